@@ -172,3 +172,23 @@ def tolerance(case):
     # Everything else is whole numbers and bit copies of rows. Two chunks would have to lie within rounding (1e-7) of
     # the k-th score for a selection to differ; neighbouring scores lie 3e-4 (tokens) to 2e-2 apart there.
     return "exact"
+
+
+def exact(case, seed):
+    """Chunk and token scores in 64 bits; the other calls' outputs are whole numbers and copies of rows."""
+    if case["kind"] != "scores":
+        return None
+    Hq, Hkv, d, L, w, c = (case[k] for k in ("Hq", "Hkv", "d", "L", "w", "c"))
+    s = prepare(case, seed)
+    P = L - w
+    chunks = torch.zeros(Hkv, -(-P // c), dtype=torch.float64, device="cuda")
+    tokens = torch.zeros(Hkv, P, dtype=torch.float64, device="cuda")
+    hidden = torch.arange(L, device="cuda")[None, :] > P + torch.arange(w, device="cuda")[:, None]
+    q = s["q"].view(Hkv, Hq // Hkv, w, d)
+    for h in range(Hkv):
+        keys = s["K"][h].double()
+        for g in range(Hq // Hkv):
+            logits = (q[h, g].double() @ keys.T) / math.sqrt(d)
+            tokens[h] += logits.masked_fill_(hidden, -math.inf).softmax(-1)[:, :P].sum(0)
+    chunks.index_add_(1, torch.arange(P, device="cuda") // c, tokens)
+    return chunks, tokens
