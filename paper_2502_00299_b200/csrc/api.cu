@@ -161,6 +161,58 @@ struct Timer {
     }
 };
 
+// What a call of the one-launch layer kernel (layer_resident.cu) wants beyond the shape.
+struct ResidentCall {
+    const void *q_obs, *K, *V;
+    void *out_K, *out_V;
+    int32_t* out_idx;              // NULL: chunk scores only
+    float* out_scores = nullptr;
+    int k = 0, n_max = 0;
+    long long kt = 0, kh = 0, vt = 0, vh = 0;   // token and head strides in elements, 0 = packed
+    const int32_t* block_table = nullptr;
+    int page_size = 0, num_pages = 0;
+    int tok_cap = 0x7fffffff;
+    bool cooperative = false;
+};
+
+// Runs the layer in the one-launch kernel where the shape fits it and `base` (header + payload, `bytes` in all) holds
+// its scratch; *done tells. A shape that does not fit, or a scratch set up for another kernel's smaller need, is left
+// to the caller's general path. Caller holds g_mu and has validated the arguments.
+int try_resident(DeviceCtx& ctx, char* base, size_t bytes, const ResidentCall& rc, int L, int Hq, int Hkv, int d, int w,
+                 int c, int C, int ctas, cudaStream_t stream, bool* done) {
+    *done = false;
+    const int R = w * (Hq / Hkv);
+    ResidentPlan plan;
+    if (C <= 0 || !make_resident_plan(L, R, Hkv, d, c, C, rc.n_max, ctas, smem_budget(ctx), &plan)) return CHUNKKV_OK;
+    if (base == nullptr || kHeaderBytes + resident_scratch_floats(plan, Hkv, C) * sizeof(float) > bytes) return CHUNKKV_OK;
+    CUtensorMap tm_q, tm_k;
+    int st = encode_bf16_3d(&tm_q, rc.q_obs, d, R, Hkv, R < 128 ? R : 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+    if (st != CHUNKKV_OK) return st;
+    st = encode_bf16_3d(&tm_k, rc.K, d, L, Hkv, L < plan.tile ? L : plan.tile, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, rc.kt, rc.kh);
+    if (st != CHUNKKV_OK) return st;
+    ResidentIO io;
+    io.L = L; io.w = w; io.R = R; io.Hkv = Hkv; io.d = d;
+    io.sl2 = static_cast<float>(1.4426950408889634 / sqrt(static_cast<double>(d)));
+    io.C = C; io.k = rc.k; io.n_max = rc.n_max;
+    io.K = rc.K; io.V = rc.V; io.out_K = rc.out_K; io.out_V = rc.out_V; io.out_idx = rc.out_idx;
+    io.out_scores = rc.out_scores;
+    io.scratch = reinterpret_cast<float*>(base + kHeaderBytes);
+    io.counters = reinterpret_cast<unsigned*>(base + kResidentCountersOffset);
+    io.status = reinterpret_cast<int*>(base);
+    io.cooperative = rc.cooperative;
+    io.k_row_elems = rc.kt; io.k_head_elems = rc.kh; io.v_row_elems = rc.vt; io.v_head_elems = rc.vh;
+    io.block_table = rc.block_table; io.page_size = rc.page_size; io.num_pages = rc.num_pages;
+    io.tok_cap = rc.tok_cap;
+    cudaError_t e;
+    {
+        Timer t(&ctx, stream, 0);
+        e = launch_layer_resident(plan, tm_q, tm_k, io, stream);
+    }
+    if (e != cudaSuccess) return cuda_fail(e);
+    *done = true;
+    return CHUNKKV_OK;
+}
+
 // Score + finalise for chunk size c. Chunk scores go to `out_scores`, or - when that is NULL -
 // to the first `extra_payload_floats` floats of the scratch payload; `*resolved` receives the
 // address used. Caller holds g_mu and has validated the arguments.
@@ -174,6 +226,19 @@ int run_score(DeviceCtx& ctx, const void* q_obs, const void* K, int L, int Hq, i
     const int R = sh.Rs;
     // with two scoring heads per KV head their chunk scores go to scratch first and are added into the output
     const size_t pair_floats = sh.shift ? round64(static_cast<size_t>(sh.Hs) * C) : 0;
+    if (out_scores != nullptr) {
+        ResidentCall rc;
+        rc.q_obs = q_obs; rc.K = K; rc.V = nullptr; rc.out_K = nullptr; rc.out_V = nullptr; rc.out_idx = nullptr;
+        rc.out_scores = out_scores;
+        rc.kt = k_row_elems; rc.kh = k_head_elems;
+        bool done;
+        int st1 = try_resident(ctx, static_cast<char*>(ctx.ws), ctx.ws_bytes, rc, L, Hq, Hkv, d, w, c, C, ctx.num_sms, stream, &done);
+        if (st1 != CHUNKKV_OK) return st1;
+        if (done) {
+            if (resolved != nullptr) *resolved = out_scores;
+            return CHUNKKV_OK;
+        }
+    }
     TokenPlan tplan;
     if (c == 1 && make_token_plan(L, w, R, sh.Hs, d, ctx.num_sms, smem_budget(ctx), &tplan)) {
         // token scores: two passes over the keys in one launch, nothing but row records in scratch
@@ -359,8 +424,8 @@ size_t chunkkv_workspace_bytes(int L, int Hq, int Hkv, int d, int w, int c) {
     size_t floats = scratch_floats_for(*ctx, L, sh.Rs, sh.Hs, d, c) + round64(static_cast<size_t>(Hkv) * C) +
                     round64(static_cast<size_t>(sh.Hs) * C);
     ResidentPlan rplan;
-    if (C > 0 && make_resident_plan(L, sh.Rs, sh.Hs, sh.shift, d, c, C, 0, ctx->num_sms, smem_budget(*ctx), &rplan)) {
-        const size_t rf = resident_scratch_floats(rplan, sh.Hs, C);
+    if (C > 0 && make_resident_plan(L, w * (Hq / Hkv), Hkv, d, c, C, 0, ctx->num_sms, smem_budget(*ctx), &rplan)) {
+        const size_t rf = resident_scratch_floats(rplan, Hkv, C);
         floats = rf > floats ? rf : floats;
     }
     return kHeaderBytes + floats * sizeof(float);
@@ -524,39 +589,16 @@ static int compress_impl(const void* q_obs, const void* K, const void* V, int L,
         // small CTAs that spread over every SM (they fit beside the other lanes' resident
         // CTAs), instead of moving the rows through its own few SMs.
         const bool split = rows_elsewhere != nullptr || (lane != nullptr && 2 * ctas <= ctx->num_sms);
-        ResidentPlan rplan;
-        if (!split && make_resident_plan(L, R, sh.Hs, sh.shift, d, c, C, n_max, ctas, smem_budget(*ctx), &rplan)) {
-            // One cooperative launch; the chunk partial sums never leave the SMs.
-            const size_t need = resident_scratch_floats(rplan, sh.Hs, C) * sizeof(float);
-            char* base;
-            if (lane != nullptr) {
-                if (kHeaderBytes + need > lane_bytes) return CHUNKKV_ENOWORKSPACE;
-                base = static_cast<char*>(lane);
-            } else {
-                st = ensure_workspace(*ctx, need);
-                if (st != CHUNKKV_OK) return st;
-                base = static_cast<char*>(ctx->ws);
-            }
-            CUtensorMap tm_q, tm_k;
-            st = encode_bf16_3d(&tm_q, q_obs, d, R, sh.Hs, R < 128 ? R : 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
-            if (st != CHUNKKV_OK) return st;
-            st = encode_bf16_3d(&tm_k, K, d, L, Hkv, L < 120 ? L : 120, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
-            if (st != CHUNKKV_OK) return st;
-            ResidentIO io;
-            io.L = L; io.w = w; io.Rs = R; io.Hs = sh.Hs; io.d = d; io.kv_shift = sh.shift;
-            io.sl2 = static_cast<float>(1.4426950408889634 / sqrt(static_cast<double>(d)));
-            io.C = C; io.k = k; io.n_max = n_max;
-            io.K = K; io.V = V; io.out_K = out_K; io.out_V = out_V; io.out_idx = out_idx;
-            io.scratch = reinterpret_cast<float*>(base + kHeaderBytes);
-            io.counters = reinterpret_cast<unsigned*>(base + kResidentCountersOffset);
-            io.status = reinterpret_cast<int*>(base);
-            io.cooperative = lane != nullptr;
-            {
-                Timer t(ctx, s, 0);
-                e = launch_layer_resident(rplan, tm_q, tm_k, io, s);
-            }
-            if (e != cudaSuccess) return cuda_fail(e);
-            return CHUNKKV_OK;
+        if (!split) {
+            // One launch; the chunk partial sums stay on chip as far as they fit there.
+            ResidentCall rc;
+            rc.q_obs = q_obs; rc.K = K; rc.V = V; rc.out_K = out_K; rc.out_V = out_V; rc.out_idx = out_idx;
+            rc.k = k; rc.n_max = n_max;
+            rc.cooperative = lane != nullptr;
+            bool done;
+            st = try_resident(*ctx, static_cast<char*>(lane != nullptr ? lane : ctx->ws), lane != nullptr ? lane_bytes : ctx->ws_bytes,
+                              rc, L, Hq, Hkv, d, w, c, C, ctas, s, &done);
+            if (st != CHUNKKV_OK || done) return st;
         }
         ScorePlan plan;
         TokenPlan tplan;
@@ -672,33 +714,13 @@ int chunkkv_compress_layer_strided(const void* q_obs, const void* K, const void*
     const int32_t* idx = reuse_idx;
     if (reuse_idx == nullptr && C > 0 && k > 0) {
         // the one-launch layer kernel takes strided keys and values as they are (tensor map and gather strides)
-        const ScoreShape sh = score_shape(Hq, Hkv, w);
-        ResidentPlan rplan;
-        if (make_resident_plan(L, sh.Rs, sh.Hs, sh.shift, d, c, C, n_max, ctx->num_sms, smem_budget(*ctx), &rplan)) {
-            st = ensure_workspace(*ctx, resident_scratch_floats(rplan, sh.Hs, C) * sizeof(float));
-            if (st != CHUNKKV_OK) return st;
-            char* base = static_cast<char*>(ctx->ws);
-            CUtensorMap tm_q, tm_k;
-            st = encode_bf16_3d(&tm_q, q_obs, d, sh.Rs, sh.Hs, sh.Rs < 128 ? sh.Rs : 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
-            if (st != CHUNKKV_OK) return st;
-            st = encode_bf16_3d(&tm_k, K, d, L, Hkv, L < 120 ? L : 120, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, k_token_stride,
-                                k_head_stride);
-            if (st != CHUNKKV_OK) return st;
-            ResidentIO io;
-            io.L = L; io.w = w; io.Rs = sh.Rs; io.Hs = sh.Hs; io.d = d; io.kv_shift = sh.shift;
-            io.sl2 = static_cast<float>(1.4426950408889634 / sqrt(static_cast<double>(d)));
-            io.C = C; io.k = k; io.n_max = n_max;
-            io.K = K; io.V = V; io.out_K = out_K; io.out_V = out_V; io.out_idx = out_idx;
-            io.scratch = reinterpret_cast<float*>(base + kHeaderBytes);
-            io.counters = reinterpret_cast<unsigned*>(base + kResidentCountersOffset);
-            io.status = reinterpret_cast<int*>(base);
-            io.cooperative = false;
-            io.k_row_elems = k_token_stride; io.k_head_elems = k_head_stride;
-            io.v_row_elems = v_token_stride; io.v_head_elems = v_head_stride;
-            e = launch_layer_resident(rplan, tm_q, tm_k, io, s);
-            if (e != cudaSuccess) return cuda_fail(e);
-            return CHUNKKV_OK;
-        }
+        ResidentCall rc;
+        rc.q_obs = q_obs; rc.K = K; rc.V = V; rc.out_K = out_K; rc.out_V = out_V; rc.out_idx = out_idx;
+        rc.k = k; rc.n_max = n_max;
+        rc.kt = k_token_stride; rc.kh = k_head_stride; rc.vt = v_token_stride; rc.vh = v_head_stride;
+        bool done;
+        st = try_resident(*ctx, static_cast<char*>(ctx->ws), ctx->ws_bytes, rc, L, Hq, Hkv, d, w, c, C, ctx->num_sms, s, &done);
+        if (st != CHUNKKV_OK || done) return st;
     }
     if (reuse_idx == nullptr) {
         float* chunk_scores = nullptr;
@@ -792,31 +814,13 @@ int chunkkv_compress_layer_paged(const void* q_obs, const void* K, const void* V
     } else {
         if (C > 0 && k > 0) {
             // the one-launch layer kernel places the kept rows through the block table itself
-            const ScoreShape sh = score_shape(Hq, Hkv, w);
-            ResidentPlan rplan;
-            if (make_resident_plan(L, sh.Rs, sh.Hs, sh.shift, d, c, C, n_max, ctx->num_sms, smem_budget(*ctx), &rplan)) {
-                st = ensure_workspace(*ctx, resident_scratch_floats(rplan, sh.Hs, C) * sizeof(float));
-                if (st != CHUNKKV_OK) return st;
-                char* base = static_cast<char*>(ctx->ws);
-                CUtensorMap tm_q, tm_k;
-                st = encode_bf16_3d(&tm_q, q_obs, d, sh.Rs, sh.Hs, sh.Rs < 128 ? sh.Rs : 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
-                if (st != CHUNKKV_OK) return st;
-                st = encode_bf16_3d(&tm_k, K, d, L, Hkv, L < 120 ? L : 120, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
-                if (st != CHUNKKV_OK) return st;
-                ResidentIO io;
-                io.L = L; io.w = w; io.Rs = sh.Rs; io.Hs = sh.Hs; io.d = d; io.kv_shift = sh.shift;
-                io.sl2 = static_cast<float>(1.4426950408889634 / sqrt(static_cast<double>(d)));
-                io.C = C; io.k = k; io.n_max = n_max;
-                io.K = K; io.V = V; io.out_K = cache_K; io.out_V = cache_V; io.out_idx = out_idx;
-                io.scratch = reinterpret_cast<float*>(base + kHeaderBytes);
-                io.counters = reinterpret_cast<unsigned*>(base + kResidentCountersOffset);
-                io.status = reinterpret_cast<int*>(base);
-                io.cooperative = false;
-                io.block_table = block_table; io.page_size = page_size; io.num_pages = num_pages;
-                e = launch_layer_resident(rplan, tm_q, tm_k, io, s);
-                if (e != cudaSuccess) return cuda_fail(e);
-                return CHUNKKV_OK;
-            }
+            ResidentCall rc;
+            rc.q_obs = q_obs; rc.K = K; rc.V = V; rc.out_K = cache_K; rc.out_V = cache_V; rc.out_idx = out_idx;
+            rc.k = k; rc.n_max = n_max;
+            rc.block_table = block_table; rc.page_size = page_size; rc.num_pages = num_pages;
+            bool done;
+            st = try_resident(*ctx, static_cast<char*>(ctx->ws), ctx->ws_bytes, rc, L, Hq, Hkv, d, w, c, C, ctx->num_sms, s, &done);
+            if (st != CHUNKKV_OK || done) return st;
         }
         float* chunk_scores = nullptr;
         if (C > 0 && k > 0) {
@@ -1111,31 +1115,13 @@ int chunkkv_compress_layer_alg1(const void* q_obs, const void* K, const void* V,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (C > 0 && k > 0) {
         // the one-launch layer kernel with Algorithm 1's chunk count and token cap
-        const ScoreShape sh = score_shape(Hq, Hkv, w);
-        ResidentPlan rplan;
-        if (make_resident_plan(L, sh.Rs, sh.Hs, sh.shift, d, c, C, n_max, ctx->num_sms, smem_budget(*ctx), &rplan)) {
-            st = ensure_workspace(*ctx, resident_scratch_floats(rplan, sh.Hs, C) * sizeof(float));
-            if (st != CHUNKKV_OK) return st;
-            char* base = static_cast<char*>(ctx->ws);
-            CUtensorMap tm_q, tm_k;
-            st = encode_bf16_3d(&tm_q, q_obs, d, sh.Rs, sh.Hs, sh.Rs < 128 ? sh.Rs : 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
-            if (st != CHUNKKV_OK) return st;
-            st = encode_bf16_3d(&tm_k, K, d, L, Hkv, L < 120 ? L : 120, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
-            if (st != CHUNKKV_OK) return st;
-            ResidentIO io;
-            io.L = L; io.w = w; io.Rs = sh.Rs; io.Hs = sh.Hs; io.d = d; io.kv_shift = sh.shift;
-            io.sl2 = static_cast<float>(1.4426950408889634 / sqrt(static_cast<double>(d)));
-            io.C = C; io.k = k; io.n_max = n_max;
-            io.K = K; io.V = V; io.out_K = out_K; io.out_V = out_V; io.out_idx = out_idx;
-            io.scratch = reinterpret_cast<float*>(base + kHeaderBytes);
-            io.counters = reinterpret_cast<unsigned*>(base + kResidentCountersOffset);
-            io.status = reinterpret_cast<int*>(base);
-            io.cooperative = false;
-            io.tok_cap = budget - w;
-            cudaError_t e2 = launch_layer_resident(rplan, tm_q, tm_k, io, s);
-            if (e2 != cudaSuccess) return cuda_fail(e2);
-            return CHUNKKV_OK;
-        }
+        ResidentCall rc;
+        rc.q_obs = q_obs; rc.K = K; rc.V = V; rc.out_K = out_K; rc.out_V = out_V; rc.out_idx = out_idx;
+        rc.k = k; rc.n_max = n_max;
+        rc.tok_cap = budget - w;
+        bool done;
+        st = try_resident(*ctx, static_cast<char*>(ctx->ws), ctx->ws_bytes, rc, L, Hq, Hkv, d, w, c, C, ctx->num_sms, s, &done);
+        if (st != CHUNKKV_OK || done) return st;
     }
     float* chunk_scores = nullptr;
     if (C > 0 && k > 0) {
@@ -1162,8 +1148,8 @@ size_t chunkkv_lane_bytes(int L, int Hq, int Hkv, int d, int w, int c, int max_c
     if (!make_score_plan(L, sh.Rs, sh.Hs, d, c, ctas, smem_budget(*ctx), true, &plan)) return 0;
     size_t floats = score_scratch_floats(plan, sh.Hs, sh.Rs) + round64(static_cast<size_t>(sh.Hs) * C);
     ResidentPlan rplan;
-    if (C > 0 && make_resident_plan(L, sh.Rs, sh.Hs, sh.shift, d, c, C, 0, ctas, smem_budget(*ctx), &rplan)) {
-        const size_t rf = resident_scratch_floats(rplan, sh.Hs, C);
+    if (C > 0 && make_resident_plan(L, w * (Hq / Hkv), Hkv, d, c, C, 0, ctas, smem_budget(*ctx), &rplan)) {
+        const size_t rf = resident_scratch_floats(rplan, Hkv, C);
         floats = rf > floats ? rf : floats;
     }
     return kHeaderBytes + floats * sizeof(float);

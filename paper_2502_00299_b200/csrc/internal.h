@@ -79,26 +79,30 @@ cudaError_t launch_layer_fused(const ScorePlan& plan, const CUtensorMap& tm_q, c
                                const ScoreArgs& args, const FusedLayerIO& io, cudaStream_t stream);
 
 // The layer kernel that keeps its chunk partial sums in tensor memory (layer_resident.cu): every CTA
-// belongs to one scoring head, `cph` CTAs per head.
+// belongs to one KV head, `cph` CTAs per head.
 struct ResidentPlan {
-    int c_static;     // 10 or 20
+    int c_static;     // 5, 8, 10, 16, 20 or 32
+    int n_mt;         // 128-row query tiles per KV head (1 or 2)
     int grid, cph;
-    int n_tiles;      // 120-key accumulator tiles per head
+    int tile, n_tiles;   // keys per accumulator tile, tiles per head
     int t_max;        // most tiles any CTA takes
+    int spp;          // chunk slots per panel (half a tile)
+    int n_on, n_off;  // panels of a CTA whose partial sums stay on chip; the others go to scratch
     int n_stages;
     int smem_bytes;
     int off_ring, ring_bytes, off_pmax, off_misc;
 };
 
 struct ResidentIO {
-    int L, w, Rs, Hs, d, kv_shift;   // Rs rows per scoring head, Hs scoring heads, KV head = scoring head >> kv_shift
+    int L, w, R, Hkv, d;  // R = w * Hq / Hkv query rows per KV head
     float sl2;
     int C, k, n_max;
     const void* K;
     const void* V;
     void* out_K;
     void* out_V;
-    int32_t* out_idx;
+    int32_t* out_idx;     // NULL: chunk scores only (out_scores)
+    float* out_scores = nullptr;   // [Hkv, C]; NULL: in scratch
     float* scratch;       // resident_scratch_floats() floats
     unsigned* counters;   // header + kResidentCountersOffset
     int* status;
@@ -112,11 +116,11 @@ struct ResidentIO {
     int tok_cap = 0x7fffffff;
 };
 
-// false when the shape does not fit this kernel (chunk size other than 10 / 20, more than 128 rows
-// per scoring head, more chunks per CTA than tensor memory holds, fewer CTAs than scoring heads).
-bool make_resident_plan(int L, int Rs, int Hs, int kv_shift, int d, int c, int C, int n_max, int max_ctas,
-                        int smem_limit, ResidentPlan* plan);
-size_t resident_scratch_floats(const ResidentPlan& plan, int Hs, int C);
+// false when the shape does not fit this kernel (a chunk size other than the six, more than 256 rows, fewer CTAs
+// than heads, kept positions or chunk scores beyond shared memory).
+bool make_resident_plan(int L, int R, int Hkv, int d, int c, int C, int n_max, int max_ctas, int smem_limit,
+                        ResidentPlan* plan);
+size_t resident_scratch_floats(const ResidentPlan& plan, int Hkv, int C);
 cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                                   const ResidentIO& io, cudaStream_t stream);
 

@@ -1,12 +1,27 @@
 // The whole layer in one cooperative launch with the chunk partial sums kept on chip
 // (ChunkKV Algorithm 3: observe-window scores, chunk scores, top-k, index_select on K and V).
 //
-// Every CTA belongs to one scoring head (a KV head, or one half of its query rows when a KV head
-// has more than 128 of them) and owns a contiguous range of that head's keys. While it streams its
+// Every CTA belongs to one KV head and owns a contiguous range of its keys. While it streams its
 // keys through the tensor cores it keeps, per query row and chunk, the sum of exp2(s - m_panel) in
 // TENSOR MEMORY (lane = query row, column = chunk of the CTA's range, 256 columns beside the two
-// accumulator buffers) and the panel maxima in shared memory, so nothing but a (max, sum) pair per
-// row and CTA ever goes to global memory before the chunk scores themselves:
+// accumulator buffers) and the panel maxima in shared memory, so for most shapes nothing but a
+// (max, sum) pair per row and CTA goes to global memory before the chunk scores themselves. A key
+// range with more panels than those 256 columns hold (long contexts, small chunks) keeps the rest
+// in scratch (L2): written and read back by the same thread, one row per lane, coalesced.
+//
+// A KV head with more than 128 query rows (two query tiles) is scored by the same CTAs: each key
+// tile is loaded once and multiplied with both query tiles, and the two pairs of epilogue groups
+// take one query tile each; with one query tile the pairs take alternate key tiles. In both cases
+// the CTA's products are numbered in issue order ("virtual tiles"), accumulator and pair = number
+// modulo 2, so one set of loops serves both.
+//
+// What bounds it (8 KV heads, d 128, B200): up to 128 rows the DRAM stream of K while scoring (13 of
+// 33.5 us at 32K tokens, c = 10) and then a chain of latencies (two hand-overs, selection, gather);
+// beyond 128 rows the special-function unit (one exponential per score element, 16 per clock and
+// SM: 78 % of that rate while scoring). Against the kernel of score.cu, which kept every partial sum
+// in scratch, loaded K once per query tile and took run-time chunk sizes: c = 16, 29695 tokens, 256 rows
+// 107 -> 41 us; c = 20, 131072 tokens, 256 rows 147 -> 134 us; chunk scores alone (c = 10, 62261
+// tokens, 128 rows, four launches) 50 -> 33 us.
 //
 //   1. score      TMA -> tcgen05.mma (128 rows x 120 keys per accumulator tile) -> epilogue
 //                 warps: one exponential per score element, chunk sums to tensor memory
@@ -19,6 +34,8 @@
 //                 and so holds the kept token positions in shared memory without a third wait;
 //                 one of them writes out_idx
 //   6. gather     the head's output rows are split evenly over its CTAs
+//
+// Without out_idx the kernel ends after step 3 (chunk scores are the result).
 //
 // Heads never wait for each other. The launch is cooperative only so that all CTAs are resident
 // while they wait for their head's other CTAs; every wait gives up after a clock limit, raises the
@@ -37,7 +54,7 @@ namespace chunkkv {
 namespace {
 
 constexpr int kRThreads = 576;               // warp 0: TMA, warp 1: UMMA issue, warps 2..17: epilogue
-constexpr int kRMiscBytes = 14336;           // records of the four epilogue groups, slices, m_i, 1 / l_i, row sums per lane quarter
+constexpr int kRMiscBytes = 10240;           // records of the four epilogue groups, slices, m_i, 1 / l_i
 
 struct ResCtl {
     unsigned long long full[kRMaxStages];
@@ -51,14 +68,16 @@ struct ResCtl {
 };
 
 struct ResArgs {
-    int L, P, w, R, Hs, d, kv_shift;   // R rows per scoring head, Hs scoring heads
+    int L, P, w, R, d;                 // R rows per KV head
+    int n_mt;                          // 128-row query tiles per KV head (1 or 2)
     float sl2;                         // log2(e) / sqrt(d)
-    int cph;                           // CTAs per scoring head (grid = Hs * cph)
+    int cph;                           // CTAs per KV head (grid = Hkv * cph)
     int n_tiles;                       // accumulator tiles per head
     int n_stages;
     int q_box_rows, k_box_rows;
     int C, k, n_max, Hkv;
     int off_ring, ring_bytes, off_pmax, off_misc;   // dynamic shared memory layout (bytes from the aligned base)
+    int n_on, n_off;                   // panels of a CTA kept on chip; room for panels in scratch
     const uint4* K;
     const uint4* V;
     long long k_row, k_head, v_row, v_head;   // 16-byte vectors between rows of a head / between heads
@@ -68,9 +87,10 @@ struct ResArgs {
     uint4* out_K;
     uint4* out_V;
     int32_t* out_idx;
-    float* cta_stat;                   // [grid, {max, sum}, 128]
-    float* scores;                     // [Hs, C]
-    unsigned* cnt_a;                   // [Hs]  hand-over 2, zero between launches
+    float* cta_stat;                   // [grid, n_mt, {max, sum}, 128]
+    float* scores;                     // [Hkv, C]
+    float* spill;                      // [grid, n_off, 1 + chunk slots per panel, 128]: panel maximum, chunk sums
+    unsigned* cnt_a;                   // [Hkv] hand-over 2, zero between launches
     unsigned* cnt_b;                   // [Hkv] hand-over 4
     unsigned* exits;                   // CTAs that left; the last one clears the counters
     int* status;
@@ -101,13 +121,18 @@ __device__ __forceinline__ bool head_handover(unsigned* counter, unsigned target
     return ctl.wait_ok != 0;
 }
 
-template <int C_STATIC>
+// BIG: two query tiles, or panels in scratch. A variant of its own: the code for either, present but not taken, costs
+// the other shapes 1.5 us of 34 (32K tokens, 128 rows).
+template <int C_STATIC, bool BIG>
 __global__ void __launch_bounds__(kRThreads, 1)
 layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                       const ResArgs a) {
-    constexpr int SPP = kRPanel / C_STATIC;          // chunk slots per panel
+    constexpr int WP = panel_keys(C_STATIC);         // keys per epilogue panel
+    constexpr int TILE = 2 * WP;                     // keys per accumulator tile
+    constexpr uint32_t STAGE = TILE * 128;           // one ring stage: a tile's keys x 64 dims
+    constexpr int SPP = WP / C_STATIC;               // chunk slots per panel
     constexpr uint32_t IDESC = umma_idesc_bf16(128, kRUmmaN);
-    static_assert(kRPanel % C_STATIC == 0, "the chunk size must divide the panel");
+    static_assert(WP % C_STATIC == 0, "the chunk size must divide the panel");
 
     extern __shared__ uint8_t smem_raw[];
     __shared__ ResCtl ctl;
@@ -122,18 +147,20 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     float* misc = reinterpret_cast<float*>(dyn + a.off_misc);
     float* rec = misc;                 // [4 groups][{max, sum}][128]
     float* slice = misc + 1024;        // [4 slices][{max, sum}][128]
-    float* gm = misc + 2048;           // [128] row maxima of the head
-    float* ginv = misc + 2176;         // [128] 1 / row sums of the head
+    float* gm = misc + 2048;           // [2 query tiles][128] row maxima of the head
+    float* ginv = misc + 2304;         // [2 query tiles][128] 1 / row sums of the head
     uint8_t* ring = dyn + a.off_ring;  // reused after scoring
     volatile int* abort_flag = &ctl.abort_flag;
     const uint32_t n_stages = static_cast<uint32_t>(a.n_stages);
 
-    const int hs = blockIdx.x / a.cph, part = blockIdx.x - hs * a.cph;
-    const int hkv = hs >> a.kv_shift;
+    const int hkv = blockIdx.x / a.cph, part = blockIdx.x - hkv * a.cph;
     // tiles are dealt out rounding up, so the head's last CTA - whose last panels take the slow, masked path -
     // is never one of those that get an extra tile
     const int t_begin = (a.n_tiles * part + a.cph - 1) / a.cph, t_end = (a.n_tiles * (part + 1) + a.cph - 1) / a.cph;
     const int nt = t_end - t_begin;
+    const int n_mt = BIG ? a.n_mt : 1;
+    const bool two = n_mt == 2;                      // two query tiles
+    const int n_vt = nt << (two ? 1 : 0);            // virtual tiles: (key tile, query tile) products of this CTA
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < a.n_stages; ++s) {
@@ -147,6 +174,8 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         mbar_init(smem_u32(&ctl.qfull), 1);
         ctl.abort_flag = 0;
         ctl.wait_ok = 1;
+        prefetch_tmap(&tm_q);            // (kernel parameters: not written by the kernel ahead of this one)
+        prefetch_tmap(&tm_k);
         fence_mbar_init();
         fence_proxy_async();
     }
@@ -167,12 +196,11 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (elect_one() && nt > 0) {
-            prefetch_tmap(&tm_q);
-            prefetch_tmap(&tm_k);
             const uint32_t qbar = smem_u32(&ctl.qfull);
-            mbar_arrive_expect_tx(qbar, static_cast<uint32_t>(KB * a.q_box_rows) * 128u);
-            for (int kb = 0; kb < KB; ++kb)
-                tma_load_3d(q_base + static_cast<uint32_t>(kb) * kRQTileBytes, &tm_q, qbar, kb * 64, 0, hs);
+            mbar_arrive_expect_tx(qbar, static_cast<uint32_t>(n_mt * KB * a.q_box_rows) * 128u);
+            for (int mt = 0; mt < n_mt; ++mt)      // (rows past R of the second tile arrive as zeros)
+                for (int kb = 0; kb < KB; ++kb)
+                    tma_load_3d(q_base + static_cast<uint32_t>(mt * KB + kb) * kRQTileBytes, &tm_q, qbar, kb * 64, mt * 128, hkv);
             const uint32_t k_bytes = static_cast<uint32_t>(a.k_box_rows) * 128u;
             uint32_t st = 0, st_par = 1;
             int issued = 0;
@@ -183,7 +211,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                     if (!ok) break;
                     const uint32_t bar = smem_u32(&ctl.full[st]);
                     mbar_arrive_expect_tx(bar, k_bytes);
-                    tma_load_3d(k_base + st * kRStageBytes, &tm_k, bar, kb * 64, t * kRTile, hkv);
+                    tma_load_3d(k_base + st * STAGE, &tm_k, bar, kb * 64, t * TILE, hkv);
                     ++issued;
                     if (++st == n_stages) { st = 0; st_par ^= 1u; }
                 }
@@ -205,62 +233,80 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         if (elect_one() && nt > 0) {
             bool ok = mbar_wait(smem_u32(&ctl.qfull), 0, abort_flag);
             uint32_t st = 0, st_par = 0;
-            for (int ti = 0; ti < nt && ok; ++ti) {
-                const int buf = ti & 1, use = ti >> 1;
-                ok = mbar_wait(smem_u32(&ctl.tempty[buf]), (use & 1) ^ 1, abort_flag);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t d_addr = tmem_base + static_cast<uint32_t>(buf * kRUmmaN);
+            for (int ti = 0, vt = 0; ti < nt && ok; ++ti) {
+                uint32_t st_kb[2] = {0u, 0u};
 #pragma unroll
                 for (int kb = 0; kb < 2; ++kb) {          // d is 64 or 128: one or two 64-element blocks
                     if (kb >= KB || !ok) break;
                     ok = mbar_wait(smem_u32(&ctl.full[st]), st_par, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint64_t b_desc = umma_desc_sw128(k_base + st * kRStageBytes);
-                    const uint64_t a_desc = umma_desc_sw128(q_base + static_cast<uint32_t>(kb) * kRQTileBytes);
-#pragma unroll
-                    for (int k4 = 0; k4 < 4; ++k4)      // k-steps advance the start address by 32 bytes
-                        umma_bf16(d_addr, a_desc + 2u * k4, b_desc + 2u * k4, IDESC, (kb > 0 || k4 > 0) ? 1u : 0u);
-                    umma_commit(smem_u32(&ctl.empty[st]));
+                    st_kb[kb] = st;
                     if (++st == n_stages) { st = 0; st_par ^= 1u; }
                 }
-                if (ok) umma_commit(smem_u32(&ctl.tfull[buf]));
+                for (int mt = 0; mt < n_mt && ok; ++mt, ++vt) {
+                    const int buf = vt & 1, use = vt >> 1;
+                    ok = mbar_wait(smem_u32(&ctl.tempty[buf]), (use & 1) ^ 1, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t d_addr = tmem_base + static_cast<uint32_t>(buf * kRUmmaN);
+#pragma unroll
+                    for (int kb = 0; kb < 2; ++kb) {
+                        if (kb >= KB) break;
+                        const uint64_t b_desc = umma_desc_sw128(k_base + st_kb[kb] * STAGE);
+                        const uint64_t a_desc = umma_desc_sw128(q_base + static_cast<uint32_t>(mt * KB + kb) * kRQTileBytes);
+#pragma unroll
+                        for (int k4 = 0; k4 < 4; ++k4)      // k-steps advance the start address by 32 bytes
+                            umma_bf16(d_addr, a_desc + 2u * k4, b_desc + 2u * k4, IDESC, (kb > 0 || k4 > 0) ? 1u : 0u);
+                    }
+                    umma_commit(smem_u32(&ctl.tfull[buf]));
+                }
+                if (!ok) break;
+#pragma unroll
+                for (int kb = 0; kb < 2; ++kb)
+                    if (kb < KB) umma_commit(smem_u32(&ctl.empty[st_kb[kb]]));
             }
         }
     } else {
         // ------------------------------------------------------------------ epilogue
         // Four groups of four warps (a group's warps cover the four tensor-memory lane quarters =
-        // the 128 query rows). The groups form two pairs that take alternate accumulator tiles;
-        // inside a pair each group takes one 60-key half of the tile.
+        // 128 query rows). The groups form two pairs that take alternate virtual tiles; inside a
+        // pair each group takes one half (panel) of the tile.
         const int grp = (warp - 2) >> 2, quarter = warp & 3;
         const int pair = grp >> 1, half = grp & 1;
-        const int row = quarter * 32 + lane;
-        const bool active = row < a.R;
-        const int last_visible = a.P + (row % a.w);      // this row sees keys j <= P + r (all < L)
+        const int row = quarter * 32 + lane;             // row of the query tile = lane of tensor memory
+        const int qrow = row + (two ? pair * 128 : 0);   // row of the KV head
+        const bool active = qrow < a.R;
+        const int last_visible = a.P + (qrow % a.w);     // this row sees keys j <= P + r (all < L)
         const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+        const uint64_t keep = l2_policy_evict_last();
         float run_m = -CUDART_INF_F, run_l = 0.f;
-        for (int ti = pair; ti < nt; ti += 2) {
-            const int use = ti >> 1;
+        for (int vt = pair; vt < n_vt; vt += 2) {
+            const int use = vt >> 1, ti = two ? use : vt;
             bool ready = true;                           // one lane polls, the warp follows
             if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[pair]), use & 1, abort_flag);
             if (!__shfl_sync(0xffffffffu, ready, 0)) break;
             tc_fence_after();
-            float v[kRPanel];
-            load_panel<kRPanel>(lane_addr + static_cast<uint32_t>(pair * kRUmmaN + half * kRPanel), v);
+            float v[WP];
+            load_panel<WP>(lane_addr + static_cast<uint32_t>(pair * kRUmmaN + half * WP), v);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&ctl.tempty[pair]));   // the buffer may be overwritten now
-            const int pl = ti * 2 + half;                // panel of this CTA
-            const int j0 = (t_begin + ti) * kRTile + half * kRPanel;
+            const int pl = vt * 2 + half;                // panel of this CTA; pl % 4 == grp
+            const int j0 = (t_begin + ti) * TILE + half * WP;
             float pr[SPP], m2, l;
             auto emit = [&](int ch, float acc) { pr[ch] = acc; };
-            if (j0 + kRPanel <= a.P)
-                panel_fast<C_STATIC, kRPanel>(v, a.sl2, emit, &m2, &l);
+            if (j0 + WP <= a.P)
+                panel_fast<C_STATIC, WP>(v, a.sl2, emit, &m2, &l);
             else
-                panel_static_tail<C_STATIC, kRPanel>(v, a.sl2, emit, j0, a.P, last_visible, &m2, &l);
-            part_store<SPP>(lane_addr + static_cast<uint32_t>(kRPartCol0 + pl * SPP), pr);
-            pmax[pl * 128 + row] = m2;
+                panel_static_tail<C_STATIC, WP>(v, a.sl2, emit, j0, a.P, last_visible, &m2, &l);
+            if (!BIG || pl < a.n_on) {
+                part_store<SPP>(lane_addr + static_cast<uint32_t>(kRPartCol0 + pl * SPP), pr);
+                pmax[pl * 128 + row] = m2;
+            } else {
+                float* sp = a.spill + (static_cast<size_t>(blockIdx.x) * a.n_off + (pl - a.n_on)) * ((SPP + 1) * 128) + row;
+                st_keep(sp, m2, keep);
+#pragma unroll
+                for (int q = 0; q < SPP; ++q) st_keep(sp + (q + 1) * 128, pr[q], keep);
+            }
             // fold into the running record: l is relative to m2, run_l to run_m
             const float nm = fmaxf(run_m, m2);
             const float s_old = (run_m == -CUDART_INF_F) ? 0.f : ex2_approx(run_m - nm);
@@ -280,36 +326,42 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 
     // ---- 2. this CTA's (max, sum) per row -> global memory; wait for the head's other CTAs
     if (ok) {
-        if (threadIdx.x < 128) {
-            const int i = threadIdx.x;
+        if (static_cast<int>(threadIdx.x) < n_mt * 128) {
+            const int i = threadIdx.x & 127;
+            const int g0 = two ? (threadIdx.x >> 7) * 2 : 0, g1 = two ? g0 + 2 : 4;   // groups that scored this query tile
             float M = -CUDART_INF_F, Ls = 0.f;
 #pragma unroll
-            for (int g = 0; g < 4; ++g) M = fmaxf(M, rec[(g * 2) * 128 + i]);
+            for (int g = 0; g < 4; ++g)
+                if (g >= g0 && g < g1) M = fmaxf(M, rec[(g * 2) * 128 + i]);
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                const float m = rec[(g * 2) * 128 + i];
-                Ls += (m == -CUDART_INF_F) ? 0.f : rec[(g * 2 + 1) * 128 + i] * ex2_approx(m - M);
-            }
-            float* dst = a.cta_stat + static_cast<size_t>(blockIdx.x) * 256;
+            for (int g = 0; g < 4; ++g)
+                if (g >= g0 && g < g1) {
+                    const float m = rec[(g * 2) * 128 + i];
+                    Ls += (m == -CUDART_INF_F) ? 0.f : rec[(g * 2 + 1) * 128 + i] * ex2_approx(m - M);
+                }
+            float* dst = a.cta_stat + (static_cast<size_t>(blockIdx.x) * n_mt + (threadIdx.x >> 7)) * 256;
             dst[i] = M;
             dst[128 + i] = Ls;
         }
-        ok = head_handover(a.cnt_a + hs, static_cast<unsigned>(a.cph), ctl);
+        ok = head_handover(a.cnt_a + hkv, static_cast<unsigned>(a.cph), ctl);
     }
 
     // ---- 3. row statistics of the head, then this CTA's chunk scores
     if (ok) {
+        // 512 threads: four (one query tile) or two (two tiles) slices of the records per row
+        const int n_sl = two ? 2 : 4;
         if (threadIdx.x < 512) {
-            const int i = threadIdx.x & 127, sl = threadIdx.x >> 7;
-            const float* src = a.cta_stat + static_cast<size_t>(hs) * a.cph * 256 + i;
+            const int i = threadIdx.x & 127, sl = (threadIdx.x >> 7) & (n_sl - 1), mt = two ? threadIdx.x >> 8 : 0;
+            const size_t step = static_cast<size_t>(n_mt) * 256;
+            const float* src = a.cta_stat + (static_cast<size_t>(hkv) * a.cph * n_mt + mt) * 256 + i;
             float M = -CUDART_INF_F, Ls = 0.f;
-            for (int j0 = sl; j0 < a.cph; j0 += 16) {     // four records in flight per thread
+            for (int j0 = sl; j0 < a.cph; j0 += 4 * n_sl) {     // four records in flight per thread
                 float rm[4], rl[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const int j = j0 + 4 * u;
-                    rm[u] = (j < a.cph) ? __ldcg(src + static_cast<size_t>(j) * 256) : -CUDART_INF_F;
-                    rl[u] = (j < a.cph) ? __ldcg(src + static_cast<size_t>(j) * 256 + 128) : 0.f;
+                    const int j = j0 + n_sl * u;
+                    rm[u] = (j < a.cph) ? __ldcg(src + j * step) : -CUDART_INF_F;
+                    rl[u] = (j < a.cph) ? __ldcg(src + j * step + 128) : 0.f;
                 }
                 float bm = M;
 #pragma unroll
@@ -320,90 +372,116 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 M = bm;
                 Ls = acc;
             }
-            slice[(sl * 2 + 0) * 128 + i] = M;
-            slice[(sl * 2 + 1) * 128 + i] = Ls;
+            slice[((threadIdx.x >> 7) * 2 + 0) * 128 + i] = M;
+            slice[((threadIdx.x >> 7) * 2 + 1) * 128 + i] = Ls;
         }
         __syncthreads();
-        if (threadIdx.x < 128) {
-            const int i = threadIdx.x;
+        if (static_cast<int>(threadIdx.x) < n_mt * 128) {
+            const int i = threadIdx.x & 127, s0 = (threadIdx.x >> 7) * n_sl;
             float M = -CUDART_INF_F, Ls = 0.f;
 #pragma unroll
-            for (int s = 0; s < 4; ++s) M = fmaxf(M, slice[(s * 2) * 128 + i]);
+            for (int s = 0; s < 4; ++s)
+                if (s >= s0 && s < s0 + n_sl) M = fmaxf(M, slice[(s * 2) * 128 + i]);
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const float m = slice[(s * 2) * 128 + i];
-                Ls += (m == -CUDART_INF_F) ? 0.f : slice[(s * 2 + 1) * 128 + i] * ex2_approx(m - M);
-            }
-            gm[i] = M;
-            ginv[i] = 1.0f / Ls;       // rows >= R are never used
+            for (int s = 0; s < 4; ++s)
+                if (s >= s0 && s < s0 + n_sl) {
+                    const float m = slice[(s * 2) * 128 + i];
+                    Ls += (m == -CUDART_INF_F) ? 0.f : slice[(s * 2 + 1) * 128 + i] * ex2_approx(m - M);
+                }
+            gm[threadIdx.x] = M;
+            ginv[threadIdx.x] = 1.0f / Ls;       // rows >= R are never used
         }
         __syncthreads();
         // chunk scores of this CTA's key range: partial sums x exp2(m_panel - m_i) / l_i, summed over
-        // the rows. A thread holds one row of up to 30 chunk slots at a time (PPB panels of its
+        // the rows. A thread holds one row of up to 32 chunk slots at a time (PPB panels of its
         // group: panels grp, grp + 4, ...); a transposing warp reduction leaves lane j with the sum
-        // over the warp's 32 rows of slot j; the four lane quarters are added through shared memory.
-        float* red = misc + 2304;      // [4 lane quarters][256 chunk slots of this CTA]
-        const int n_pl = 2 * nt;
+        // over the warp's 32 rows of slot j; the lane quarters (and query tiles) are added through
+        // shared memory (the K ring is idle now).
+        float* red = reinterpret_cast<float*>(ring);     // [query tiles x 4 lane quarters][chunk slots of this CTA]
+        const int n_local = nt * (TILE / C_STATIC);      // chunk slots of this CTA
+        const int n_pl = 2 * n_vt;
         if (warp >= 2) {
             const int grp = (warp - 2) >> 2, quarter = warp & 3;
-            const int row = quarter * 32 + lane;
-            const bool active = row < a.R;
+            const int row = quarter * 32 + lane, mt = two ? grp >> 1 : 0;
+            const bool active = mt * 128 + row < a.R;
             const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-            const float mi = gm[row], li = ginv[row];
-            constexpr int PPB = 30 / SPP;                // panels per block of 32 values (30 used)
+            const float mi = gm[mt * 128 + row], li = ginv[mt * 128 + row];
+            const uint64_t drop = l2_policy_evict_first();   // the sums in scratch are dead once read
+            constexpr int PPB = 32 / SPP;                // panels per block of up to 32 values
             for (int b0 = 0; grp + 4 * b0 < n_pl; b0 += PPB) {
-                float v[32];
+                float v[32], pm[PPB];
+                // (panel numbers clamped: every lane issues the same loads) A block that is on chip as a whole - every
+                // block of most shapes - takes its loads without a branch between them, so that they overlap.
+                if (!BIG || min(grp + 4 * (b0 + PPB - 1), n_pl - 1) < a.n_on) {
 #pragma unroll
-                for (int u = 0; u < PPB; ++u) {
-                    const int pl = min(grp + 4 * (b0 + u), n_pl - 1);   // clamped: every lane issues the same loads
-                    part_load<SPP>(lane_addr + static_cast<uint32_t>(kRPartCol0 + pl * SPP), &v[u * SPP]);
+                    for (int u = 0; u < PPB; ++u) {
+                        const int pl = min(grp + 4 * (b0 + u), n_pl - 1);
+                        part_load<SPP>(lane_addr + static_cast<uint32_t>(kRPartCol0 + pl * SPP), &v[u * SPP]);
+                        pm[u] = pmax[pl * 128 + row];
+                    }
+                } else {
+#pragma unroll
+                    for (int u = 0; u < PPB; ++u) {
+                        const int pl = min(grp + 4 * (b0 + u), n_pl - 1);
+                        if (pl < a.n_on) {
+                            part_load<SPP>(lane_addr + static_cast<uint32_t>(kRPartCol0 + pl * SPP), &v[u * SPP]);
+                            pm[u] = pmax[pl * 128 + row];
+                        } else {
+                            const float* sp = a.spill + (static_cast<size_t>(blockIdx.x) * a.n_off + (pl - a.n_on)) * ((SPP + 1) * 128) + row;
+                            pm[u] = ld_drop(sp, drop);
+#pragma unroll
+                            for (int q = 0; q < SPP; ++q) v[u * SPP + q] = ld_drop(sp + (q + 1) * 128, drop);
+                        }
+                    }
                 }
                 tmem_ld_wait();
-                v[30] = 0.f;
-                v[31] = 0.f;
+#pragma unroll
+                for (int e = PPB * SPP; e < 32; ++e) v[e] = 0.f;
 #pragma unroll
                 for (int u = 0; u < PPB; ++u) {
-                    const int pl = grp + 4 * (b0 + u);
-                    const bool have = active && pl < n_pl;
-                    const float f = have ? ex2_approx(pmax[min(pl, n_pl - 1) * 128 + row] - mi) * li : 0.f;
+                    const bool have = active && grp + 4 * (b0 + u) < n_pl;
+                    const float f = have ? ex2_approx(pm[u] - mi) * li : 0.f;
 #pragma unroll
                     for (int s = 0; s < SPP; ++s) v[u * SPP + s] = have ? v[u * SPP + s] * f : 0.f;
                 }
                 const float tot = warp_transpose_reduce(v, lane);
                 const int pl = grp + 4 * (b0 + lane / SPP);
-                if (lane < 30 && pl < n_pl) red[quarter * 256 + pl * SPP + lane % SPP] = tot;
+                if (lane < PPB * SPP && pl < n_pl) {
+                    const int kp = two ? (pl >> 2) * 2 + (pl & 1) : pl;      // panel of the key range
+                    red[(mt * 4 + quarter) * n_local + kp * SPP + lane % SPP] = tot;
+                }
             }
         }
         tc_fence_before();
         __syncthreads();
-        const int n_local = nt * (kRTile / C_STATIC);    // chunk slots of this CTA
-        const int ch0 = t_begin * (kRTile / C_STATIC);   // its first chunk
+        const int ch0 = t_begin * (TILE / C_STATIC);     // this CTA's first chunk
         for (int lc = threadIdx.x; lc < n_local; lc += kRThreads)
-            if (ch0 + lc < a.C)
-                a.scores[static_cast<size_t>(hs) * a.C + ch0 + lc] =
-                    (red[lc] + red[256 + lc]) + (red[512 + lc] + red[768 + lc]);
+            if (ch0 + lc < a.C) {
+                const float* r = red + lc;
+                float t = (r[0] + r[n_local]) + (r[2 * n_local] + r[3 * n_local]);
+                if (two) t += (r[4 * n_local] + r[5 * n_local]) + (r[6 * n_local] + r[7 * n_local]);
+                a.scores[static_cast<size_t>(hkv) * a.C + ch0 + lc] = t;
+            }
     }
     // ---- 4. wait for the KV head's other CTAs, 5. select, 6. gather
-    if (ok) ok = head_handover(a.cnt_b + hkv, static_cast<unsigned>(a.cph) << a.kv_shift, ctl);
-    if (ok) {
+    if (ok && a.out_idx != nullptr) ok = head_handover(a.cnt_b + hkv, static_cast<unsigned>(a.cph), ctl);
+    if (ok && a.out_idx != nullptr) {
         SelectSmem& ss = *reinterpret_cast<SelectSmem*>(ring);
         constexpr size_t kSelBytes = (sizeof(SelectSmem) + 127) & ~size_t(127);
         int32_t* sidx = reinterpret_cast<int32_t*>(ring + kSelBytes);          // [n_max] kept positions of the head
-        const float* sc = a.scores + (static_cast<size_t>(hkv) << a.kv_shift) * a.C;
-        const float* sc2 = a.kv_shift ? sc + a.C : nullptr;
+        const float* sc = a.scores + static_cast<size_t>(hkv) * a.C;
         if (a.C <= kRThreads * 6) {
-            select_head_regs<6>(sc, sc2, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, sidx, ss, a.tok_cap);
+            select_head_regs<6>(sc, nullptr, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, sidx, ss, a.tok_cap);
         } else {
             const size_t idx_bytes = (static_cast<size_t>(a.n_max) * 4 + 127) & ~size_t(127);
             uint32_t* kbuf = reinterpret_cast<uint32_t*>(ring + kSelBytes + idx_bytes);
             const bool fits = kSelBytes + idx_bytes + static_cast<size_t>(a.C) * 4 <= static_cast<size_t>(a.ring_bytes);
             if (fits)
-                select_head_smem(sc, sc2, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, sidx, ss, kbuf, a.tok_cap);
+                select_head_smem(sc, nullptr, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, sidx, ss, kbuf, a.tok_cap);
             else
-                select_head_rows(sc, sc2, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, sidx, ss, nullptr);
+                select_head_rows(sc, nullptr, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, sidx, ss, nullptr, a.tok_cap);
         }
-        const int Q = a.cph << a.kv_shift;               // CTAs of this KV head
-        const int q = static_cast<int>(blockIdx.x) - (hkv << a.kv_shift) * a.cph;
+        const int Q = a.cph, q = part;                   // CTAs of this KV head
         if (q == 0) {
             int32_t* dst = a.out_idx + static_cast<size_t>(hkv) * a.n_max;
             for (int n = threadIdx.x; n < a.n_max; n += kRThreads) dst[n] = sidx[n];
@@ -437,46 +515,63 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         // abandoned wait the counters are left as they are; chunkkv_device_status clears them.)
         const unsigned old = atomicAdd(a.exits, 1u);
         if (old + 1u == gridDim.x) {
-            for (int h = 0; h < a.Hs; ++h) a.cnt_a[h] = 0u;
-            for (int h = 0; h < a.Hkv; ++h) a.cnt_b[h] = 0u;
+            for (int h = 0; h < a.Hkv; ++h) { a.cnt_a[h] = 0u; a.cnt_b[h] = 0u; }
             *a.exits = 0u;
             __threadfence();
         }
     }
 }
 
-}  // namespace
-
-size_t resident_scratch_floats(const ResidentPlan& plan, int Hs, int C) {
-    return static_cast<size_t>(plan.grid) * 256 + ((static_cast<size_t>(Hs) * C + 63) & ~static_cast<size_t>(63));
+template <int C_STATIC>
+const void* kernel_of(bool big) {
+    return big ? reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, true>)
+               : reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, false>);
 }
 
-bool make_resident_plan(int L, int Rs, int Hs, int kv_shift, int d, int c, int C, int n_max, int max_ctas,
-                        int smem_limit, ResidentPlan* plan) {
-    if (c != 10 && c != 20) return false;
-    if (Rs < 1 || Rs > 128 || (d != 64 && d != 128) || L < 1 || C < 1 || Hs < 1 || Hs > kResidentMaxHeads) return false;
-    if (max_ctas < Hs) return false;
+}  // namespace
+
+size_t resident_scratch_floats(const ResidentPlan& plan, int Hkv, int C) {
+    return static_cast<size_t>(plan.grid) * plan.n_mt * 256 + ((static_cast<size_t>(Hkv) * C + 63) & ~static_cast<size_t>(63)) +
+           static_cast<size_t>(plan.grid) * plan.n_off * (plan.spp + 1) * 128;
+}
+
+bool make_resident_plan(int L, int R, int Hkv, int d, int c, int C, int n_max, int max_ctas, int smem_limit,
+                        ResidentPlan* plan) {
+    // chunk sizes that divide a panel of 60 or 64 keys and leave at least two chunks in it; the others (and token
+    // level, where a partial sum per chunk would be the score matrix itself) take other kernels
+    if (c != 5 && c != 8 && c != 10 && c != 16 && c != 20 && c != 32) return false;
+    if (R < 1 || R > 256 || (d != 64 && d != 128) || L < 1 || C < 1 || Hkv < 1 || Hkv > kResidentMaxHeads) return false;
+    if (max_ctas < Hkv) return false;
     ResidentPlan p{};
     p.c_static = c;
-    p.cph = max_ctas / Hs;
-    p.grid = p.cph * Hs;
-    p.n_tiles = (L + kRTile - 1) / kRTile;
+    p.n_mt = R > 128 ? 2 : 1;
+    const int tile = 2 * panel_keys(c);
+    p.spp = panel_keys(c) / c;
+    p.tile = tile;
+    p.n_tiles = (L + tile - 1) / tile;
+    p.cph = max_ctas / Hkv;
+    if (p.cph > p.n_tiles) p.cph = p.n_tiles;                       // a CTA without keys would only lengthen the hand-overs
+    p.grid = p.cph * Hkv;
     p.t_max = (p.n_tiles + p.cph - 1) / p.cph;
-    if (p.t_max * (kRTile / c) > kRPartCols) return false;          // the chunk partial sums must fit tensor memory
-    const int KB = d / 64;
-    const int q_bytes = KB * kRQTileBytes;
-    const int pmax_bytes = p.t_max * 2 * 128 * 4;
+    const int n_pl = 2 * p.n_mt * p.t_max;                          // panels of a CTA
+    p.n_on = kRPartCols / p.spp;
+    if (p.n_on > n_pl) p.n_on = n_pl;
+    p.n_off = n_pl - p.n_on;
+    const int KB = d / 64, stage = tile * 128;
+    const int q_bytes = p.n_mt * KB * kRQTileBytes;
+    const int pmax_bytes = p.n_on * 128 * 4;
     const int fixed = 1024 /* alignment */ + q_bytes + 1024 /* tail of the last stage's UMMA read */ + pmax_bytes + kRMiscBytes;
-    int ns = (smem_limit - fixed) / kRStageBytes;
+    int ns = (smem_limit - fixed) / stage;
     if (ns > kRMaxStages) ns = kRMaxStages;
     if (ns < 2 * KB) return false;
     p.n_stages = ns;
     p.off_ring = q_bytes;
-    p.ring_bytes = ns * kRStageBytes + 1024;
+    p.ring_bytes = ns * stage + 1024;
     p.off_pmax = p.off_ring + p.ring_bytes;
     p.off_misc = p.off_pmax + pmax_bytes;
     p.smem_bytes = 1024 + p.off_misc + kRMiscBytes;
-    // after scoring the ring holds the selection scratch and the kept positions
+    // after scoring the ring holds the row sums of the chunk scores, then the selection scratch and the kept positions
+    if (static_cast<size_t>(p.n_mt) * 4 * p.t_max * (tile / c) * 4 > static_cast<size_t>(p.ring_bytes)) return false;
     const size_t sel_bytes = ((sizeof(SelectSmem) + 127) & ~size_t(127)) + ((static_cast<size_t>(n_max) * 4 + 127) & ~size_t(127));
     if (sel_bytes > static_cast<size_t>(p.ring_bytes)) return false;
     *plan = p;
@@ -486,12 +581,13 @@ bool make_resident_plan(int L, int Rs, int Hs, int kv_shift, int d, int c, int C
 cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                                   const ResidentIO& io, cudaStream_t stream) {
     ResArgs a{};
-    a.L = io.L; a.P = io.L - io.w; a.w = io.w; a.R = io.Rs; a.Hs = io.Hs; a.d = io.d; a.kv_shift = io.kv_shift;
+    a.L = io.L; a.P = io.L - io.w; a.w = io.w; a.R = io.R; a.d = io.d; a.n_mt = plan.n_mt;
     a.sl2 = io.sl2;
     a.cph = plan.cph; a.n_tiles = plan.n_tiles; a.n_stages = plan.n_stages;
-    a.q_box_rows = io.Rs < 128 ? io.Rs : 128;
-    a.k_box_rows = io.L < kRTile ? io.L : kRTile;
-    a.C = io.C; a.k = io.k; a.n_max = io.n_max; a.Hkv = io.Hs >> io.kv_shift;
+    a.q_box_rows = io.R < 128 ? io.R : 128;
+    a.k_box_rows = io.L < plan.tile ? io.L : plan.tile;
+    a.C = io.C; a.k = io.k; a.n_max = io.n_max; a.Hkv = io.Hkv;
+    a.n_on = plan.n_on; a.n_off = plan.n_off;
     a.off_ring = plan.off_ring; a.ring_bytes = plan.ring_bytes; a.off_pmax = plan.off_pmax; a.off_misc = plan.off_misc;
     a.K = static_cast<const uint4*>(io.K); a.V = static_cast<const uint4*>(io.V);
     a.block_table = io.block_table; a.page_size = io.page_size; a.num_pages = io.num_pages;
@@ -505,18 +601,30 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     }
     a.out_K = static_cast<uint4*>(io.out_K); a.out_V = static_cast<uint4*>(io.out_V); a.out_idx = io.out_idx;
     a.cta_stat = io.scratch;
-    a.scores = io.scratch + static_cast<size_t>(plan.grid) * 256;
+    float* scores = io.scratch + static_cast<size_t>(plan.grid) * plan.n_mt * 256;
+    a.scores = io.out_scores ? io.out_scores : scores;
+    a.spill = scores + ((static_cast<size_t>(io.Hkv) * io.C + 63) & ~static_cast<size_t>(63));
     a.exits = io.counters;
     a.cnt_a = io.counters + 16;
     a.cnt_b = io.counters + 16 + kResidentMaxHeads;
     a.status = io.status;
-    const void* kern = plan.c_static == 10 ? reinterpret_cast<const void*>(layer_resident_kernel<10>)
-                                           : reinterpret_cast<const void*>(layer_resident_kernel<20>);
-    static int smem_set[2][64] = {{0}};
+    const bool big = plan.n_mt == 2 || plan.n_off > 0;
+    const void* kern = nullptr;
+    int v = 0;
+    switch (plan.c_static) {
+        case 5: kern = kernel_of<5>(big); v = 0; break;
+        case 8: kern = kernel_of<8>(big); v = 1; break;
+        case 10: kern = kernel_of<10>(big); v = 2; break;
+        case 16: kern = kernel_of<16>(big); v = 3; break;
+        case 20: kern = kernel_of<20>(big); v = 4; break;
+        case 32: kern = kernel_of<32>(big); v = 5; break;
+        default: return cudaErrorInvalidValue;
+    }
+    v += big ? 6 : 0;
+    static int smem_set[12][64] = {{0}};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    const int v = plan.c_static == 10 ? 0 : 1;
     if (dev < 0 || dev >= 64 || smem_set[v][dev] < plan.smem_bytes) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
         if (e != cudaSuccess) return e;

@@ -1,0 +1,62 @@
+"""The one-launch layer kernel over its whole range: every chunk size it is built for, one and two query tiles,
+key ranges whose partial sums do not fit on chip, last tiles and chunks of any length, strided inputs, paged outputs.
+Tolerances as in test_gpu_parity.py."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import chunkkv_oracle as ora
+from tests.helpers import (assert_gather_exact, assert_scores_close, assert_selection_matches, bits_of, guarded_outputs,
+                           to_dev)
+from workloads import CONFIGS, make_layer, scaled
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ck():
+    import paper_2502_00299_b200 as ck
+    assert torch.cuda.is_available()
+    return ck
+
+
+def _layer(Hq, Hkv, d, L, w, c, budget, seed=0):
+    wl = scaled(CONFIGS[1], Hq=Hq, Hkv=Hkv, d=d, L=L, w=w, c=c, budget=budget, seed=900 + seed, planted_count=2,
+                sink_tokens=1)
+    return wl, make_layer(wl)
+
+
+# a CTA takes ceil(ceil(L / tile) / (148 / Hkv)) key tiles (tile = 120 keys, 128 for c = 8, 16, 32); partial sums beyond
+# 256 / (chunks per half tile) panels go to scratch
+CASES = [
+    (8, 2, 64, 2048, 16, 5), (8, 2, 64, 121, 16, 8), (8, 2, 64, 129, 16, 16), (4, 4, 128, 33, 32, 32), (2, 1, 128, 20, 16, 5),
+    (28, 4, 128, 3000, 32, 10), (28, 4, 128, 1500, 16, 32),          # 224 rows: tiles of 128 and 96; 112 rows
+    (15, 3, 64, 1203, 43, 20), (64, 8, 128, 2047, 32, 16),           # 215 rows (odd); 256 rows
+    (64, 16, 64, 9 * 120 * 11 + 7, 16, 5),                           # 64 rows, 22 panels of which 21 fit
+    (64, 16, 64, 9 * 120 * 22, 16, 10), (32, 32, 64, 4 * 128 * 17 + 1, 8, 8), (32, 32, 64, 4 * 128 * 33 - 3, 8, 16),
+    (128, 32, 64, 4 * 120 * 23 + 61, 64, 20), (64, 32, 128, 4 * 128 * 33 + 65, 128, 32),     # 256 rows, in scratch from panel 86 / 129
+]
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,L,w,c", CASES)
+def test_layer_and_chunk_scores(ck, Hq, Hkv, d, L, w, c):
+    budget = w + c * max(1, (L - w) // (4 * c)) + 1
+    wl, x = _layer(Hq, Hkv, d, L, w, c, budget, seed=L)
+    q, K, V = to_dev(x.q_obs), to_dev(x.K), to_dev(x.V)
+    t = ora.token_scores(x.q_obs, x.K, Hq, Hkv, w)
+    s = ora.chunk_scores(t, c)
+    cs, _ = ck.score(q, K, w, c)
+    assert_scores_close(cs.cpu().numpy(), s, w * Hq // Hkv, L, "chunk scores")
+    gK, gV, gI = guarded_outputs(Hkv, ck.out_len(L, w, c, budget), d)
+    oK, oV, idx = ck.compress_layer(q, K, V, Hq, w, c, budget, out_K=gK.t, out_V=gV.t, out_idx=gI.t)
+    assert ck.device_status() == 0
+    for g in (gK, gV, gI):
+        g.check()
+    idx = idx.cpu().numpy()
+    assert_selection_matches(idx, s, L, w, c, budget)
+    assert_gather_exact(bits_of(oK), bits_of(oV), idx, x.K, x.V)
+    # token-major inputs: same scores and so the same selection and rows
+    Kt, Vt = (a.permute(1, 0, 2).contiguous().permute(1, 0, 2) for a in (K, V))
+    sK, sV, sidx = ck.compress_layer_strided(q, Kt, Vt, Hq, w, c, budget)
+    assert np.array_equal(sidx.cpu().numpy(), idx) and torch.equal(sK, oK) and torch.equal(sV, oV)
+
