@@ -845,6 +845,13 @@ static int model_args_ok(int n_layers, int reuse_depth) {
     return CHUNKKV_OK;
 }
 
+// Most computed layers that one launch of the persistent kernel takes.
+static int model_launch_computes(int n_layers, int reuse_depth) {
+    const int per_launch = n_layers < kModelMaxLayers ? n_layers : kModelMaxLayers;
+    const int n = (per_launch + reuse_depth - 1) / reuse_depth + 1;
+    return n < kModelMaxCompute ? n : kModelMaxCompute;
+}
+
 size_t chunkkv_model_workspace_bytes(int n_layers, int L, int Hq, int Hkv, int d, int w, int c, int budget,
                                      int reuse_depth) {
     if (model_args_ok(n_layers, reuse_depth) != CHUNKKV_OK || check_sizes(L, w, c, budget) != CHUNKKV_OK) return 0;
@@ -853,15 +860,12 @@ size_t chunkkv_model_workspace_bytes(int n_layers, int L, int Hq, int Hkv, int d
     std::lock_guard<std::mutex> lk(g_mu);
     DeviceCtx* ctx;
     if (get_ctx(&ctx) != CHUNKKV_OK) return 0;
-    const ScoreShape sh = score_shape(Hq, Hkv, w);
     const int C = (L - w + c - 1) / c;
     const int k = chunkkv_num_kept_chunks(L, w, c, budget);
     ModelPlan mp;
     size_t need = per_layer;
-    if (C > 0 && k > 0 && make_model_plan(L, sh.Rs, sh.Hs, sh.shift, d, c, C, k, ctx->num_sms, smem_budget(*ctx), &mp)) {
-        const int per_launch = n_layers < kModelMaxLayers ? n_layers : kModelMaxLayers;
-        const int n_compute = (per_launch + reuse_depth - 1) / reuse_depth + 1;
-        const size_t m = kHeaderBytes + model_scratch_floats(mp, sh.Hs, sh.shift, C, n_compute) * sizeof(float);
+    if (C > 0 && k > 0 && make_model_plan(L, w * (Hq / Hkv), Hkv, d, c, C, k, ctx->num_sms, smem_budget(*ctx), &mp)) {
+        const size_t m = kHeaderBytes + model_scratch_floats(mp, Hkv, C, model_launch_computes(n_layers, reuse_depth)) * sizeof(float);
         need = m > need ? m : need;
     }
     return need;
@@ -900,15 +904,18 @@ static int compress_model_impl(int n_layers, const void* const* q_obs, const voi
     ModelPlan mp;
     bool persistent = false;
     DeviceCtx* ctx = nullptr;
-    ScoreShape sh = score_shape(Hq, Hkv, w);
+    const int R = w * (Hq / Hkv);
     {
         std::lock_guard<std::mutex> lk(g_mu);
         st = get_ctx(&ctx);
         if (st != CHUNKKV_OK) return st;
         // paged outputs run layer by layer: the one-launch layer kernel places rows through the block table with all
         // its threads, which measured faster (35 us per layer) than the persistent kernel's copy warp doing it (41 us)
+        // (a scratch set up for the layer calls only is used by the layer calls)
         persistent = !paged && C > 0 && k > 0 &&
-                     make_model_plan(L, sh.Rs, sh.Hs, sh.shift, d, c, C, k, ctx->num_sms, smem_budget(*ctx), &mp);
+                     make_model_plan(L, R, Hkv, d, c, C, k, ctx->num_sms, smem_budget(*ctx), &mp) &&
+                     ensure_workspace(*ctx, model_scratch_floats(mp, Hkv, C, model_launch_computes(n_layers, reuse_depth)) *
+                                                sizeof(float)) == CHUNKKV_OK;
     }
     if (!persistent) {
         // layer by layer: Algorithm 2's call sequence over chunkkv_compress_layer
@@ -938,7 +945,7 @@ static int compress_model_impl(int n_layers, const void* const* q_obs, const voi
         int n_compute = 0;
         while (l1 < n_layers) {
             const int group_end = (l1 + reuse_depth < n_layers) ? l1 + reuse_depth : n_layers;
-            if (group_end - l0 > kModelMaxLayers && l1 > l0) break;
+            if ((group_end - l0 > kModelMaxLayers || n_compute == kModelMaxCompute) && l1 > l0) break;
             if (group_end - l0 > kModelMaxLayers) {         // a single reuse group longer than a launch: split it
                 l1 = l0 + kModelMaxLayers;
                 if (n_compute == 0) n_compute = 1;
@@ -948,7 +955,7 @@ static int compress_model_impl(int n_layers, const void* const* q_obs, const voi
             ++n_compute;
         }
         const int n = l1 - l0;
-        const size_t need = model_scratch_floats(mp, sh.Hs, sh.shift, C, n_compute) * sizeof(float);
+        const size_t need = model_scratch_floats(mp, Hkv, C, n_compute) * sizeof(float);
         st = ensure_workspace(*ctx, need);
         if (st != CHUNKKV_OK) return st;
         char* base = static_cast<char*>(ctx->ws);
@@ -959,10 +966,9 @@ static int compress_model_impl(int n_layers, const void* const* q_obs, const voi
             lay[i].K = K[l]; lay[i].V = V[l]; lay[i].out_K = out_K[l]; lay[i].out_V = out_V[l]; lay[i].out_idx = out_idx[l];
             lay[i].computes = computes;
             if (computes) {
-                st = encode_bf16_3d(&tm_q[nc], q_obs[l], d, sh.Rs, sh.Hs, sh.Rs < 128 ? sh.Rs : 128,
-                                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+                st = encode_bf16_3d(&tm_q[nc], q_obs[l], d, R, Hkv, R < 128 ? R : 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
                 if (st != CHUNKKV_OK) return st;
-                st = encode_bf16_3d(&tm_k[nc], K[l], d, L, Hkv, L < 120 ? L : 120, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, kt, kh);
+                st = encode_bf16_3d(&tm_k[nc], K[l], d, L, Hkv, L < mp.tile ? L : mp.tile, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, kt, kh);
                 if (st != CHUNKKV_OK) return st;
                 ++nc;
             }
@@ -990,7 +996,7 @@ static int compress_model_impl(int n_layers, const void* const* q_obs, const voi
             continue;
         }
         ModelIO io;
-        io.L = L; io.w = w; io.Rs = sh.Rs; io.Hs = sh.Hs; io.d = d; io.kv_shift = sh.shift;
+        io.L = L; io.w = w; io.R = R; io.Hkv = Hkv; io.d = d;
         io.sl2 = static_cast<float>(1.4426950408889634 / sqrt(static_cast<double>(d)));
         io.C = C; io.k = k; io.n_max = n_max;
         io.scratch = reinterpret_cast<float*>(base + kHeaderBytes);

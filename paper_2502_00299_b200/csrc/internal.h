@@ -126,18 +126,21 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
 
 // The persistent kernel that runs many layers per launch (model_kernel.cu). Same tiling as the
 // layer kernel above, plus two tail warps per CTA that select and copy rows behind the scoring.
-constexpr int kModelMaxLayers = 32;     // layers per launch (computed + reusing)
+constexpr int kModelMaxLayers = 96;     // layers per launch (computed + reusing)
 constexpr int kModelMaxCompute = 32;    // computed layers per launch
 
 struct ModelPlan {
-    int c_static, grid, cph, n_tiles, t_max, n_stages, smem_bytes;
+    int c_static, n_mt, grid, cph, tile, n_tiles, t_max, spp, n_stages, smem_bytes;
+    bool big;                    // two query tiles or a ring of partial sums that continues in scratch
+    int ring_on, ring;           // panels of the ring on chip, in all
+    int copy_slots;
     int n_score, n_sel;          // scoring CTAs, selector CTAs (grid = n_score + n_sel)
     int sel_row_bytes, sel_keys_fit;
     int off_ring, off_pmax, off_misc, off_tail, stage_slot_bytes;
 };
 
 struct ModelIO {
-    int L, w, Rs, Hs, d, kv_shift;
+    int L, w, R, Hkv, d;         // R query rows per KV head
     float sl2;
     int C, k, n_max;
     float* scratch;       // model_scratch_floats() floats
@@ -156,9 +159,8 @@ struct ModelLayerIO {
     bool computes;        // false: gather with the indices of the nearest computed layer before it
 };
 
-bool make_model_plan(int L, int Rs, int Hs, int kv_shift, int d, int c, int C, int k, int max_ctas, int smem_limit,
-                     ModelPlan* plan);
-size_t model_scratch_floats(const ModelPlan& plan, int Hs, int kv_shift, int C, int n_compute);
+bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, ModelPlan* plan);
+size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute);
 // layers[0] must compute; tm_q / tm_k hold one tensor map per computed layer, in order.
 cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtensorMap* tm_q, const CUtensorMap* tm_k,
                          const ModelLayerIO* layers, int n_layers, cudaStream_t stream);

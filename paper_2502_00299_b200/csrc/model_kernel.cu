@@ -2,12 +2,17 @@
 // computed layer): a persistent version of the layer kernel of layer_resident.cu in which the
 // steps of successive layers overlap inside every CTA.
 //
-// A CTA belongs to one scoring head and one key range for the whole launch. Its warps have roles:
+// A CTA belongs to one KV head and one key range for the whole launch. A KV head with more than 128
+// query rows has two query tiles: each key tile is loaded once and multiplied with both. The CTA's
+// (key tile, query tile) products are "virtual tiles" in issue order; its panels (half a virtual
+// tile each) are numbered through the launch, and a panel's accumulator, epilogue group and ring slot
+// all follow from that number. Its warps have roles:
 //   warp 0         TMA producer: streams the Q tile and the CTA's K tiles of layer after layer
 //                  through the shared-memory ring, as far ahead as the ring allows
 //   warp 1         tcgen05.mma issuer
 //   warps 2..17    epilogue, four groups of four warps: one exponential per score element, chunk sums
-//                  into a ring of tensor-memory columns that holds more than one layer; at the end
+//                  into a ring of tensor-memory columns that holds more than one layer (the part of
+//                  the ring that does not fit there lies in scratch: long contexts, small chunks); at the end
 //                  of a layer a group leaves its per-row (max, sum) in shared memory and goes straight
 //                  on with the next layer; when the head's row statistics have arrived (normally long
 //                  before they are needed) it contracts the partial sums it wrote itself over the rows
@@ -39,31 +44,45 @@ namespace {
 
 constexpr int kMThreads = 640;          // warp 0: TMA, warp 1: UMMA issue, warps 2..17: epilogue, warp 18: row copies, warp 19: row statistics
                                         // (five warps per scheduler: a sixth would cut every thread to 80 registers)
-constexpr int kMMiscBytes = 18432;      // epilogue: group records (two slots), m_i, 1 / l_i, row sums per lane quarter
-constexpr int kMSlots = 8;              // staging slots of the row copies
-// Tensor memory: three 64-column accumulators (one 60-key panel of a tile each, in rotation; the
+constexpr int kMMiscBytes = 16384;      // epilogue: group records (two slots), m_i, 1 / l_i, row sums per lane quarter
+constexpr int kMSlots = 8;              // most staging slots of the row copies
+constexpr int kMSegSlots = 64;          // chunk slots a group contracts between two barriers
+// Tensor memory, small variant: three 64-column accumulators (one 60-key panel of a tile each, in rotation; the
 // second panel of a tile is computed on keys 56 .. 119 so that its operand starts on a swizzle-atom
 // boundary, and begins at column 4), and 320 columns of chunk partial sums: a ring that holds one
 // layer and two thirds of the next at c = 10, so the statistics of a layer have most of the next
 // layer's scoring time to travel before its contraction needs them.
+// Big variant: two 128-column accumulators (a whole virtual tile each, one per pair of epilogue groups) and 256
+// columns of the ring, which continues in scratch. Half as many products to issue, each at the tensor pipe's rate
+// (an N = 64 product takes 48 clocks, an N = 128 one 64: the query tile is read from shared memory for each), which
+// two query tiles need: with three 64-column accumulators a 256-row layer spent 45 % of its time waiting for products.
 constexpr int kMAccN = 64;
 constexpr int kMAccBufs = 3;
 constexpr int kMAccSlots = 12;                     // (buffer, epilogue group) pairs: lcm(3 buffers, 4 groups)
 constexpr int kMAcc1Row = 56;
-constexpr int kMPartCol0 = kMAccBufs * kMAccN;
-constexpr int kMPartCols = 512 - kMPartCol0;
+__host__ __device__ constexpr int model_part_col0(bool big) { return big ? 2 * kRUmmaN : kMAccBufs * kMAccN; }
 // Ring sizes are multiples of the four epilogue groups: a panel's ring slot is its number (since the
 // start of the launch) modulo the ring size and its group is that number modulo 4, so a ring slot
-// is only ever reused by the group that wrote and contracted its previous contents.
-constexpr int kMRingPanels10 = kMPartCols / 6 / 4 * 4;   // c = 10: 6 chunk columns per panel
-constexpr int kMRingPanels20 = 84;                       // c = 20: 3 per panel; more would only cost shared memory
-static_assert(kMRingPanels10 % 4 == 0 && kMRingPanels20 % 4 == 0 && kMRingPanels20 * 3 <= kMPartCols, "ring sizes");
+// is only ever reused by the group that wrote and contracted its previous contents. Panels held on chip:
+// the small variant keeps panel maxima in shared memory (a row set per panel: at most 84 panels, fewer where
+// more would only cost ring stages), the big one beside the sums in tensor memory.
+__host__ __device__ constexpr int model_ring_panels(int c, bool big) {
+    const int spp = panel_keys(c) / c;
+    const int fit = (512 - model_part_col0(big)) / (big ? spp + 1 : spp) / 4 * 4;
+    return big ? fit : (c >= 32 ? 64 : (c == 16 ? 72 : (fit > 84 ? 84 : fit)));
+}
+// Staging slots of the row copies: as many as fit about 40 KB (a slot holds a chunk's K and V rows)
+__host__ __device__ constexpr int model_copy_slots(int c, int d) {
+    const int n = 40960 / (4 * c * d);
+    return n > kMSlots ? kMSlots : (n < 3 ? 3 : n);
+}
 constexpr int kBarGroup = 2;                       // named barriers 2 .. 5: the four warps of an epilogue group
 
 struct ModelCtl {
     unsigned long long full[kRMaxStages];
     unsigned long long empty[kRMaxStages];
     unsigned long long tfull[kMAccSlots];      // by panel number modulo 12: one (accumulator, epilogue group) pair each
+                                               // (big variant: the first two, one per accumulator)
     unsigned long long tempty[kMAccSlots];
     unsigned long long qfull;
     unsigned long long qempty;
@@ -92,21 +111,25 @@ struct ModelParams {
     CUtensorMap tm_k[kModelMaxCompute];
     ModelLayer layer[kModelMaxLayers];
     int n_layers, n_compute;
-    int L, P, w, R, Hs, d, kv_shift;
+    int L, P, w, R, d;
+    int n_mt;              // 128-row query tiles per KV head (1 or 2)
     float sl2;
     int cph, n_tiles, n_stages, q_box_rows, k_box_rows;
     int C, k, n_max, Hkv;
     int Cpad;              // row stride of the chunk scores (C rounded up to a multiple of 4: rows stay 16-byte aligned)
-    int n_score, n_sel;    // scoring CTAs (Hs * cph) and selector CTAs (the rest of the grid)
+    int n_score, n_sel;    // scoring CTAs (Hkv * cph) and selector CTAs (the rest of the grid)
+    int ring_on, ring;     // big variant: panels of the ring in tensor memory, panels of the ring in all
+    int copy_slots;
     int sel_row_bytes;     // bytes of one kept-chunk list: 4 header ints + the kept chunk ids, padded to 16 bytes
     int sel_keys_fit;      // selector: the keys of a head fit its shared memory (many chunks per thread)
     int off_ring, off_pmax, off_misc, off_tail, stage_slot_bytes;
     // bytes between consecutive rows of a head and between heads of K and of V (packed: d * 2 and L * d * 2)
     long long k_row_bytes, k_head_bytes, v_row_bytes, v_head_bytes;
-    float* cta_stat;       // [2 (slot parity)][grid][{max, sum}][128]
-    float* scores;         // [n_compute][Hs][Cpad]
-    unsigned* cnt_a;       // [Hs]
-    unsigned* cnt_b;       // [Hs]   chunk scores of a slot announced by the scoring CTAs
+    float* cta_stat;       // [2 (slot parity)][grid][n_mt][{max, sum}][128]
+    float* scores;         // [n_compute][Hkv][n_mt][Cpad]
+    float* spill;          // [scoring CTA][ring - ring_on][1 + chunk slots per panel][128]: panel maximum, chunk sums
+    unsigned* cnt_a;       // [Hkv]
+    unsigned* cnt_b;       // [Hkv]  chunk scores of a slot announced by the scoring CTAs
     unsigned* cnt_c;       // [Hkv]  kept-chunk lists announced by the selector CTAs
     int* sel_rows;         // [n_compute][Hkv][sel_row_bytes / 4]
     unsigned* exits;
@@ -217,19 +240,17 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
         for (int hkv = sid; hkv < p.Hkv; hkv += p.n_sel) {
             if (threadIdx.x == 0) {
                 const unsigned target = static_cast<unsigned>(s + 1) * p.cph;
-                bool w_ok = wait_counter(p.cnt_b + (hkv << p.kv_shift), target, flag + 1, 100);
-                if (w_ok && p.kv_shift) w_ok = wait_counter(p.cnt_b + (hkv << p.kv_shift) + 1, target, flag + 1, 100);
+                const bool w_ok = wait_counter(p.cnt_b + hkv, target, flag + 1, 100);
                 asm volatile("fence.acq_rel.gpu;" ::: "memory");
                 flag[0] = w_ok ? 1 : 0;
             }
             __syncthreads();
             if (!flag[0]) return false;
-            const float* sc = p.scores + (static_cast<size_t>(s) * p.Hs + (hkv << p.kv_shift)) * p.Cpad;
-            const float* sc2 = p.kv_shift ? sc + p.Cpad : nullptr;
+            const float* sc = p.scores + (static_cast<size_t>(s) * p.Hkv + hkv) * p.n_mt * p.Cpad;
+            const float* sc2 = p.n_mt == 2 ? sc + p.Cpad : nullptr;
             if (p.C <= kMThreads * 8)
                 select_head_regs<8>(sc, sc2, p.L, p.w, C_STATIC, p.C, p.k, p.n_max, sidx, ss);
-            else
-{
+            else {
                 if (p.sel_keys_fit)
                     select_head_smem(sc, sc2, p.L, p.w, C_STATIC, p.C, p.k, p.n_max, sidx, ss, kbuf);
                 else
@@ -262,12 +283,19 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
 }
 
 // STRIDED: the rows of a head are not adjacent in memory (e.g. token-major caches): the copy thread moves
-// kept rows one at a time. A variant of its own, so that the packed kernel's code is exactly what it was.
-template <int C_STATIC, bool STRIDED>
+// kept rows one at a time. BIG: two query tiles, or a ring that reaches into scratch. Variants of their own, so that
+// the kernel for packed caches and up to 128 rows is exactly what it was.
+template <int C_STATIC, bool STRIDED, bool BIG>
 __global__ void __launch_bounds__(kMThreads, 1)
 model_kernel(const __grid_constant__ ModelParams p) {
-    constexpr int SPP = kRPanel / C_STATIC;
-    constexpr uint32_t IDESC = umma_idesc_bf16(128, kMAccN);
+    constexpr int WP = panel_keys(C_STATIC);
+    constexpr int TILE = 2 * WP;
+    constexpr uint32_t STAGE = TILE * 128;
+    constexpr int SPP = WP / C_STATIC;
+    constexpr int ACC1 = WP == 64 ? 64 : kMAcc1Row;       // first key of a tile's second product (a swizzle-atom boundary)
+    constexpr int COL1 = WP - ACC1;                       // accumulator column its panel begins at
+    constexpr int PART0 = model_part_col0(BIG);
+    constexpr uint32_t IDESC = umma_idesc_bf16(128, BIG ? kRUmmaN : kMAccN);
 
     extern __shared__ uint8_t smem_raw[];
     __shared__ ModelCtl ctl;
@@ -280,9 +308,9 @@ model_kernel(const __grid_constant__ ModelParams p) {
     const uint32_t k_base = smem_base + static_cast<uint32_t>(p.off_ring);
     float* pmax = reinterpret_cast<float*>(dyn + p.off_pmax);
     float* misc = reinterpret_cast<float*>(dyn + p.off_misc);
-    float* rec = misc;                 // [4 groups][{max, sum}][128]; the odd slots' copy sits at misc + 3584
-    float* gstat = misc + 1024;        // [2 (slot parity)][{m_i, 1 / l_i}][128]
-    float* red = misc + 2304;          // [4 lane quarters][256 chunk slots]
+    float* rec = misc;                 // [4 groups][{max, sum}][128]; the odd slots' copy sits at misc + 3072
+    float* gstat = misc + 1024;        // [2 (slot parity)][2 query tiles][{m_i, 1 / l_i}][128]
+    float* red = misc + 2048;          // [4 groups][4 lane quarters][kMSegSlots]
     volatile int* abort_flag = &ctl.abort_flag;
     const uint32_t n_stages = static_cast<uint32_t>(p.n_stages);
 
@@ -298,20 +326,21 @@ model_kernel(const __grid_constant__ ModelParams p) {
             if (!s_ok) atomicExch(p.status, 1);
             const unsigned old = atomicAdd(p.exits, 1u);
             if (old + 1u == gridDim.x) {
-                for (int h = 0; h < p.Hs; ++h) { p.cnt_a[h] = 0u; p.cnt_b[h] = 0u; }
-                for (int h = 0; h < p.Hkv; ++h) p.cnt_c[h] = 0u;
+                for (int h = 0; h < p.Hkv; ++h) { p.cnt_a[h] = 0u; p.cnt_b[h] = 0u; p.cnt_c[h] = 0u; }
                 *p.exits = 0u;
                 __threadfence();
             }
         }
         return;
     }
-    const int hs = blockIdx.x / p.cph, part = blockIdx.x - hs * p.cph;
-    const int hkv = hs >> p.kv_shift;
+    const int hkv = blockIdx.x / p.cph, part = blockIdx.x - hkv * p.cph;
     // tiles are dealt out rounding up, so the head's last CTA - whose last panels take the slow, masked path -
     // is never one of those that get an extra tile
     const int t_begin = (p.n_tiles * part + p.cph - 1) / p.cph, t_end = (p.n_tiles * (part + 1) + p.cph - 1) / p.cph;
     const int nt = t_end - t_begin;
+    const int n_mt = BIG ? p.n_mt : 1;
+    const bool two = n_mt == 2;
+    const int n_vt = two ? 2 * nt : nt;              // virtual tiles of this CTA per layer
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.n_stages; ++s) {
@@ -320,7 +349,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
         }
         for (int b = 0; b < kMAccSlots; ++b) {
             mbar_init(smem_u32(&ctl.tfull[b]), 1);
-            mbar_init(smem_u32(&ctl.tempty[b]), 4);
+            mbar_init(smem_u32(&ctl.tempty[b]), BIG ? 8 : 4);      // one arrival per reading warp
         }
         mbar_init(smem_u32(&ctl.qfull), 1);
         mbar_init(smem_u32(&ctl.qempty), 1);
@@ -351,7 +380,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
         // ------------------------------------------------------------------ TMA producer
         if (elect_one() && nt > 0) {
             const uint32_t qbar = smem_u32(&ctl.qfull);
-            const uint32_t q_bytes = static_cast<uint32_t>(KB * p.q_box_rows) * 128u;
+            const uint32_t q_bytes = static_cast<uint32_t>(n_mt * KB * p.q_box_rows) * 128u;
             const uint32_t k_bytes = static_cast<uint32_t>(p.k_box_rows) * 128u;
             uint32_t st = 0, st_par = 1;
             int issued = 0;
@@ -363,15 +392,16 @@ model_kernel(const __grid_constant__ ModelParams p) {
                 if (s > 0) ok = mbar_wait(smem_u32(&ctl.qempty), (s - 1) & 1, abort_flag);
                 if (!ok) break;
                 mbar_arrive_expect_tx(qbar, q_bytes);
-                for (int kb = 0; kb < KB; ++kb)
-                    tma_load_3d(q_base + static_cast<uint32_t>(kb) * kRQTileBytes, &p.tm_q[s], qbar, kb * 64, 0, hs);
+                for (int mt = 0; mt < n_mt; ++mt)    // (rows past R of the second tile arrive as zeros)
+                    for (int kb = 0; kb < KB; ++kb)
+                        tma_load_3d(q_base + static_cast<uint32_t>(mt * KB + kb) * kRQTileBytes, &p.tm_q[s], qbar, kb * 64, mt * 128, hkv);
                 for (int t = t_begin; t < t_end && ok; ++t) {
                     for (int kb = 0; kb < KB; ++kb) {
                         ok = mbar_wait(smem_u32(&ctl.empty[st]), st_par, abort_flag);
                         if (!ok) break;
                         const uint32_t bar = smem_u32(&ctl.full[st]);
                         mbar_arrive_expect_tx(bar, k_bytes);
-                        tma_load_3d(k_base + st * kRStageBytes, &p.tm_k[s], bar, kb * 64, t * kRTile, hkv);
+                        tma_load_3d(k_base + st * STAGE, &p.tm_k[s], bar, kb * 64, t * TILE, hkv);
                         ++issued;
                         if (++st == n_stages) { st = 0; st_par ^= 1u; }
                     }
@@ -392,11 +422,12 @@ model_kernel(const __grid_constant__ ModelParams p) {
         // ------------------------------------------------------------------ UMMA issuer
         if (elect_one() && nt > 0) {
             uint32_t st = 0, st_par = 0;
-            int tg = 0;                  // tiles issued so far (all layers); the epilogue pair tg & 1 reads tile tg
+            uint32_t buf = 0, aslot = 0, e_slot = kMAccSlots - kMAccBufs, e_par = 1;   // small: accumulator, (accumulator, group) slot; slot to wait for
+            int vg = 0;                  // virtual tiles issued so far (all layers); the epilogue pair vg & 1 reads tile vg
             bool ok = true;
             for (int s = 0; s < p.n_compute && ok; ++s) {
                 ok = mbar_wait(smem_u32(&ctl.qfull), s & 1, abort_flag);
-                for (int ti = 0; ti < nt && ok; ++ti, ++tg) {
+                for (int ti = 0; ti < nt && ok; ++ti) {
                     uint32_t st_kb[2] = {0u, 0u};
 #pragma unroll
                     for (int kb = 0; kb < 2; ++kb) {
@@ -406,28 +437,47 @@ model_kernel(const __grid_constant__ ModelParams p) {
                         if (++st == n_stages) { st = 0; st_par ^= 1u; }
                     }
                     if (!ok) break;
+                    for (int mt = 0; mt < n_mt && ok; ++mt, ++vg) {
+                        if constexpr (BIG) {
+                            const uint32_t ab = vg & 1;
+                            ok = mbar_wait(smem_u32(&ctl.tempty[ab]), ((vg >> 1) & 1) ^ 1, abort_flag);
+                            if (!ok) break;
+                            tc_fence_after();
+                            const uint32_t d_addr = tmem_base + ab * kRUmmaN;
 #pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        // panel pc goes to accumulator pc % 3, which panel pc - 3 used last
-                        const int pc = 2 * tg + half;
-                        if (pc >= kMAccBufs) {
-                            const int prev = pc - kMAccBufs;
-                            ok = mbar_wait(smem_u32(&ctl.tempty[prev % kMAccSlots]), (prev / kMAccSlots) & 1, abort_flag);
+                            for (int kb = 0; kb < 2; ++kb) {
+                                if (kb >= KB) break;
+                                const uint64_t b_desc = umma_desc_sw128(k_base + st_kb[kb] * STAGE);
+                                const uint64_t a_desc = umma_desc_sw128(q_base + static_cast<uint32_t>(mt * KB + kb) * kRQTileBytes);
+#pragma unroll
+                                for (int k4 = 0; k4 < 4; ++k4)
+                                    umma_bf16(d_addr, a_desc + 2u * k4, b_desc + 2u * k4, IDESC, (kb > 0 || k4 > 0) ? 1u : 0u);
+                            }
+                            umma_commit(smem_u32(&ctl.tfull[ab]));
+                        } else {
+#pragma unroll
+                            for (int half = 0; half < 2; ++half) {
+                                // a panel goes to accumulator (panel number % 3), which the third panel before it used last:
+                                // wait until that one's group has read it (the first three panels find a fresh barrier)
+                                ok = mbar_wait(smem_u32(&ctl.tempty[e_slot]), e_par, abort_flag);
+                                if (++e_slot == kMAccSlots) { e_slot = 0; e_par ^= 1u; }
+                                if (!ok) break;
+                                tc_fence_after();
+                                const uint32_t d_addr = tmem_base + buf * kMAccN;
+#pragma unroll
+                                for (int kb = 0; kb < 2; ++kb) {
+                                    if (kb >= KB) break;
+                                    const uint64_t b_desc = umma_desc_sw128(k_base + st_kb[kb] * STAGE + static_cast<uint32_t>(half * ACC1 * 128));
+                                    const uint64_t a_desc = umma_desc_sw128(q_base + static_cast<uint32_t>(kb) * kRQTileBytes);
+#pragma unroll
+                                    for (int k4 = 0; k4 < 4; ++k4)
+                                        umma_bf16(d_addr, a_desc + 2u * k4, b_desc + 2u * k4, IDESC, (kb > 0 || k4 > 0) ? 1u : 0u);
+                                }
+                                umma_commit(smem_u32(&ctl.tfull[aslot]));
+                                if (++buf == kMAccBufs) buf = 0;
+                                if (++aslot == kMAccSlots) aslot = 0;
+                            }
                         }
-                        if (!ok) break;
-                        tc_fence_after();
-                        const uint32_t d_addr = tmem_base + static_cast<uint32_t>((pc % kMAccBufs) * kMAccN);
-#pragma unroll
-                        for (int kb = 0; kb < 2; ++kb) {
-                            if (kb >= KB) break;
-                            const uint64_t b_desc =
-                                umma_desc_sw128(k_base + st_kb[kb] * kRStageBytes + static_cast<uint32_t>(half * kMAcc1Row * 128));
-                            const uint64_t a_desc = umma_desc_sw128(q_base + static_cast<uint32_t>(kb) * kRQTileBytes);
-#pragma unroll
-                            for (int k4 = 0; k4 < 4; ++k4)
-                                umma_bf16(d_addr, a_desc + 2u * k4, b_desc + 2u * k4, IDESC, (kb > 0 || k4 > 0) ? 1u : 0u);
-                        }
-                        umma_commit(smem_u32(&ctl.tfull[pc % kMAccSlots]));
                     }
                     if (!ok) break;
 #pragma unroll
@@ -447,44 +497,62 @@ model_kernel(const __grid_constant__ ModelParams p) {
         const int grp = (warp - 2) >> 2, quarter = warp & 3;
         const int gt = threadIdx.x - 64 - grp * 128;    // 0 .. 127 within the group
         const int pair = grp >> 1, half = grp & 1;
-        const int row = quarter * 32 + lane;
-        const bool active = row < p.R;
-        const int last_visible = p.P + (row % p.w);
+        const int row = quarter * 32 + lane;             // row of the query tile = lane of tensor memory
+        const int qrow = row + (two ? pair * 128 : 0);   // row of the KV head (two query tiles: a pair takes one of them)
+        const bool active = qrow < p.R;
+        const int last_visible = p.P + (qrow % p.w);
         const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
-        const int n_pl = 2 * nt;
-        constexpr int PR = (C_STATIC == 10) ? kMRingPanels10 : kMRingPanels20;     // panels in the rings
-        const int ahead = max(0, min(nt, (PR - n_pl) / 2));   // tiles of the next layer scored before the contraction
-        const int ch0 = t_begin * (kRTile / C_STATIC);
+        const int n_pl = 2 * n_vt;
+        const int PR = BIG ? p.ring : model_ring_panels(C_STATIC, false);          // panels in the ring
+        constexpr int PCOLS = BIG ? SPP + 1 : SPP;                                  // tensor-memory columns of a panel
+        const int ahead = max(0, min(n_vt, (PR - n_pl) / 2));   // virtual tiles of the next layer scored before the contraction
+        const int ch0 = t_begin * (TILE / C_STATIC);
+        const uint64_t keep = l2_policy_evict_last(), drop = l2_policy_evict_first();
+        float* spill = BIG ? p.spill + static_cast<size_t>(blockIdx.x) * (p.ring - p.ring_on) * ((SPP + 1) * 128) + row : nullptr;
         bool ok = true;
         float run_m = -CUDART_INF_F, run_l = 0.f;
-        // tiles [ti_lo, ti_hi) of slot s that belong to this thread's pair
-        auto do_tiles = [&](int s, int ti_lo, int ti_hi) {
+        // virtual tiles [v_lo, v_hi) of slot s that belong to this thread's pair
+        auto do_tiles = [&](int s, int v_lo, int v_hi) {
             if (!ok) return;
-            const int tg0 = s * nt, pbase = (s * n_pl) % PR;
-            for (int ti = ti_lo + ((pair - ((tg0 + ti_lo) & 1)) & 1); ti < ti_hi; ti += 2) {
-                const int pc = 2 * (tg0 + ti) + half;        // panel number since the start of the launch
-                const int aslot = pc % kMAccSlots;
+            const int vg0 = s * n_vt, pbase = (s * n_pl) % PR;
+            for (int vt = v_lo + ((pair - ((vg0 + v_lo) & 1)) & 1); vt < v_hi; vt += 2) {
+                const int ti = two ? vt >> 1 : vt;
+                const int pc = 2 * (vg0 + vt) + half;        // panel number since the start of the launch
+                const int aslot = BIG ? pair : pc % kMAccSlots;
+                const int use = BIG ? (vg0 + vt) >> 1 : pc / kMAccSlots;
+                const int acol = BIG ? pair * kRUmmaN + half * WP : (pc % kMAccBufs) * kMAccN + half * COL1;
                 bool ready = true;
-                if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[aslot]), (pc / kMAccSlots) & 1, abort_flag);
+                if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[aslot]), use & 1, abort_flag);
                 if (!__shfl_sync(0xffffffffu, ready, 0)) { ok = false; break; }
                 tc_fence_after();
-                float v[kRPanel];
-                load_panel<kRPanel>(lane_addr + static_cast<uint32_t>((pc % kMAccBufs) * kMAccN + half * (kRPanel - kMAcc1Row)), v);
+                float v[WP];
+                load_panel<WP>(lane_addr + static_cast<uint32_t>(acol), v);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctl.tempty[aslot]));
-                const int pl = ti * 2 + half;
+                const int pl = vt * 2 + half;
                 int slot = pbase + pl;
                 slot -= (slot >= PR) ? PR : 0;
-                const int j0 = (t_begin + ti) * kRTile + half * kRPanel;
-                float pr[SPP], m2, l;
+                const int j0 = (t_begin + ti) * TILE + half * WP;
+                float pr[PCOLS], m2, l;          // (big variant: the panel maximum behind the chunk sums)
                 auto emit = [&](int ch, float acc) { pr[ch] = acc; };
-                if (j0 + kRPanel <= p.P)
-                    panel_fast<C_STATIC, kRPanel>(v, p.sl2, emit, &m2, &l);
+                if (j0 + WP <= p.P)
+                    panel_fast<C_STATIC, WP>(v, p.sl2, emit, &m2, &l);
                 else
-                    panel_static_tail<C_STATIC, kRPanel>(v, p.sl2, emit, j0, p.P, last_visible, &m2, &l);
-                part_store<SPP>(lane_addr + static_cast<uint32_t>(kMPartCol0 + slot * SPP), pr);
-                pmax[slot * 128 + row] = m2;
+                    panel_static_tail<C_STATIC, WP>(v, p.sl2, emit, j0, p.P, last_visible, &m2, &l);
+                if constexpr (BIG) {
+                    pr[SPP] = m2;
+                    if (slot < p.ring_on) {
+                        part_store<PCOLS>(lane_addr + static_cast<uint32_t>(PART0 + slot * PCOLS), pr);
+                    } else {
+                        float* sp = spill + static_cast<size_t>(slot - p.ring_on) * (PCOLS * 128);
+#pragma unroll
+                        for (int q = 0; q < PCOLS; ++q) st_keep(sp + q * 128, pr[q], keep);
+                    }
+                } else {
+                    part_store<SPP>(lane_addr + static_cast<uint32_t>(PART0 + slot * SPP), pr);
+                    pmax[slot * 128 + row] = m2;
+                }
                 const float nm = fmaxf(run_m, m2);
                 const float s_old = (run_m == -CUDART_INF_F) ? 0.f : ex2_approx(run_m - nm);
                 const float s_new = (m2 == -CUDART_INF_F) ? 0.f : ex2_approx(m2 - nm);
@@ -495,7 +563,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
         // end of slot s: this group's (max, sum) per row -> shared memory; the statistics warp merges the four
         // groups, stores the CTA's record and announces it (no block-wide barrier on the scoring warps' path)
         auto publish = [&](int s) {
-            float* rc = rec + (s & 1) * 3584;
+            float* rc = rec + (s & 1) * 3072;
             rc[(grp * 2 + 0) * 128 + row] = active ? run_m : -CUDART_INF_F;
             rc[(grp * 2 + 1) * 128 + row] = active ? run_l : 0.f;
             run_m = -CUDART_INF_F;
@@ -507,50 +575,84 @@ model_kernel(const __grid_constant__ ModelParams p) {
         // scored itself - every thread reads back the tensor-memory columns and panel maxima it wrote -
         // so the only synchronisation is among the group's four warps (the four lane quarters of a sum).
         auto contract = [&](int s) -> bool {
-            const int tg0 = s * nt, pbase = (s * n_pl) % PR;
+            const int vg0 = s * n_vt, pbase = (s * n_pl) % PR;
             // first panel of the slot that this group scored; its others follow every fourth panel
-            const int g1 = 2 * (((grp >> 1) - tg0) & 1) + half;
+            const int g1 = 2 * ((pair - vg0) & 1) + half;
             bool ready = true;
             if (lane == 0) ready = mbar_wait(smem_u32(&ctl.stat_full[s & 1]), (s >> 1) & 1, abort_flag);
             if (!__shfl_sync(0xffffffffu, ready, 0)) ok = false;   // (the failed wait has raised the abort flag)
             tmem_st_wait();
             // the group's previous sums have been read by all its warps; and a uniform decision to go on
             if (named_barrier_or(kBarGroup + grp, 128, !ok || ctl.abort_flag != 0)) return false;
-            const float* gm = gstat + (s & 1) * 256;
+            const float* gm = gstat + (s & 1) * 512 + (two ? pair * 256 : 0);
             const float mi = gm[row], li = gm[128 + row];
-            constexpr int PPB = 30 / SPP;
-            for (int b0 = 0; g1 + 4 * b0 < n_pl; b0 += PPB) {
-                float v[32];
-                int slot_of[PPB];
+            float* rg = red + grp * (4 * kMSegSlots);
+            float* sc_out = p.scores + ((static_cast<size_t>(s) * p.Hkv + hkv) * n_mt + (two ? pair : 0)) * p.Cpad;
+            constexpr int PPB = 32 / SPP;                    // panels per block of up to 32 values
+            constexpr int BPS = kMSegSlots / (PPB * SPP);    // blocks per segment
+            const int own = (n_pl - g1 + 3) / 4;             // panels of this group
+            for (int s0 = 0; s0 < own; s0 += PPB * BPS) {
+                // (the previous segment's sums have been read: a barrier lies between)
+                if (s0 > 0) named_barrier(kBarGroup + grp, 128);
+                for (int b0 = s0; b0 < min(own, s0 + PPB * BPS); b0 += PPB) {
+                    float v[32], pm[PPB];
+                    int slot_of[PPB];
 #pragma unroll
-                for (int u = 0; u < PPB; ++u) {
-                    const int pl = min(g1 + 4 * (b0 + u), n_pl - 1);
-                    int slot = pbase + pl;
-                    slot -= (slot >= PR) ? PR : 0;
-                    slot_of[u] = slot;
-                    part_load<SPP>(lane_addr + static_cast<uint32_t>(kMPartCol0 + slot * SPP), &v[u * SPP]);
+                    for (int u = 0; u < PPB; ++u) {
+                        const int pl = min(g1 + 4 * (b0 + u), n_pl - 1);
+                        int slot = pbase + pl;
+                        slot -= (slot >= PR) ? PR : 0;
+                        slot_of[u] = slot;
+                    }
+                    if constexpr (BIG) {
+                        float vp[PPB * PCOLS];
+#pragma unroll
+                        for (int u = 0; u < PPB; ++u) {
+                            if (slot_of[u] < p.ring_on) {
+                                part_load<PCOLS>(lane_addr + static_cast<uint32_t>(PART0 + slot_of[u] * PCOLS), &vp[u * PCOLS]);
+                            } else {
+                                const float* sp = spill + static_cast<size_t>(slot_of[u] - p.ring_on) * (PCOLS * 128);
+#pragma unroll
+                                for (int q = 0; q < PCOLS; ++q) vp[u * PCOLS + q] = ld_drop(sp + q * 128, drop);
+                            }
+                        }
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int u = 0; u < PPB; ++u) {
+                            pm[u] = vp[u * PCOLS + SPP];
+#pragma unroll
+                            for (int q = 0; q < SPP; ++q) v[u * SPP + q] = vp[u * PCOLS + q];
+                        }
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < PPB; ++u)
+                            part_load<SPP>(lane_addr + static_cast<uint32_t>(PART0 + slot_of[u] * SPP), &v[u * SPP]);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int u = 0; u < PPB; ++u) pm[u] = pmax[slot_of[u] * 128 + row];
+                    }
+#pragma unroll
+                    for (int e = PPB * SPP; e < 32; ++e) v[e] = 0.f;
+#pragma unroll
+                    for (int u = 0; u < PPB; ++u) {
+                        const bool have = active && b0 + u < own;
+                        const float f = have ? ex2_approx(pm[u] - mi) * li : 0.f;
+#pragma unroll
+                        for (int q = 0; q < SPP; ++q) v[u * SPP + q] = have ? v[u * SPP + q] * f : 0.f;
+                    }
+                    const float tot = warp_transpose_reduce(v, lane);
+                    if (lane < PPB * SPP) rg[quarter * kMSegSlots + (b0 - s0) * SPP + lane] = tot;
                 }
-                tmem_ld_wait();
-                v[30] = 0.f;
-                v[31] = 0.f;
-#pragma unroll
-                for (int u = 0; u < PPB; ++u) {
-                    const int pl = g1 + 4 * (b0 + u);
-                    const bool have = active && pl < n_pl;
-                    const float f = have ? ex2_approx(pmax[slot_of[u] * 128 + row] - mi) * li : 0.f;
-#pragma unroll
-                    for (int q = 0; q < SPP; ++q) v[u * SPP + q] = have ? v[u * SPP + q] * f : 0.f;
+                named_barrier(kBarGroup + grp, 128);
+                // chunk slots of this segment's panels (at most kMSegSlots)
+                const int n_own = min(own - s0, PPB * BPS) * SPP;
+                if (gt < n_own) {
+                    const int pl = g1 + 4 * (s0 + gt / SPP);
+                    const int kp = two ? (pl >> 2) * 2 + (pl & 1) : pl;          // panel of the key range
+                    const int ch = ch0 + kp * SPP + gt % SPP;
+                    if (ch < p.C)
+                        sc_out[ch] = (rg[gt] + rg[kMSegSlots + gt]) + (rg[2 * kMSegSlots + gt] + rg[3 * kMSegSlots + gt]);
                 }
-                const float tot = warp_transpose_reduce(v, lane);
-                const int pl = g1 + 4 * (b0 + lane / SPP);
-                if (lane < 30 && pl < n_pl) red[quarter * 256 + pl * SPP + lane % SPP] = tot;
-            }
-            named_barrier(kBarGroup + grp, 128);
-            float* sc_out = p.scores + (static_cast<size_t>(s) * p.Hs + hs) * p.Cpad;
-            const int n_own = (n_pl - g1 + 3) / 4 * SPP;     // chunk slots of this group's panels
-            for (int i = gt; i < n_own; i += 128) {
-                const int lc = (g1 + 4 * (i / SPP)) * SPP + i % SPP;
-                if (ch0 + lc < p.C) sc_out[ch0 + lc] = (red[lc] + red[256 + lc]) + (red[512 + lc] + red[768 + lc]);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&ctl.sc_done[s & 1]));      // announced by the statistics warp
@@ -560,7 +662,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
             if (s < p.n_compute) do_tiles(s, 0, ahead);
             if (s > 0 && !contract(s - 1)) break;
             if (s < p.n_compute) {
-                do_tiles(s, ahead, nt);
+                do_tiles(s, ahead, n_vt);
                 publish(s);
             }
         }
@@ -583,46 +685,52 @@ model_kernel(const __grid_constant__ ModelParams p) {
                 // four groups (this lane: rows 4 lane .. 4 lane + 3), store the CTA's record and announce it.
                 // release: the record stores of the whole warp, ordered by __syncwarp, are visible to whoever
                 // sees the count
-                const float* rc = rec + (s & 1) * 3584;
-                float Mo[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}, So[4] = {0.f, 0.f, 0.f, 0.f};
-                float4 m[4], l[4];
+                const float* rc = rec + (s & 1) * 3072;
+                for (int mt = 0; mt < n_mt; ++mt) {
+                    float Mo[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}, So[4] = {0.f, 0.f, 0.f, 0.f};
+                    float4 m[4], l[4];
+                    const int n_g = two ? 2 : 4;         // groups that scored this query tile
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    m[g] = *reinterpret_cast<const float4*>(rc + (g * 2) * 128 + r0);
-                    l[g] = *reinterpret_cast<const float4*>(rc + (g * 2 + 1) * 128 + r0);
+                    for (int g = 0; g < 4; ++g) {
+                        const int gg = two ? mt * 2 + (g & 1) : g;
+                        m[g] = *reinterpret_cast<const float4*>(rc + (gg * 2) * 128 + r0);
+                        l[g] = *reinterpret_cast<const float4*>(rc + (gg * 2 + 1) * 128 + r0);
+                    }
+                    merge_batch<4>(Mo, So, m, l, n_g);
+                    float* dst = p.cta_stat + ((static_cast<size_t>(s & 1) * gridDim.x + blockIdx.x) * n_mt + mt) * 256;
+                    *reinterpret_cast<float4*>(dst + r0) = make_float4(Mo[0], Mo[1], Mo[2], Mo[3]);
+                    *reinterpret_cast<float4*>(dst + 128 + r0) = make_float4(So[0], So[1], So[2], So[3]);
                 }
-                merge_batch<4>(Mo, So, m, l, 4);
-                float* dst = p.cta_stat + (static_cast<size_t>(s & 1) * gridDim.x + blockIdx.x) * 256;
-                *reinterpret_cast<float4*>(dst + r0) = make_float4(Mo[0], Mo[1], Mo[2], Mo[3]);
-                *reinterpret_cast<float4*>(dst + 128 + r0) = make_float4(So[0], So[1], So[2], So[3]);
                 __syncwarp();
             }
-            if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.cnt_a + hs) : "memory");
-            if (!wait_counter_warp(p.cnt_a + hs, static_cast<unsigned>(s + 1) * p.cph, abort_flag)) break;
-            const float* src = p.cta_stat + (static_cast<size_t>(s & 1) * gridDim.x + static_cast<size_t>(hs) * p.cph) * 256;
-            float M[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}, S[4] = {0.f, 0.f, 0.f, 0.f};
+            if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.cnt_a + hkv) : "memory");
+            if (!wait_counter_warp(p.cnt_a + hkv, static_cast<unsigned>(s + 1) * p.cph, abort_flag)) break;
             // the head's records straight from the L2 (they were written by other SMs; every lane has
             // acquired the counter), six CTAs' worth of loads in flight per lane
-            for (int j0 = 0; j0 < p.cph; j0 += 6) {
-                float4 m[6], l[6];
+            for (int mt = 0; mt < n_mt; ++mt) {
+                const size_t step = static_cast<size_t>(n_mt) * 256;
+                const float* src = p.cta_stat + ((static_cast<size_t>(s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * n_mt + mt) * 256;
+                float M[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}, S[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int j0 = 0; j0 < p.cph; j0 += 6) {
+                    float4 m[6], l[6];
 #pragma unroll
-                for (int j = 0; j < 6; ++j) {
-                    const int jj = min(j0 + j, p.cph - 1);
-                    m[j] = __ldcg(reinterpret_cast<const float4*>(src + static_cast<size_t>(jj) * 256 + r0));
-                    l[j] = __ldcg(reinterpret_cast<const float4*>(src + static_cast<size_t>(jj) * 256 + 128 + r0));
+                    for (int j = 0; j < 6; ++j) {
+                        const int jj = min(j0 + j, p.cph - 1);
+                        m[j] = __ldcg(reinterpret_cast<const float4*>(src + jj * step + r0));
+                        l[j] = __ldcg(reinterpret_cast<const float4*>(src + jj * step + 128 + r0));
+                    }
+                    merge_batch<6>(M, S, m, l, p.cph - j0);
                 }
-                merge_batch<6>(M, S, m, l, p.cph - j0);
+                float* gm = gstat + (s & 1) * 512 + mt * 256;
+                *reinterpret_cast<float4*>(gm + r0) = make_float4(M[0], M[1], M[2], M[3]);
+                *reinterpret_cast<float4*>(gm + 128 + r0) = make_float4(1.0f / S[0], 1.0f / S[1], 1.0f / S[2], 1.0f / S[3]);
             }
-            if (!ok) break;
-            float* gm = gstat + (s & 1) * 256;
-            *reinterpret_cast<float4*>(gm + r0) = make_float4(M[0], M[1], M[2], M[3]);
-            *reinterpret_cast<float4*>(gm + 128 + r0) = make_float4(1.0f / S[0], 1.0f / S[1], 1.0f / S[2], 1.0f / S[3]);
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(smem_u32(&ctl.stat_full[s & 1]));
                 // the epilogue forms the slot's chunk scores next; announce them when they are stored
                 if (mbar_wait(smem_u32(&ctl.sc_done[s & 1]), static_cast<uint32_t>(s >> 1) & 1u, abort_flag))
-                    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.cnt_b + hs) : "memory");
+                    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.cnt_b + hkv) : "memory");
                 else
                     ok = false;
             }
@@ -640,8 +748,9 @@ model_kernel(const __grid_constant__ ModelParams p) {
             int* row = reinterpret_cast<int*>(tbase);        // [4 + kkpad]: n_tok, -, -, -, kept chunk ids
             const uint32_t stage0 = smem_u32(tbase + p.sel_row_bytes);
             const int* sel = row + 4;
-            const int Q = p.cph << p.kv_shift;               // CTAs of this KV head
-            const int q = static_cast<int>(blockIdx.x) - (hkv << p.kv_shift) * p.cph;
+            const int Q = p.cph, q = part;                   // CTAs of this KV head
+            constexpr uint32_t kSl = C_STATIC <= 10 ? kMSlots : 0;   // staging slots where every head dim has the most
+            const uint32_t n_slots = kSl ? kSl : static_cast<uint32_t>(p.copy_slots);
             const int kk = min(p.k, p.C);
             const int wu = (p.w + C_STATIC - 1) / C_STATIC;  // the window as pseudo-chunks of up to c rows
             const int U = kk + wu;                           // copy units of the head
@@ -650,7 +759,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
             const int n_units = u_end - u_begin;
             const uint32_t row_bytes = static_cast<uint32_t>(p.d) * 2u;
             const uint32_t half_slot = static_cast<uint32_t>(p.stage_slot_bytes) / 2u;
-            uint32_t g_issued = 0;                           // units loaded so far (all layers): slot = g % kMSlots
+            uint32_t g_issued = 0;                           // units loaded so far (all layers): slot = g % n_slots
             bool ok = true;
             for (int li = 0; li < p.n_layers && ok;) {
                 const int s = p.layer[li].slot;
@@ -697,7 +806,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                     auto issue_load = [&](int idx) {
                         int sr, dr, rows;
                         unit(u_begin + idx, sr, dr, rows);
-                        const uint32_t slot = (g_issued + idx) % kMSlots;
+                        const uint32_t slot = (g_issued + idx) % n_slots;
                         const uint32_t bytes = static_cast<uint32_t>(rows) * row_bytes;
                         const uint32_t bar = smem_u32(&ctl.gfull[slot]);
                         if (lane == 0) mbar_arrive_expect_tx(bar, 2u * bytes);
@@ -715,12 +824,12 @@ model_kernel(const __grid_constant__ ModelParams p) {
                             }
                         }
                     };
-                    // loads run kMSlots - 1 units ahead of the stores
-                    for (; loaded < n_units && loaded < kMSlots - 1; ++loaded) issue_load(loaded);
+                    // loads run n_slots - 1 units ahead of the stores
+                    for (; loaded < n_units && loaded < static_cast<int>(n_slots) - 1; ++loaded) issue_load(loaded);
                     for (int idx = 0; idx < n_units && ok; ++idx) {
                         const uint32_t gi = g_issued + idx;
-                        const uint32_t slot = gi % kMSlots;
-                        if (lane == 0) ok = mbar_wait(smem_u32(&ctl.gfull[slot]), (gi / kMSlots) & 1u, abort_flag);
+                        const uint32_t slot = gi % n_slots;
+                        if (lane == 0) ok = mbar_wait(smem_u32(&ctl.gfull[slot]), (gi / n_slots) & 1u, abort_flag);
                         if constexpr (STRIDED) ok = __shfl_sync(0xffffffffu, ok, 0);
                         if (!ok) break;
                         int sr, dr, rows;
@@ -761,8 +870,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
         if (ctl.abort_flag) atomicExch(p.status, 1);
         const unsigned old = atomicAdd(p.exits, 1u);
         if (old + 1u == gridDim.x) {
-            for (int h = 0; h < p.Hs; ++h) { p.cnt_a[h] = 0u; p.cnt_b[h] = 0u; }
-            for (int h = 0; h < p.Hkv; ++h) p.cnt_c[h] = 0u;
+            for (int h = 0; h < p.Hkv; ++h) { p.cnt_a[h] = 0u; p.cnt_b[h] = 0u; p.cnt_c[h] = 0u; }
             *p.exits = 0u;
             __threadfence();
         }
@@ -771,41 +879,53 @@ model_kernel(const __grid_constant__ ModelParams p) {
 
 }  // namespace
 
-bool make_model_plan(int L, int Rs, int Hs, int kv_shift, int d, int c, int C, int k, int max_ctas, int smem_limit,
-                     ModelPlan* plan) {
-    if (c != 10 && c != 20) return false;
-    if (Rs < 1 || Rs > 128 || (d != 64 && d != 128) || L < 1 || C < 1 || k < 1 || Hs < 1 || Hs > kResidentMaxHeads)
+bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, ModelPlan* plan) {
+    if (c != 5 && c != 8 && c != 10 && c != 16 && c != 20 && c != 32) return false;
+    if (R < 1 || R > 256 || (d != 64 && d != 128) || L < 1 || C < 1 || k < 1 || Hkv < 1 || Hkv > kResidentMaxHeads)
         return false;
-    const int Hkv = Hs >> kv_shift;
     const int kk = k < C ? k : C;
     if (kk > kSelCap) return false;                          // the selector stages the kept chunk ids in shared memory
-    if (max_ctas < Hs + 1) return false;
+    if (max_ctas < Hkv + 1) return false;
     ModelPlan p{};
     p.c_static = c;
+    p.n_mt = R > 128 ? 2 : 1;
+    p.tile = 2 * panel_keys(c);
+    p.spp = panel_keys(c) / c;
+    p.n_tiles = (L + p.tile - 1) / p.tile;
     // a few CTAs do nothing but select (they take the SMs the scoring grid would leave idle anyway)
     p.n_sel = Hkv < 4 ? Hkv : 4;
-    if (max_ctas - p.n_sel < Hs) p.n_sel = max_ctas - Hs;
-    p.cph = (max_ctas - p.n_sel) / Hs;
-    p.n_score = p.cph * Hs;
+    if (max_ctas - p.n_sel < Hkv) p.n_sel = max_ctas - Hkv;
+    p.cph = (max_ctas - p.n_sel) / Hkv;
+    if (p.cph > p.n_tiles) p.cph = p.n_tiles;
+    p.n_score = p.cph * Hkv;
     p.grid = p.n_score + p.n_sel;
-    p.n_tiles = (L + kRTile - 1) / kRTile;
     p.t_max = (p.n_tiles + p.cph - 1) / p.cph;
-    const int ring_panels = c == 10 ? kMRingPanels10 : kMRingPanels20;
-    // a layer's chunk scores are summed in a 4 x 256-float buffer, its panels must fit the rings
-    if (p.t_max * (kRTile / c) > 252 || 2 * p.t_max > ring_panels) return false;
-    const int KB = d / 64;
-    const int q_bytes = KB * kRQTileBytes;
-    const int pmax_bytes = ring_panels * 128 * 4;            // the panel-maxima ring: one row set per ring panel
+    // Panels of a CTA and layer; the ring should hold them and at least kMinAhead of the next layer, whose scoring
+    // hides the exchange of row statistics. Where tensor memory holds fewer the ring continues in scratch.
+    constexpr int kMinAhead = 8, kBigAhead = 24;
+    const int n_pl = 2 * p.n_mt * p.t_max;
+    p.big = p.n_mt == 2 || n_pl + kMinAhead > model_ring_panels(c, false);
+    if (p.big) {
+        p.ring_on = model_ring_panels(c, true);
+        p.ring = (n_pl + (kBigAhead < n_pl ? kBigAhead : n_pl) + 3) / 4 * 4;
+        if (p.ring < p.ring_on) p.ring = p.ring_on;
+    } else {
+        p.ring_on = p.ring = model_ring_panels(c, false);
+    }
+    const int KB = d / 64, stage = p.tile * 128;
+    const int q_bytes = p.n_mt * KB * kRQTileBytes;
+    const int pmax_bytes = p.big ? 0 : p.ring * 128 * 4;     // the panel-maxima ring: one row set per ring panel
+    p.copy_slots = c <= 10 ? kMSlots : model_copy_slots(c, d);
     p.stage_slot_bytes = 2 * c * d * 2;                        // K rows and V rows of one chunk
     p.sel_row_bytes = ((4 + kk) * 4 + 127) & ~127;
-    const int tail_bytes = p.sel_row_bytes + kMSlots * p.stage_slot_bytes + 128;
+    const int tail_bytes = p.sel_row_bytes + p.copy_slots * p.stage_slot_bytes + 128;
     const int fixed = 1024 + q_bytes + 1024 + pmax_bytes + kMMiscBytes + tail_bytes;
-    int ns = (smem_limit - 512 - fixed) / kRStageBytes;           // (the control block is larger than the layer kernel's)
+    int ns = (smem_limit - 512 - fixed) / stage;               // (the control block is larger than the layer kernel's)
     if (ns > kRMaxStages) ns = kRMaxStages;
     if (ns < 2 * KB + 1) return false;
     p.n_stages = ns;
     p.off_ring = q_bytes;
-    p.off_pmax = p.off_ring + ns * kRStageBytes + 1024;
+    p.off_pmax = p.off_ring + ns * stage + 1024;
     p.off_misc = p.off_pmax + pmax_bytes;
     p.off_tail = p.off_misc + kMMiscBytes;
     p.smem_bytes = 1024 + p.off_tail + tail_bytes;
@@ -818,9 +938,19 @@ bool make_model_plan(int L, int Rs, int Hs, int kv_shift, int d, int c, int C, i
     return true;
 }
 
-size_t model_scratch_floats(const ModelPlan& plan, int Hs, int kv_shift, int C, int n_compute) {
-    return static_cast<size_t>(2) * plan.grid * 256 + static_cast<size_t>(n_compute) * Hs * ((C + 3) & ~3) +
-           static_cast<size_t>(n_compute) * (Hs >> kv_shift) * (plan.sel_row_bytes / 4) + 64;
+size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute) {
+    return static_cast<size_t>(2) * plan.grid * plan.n_mt * 256 + static_cast<size_t>(n_compute) * Hkv * plan.n_mt * ((C + 3) & ~3) +
+           static_cast<size_t>(n_compute) * Hkv * (plan.sel_row_bytes / 4) + 64 +
+           static_cast<size_t>(plan.n_score) * (plan.ring - plan.ring_on) * (plan.spp + 1) * 128;
+}
+
+template <int C_STATIC>
+static const void* model_kernel_of(bool strided, bool big) {
+    if (big)
+        return strided ? reinterpret_cast<const void*>(model_kernel<C_STATIC, true, true>)
+                       : reinterpret_cast<const void*>(model_kernel<C_STATIC, false, true>);
+    return strided ? reinterpret_cast<const void*>(model_kernel<C_STATIC, true, false>)
+                   : reinterpret_cast<const void*>(model_kernel<C_STATIC, false, false>);
 }
 
 cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtensorMap* tm_q, const CUtensorMap* tm_k,
@@ -845,37 +975,47 @@ cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtenso
     }
     p.n_layers = n_layers;
     p.n_compute = n_compute;
-    p.L = io.L; p.P = io.L - io.w; p.w = io.w; p.R = io.Rs; p.Hs = io.Hs; p.d = io.d; p.kv_shift = io.kv_shift;
+    p.L = io.L; p.P = io.L - io.w; p.w = io.w; p.R = io.R; p.d = io.d; p.n_mt = plan.n_mt;
     p.sl2 = io.sl2;
     p.k_row_bytes = 2 * (io.k_row_elems ? io.k_row_elems : io.d);
     p.v_row_bytes = 2 * (io.v_row_elems ? io.v_row_elems : io.d);
     p.k_head_bytes = 2 * (io.k_head_elems ? io.k_head_elems : static_cast<long long>(io.L) * io.d);
     p.v_head_bytes = 2 * (io.v_head_elems ? io.v_head_elems : static_cast<long long>(io.L) * io.d);
     p.cph = plan.cph; p.n_tiles = plan.n_tiles; p.n_stages = plan.n_stages;
-    p.q_box_rows = io.Rs < 128 ? io.Rs : 128;
-    p.k_box_rows = io.L < kRTile ? io.L : kRTile;
-    p.C = io.C; p.k = io.k; p.n_max = io.n_max; p.Hkv = io.Hs >> io.kv_shift;
+    p.q_box_rows = io.R < 128 ? io.R : 128;
+    p.k_box_rows = io.L < plan.tile ? io.L : plan.tile;
+    p.C = io.C; p.k = io.k; p.n_max = io.n_max; p.Hkv = io.Hkv;
+    p.ring_on = plan.ring_on; p.ring = plan.ring; p.copy_slots = plan.copy_slots;
     p.Cpad = (io.C + 3) & ~3;
     p.n_score = plan.n_score; p.n_sel = plan.n_sel;
     p.sel_row_bytes = plan.sel_row_bytes; p.sel_keys_fit = plan.sel_keys_fit;
     p.off_ring = plan.off_ring; p.off_pmax = plan.off_pmax; p.off_misc = plan.off_misc; p.off_tail = plan.off_tail;
     p.stage_slot_bytes = plan.stage_slot_bytes;
     p.cta_stat = io.scratch;
-    p.scores = io.scratch + static_cast<size_t>(2) * plan.grid * 256;
-    p.sel_rows = reinterpret_cast<int*>(p.scores + static_cast<size_t>(n_compute) * io.Hs * p.Cpad);   // 16-byte aligned: Cpad % 4 == 0
+    p.scores = io.scratch + static_cast<size_t>(2) * plan.grid * plan.n_mt * 256;
+    p.sel_rows = reinterpret_cast<int*>(p.scores + static_cast<size_t>(n_compute) * io.Hkv * plan.n_mt * p.Cpad);   // 16-byte aligned: Cpad % 4 == 0
+    p.spill = reinterpret_cast<float*>(p.sel_rows) + static_cast<size_t>(n_compute) * io.Hkv * (plan.sel_row_bytes / 4);
     p.exits = io.counters;
     p.cnt_a = io.counters + 16;
     p.cnt_b = io.counters + 16 + kResidentMaxHeads;
     p.cnt_c = io.counters + 16 + 2 * kResidentMaxHeads;
     p.status = io.status;
     const bool strided = io.k_row_elems != 0 || io.v_row_elems != 0 || io.k_head_elems != 0 || io.v_head_elems != 0;
-    const void* kern = plan.c_static == 10
-                           ? (strided ? reinterpret_cast<const void*>(model_kernel<10, true>) : reinterpret_cast<const void*>(model_kernel<10, false>))
-                           : (strided ? reinterpret_cast<const void*>(model_kernel<20, true>) : reinterpret_cast<const void*>(model_kernel<20, false>));
-    static int smem_set[4][64] = {{0}};
+    const void* kern = nullptr;
+    int v = 0;
+    switch (plan.c_static) {
+        case 5: kern = model_kernel_of<5>(strided, plan.big); v = 0; break;
+        case 8: kern = model_kernel_of<8>(strided, plan.big); v = 1; break;
+        case 10: kern = model_kernel_of<10>(strided, plan.big); v = 2; break;
+        case 16: kern = model_kernel_of<16>(strided, plan.big); v = 3; break;
+        case 20: kern = model_kernel_of<20>(strided, plan.big); v = 4; break;
+        case 32: kern = model_kernel_of<32>(strided, plan.big); v = 5; break;
+        default: break;
+    }
+    v += (strided ? 6 : 0) + (plan.big ? 12 : 0);
+    static int smem_set[24][64] = {{0}};
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    const int v = (plan.c_static == 10 ? 0 : 1) + (strided ? 2 : 0);
+    cudaError_t e = kern != nullptr ? cudaGetDevice(&dev) : cudaErrorInvalidValue;
     if (e == cudaSuccess && (dev < 0 || dev >= 64 || smem_set[v][dev] < plan.smem_bytes)) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
         if (e == cudaSuccess && dev >= 0 && dev < 64) smem_set[v][dev] = plan.smem_bytes;

@@ -20,23 +20,22 @@ constexpr int kRQTileBytes = 128 * 128;
 // Keys per epilogue panel (half a tile) for a chunk size: a multiple of it, so that no chunk straddles panels.
 __host__ __device__ constexpr int panel_keys(int c) { return (c == 8 || c == 16 || c == 32) ? 64 : kRPanel; }
 
-// Chunk partial sums of a panel (SPP = panel_keys / c of them) to and from consecutive tensor-memory columns.
-template <int SPP>
-__device__ __forceinline__ void part_store(uint32_t taddr, const float (&p)[SPP]) {
-    static_assert(SPP == 12 || SPP == 8 || SPP == 6 || SPP == 4 || SPP == 3 || SPP == 2, "chunk slots per panel");
-    constexpr int X4 = SPP / 4 * 4, X2 = X4 + (SPP & 2);
+// A panel's chunk partial sums to and from consecutive tensor-memory columns.
+template <int N>
+__device__ __forceinline__ void part_store(uint32_t taddr, const float (&p)[N]) {
+    constexpr int X4 = N / 4 * 4, X2 = X4 + (N & 2);
 #pragma unroll
     for (int o = 0; o < X4; o += 4) tmem_st_x4(taddr + o, &p[o]);
-    if constexpr ((SPP & 2) != 0) tmem_st_x2(taddr + X4, &p[X4]);
-    if constexpr ((SPP & 1) != 0) tmem_st_x1(taddr + X2, &p[X2]);
+    if constexpr ((N & 2) != 0) tmem_st_x2(taddr + X4, &p[X4]);
+    if constexpr ((N & 1) != 0) tmem_st_x1(taddr + X2, &p[X2]);
 }
-template <int SPP>
+template <int N>
 __device__ __forceinline__ void part_load(uint32_t taddr, float* p) {
-    constexpr int X4 = SPP / 4 * 4, X2 = X4 + (SPP & 2);
+    constexpr int X4 = N / 4 * 4, X2 = X4 + (N & 2);
 #pragma unroll
     for (int o = 0; o < X4; o += 4) tmem_ld_x4(taddr + o, p + o);
-    if constexpr ((SPP & 2) != 0) tmem_ld_x2(taddr + X4, p + X4);
-    if constexpr ((SPP & 1) != 0) tmem_ld_x1(taddr + X2, p + X2);
+    if constexpr ((N & 2) != 0) tmem_ld_x2(taddr + X4, p + X4);
+    if constexpr ((N & 1) != 0) tmem_ld_x1(taddr + X2, p + X2);
 }
 
 // Sum of 32 values per lane over the 32 lanes of a warp, transposed: lane j returns the sum over

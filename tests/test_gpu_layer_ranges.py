@@ -60,3 +60,41 @@ def test_layer_and_chunk_scores(ck, Hq, Hkv, d, L, w, c):
     sK, sV, sidx = ck.compress_layer_strided(q, Kt, Vt, Hq, w, c, budget)
     assert np.array_equal(sidx.cpu().numpy(), idx) and torch.equal(sK, oK) and torch.equal(sV, oV)
 
+
+# a model call's CTA takes ceil(ceil(L / tile) / (144 / Hkv)) key tiles of every layer; its ring of partial sums continues in
+# scratch where a layer and eight panels more do not fit on chip, and always has both forms with two query tiles
+MODEL_CASES = [
+    (8, 2, 64, 2048, 16, 5, 3, 1), (28, 4, 128, 3000, 32, 10, 4, 2), (4, 4, 128, 1300, 32, 32, 5, 2),
+    (64, 16, 64, 9 * 120 * 11 + 7, 16, 5, 3, 2), (64, 16, 64, 9 * 128 * 18, 16, 8, 3, 1), (64, 16, 64, 9 * 120 * 23 - 50, 16, 10, 4, 1),
+    (128, 32, 64, 4 * 120 * 15 + 61, 64, 20, 4, 1), (128, 32, 64, 4 * 128 * 12, 64, 16, 3, 1), (64, 32, 128, 4 * 128 * 20, 128, 32, 2, 1),
+    (8, 2, 64, 600, 16, 10, 100, 98),                     # a reuse group longer than a launch
+]
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,L,w,c,n_layers,n_reuse", MODEL_CASES)
+def test_model_call(ck, Hq, Hkv, d, L, w, c, n_layers, n_reuse):
+    budget = w + c * max(1, (L - w) // (4 * c)) + 1
+    wl = scaled(CONFIGS[1], Hq=Hq, Hkv=Hkv, d=d, L=L, w=w, c=c, budget=budget, seed=950 + L, planted_count=2, sink_tokens=1)
+    xs = [make_layer(wl, layer=i) for i in range(min(n_layers, 5))]
+    pick = [min(i, 4) for i in range(n_layers)]
+    on = [(to_dev(x.q_obs), to_dev(x.K), to_dev(x.V)) for x in xs]
+    dev = [on[p] for p in pick]
+    guards = [guarded_outputs(Hkv, ck.out_len(L, w, c, budget), d) for _ in range(n_layers)]
+    for _ in range(2):                                    # the second call finds the counters and scratch of the first
+        outs = ck.compress_model(dev, Hq, w, c, budget, n_reuse, outs=[tuple(g.t for g in gs) for gs in guards])
+        assert ck.device_status() == 0
+    for gs in guards:
+        for g in gs:
+            g.check()
+    for l, (oK, oV, idx) in enumerate(outs):
+        x, src = xs[pick[l]], l // n_reuse * n_reuse
+        if l == src:
+            t = ora.token_scores(x.q_obs, x.K, Hq, Hkv, w)
+            assert_selection_matches(idx.cpu().numpy(), ora.chunk_scores(t, c), L, w, c, budget)
+        else:
+            assert torch.equal(idx, outs[src][2])
+        if l < 5 or l > n_layers - 3:
+            assert_gather_exact(bits_of(oK), bits_of(oV), idx.cpu().numpy(), x.K, x.V)
+    major = [(q, *(a.permute(1, 0, 2).contiguous().permute(1, 0, 2) for a in (K, V))) for q, K, V in on]
+    for a, b in zip(ck.compress_model_strided([major[p] for p in pick], Hq, w, c, budget, n_reuse), outs):
+        assert all(torch.equal(s, t) for s, t in zip(a, b))
