@@ -31,9 +31,9 @@
 //                 partial sums over the rows: chunk scores of its key range -> global memory
 //   4. hand-over  per KV head, until all of its chunk scores are there (bounded wait)
 //   5. select     every CTA of the head runs the same exact top-k over the head's chunk scores
-//                 and so holds the kept token positions in shared memory without a third wait;
-//                 one of them writes out_idx
-//   6. gather     the head's output rows are split evenly over its CTAs
+//                 and so holds the kept chunks in shared memory without a third wait
+//   6. gather     the head's output positions are split evenly over its CTAs: each expands its
+//                 share to token positions, writes them to out_idx and moves their rows
 //
 // Without out_idx the kernel ends after step 3 (chunk scores are the result).
 //
@@ -88,7 +88,8 @@ struct ResArgs {
     uint4* out_V;
     int32_t* out_idx;
     float* cta_stat;                   // [grid, n_mt, {max, sum}, 128]
-    float* scores;                     // [Hkv, C]
+    float* scores;                     // [Hkv, score_row]
+    int score_row;                     // C, or C rounded up to a multiple of 4 in scratch (16-byte aligned rows)
     float* spill;                      // [grid, n_off, 1 + chunk slots per panel, 128]: panel maximum, chunk sums
     unsigned* cnt_a;                   // [Hkv] hand-over 2, zero between launches
     unsigned* cnt_b;                   // [Hkv] hand-over 4
@@ -460,7 +461,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 const float* r = red + lc;
                 float t = (r[0] + r[n_local]) + (r[2 * n_local] + r[3 * n_local]);
                 if (two) t += (r[4 * n_local] + r[5 * n_local]) + (r[6 * n_local] + r[7 * n_local]);
-                a.scores[static_cast<size_t>(hkv) * a.C + ch0 + lc] = t;
+                a.scores[static_cast<size_t>(hkv) * a.score_row + ch0 + lc] = t;
             }
     }
     // ---- 4. wait for the KV head's other CTAs, 5. select, 6. gather
@@ -468,26 +469,35 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     if (ok && a.out_idx != nullptr) {
         SelectSmem& ss = *reinterpret_cast<SelectSmem*>(ring);
         constexpr size_t kSelBytes = (sizeof(SelectSmem) + 127) & ~size_t(127);
-        int32_t* sidx = reinterpret_cast<int32_t*>(ring + kSelBytes);          // [n_max] kept positions of the head
-        const float* sc = a.scores + static_cast<size_t>(hkv) * a.C;
-        if (a.C <= kRThreads * 6) {
-            select_head_regs<6>(sc, nullptr, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, sidx, ss, a.tok_cap);
-        } else {
-            const size_t idx_bytes = (static_cast<size_t>(a.n_max) * 4 + 127) & ~size_t(127);
-            uint32_t* kbuf = reinterpret_cast<uint32_t*>(ring + kSelBytes + idx_bytes);
-            const bool fits = kSelBytes + idx_bytes + static_cast<size_t>(a.C) * 4 <= static_cast<size_t>(a.ring_bytes);
-            if (fits)
-                select_head_smem(sc, nullptr, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, sidx, ss, kbuf, a.tok_cap);
-            else
-                select_head_rows(sc, nullptr, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, sidx, ss, nullptr, a.tok_cap);
-        }
+        const float* sc = a.scores + static_cast<size_t>(hkv) * a.score_row;
         const int Q = a.cph, q = part;                   // CTAs of this KV head
-        if (q == 0) {
-            int32_t* dst = a.out_idx + static_cast<size_t>(hkv) * a.n_max;
-            for (int n = threadIdx.x; n < a.n_max; n += kRThreads) dst[n] = sidx[n];
-        }
         const int r_begin = static_cast<int>(static_cast<long long>(a.n_max) * q / Q);
         const int r_end = static_cast<int>(static_cast<long long>(a.n_max) * (q + 1) / Q);
+        int32_t* sidx = reinterpret_cast<int32_t*>(ring + kSelBytes);          // kept positions [r_begin, r_end) of the head
+        int32_t* out_idx = a.out_idx + static_cast<size_t>(hkv) * a.n_max;
+        const size_t idx_bytes = (static_cast<size_t>(r_end - r_begin) * 4 + 127) & ~size_t(127);
+        uint32_t* kbuf = reinterpret_cast<uint32_t*>(ring + kSelBytes + idx_bytes);
+        const bool fits = kSelBytes + idx_bytes + static_cast<size_t>(a.C) * 4 <= static_cast<size_t>(a.ring_bytes);
+        if (min(a.k, a.C) <= kSelCap && a.C <= kSelMaxChunks && (fits || a.C <= kRThreads * 16)) {
+            if (a.C <= kRThreads * 8)
+                select_core<8>(sc, nullptr, a.C, a.k, ss, nullptr);
+            else if (a.C <= kRThreads * 16)
+                select_core<16>(sc, nullptr, a.C, a.k, ss, nullptr);
+            else
+                select_core<0>(sc, nullptr, a.C, a.k, ss, kbuf);
+            // every CTA holds the head's kept chunks: it expands, writes and gathers its own share of the positions
+            const int n_tok = select_tokens(a.P, C_STATIC, a.C, a.k, ss, a.tok_cap);
+            for (int n = r_begin + threadIdx.x; n < r_end; n += kRThreads) {
+                const int pos = select_position(ss, n, n_tok, C_STATIC, a.P, a.w);
+                sidx[n - r_begin] = pos;
+                out_idx[n] = pos;
+            }
+        } else {
+            // very many chunks: every CTA of the head writes the same positions to out_idx and takes its share from there
+            select_head_rows(sc, nullptr, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, out_idx, ss, fits ? kbuf : nullptr, a.tok_cap);
+            for (int n = r_begin + threadIdx.x; n < r_end; n += kRThreads) sidx[n - r_begin] = out_idx[n];
+        }
+        __syncthreads();
         const int vpr = a.d >> 3;
         const int rows_per_pass = (kRThreads / vpr) * kGatherRowsPerThread;
         // packed outputs: this head's block; paged outputs: the cache base (rows are placed through the block table)
@@ -496,11 +506,11 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         for (int n0 = r_begin; n0 < r_end; n0 += rows_per_pass) {
             if (vpr == 16)
                 gather_rows<16, false>(a.K + static_cast<size_t>(hkv) * a.k_head, a.V + static_cast<size_t>(hkv) * a.v_head,
-                                       sidx, a.L, r_end, n0, threadIdx.x, kRThreads, a.out_K + head_out * 16,
+                                       sidx - r_begin, a.L, r_end, n0, threadIdx.x, kRThreads, a.out_K + head_out * 16,
                                        a.out_V + head_out * 16, nullptr, a.k_row, a.v_row, pg);
             else
                 gather_rows<8, false>(a.K + static_cast<size_t>(hkv) * a.k_head, a.V + static_cast<size_t>(hkv) * a.v_head,
-                                      sidx, a.L, r_end, n0, threadIdx.x, kRThreads, a.out_K + head_out * 8,
+                                      sidx - r_begin, a.L, r_end, n0, threadIdx.x, kRThreads, a.out_K + head_out * 8,
                                       a.out_V + head_out * 8, nullptr, a.k_row, a.v_row, pg);
         }
     }
@@ -531,7 +541,7 @@ const void* kernel_of(bool big) {
 }  // namespace
 
 size_t resident_scratch_floats(const ResidentPlan& plan, int Hkv, int C) {
-    return static_cast<size_t>(plan.grid) * plan.n_mt * 256 + ((static_cast<size_t>(Hkv) * C + 63) & ~static_cast<size_t>(63)) +
+    return static_cast<size_t>(plan.grid) * plan.n_mt * 256 + ((static_cast<size_t>(Hkv) * ((C + 3) & ~3) + 63) & ~static_cast<size_t>(63)) +
            static_cast<size_t>(plan.grid) * plan.n_off * (plan.spp + 1) * 128;
 }
 
@@ -572,7 +582,8 @@ bool make_resident_plan(int L, int R, int Hkv, int d, int c, int C, int n_max, i
     p.smem_bytes = 1024 + p.off_misc + kRMiscBytes;
     // after scoring the ring holds the row sums of the chunk scores, then the selection scratch and the kept positions
     if (static_cast<size_t>(p.n_mt) * 4 * p.t_max * (tile / c) * 4 > static_cast<size_t>(p.ring_bytes)) return false;
-    const size_t sel_bytes = ((sizeof(SelectSmem) + 127) & ~size_t(127)) + ((static_cast<size_t>(n_max) * 4 + 127) & ~size_t(127));
+    const size_t own = static_cast<size_t>(n_max) / p.cph + 1;      // kept positions of a CTA
+    const size_t sel_bytes = ((sizeof(SelectSmem) + 127) & ~size_t(127)) + ((own * 4 + 127) & ~size_t(127));
     if (sel_bytes > static_cast<size_t>(p.ring_bytes)) return false;
     *plan = p;
     return true;
@@ -603,7 +614,8 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     a.cta_stat = io.scratch;
     float* scores = io.scratch + static_cast<size_t>(plan.grid) * plan.n_mt * 256;
     a.scores = io.out_scores ? io.out_scores : scores;
-    a.spill = scores + ((static_cast<size_t>(io.Hkv) * io.C + 63) & ~static_cast<size_t>(63));
+    a.score_row = io.out_scores ? io.C : (io.C + 3) & ~3;
+    a.spill = scores + ((static_cast<size_t>(io.Hkv) * ((io.C + 3) & ~3) + 63) & ~static_cast<size_t>(63));
     a.exits = io.counters;
     a.cnt_a = io.counters + 16;
     a.cnt_b = io.counters + 16 + kResidentMaxHeads;

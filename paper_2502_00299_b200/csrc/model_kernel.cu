@@ -225,12 +225,9 @@ template <int C_STATIC>
 __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn, int* flag_smem) {
     SelectSmem& ss = *reinterpret_cast<SelectSmem*>(dyn);
     constexpr size_t kSelBytes = (sizeof(SelectSmem) + 127) & ~size_t(127);
-    int32_t* sidx = reinterpret_cast<int32_t*>(dyn + kSelBytes);                  // [n_max] kept positions
-    const size_t idx_bytes = (static_cast<size_t>(p.n_max) * 4 + 127) & ~size_t(127);
-    uint32_t* kbuf = reinterpret_cast<uint32_t*>(dyn + kSelBytes + idx_bytes);    // keys, when there are many chunks per thread
+    uint32_t* kbuf = reinterpret_cast<uint32_t*>(dyn + kSelBytes);    // keys, when there are many chunks per thread
     const int sid = static_cast<int>(blockIdx.x) - p.n_score;
     const int kk = min(p.k, p.C);
-    const int tail_rows = (p.C > 0) ? (p.P - (p.C - 1) * C_STATIC) : 0;
     const int row_ints = p.sel_row_bytes / 4;
     volatile int* flag = flag_smem;
     for (int li = 0; li < p.n_layers;) {
@@ -249,28 +246,31 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
             const float* sc = p.scores + (static_cast<size_t>(s) * p.Hkv + hkv) * p.n_mt * p.Cpad;
             const float* sc2 = p.n_mt == 2 ? sc + p.Cpad : nullptr;
             if (p.C <= kMThreads * 8)
-                select_head_regs<8>(sc, sc2, p.L, p.w, C_STATIC, p.C, p.k, p.n_max, sidx, ss);
-            else {
-                if (p.sel_keys_fit)
-                    select_head_smem(sc, sc2, p.L, p.w, C_STATIC, p.C, p.k, p.n_max, sidx, ss, kbuf);
-                else
-                    select_head_rows(sc, sc2, p.L, p.w, C_STATIC, p.C, p.k, p.n_max, sidx, ss, nullptr);
-            }
-            const int n_tok = kk * C_STATIC - ((ss.last_kept && kk > 0) ? (C_STATIC - tail_rows) : 0);
+                select_core<8>(sc, sc2, p.C, p.k, ss, nullptr);
+            else if (p.C <= kMThreads * 16)
+                select_core<16>(sc, sc2, p.C, p.k, ss, nullptr);
+            else if (p.sel_keys_fit)
+                select_core<0>(sc, sc2, p.C, p.k, ss, kbuf);
+            else
+                select_head_rows(sc, sc2, p.L, p.w, C_STATIC, p.C, p.k, p.n_max, p.layer[li].out_idx + static_cast<size_t>(hkv) * p.n_max,
+                                 ss, nullptr);
+            const int n_tok = select_tokens(p.P, C_STATIC, p.C, p.k, ss);
             // the kept-chunk list for the copy threads: [n_tok, -, -, -, chunk ids]
             int* row = p.sel_rows + (static_cast<size_t>(s) * p.Hkv + hkv) * row_ints;
             if (threadIdx.x == 0) row[0] = n_tok;
             for (int r = threadIdx.x; r < kk; r += kMThreads) row[4 + r] = ss.sel[r];
             const int vpr = p.d >> 3;
-            for (int lj = li; lj < lj_end; ++lj) {
-                const ModelLayer& ly = p.layer[lj];
-                int32_t* dst = ly.out_idx + static_cast<size_t>(hkv) * p.n_max;
-                for (int n = threadIdx.x; n < p.n_max; n += kMThreads) dst[n] = sidx[n];
-                uint4* zk = ly.out_K + (static_cast<size_t>(hkv) * p.n_max + n_tok + p.w) * vpr;
-                uint4* zv = ly.out_V + (static_cast<size_t>(hkv) * p.n_max + n_tok + p.w) * vpr;
-                const int nz = (p.n_max - n_tok - p.w) * vpr;
-                for (int i = threadIdx.x; i < nz; i += kMThreads) { zk[i] = make_uint4(0, 0, 0, 0); zv[i] = make_uint4(0, 0, 0, 0); }
+            for (int n = threadIdx.x; n < p.n_max; n += kMThreads) {
+                const int pos = select_position(ss, n, n_tok, C_STATIC, p.P, p.w);
+                for (int lj = li; lj < lj_end; ++lj) p.layer[lj].out_idx[static_cast<size_t>(hkv) * p.n_max + n] = pos;
             }
+            const int nz = (p.n_max - n_tok - p.w) * vpr;
+            if (nz > 0)
+                for (int lj = li; lj < lj_end; ++lj) {
+                    uint4* zk = p.layer[lj].out_K + (static_cast<size_t>(hkv) * p.n_max + n_tok + p.w) * vpr;
+                    uint4* zv = p.layer[lj].out_V + (static_cast<size_t>(hkv) * p.n_max + n_tok + p.w) * vpr;
+                    for (int i = threadIdx.x; i < nz; i += kMThreads) { zk[i] = make_uint4(0, 0, 0, 0); zv[i] = make_uint4(0, 0, 0, 0); }
+                }
             __syncthreads();
             if (threadIdx.x == 0) {
                 unsigned old;   // release: the list and the positions written above are visible to whoever sees the count
@@ -884,7 +884,7 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_
     if (R < 1 || R > 256 || (d != 64 && d != 128) || L < 1 || C < 1 || k < 1 || Hkv < 1 || Hkv > kResidentMaxHeads)
         return false;
     const int kk = k < C ? k : C;
-    if (kk > kSelCap) return false;                          // the selector stages the kept chunk ids in shared memory
+    if (kk > kSelCap || C > kSelMaxChunks) return false;     // the selector stages the kept chunk ids in shared memory
     if (max_ctas < Hkv + 1) return false;
     ModelPlan p{};
     p.c_static = c;
@@ -929,9 +929,8 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_
     p.off_misc = p.off_pmax + pmax_bytes;
     p.off_tail = p.off_misc + kMMiscBytes;
     p.smem_bytes = 1024 + p.off_tail + tail_bytes;
-    // the selector CTAs use the same allocation for their scratch, the kept positions and (many chunks) the keys
-    const size_t n_max = static_cast<size_t>(kk) * c + 4096;      // (w <= 256 rows; generous)
-    const size_t sel_need = ((sizeof(SelectSmem) + 127) & ~size_t(127)) + ((n_max * 4 + 127) & ~size_t(127));
+    // the selector CTAs use the same allocation for their scratch and (many chunks) the keys
+    const size_t sel_need = (sizeof(SelectSmem) + 127) & ~size_t(127);
     if (sel_need + 1024 > static_cast<size_t>(p.smem_bytes)) return false;
     p.sel_keys_fit = (sel_need + static_cast<size_t>(C) * 4 + 1024 <= static_cast<size_t>(p.smem_bytes)) ? 1 : 0;
     *plan = p;

@@ -857,19 +857,20 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             const float* sc = la.chunk_scores + (static_cast<size_t>(h) << a.kv_shift) * la.C;
             const float* sc2 = a.kv_shift ? sc + la.C : nullptr;        // the head's second scoring head
             int32_t* out = la.out_idx + static_cast<size_t>(h) * la.n_max;
-            if (la.C <= kThreads * 6) {
-                select_head_regs<6>(sc, sc2, a.L, a.w, a.c, la.C, la.k, la.n_max, out, ss);
+            const bool sel_staged = min(la.k, la.C) <= kSelCap && la.C <= kSelMaxChunks;
+            if (sel_staged && la.C <= kThreads * 8) {
+                select_head<8>(sc, sc2, a.L, a.w, a.c, la.C, la.k, la.n_max, out, ss, nullptr);
             } else {
                 // keys go to the idle dynamic shared memory behind the selection scratch; if they do
                 // not fit there (token-level selection of very long sequences) they replace the
                 // chunk scores, which nothing reads after the selection
                 uint32_t* kbuf = reinterpret_cast<uint32_t*>(dyn + ((sizeof(SelectSmem) + 127) & ~size_t(127)));
                 const bool fits = static_cast<size_t>(la.C) * 4 + sizeof(SelectSmem) + 256 <= static_cast<size_t>(g.dyn_bytes);
-                if (fits)
-                    select_head_smem(sc, sc2, a.L, a.w, a.c, la.C, la.k, la.n_max, out, ss, kbuf);
+                if (fits && sel_staged)
+                    select_head<0>(sc, sc2, a.L, a.w, a.c, la.C, la.k, la.n_max, out, ss, kbuf);
                 else
                     select_head_rows(sc, sc2, a.L, a.w, a.c, la.C, la.k, la.n_max, out, ss,
-                                     reinterpret_cast<uint32_t*>(const_cast<float*>(sc)));
+                                     fits ? kbuf : reinterpret_cast<uint32_t*>(const_cast<float*>(sc)));
             }
         }
         if (rows_elsewhere) return;

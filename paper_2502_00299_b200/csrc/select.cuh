@@ -7,21 +7,19 @@
 // ties go to the lower chunk id. Token positions are written directly in ascending order: no
 // mask, no sort.
 //
-// select_head_regs (a few chunks per thread): each thread owns a contiguous run of chunk ids and
-// keeps their keys in registers; the threshold comes from an adaptive radix select (2048 equal
-// sub-intervals of [min key, max key], repeated on the sub-interval that holds the k-th largest
-// until few enough keys remain to rank directly). One block-wide prefix sum over the threads'
-// (#above, #equal) gives the ranks.
+// select_core (keys in registers or in shared memory): the threshold comes from an adaptive radix select (2048
+// equal sub-intervals of [min key, max key], repeated on the sub-interval that holds the k-th largest
+// until few enough keys remain to rank directly).
 //
-// select_head_rows (many chunks per thread, e.g. token-level selection of tens of thousands of
-// keys): unrolled code over registers would spill and spend its time fetching instructions that
-// run once, so this body is short rolled loops over a key buffer (shared memory where it fits).
-// Each warp owns a contiguous block of chunk ids and walks it in rows of 32 consecutive ids, one
-// per lane: accesses are coalesced and the order inside a row is the lane order. In the first
+// select_head_rows (keys nowhere or in a buffer of any kind; any number of kept chunks): 8 bits of the key at a time in
+// short rolled loops. In the first
 // pass every lane counts the four bins around the warp's first key in registers and the warp
 // adds its totals once; any other bin, and every bin of the later passes, takes one
-// shared-memory atomic per key. Ranks come from warp ballots plus one block-wide prefix sum
-// over the warps' (#above, #equal) totals.
+// shared-memory atomic per key.
+//
+// In both, each warp owns a contiguous block of chunk ids and walks it in rows of 32 consecutive ids, one
+// per lane: accesses are coalesced and the order inside a row is the lane order; ranks come from warp ballots plus the
+// warps' (#above, #equal) totals.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -29,11 +27,12 @@
 namespace chunkkv {
 
 constexpr int kSelMaxWarps = 32;
-constexpr int kSelCap = 4096;         // kept-chunk ids staged for coalesced index writes
+constexpr int kSelCap = 8192;         // kept-chunk ids staged for coalesced index writes (16 bits each)
+constexpr int kSelMaxChunks = 65535;  // most chunks of a head for which ids are staged
 
 struct SelectSmem {
-    unsigned short whist[kSelMaxWarps][256];
-    int sel[kSelCap];
+    alignas(16) unsigned short whist[kSelMaxWarps][256];
+    alignas(16) unsigned short sel[kSelCap];
     int hist[256];
     unsigned long long warp_sums[kSelMaxWarps + 1];
     int warp_tot[kSelMaxWarps];
@@ -41,6 +40,7 @@ struct SelectSmem {
     int need;
     int bin_count;
     int n_cand;
+    int need_eq;
     int last_kept;
 };
 
@@ -49,9 +49,11 @@ __device__ __forceinline__ uint32_t select_order_key(float x) {
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);     // larger float <=> larger key
 }
 
-// Selection for a few chunks per thread. All threads of the CTA must call this (it uses
-// __syncthreads); blockDim.x must be a multiple of 32, at least 512 and at most 1024. Every thread
-// keeps up to KPT keys in registers, which needs C <= blockDim.x * KPT.
+// The one-CTA selection proper: leaves the ids of the kept chunks in ascending order in sm.sel (kk = min(k, C) of
+// them; kk <= kSelCap, C <= kSelMaxChunks) and sm.last_kept. All threads of the CTA must call this (it uses __syncthreads);
+// blockDim.x must be a multiple of 32, at least 512 and at most 1024.
+// KPT > 0: every thread keeps up to KPT keys in registers, which needs C <= blockDim.x * KPT and kbuf is not used.
+// KPT = 0: the keys live in kbuf (shared memory, room for C).
 // sc2 != NULL: the head's scores are sc[ch] + sc2[ch] (a KV head scored as two heads of half the rows).
 //
 // The k-th largest key is found by an adaptive radix select: the keys of interest always lie in a
@@ -61,55 +63,103 @@ __device__ __forceinline__ uint32_t select_order_key(float x) {
 // keys) already leaves a handful of candidates; as soon as at most kSelCandCap keys remain they are
 // ranked against each other directly. Ties and degenerate inputs (all keys equal) end with
 // span = 0, i.e. a single key value. Exact for any input.
+//
+// What bounds it is a chain of latencies - about ten block-wide steps on a few thousand keys - and, inside the steps,
+// instructions that a quarter of the lanes execute at a time (population counts, shared atomics). Keys in registers: a
+// thread owns a run of KPT or fewer consecutive ids, loaded 16 bytes at a time where the scores are aligned, so that the
+// order inside a warp is one packed prefix sum over its lanes and the list is written without branches. Keys in shared
+// memory: warp v owns a block of consecutive ids and walks it in rows of 32, one id per lane, with ballots for the order.
+// Totals of warps are combined by one shared-memory read per lane and a warp reduction.
+// 3274 keys, 640 threads, in clocks: 11.2k with scalar loads (2.2k), a loop over the warps for the minimum and maximum
+// (1.1k) and branches per key for the candidates (1.2k) and the list (2.1k); about 6.5k in this form.
 constexpr int kSelBins = 2048;
-constexpr int kSelCandCap = 1024;
+constexpr int kSelCandCap = 128;
 
 template <int KPT>
-__device__ __forceinline__ void select_head_regs(const float* sc, const float* sc2, int L, int w, int c,
-                                            int C, int k, int n_max, int32_t* out, SelectSmem& sm,
-                                            int tok_cap = 0x7fffffff) {
-    static_assert(KPT > 0, "keys live in registers");
+__device__ __forceinline__ void select_core(const float* sc, const float* sc2, int C, int k, SelectSmem& sm, uint32_t* kbuf) {
     constexpr unsigned kFull = 0xffffffffu;
-    auto score_at = [&](int ch) { return sc2 != nullptr ? __ldcg(sc + ch) + __ldcg(sc2 + ch) : __ldcg(sc + ch); };
-    const int P = L - w;
+    constexpr bool REGS = KPT > 0;
+    constexpr int UN = REGS ? KPT : 4;                       // unrolling of the loops over a warp's rows
     const int nt = blockDim.x, nwarps = nt >> 5;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool keep_all = (k >= C);
     const int kk = min(k, C);
+    // registers: thread t owns the ids [t per, (t + 1) per); shared memory: lane l of warp v the ids id0 + 32 u, u < per
+    const int per = REGS ? 4 * ((C + 4 * nt - 1) / (4 * nt)) : (C + nt - 1) / nt;
+    const int rows = REGS ? KPT : per;
+    const int id0 = REGS ? tid * per : warp * per * 32 + lane;
+    const int own = REGS ? max(0, min(per, C - id0)) : 0;    // ids of this thread
+    uint32_t keys[REGS ? KPT : 1];
+    auto have = [&](int u) { return REGS ? u < own : (u < per && id0 + 32 * u < C); };
+    auto key_at = [&](int u) -> uint32_t { return REGS ? keys[REGS ? u : 0] : kbuf[id0 + 32 * u]; };
 
-    // thread t owns chunk ids [c0, c1)
-    const int per = (C + nt - 1) / nt;
-    const int c0 = min(tid * per, C), c1 = min(c0 + per, C);
-    uint32_t keys[KPT];
-    if (kk > 0 && !keep_all) {
-#pragma unroll
-        for (int u = 0; u < KPT; ++u) keys[u] = (c0 + u < c1) ? select_order_key(score_at(c0 + u)) : 0u;
-    }
-    if (tid == 0) sm.last_kept = 0;
-
+    if (tid == 0) { sm.last_kept = 0; sm.n_cand = 0; }
     uint32_t thresh = 0;   // key of the k-th largest score
     int need_eq = 0;       // how many chunks equal to the threshold are kept
     if (!keep_all && kk > 0) {
         int* hist = reinterpret_cast<int*>(&sm.whist[0][0]);            // kSelBins counters
         uint32_t* cand = reinterpret_cast<uint32_t*>(&sm.sel[0]);       // kSelCandCap keys (sel is written later)
-        // smallest and largest key of the head
         uint32_t lo = 0xffffffffu, hi = 0u;
+        if constexpr (REGS) {
+            float v[KPT];                                    // (all loads before the first use)
+            const bool vec = ((reinterpret_cast<uintptr_t>(sc) | reinterpret_cast<uintptr_t>(sc2)) & 15u) == 0 && own == KPT;
+            if (vec) {
 #pragma unroll
-        for (int u = 0; u < KPT; ++u)
-            if (c0 + u < c1) { lo = min(lo, keys[u]); hi = max(hi, keys[u]); }
+                for (int u = 0; u < KPT; u += 4) {
+                    const float4 f = __ldcg(reinterpret_cast<const float4*>(sc + id0 + u));
+                    v[u] = f.x; v[u + 1] = f.y; v[u + 2] = f.z; v[u + 3] = f.w;
+                }
+                if (sc2 != nullptr) {
+#pragma unroll
+                    for (int u = 0; u < KPT; u += 4) {
+                        const float4 f = __ldcg(reinterpret_cast<const float4*>(sc2 + id0 + u));
+                        v[u] += f.x; v[u + 1] += f.y; v[u + 2] += f.z; v[u + 3] += f.w;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < KPT; ++u) v[u] = have(u) ? __ldcg(sc + id0 + u) : 0.f;
+                if (sc2 != nullptr) {
+#pragma unroll
+                    for (int u = 0; u < KPT; ++u) v[u] += have(u) ? __ldcg(sc2 + id0 + u) : 0.f;
+                }
+            }
+            for (int i = tid; i < kSelBins; i += nt) hist[i] = 0;
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) {
+                keys[u] = select_order_key(v[u]);
+                if (have(u)) { lo = min(lo, keys[u]); hi = max(hi, keys[u]); }
+            }
+        } else {
+            for (int i = tid; i < kSelBins; i += nt) hist[i] = 0;
+            constexpr int kB = 16;                           // loads in flight per thread
+#pragma unroll 1
+            for (int u0 = 0; u0 < rows; u0 += kB) {
+                float v[kB];
+#pragma unroll
+                for (int q = 0; q < kB; ++q) v[q] = __ldcg(sc + min(id0 + 32 * min(u0 + q, rows - 1), C - 1));
+                if (sc2 != nullptr) {
+#pragma unroll
+                    for (int q = 0; q < kB; ++q) v[q] += __ldcg(sc2 + min(id0 + 32 * min(u0 + q, rows - 1), C - 1));
+                }
+#pragma unroll
+                for (int q = 0; q < kB; ++q)
+                    if (have(u0 + q)) {
+                        const uint32_t key = select_order_key(v[q]);
+                        kbuf[id0 + 32 * (u0 + q)] = key;     // (read back by this thread only)
+                        lo = min(lo, key);
+                        hi = max(hi, key);
+                    }
+            }
+        }
         lo = __reduce_min_sync(kFull, lo);
         hi = __reduce_max_sync(kFull, hi);
         if (lane == 0) sm.warp_sums[warp] = (static_cast<unsigned long long>(hi) << 32) | lo;
-        for (int i = tid; i < kSelBins; i += nt) hist[i] = 0;
-        if (tid == 0) sm.n_cand = 0;
         __syncthreads();
-        uint32_t base = 0xffffffffu, top = 0u;
-        for (int wv = 0; wv < nwarps; ++wv) {
-            const unsigned long long v = sm.warp_sums[wv];
-            base = min(base, static_cast<uint32_t>(v));
-            top = max(top, static_cast<uint32_t>(v >> 32));
-        }
-        uint32_t span = top - base;          // the keys of interest lie in [base, base + span]
+        // smallest and largest key of the head
+        const unsigned long long mm = sm.warp_sums[lane < nwarps ? lane : 0];
+        uint32_t base = __reduce_min_sync(kFull, static_cast<uint32_t>(mm));
+        uint32_t span = __reduce_max_sync(kFull, static_cast<uint32_t>(mm >> 32)) - base;   // the keys of interest lie in [base, base + span]
         int need = k;                        // the need-th largest of them is the threshold
         for (int round = 0;; ++round) {
             if (span == 0u) { thresh = base; need_eq = need; break; }
@@ -118,18 +168,20 @@ __device__ __forceinline__ void select_head_regs(const float* sc, const float* s
                 for (int i = tid; i < kSelBins; i += nt) hist[i] = 0;
                 __syncthreads();
             }
-#pragma unroll
-            for (int u = 0; u < KPT; ++u) {
-                const uint32_t dlt = keys[u] - base;
-                if (c0 + u < c1 && keys[u] >= base && dlt <= span) atomicAdd(&hist[dlt >> shift], 1);
-            }
+#pragma unroll UN
+            for (int u = 0; u < rows; ++u)
+                if (have(u)) {
+                    const uint32_t dlt = key_at(u) - base;   // (a key below base wraps to more than span: base + span is a key's value)
+                    if (dlt <= span) atomicAdd(&hist[dlt >> shift], 1);
+                }
             __syncthreads();
             // thread t < 512 owns bins 2047 - 4t .. 2044 - 4t, so a prefix over threads counts from the top
-            int cnt[4] = {0, 0, 0, 0}, sum = 0;
+            int cnt[4] = {0, 0, 0, 0};
             if (tid < kSelBins / 4) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) { cnt[q] = hist[kSelBins - 1 - 4 * tid - q]; sum += cnt[q]; }
+                const int4 b4 = *reinterpret_cast<const int4*>(hist + kSelBins - 4 - 4 * tid);
+                cnt[0] = b4.w; cnt[1] = b4.z; cnt[2] = b4.y; cnt[3] = b4.x;
             }
+            const int sum = (cnt[0] + cnt[1]) + (cnt[2] + cnt[3]);
             int inc = sum;
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
@@ -138,9 +190,7 @@ __device__ __forceinline__ void select_head_regs(const float* sc, const float* s
             }
             if (lane == 31) sm.warp_tot[warp] = inc;
             __syncthreads();
-            int before = 0;
-            for (int wv = 0; wv < warp; ++wv) before += sm.warp_tot[wv];
-            inc += before;
+            inc += __reduce_add_sync(kFull, lane < warp ? sm.warp_tot[lane] : 0);
             if (tid < kSelBins / 4 && inc - sum < need && need <= inc) {     // exactly one thread
                 int above = inc - sum, q = 0, cq = cnt[0];
 #pragma unroll
@@ -155,293 +205,125 @@ __device__ __forceinline__ void select_head_regs(const float* sc, const float* s
             const int n_bin = sm.bin_count;
             need = sm.need;
             const uint32_t sub = bin << shift;
-            const uint32_t width = (shift >= 32) ? 0xffffffffu : ((1u << shift) - 1u);
-            base += sub;
-            span = min(width, span - sub);
-            if (n_bin <= kSelCandCap) {
-                // few keys left: rank them against each other
-#pragma unroll
-                for (int u = 0; u < KPT; ++u) {
-                    const uint32_t dlt = keys[u] - base;
-                    if (c0 + u < c1 && keys[u] >= base && dlt <= span) cand[atomicAdd(&sm.n_cand, 1)] = keys[u];
-                }
-                __syncthreads();
-                for (int j = tid; j < n_bin; j += nt) {
-                    const uint32_t v = cand[j];
-                    int gt = 0, ge = 0;
-                    for (int i = 0; i < n_bin; ++i) { gt += cand[i] > v; ge += cand[i] >= v; }
-                    if (gt < need && need <= ge) { sm.prefix = v; sm.need = need - gt; }   // same values from every writer
-                }
-                __syncthreads();
-                thresh = sm.prefix;
-                need_eq = sm.need;
-                break;
-            }
-        }
-        __syncthreads();       // cand (= sel) and the shared words are reused below
-    }
-
-    // Ordered sweep over the chunk ids.
-    const bool stage_sel = kk <= kSelCap;
-    if (kk > 0) {
-        unsigned gt_n = 0, eq_n = 0;
-        if (keep_all) gt_n = c1 - c0;
-        else {
-#pragma unroll
-            for (int u = 0; u < KPT; ++u)
-                if (c0 + u < c1) { gt_n += keys[u] > thresh; eq_n += keys[u] == thresh; }
-        }
-        // block-wide exclusive prefix of the packed pair (eq in the high half, gt in the low half)
-        const unsigned long long mine = (static_cast<unsigned long long>(eq_n) << 32) | gt_n;
-        unsigned long long inc = mine;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const unsigned long long n = __shfl_up_sync(kFull, inc, off);
-            if (lane >= off) inc += n;
-        }
-        if (lane == 31) sm.warp_sums[warp] = inc;
-        __syncthreads();
-        if (warp == 0) {
-            const unsigned long long s = (lane < nwarps) ? sm.warp_sums[lane] : 0ull;
-            unsigned long long sinc = s;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const unsigned long long n = __shfl_up_sync(kFull, sinc, off);
-                if (lane >= off) sinc += n;
-            }
-            sm.warp_sums[lane] = sinc - s;
-        }
-        __syncthreads();
-        const unsigned long long excl = sm.warp_sums[warp] + inc - mine;
-        int gt_before = static_cast<int>(excl & 0xffffffffu), eq_before = static_cast<int>(excl >> 32);
-        auto visit = [&](int ch, uint32_t key) {
-            const bool gt = keep_all || key > thresh;
-            const bool eq = !keep_all && key == thresh;
-            if (gt || (eq && eq_before < need_eq)) {
-                const int rank = gt_before + min(eq_before, need_eq);
-                if (stage_sel) sm.sel[rank] = ch;
-                else {
-                    const int j0 = ch * c, len = min(c, P - j0);
-                    int32_t* dst = out + static_cast<size_t>(rank) * c;
-                    for (int t = 0; t < len; ++t)
-                        if (rank * c + t < tok_cap) dst[t] = j0 + t;
-                }
-                if (ch == C - 1) sm.last_kept = 1;
-            }
-            gt_before += gt;
-            eq_before += eq;
-        };
-        if (!keep_all) {
-#pragma unroll
-            for (int u = 0; u < KPT; ++u)
-                if (c0 + u < c1) visit(c0 + u, keys[u]);
-        } else {
-            for (int ch = c0; ch < c1; ++ch) visit(ch, 0u);
-        }
-    }
-    __syncthreads();
-    // Every kept chunk is full except possibly chunk C-1, which can only be the last kept one.
-    const int tail = (C > 0) ? (P - (C - 1) * c) : 0;
-    // tok_cap: at most this many tokens of the kept chunks are emitted, lowest positions first
-    // (Algorithm 1 keeps the first L_max - w selected tokens); no cap by default
-    const int n_tok = min(kk * c - ((sm.last_kept && kk > 0) ? (c - tail) : 0), tok_cap);
-    if (stage_sel)
-        for (int r = tid; r < kk; r += nt) {            // one kept chunk per thread: its c positions
-            const int j0 = sm.sel[r] * c, n0 = r * c;
-            for (int t = 0; t < c; ++t)
-                if (n0 + t < n_tok) out[n0 + t] = j0 + t;
-        }
-    for (int i = tid; i < w; i += nt) out[n_tok + i] = P + i;
-    for (int i = n_tok + w + tid; i < n_max; i += nt) out[i] = -1;
-    __syncthreads();     // shared state may be reused by the caller
-}
-
-// The same selection with the keys of the head in a shared-memory buffer (kbuf, room for C keys)
-// instead of registers: for heads with many chunks per thread (token-level selection: tens of
-// thousands of keys). Same adaptive radix select and ordered sweep as select_head_regs; the passes
-// over the keys are strided loops (coalesced, conflict-free), the sweep walks thread-contiguous runs.
-// All threads of the CTA must call it; blockDim.x a multiple of 32, at least 512, at most 1024.
-__device__ __forceinline__ void select_head_smem(const float* sc, const float* sc2, int L, int w, int c, int C, int k,
-                                                 int n_max, int32_t* out, SelectSmem& sm, uint32_t* kbuf,
-                                                 int tok_cap = 0x7fffffff) {
-    constexpr unsigned kFull = 0xffffffffu;
-    const int P = L - w;
-    const int nt = blockDim.x, nwarps = nt >> 5;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool keep_all = (k >= C);
-    const int kk = min(k, C);
-    if (tid == 0) sm.last_kept = 0;
-    uint32_t thresh = 0;
-    int need_eq = 0;
-    if (!keep_all && kk > 0) {
-        int* hist = reinterpret_cast<int*>(&sm.whist[0][0]);
-        uint32_t* cand = reinterpret_cast<uint32_t*>(&sm.sel[0]);
-        uint32_t lo = 0xffffffffu, hi = 0u;
-        constexpr int kB = 16;                             // loads in flight per thread
-#pragma unroll 1
-        for (int ch0 = tid; ch0 < C; ch0 += kB * nt) {
-            float v[kB];
-#pragma unroll
-            for (int q = 0; q < kB; ++q) v[q] = __ldcg(sc + min(ch0 + q * nt, C - 1));
-            if (sc2 != nullptr) {
-#pragma unroll
-                for (int q = 0; q < kB; ++q) v[q] += __ldcg(sc2 + min(ch0 + q * nt, C - 1));
-            }
-#pragma unroll
-            for (int q = 0; q < kB; ++q)
-                if (ch0 + q * nt < C) {
-                    const uint32_t key = select_order_key(v[q]);
-                    kbuf[ch0 + q * nt] = key;
-                    lo = min(lo, key);
-                    hi = max(hi, key);
-                }
-        }
-        lo = __reduce_min_sync(kFull, lo);
-        hi = __reduce_max_sync(kFull, hi);
-        if (lane == 0) sm.warp_sums[warp] = (static_cast<unsigned long long>(hi) << 32) | lo;
-        for (int i = tid; i < kSelBins; i += nt) hist[i] = 0;
-        if (tid == 0) sm.n_cand = 0;
-        __syncthreads();
-        uint32_t base = 0xffffffffu, top = 0u;
-        for (int wv = 0; wv < nwarps; ++wv) {
-            const unsigned long long v = sm.warp_sums[wv];
-            base = min(base, static_cast<uint32_t>(v));
-            top = max(top, static_cast<uint32_t>(v >> 32));
-        }
-        uint32_t span = top - base;
-        int need = k;
-        for (int round = 0;; ++round) {
-            if (span == 0u) { thresh = base; need_eq = need; break; }
-            const int shift = max(0, 21 - __clz(span));
-            if (round > 0) {
-                for (int i = tid; i < kSelBins; i += nt) hist[i] = 0;
-                __syncthreads();
-            }
-#pragma unroll 4
-            for (int ch = tid; ch < C; ch += nt) {
-                const uint32_t key = kbuf[ch], dlt = key - base;
-                if (key >= base && dlt <= span) atomicAdd(&hist[dlt >> shift], 1);
-            }
-            __syncthreads();
-            int cnt[4] = {0, 0, 0, 0}, sum = 0;
-            if (tid < kSelBins / 4) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) { cnt[q] = hist[kSelBins - 1 - 4 * tid - q]; sum += cnt[q]; }
-            }
-            int inc = sum;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int n = __shfl_up_sync(kFull, inc, off);
-                if (lane >= off) inc += n;
-            }
-            if (lane == 31) sm.warp_tot[warp] = inc;
-            __syncthreads();
-            int before = 0;
-            for (int wv = 0; wv < warp; ++wv) before += sm.warp_tot[wv];
-            inc += before;
-            if (tid < kSelBins / 4 && inc - sum < need && need <= inc) {
-                int above = inc - sum, q = 0, cq = cnt[0];
-#pragma unroll
-                for (int t = 0; t < 3; ++t)
-                    if (q == t && above + cnt[t] < need) { above += cnt[t]; q = t + 1; cq = cnt[t + 1]; }
-                sm.prefix = static_cast<uint32_t>(kSelBins - 1 - 4 * tid - q);
-                sm.need = need - above;
-                sm.bin_count = cq;
-            }
-            __syncthreads();
-            const uint32_t bin = sm.prefix;
-            const int n_bin = sm.bin_count;
-            need = sm.need;
-            const uint32_t sub = bin << shift;
             base += sub;
             span = min((1u << shift) - 1u, span - sub);
             if (n_bin <= kSelCandCap) {
+                // few keys left: rank them against each other
+                if constexpr (REGS) {
+                    unsigned hits = 0;
+#pragma unroll
+                    for (int u = 0; u < KPT; ++u) hits |= (have(u) && keys[u] - base <= span) ? 1u << u : 0u;
+                    if (hits != 0) {
+                        int at = atomicAdd(&sm.n_cand, __popc(hits));
+#pragma unroll
+                        for (int u = 0; u < KPT; ++u)
+                            if (hits >> u & 1u) cand[at++] = keys[u];
+                    }
+                } else {
 #pragma unroll 4
-                for (int ch = tid; ch < C; ch += nt) {
-                    const uint32_t key = kbuf[ch], dlt = key - base;
-                    if (key >= base && dlt <= span) cand[atomicAdd(&sm.n_cand, 1)] = key;
+                    for (int u = 0; u < rows; ++u)
+                        if (have(u) && key_at(u) - base <= span) cand[atomicAdd(&sm.n_cand, 1)] = key_at(u);
                 }
                 __syncthreads();
-                for (int j = tid; j < n_bin; j += nt) {
-                    const uint32_t v = cand[j];
+                if (tid < n_bin) {
+                    const uint32_t v = cand[tid];
                     int gt = 0, ge = 0;
-                    for (int i = 0; i < n_bin; ++i) { gt += cand[i] > v; ge += cand[i] >= v; }
-                    if (gt < need && need <= ge) { sm.prefix = v; sm.need = need - gt; }
+#pragma unroll 8
+                    for (int i = 0; i < n_bin; ++i) { const uint32_t x = cand[i]; gt += x > v; ge += x >= v; }
+                    if (gt < need && need <= ge) { sm.prefix = v; sm.need_eq = need - gt; }   // same values from every writer
                 }
                 __syncthreads();
                 thresh = sm.prefix;
-                need_eq = sm.need;
+                need_eq = sm.need_eq;
                 break;
             }
         }
-        __syncthreads();
     }
-    // ordered sweep: warp v owns the contiguous ids [v * rows * 32, (v + 1) * rows * 32) and walks them in
-    // rows of 32 consecutive ids, one per lane; ballots give a row's (#above, #equal) in lane order
-    const bool stage_sel = kk <= kSelCap;
-    if (kk > 0) {
+
+    // Ordered sweep over the chunk ids: a kept chunk's rank is the number of kept ones before it, (#above) + min(#equal,
+    // ties to keep). (#equal << 16 | #above) of a thread or warp fits 32 bits, and so do the totals: fewer than k keys lie
+    // above the threshold, C <= kSelMaxChunks.
+    if (kk > 0 && keep_all) {
+        for (int ch = tid; ch < C; ch += nt) sm.sel[ch] = static_cast<unsigned short>(ch);
+        if (tid == 0) sm.last_kept = 1;
+    } else if (kk > 0 && REGS) {
+        unsigned mine = 0;
+#pragma unroll
+        for (int u = 0; u < KPT; ++u) mine += have(u) ? (keys[u] > thresh ? 1u : (keys[u] == thresh ? 0x10000u : 0u)) : 0u;
+        unsigned inc = mine;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const unsigned n = __shfl_up_sync(kFull, inc, off);
+            if (lane >= off) inc += n;
+        }
+        if (lane == 31) sm.warp_tot[warp] = static_cast<int>(inc);
+        __syncthreads();                 // (also: cand, which shares its words with sel, is no longer read)
+        inc += __reduce_add_sync(kFull, lane < warp ? static_cast<unsigned>(sm.warp_tot[lane]) : 0u) - mine;
+        int eq_before = static_cast<int>(inc >> 16);
+        int rank = static_cast<int>(inc & 0xffffu) + min(eq_before, need_eq);
+#pragma unroll
+        for (int u = 0; u < KPT; ++u) {
+            const bool eq = have(u) && keys[u] == thresh;
+            const bool kept = have(u) && (keys[u] > thresh || (eq && eq_before < need_eq));
+            if (kept) sm.sel[rank] = static_cast<unsigned short>(id0 + u);
+            if (kept && id0 + u == C - 1) sm.last_kept = 1;
+            rank += kept;
+            eq_before += eq;
+        }
+    } else if (kk > 0) {
         const unsigned lt_mask = (1u << lane) - 1u;
-        const int rows = (C + nt - 1) / nt;
-        const int base_id = warp * rows * 32 + lane;
         unsigned gt_n = 0, eq_n = 0;
 #pragma unroll 4
         for (int u = 0; u < rows; ++u) {
-            const int ch = base_id + 32 * u;
-            const uint32_t key = (ch < C && !keep_all) ? kbuf[ch] : 0u;
-            gt_n += __popc(__ballot_sync(kFull, ch < C && (keep_all || key > thresh)));
-            eq_n += __popc(__ballot_sync(kFull, ch < C && !keep_all && key == thresh));
+            const uint32_t key = have(u) ? key_at(u) : 0u;
+            gt_n += __popc(__ballot_sync(kFull, have(u) && key > thresh));
+            eq_n += __popc(__ballot_sync(kFull, have(u) && key == thresh));
         }
-        if (lane == 0) sm.warp_sums[warp] = (static_cast<unsigned long long>(eq_n) << 32) | gt_n;
-        __syncthreads();
-        if (warp == 0) {
-            const unsigned long long s = (lane < nwarps) ? sm.warp_sums[lane] : 0ull;
-            unsigned long long sinc = s;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const unsigned long long n = __shfl_up_sync(kFull, sinc, off);
-                if (lane >= off) sinc += n;
-            }
-            sm.warp_sums[lane] = sinc - s;
-        }
-        __syncthreads();
-        const unsigned long long excl = sm.warp_sums[warp];
-        int gt_run = static_cast<int>(excl & 0xffffffffu), eq_run = static_cast<int>(excl >> 32);
-#pragma unroll 2
+        if (lane == 0) sm.warp_tot[warp] = static_cast<int>(eq_n << 16 | gt_n);
+        __syncthreads();                 // (also: cand, which shares its words with sel, is no longer read)
+        const unsigned tot = __reduce_add_sync(kFull, lane < warp ? static_cast<unsigned>(sm.warp_tot[lane]) : 0u);
+        unsigned gt_run = tot & 0xffffu, eq_run = tot >> 16;
+#pragma unroll 4
         for (int u = 0; u < rows; ++u) {
-            const int ch = base_id + 32 * u;
-            const uint32_t key = (ch < C && !keep_all) ? kbuf[ch] : 0u;
-            const bool gt = ch < C && (keep_all || key > thresh);
-            const bool eq = ch < C && !keep_all && key == thresh;
+            const uint32_t key = have(u) ? key_at(u) : 0u;
+            const bool gt = have(u) && key > thresh, eq = have(u) && key == thresh;
             const unsigned gtm = __ballot_sync(kFull, gt), eqm = __ballot_sync(kFull, eq);
             const int gt_before = gt_run + __popc(gtm & lt_mask);
-            const int eq_before = eq_run + __popc(eqm & lt_mask);
+            const int eq_before = eq_run + (eqm ? __popc(eqm & lt_mask) : 0);
             if (gt || (eq && eq_before < need_eq)) {
-                const int rank = gt_before + min(eq_before, need_eq);
-                if (stage_sel) sm.sel[rank] = ch;
-                else {
-                    const int j0 = ch * c, len = min(c, P - j0);
-                    int32_t* dst = out + static_cast<size_t>(rank) * c;
-                    for (int t = 0; t < len; ++t)
-                        if (rank * c + t < tok_cap) dst[t] = j0 + t;
-                }
-                if (ch == C - 1) sm.last_kept = 1;
+                sm.sel[gt_before + min(eq_before, need_eq)] = static_cast<unsigned short>(id0 + 32 * u);
+                if (id0 + 32 * u == C - 1) sm.last_kept = 1;
             }
             gt_run += __popc(gtm);
-            eq_run += __popc(eqm);
+            eq_run += eqm ? __popc(eqm) : 0;
         }
     }
     __syncthreads();
+}
+
+// Tokens of the kept chunks that are emitted: every kept chunk is full except possibly chunk C - 1, which can only be
+// the last kept one. tok_cap: at most this many, lowest positions first (Algorithm 1 keeps the first L_max - w
+// selected tokens); no cap by default.
+__device__ __forceinline__ int select_tokens(int P, int c, int C, int k, const SelectSmem& sm, int tok_cap = 0x7fffffff) {
+    const int kk = min(k, C);
     const int tail = (C > 0) ? (P - (C - 1) * c) : 0;
-    const int n_tok = min(kk * c - ((sm.last_kept && kk > 0) ? (c - tail) : 0), tok_cap);
-    if (stage_sel)
-        for (int r = tid; r < kk; r += nt) {
-            const int j0 = sm.sel[r] * c, n0 = r * c;
-            for (int t = 0; t < c; ++t)
-                if (n0 + t < n_tok) out[n0 + t] = j0 + t;
-        }
-    for (int i = tid; i < w; i += nt) out[n_tok + i] = P + i;
-    for (int i = n_tok + w + tid; i < n_max; i += nt) out[i] = -1;
-    __syncthreads();
+    return min(kk * c - ((sm.last_kept && kk > 0) ? (c - tail) : 0), tok_cap);
+}
+
+// Kept position n of [0, n_max): tokens of the kept chunks ascending, then the window, then -1.
+__device__ __forceinline__ int select_position(const SelectSmem& sm, int n, int n_tok, int c, int P, int w) {
+    if (n < n_tok) { const int r = n / c; return sm.sel[r] * c + (n - r * c); }
+    return n < n_tok + w ? P + (n - n_tok) : -1;
+}
+
+// The whole selection of a head into out[n_max], keys in registers (KPT > 0) or in kbuf; conditions as select_core.
+template <int KPT>
+__device__ __forceinline__ void select_head(const float* sc, const float* sc2, int L, int w, int c, int C, int k, int n_max,
+                                            int32_t* out, SelectSmem& sm, uint32_t* kbuf, int tok_cap = 0x7fffffff) {
+    select_core<KPT>(sc, sc2, C, k, sm, kbuf);
+    const int P = L - w, n_tok = select_tokens(P, c, C, k, sm, tok_cap);
+    for (int n = threadIdx.x; n < n_max; n += blockDim.x) out[n] = select_position(sm, n, n_tok, c, P, w);
+    __syncthreads();     // shared state may be reused by the caller
 }
 
 // Selection for many chunks per thread. All threads of the CTA must call this (it uses
@@ -567,7 +449,7 @@ __device__ __forceinline__ void select_head_rows(const float* sc, const float* s
     }
 
     // Ordered sweep over the chunk ids: ballots give a row's (#above, #equal) in lane order.
-    const bool stage_sel = kk <= kSelCap;
+    const bool stage_sel = kk <= kSelCap && C <= kSelMaxChunks;
     if (kk > 0) {
         auto row_flags = [&](int ch, unsigned& gtm, unsigned& eqm, bool& gt, bool& eq) {
             const bool valid = ch < C;
@@ -613,7 +495,7 @@ __device__ __forceinline__ void select_head_rows(const float* sc, const float* s
             const int eq_before = eq_run + __popc(eqm & lt_mask);
             if (gt || (eq && eq_before < need_eq)) {
                 const int rank = gt_before + min(eq_before, need_eq);
-                if (stage_sel) sm.sel[rank] = ch;
+                if (stage_sel) sm.sel[rank] = static_cast<unsigned short>(ch);
                 else {
                     const int j0 = ch * c, len = min(c, P - j0);
                     int32_t* dst = out + static_cast<size_t>(rank) * c;
