@@ -121,17 +121,19 @@ int check_sizes(int L, int w, int c, int budget) {
 }
 
 // row_elems / head_elems: elements between consecutive rows of a head and between heads; 0 = packed [heads, rows, d]
+// Boxes of 64 elements x box_rows in the 128-byte swizzle of the tensor cores' operands, or (whole_rows) of d elements x
+// box_rows, unswizzled: rows as they are.
 int encode_bf16_3d(CUtensorMap* tm, const void* base, int d, long long rows, int heads, int box_rows,
-                   CUtensorMapL2promotion promo, long long row_elems = 0, long long head_elems = 0) {
+                   CUtensorMapL2promotion promo, long long row_elems = 0, long long head_elems = 0, bool whole_rows = false) {
     cuuint64_t dims[3] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(rows),
                           static_cast<cuuint64_t>(heads)};
     if (row_elems == 0) row_elems = d;
     if (head_elems == 0) head_elems = rows * d;
     cuuint64_t strides[2] = {static_cast<cuuint64_t>(row_elems) * 2, static_cast<cuuint64_t>(head_elems) * 2};
-    cuuint32_t box[3] = {64, static_cast<cuuint32_t>(box_rows), 1};
+    cuuint32_t box[3] = {static_cast<cuuint32_t>(whole_rows ? d : 64), static_cast<cuuint32_t>(box_rows), 1};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = g_encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
-                          box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, promo,
+                          box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, whole_rows ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B, promo,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         g_last_cuda_error = 100000 + static_cast<int>(r);
@@ -937,17 +939,19 @@ static int compress_model_impl(int n_layers, const void* const* q_obs, const voi
         return CHUNKKV_OK;
     }
     std::lock_guard<std::mutex> lk(g_mu);
-    std::vector<CUtensorMap> tm_q(kModelMaxCompute), tm_k(kModelMaxCompute);
+    std::vector<CUtensorMap> tm_q(kModelMaxCompute), tm_k(kModelMaxCompute), tm_rk(strided ? kModelMaxStrided : 0),
+        tm_rv(strided ? kModelMaxStrided : 0);
     std::vector<ModelLayerIO> lay(kModelMaxLayers);
+    const int max_layers = strided ? kModelMaxStrided : kModelMaxLayers;
     for (int l0 = 0; l0 < n_layers;) {
-        // a launch takes whole reuse groups, at most kModelMaxLayers layers
+        // a launch takes whole reuse groups, at most max_layers layers
         int l1 = l0;
         int n_compute = 0;
         while (l1 < n_layers) {
             const int group_end = (l1 + reuse_depth < n_layers) ? l1 + reuse_depth : n_layers;
-            if ((group_end - l0 > kModelMaxLayers || n_compute == kModelMaxCompute) && l1 > l0) break;
-            if (group_end - l0 > kModelMaxLayers) {         // a single reuse group longer than a launch: split it
-                l1 = l0 + kModelMaxLayers;
+            if ((group_end - l0 > max_layers || n_compute == kModelMaxCompute) && l1 > l0) break;
+            if (group_end - l0 > max_layers) {              // a single reuse group longer than a launch: split it
+                l1 = l0 + max_layers;
                 if (n_compute == 0) n_compute = 1;
                 break;
             }
@@ -965,6 +969,13 @@ static int compress_model_impl(int n_layers, const void* const* q_obs, const voi
             const bool computes = (l % reuse_depth) == 0;
             lay[i].K = K[l]; lay[i].V = V[l]; lay[i].out_K = out_K[l]; lay[i].out_V = out_V[l]; lay[i].out_idx = out_idx[l];
             lay[i].computes = computes;
+            if (strided) {
+                const int rows = c < L ? c : L;
+                st = encode_bf16_3d(&tm_rk[i], K[l], d, L, Hkv, rows, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, kt, kh, true);
+                if (st != CHUNKKV_OK) return st;
+                st = encode_bf16_3d(&tm_rv[i], V[l], d, L, Hkv, rows, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, vt, vh, true);
+                if (st != CHUNKKV_OK) return st;
+            }
             if (computes) {
                 st = encode_bf16_3d(&tm_q[nc], q_obs[l], d, R, Hkv, R < 128 ? R : 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
                 if (st != CHUNKKV_OK) return st;
@@ -1002,11 +1013,11 @@ static int compress_model_impl(int n_layers, const void* const* q_obs, const voi
         io.scratch = reinterpret_cast<float*>(base + kHeaderBytes);
         io.counters = reinterpret_cast<unsigned*>(base + kResidentCountersOffset);
         io.status = reinterpret_cast<int*>(base);
-        io.k_row_elems = kt; io.k_head_elems = kh; io.v_row_elems = vt; io.v_head_elems = vh;
         cudaError_t e;
         {
             Timer t(ctx, s, 0);
-            e = launch_model(mp, io, tm_q.data(), tm_k.data(), lay.data(), n, s);
+            e = launch_model(mp, io, tm_q.data(), tm_k.data(), strided ? tm_rk.data() : nullptr, strided ? tm_rv.data() : nullptr,
+                             lay.data(), n, s);
         }
         if (e != cudaSuccess) return cuda_fail(e);
         l0 = l1;

@@ -128,11 +128,13 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
 // layer kernel above, plus two tail warps per CTA that select and copy rows behind the scoring.
 constexpr int kModelMaxLayers = 96;     // layers per launch (computed + reusing)
 constexpr int kModelMaxCompute = 32;    // computed layers per launch
+constexpr int kModelMaxStrided = 48;    // layers per launch whose rows are fetched through tensor maps
 
 struct ModelPlan {
     int c_static, n_mt, grid, cph, tile, n_tiles, t_max, spp, n_stages, smem_bytes;
     bool big;                    // two query tiles or a ring of partial sums that continues in scratch
     int ring_on, ring;           // panels of the ring on chip, in all
+    int ahead, stride;           // big: when a group contracts the layer before (own panels)
     int copy_slots;
     int n_score, n_sel;          // scoring CTAs, selector CTAs (grid = n_score + n_sel)
     int sel_row_bytes, sel_keys_fit;
@@ -146,8 +148,6 @@ struct ModelIO {
     float* scratch;       // model_scratch_floats() floats
     unsigned* counters;   // header + kResidentCountersOffset
     int* status;
-    // elements between consecutive rows of a head and between heads of K and of V (all layers); 0 = packed
-    long long k_row_elems = 0, k_head_elems = 0, v_row_elems = 0, v_head_elems = 0;
 };
 
 struct ModelLayerIO {
@@ -161,9 +161,11 @@ struct ModelLayerIO {
 
 bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, ModelPlan* plan);
 size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute);
-// layers[0] must compute; tm_q / tm_k hold one tensor map per computed layer, in order.
+// layers[0] must compute; tm_q / tm_k hold one tensor map per computed layer, in order; tm_rk / tm_rv one per layer (boxes
+// of one chunk's rows) where keys and values are not packed, else NULL.
 cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtensorMap* tm_q, const CUtensorMap* tm_k,
-                         const ModelLayerIO* layers, int n_layers, cudaStream_t stream);
+                         const CUtensorMap* tm_rk, const CUtensorMap* tm_rv, const ModelLayerIO* layers, int n_layers,
+                         cudaStream_t stream);
 
 // Token scores in one launch, two passes over the keys (token_kernel.cu).
 struct TokenPlan {

@@ -7,7 +7,7 @@
 // accumulator buffers) and the panel maxima in shared memory, so for most shapes nothing but a
 // (max, sum) pair per row and CTA goes to global memory before the chunk scores themselves. A key
 // range with more panels than those 256 columns hold (long contexts, small chunks) keeps the rest
-// in scratch (L2): written and read back by the same thread, one row per lane, coalesced.
+// in scratch (L2): written and read back by the same thread, 16 bytes at a time.
 //
 // A KV head with more than 128 query rows (two query tiles) is scored by the same CTAs: each key
 // tile is loaded once and multiplied with both query tiles, and the two pairs of epilogue groups
@@ -90,7 +90,7 @@ struct ResArgs {
     float* cta_stat;                   // [grid, n_mt, {max, sum}, 128]
     float* scores;                     // [Hkv, score_row]
     int score_row;                     // C, or C rounded up to a multiple of 4 in scratch (16-byte aligned rows)
-    float* spill;                      // [grid, n_off, 1 + chunk slots per panel, 128]: panel maximum, chunk sums
+    float* spill;                      // [grid, n_off, (chunk slots per panel + 1) * 128]: chunk sums, panel maximum
     unsigned* cnt_a;                   // [Hkv] hand-over 2, zero between launches
     unsigned* cnt_b;                   // [Hkv] hand-over 4
     unsigned* exits;                   // CTAs that left; the last one clears the counters
@@ -103,19 +103,16 @@ __device__ __forceinline__ bool head_handover(unsigned* counter, unsigned target
     __syncthreads();
     if (threadIdx.x == 0) {
         bool ok = true;
-        unsigned old;
-        // release: what this CTA wrote before the barrier above becomes visible to the others
-        asm volatile("atom.add.release.gpu.u32 %0, [%1], 1;" : "=r"(old) : "l"(counter) : "memory");
-        if (old + 1u < target) {
-            const long long t0 = clock64();
+        // release: what this CTA wrote before the barrier above becomes visible to whoever acquires the count (and, behind
+        // the barrier below, to the whole CTA); without a result the first poll follows at once
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
+        const long long t0 = clock64();
+        for (;;) {
             unsigned cur;
-            for (;;) {
-                asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(cur) : "l"(counter) : "memory");
-                if (cur >= target) break;
-                if (clock64() - t0 > kWaitLimitClocks) { ok = false; break; }
-            }
+            asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(cur) : "l"(counter) : "memory");
+            if (cur >= target) break;
+            if (clock64() - t0 > kWaitLimitClocks) { ok = false; break; }
         }
-        asm volatile("fence.acq_rel.gpu;" ::: "memory");
         ctl.wait_ok = ok ? 1 : 0;
     }
     __syncthreads();
@@ -303,10 +300,11 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 part_store<SPP>(lane_addr + static_cast<uint32_t>(kRPartCol0 + pl * SPP), pr);
                 pmax[pl * 128 + row] = m2;
             } else {
-                float* sp = a.spill + (static_cast<size_t>(blockIdx.x) * a.n_off + (pl - a.n_on)) * ((SPP + 1) * 128) + row;
-                st_keep(sp, m2, keep);
+                float rec_[SPP + 1];
 #pragma unroll
-                for (int q = 0; q < SPP; ++q) st_keep(sp + (q + 1) * 128, pr[q], keep);
+                for (int q = 0; q < SPP; ++q) rec_[q] = pr[q];
+                rec_[SPP] = m2;
+                spill_store<SPP + 1>(a.spill + (static_cast<size_t>(blockIdx.x) * a.n_off + (pl - a.n_on)) * ((SPP + 1) * 128), row, rec_, keep);
             }
             // fold into the running record: l is relative to m2, run_l to run_m
             const float nm = fmaxf(run_m, m2);
@@ -356,20 +354,22 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             const size_t step = static_cast<size_t>(n_mt) * 256;
             const float* src = a.cta_stat + (static_cast<size_t>(hkv) * a.cph * n_mt + mt) * 256 + i;
             float M = -CUDART_INF_F, Ls = 0.f;
-            for (int j0 = sl; j0 < a.cph; j0 += 4 * n_sl) {     // four records in flight per thread
-                float rm[4], rl[4];
+            // records in flight per thread: enough for one round trip where a head has 18 CTAs (8 heads)
+            constexpr int kF = BIG ? 9 : 5;
+            for (int j0 = sl; j0 < a.cph; j0 += kF * n_sl) {
+                float rm[kF], rl[kF];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
+                for (int u = 0; u < kF; ++u) {
                     const int j = j0 + n_sl * u;
                     rm[u] = (j < a.cph) ? __ldcg(src + j * step) : -CUDART_INF_F;
                     rl[u] = (j < a.cph) ? __ldcg(src + j * step + 128) : 0.f;
                 }
                 float bm = M;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) bm = fmaxf(bm, rm[u]);
+                for (int u = 0; u < kF; ++u) bm = fmaxf(bm, rm[u]);
                 float acc = (M == -CUDART_INF_F) ? 0.f : Ls * ex2_approx(M - bm);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) acc += (rm[u] == -CUDART_INF_F) ? 0.f : rl[u] * ex2_approx(rm[u] - bm);
+                for (int u = 0; u < kF; ++u) acc += (rm[u] == -CUDART_INF_F) ? 0.f : rl[u] * ex2_approx(rm[u] - bm);
                 M = bm;
                 Ls = acc;
             }
@@ -428,10 +428,11 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                             part_load<SPP>(lane_addr + static_cast<uint32_t>(kRPartCol0 + pl * SPP), &v[u * SPP]);
                             pm[u] = pmax[pl * 128 + row];
                         } else {
-                            const float* sp = a.spill + (static_cast<size_t>(blockIdx.x) * a.n_off + (pl - a.n_on)) * ((SPP + 1) * 128) + row;
-                            pm[u] = ld_drop(sp, drop);
+                            float rec_[SPP + 1];
+                            spill_load<SPP + 1>(a.spill + (static_cast<size_t>(blockIdx.x) * a.n_off + (pl - a.n_on)) * ((SPP + 1) * 128), row, rec_, drop);
+                            pm[u] = rec_[SPP];
 #pragma unroll
-                            for (int q = 0; q < SPP; ++q) v[u * SPP + q] = ld_drop(sp + (q + 1) * 128, drop);
+                            for (int q = 0; q < SPP; ++q) v[u * SPP + q] = rec_[q];
                         }
                     }
                 }

@@ -46,7 +46,7 @@ constexpr int kMThreads = 640;          // warp 0: TMA, warp 1: UMMA issue, warp
                                         // (five warps per scheduler: a sixth would cut every thread to 80 registers)
 constexpr int kMMiscBytes = 16384;      // epilogue: group records (two slots), m_i, 1 / l_i, row sums per lane quarter
 constexpr int kMSlots = 8;              // most staging slots of the row copies
-constexpr int kMSegSlots = 64;          // chunk slots a group contracts between two barriers
+constexpr int kMBlkSlots = 32;          // room for the chunk slots of one contraction block
 // Tensor memory, small variant: three 64-column accumulators (one 60-key panel of a tile each, in rotation; the
 // second panel of a tile is computed on keys 56 .. 119 so that its operand starts on a swizzle-atom
 // boundary, and begins at column 4), and 320 columns of chunk partial sums: a ring that holds one
@@ -118,23 +118,29 @@ struct ModelParams {
     int C, k, n_max, Hkv;
     int Cpad;              // row stride of the chunk scores (C rounded up to a multiple of 4: rows stay 16-byte aligned)
     int n_score, n_sel;    // scoring CTAs (Hkv * cph) and selector CTAs (the rest of the grid)
+    int strided;           // rows of a head are not adjacent in memory: kept rows are fetched through tm_rk / tm_rv
+    int copy_box_bytes;    // bytes of such a box
     int ring_on, ring;     // big variant: panels of the ring in tensor memory, panels of the ring in all
+    int ahead, stride;     // big variant: own panels of a layer that a group scores before the contraction of the layer before,
+                           // and between two blocks of it
     int copy_slots;
     int sel_row_bytes;     // bytes of one kept-chunk list: 4 header ints + the kept chunk ids, padded to 16 bytes
     int sel_keys_fit;      // selector: the keys of a head fit its shared memory (many chunks per thread)
     int off_ring, off_pmax, off_misc, off_tail, stage_slot_bytes;
-    // bytes between consecutive rows of a head and between heads of K and of V (packed: d * 2 and L * d * 2)
-    long long k_row_bytes, k_head_bytes, v_row_bytes, v_head_bytes;
     float* cta_stat;       // [2 (slot parity)][grid][n_mt][{max, sum}][128]
     float* scores;         // [n_compute][Hkv][n_mt][Cpad]
-    float* spill;          // [scoring CTA][ring - ring_on][1 + chunk slots per panel][128]: panel maximum, chunk sums
+    float* spill;          // [scoring CTA][ring - ring_on][(chunk slots per panel + 1) * 128]: chunk sums, panel maximum
     unsigned* cnt_a;       // [Hkv]
     unsigned* cnt_b;       // [Hkv]  chunk scores of a slot announced by the scoring CTAs
     unsigned* cnt_c;       // [Hkv]  kept-chunk lists announced by the selector CTAs
     int* sel_rows;         // [n_compute][Hkv][sel_row_bytes / 4]
     unsigned* exits;
     int* status;
+    // strided caches: boxes of one chunk's rows of K and of V, per layer (a launch takes at most kModelMaxStrided then)
+    CUtensorMap tm_rk[kModelMaxStrided];
+    CUtensorMap tm_rv[kModelMaxStrided];
 };
+static_assert(sizeof(ModelParams) <= 32764, "kernel parameters");
 
 // ---- bulk asynchronous copies (no multicast): global -> this CTA's shared memory with byte-counted
 //      completion on an mbarrier, and shared -> global in bulk groups
@@ -282,10 +288,9 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
     return true;
 }
 
-// STRIDED: the rows of a head are not adjacent in memory (e.g. token-major caches): the copy thread moves
-// kept rows one at a time. BIG: two query tiles, or a ring that reaches into scratch. Variants of their own, so that
-// the kernel for packed caches and up to 128 rows is exactly what it was.
-template <int C_STATIC, bool STRIDED, bool BIG>
+// BIG: two query tiles, or a ring that reaches into scratch. A variant of its own, so that the kernel for up to 128 rows
+// carries none of it.
+template <int C_STATIC, bool BIG>
 __global__ void __launch_bounds__(kMThreads, 1)
 model_kernel(const __grid_constant__ ModelParams p) {
     constexpr int WP = panel_keys(C_STATIC);
@@ -309,8 +314,8 @@ model_kernel(const __grid_constant__ ModelParams p) {
     float* pmax = reinterpret_cast<float*>(dyn + p.off_pmax);
     float* misc = reinterpret_cast<float*>(dyn + p.off_misc);
     float* rec = misc;                 // [4 groups][{max, sum}][128]; the odd slots' copy sits at misc + 3072
-    float* gstat = misc + 1024;        // [2 (slot parity)][2 query tiles][{m_i, 1 / l_i}][128]
-    float* red = misc + 2048;          // [4 groups][4 lane quarters][kMSegSlots]
+    float* gstat = misc + 1024;        // [2 (slot parity)][{m_i, 1 / l_i}][128]; big variant: [4 groups][{m_i, 1 / l_i}][128]
+    float* red = misc + 2048;          // [4 groups][block parity][4 lane quarters][kMBlkSlots]
     volatile int* abort_flag = &ctl.abort_flag;
     const uint32_t n_stages = static_cast<uint32_t>(p.n_stages);
 
@@ -490,10 +495,9 @@ model_kernel(const __grid_constant__ ModelParams p) {
     } else if (warp < 18) {
         // ------------------------------------------------------------------ epilogue
         // The chunk partial sums and panel maxima of a layer live in rings (tensor-memory columns,
-        // shared memory) that hold more than one layer's worth, so after its last tile of layer s a
-        // thread only publishes the CTA's row records and goes straight on with the first `ahead`
-        // tiles of layer s + 1; the chunk scores of layer s are formed after those, when the other
-        // CTAs' records have long arrived and the statistics warp has merged them.
+        // shared memory, scratch) that hold more than one layer's worth, so after its last tile of layer s a
+        // thread only publishes the CTA's row records and goes straight on with layer s + 1; the chunk scores
+        // of layer s are formed between its panels.
         const int grp = (warp - 2) >> 2, quarter = warp & 3;
         const int gt = threadIdx.x - 64 - grp * 128;    // 0 .. 127 within the group
         const int pair = grp >> 1, half = grp & 1;
@@ -505,17 +509,145 @@ model_kernel(const __grid_constant__ ModelParams p) {
         const int n_pl = 2 * n_vt;
         const int PR = BIG ? p.ring : model_ring_panels(C_STATIC, false);          // panels in the ring
         constexpr int PCOLS = BIG ? SPP + 1 : SPP;                                  // tensor-memory columns of a panel
-        const int ahead = max(0, min(n_vt, (PR - n_pl) / 2));   // virtual tiles of the next layer scored before the contraction
         const int ch0 = t_begin * (TILE / C_STATIC);
         const uint64_t keep = l2_policy_evict_last(), drop = l2_policy_evict_first();
-        float* spill = BIG ? p.spill + static_cast<size_t>(blockIdx.x) * (p.ring - p.ring_on) * ((SPP + 1) * 128) + row : nullptr;
+        float* spill = BIG ? p.spill + static_cast<size_t>(blockIdx.x) * (p.ring - p.ring_on) * ((SPP + 1) * 128) : nullptr;
         bool ok = true;
         float run_m = -CUDART_INF_F, run_l = 0.f;
-        // virtual tiles [v_lo, v_hi) of slot s that belong to this thread's pair
-        auto do_tiles = [&](int s, int v_lo, int v_hi) {
-            if (!ok) return;
+        // Contraction of a layer's partial sums into chunk scores, one block of panels at a time, between the panels of the next
+        // layer: a group contracts the panels it scored itself - every thread reads back the tensor-memory columns (or
+        // scratch) it wrote - so the only synchronisation is among the group's four warps (the four lane quarters of a
+        // sum). It starts once `ahead` of the group's own panels of the next layer are scored, so that the row statistics
+        // have arrived, and goes on block by panel, so that the groups' round trips and shuffles overlap the other groups'
+        // exponentials. A block holds more panels than are scored between two blocks, and the ring more than a layer and
+        // `ahead` panels per group: a slot is contracted before it is written again. (Big variant: `stride` panels between
+        // two blocks and the groups a part of it apart, so that mostly one group at a time waits for scratch; the ring then
+        // holds `stride` panels per group more.)
+        constexpr int PPB = 32 / SPP;                        // panels per block of up to 32 values
+        const int ahead = BIG ? p.ahead + grp * p.stride / 4 : max(0, (PR - n_pl) / 4);           // own panels
+        int next_blk = ahead;                                // own panel before which the next block is due
+        float* rg = red + grp * (8 * kMBlkSlots);            // [block parity][4 lane quarters][kMBlkSlots]
+        int c_s = 0, c_blk = 0, c_left = 0, c_par = 0;       // layer, next block, blocks left, parity of the block count
+        // false: a wait of some warp of the group was abandoned, all four leave
+        auto contract_block = [&]() -> bool {
+            const int vg0 = c_s * n_vt, pbase = (c_s * n_pl) % PR;
+            // first panel of the layer that this group scored; its others follow every fourth panel
+            const int g1 = 2 * ((pair - vg0) & 1) + half;
+            const int own = (n_pl - g1 + 3) / 4, b0 = c_blk * PPB;
+            if (c_blk == 0) {
+                bool ready = true;
+                if (lane == 0) ready = mbar_wait(smem_u32(&ctl.stat_full[c_s & 1]), (c_s >> 1) & 1, abort_flag);
+                if (!__shfl_sync(0xffffffffu, ready, 0)) ok = false;   // (the failed wait has raised the abort flag)
+                tmem_st_wait();
+                if constexpr (BIG) {
+                    // every record of the head is there (the statistics warp has seen the count): each thread merges those of
+                    // its row, straight from the L2. 18 records of two query tiles took the statistics warp 8 us beside four
+                    // busy warps, 128 threads a group take 1.5.
+                    float M = -CUDART_INF_F, S = 0.f;
+                    const size_t step = static_cast<size_t>(n_mt) * 256;
+                    const float* src = p.cta_stat + ((static_cast<size_t>(c_s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * n_mt +
+                                                     (two ? pair : 0)) * 256 + row;
+                    for (int j0 = 0; ok && j0 < p.cph; j0 += 9) {
+                        float rm[9], rl[9];
+#pragma unroll
+                        for (int j = 0; j < 9; ++j) {
+                            const bool in = j0 + j < p.cph;
+                            rm[j] = in ? __ldcg(src + (j0 + j) * step) : -CUDART_INF_F;
+                            rl[j] = in ? __ldcg(src + (j0 + j) * step + 128) : 0.f;
+                        }
+                        float bm = M;
+#pragma unroll
+                        for (int j = 0; j < 9; ++j) bm = fmaxf(bm, rm[j]);
+                        float acc = (M == -CUDART_INF_F) ? 0.f : S * ex2_approx(M - bm);
+#pragma unroll
+                        for (int j = 0; j < 9; ++j) acc += (rm[j] == -CUDART_INF_F) ? 0.f : rl[j] * ex2_approx(rm[j] - bm);
+                        M = bm;
+                        S = acc;
+                    }
+                    gstat[grp * 256 + row] = M;                // (read back by this thread only)
+                    gstat[grp * 256 + 128 + row] = 1.0f / S;
+                }
+            }
+            const float* gm = gstat + (BIG ? grp : c_s & 1) * 256;
+            const float mi = gm[row], li = gm[128 + row];
+            float* rb = rg + c_par * (4 * kMBlkSlots);
+            if (own > 0) {
+                float v[32], pm[PPB];
+                int slot_of[PPB];
+#pragma unroll
+                for (int u = 0; u < PPB; ++u) {
+                    const int pl = min(g1 + 4 * (b0 + u), n_pl - 1);
+                    int slot = pbase + pl;
+                    slot -= (slot >= PR) ? PR : 0;
+                    slot_of[u] = slot;
+                }
+                if constexpr (BIG) {
+                    float vp[PPB * PCOLS];
+#pragma unroll
+                    for (int u = 0; u < PPB; ++u) {
+                        if (slot_of[u] < p.ring_on) {
+                            part_load<PCOLS>(lane_addr + static_cast<uint32_t>(PART0 + slot_of[u] * PCOLS), &vp[u * PCOLS]);
+                        } else {
+                            spill_load<PCOLS>(spill + static_cast<size_t>(slot_of[u] - p.ring_on) * (PCOLS * 128), row, &vp[u * PCOLS], drop);
+                        }
+                    }
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int u = 0; u < PPB; ++u) {
+                        pm[u] = vp[u * PCOLS + SPP];
+#pragma unroll
+                        for (int q = 0; q < SPP; ++q) v[u * SPP + q] = vp[u * PCOLS + q];
+                    }
+                } else {
+#pragma unroll
+                    for (int u = 0; u < PPB; ++u)
+                        part_load<SPP>(lane_addr + static_cast<uint32_t>(PART0 + slot_of[u] * SPP), &v[u * SPP]);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int u = 0; u < PPB; ++u) pm[u] = pmax[slot_of[u] * 128 + row];
+                }
+#pragma unroll
+                for (int e = PPB * SPP; e < 32; ++e) v[e] = 0.f;
+#pragma unroll
+                for (int u = 0; u < PPB; ++u) {
+                    const bool have = active && b0 + u < own;
+                    const float f = have ? ex2_approx(pm[u] - mi) * li : 0.f;
+#pragma unroll
+                    for (int q = 0; q < SPP; ++q) v[u * SPP + q] = have ? v[u * SPP + q] * f : 0.f;
+                }
+                rb[quarter * kMBlkSlots + lane] = warp_transpose_reduce(v, lane);
+            }
+            // the block's sums are there; and a uniform decision to go on (the two halves of rg alternate: a half is written
+            // again only after the next block's barrier, which its readers reach behind their reads)
+            if (named_barrier_or(kBarGroup + grp, 128, !ok || ctl.abort_flag != 0)) return false;
+            if (gt < min(own - b0, PPB) * SPP) {
+                const int pl = g1 + 4 * (b0 + gt / SPP);
+                const int kp = two ? (pl >> 2) * 2 + (pl & 1) : pl;          // panel of the key range
+                const int ch = ch0 + kp * SPP + gt % SPP;
+                if (ch < p.C)
+                    p.scores[((static_cast<size_t>(c_s) * p.Hkv + hkv) * n_mt + (two ? pair : 0)) * p.Cpad + ch] =
+                        (rb[gt] + rb[kMBlkSlots + gt]) + (rb[2 * kMBlkSlots + gt] + rb[3 * kMBlkSlots + gt]);
+            }
+            ++c_blk;
+            c_par ^= 1;
+            if (--c_left == 0) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ctl.sc_done[c_s & 1]));      // announced by the statistics warp
+            }
+            return true;
+        };
+        bool alive = true;
+        // the panels of slot s that belong to this thread's group, and the contraction of the layer before
+        auto do_layer = [&](int s) {
             const int vg0 = s * n_vt, pbase = (s * n_pl) % PR;
-            for (int vt = v_lo + ((pair - ((vg0 + v_lo) & 1)) & 1); vt < v_hi; vt += 2) {
+            int done = 0;
+            next_blk = ahead;
+            for (int vt = (pair - vg0) & 1; vt < n_vt; vt += 2, ++done) {
+                if (c_left > 0 && done >= next_blk) {
+                    if (!contract_block()) { alive = false; return; }
+                    if constexpr (BIG) next_blk += p.stride;
+                }
+                if (!ok) continue;           // (an abandoned wait: only the group's barriers are still kept)
                 const int ti = two ? vt >> 1 : vt;
                 const int pc = 2 * (vg0 + vt) + half;        // panel number since the start of the launch
                 const int aslot = BIG ? pair : pc % kMAccSlots;
@@ -523,7 +655,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                 const int acol = BIG ? pair * kRUmmaN + half * WP : (pc % kMAccBufs) * kMAccN + half * COL1;
                 bool ready = true;
                 if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[aslot]), use & 1, abort_flag);
-                if (!__shfl_sync(0xffffffffu, ready, 0)) { ok = false; break; }
+                if (!__shfl_sync(0xffffffffu, ready, 0)) { ok = false; continue; }
                 tc_fence_after();
                 float v[WP];
                 load_panel<WP>(lane_addr + static_cast<uint32_t>(acol), v);
@@ -545,9 +677,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                     if (slot < p.ring_on) {
                         part_store<PCOLS>(lane_addr + static_cast<uint32_t>(PART0 + slot * PCOLS), pr);
                     } else {
-                        float* sp = spill + static_cast<size_t>(slot - p.ring_on) * (PCOLS * 128);
-#pragma unroll
-                        for (int q = 0; q < PCOLS; ++q) st_keep(sp + q * 128, pr[q], keep);
+                        spill_store<PCOLS>(spill + static_cast<size_t>(slot - p.ring_on) * (PCOLS * 128), row, pr, keep);
                     }
                 } else {
                     part_store<SPP>(lane_addr + static_cast<uint32_t>(PART0 + slot * SPP), pr);
@@ -571,99 +701,15 @@ model_kernel(const __grid_constant__ ModelParams p) {
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&ctl.pub_done[s & 1]));
         };
-        // Chunk scores of slot s from the partial sums in the rings. A group contracts the panels it
-        // scored itself - every thread reads back the tensor-memory columns and panel maxima it wrote -
-        // so the only synchronisation is among the group's four warps (the four lane quarters of a sum).
-        auto contract = [&](int s) -> bool {
-            const int vg0 = s * n_vt, pbase = (s * n_pl) % PR;
-            // first panel of the slot that this group scored; its others follow every fourth panel
-            const int g1 = 2 * ((pair - vg0) & 1) + half;
-            bool ready = true;
-            if (lane == 0) ready = mbar_wait(smem_u32(&ctl.stat_full[s & 1]), (s >> 1) & 1, abort_flag);
-            if (!__shfl_sync(0xffffffffu, ready, 0)) ok = false;   // (the failed wait has raised the abort flag)
-            tmem_st_wait();
-            // the group's previous sums have been read by all its warps; and a uniform decision to go on
-            if (named_barrier_or(kBarGroup + grp, 128, !ok || ctl.abort_flag != 0)) return false;
-            const float* gm = gstat + (s & 1) * 512 + (two ? pair * 256 : 0);
-            const float mi = gm[row], li = gm[128 + row];
-            float* rg = red + grp * (4 * kMSegSlots);
-            float* sc_out = p.scores + ((static_cast<size_t>(s) * p.Hkv + hkv) * n_mt + (two ? pair : 0)) * p.Cpad;
-            constexpr int PPB = 32 / SPP;                    // panels per block of up to 32 values
-            constexpr int BPS = kMSegSlots / (PPB * SPP);    // blocks per segment
-            const int own = (n_pl - g1 + 3) / 4;             // panels of this group
-            for (int s0 = 0; s0 < own; s0 += PPB * BPS) {
-                // (the previous segment's sums have been read: a barrier lies between)
-                if (s0 > 0) named_barrier(kBarGroup + grp, 128);
-                for (int b0 = s0; b0 < min(own, s0 + PPB * BPS); b0 += PPB) {
-                    float v[32], pm[PPB];
-                    int slot_of[PPB];
-#pragma unroll
-                    for (int u = 0; u < PPB; ++u) {
-                        const int pl = min(g1 + 4 * (b0 + u), n_pl - 1);
-                        int slot = pbase + pl;
-                        slot -= (slot >= PR) ? PR : 0;
-                        slot_of[u] = slot;
-                    }
-                    if constexpr (BIG) {
-                        float vp[PPB * PCOLS];
-#pragma unroll
-                        for (int u = 0; u < PPB; ++u) {
-                            if (slot_of[u] < p.ring_on) {
-                                part_load<PCOLS>(lane_addr + static_cast<uint32_t>(PART0 + slot_of[u] * PCOLS), &vp[u * PCOLS]);
-                            } else {
-                                const float* sp = spill + static_cast<size_t>(slot_of[u] - p.ring_on) * (PCOLS * 128);
-#pragma unroll
-                                for (int q = 0; q < PCOLS; ++q) vp[u * PCOLS + q] = ld_drop(sp + q * 128, drop);
-                            }
-                        }
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int u = 0; u < PPB; ++u) {
-                            pm[u] = vp[u * PCOLS + SPP];
-#pragma unroll
-                            for (int q = 0; q < SPP; ++q) v[u * SPP + q] = vp[u * PCOLS + q];
-                        }
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < PPB; ++u)
-                            part_load<SPP>(lane_addr + static_cast<uint32_t>(PART0 + slot_of[u] * SPP), &v[u * SPP]);
-                        tmem_ld_wait();
-#pragma unroll
-                        for (int u = 0; u < PPB; ++u) pm[u] = pmax[slot_of[u] * 128 + row];
-                    }
-#pragma unroll
-                    for (int e = PPB * SPP; e < 32; ++e) v[e] = 0.f;
-#pragma unroll
-                    for (int u = 0; u < PPB; ++u) {
-                        const bool have = active && b0 + u < own;
-                        const float f = have ? ex2_approx(pm[u] - mi) * li : 0.f;
-#pragma unroll
-                        for (int q = 0; q < SPP; ++q) v[u * SPP + q] = have ? v[u * SPP + q] * f : 0.f;
-                    }
-                    const float tot = warp_transpose_reduce(v, lane);
-                    if (lane < PPB * SPP) rg[quarter * kMSegSlots + (b0 - s0) * SPP + lane] = tot;
-                }
-                named_barrier(kBarGroup + grp, 128);
-                // chunk slots of this segment's panels (at most kMSegSlots)
-                const int n_own = min(own - s0, PPB * BPS) * SPP;
-                if (gt < n_own) {
-                    const int pl = g1 + 4 * (s0 + gt / SPP);
-                    const int kp = two ? (pl >> 2) * 2 + (pl & 1) : pl;          // panel of the key range
-                    const int ch = ch0 + kp * SPP + gt % SPP;
-                    if (ch < p.C)
-                        sc_out[ch] = (rg[gt] + rg[kMSegSlots + gt]) + (rg[2 * kMSegSlots + gt] + rg[3 * kMSegSlots + gt]);
-                }
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&ctl.sc_done[s & 1]));      // announced by the statistics warp
-            return true;
-        };
-        for (int s = 0; s <= p.n_compute; ++s) {
-            if (s < p.n_compute) do_tiles(s, 0, ahead);
-            if (s > 0 && !contract(s - 1)) break;
-            if (s < p.n_compute) {
-                do_tiles(s, ahead, n_vt);
+        for (int s = 0; s <= p.n_compute && alive; ++s) {
+            if (s < p.n_compute) do_layer(s);
+            while (alive && c_left > 0) alive = contract_block();
+            if (alive && s < p.n_compute) {
                 publish(s);
+                const int own = (n_pl - (2 * ((pair - s * n_vt) & 1) + half) + 3) / 4;
+                c_s = s;
+                c_blk = 0;
+                c_left = max(1, (own + PPB - 1) / PPB);
             }
         }
         if (!ok && lane == 0) ctl.abort_flag = 1;
@@ -705,23 +751,22 @@ model_kernel(const __grid_constant__ ModelParams p) {
             }
             if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.cnt_a + hkv) : "memory");
             if (!wait_counter_warp(p.cnt_a + hkv, static_cast<unsigned>(s + 1) * p.cph, abort_flag)) break;
-            // the head's records straight from the L2 (they were written by other SMs; every lane has
-            // acquired the counter), six CTAs' worth of loads in flight per lane
-            for (int mt = 0; mt < n_mt; ++mt) {
-                const size_t step = static_cast<size_t>(n_mt) * 256;
-                const float* src = p.cta_stat + ((static_cast<size_t>(s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * n_mt + mt) * 256;
+            if constexpr (!BIG) {
+                // the head's records straight from the L2 (they were written by other SMs; every lane has
+                // acquired the counter), nine CTAs' worth of loads in flight per lane
+                const float* src = p.cta_stat + (static_cast<size_t>(s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * 256;
                 float M[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}, S[4] = {0.f, 0.f, 0.f, 0.f};
-                for (int j0 = 0; j0 < p.cph; j0 += 6) {
-                    float4 m[6], l[6];
+                for (int j0 = 0; j0 < p.cph; j0 += 9) {
+                    float4 m[9], l[9];
 #pragma unroll
-                    for (int j = 0; j < 6; ++j) {
+                    for (int j = 0; j < 9; ++j) {
                         const int jj = min(j0 + j, p.cph - 1);
-                        m[j] = __ldcg(reinterpret_cast<const float4*>(src + jj * step + r0));
-                        l[j] = __ldcg(reinterpret_cast<const float4*>(src + jj * step + 128 + r0));
+                        m[j] = __ldcg(reinterpret_cast<const float4*>(src + static_cast<size_t>(jj) * 256 + r0));
+                        l[j] = __ldcg(reinterpret_cast<const float4*>(src + static_cast<size_t>(jj) * 256 + 128 + r0));
                     }
-                    merge_batch<6>(M, S, m, l, p.cph - j0);
+                    merge_batch<9>(M, S, m, l, p.cph - j0);
                 }
-                float* gm = gstat + (s & 1) * 512 + mt * 256;
+                float* gm = gstat + (s & 1) * 256;
                 *reinterpret_cast<float4*>(gm + r0) = make_float4(M[0], M[1], M[2], M[3]);
                 *reinterpret_cast<float4*>(gm + 128 + r0) = make_float4(1.0f / S[0], 1.0f / S[1], 1.0f / S[2], 1.0f / S[3]);
             }
@@ -741,9 +786,9 @@ model_kernel(const __grid_constant__ ModelParams p) {
         // One thread: waits until the selector CTA has published the head's kept-chunk list of a
         // slot, fetches the list, and moves this CTA's share of the rows - whole chunks and window
         // pieces - through the staging slots with bulk copies, for the computed layer and for every
-        // layer that reuses its indices. (Strided variant: the whole warp runs this loop in step - lane 0 waits,
-        // stores and keeps the books, every lane issues the copy of one source row.)
-        if (STRIDED || lane == 0) {
+        // layer that reuses its indices. Rows that are not adjacent in memory (e.g. token-major caches)
+        // arrive through tensor maps whose box is a chunk: one copy as well, whatever the strides.
+        if (lane == 0) {
             uint8_t* tbase = dyn + p.off_tail;
             int* row = reinterpret_cast<int*>(tbase);        // [4 + kkpad]: n_tok, -, -, -, kept chunk ids
             const uint32_t stage0 = smem_u32(tbase + p.sel_row_bytes);
@@ -763,7 +808,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
             bool ok = true;
             for (int li = 0; li < p.n_layers && ok;) {
                 const int s = p.layer[li].slot;
-                if (lane == 0) {
+                {
                     ok = wait_counter(p.cnt_c + hkv, static_cast<unsigned>(s + 1), abort_flag, 200);
                     if (ok) {
                         asm volatile("fence.acq_rel.gpu;" ::: "memory");
@@ -775,10 +820,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                                   static_cast<uint32_t>(p.sel_row_bytes), bar);
                     }
                 }
-                if constexpr (STRIDED) ok = __shfl_sync(0xffffffffu, ok, 0);
-                // (every lane that reads the list waits for it itself)
                 if (ok) ok = mbar_wait(smem_u32(&ctl.sfull), static_cast<uint32_t>(s) & 1u, abort_flag);
-                if constexpr (STRIDED) ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 const int n_tok = row[0];
                 auto unit = [&](int u, int& src_row, int& dst_row, int& rows) {
@@ -796,10 +838,8 @@ model_kernel(const __grid_constant__ ModelParams p) {
                 int lj = li;
                 do {
                     const ModelLayer& ly = p.layer[lj];
-                    const char* Kh = reinterpret_cast<const char*>(ly.K) +
-                                     (STRIDED ? static_cast<size_t>(hkv) * p.k_head_bytes : static_cast<size_t>(hkv) * p.L * row_bytes);
-                    const char* Vh = reinterpret_cast<const char*>(ly.V) +
-                                     (STRIDED ? static_cast<size_t>(hkv) * p.v_head_bytes : static_cast<size_t>(hkv) * p.L * row_bytes);
+                    const char* Kh = reinterpret_cast<const char*>(ly.K) + static_cast<size_t>(hkv) * p.L * row_bytes;
+                    const char* Vh = reinterpret_cast<const char*>(ly.V) + static_cast<size_t>(hkv) * p.L * row_bytes;
                     char* oK = reinterpret_cast<char*>(ly.out_K) + static_cast<size_t>(hkv) * p.n_max * row_bytes;
                     char* oV = reinterpret_cast<char*>(ly.out_V) + static_cast<size_t>(hkv) * p.n_max * row_bytes;
                     int loaded = 0;
@@ -807,21 +847,18 @@ model_kernel(const __grid_constant__ ModelParams p) {
                         int sr, dr, rows;
                         unit(u_begin + idx, sr, dr, rows);
                         const uint32_t slot = (g_issued + idx) % n_slots;
-                        const uint32_t bytes = static_cast<uint32_t>(rows) * row_bytes;
                         const uint32_t bar = smem_u32(&ctl.gfull[slot]);
-                        if (lane == 0) mbar_arrive_expect_tx(bar, 2u * bytes);
-                        if constexpr (!STRIDED) {
-                            bulk_load(stage0 + slot * p.stage_slot_bytes, Kh + static_cast<size_t>(sr) * row_bytes, bytes, bar);
-                            bulk_load(stage0 + slot * p.stage_slot_bytes + half_slot, Vh + static_cast<size_t>(sr) * row_bytes, bytes, bar);
+                        const uint32_t dst = stage0 + slot * p.stage_slot_bytes;
+                        if (!p.strided) {
+                            const uint32_t bytes = static_cast<uint32_t>(rows) * row_bytes;
+                            mbar_arrive_expect_tx(bar, 2u * bytes);
+                            bulk_load(dst, Kh + static_cast<size_t>(sr) * row_bytes, bytes, bar);
+                            bulk_load(dst + half_slot, Vh + static_cast<size_t>(sr) * row_bytes, bytes, bar);
                         } else {
-                            // rows of a chunk are not adjacent in memory (e.g. a token-major cache): lane r copies row r
-                            __syncwarp();             // the byte count is on the barrier before any copy can complete
-                            if (lane < rows) {
-                                bulk_load(stage0 + slot * p.stage_slot_bytes + static_cast<uint32_t>(lane) * row_bytes,
-                                          Kh + static_cast<size_t>(sr + lane) * p.k_row_bytes, row_bytes, bar);
-                                bulk_load(stage0 + slot * p.stage_slot_bytes + half_slot + static_cast<uint32_t>(lane) * row_bytes,
-                                          Vh + static_cast<size_t>(sr + lane) * p.v_row_bytes, row_bytes, bar);
-                            }
+                            // (a box is always whole: rows past the chunk's or window's end are not stored, past L they are zeros)
+                            mbar_arrive_expect_tx(bar, 2u * static_cast<uint32_t>(p.copy_box_bytes));
+                            tma_load_3d(dst, &p.tm_rk[lj], bar, 0, sr, hkv);
+                            tma_load_3d(dst + half_slot, &p.tm_rv[lj], bar, 0, sr, hkv);
                         }
                     };
                     // loads run n_slots - 1 units ahead of the stores
@@ -829,34 +866,31 @@ model_kernel(const __grid_constant__ ModelParams p) {
                     for (int idx = 0; idx < n_units && ok; ++idx) {
                         const uint32_t gi = g_issued + idx;
                         const uint32_t slot = gi % n_slots;
-                        if (lane == 0) ok = mbar_wait(smem_u32(&ctl.gfull[slot]), (gi / n_slots) & 1u, abort_flag);
-                        if constexpr (STRIDED) ok = __shfl_sync(0xffffffffu, ok, 0);
+                        ok = mbar_wait(smem_u32(&ctl.gfull[slot]), (gi / n_slots) & 1u, abort_flag);
                         if (!ok) break;
                         int sr, dr, rows;
                         unit(u_begin + idx, sr, dr, rows);
                         const uint32_t bytes = static_cast<uint32_t>(rows) * row_bytes;
-                        if (lane == 0) {
+                        {
                             bulk_store(oK + static_cast<size_t>(dr) * row_bytes, stage0 + slot * p.stage_slot_bytes, bytes);
                             bulk_store(oV + static_cast<size_t>(dr) * row_bytes, stage0 + slot * p.stage_slot_bytes + half_slot, bytes);
                             bulk_commit();
                         }
                         if (loaded < n_units) {
                             // the slot the next load takes was stored one unit ago: all but the newest group have been read
-                            if (lane == 0) bulk_wait_read<1>();
-                            if constexpr (STRIDED) __syncwarp();
+                            bulk_wait_read<1>();
                             issue_load(loaded);
                             ++loaded;
                         }
                     }
-                    if (lane == 0) bulk_wait_read<0>();          // the slots are reused by the next layer's first loads
-                    if constexpr (STRIDED) __syncwarp();
+                    bulk_wait_read<0>();          // the slots are reused by the next layer's first loads
                     g_issued += static_cast<uint32_t>(n_units);
                     ++lj;
                 } while (ok && lj < p.n_layers && !p.layer[lj].computes);
                 li = lj;
             }
-            if (lane == 0) bulk_wait_all();
-            if (!ok && lane == 0) ctl.abort_flag = 1;
+            bulk_wait_all();
+            if (!ok) ctl.abort_flag = 1;
         }
     }
 
@@ -902,12 +936,19 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_
     p.t_max = (p.n_tiles + p.cph - 1) / p.cph;
     // Panels of a CTA and layer; the ring should hold them and at least kMinAhead of the next layer, whose scoring
     // hides the exchange of row statistics. Where tensor memory holds fewer the ring continues in scratch.
-    constexpr int kMinAhead = 8, kBigAhead = 24;
+    constexpr int kMinAhead = 8, kBigAhead = 5;
     const int n_pl = 2 * p.n_mt * p.t_max;
     p.big = p.n_mt == 2 || n_pl + kMinAhead > model_ring_panels(c, false);
+    p.ahead = p.stride = 0;
     if (p.big) {
+        // per epilogue group: kBigAhead panels (about 10 us) until the statistics are there, then a block of the contraction
+        // every `stride` panels so that the last one is done near the end of the layer
+        const int own = (n_pl + 3) / 4, ppb = 32 / p.spp, blocks = (own + ppb - 1) / ppb;
+        p.ahead = own < kBigAhead ? own : kBigAhead;
+        p.stride = (own - p.ahead) / blocks;
+        p.stride = p.stride < 1 ? 1 : (p.stride > ppb ? ppb : p.stride);
         p.ring_on = model_ring_panels(c, true);
-        p.ring = (n_pl + (kBigAhead < n_pl ? kBigAhead : n_pl) + 3) / 4 * 4;
+        p.ring = (n_pl + 4 * (p.ahead + p.stride) + 3) / 4 * 4;
         if (p.ring < p.ring_on) p.ring = p.ring_on;
     } else {
         p.ring_on = p.ring = model_ring_panels(c, false);
@@ -944,16 +985,13 @@ size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute
 }
 
 template <int C_STATIC>
-static const void* model_kernel_of(bool strided, bool big) {
-    if (big)
-        return strided ? reinterpret_cast<const void*>(model_kernel<C_STATIC, true, true>)
-                       : reinterpret_cast<const void*>(model_kernel<C_STATIC, false, true>);
-    return strided ? reinterpret_cast<const void*>(model_kernel<C_STATIC, true, false>)
-                   : reinterpret_cast<const void*>(model_kernel<C_STATIC, false, false>);
+static const void* model_kernel_of(bool big) {
+    return big ? reinterpret_cast<const void*>(model_kernel<C_STATIC, true>) : reinterpret_cast<const void*>(model_kernel<C_STATIC, false>);
 }
 
 cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtensorMap* tm_q, const CUtensorMap* tm_k,
-                         const ModelLayerIO* layers, int n_layers, cudaStream_t stream) {
+                         const CUtensorMap* tm_rk, const CUtensorMap* tm_rv, const ModelLayerIO* layers, int n_layers,
+                         cudaStream_t stream) {
     ModelParams* pp = new ModelParams();        // too large for the host stack frame of every caller; copied at launch
     ModelParams& p = *pp;
     int n_compute = 0;
@@ -976,15 +1014,15 @@ cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtenso
     p.n_compute = n_compute;
     p.L = io.L; p.P = io.L - io.w; p.w = io.w; p.R = io.R; p.d = io.d; p.n_mt = plan.n_mt;
     p.sl2 = io.sl2;
-    p.k_row_bytes = 2 * (io.k_row_elems ? io.k_row_elems : io.d);
-    p.v_row_bytes = 2 * (io.v_row_elems ? io.v_row_elems : io.d);
-    p.k_head_bytes = 2 * (io.k_head_elems ? io.k_head_elems : static_cast<long long>(io.L) * io.d);
-    p.v_head_bytes = 2 * (io.v_head_elems ? io.v_head_elems : static_cast<long long>(io.L) * io.d);
+    p.strided = tm_rk != nullptr ? 1 : 0;
+    p.copy_box_bytes = (plan.c_static < io.L ? plan.c_static : io.L) * io.d * 2;
+    if (p.strided)
+        for (int i = 0; i < n_layers; ++i) { p.tm_rk[i] = tm_rk[i]; p.tm_rv[i] = tm_rv[i]; }
     p.cph = plan.cph; p.n_tiles = plan.n_tiles; p.n_stages = plan.n_stages;
     p.q_box_rows = io.R < 128 ? io.R : 128;
     p.k_box_rows = io.L < plan.tile ? io.L : plan.tile;
     p.C = io.C; p.k = io.k; p.n_max = io.n_max; p.Hkv = io.Hkv;
-    p.ring_on = plan.ring_on; p.ring = plan.ring; p.copy_slots = plan.copy_slots;
+    p.ring_on = plan.ring_on; p.ring = plan.ring; p.ahead = plan.ahead; p.stride = plan.stride; p.copy_slots = plan.copy_slots;
     p.Cpad = (io.C + 3) & ~3;
     p.n_score = plan.n_score; p.n_sel = plan.n_sel;
     p.sel_row_bytes = plan.sel_row_bytes; p.sel_keys_fit = plan.sel_keys_fit;
@@ -999,20 +1037,19 @@ cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtenso
     p.cnt_b = io.counters + 16 + kResidentMaxHeads;
     p.cnt_c = io.counters + 16 + 2 * kResidentMaxHeads;
     p.status = io.status;
-    const bool strided = io.k_row_elems != 0 || io.v_row_elems != 0 || io.k_head_elems != 0 || io.v_head_elems != 0;
     const void* kern = nullptr;
     int v = 0;
     switch (plan.c_static) {
-        case 5: kern = model_kernel_of<5>(strided, plan.big); v = 0; break;
-        case 8: kern = model_kernel_of<8>(strided, plan.big); v = 1; break;
-        case 10: kern = model_kernel_of<10>(strided, plan.big); v = 2; break;
-        case 16: kern = model_kernel_of<16>(strided, plan.big); v = 3; break;
-        case 20: kern = model_kernel_of<20>(strided, plan.big); v = 4; break;
-        case 32: kern = model_kernel_of<32>(strided, plan.big); v = 5; break;
+        case 5: kern = model_kernel_of<5>(plan.big); v = 0; break;
+        case 8: kern = model_kernel_of<8>(plan.big); v = 1; break;
+        case 10: kern = model_kernel_of<10>(plan.big); v = 2; break;
+        case 16: kern = model_kernel_of<16>(plan.big); v = 3; break;
+        case 20: kern = model_kernel_of<20>(plan.big); v = 4; break;
+        case 32: kern = model_kernel_of<32>(plan.big); v = 5; break;
         default: break;
     }
-    v += (strided ? 6 : 0) + (plan.big ? 12 : 0);
-    static int smem_set[24][64] = {{0}};
+    v += plan.big ? 6 : 0;
+    static int smem_set[12][64] = {{0}};
     int dev = 0;
     cudaError_t e = kern != nullptr ? cudaGetDevice(&dev) : cudaErrorInvalidValue;
     if (e == cudaSuccess && (dev < 0 || dev >= 64 || smem_set[v][dev] < plan.smem_bytes)) {
