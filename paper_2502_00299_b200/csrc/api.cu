@@ -242,32 +242,34 @@ int run_score(DeviceCtx& ctx, const void* q_obs, const void* K, int L, int Hq, i
         }
     }
     TokenPlan tplan;
-    if (c == 1 && make_token_plan(L, w, R, sh.Hs, d, ctx.num_sms, smem_budget(ctx), &tplan)) {
+    const int rows = w * (Hq / Hkv);
+    if (c == 1 && make_token_plan(L, w, rows, Hkv, d, ctx.num_sms, smem_budget(ctx), &tplan)) {
         // token scores: two passes over the keys in one launch, nothing but row records in scratch
-        const size_t tfloats = extra_payload_floats + pair_floats + static_cast<size_t>(tplan.grid) * 256;
+        const size_t pair_t = tplan.n_mt == 2 ? round64(static_cast<size_t>(tplan.Hs) * C) : 0;
+        const size_t tfloats = extra_payload_floats + pair_t + static_cast<size_t>(tplan.grid) * 256;
         int st2 = ensure_workspace(ctx, tfloats * sizeof(float));
         if (st2 != CHUNKKV_OK) return st2;
         float* payload = reinterpret_cast<float*>(static_cast<char*>(ctx.ws) + kHeaderBytes);
         if (out_scores == nullptr) out_scores = payload;
         if (resolved != nullptr) *resolved = out_scores;
-        float* head_scores = sh.shift ? payload + extra_payload_floats : out_scores;
+        float* head_scores = pair_t ? payload + extra_payload_floats : out_scores;
         CUtensorMap tq, tk;
-        st2 = encode_bf16_3d(&tq, q_obs, d, R, sh.Hs, R < 128 ? R : 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+        st2 = encode_bf16_3d(&tq, q_obs, d, rows, Hkv, 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
         if (st2 != CHUNKKV_OK) return st2;
-        st2 = encode_bf16_3d(&tk, K, d, L, Hkv, L < 120 ? L : 120, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, k_row_elems, k_head_elems);
+        st2 = encode_bf16_3d(&tk, K, d, L, Hkv, L < 128 ? L : 128, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, k_row_elems, k_head_elems);
         if (st2 != CHUNKKV_OK) return st2;
         TokenIO io;
-        io.L = L; io.w = w; io.Rs = R; io.Hs = sh.Hs; io.d = d; io.kv_shift = sh.shift;
+        io.L = L; io.w = w; io.R = rows; io.d = d;
         io.sl2 = static_cast<float>(1.4426950408889634 / sqrt(static_cast<double>(d)));
         io.token_scores = head_scores;
-        io.scratch = payload + extra_payload_floats + pair_floats;
+        io.scratch = payload + extra_payload_floats + pair_t;
         io.counters = reinterpret_cast<unsigned*>(static_cast<char*>(ctx.ws) + kResidentCountersOffset);
         io.status = static_cast<int*>(ctx.ws);
         cudaError_t e2;
         {
             Timer t(&ctx, stream, 0);
             e2 = launch_token_scores(tplan, tq, tk, io, stream);
-            if (e2 == cudaSuccess && sh.shift) e2 = launch_pair_sum(head_scores, out_scores, Hkv, C, stream);
+            if (e2 == cudaSuccess && pair_t) e2 = launch_pair_sum(head_scores, out_scores, Hkv, C, stream);
         }
         if (e2 != cudaSuccess) return cuda_fail(e2);
         return CHUNKKV_OK;
@@ -489,11 +491,12 @@ int chunkkv_score(const void* q_obs, const void* K, int L, int Hq, int Hkv, int 
     st = get_ctx(&ctx);
     if (st != CHUNKKV_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    st = run_score(*ctx, q_obs, K, L, Hq, Hkv, d, w, c, out_chunk_scores, 0, nullptr, s);
-    if (st != CHUNKKV_OK) return st;
-    if (out_token_scores != nullptr)
-        st = run_score(*ctx, q_obs, K, L, Hq, Hkv, d, w, 1, out_token_scores, 0, nullptr, s);
-    return st;
+    if (out_token_scores == nullptr) return run_score(*ctx, q_obs, K, L, Hq, Hkv, d, w, c, out_chunk_scores, 0, nullptr, s);
+    // with the token scores at hand a chunk's score is a sum of c of them: no second pass over keys and exponentials
+    st = run_score(*ctx, q_obs, K, L, Hq, Hkv, d, w, 1, out_token_scores, 0, nullptr, s);
+    if (st != CHUNKKV_OK || L == w) return st;
+    cudaError_t e = launch_chunk_sum(out_token_scores, out_chunk_scores, Hkv, L - w, c, s);
+    return e == cudaSuccess ? CHUNKKV_OK : cuda_fail(e);
 }
 
 int chunkkv_select(const float* chunk_scores, int L, int Hkv, int w, int c, int budget,
@@ -606,7 +609,7 @@ static int compress_impl(const void* q_obs, const void* K, const void* V, int L,
         TokenPlan tplan;
         // token-level layers on the whole GPU: the two-pass token-score kernel, then select and gather
         const bool token_path = c == 1 && lane == nullptr && rows_elsewhere == nullptr &&
-                                make_token_plan(L, w, R, sh.Hs, d, ctx->num_sms, smem_budget(*ctx), &tplan);
+                                make_token_plan(L, w, w * (Hq / Hkv), Hkv, d, ctx->num_sms, smem_budget(*ctx), &tplan);
         if (!token_path && make_score_plan(L, R, sh.Hs, d, c, ctas, smem_budget(*ctx), true, &plan)) {
             // One cooperative launch for the whole layer.
             const size_t need = (cs_floats + score_scratch_floats(plan, sh.Hs, R)) * sizeof(float);

@@ -169,19 +169,23 @@ cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtenso
 
 // Token scores in one launch, two passes over the keys (token_kernel.cu).
 struct TokenPlan {
+    int n_mt, Hs;         // scoring heads per KV head (1 or 2: more than 128 rows), in all
     int grid, cph, n_tiles, n_tiles_prefix, n_stages, smem_bytes, off_ring, off_misc;
 };
 struct TokenIO {
-    int L, w, Rs, Hs, d, kv_shift;
+    int L, w, R, d;       // R = w * Hq / Hkv query rows per KV head
     float sl2;
     float* token_scores;  // [Hs][P]
     float* scratch;       // grid * 256 floats
     unsigned* counters;   // header + kResidentCountersOffset
     int* status;
 };
-bool make_token_plan(int L, int w, int Rs, int Hs, int d, int max_ctas, int smem_limit, TokenPlan* plan);
+bool make_token_plan(int L, int w, int R, int Hkv, int d, int max_ctas, int smem_limit, TokenPlan* plan);
+// tm_q: [Hkv heads, R rows] with boxes of 128 rows; tm_k: boxes of min(L, 128) rows.
 cudaError_t launch_token_scores(const TokenPlan& plan, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                                 const TokenIO& io, cudaStream_t stream);
+// out[h][ch] = sum of the token scores of chunk ch (the last one clipped at P).
+cudaError_t launch_chunk_sum(const float* token_scores, float* out, int Hkv, int P, int c, cudaStream_t stream);
 
 cudaError_t launch_finalize(const ScorePlan& plan, const ScoreArgs& args, int C, float* out_scores,
                             int num_sms, cudaStream_t stream);

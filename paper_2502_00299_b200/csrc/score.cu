@@ -1144,6 +1144,54 @@ finalize_panels_kernel(const ScoreArgs a, const FinGeom g, float* __restrict__ o
     contract_panels_aligned<RV, PP, SB>(a, g, h, p_lo, p_hi, rs, rs + 256, out);
 }
 
+// A thread per chunk (its token scores come through the L1, which the chunks of a warp share), or a warp per chunk of
+// many tokens; fixed order of summation either way.
+template <bool WARP>
+__global__ void __launch_bounds__(256)
+chunk_sum_kernel(const float* tokens, float* out, int P, int c, int C, size_t n) {
+    // launched as a programmatic dependent of the token-score kernel
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const size_t t = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const size_t i = WARP ? t >> 5 : t;
+    if (i >= n) return;
+    const size_t h = i / C;
+    const int ch = static_cast<int>(i - h * C), j0 = ch * c, len = min(c, P - j0);
+    const float* src = tokens + h * P + j0;
+    float s = 0.f;
+    if constexpr (WARP) {
+        const int lane = threadIdx.x & 31;
+        for (int u = lane; u < len; u += 32) s += src[u];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane == 0) out[i] = s;
+    } else {
+        float s1 = 0.f;
+#pragma unroll 4
+        for (int u = 0; u + 1 < len; u += 2) { s += src[u]; s1 += src[u + 1]; }
+        if (len & 1) s += src[len - 1];
+        out[i] = s + s1;
+    }
+}
+
+cudaError_t launch_chunk_sum(const float* token_scores, float* out, int Hkv, int P, int c, cudaStream_t stream) {
+    const int C = (P + c - 1) / c;
+    const size_t n = static_cast<size_t>(Hkv) * C;
+    if (n == 0) return cudaSuccess;
+    const bool warp = c > 64;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>((n * (warp ? 32 : 1) + 255) / 256));
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (warp) return cudaLaunchKernelEx(&cfg, chunk_sum_kernel<true>, token_scores, out, P, c, C, n);
+    return cudaLaunchKernelEx(&cfg, chunk_sum_kernel<false>, token_scores, out, P, c, C, n);
+}
+
 cudaError_t launch_pair_sum(const float* in, float* out, int Hkv, int C, cudaStream_t stream) {
     const size_t n = static_cast<size_t>(Hkv) * C;
     if (n == 0) return cudaSuccess;

@@ -6,9 +6,14 @@
 // score matrix, so this kernel walks its keys twice instead, in one launch: pass 1 only folds the
 // per-row (max, sum) of the CTA's key range; the CTAs of a head exchange those records (one
 // bounded hand-over per head); pass 2 recomputes the same tiles (the keys come back from L2),
-// normalises every element with the final row statistics and sums over the 128 rows with a
-// transposing warp reduction, so only the token scores are written. Same tiling, producer / issuer
-// / epilogue roles and bounded waits as layer_resident.cu.
+// normalises every element with the final row statistics and sums over the rows. Pass 1 multiplies
+// query rows x keys (a thread owns a row, so maximum and sum over keys stay in the thread); pass 2 multiplies
+// keys x query rows - the same two shared-memory operands with their roles exchanged - so that a thread owns a
+// key and the sum over the rows stays in the thread as well: it stores token scores and nothing else. (With
+// rows in lanes in both passes the sum over rows was a transposing warp reduction, four instructions per element
+// and four warps to meet on every panel: 15 us of a 32768-token layer's pass 2, 128 rows, against the
+// special-function unit's 7; the layer went from 56.7 to 49.6 us.) Each of the four epilogue groups has an accumulator of its own, 128 keys x 128 rows.
+// A KV head with more than 128 query rows is scored as two heads of 128 and the rest.
 #include "internal.h"
 #include "panels.cuh"
 #include "ptx.cuh"
@@ -21,13 +26,17 @@ namespace chunkkv {
 namespace {
 
 constexpr int kTThreads = 576;
-constexpr int kTMiscBytes = 20480;     // group records, slices, m_i, 1 / l_i, per-group column sums (two buffers)
+constexpr int kTMiscBytes = 9216;      // group records, slices, m_i, 1 / l_i
+constexpr int kTPanel = 64;            // keys per epilogue panel in pass 1, query rows per step in pass 2
+constexpr int kTTile = 128;            // keys per tile: both operands of a product have 128 rows
+constexpr uint32_t kTStageBytes = kTTile * 128;
+constexpr int kTBufs = 4;              // accumulators of 128 columns: all of tensor memory, one per epilogue group
 
 struct TokCtl {
     unsigned long long full[kRMaxStages];
     unsigned long long empty[kRMaxStages];
-    unsigned long long tfull[2];
-    unsigned long long tempty[2];
+    unsigned long long tfull[kTBufs];
+    unsigned long long tempty[kTBufs];
     unsigned long long qfull;
     uint32_t tmem_base;
     int abort_flag;
@@ -35,7 +44,8 @@ struct TokCtl {
 };
 
 struct TokArgs {
-    int L, P, w, R, Hs, d, kv_shift;
+    int L, P, w, R, Hs, d;
+    int n_mt;              // scoring heads per KV head (1 or 2): scoring head v scores rows [128 (v % n_mt), ...) of KV head v / n_mt
     float sl2;
     int cph, n_tiles, n_tiles_prefix, n_stages, q_box_rows, k_box_rows;
     int off_ring, off_misc;
@@ -49,7 +59,7 @@ struct TokArgs {
 __global__ void __launch_bounds__(kTThreads, 1)
 token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const TokArgs a) {
-    constexpr uint32_t IDESC = umma_idesc_bf16(128, kRUmmaN);
+    constexpr uint32_t IDESC = umma_idesc_bf16(128, 128);
     extern __shared__ uint8_t smem_raw[];
     __shared__ TokCtl ctl;
 
@@ -62,14 +72,14 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     float* misc = reinterpret_cast<float*>(dyn + a.off_misc);
     float* rec = misc;                 // [4 groups][{max, sum}][128]
     float* slice = misc + 1024;        // [4 slices][{max, sum}][128]
-    float* gm = misc + 2048;           // [128]
-    float* ginv = misc + 2176;         // [128]
-    float* qsum = misc + 2304;         // [4 groups][2 buffers][4 lane quarters][64]
+    float* nrm = misc + 2048;          // [128] -m_i
+    float* inv = misc + 2176;          // [128] 1 / l_i
     volatile int* abort_flag = &ctl.abort_flag;
     const uint32_t n_stages = static_cast<uint32_t>(a.n_stages);
 
     const int hs = blockIdx.x / a.cph, part = blockIdx.x - hs * a.cph;
-    const int hkv = hs >> a.kv_shift;
+    const int hkv = a.n_mt == 2 ? hs >> 1 : hs, row0 = a.n_mt == 2 ? (hs & 1) * 128 : 0;
+    const int R = min(128, a.R - row0);              // rows of this scoring head
     const int t_begin = a.n_tiles * part / a.cph, t_end = a.n_tiles * (part + 1) / a.cph;
     const int nt = t_end - t_begin;
     const int nt2 = max(0, min(t_end, a.n_tiles_prefix) - t_begin);   // tiles of pass 2: those that hold prefix keys
@@ -79,18 +89,20 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             mbar_init(smem_u32(&ctl.full[s]), 1);
             mbar_init(smem_u32(&ctl.empty[s]), 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < kTBufs; ++b) {
             mbar_init(smem_u32(&ctl.tfull[b]), 1);
-            mbar_init(smem_u32(&ctl.tempty[b]), 8);
+            mbar_init(smem_u32(&ctl.tempty[b]), 4);
         }
         mbar_init(smem_u32(&ctl.qfull), 1);
         ctl.abort_flag = 0;
         ctl.wait_ok = 1;
+        prefetch_tmap(&tm_q);            // (kernel parameters: not written by the kernel ahead of this one)
+        prefetch_tmap(&tm_k);
         fence_mbar_init();
         fence_proxy_async();
     }
     if (warp == 1) {
-        tmem_alloc(smem_u32(&ctl.tmem_base), 256);
+        tmem_alloc(smem_u32(&ctl.tmem_base), 512);
         tmem_relinquish();
     }
     tc_fence_before();
@@ -105,12 +117,10 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer: the key range, twice
         if (elect_one() && nt > 0) {
-            prefetch_tmap(&tm_q);
-            prefetch_tmap(&tm_k);
             const uint32_t qbar = smem_u32(&ctl.qfull);
             mbar_arrive_expect_tx(qbar, static_cast<uint32_t>(KB * a.q_box_rows) * 128u);
             for (int kb = 0; kb < KB; ++kb)
-                tma_load_3d(q_base + static_cast<uint32_t>(kb) * kRQTileBytes, &tm_q, qbar, kb * 64, 0, hs);
+                tma_load_3d(q_base + static_cast<uint32_t>(kb) * kRQTileBytes, &tm_q, qbar, kb * 64, row0, hkv);   // (rows past R arrive as zeros)
             const uint32_t k_bytes = static_cast<uint32_t>(a.k_box_rows) * 128u;
             uint32_t st = 0, st_par = 1;
             int issued = 0;
@@ -125,7 +135,7 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                         if (!ok) break;
                         const uint32_t bar = smem_u32(&ctl.full[st]);
                         mbar_arrive_expect_tx(bar, k_bytes);
-                        tma_load_3d(k_base + st * kRStageBytes, &tm_k, bar, kb * 64, t * kRTile, hkv);
+                        tma_load_3d(k_base + st * kTStageBytes, &tm_k, bar, kb * 64, t * kTTile, hkv);
                         ++issued;
                         if (++st == n_stages) { st = 0; st_par ^= 1u; }
                     }
@@ -148,19 +158,21 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             bool ok = mbar_wait(smem_u32(&ctl.qfull), 0, abort_flag);
             uint32_t st = 0, st_par = 0;
             for (int tg = 0; tg < nt + nt2 && ok; ++tg) {
-                const int buf = tg & 1, use = tg >> 1;
+                const int buf = tg % kTBufs, use = tg / kTBufs;
                 ok = mbar_wait(smem_u32(&ctl.tempty[buf]), (use & 1) ^ 1, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t d_addr = tmem_base + static_cast<uint32_t>(buf * kRUmmaN);
+                const uint32_t d_addr = tmem_base + static_cast<uint32_t>(buf * 128);
+                const bool keys_first = tg >= nt;        // pass 2: lanes are keys
 #pragma unroll
                 for (int kb = 0; kb < 2; ++kb) {
                     if (kb >= KB || !ok) break;
                     ok = mbar_wait(smem_u32(&ctl.full[st]), st_par, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint64_t b_desc = umma_desc_sw128(k_base + st * kRStageBytes);
-                    const uint64_t a_desc = umma_desc_sw128(q_base + static_cast<uint32_t>(kb) * kRQTileBytes);
+                    const uint64_t k_desc = umma_desc_sw128(k_base + st * kTStageBytes);
+                    const uint64_t q_desc = umma_desc_sw128(q_base + static_cast<uint32_t>(kb) * kRQTileBytes);
+                    const uint64_t a_desc = keys_first ? k_desc : q_desc, b_desc = keys_first ? q_desc : k_desc;
 #pragma unroll
                     for (int k4 = 0; k4 < 4; ++k4)
                         umma_bf16(d_addr, a_desc + 2u * k4, b_desc + 2u * k4, IDESC, (kb > 0 || k4 > 0) ? 1u : 0u);
@@ -174,36 +186,40 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         // ------------------------------------------------------------------ epilogue
         const int et = threadIdx.x - 64;
         const int grp = (warp - 2) >> 2, quarter = warp & 3;
-        const int pair = grp >> 1, half = grp & 1;
-        const int row = quarter * 32 + lane;
-        const bool active = row < a.R;
-        const int last_visible = a.P + (row % a.w);
-        const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+        const int row = quarter * 32 + lane;             // lane of tensor memory: query row in pass 1, key in pass 2
+        const bool active = row < R;
+        const int last_visible = a.P + ((row0 + row) % a.w);
+        const uint32_t acc = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(grp * 128);
+        int tg = grp;                                    // this group's next tile, counted over both passes; tile tg uses accumulator tg % 4
         // ---- pass 1: (max, sum of exp2) per row over this CTA's keys
         float run_m = -CUDART_INF_F, run_l = 0.f;
-        for (int ti = pair; ti < nt; ti += 2) {
-            const int use = ti >> 1;
+        for (; tg < nt; tg += kTBufs) {
             bool ready = true;
-            if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[pair]), use & 1, abort_flag);
+            if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[grp]), (tg / kTBufs) & 1, abort_flag);
             if (!__shfl_sync(0xffffffffu, ready, 0)) break;
             tc_fence_after();
-            float v[kRPanel];
-            load_panel<kRPanel>(lane_addr + static_cast<uint32_t>(pair * kRUmmaN + half * kRPanel), v);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&ctl.tempty[pair]));
-            const int j0 = (t_begin + ti) * kRTile + half * kRPanel;
-            float m2, l;
-            auto emit = [](int, float) {};
-            if (j0 + kRPanel <= a.P)
-                panel_fast<10, kRPanel>(v, a.sl2, emit, &m2, &l);
-            else
-                panel_static_tail<10, kRPanel>(v, a.sl2, emit, j0, a.P, last_visible, &m2, &l);
-            const float nm = fmaxf(run_m, m2);
-            const float s_old = (run_m == -CUDART_INF_F) ? 0.f : ex2_approx(run_m - nm);
-            const float s_new = (m2 == -CUDART_INF_F) ? 0.f : ex2_approx(m2 - nm);
-            run_l = run_l * s_old + l * s_new;
-            run_m = nm;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                float v[kTPanel];
+                load_panel<kTPanel>(acc + static_cast<uint32_t>(half * kTPanel), v);
+                if (half == 1) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&ctl.tempty[grp]));
+                }
+                const int j0 = (t_begin + tg) * kTTile + half * kTPanel;
+                float m2, l;
+                auto emit = [](int, float) {};
+                if (j0 + kTPanel <= a.P)
+                    panel_fast<8, kTPanel>(v, a.sl2, emit, &m2, &l);
+                else
+                    panel_static_tail<8, kTPanel>(v, a.sl2, emit, j0, a.P, last_visible, &m2, &l);
+                const float nm = fmaxf(run_m, m2);
+                const float s_old = (run_m == -CUDART_INF_F) ? 0.f : ex2_approx(run_m - nm);
+                const float s_new = (m2 == -CUDART_INF_F) ? 0.f : ex2_approx(m2 - nm);
+                run_l = run_l * s_old + l * s_new;
+                run_m = nm;
+            }
         }
         rec[(grp * 2 + 0) * 128 + row] = active ? run_m : -CUDART_INF_F;
         rec[(grp * 2 + 1) * 128 + row] = active ? run_l : 0.f;
@@ -221,19 +237,15 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             }
             named_barrier(1, 512);
             if (et == 0) {
-                unsigned old;
-                asm volatile("atom.add.release.gpu.u32 %0, [%1], 1;" : "=r"(old) : "l"(a.cnt_a + hs) : "memory");
+                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.cnt_a + hs) : "memory");
                 bool w_ok = true;
-                if (old + 1u < static_cast<unsigned>(a.cph)) {
-                    const long long t0 = clock64();
+                const long long t0 = clock64();
+                for (;;) {
                     unsigned cur;
-                    for (;;) {
-                        asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(cur) : "l"(a.cnt_a + hs) : "memory");
-                        if (cur >= static_cast<unsigned>(a.cph)) break;
-                        if (clock64() - t0 > kWaitLimitClocks) { w_ok = false; ctl.abort_flag = 1; break; }
-                    }
+                    asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(cur) : "l"(a.cnt_a + hs) : "memory");
+                    if (cur >= static_cast<unsigned>(a.cph)) break;
+                    if (clock64() - t0 > kWaitLimitClocks) { w_ok = false; ctl.abort_flag = 1; break; }
                 }
-                asm volatile("fence.acq_rel.gpu;" ::: "memory");
                 ctl.wait_ok = w_ok ? 1 : 0;
             }
             named_barrier(1, 512);
@@ -243,16 +255,16 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             const int i = et & 127, sl = et >> 7;
             const float* src = a.cta_stat + static_cast<size_t>(hs) * a.cph * 256 + i;
             float M = -CUDART_INF_F, Ls = 0.f;
-            for (int j0 = sl; j0 < a.cph; j0 += 16) {
-                float rm[4], rl[4];
+            for (int j0 = sl; j0 < a.cph; j0 += 20) {        // five records in flight per thread
+                float rm[5], rl[5];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
+                for (int u = 0; u < 5; ++u) {
                     const int j = j0 + 4 * u;
                     rm[u] = (j < a.cph) ? __ldcg(src + static_cast<size_t>(j) * 256) : -CUDART_INF_F;
                     rl[u] = (j < a.cph) ? __ldcg(src + static_cast<size_t>(j) * 256 + 128) : 0.f;
                 }
 #pragma unroll
-                for (int u = 0; u < 4; ++u) merge_ml(M, Ls, rm[u], rl[u]);
+                for (int u = 0; u < 5; ++u) merge_ml(M, Ls, rm[u], rl[u]);
             }
             slice[(sl * 2 + 0) * 128 + i] = M;
             slice[(sl * 2 + 1) * 128 + i] = Ls;
@@ -261,47 +273,49 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 float M2 = -CUDART_INF_F, L2 = 0.f;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) merge_ml(M2, L2, slice[(q * 2) * 128 + et], slice[(q * 2 + 1) * 128 + et]);
-                gm[et] = M2;
-                ginv[et] = log2f(L2);          // the normaliser goes into the exponent: exp2(s - m_i - log2 l_i)
+                // (a row past R is all zeros, its scores 0: a maximum beyond every exponent makes its share 0)
+                nrm[et] = et < R ? -M2 : -1e30f;
+                inv[et] = et < R ? 1.0f / L2 : 0.f;
             }
             named_barrier(1, 512);
-            // ---- pass 2: the same tiles again, normalised, summed over the rows
-            const float nm = active ? -(gm[row] + ginv[row]) : 0.f;
+            // ---- pass 2: the same tiles again, backwards, keys in lanes: normalised and summed over the rows
             float* out = a.token_scores + static_cast<size_t>(hs) * a.P;
-            int mine = 0;                                  // tiles this group has taken in pass 2 (column-sum buffer = mine & 1)
-            for (int ti = (pair - (nt & 1)) & 1; ti < nt2; ti += 2, ++mine) {
-                const int tg = nt + ti, use = tg >> 1;
+            const unsigned long long s2 = pack2(a.sl2, a.sl2);
+            const int n_half = R > kTPanel ? 2 : 1;
+            for (; tg < nt + nt2; tg += kTBufs) {
                 bool ready = true;
-                if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[pair]), use & 1, abort_flag);
-                ready = __shfl_sync(0xffffffffu, ready, 0);
-                float* qs = qsum + ((grp * 2 + (mine & 1)) * 4 + quarter) * 64;
-                if (ready) {
-                    tc_fence_after();
-                    float v[kRPanel];
-                    load_panel<kRPanel>(lane_addr + static_cast<uint32_t>(pair * kRUmmaN + half * kRPanel), v);
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&ctl.tempty[pair]));
-#pragma unroll
-                    for (int b = 0; b < 2; ++b) {
-                        float x[32];
-#pragma unroll
-                        for (int u = 0; u < 30; ++u)      // (an inactive row holds garbage: select, do not multiply)
-                            x[u] = active ? ex2_approx(fmaf(v[b * 30 + u], a.sl2, nm)) : 0.f;
-                        x[30] = 0.f;
-                        x[31] = 0.f;
-                        const float tot = warp_transpose_reduce(x, lane);
-                        if (lane < 30) qs[b * 30 + lane] = tot;
+                if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[grp]), (tg / kTBufs) & 1, abort_flag);
+                if (!__shfl_sync(0xffffffffu, ready, 0)) break;
+                tc_fence_after();
+                float t = 0.f;
+                for (int half = 0; half < n_half; ++half) {
+                    float v[kTPanel];
+                    load_panel<kTPanel>(acc + static_cast<uint32_t>(half * kTPanel), v);
+                    if (half == n_half - 1) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&ctl.tempty[grp]));
                     }
+                    const float4* n4 = reinterpret_cast<const float4*>(nrm + half * kTPanel);
+                    const float4* i4 = reinterpret_cast<const float4*>(inv + half * kTPanel);
+                    // eight chains of eight terms, added as a tree
+                    unsigned long long sum[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+                    for (int u = 0; u < kTPanel / 4; ++u) {
+                        const float4 n = n4[u], iv = i4[u];              // (the same address in every lane)
+                        float x0, x1, x2, x3;
+                        unpack2(fma2(pack2(v[4 * u], v[4 * u + 1]), s2, pack2(n.x, n.y)), x0, x1);
+                        unpack2(fma2(pack2(v[4 * u + 2], v[4 * u + 3]), s2, pack2(n.z, n.w)), x2, x3);
+                        unsigned long long* a2 = &sum[2 * (u & 1)];
+                        a2[0] = fma2(pack2(ex2_approx(x0), ex2_approx(x1)), pack2(iv.x, iv.y), a2[0]);
+                        a2[1] = fma2(pack2(ex2_approx(x2), ex2_approx(x3)), pack2(iv.z, iv.w), a2[1]);
+                    }
+                    float lo, hi;
+                    unpack2(add2(add2(sum[0], sum[1]), add2(sum[2], sum[3])), lo, hi);
+                    t += lo + hi;
                 }
-                named_barrier(2 + grp, 128);               // the four lane quarters of this panel are in shared memory
-                if (ctl.abort_flag) break;                 // same answer in the four warps of the group
-                const int gt = threadIdx.x - 64 - grp * 128;   // 0 .. 127 within the group
-                const int j = (t_begin + nt2 - 1 - ti) * kRTile + half * kRPanel + gt;      // (pass 2 runs backwards)
-                if (gt < kRPanel && j < a.P) {
-                    const float* q0 = qsum + ((grp * 2 + (mine & 1)) * 4) * 64 + gt;
-                    out[j] = (q0[0] + q0[64]) + (q0[128] + q0[192]);
-                }
+                const int j = (t_begin + nt2 - 1 - (tg - nt)) * kTTile + row;
+                if (j < a.P) out[j] = t;
             }
         }
     }
@@ -310,7 +324,7 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 256);
+        tmem_dealloc(tmem_base, 512);
     }
     if (threadIdx.x == 0) {
         if (ctl.abort_flag) atomicExch(a.status, 1);
@@ -325,23 +339,26 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 
 }  // namespace
 
-bool make_token_plan(int L, int w, int Rs, int Hs, int d, int max_ctas, int smem_limit, TokenPlan* plan) {
-    if (Rs < 1 || Rs > 128 || (d != 64 && d != 128) || L < 1 || L - w < 1 || Hs < 1 || Hs > kResidentMaxHeads) return false;
+bool make_token_plan(int L, int w, int R, int Hkv, int d, int max_ctas, int smem_limit, TokenPlan* plan) {
+    const int n_mt = R > 128 ? 2 : 1, Hs = Hkv * n_mt;
+    if (R < 1 || R > 256 || (d != 64 && d != 128) || L < 1 || L - w < 1 || Hs < 1 || Hs > kResidentMaxHeads) return false;
     if (max_ctas < Hs) return false;
     TokenPlan p{};
+    p.n_mt = n_mt;
+    p.Hs = Hs;
     p.cph = max_ctas / Hs;
     p.grid = p.cph * Hs;
-    p.n_tiles = (L + kRTile - 1) / kRTile;
-    p.n_tiles_prefix = (L - w + kRTile - 1) / kRTile;
+    p.n_tiles = (L + kTTile - 1) / kTTile;
+    p.n_tiles_prefix = (L - w + kTTile - 1) / kTTile;
     const int KB = d / 64;
     const int q_bytes = KB * kRQTileBytes;
     const int fixed = 1024 + q_bytes + 1024 + kTMiscBytes;
-    int ns = (smem_limit - fixed) / kRStageBytes;
+    int ns = (smem_limit - fixed) / static_cast<int>(kTStageBytes);
     if (ns > kRMaxStages) ns = kRMaxStages;
     if (ns < 2 * KB) return false;
     p.n_stages = ns;
     p.off_ring = q_bytes;
-    p.off_misc = p.off_ring + ns * kRStageBytes + 1024;
+    p.off_misc = p.off_ring + ns * static_cast<int>(kTStageBytes) + 1024;
     p.smem_bytes = 1024 + p.off_misc + kTMiscBytes;
     *plan = p;
     return true;
@@ -350,11 +367,11 @@ bool make_token_plan(int L, int w, int Rs, int Hs, int d, int max_ctas, int smem
 cudaError_t launch_token_scores(const TokenPlan& plan, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                                 const TokenIO& io, cudaStream_t stream) {
     TokArgs a{};
-    a.L = io.L; a.P = io.L - io.w; a.w = io.w; a.R = io.Rs; a.Hs = io.Hs; a.d = io.d; a.kv_shift = io.kv_shift;
+    a.L = io.L; a.P = io.L - io.w; a.w = io.w; a.R = io.R; a.Hs = plan.Hs; a.d = io.d; a.n_mt = plan.n_mt;
     a.sl2 = io.sl2;
     a.cph = plan.cph; a.n_tiles = plan.n_tiles; a.n_tiles_prefix = plan.n_tiles_prefix; a.n_stages = plan.n_stages;
-    a.q_box_rows = io.Rs < 128 ? io.Rs : 128;
-    a.k_box_rows = io.L < kRTile ? io.L : kRTile;
+    a.q_box_rows = 128;                  // (rows past R arrive as zeros)
+    a.k_box_rows = io.L < kTTile ? io.L : kTTile;
     a.off_ring = plan.off_ring; a.off_misc = plan.off_misc;
     a.cta_stat = io.scratch;
     a.token_scores = io.token_scores;

@@ -98,3 +98,22 @@ def test_model_call(ck, Hq, Hkv, d, L, w, c, n_layers, n_reuse):
     major = [(q, *(a.permute(1, 0, 2).contiguous().permute(1, 0, 2) for a in (K, V))) for q, K, V in on]
     for a, b in zip(ck.compress_model_strided([major[p] for p in pick], Hq, w, c, budget, n_reuse), outs):
         assert all(torch.equal(s, t) for s, t in zip(a, b))
+
+
+# token scores: 128-key tiles, one or two scoring heads per KV head (128 rows and the rest), two passes
+@pytest.mark.parametrize("Hq,Hkv,d,L,w,c", [
+    (8, 2, 64, 2048, 16, 7), (28, 4, 128, 1500, 32, 13), (15, 3, 64, 1203, 43, 300), (4, 1, 128, 129, 1, 100), (64, 8, 128, 20 * 128, 32, 64),
+    (32, 8, 64, 18 * 128 * 5 + 1, 16, 3), (4, 2, 128, 40, 32, 65), (256, 1, 64, 700, 1, 1), (4, 4, 64, 127 + 16, 16, 2),
+])
+def test_token_scores_and_chunk_scores_with_and_without_them(ck, Hq, Hkv, d, L, w, c):
+    wl, x = _layer(Hq, Hkv, d, L, w, c, w, seed=L + c)
+    q, K = to_dev(x.q_obs), to_dev(x.K)
+    t = ora.token_scores(x.q_obs, x.K, Hq, Hkv, w)
+    s = ora.chunk_scores(t, c)
+    cs, ts = ck.score(q, K, w, c, want_token_scores=True)
+    alone, none = ck.score(q, K, w, c)
+    assert ck.device_status() == 0 and none is None
+    R = w * Hq // Hkv
+    assert_scores_close(ts.cpu().numpy(), t, R, L, "token scores")
+    assert_scores_close(cs.cpu().numpy(), s, R, L, "chunk scores beside token scores")
+    assert_scores_close(alone.cpu().numpy(), s, R, L, "chunk scores alone")
