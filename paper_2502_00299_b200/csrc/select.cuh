@@ -71,7 +71,7 @@ __device__ __forceinline__ uint32_t select_order_key(float x) {
 // memory: warp v owns a block of consecutive ids and walks it in rows of 32, one id per lane, with ballots for the order.
 // Totals of warps are combined by one shared-memory read per lane and a warp reduction.
 // 3274 keys, 640 threads, in clocks: 11.2k with scalar loads (2.2k), a loop over the warps for the minimum and maximum
-// (1.1k) and branches per key for the candidates (1.2k) and the list (2.1k); about 6.5k in this form.
+// (1.1k) and branches per key for the candidates (1.2k) and the list (2.1k); 7.2k in this form (a selector CTA of the model kernel; 12.2k there before).
 constexpr int kSelBins = 2048;
 constexpr int kSelCandCap = 128;
 
