@@ -20,6 +20,7 @@
 #include "resident.cuh"
 
 #include <math_constants.h>
+#include <type_traits>
 
 namespace chunkkv {
 
@@ -273,8 +274,7 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 float M2 = -CUDART_INF_F, L2 = 0.f;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) merge_ml(M2, L2, slice[(q * 2) * 128 + et], slice[(q * 2 + 1) * 128 + et]);
-                // (a row past R is all zeros, its scores 0: a maximum beyond every exponent makes its share 0)
-                nrm[et] = et < R ? -M2 : -1e30f;
+                nrm[et] = -M2;
                 inv[et] = et < R ? 1.0f / L2 : 0.f;
             }
             named_barrier(1, 512);
@@ -282,6 +282,32 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             float* out = a.token_scores + static_cast<size_t>(hs) * a.P;
             const unsigned long long s2 = pack2(a.sl2, a.sl2);
             const int n_half = R > kTPanel ? 2 : 1;
+            // A key's sum over the rows r0 .. r0 + 63 of this scoring head, as eight chains of eight terms added as a tree. A
+            // column past R is left out by selection, not by a factor 0: it is the product of a zero row, which is NaN for a
+            // key with an infinite component.
+            auto sum_rows = [&](auto all, int r0, const float (&v)[kTPanel]) -> float {
+                constexpr bool ALL = decltype(all)::value;               // every one of the 64 rows exists
+                const float4* n4 = reinterpret_cast<const float4*>(nrm + r0);
+                const float4* i4 = reinterpret_cast<const float4*>(inv + r0);
+                unsigned long long sum[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+                for (int u = 0; u < kTPanel / 4; ++u) {
+                    const int left = ALL ? 4 : R - r0 - 4 * u;           // rows of this group of four
+                    if (left <= 0) break;
+                    const float4 n = n4[u], iv = i4[u];                  // (the same address in every lane)
+                    float x0, x1, x2, x3;
+                    unpack2(fma2(pack2(v[4 * u], v[4 * u + 1]), s2, pack2(n.x, n.y)), x0, x1);
+                    unpack2(fma2(pack2(v[4 * u + 2], v[4 * u + 3]), s2, pack2(n.z, n.w)), x2, x3);
+                    const float e0 = ex2_approx(x0), e1 = left > 1 ? ex2_approx(x1) : 0.f;
+                    const float e2 = left > 2 ? ex2_approx(x2) : 0.f, e3 = left > 3 ? ex2_approx(x3) : 0.f;
+                    unsigned long long* a2 = &sum[2 * (u & 1)];
+                    a2[0] = fma2(pack2(e0, e1), pack2(iv.x, iv.y), a2[0]);
+                    a2[1] = fma2(pack2(e2, e3), pack2(iv.z, iv.w), a2[1]);
+                }
+                float lo, hi;
+                unpack2(add2(add2(sum[0], sum[1]), add2(sum[2], sum[3])), lo, hi);
+                return lo + hi;
+            };
             for (; tg < nt + nt2; tg += kTBufs) {
                 bool ready = true;
                 if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[grp]), (tg / kTBufs) & 1, abort_flag);
@@ -296,23 +322,7 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&ctl.tempty[grp]));
                     }
-                    const float4* n4 = reinterpret_cast<const float4*>(nrm + half * kTPanel);
-                    const float4* i4 = reinterpret_cast<const float4*>(inv + half * kTPanel);
-                    // eight chains of eight terms, added as a tree
-                    unsigned long long sum[4] = {0ull, 0ull, 0ull, 0ull};
-#pragma unroll
-                    for (int u = 0; u < kTPanel / 4; ++u) {
-                        const float4 n = n4[u], iv = i4[u];              // (the same address in every lane)
-                        float x0, x1, x2, x3;
-                        unpack2(fma2(pack2(v[4 * u], v[4 * u + 1]), s2, pack2(n.x, n.y)), x0, x1);
-                        unpack2(fma2(pack2(v[4 * u + 2], v[4 * u + 3]), s2, pack2(n.z, n.w)), x2, x3);
-                        unsigned long long* a2 = &sum[2 * (u & 1)];
-                        a2[0] = fma2(pack2(ex2_approx(x0), ex2_approx(x1)), pack2(iv.x, iv.y), a2[0]);
-                        a2[1] = fma2(pack2(ex2_approx(x2), ex2_approx(x3)), pack2(iv.z, iv.w), a2[1]);
-                    }
-                    float lo, hi;
-                    unpack2(add2(add2(sum[0], sum[1]), add2(sum[2], sum[3])), lo, hi);
-                    t += lo + hi;
+                    t += (half + 1) * kTPanel <= R ? sum_rows(std::true_type{}, half * kTPanel, v) : sum_rows(std::false_type{}, half * kTPanel, v);
                 }
                 const int j = (t_begin + nt2 - 1 - (tg - nt)) * kTTile + row;
                 if (j < a.P) out[j] = t;
