@@ -37,7 +37,8 @@ __device__ __forceinline__ void panel_fast(float (&v)[WP], float sl2, Emit emit,
         m1 = fmax3(m1, v[u + 2], v[u + 3]);
     }
     const float mx = fmaxf(m0, m1);
-    const float neg_m2 = -mx * sl2;
+    // (a row whose keys of the panel all have the logit -inf: exponentials of -inf, not of -inf + inf)
+    const float neg_m2 = (mx == -CUDART_INF_F) ? 0.f : -mx * sl2;
     float l = 0.f;
     if constexpr (C % 2 == 0) {
         // Two columns per instruction: scale-and-shift and the chunk sums run on packed pairs

@@ -52,3 +52,25 @@ def _check(ck, Hq, Hkv, d, L, w, c, hidden):
 @pytest.mark.parametrize("c", [1, 7])
 def test_single_keys_without_attention_at_token_level(ck, Hq, Hkv, d, w, c):
     _check(ck, Hq, Hkv, d, 1500, w, c, [3, 77, 300, 301, 640, 1499 - w])
+
+
+# runs that cover whole panels (60 or 64 keys of a row): a CTA's first panel, panels between others, everything up to the window
+@pytest.mark.parametrize("Hq,Hkv,d,L,w", [(32, 8, 128, 1500, 32), (64, 8, 64, 9000, 32), (4, 4, 64, 700, 8), (32, 32, 64, 4 * 128 * 17 + 1, 8)])
+@pytest.mark.parametrize("c", [1, 5, 7, 8, 10, 16, 20, 32])
+def test_runs_of_keys_without_attention(ck, Hq, Hkv, d, L, w, c):
+    _check(ck, Hq, Hkv, d, L, w, c, [*range(200, 520), *range(L - w - 150, L - w)])
+
+
+@pytest.mark.parametrize("c", [5, 8, 10, 16, 20, 32])
+@pytest.mark.parametrize("Hq", [8, 64])
+def test_model_call_with_runs_of_keys_without_attention(ck, Hq, c):
+    Hkv, d, L, w = 8, 64, 6000, 32
+    hidden = [*range(200, 520), *range(L - w - 150, L - w)]
+    xs = [_inputs(Hq, Hkv, d, L, w, hidden, seed=c + i) for i in range(3)]
+    budget = w + c * ((L - w) // (4 * c))
+    outs = ck.compress_model([tuple(map(to_dev, x)) for x in xs], Hq, w, c, budget, 1)
+    assert ck.device_status() == 0
+    for (q, K, V), (oK, oV, idx) in zip(xs, outs):
+        s = ora.chunk_scores(ora.token_scores(q, K, Hq, Hkv, w), c)
+        assert_selection_matches(idx.cpu().numpy(), s, L, w, c, budget)
+        assert_gather_exact(bits_of(oK), bits_of(oV), idx.cpu().numpy(), K, V)
