@@ -123,9 +123,11 @@ CHUNKKV_API int chunkkv_score(const void* q_obs, const void* K, int L, int Hq, i
  * exits).
  *
  * Same arguments, layouts and result as chunkkv_score without the token-score output:
- * out_chunk_scores [Hkv, C] f32. Shapes whose chunkkv_workspace_bytes(L, Hq, Hkv, d, w, c)
- * exceeds 8 MiB are rejected with CHUNKKV_ETOOLARGE, shapes outside the library's limits with
- * CHUNKKV_EINVAL_SHAPE, and nothing is launched.
+ * out_chunk_scores [Hkv, C] f32 (it always runs the kernels that keep their partial sums in scratch,
+ * so the last bits may differ from chunkkv_score's). Shapes for which those kernels need more than
+ * 8 MiB of scratch are rejected with CHUNKKV_ETOOLARGE, shapes outside the library's limits with
+ * CHUNKKV_EINVAL_SHAPE, and nothing is launched. Every shape whose chunkkv_workspace_bytes(...) is
+ * at most 8 MiB fits; one above it may fit, where that size is the layer kernel's.
  *
  * The first call on each device looks up the device address of the array (with that device
  * current). The CUDA runtime loads device code lazily, so that first call is also the moment the

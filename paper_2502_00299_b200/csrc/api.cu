@@ -322,6 +322,16 @@ size_t scratch_floats_for(const DeviceCtx& ctx, int L, int R, int Hkv, int d, in
     return n;
 }
 
+// Bytes of scratch of the calls that score with the kernels of score.cu: the chunk scores of the KV heads, those of the
+// scoring heads, and the kernels' own scratch.
+size_t score_path_bytes(const DeviceCtx& ctx, int L, int Hq, int Hkv, int d, int w, int c) {
+    const ScoreShape sh = score_shape(Hq, Hkv, w);
+    const int C = (L - w + c - 1) / c;
+    const size_t floats = scratch_floats_for(ctx, L, sh.Rs, sh.Hs, d, c) + round64(static_cast<size_t>(Hkv) * C) +
+                          round64(static_cast<size_t>(sh.Hs) * C);
+    return kHeaderBytes + floats * sizeof(float);
+}
+
 }  // namespace
 
 namespace chunkkv {
@@ -335,6 +345,13 @@ int check_heads(int L, int Hq, int Hkv, int d, int w) {
     if (Hkv > 65535) return CHUNKKV_EINVAL_SHAPE;
     if (static_cast<long long>(Hkv) * L >= (1LL << 23)) return CHUNKKV_EINVAL_SHAPE;   // 32-bit row arithmetic in the kernels
     return CHUNKKV_OK;
+}
+
+// Bytes of scratch (header included) that score_with_scratch needs for a shape within the limits; 0 without a device.
+size_t score_with_scratch_bytes(int L, int Hq, int Hkv, int d, int w, int c) {
+    std::lock_guard<std::mutex> lk(g_mu);
+    DeviceCtx* ctx;
+    return get_ctx(&ctx) == CHUNKKV_OK ? score_path_bytes(*ctx, L, Hq, Hkv, d, w, c) : 0;
 }
 
 // Scoring into caller-supplied scratch (256-byte header + payload). Used by the fixed-scratch
@@ -422,17 +439,14 @@ size_t chunkkv_workspace_bytes(int L, int Hq, int Hkv, int d, int w, int c) {
     std::lock_guard<std::mutex> lk(g_mu);
     DeviceCtx* ctx;
     if (get_ctx(&ctx) != CHUNKKV_OK) return 0;
-    const ScoreShape sh = score_shape(Hq, Hkv, w);
     const int C = (L - w + c - 1) / c;
-    // chunk scores of the KV heads, those of the scoring heads, and the scoring kernels' scratch
-    size_t floats = scratch_floats_for(*ctx, L, sh.Rs, sh.Hs, d, c) + round64(static_cast<size_t>(Hkv) * C) +
-                    round64(static_cast<size_t>(sh.Hs) * C);
+    size_t bytes = score_path_bytes(*ctx, L, Hq, Hkv, d, w, c);
     ResidentPlan rplan;
     if (C > 0 && make_resident_plan(L, w * (Hq / Hkv), Hkv, d, c, C, 0, ctx->num_sms, smem_budget(*ctx), &rplan)) {
-        const size_t rf = resident_scratch_floats(rplan, Hkv, C);
-        floats = rf > floats ? rf : floats;
+        const size_t rb = kHeaderBytes + resident_scratch_floats(rplan, Hkv, C) * sizeof(float);
+        bytes = rb > bytes ? rb : bytes;
     }
-    return kHeaderBytes + floats * sizeof(float);
+    return bytes;
 }
 
 int chunkkv_set_workspace(void* dev_ptr, size_t bytes) {

@@ -226,6 +226,7 @@ cudaError_t launch_gather_shared_sms(const void* K, const void* V, const int32_t
 // Scoring (score + finalisation kernels) into caller-supplied scratch: a 256-byte header whose
 // first word is the device status word, then the payload. Returns a CHUNKKV_* status;
 // CHUNKKV_ETOOLARGE if scratch_bytes is too small. Allocates nothing.
+size_t score_with_scratch_bytes(int L, int Hq, int Hkv, int d, int w, int c);
 int score_with_scratch(const void* q_obs, const void* K, int L, int Hq, int Hkv, int d, int w, int c,
                        float* out_scores, void* scratch, size_t scratch_bytes, cudaStream_t stream);
 

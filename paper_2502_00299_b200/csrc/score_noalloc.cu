@@ -59,8 +59,8 @@ extern "C" int chunkkv_score_noalloc(const void* q_obs, const void* K, int L, in
     if (((reinterpret_cast<uintptr_t>(q_obs) | reinterpret_cast<uintptr_t>(K) |
           reinterpret_cast<uintptr_t>(out_chunk_scores)) & 15u) != 0)
         return CHUNKKV_EINVAL_ALIGN;
-    // The documented limit is phrased in terms of the public size query, so callers can test it.
-    const size_t need = chunkkv_workspace_bytes(L, Hq, Hkv, d, w, c);
+    // what the kernels launched here need, not what chunkkv_workspace_bytes reserves for the layer kernel as well
+    const size_t need = chunkkv::score_with_scratch_bytes(L, Hq, Hkv, d, w, c);
     if (need == 0) return CHUNKKV_EINVAL_SHAPE;
     if (need > kScratchBytes) return CHUNKKV_ETOOLARGE;
     void* scratch = nullptr;

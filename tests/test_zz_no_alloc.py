@@ -81,3 +81,19 @@ def test_noalloc_refuses_what_does_not_fit_before_launching():
     # a shape outside the library's limits (Hkv * L >= 2^23 keys) is a shape error here as everywhere
     assert ck.lib.chunkkv_score_noalloc(q.data_ptr(), K.data_ptr(), 1 << 20, 8, 8, 128, 1, 64, out.data_ptr(), None) == -2
     assert ck.lib.chunkkv_score_noalloc_status(None) == 0
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,L,w,c", [(8, 8, 128, 131072, 8, 10), (32, 32, 64, 16000, 8, 10), (4, 4, 64, 131072, 2, 5)])
+def test_noalloc_takes_long_contexts_with_few_rows(Hq, Hkv, d, L, w, c):
+    # their partial sums are a few MB in the kernels of this entry point, whatever the layer kernel's scratch is
+    ck = _lib()
+    g = torch.Generator(device="cuda").manual_seed(L + c)
+    q = torch.randn(Hq, w, d, device="cuda", generator=g).to(torch.bfloat16)
+    K = torch.randn(Hkv, L, d, device="cuda", dtype=torch.bfloat16, generator=g)
+    ref, _ = ck.score(q, K, w, c)
+    out = Guarded((Hkv, ck.num_chunks(L, w, c)), torch.float32)
+    st = _noalloc(ck, q, K, Hq, w, c, out.t)
+    assert st == 0, ck.strerror(st)
+    assert ck.lib.chunkkv_score_noalloc_status(torch.cuda.current_stream().cuda_stream or None) == 0
+    out.check("out_chunk_scores")
+    assert_scores_close(out.t.cpu().numpy(), ref.cpu().numpy().astype(np.float64), w * Hq // Hkv, L, "noalloc vs chunkkv_score")
