@@ -200,7 +200,6 @@ int try_resident(DeviceCtx& ctx, char* base, size_t bytes, const ResidentCall& r
     io.out_scores = rc.out_scores;
     io.scratch = reinterpret_cast<float*>(base + kHeaderBytes);
     io.counters = reinterpret_cast<unsigned*>(base + kResidentCountersOffset);
-    io.status = reinterpret_cast<int*>(base);
     io.cooperative = rc.cooperative;
     io.k_row_elems = rc.kt; io.k_head_elems = rc.kh; io.v_row_elems = rc.vt; io.v_head_elems = rc.vh;
     io.block_table = rc.block_table; io.page_size = rc.page_size; io.num_pages = rc.num_pages;

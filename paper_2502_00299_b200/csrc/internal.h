@@ -104,8 +104,7 @@ struct ResidentIO {
     int32_t* out_idx;     // NULL: chunk scores only (out_scores)
     float* out_scores = nullptr;   // [Hkv, C]; NULL: in scratch
     float* scratch;       // resident_scratch_floats() floats
-    unsigned* counters;   // header + kResidentCountersOffset
-    int* status;
+    unsigned* counters;   // header + kResidentCountersOffset (the status word is the header's first)
     bool cooperative;     // cooperative launch (lanes: several launches share the GPU) instead of a programmatic dependent one
     // elements between consecutive rows of a head and between heads of K and of V; 0 = packed [Hkv, L, d]
     long long k_row_elems = 0, k_head_elems = 0, v_row_elems = 0, v_head_elems = 0;

@@ -91,11 +91,16 @@ struct ResArgs {
     float* scores;                     // [Hkv, score_row]
     int score_row;                     // C, or C rounded up to a multiple of 4 in scratch (16-byte aligned rows)
     float* spill;                      // [grid, n_off, (chunk slots per panel + 1) * 128]: chunk sums, panel maximum
-    unsigned* cnt_a;                   // [Hkv] hand-over 2, zero between launches
-    unsigned* cnt_b;                   // [Hkv] hand-over 4
-    unsigned* exits;                   // CTAs that left; the last one clears the counters
-    int* status;
+    unsigned* counters;                // header + kResidentCountersOffset, zero between launches
+
+    __device__ unsigned* exits() const { return counters; }              // CTAs that left; the last one clears the counters
+    __device__ unsigned* cnt_a(int h) const { return counters + 16 + h; }                          // hand-over 2 of a KV head
+    __device__ unsigned* cnt_b(int h) const { return counters + 16 + kResidentMaxHeads + h; }      // hand-over 4
+    __device__ int* status() const { return reinterpret_cast<int*>(counters) - kResidentCountersOffset / sizeof(int); }
 };
+// The launch costs the host more with more parameter bytes than this: 488 -> 504 bytes took 0.45 us of a serving layer's 30.3
+// (a launch between other kernels' launches; hence the addresses above that follow from one pointer).
+static_assert(2 * sizeof(CUtensorMap) + sizeof(ResArgs) <= 488, "kernel parameters");
 
 // One thread publishes this CTA's arrival on `counter` and waits until `target` CTAs have arrived.
 // Block-wide: every thread calls it; returns false if the wait was abandoned.
@@ -342,7 +347,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             dst[i] = M;
             dst[128 + i] = Ls;
         }
-        ok = head_handover(a.cnt_a + hkv, static_cast<unsigned>(a.cph), ctl);
+        ok = head_handover(a.cnt_a(hkv), static_cast<unsigned>(a.cph), ctl);
     }
 
     // ---- 3. row statistics of the head, then this CTA's chunk scores
@@ -466,7 +471,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             }
     }
     // ---- 4. wait for the KV head's other CTAs, 5. select, 6. gather
-    if (ok && a.out_idx != nullptr) ok = head_handover(a.cnt_b + hkv, static_cast<unsigned>(a.cph), ctl);
+    if (ok && a.out_idx != nullptr) ok = head_handover(a.cnt_b(hkv), static_cast<unsigned>(a.cph), ctl);
     if (ok && a.out_idx != nullptr) {
         SelectSmem& ss = *reinterpret_cast<SelectSmem*>(ring);
         constexpr size_t kSelBytes = (sizeof(SelectSmem) + 127) & ~size_t(127);
@@ -521,13 +526,13 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         tmem_dealloc(tmem_base, 512);
     }
     if (threadIdx.x == 0) {
-        if (!ok) atomicExch(a.status, 1);
+        if (!ok) atomicExch(a.status(), 1);
         // The last CTA to leave clears the hand-over counters for the next launch. (After an
         // abandoned wait the counters are left as they are; chunkkv_device_status clears them.)
-        const unsigned old = atomicAdd(a.exits, 1u);
+        const unsigned old = atomicAdd(a.exits(), 1u);
         if (old + 1u == gridDim.x) {
-            for (int h = 0; h < a.Hkv; ++h) { a.cnt_a[h] = 0u; a.cnt_b[h] = 0u; }
-            *a.exits = 0u;
+            for (int h = 0; h < a.Hkv; ++h) { *a.cnt_a(h) = 0u; *a.cnt_b(h) = 0u; }
+            *a.exits() = 0u;
             __threadfence();
         }
     }
@@ -617,10 +622,7 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     a.scores = io.out_scores ? io.out_scores : scores;
     a.score_row = io.out_scores ? io.C : (io.C + 3) & ~3;
     a.spill = scores + ((static_cast<size_t>(io.Hkv) * ((io.C + 3) & ~3) + 63) & ~static_cast<size_t>(63));
-    a.exits = io.counters;
-    a.cnt_a = io.counters + 16;
-    a.cnt_b = io.counters + 16 + kResidentMaxHeads;
-    a.status = io.status;
+    a.counters = io.counters;
     const bool big = plan.n_mt == 2 || plan.n_off > 0;
     const void* kern = nullptr;
     int v = 0;
