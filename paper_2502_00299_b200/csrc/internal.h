@@ -88,6 +88,7 @@ struct ResidentPlan {
     int t_max;        // most tiles any CTA takes
     int spp;          // chunk slots per panel (half a tile)
     int n_on, n_off;  // panels of a CTA whose partial sums stay on chip; the others go to scratch
+    int spill_rows;   // rows of a panel's record in scratch
     int n_stages;
     int smem_bytes;
     int off_ring, ring_bytes, off_pmax, off_misc;
@@ -133,6 +134,7 @@ struct ModelPlan {
     int c_static, n_mt, grid, cph, tile, n_tiles, t_max, spp, n_stages, smem_bytes;
     bool big;                    // two query tiles or a ring of partial sums that continues in scratch
     int ring_on, ring;           // panels of the ring on chip, in all
+    int spill_rows;              // rows of a panel's record in scratch (whole warps)
     int ahead, stride;           // big: when a group contracts the layer before (own panels)
     int copy_slots;
     int n_score, n_sel;          // scoring CTAs, selector CTAs (grid = n_score + n_sel)

@@ -78,6 +78,7 @@ struct ResArgs {
     int C, k, n_max, Hkv;
     int off_ring, ring_bytes, off_pmax, off_misc;   // dynamic shared memory layout (bytes from the aligned base)
     int n_on, n_off;                   // panels of a CTA kept on chip; room for panels in scratch
+    int spill_rows;                    // rows of a panel's record in scratch
     const uint4* K;
     const uint4* V;
     long long k_row, k_head, v_row, v_head;   // 16-byte vectors between rows of a head / between heads
@@ -90,7 +91,7 @@ struct ResArgs {
     float* cta_stat;                   // [grid, n_mt, {max, sum}, 128]
     float* scores;                     // [Hkv, score_row]
     int score_row;                     // C, or C rounded up to a multiple of 4 in scratch (16-byte aligned rows)
-    float* spill;                      // [grid, n_off, (chunk slots per panel + 1) * 128]: chunk sums, panel maximum
+    float* spill;                      // [grid, n_off, (chunk slots per panel + 1) * spill_rows]: chunk sums, panel maximum
     unsigned* counters;                // header + kResidentCountersOffset, zero between launches
 
     __device__ unsigned* exits() const { return counters; }              // CTAs that left; the last one clears the counters
@@ -309,7 +310,11 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 #pragma unroll
                 for (int q = 0; q < SPP; ++q) rec_[q] = pr[q];
                 rec_[SPP] = m2;
-                spill_store<SPP + 1>(a.spill + (static_cast<size_t>(blockIdx.x) * a.n_off + (pl - a.n_on)) * ((SPP + 1) * 128), row, rec_, keep);
+                const size_t at = static_cast<size_t>(blockIdx.x) * a.n_off + (pl - a.n_on);
+                if (a.spill_rows == 128)
+                    spill_store<SPP + 1, 128>(a.spill + at * ((SPP + 1) * 128), 128, row, rec_, keep);
+                else if (active)
+                    spill_store<SPP + 1, 0>(a.spill + at * ((SPP + 1) * a.spill_rows), a.spill_rows, row, rec_, keep);
             }
             // fold into the running record: l is relative to m2, run_l to run_m
             const float nm = fmaxf(run_m, m2);
@@ -411,6 +416,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             const int row = quarter * 32 + lane, mt = two ? grp >> 1 : 0;
             const bool active = mt * 128 + row < a.R;
             const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+            const int srow = active ? row : 0;           // (rows that do not exist have no record)
             const float mi = gm[mt * 128 + row], li = ginv[mt * 128 + row];
             const uint64_t drop = l2_policy_evict_first();   // the sums in scratch are dead once read
             constexpr int PPB = 32 / SPP;                // panels per block of up to 32 values
@@ -434,7 +440,11 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                             pm[u] = pmax[pl * 128 + row];
                         } else {
                             float rec_[SPP + 1];
-                            spill_load<SPP + 1>(a.spill + (static_cast<size_t>(blockIdx.x) * a.n_off + (pl - a.n_on)) * ((SPP + 1) * 128), row, rec_, drop);
+                            const size_t at = static_cast<size_t>(blockIdx.x) * a.n_off + (pl - a.n_on);
+                            if (a.spill_rows == 128)
+                                spill_load<SPP + 1, 128>(a.spill + at * ((SPP + 1) * 128), 128, row, rec_, drop);
+                            else
+                                spill_load<SPP + 1, 0>(a.spill + at * ((SPP + 1) * a.spill_rows), a.spill_rows, srow, rec_, drop);
                             pm[u] = rec_[SPP];
 #pragma unroll
                             for (int q = 0; q < SPP; ++q) v[u * SPP + q] = rec_[q];
@@ -548,7 +558,7 @@ const void* kernel_of(bool big) {
 
 size_t resident_scratch_floats(const ResidentPlan& plan, int Hkv, int C) {
     return static_cast<size_t>(plan.grid) * plan.n_mt * 256 + ((static_cast<size_t>(Hkv) * ((C + 3) & ~3) + 63) & ~static_cast<size_t>(63)) +
-           static_cast<size_t>(plan.grid) * plan.n_off * (plan.spp + 1) * 128;
+           static_cast<size_t>(plan.grid) * plan.n_off * (plan.spp + 1) * plan.spill_rows;
 }
 
 bool make_resident_plan(int L, int R, int Hkv, int d, int c, int C, int n_max, int max_ctas, int smem_limit,
@@ -573,6 +583,7 @@ bool make_resident_plan(int L, int R, int Hkv, int d, int c, int C, int n_max, i
     p.n_on = kRPartCols / p.spp;
     if (p.n_on > n_pl) p.n_on = n_pl;
     p.n_off = n_pl - p.n_on;
+    p.spill_rows = R < 128 ? (R + 3) & ~3 : 128;                    // 16-byte aligned records of the rows that exist
     const int KB = d / 64, stage = tile * 128;
     const int q_bytes = p.n_mt * KB * kRQTileBytes;
     const int pmax_bytes = p.n_on * 128 * 4;
@@ -604,7 +615,7 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     a.q_box_rows = io.R < 128 ? io.R : 128;
     a.k_box_rows = io.L < plan.tile ? io.L : plan.tile;
     a.C = io.C; a.k = io.k; a.n_max = io.n_max; a.Hkv = io.Hkv;
-    a.n_on = plan.n_on; a.n_off = plan.n_off;
+    a.n_on = plan.n_on; a.n_off = plan.n_off; a.spill_rows = plan.spill_rows;
     a.off_ring = plan.off_ring; a.ring_bytes = plan.ring_bytes; a.off_pmax = plan.off_pmax; a.off_misc = plan.off_misc;
     a.K = static_cast<const uint4*>(io.K); a.V = static_cast<const uint4*>(io.V);
     a.block_table = io.block_table; a.page_size = io.page_size; a.num_pages = io.num_pages;

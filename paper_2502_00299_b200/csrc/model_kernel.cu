@@ -121,6 +121,7 @@ struct ModelParams {
     int strided;           // rows of a head are not adjacent in memory: kept rows are fetched through tm_rk / tm_rv
     int copy_box_bytes;    // bytes of such a box
     int ring_on, ring;     // big variant: panels of the ring in tensor memory, panels of the ring in all
+    int spill_rows;        // rows of a panel's record in scratch (whole warps)
     int ahead, stride;     // big variant: own panels of a layer that a group scores before the contraction of the layer before,
                            // and between two blocks of it
     int copy_slots;
@@ -129,7 +130,7 @@ struct ModelParams {
     int off_ring, off_pmax, off_misc, off_tail, stage_slot_bytes;
     float* cta_stat;       // [2 (slot parity)][grid][n_mt][{max, sum}][128]
     float* scores;         // [n_compute][Hkv][n_mt][Cpad]
-    float* spill;          // [scoring CTA][ring - ring_on][(chunk slots per panel + 1) * 128]: chunk sums, panel maximum
+    float* spill;          // per scoring CTA: [ring - ring_on][rows / 32][chunk sums, panel maximum][32 rows], and the blocks of warps without rows
     unsigned* cnt_a;       // [Hkv]
     unsigned* cnt_b;       // [Hkv]  chunk scores of a slot announced by the scoring CTAs
     unsigned* cnt_c;       // [Hkv]  kept-chunk lists announced by the selector CTAs
@@ -511,7 +512,17 @@ model_kernel(const __grid_constant__ ModelParams p) {
         constexpr int PCOLS = BIG ? SPP + 1 : SPP;                                  // tensor-memory columns of a panel
         const int ch0 = t_begin * (TILE / C_STATIC);
         const uint64_t keep = l2_policy_evict_last(), drop = l2_policy_evict_first();
-        float* spill = BIG ? p.spill + static_cast<size_t>(blockIdx.x) * (p.ring - p.ring_on) * ((SPP + 1) * 128) : nullptr;
+        // A panel's record in scratch: a block of 32 rows for every warp that has rows, with constant offsets inside it. A warp
+        // that has none does the same with one block of its own behind the records (it would cost the others more to branch).
+        float* spill = nullptr;
+        size_t spill_step = 0;                           // between the records of two ring slots
+        if constexpr (BIG) {
+            const int off = p.ring - p.ring_on, n_w = p.spill_rows / 32;
+            const size_t cta = static_cast<size_t>(blockIdx.x) * (static_cast<size_t>(off) * n_w + 4 * (4 - n_w)) * (PCOLS * 32);
+            const bool have_rows = quarter < n_w;
+            spill = p.spill + cta + (have_rows ? quarter : off * n_w + grp * (4 - n_w) + quarter - n_w) * (PCOLS * 32);
+            spill_step = have_rows ? PCOLS * p.spill_rows : 0;
+        }
         bool ok = true;
         float run_m = -CUDART_INF_F, run_l = 0.f;
         // Contraction of a layer's partial sums into chunk scores, one block of panels at a time, between the panels of the next
@@ -588,7 +599,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                         if (slot_of[u] < p.ring_on) {
                             part_load<PCOLS>(lane_addr + static_cast<uint32_t>(PART0 + slot_of[u] * PCOLS), &vp[u * PCOLS]);
                         } else {
-                            spill_load<PCOLS>(spill + static_cast<size_t>(slot_of[u] - p.ring_on) * (PCOLS * 128), row, &vp[u * PCOLS], drop);
+                            spill_load<PCOLS, 32>(spill + (slot_of[u] - p.ring_on) * spill_step, 32, lane, &vp[u * PCOLS], drop);
                         }
                     }
                     tmem_ld_wait();
@@ -677,7 +688,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                     if (slot < p.ring_on) {
                         part_store<PCOLS>(lane_addr + static_cast<uint32_t>(PART0 + slot * PCOLS), pr);
                     } else {
-                        spill_store<PCOLS>(spill + static_cast<size_t>(slot - p.ring_on) * (PCOLS * 128), row, pr, keep);
+                        spill_store<PCOLS, 32>(spill + (slot - p.ring_on) * spill_step, 32, lane, pr, keep);
                     }
                 } else {
                     part_store<SPP>(lane_addr + static_cast<uint32_t>(PART0 + slot * SPP), pr);
@@ -953,6 +964,7 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_
     } else {
         p.ring_on = p.ring = model_ring_panels(c, false);
     }
+    p.spill_rows = R < 128 ? (R + 31) & ~31 : 128;
     const int KB = d / 64, stage = p.tile * 128;
     const int q_bytes = p.n_mt * KB * kRQTileBytes;
     const int pmax_bytes = p.big ? 0 : p.ring * 128 * 4;     // the panel-maxima ring: one row set per ring panel
@@ -978,10 +990,18 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_
     return true;
 }
 
+// Scratch of a scoring CTA for the part of the ring that is not on chip: the records, and four groups' blocks for the warps
+// without rows.
+static size_t model_spill_floats(const ModelPlan& plan) {
+    if (plan.ring == plan.ring_on) return 0;
+    const size_t n_w = plan.spill_rows / 32;
+    return ((plan.ring - plan.ring_on) * n_w + 4 * (4 - n_w)) * (plan.spp + 1) * 32;
+}
+
 size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute) {
     return static_cast<size_t>(2) * plan.grid * plan.n_mt * 256 + static_cast<size_t>(n_compute) * Hkv * plan.n_mt * ((C + 3) & ~3) +
            static_cast<size_t>(n_compute) * Hkv * (plan.sel_row_bytes / 4) + 64 +
-           static_cast<size_t>(plan.n_score) * (plan.ring - plan.ring_on) * (plan.spp + 1) * 128;
+           static_cast<size_t>(plan.n_score) * model_spill_floats(plan);
 }
 
 template <int C_STATIC>
@@ -1022,7 +1042,7 @@ cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtenso
     p.q_box_rows = io.R < 128 ? io.R : 128;
     p.k_box_rows = io.L < plan.tile ? io.L : plan.tile;
     p.C = io.C; p.k = io.k; p.n_max = io.n_max; p.Hkv = io.Hkv;
-    p.ring_on = plan.ring_on; p.ring = plan.ring; p.ahead = plan.ahead; p.stride = plan.stride; p.copy_slots = plan.copy_slots;
+    p.ring_on = plan.ring_on; p.ring = plan.ring; p.spill_rows = plan.spill_rows; p.ahead = plan.ahead; p.stride = plan.stride; p.copy_slots = plan.copy_slots;
     p.Cpad = (io.C + 3) & ~3;
     p.n_score = plan.n_score; p.n_sel = plan.n_sel;
     p.sel_row_bytes = plan.sel_row_bytes; p.sel_keys_fit = plan.sel_keys_fit;

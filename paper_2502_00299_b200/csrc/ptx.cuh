@@ -108,28 +108,31 @@ __device__ __forceinline__ float4 ld_last_use(const float4* p, uint64_t policy) 
     return v;
 }
 
-// N floats of each of 128 threads (rows) in scratch: whole groups of four as 16-byte vectors, the rest one by one, each
-// adjacent for adjacent rows, so that a warp's accesses are whole lines and nothing is padded.
-template <int N>
-__device__ __forceinline__ void spill_store(float* p, int row, const float (&v)[N], uint64_t policy) {
+// N floats of each of `rows` threads (a multiple of 4) in scratch: whole groups of four as 16-byte vectors, the rest one by
+// one, each adjacent for adjacent rows, so that a warp's accesses are whole lines and nothing is padded.
+// ROWS > 0: that many rows, so that the offsets are constants.
+template <int N, int ROWS>
+__device__ __forceinline__ void spill_store(float* p, int rows, int row, const float (&v)[N], uint64_t policy) {
+    const int n = ROWS > 0 ? ROWS : rows;
 #pragma unroll
     for (int o = 0; o + 4 <= N; o += 4)
-        asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p + o * 128 + row * 4), "f"(v[o]),
+        asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p + o * n + row * 4), "f"(v[o]),
                      "f"(v[o + 1]), "f"(v[o + 2]), "f"(v[o + 3]), "l"(policy)
                      : "memory");
 #pragma unroll
-    for (int o = N / 4 * 4; o < N; ++o) st_keep(p + o * 128 + row, v[o], policy);
+    for (int o = N / 4 * 4; o < N; ++o) st_keep(p + o * n + row, v[o], policy);
 }
-template <int N>
-__device__ __forceinline__ void spill_load(const float* p, int row, float* v, uint64_t policy) {
+template <int N, int ROWS>
+__device__ __forceinline__ void spill_load(const float* p, int rows, int row, float* v, uint64_t policy) {
+    const int n = ROWS > 0 ? ROWS : rows;
 #pragma unroll
     for (int o = 0; o + 4 <= N; o += 4) {
-        const float4 f = ld_last_use(reinterpret_cast<const float4*>(p + o * 128 + row * 4), policy);
+        const float4 f = ld_last_use(reinterpret_cast<const float4*>(p + o * n + row * 4), policy);
         v[o] = f.x; v[o + 1] = f.y; v[o + 2] = f.z; v[o + 3] = f.w;
     }
 #pragma unroll
     for (int o = N / 4 * 4; o < N; ++o)
-        asm volatile("ld.global.cg.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v[o]) : "l"(p + o * 128 + row), "l"(policy));
+        asm volatile("ld.global.cg.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v[o]) : "l"(p + o * n + row), "l"(policy));
 }
 
 // ----------------------------------------------------------------------------- tcgen05

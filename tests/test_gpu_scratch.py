@@ -1,0 +1,60 @@
+"""Scratch of the one-launch layer kernel and of the persistent model kernel where their partial sums do not all stay on chip:
+how much a shape asks for, and that a call writes nothing outside it."""
+import numpy as np
+import pytest
+import torch
+
+from tests.helpers import Guarded
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ck():
+    import paper_2502_00299_b200 as ck
+    assert torch.cuda.is_available()
+    yield ck
+    ck.set_workspace(None)
+
+
+def _layer(Hq, Hkv, d, L, w, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    q = torch.randn(Hq, w, d, device="cuda", generator=g).to(torch.bfloat16)
+    K, V = (torch.randn(Hkv, L, d, device="cuda", dtype=torch.bfloat16, generator=g) for _ in range(2))
+    return q, K, V
+
+
+def test_scratch_grows_with_the_rows_that_exist(ck):
+    # off-chip records are as wide as the rows: a few rows ask for a few MB, whatever 128 rows ask for
+    for Hq, Hkv, d, L, w, c, limit in ((8, 8, 128, 131072, 8, 10, 7.0), (8, 8, 128, 131072, 8, 5, 14.0), (8, 8, 128, 131072, 16, 5, 22.0),
+                                       (32, 32, 64, 16000, 8, 10, 4.2), (32, 32, 64, 65536, 8, 10, 12.0), (8, 8, 128, 131072, 1, 5, 6.5)):
+        assert ck.workspace_bytes(L, Hq, Hkv, d, w, c) <= limit * 2 ** 20, (Hq, Hkv, L, w, c)
+
+
+# shapes with off-chip records: one and two query tiles, rows no multiple of 4 or 32, few rows
+SPILL = [(64, 16, 64, 9 * 120 * 22, 16, 10), (64, 32, 64, 4 * 120 * 30 + 7, 5, 5), (32, 32, 64, 4 * 128 * 33 - 3, 8, 8), (32, 32, 64, 4 * 120 * 23 + 1, 1, 5),
+         (128, 32, 64, 4 * 120 * 23 + 61, 64, 20), (96, 32, 64, 4 * 128 * 40, 64, 16), (28 * 8, 32, 64, 4 * 120 * 20, 32, 10)]
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,L,w,c", SPILL)
+def test_layer_and_model_calls_stay_inside_their_scratch(ck, Hq, Hkv, d, L, w, c):
+    budget = w + c * ((L - w) // (5 * c))
+    xs = [_layer(Hq, Hkv, d, L, w, seed=L + i) for i in range(3)]
+    ck.set_workspace(None)
+    free = [ck.compress_layer(*x, Hq, w, c, budget) for x in xs]           # (scratch with room to spare)
+    scores = [ck.score(x[0], x[1], w, c)[0] for x in xs]
+    ws = Guarded((ck.workspace_bytes(L, Hq, Hkv, d, w, c),), torch.uint8)
+    ck.set_workspace(ws.t)
+    for x, want, s in zip(xs, free, scores):
+        got = ck.compress_layer(*x, Hq, w, c, budget)
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+        assert torch.equal(ck.score(x[0], x[1], w, c)[0], s)
+    assert ck.device_status() == 0
+    ws.check("layer scratch")
+    ws = Guarded((int(ck.lib.chunkkv_model_workspace_bytes(len(xs), L, Hq, Hkv, d, w, c, budget, 1)),), torch.uint8)
+    ck.set_workspace(ws.t)
+    for _ in range(2):
+        for got, want in zip(ck.compress_model(xs, Hq, w, c, budget, 1), free):
+            assert all(torch.equal(a, b) for a, b in zip(got, want))
+    assert ck.device_status() == 0
+    ws.check("model scratch")
