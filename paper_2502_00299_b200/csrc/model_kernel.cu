@@ -549,6 +549,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                 bool ready = true;
                 if (lane == 0) ready = mbar_wait(smem_u32(&ctl.stat_full[c_s & 1]), (c_s >> 1) & 1, abort_flag);
                 if (!__shfl_sync(0xffffffffu, ready, 0)) ok = false;   // (the failed wait has raised the abort flag)
+                __syncwarp();          // orders the other lanes' reads below behind the wait; a shuffle alone does not
                 tmem_st_wait();
                 if constexpr (BIG) {
                     // every record of the head is there (the statistics warp has seen the count): each thread merges those of
@@ -737,6 +738,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
             if (lane == 0)
                 w_ok = mbar_wait(smem_u32(&ctl.pub_done[s & 1]), static_cast<uint32_t>(s >> 1) & 1u, abort_flag);
             if (!__shfl_sync(0xffffffffu, w_ok, 0)) break;
+            __syncwarp();              // (as above: the other lanes read what the epilogue warps left in shared memory)
             {
                 // every epilogue warp has left its group's (max, sum) per row in shared memory: merge the
                 // four groups (this lane: rows 4 lane .. 4 lane + 3), store the CTA's record and announce it.
