@@ -883,7 +883,7 @@ size_t chunkkv_model_workspace_bytes(int n_layers, int L, int Hq, int Hkv, int d
     ModelPlan mp;
     size_t need = per_layer;
     if (C > 0 && k > 0 && make_model_plan(L, w * (Hq / Hkv), Hkv, d, c, C, k, ctx->num_sms, smem_budget(*ctx), &mp)) {
-        const size_t m = kHeaderBytes + model_scratch_floats(mp, Hkv, C, model_launch_computes(n_layers, reuse_depth)) * sizeof(float);
+        const size_t m = kHeaderBytes + model_scratch_floats(mp, Hkv, C, model_launch_computes(n_layers, reuse_depth), true) * sizeof(float);
         need = m > need ? m : need;
     }
     return need;

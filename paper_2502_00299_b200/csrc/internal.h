@@ -134,6 +134,7 @@ struct ModelPlan {
     int c_static, n_mt, grid, cph, tile, n_tiles, t_max, spp, n_stages, smem_bytes;
     bool big;                    // two query tiles or a ring of partial sums that continues in scratch
     int ring_on, ring;           // panels of the ring on chip, in all
+    int ring_reserve;            // at least `ring`, and never smaller for a longer sequence
     int spill_rows;              // rows of a panel's record in scratch (whole warps)
     int ahead, stride;           // big: when a group contracts the layer before (own panels)
     int copy_slots;
@@ -161,7 +162,8 @@ struct ModelLayerIO {
 };
 
 bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, ModelPlan* plan);
-size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute);
+// What a launch uses; with `reserve` what a caller is told to provide, which a shorter sequence never exceeds.
+size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute, bool reserve = false);
 // layers[0] must compute; tm_q / tm_k hold one tensor map per computed layer, in order; tm_rk / tm_rv one per layer (boxes
 // of one chunk's rows) where keys and values are not packed, else NULL.
 cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtensorMap* tm_q, const CUtensorMap* tm_k,

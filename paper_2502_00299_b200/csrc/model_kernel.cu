@@ -515,7 +515,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
         // A panel's record in scratch: a block of 32 rows for every warp that has rows, with constant offsets inside it. A warp
         // that has none does the same with one block of its own behind the records (it would cost the others more to branch).
         float* spill = nullptr;
-        size_t spill_step = 0;                           // between the records of two ring slots
+        int spill_step = 0;                              // between the records of two ring slots
         if constexpr (BIG) {
             const int off = p.ring - p.ring_on, n_w = p.spill_rows / 32;
             const size_t cta = static_cast<size_t>(blockIdx.x) * (static_cast<size_t>(off) * n_w + 4 * (4 - n_w)) * (PCOLS * 32);
@@ -963,8 +963,12 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_
         p.ring_on = model_ring_panels(c, true);
         p.ring = (n_pl + 4 * (p.ahead + p.stride) + 3) / 4 * 4;
         if (p.ring < p.ring_on) p.ring = p.ring_on;
+        // (`stride` falls where another block begins, and the ring with it)
+        const int widest = own - p.ahead < 1 ? 1 : (own - p.ahead > ppb ? ppb : own - p.ahead);
+        p.ring_reserve = (n_pl + 4 * (p.ahead + widest) + 3) / 4 * 4;
+        if (p.ring_reserve < p.ring_on) p.ring_reserve = p.ring_on;
     } else {
-        p.ring_on = p.ring = model_ring_panels(c, false);
+        p.ring_on = p.ring = p.ring_reserve = model_ring_panels(c, false);
     }
     p.spill_rows = R < 128 ? (R + 31) & ~31 : 128;
     const int KB = d / 64, stage = p.tile * 128;
@@ -994,16 +998,16 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_
 
 // Scratch of a scoring CTA for the part of the ring that is not on chip: the records, and four groups' blocks for the warps
 // without rows.
-static size_t model_spill_floats(const ModelPlan& plan) {
-    if (plan.ring == plan.ring_on) return 0;
+static size_t model_spill_floats(const ModelPlan& plan, int ring) {
+    if (ring <= plan.ring_on) return 0;
     const size_t n_w = plan.spill_rows / 32;
-    return ((plan.ring - plan.ring_on) * n_w + 4 * (4 - n_w)) * (plan.spp + 1) * 32;
+    return ((ring - plan.ring_on) * n_w + 4 * (4 - n_w)) * (plan.spp + 1) * 32;
 }
 
-size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute) {
+size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute, bool reserve) {
     return static_cast<size_t>(2) * plan.grid * plan.n_mt * 256 + static_cast<size_t>(n_compute) * Hkv * plan.n_mt * ((C + 3) & ~3) +
            static_cast<size_t>(n_compute) * Hkv * (plan.sel_row_bytes / 4) + 64 +
-           static_cast<size_t>(plan.n_score) * model_spill_floats(plan);
+           static_cast<size_t>(plan.n_score) * model_spill_floats(plan, reserve ? plan.ring_reserve : plan.ring);
 }
 
 template <int C_STATIC>

@@ -58,3 +58,11 @@ def test_layer_and_model_calls_stay_inside_their_scratch(ck, Hq, Hkv, d, L, w, c
             assert all(torch.equal(a, b) for a, b in zip(got, want))
     assert ck.device_status() == 0
     ws.check("model scratch")
+
+
+@pytest.mark.parametrize("Hq,Hkv,w,c", [(32, 8, 32, 20), (64, 8, 32, 10), (64, 8, 32, 5), (8, 8, 8, 5), (28, 4, 32, 16), (32, 8, 32, 32)])
+def test_model_scratch_never_shrinks_for_a_longer_sequence(ck, Hq, Hkv, w, c):
+    # so that a buffer sized for the longest prompt holds every shorter one
+    lens = [*range(129400, 129700, 4), *range(w, 140000, 97)]
+    need = [ck.lib.chunkkv_model_workspace_bytes(32, L, Hq, Hkv, 128, w, c, 4096, 1) for L in sorted(lens)]
+    assert all(a <= b for a, b in zip(need, need[1:])), [L for L, a, b in zip(sorted(lens)[1:], need, need[1:]) if a > b][:5]
