@@ -230,12 +230,17 @@ CHUNKKV_API int chunkkv_compress_layer_strided(const void* q_obs, const void* K,
  *                                        that reuse indices. The arrays are read during the call
  *                                        only. Output buffers of different layers must not overlap.
  * Same results as the corresponding sequence of chunkkv_compress_layer calls. Where the shape
- * allows (chunk size 10 or 20, at most 128 query rows per KV head or an even number of grouped query
- * heads, key range per SM within tensor memory) the layers run through one persistent kernel per
- * group of up to 32 layers in which scoring layer l + 1 overlaps selecting and gathering layer l;
- * otherwise they run layer by layer. Needs a workspace of chunkkv_model_workspace_bytes(...) bytes
- * (chunkkv_set_workspace); returns CHUNKKV_ENOWORKSPACE otherwise. Queued on `stream`; the calls of
- * one device that use the workspace must be ordered.
+ * allows (chunk size 5, 8, 10, 16, 20 or 32, at most 65535 chunks of which at most 8192 are kept, more SMs
+ * than KV heads) the layers run through one persistent kernel per group of up to 96 layers (48 with
+ * strided inputs), 32 of them computed, in which scoring layer l + 1 overlaps selecting and gathering
+ * layer l; otherwise they run layer by layer.
+ *
+ * Needs a workspace of chunkkv_model_workspace_bytes(...) bytes (chunkkv_set_workspace), which never
+ * shrinks for a longer sequence. With less, calls with chunk size 10 or 20, at most 128 query rows per
+ * KV head or an even number of grouped query heads, and at most 252 / (120 / c) tiles of 120 keys per
+ * SM return CHUNKKV_ENOWORKSPACE; the other shapes run layer by layer where chunkkv_workspace_bytes(...)
+ * are there (slower; the same results), and return CHUNKKV_ENOWORKSPACE where not. Queued on `stream`;
+ * the calls of one device that use the workspace must be ordered.
  */
 CHUNKKV_API size_t chunkkv_model_workspace_bytes(int n_layers, int L, int Hq, int Hkv, int d, int w, int c,
                                                  int budget, int reuse_depth);

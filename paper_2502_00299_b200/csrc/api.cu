@@ -870,6 +870,18 @@ static int model_launch_computes(int n_layers, int reuse_depth) {
     return n < kModelMaxCompute ? n : kModelMaxCompute;
 }
 
+// Whether a model call of this shape is refused on a scratch that does not hold the persistent kernel's: chunk sizes 10 and 20
+// with at most 128 query rows to a scoring head (a KV head, or half of an even group) and at most 252 chunk slots of
+// it to a CTA. The other shapes that the kernel takes run layer by layer on a scratch of the layer calls.
+static bool model_scratch_required(int num_sms, int L, int R, int G, int Hkv, int c) {
+    if ((c != 10 && c != 20) || (R > 128 && G % 2 != 0)) return false;
+    const int heads = R > 128 ? 2 * Hkv : Hkv;
+    if (num_sms <= heads || heads > kResidentMaxHeads) return false;
+    const int sel = Hkv < 4 ? Hkv : 4, ctas = num_sms - sel < heads ? heads : num_sms - sel, cph = ctas / heads;
+    const int tiles = (L + 119) / 120, per_cta = (tiles + cph - 1) / cph;
+    return per_cta * (120 / c) <= 252;
+}
+
 size_t chunkkv_model_workspace_bytes(int n_layers, int L, int Hq, int Hkv, int d, int w, int c, int budget,
                                      int reuse_depth) {
     if (model_args_ok(n_layers, reuse_depth) != CHUNKKV_OK || check_sizes(L, w, c, budget) != CHUNKKV_OK) return 0;
@@ -929,11 +941,11 @@ static int compress_model_impl(int n_layers, const void* const* q_obs, const voi
         if (st != CHUNKKV_OK) return st;
         // paged outputs run layer by layer: the one-launch layer kernel places rows through the block table with all
         // its threads, which measured faster (35 us per layer) than the persistent kernel's copy warp doing it (41 us)
-        // (a scratch set up for the layer calls only is used by the layer calls)
-        persistent = !paged && C > 0 && k > 0 &&
-                     make_model_plan(L, R, Hkv, d, c, C, k, ctx->num_sms, smem_budget(*ctx), &mp) &&
-                     ensure_workspace(*ctx, model_scratch_floats(mp, Hkv, C, model_launch_computes(n_layers, reuse_depth)) *
-                                                sizeof(float)) == CHUNKKV_OK;
+        if (!paged && C > 0 && k > 0 && make_model_plan(L, R, Hkv, d, c, C, k, ctx->num_sms, smem_budget(*ctx), &mp)) {
+            st = ensure_workspace(*ctx, model_scratch_floats(mp, Hkv, C, model_launch_computes(n_layers, reuse_depth)) * sizeof(float));
+            if (st != CHUNKKV_OK && model_scratch_required(ctx->num_sms, L, R, Hq / Hkv, Hkv, c)) return st;
+            persistent = st == CHUNKKV_OK;
+        }
     }
     if (!persistent) {
         // layer by layer: Algorithm 2's call sequence over chunkkv_compress_layer

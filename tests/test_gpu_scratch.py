@@ -1,6 +1,7 @@
 """Scratch of the one-launch layer kernel and of the persistent model kernel where their partial sums do not all stay on chip:
 how much a shape asks for, and that a call writes nothing outside it."""
-import numpy as np
+import ctypes
+
 import pytest
 import torch
 
@@ -66,3 +67,38 @@ def test_model_scratch_never_shrinks_for_a_longer_sequence(ck, Hq, Hkv, w, c):
     lens = [*range(129400, 129700, 4), *range(w, 140000, 97)]
     need = [ck.lib.chunkkv_model_workspace_bytes(32, L, Hq, Hkv, 128, w, c, 4096, 1) for L in sorted(lens)]
     assert all(a <= b for a, b in zip(need, need[1:])), [L for L, a, b in zip(sorted(lens)[1:], need, need[1:]) if a > b][:5]
+
+
+@pytest.mark.parametrize("Hq,c,L,refused", [(8, 10, 20000, True), (8, 20, 20000, True), (8, 16, 20000, False), (8, 5, 9000, False),
+                                            (8, 10, 120000, False)])
+def test_model_call_on_a_scratch_of_the_layer_calls(ck, Hq, c, L, refused):
+    # chunk sizes 10 and 20 need the model's scratch, as they always have, unless a CTA's key range is too long; the others
+    # run layer by layer on the layer calls' scratch
+    Hkv, d, w, n = 8, 64, 4, 96
+    budget = w + c * (L // (6 * c))
+    x = _layer(Hq, Hkv, d, L, w, seed=L + c)
+    n_max = ck.out_len(L, w, c, budget)
+    need, layers = (int(ck.lib.chunkkv_model_workspace_bytes(n, L, Hq, Hkv, d, w, c, budget, 3)), ck.workspace_bytes(L, Hq, Hkv, d, w, c))
+    assert layers < need
+    ck.set_workspace(None)
+    want = ck.compress_layer(*x, Hq, w, c, budget)
+    out = (torch.empty(n, Hkv, n_max, d, dtype=torch.bfloat16, device="cuda"), torch.empty(n, Hkv, n_max, d, dtype=torch.bfloat16, device="cuda"),
+           torch.full((n, Hkv, n_max), -7, dtype=torch.int32, device="cuda"))
+    arr = ctypes.c_void_p * n
+    ptrs = [arr(*[t.data_ptr()] * n) for t in x] + [arr(*[o[l].data_ptr() for l in range(n)]) for o in out]
+
+    def call(ws):
+        ck.set_workspace(ws)
+        return ck.lib.chunkkv_compress_model(n, *ptrs[:3], L, Hq, Hkv, d, w, c, budget, 3, *ptrs[3:], None)
+
+    def same():
+        assert ck.device_status() == 0
+        return all(torch.equal(o[l], v) for o, v in zip((out[0], out[1], out[2]), want) for l in (0, 1, n - 1))
+
+    ws = Guarded((layers,), torch.uint8)
+    assert call(ws.t) == (-4 if refused else 0)
+    assert bool((out[2] == -7).all()) if refused else same()
+    ws.check("layer scratch")
+    out[2].fill_(-7)
+    assert call(Guarded((need,), torch.uint8).t) == 0 and same()
+    assert call(torch.empty(4096, dtype=torch.uint8, device="cuda")) == -4
