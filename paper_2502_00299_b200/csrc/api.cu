@@ -188,7 +188,7 @@ int try_resident(DeviceCtx& ctx, char* base, size_t bytes, const ResidentCall& r
     if (C <= 0 || !make_resident_plan(L, R, Hkv, d, c, C, rc.n_max, ctas, smem_budget(ctx), &plan)) return CHUNKKV_OK;
     if (base == nullptr || kHeaderBytes + resident_scratch_floats(plan, Hkv, C) * sizeof(float) > bytes) return CHUNKKV_OK;
     CUtensorMap tm_q, tm_k;
-    int st = encode_bf16_3d(&tm_q, rc.q_obs, d, R, Hkv, R < 128 ? R : 128, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
+    int st = encode_bf16_3d(&tm_q, rc.q_obs, d, R, Hkv, resident_q_box_rows(plan, R), CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
     if (st != CHUNKKV_OK) return st;
     st = encode_bf16_3d(&tm_k, rc.K, d, L, Hkv, L < plan.tile ? L : plan.tile, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, rc.kt, rc.kh);
     if (st != CHUNKKV_OK) return st;

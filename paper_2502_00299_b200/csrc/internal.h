@@ -83,7 +83,8 @@ cudaError_t launch_layer_fused(const ScorePlan& plan, const CUtensorMap& tm_q, c
 struct ResidentPlan {
     int c_static;     // 5, 8, 10, 16, 20 or 32
     int n_mt;         // 128-row query tiles per KV head (1 or 2)
-    int grid, cph;
+    int shift;        // 1: more than 128 rows are scored as two heads of half the rows instead
+    int grid, cph;    // CTAs, and per scoring head
     int tile, n_tiles;   // keys per accumulator tile, tiles per head
     int t_max;        // most tiles any CTA takes
     int spp;          // chunk slots per panel (half a tile)
@@ -120,6 +121,8 @@ struct ResidentIO {
 // than heads, kept positions or chunk scores beyond shared memory).
 bool make_resident_plan(int L, int R, int Hkv, int d, int c, int C, int n_max, int max_ctas, int smem_limit,
                         ResidentPlan* plan);
+// Rows of a box of the query tensor map.
+inline int resident_q_box_rows(const ResidentPlan& plan, int R) { return plan.shift ? (R + 1) / 2 : (R < 128 ? R : 128); }
 size_t resident_scratch_floats(const ResidentPlan& plan, int Hkv, int C);
 cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                                   const ResidentIO& io, cudaStream_t stream);

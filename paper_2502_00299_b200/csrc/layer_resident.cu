@@ -1,7 +1,7 @@
-// The whole layer in one cooperative launch with the chunk partial sums kept on chip
+// The whole layer in one launch with the chunk partial sums kept on chip
 // (ChunkKV Algorithm 3: observe-window scores, chunk scores, top-k, index_select on K and V).
 //
-// Every CTA belongs to one KV head and owns a contiguous range of its keys. While it streams its
+// Every CTA belongs to one scoring head and owns a contiguous range of its keys. While it streams its
 // keys through the tensor cores it keeps, per query row and chunk, the sum of exp2(s - m_panel) in
 // TENSOR MEMORY (lane = query row, column = chunk of the CTA's range, 256 columns beside the two
 // accumulator buffers) and the panel maxima in shared memory, so for most shapes nothing but a
@@ -9,37 +9,43 @@
 // range with more panels than those 256 columns hold (long contexts, small chunks) keeps the rest
 // in scratch (L2): written and read back by the same thread, 16 bytes at a time.
 //
-// A KV head with more than 128 query rows (two query tiles) is scored by the same CTAs: each key
-// tile is loaded once and multiplied with both query tiles, and the two pairs of epilogue groups
-// take one query tile each; with one query tile the pairs take alternate key tiles. In both cases
-// the CTA's products are numbered in issue order ("virtual tiles"), accumulator and pair = number
-// modulo 2, so one set of loops serves both.
+// A KV head is one scoring head where it has at most 128 query rows. With more, one of two forms:
+//   - two scoring heads of half the rows each, with half the CTAs each, where all their panels stay on chip; the two
+//     vectors of chunk scores are added in the selection;
+//   - two query tiles, scored by the same CTAs: each key tile is loaded once and multiplied with both, and the two pairs
+//     of epilogue groups take one query tile each; with one query tile the pairs take alternate key tiles. In both cases
+//     the CTA's products are numbered in issue order ("virtual tiles"), accumulator and pair = number modulo 2, so one set
+//     of loops serves both.
+// Two heads are the faster form wherever their panels stay on chip (device times, two tiles -> two heads; 64 heads over 8,
+// c = 10: 1024 tokens 15.8 -> 13.9 us, 4096 18.3 -> 16.5, 10248 22.7 -> 20.8, 20480 31.0 -> 29.2; c = 20, 45000 tokens 50.5 -> 48.9;
+// 16 over 2, 8192 tokens 18.2 -> 15.6): a CTA has half the exponentials to do between the latencies of its chain, twice as
+// many CTAs gather, and K's second reading is an L2 hit. Past that the partial sums in scratch would double as well.
 //
-// What bounds it (8 KV heads, d 128, B200): up to 128 rows the DRAM stream of K while scoring (13 of
-// 33.5 us at 32K tokens, c = 10) and then a chain of latencies (two hand-overs, selection, gather);
+// What bounds it (8 KV heads, d 128, B200): up to 128 rows the DRAM stream of K while scoring (12 of
+// 30 us on the device at 32K tokens, c = 10) and then a chain of latencies (two hand-overs, selection, gather);
 // beyond 128 rows the special-function unit (one exponential per score element, 16 per clock and
-// SM: 78 % of that rate while scoring). Against the kernel of score.cu, which kept every partial sum
-// in scratch, loaded K once per query tile and took run-time chunk sizes: c = 16, 29695 tokens, 256 rows
-// 107 -> 41 us; c = 20, 131072 tokens, 256 rows 147 -> 134 us; chunk scores alone (c = 10, 62261
-// tokens, 128 rows, four launches) 50 -> 33 us.
+// SM: 78 % of that rate while scoring). Against the kernel of score.cu, which keeps every partial sum
+// in scratch, loads K once per query tile and takes run-time chunk sizes: c = 16, 32768 tokens, 256 rows
+// 121 -> 41 us; c = 20, 131072 tokens, 256 rows 161 -> 139 us; chunk scores alone (c = 10, 32768
+// tokens, 128 rows, four launches) 32 -> 20 us.
 //
-//   1. score      TMA -> tcgen05.mma (128 rows x 120 keys per accumulator tile) -> epilogue
+//   1. score      TMA -> tcgen05.mma (128 rows x 120 or 128 keys per accumulator tile) -> epilogue
 //                 warps: one exponential per score element, chunk sums to tensor memory
 //   2. hand-over  the CTAs of a scoring head publish their per-row (max, sum) and wait for one
 //                 another on a per-head counter (bounded wait)
 //   3. contract   every CTA merges the head's records into m_i and 1 / l_i and contracts its own
 //                 partial sums over the rows: chunk scores of its key range -> global memory
 //   4. hand-over  per KV head, until all of its chunk scores are there (bounded wait)
-//   5. select     every CTA of the head runs the same exact top-k over the head's chunk scores
+//   5. select     every CTA of the KV head runs the same exact top-k over the head's chunk scores
 //                 and so holds the kept chunks in shared memory without a third wait
 //   6. gather     the head's output positions are split evenly over its CTAs: each expands its
 //                 share to token positions, writes them to out_idx and moves their rows
 //
 // Without out_idx the kernel ends after step 3 (chunk scores are the result).
 //
-// Heads never wait for each other. The launch is cooperative only so that all CTAs are resident
-// while they wait for their head's other CTAs; every wait gives up after a clock limit, raises the
-// device status word and lets the CTA leave.
+// Heads never wait for each other. All CTAs of a launch are resident while they wait for their head's other CTAs: at
+// most one per SM, and a cooperative launch where several launches share the GPU (lanes); every wait gives up after a
+// clock limit, raises the device status word and lets the CTA leave.
 #include "gather.cuh"
 #include "internal.h"
 #include "panels.cuh"
@@ -70,11 +76,12 @@ struct ResCtl {
 struct ResArgs {
     int L, P, w, R, d;                 // R rows per KV head
     int n_mt;                          // 128-row query tiles per KV head (1 or 2)
+    int shift;                         // 1: the rows of a KV head are scored as two heads of q_rows and the rest
+    int q_rows;                        // rows of a box of the query tensor map: 128, fewer, or the half's
     float sl2;                         // log2(e) / sqrt(d)
-    int cph;                           // CTAs per KV head (grid = Hkv * cph)
+    int cph;                           // CTAs per scoring head (a KV head, or one of its halves)
     int n_tiles;                       // accumulator tiles per head
     int n_stages;
-    int q_box_rows, k_box_rows;
     int C, k, n_max, Hkv;
     int off_ring, ring_bytes, off_pmax, off_misc;   // dynamic shared memory layout (bytes from the aligned base)
     int n_on, n_off;                   // panels of a CTA kept on chip; room for panels in scratch
@@ -95,8 +102,8 @@ struct ResArgs {
     unsigned* counters;                // header + kResidentCountersOffset, zero between launches
 
     __device__ unsigned* exits() const { return counters; }              // CTAs that left; the last one clears the counters
-    __device__ unsigned* cnt_a(int h) const { return counters + 16 + h; }                          // hand-over 2 of a KV head
-    __device__ unsigned* cnt_b(int h) const { return counters + 16 + kResidentMaxHeads + h; }      // hand-over 4
+    __device__ unsigned* cnt_a(int h) const { return counters + 16 + h; }                          // hand-over 2 of a scoring head
+    __device__ unsigned* cnt_b(int h) const { return counters + 16 + kResidentMaxHeads + h; }      // hand-over 4 of a KV head
     __device__ int* status() const { return reinterpret_cast<int*>(counters) - kResidentCountersOffset / sizeof(int); }
 };
 // The launch costs the host more with more parameter bytes than this: 488 -> 504 bytes took 0.45 us of a serving layer's 30.3
@@ -157,7 +164,9 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     volatile int* abort_flag = &ctl.abort_flag;
     const uint32_t n_stages = static_cast<uint32_t>(a.n_stages);
 
-    const int hkv = blockIdx.x / a.cph, part = blockIdx.x - hkv * a.cph;
+    const int hs = blockIdx.x / a.cph, part = blockIdx.x - hs * a.cph;      // scoring head, key range
+    const int hkv = BIG ? hs : hs >> a.shift, row0 = BIG ? 0 : (hs & a.shift) * a.q_rows;
+    const int n_rows = BIG ? a.R : (a.shift ? (row0 ? a.R - row0 : a.q_rows) : a.R);   // rows of the scoring head
     // tiles are dealt out rounding up, so the head's last CTA - whose last panels take the slow, masked path -
     // is never one of those that get an extra tile
     const int t_begin = (a.n_tiles * part + a.cph - 1) / a.cph, t_end = (a.n_tiles * (part + 1) + a.cph - 1) / a.cph;
@@ -201,11 +210,11 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         // ------------------------------------------------------------------ TMA producer
         if (elect_one() && nt > 0) {
             const uint32_t qbar = smem_u32(&ctl.qfull);
-            mbar_arrive_expect_tx(qbar, static_cast<uint32_t>(n_mt * KB * a.q_box_rows) * 128u);
+            mbar_arrive_expect_tx(qbar, static_cast<uint32_t>(n_mt * KB * a.q_rows) * 128u);
             for (int mt = 0; mt < n_mt; ++mt)      // (rows past R of the second tile arrive as zeros)
                 for (int kb = 0; kb < KB; ++kb)
-                    tma_load_3d(q_base + static_cast<uint32_t>(mt * KB + kb) * kRQTileBytes, &tm_q, qbar, kb * 64, mt * 128, hkv);
-            const uint32_t k_bytes = static_cast<uint32_t>(a.k_box_rows) * 128u;
+                    tma_load_3d(q_base + static_cast<uint32_t>(mt * KB + kb) * kRQTileBytes, &tm_q, qbar, kb * 64, row0 + mt * 128, hkv);
+            const uint32_t k_bytes = static_cast<uint32_t>(min(a.L, TILE)) * 128u;
             uint32_t st = 0, st_par = 1;
             int issued = 0;
             bool ok = true;
@@ -278,8 +287,8 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         const int pair = grp >> 1, half = grp & 1;
         const int row = quarter * 32 + lane;             // row of the query tile = lane of tensor memory
         const int qrow = row + (two ? pair * 128 : 0);   // row of the KV head
-        const bool active = qrow < a.R;
-        const int last_visible = a.P + (qrow % a.w);     // this row sees keys j <= P + r (all < L)
+        const bool active = qrow < n_rows;
+        const int last_visible = a.P + ((row0 + qrow) % a.w);     // this row sees keys j <= P + r (all < L)
         const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
         const uint64_t keep = l2_policy_evict_last();
         float run_m = -CUDART_INF_F, run_l = 0.f;
@@ -352,7 +361,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             dst[i] = M;
             dst[128 + i] = Ls;
         }
-        ok = head_handover(a.cnt_a(hkv), static_cast<unsigned>(a.cph), ctl);
+        ok = head_handover(a.cnt_a(hs), static_cast<unsigned>(a.cph), ctl);
     }
 
     // ---- 3. row statistics of the head, then this CTA's chunk scores
@@ -362,7 +371,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         if (threadIdx.x < 512) {
             const int i = threadIdx.x & 127, sl = (threadIdx.x >> 7) & (n_sl - 1), mt = two ? threadIdx.x >> 8 : 0;
             const size_t step = static_cast<size_t>(n_mt) * 256;
-            const float* src = a.cta_stat + (static_cast<size_t>(hkv) * a.cph * n_mt + mt) * 256 + i;
+            const float* src = a.cta_stat + (static_cast<size_t>(hs) * a.cph * n_mt + mt) * 256 + i;
             float M = -CUDART_INF_F, Ls = 0.f;
             // records in flight per thread: enough for one round trip where a head has 18 CTAs (8 heads)
             constexpr int kF = BIG ? 9 : 5;
@@ -414,7 +423,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         if (warp >= 2) {
             const int grp = (warp - 2) >> 2, quarter = warp & 3;
             const int row = quarter * 32 + lane, mt = two ? grp >> 1 : 0;
-            const bool active = mt * 128 + row < a.R;
+            const bool active = mt * 128 + row < n_rows;
             const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
             const int srow = active ? row : 0;           // (rows that do not exist have no record)
             const float mi = gm[mt * 128 + row], li = ginv[mt * 128 + row];
@@ -477,16 +486,18 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 const float* r = red + lc;
                 float t = (r[0] + r[n_local]) + (r[2 * n_local] + r[3 * n_local]);
                 if (two) t += (r[4 * n_local] + r[5 * n_local]) + (r[6 * n_local] + r[7 * n_local]);
-                a.scores[static_cast<size_t>(hkv) * a.score_row + ch0 + lc] = t;
+                a.scores[static_cast<size_t>(hs) * a.score_row + ch0 + lc] = t;
             }
     }
     // ---- 4. wait for the KV head's other CTAs, 5. select, 6. gather
-    if (ok && a.out_idx != nullptr) ok = head_handover(a.cnt_b(hkv), static_cast<unsigned>(a.cph), ctl);
+    if (ok && a.out_idx != nullptr) ok = head_handover(a.cnt_b(hkv), static_cast<unsigned>(a.cph << (BIG ? 0 : a.shift)), ctl);
     if (ok && a.out_idx != nullptr) {
         SelectSmem& ss = *reinterpret_cast<SelectSmem*>(ring);
         constexpr size_t kSelBytes = (sizeof(SelectSmem) + 127) & ~size_t(127);
-        const float* sc = a.scores + static_cast<size_t>(hkv) * a.score_row;
-        const int Q = a.cph, q = part;                   // CTAs of this KV head
+        const int shift = BIG ? 0 : a.shift;
+        const float* sc = a.scores + (static_cast<size_t>(hkv) << shift) * a.score_row;
+        const float* sc2 = shift ? sc + a.score_row : nullptr;           // the other half's chunk scores are added
+        const int Q = a.cph << shift, q = (hs & shift) * a.cph + part;   // CTAs of this KV head
         const int r_begin = static_cast<int>(static_cast<long long>(a.n_max) * q / Q);
         const int r_end = static_cast<int>(static_cast<long long>(a.n_max) * (q + 1) / Q);
         int32_t* sidx = reinterpret_cast<int32_t*>(ring + kSelBytes);          // kept positions [r_begin, r_end) of the head
@@ -496,11 +507,11 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         const bool fits = kSelBytes + idx_bytes + static_cast<size_t>(a.C) * 4 <= static_cast<size_t>(a.ring_bytes);
         if (min(a.k, a.C) <= kSelCap && a.C <= kSelMaxChunks && (fits || a.C <= kRThreads * 16)) {
             if (a.C <= kRThreads * 8)
-                select_core<8>(sc, nullptr, a.C, a.k, ss, nullptr);
+                select_core<8>(sc, sc2, a.C, a.k, ss, nullptr);
             else if (a.C <= kRThreads * 16)
-                select_core<16>(sc, nullptr, a.C, a.k, ss, nullptr);
+                select_core<16>(sc, sc2, a.C, a.k, ss, nullptr);
             else
-                select_core<0>(sc, nullptr, a.C, a.k, ss, kbuf);
+                select_core<0>(sc, sc2, a.C, a.k, ss, kbuf);
             // every CTA holds the head's kept chunks: it expands, writes and gathers its own share of the positions
             const int n_tok = select_tokens(a.P, C_STATIC, a.C, a.k, ss, a.tok_cap);
             for (int n = r_begin + threadIdx.x; n < r_end; n += kRThreads) {
@@ -510,7 +521,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             }
         } else {
             // very many chunks: every CTA of the head writes the same positions to out_idx and takes its share from there
-            select_head_rows(sc, nullptr, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, out_idx, ss, fits ? kbuf : nullptr, a.tok_cap);
+            select_head_rows(sc, sc2, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, out_idx, ss, fits ? kbuf : nullptr, a.tok_cap);
             for (int n = r_begin + threadIdx.x; n < r_end; n += kRThreads) sidx[n - r_begin] = out_idx[n];
         }
         __syncthreads();
@@ -541,7 +552,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         // abandoned wait the counters are left as they are; chunkkv_device_status clears them.)
         const unsigned old = atomicAdd(a.exits(), 1u);
         if (old + 1u == gridDim.x) {
-            for (int h = 0; h < a.Hkv; ++h) { *a.cnt_a(h) = 0u; *a.cnt_b(h) = 0u; }
+            for (int h = 0; h < a.Hkv << a.shift; ++h) { *a.cnt_a(h) = 0u; *a.cnt_b(h) = 0u; }
             *a.exits() = 0u;
             __threadfence();
         }
@@ -557,27 +568,36 @@ const void* kernel_of(bool big) {
 }  // namespace
 
 size_t resident_scratch_floats(const ResidentPlan& plan, int Hkv, int C) {
-    return static_cast<size_t>(plan.grid) * plan.n_mt * 256 + ((static_cast<size_t>(Hkv) * ((C + 3) & ~3) + 63) & ~static_cast<size_t>(63)) +
+    return static_cast<size_t>(plan.grid) * plan.n_mt * 256 + (((static_cast<size_t>(Hkv) << plan.shift) * ((C + 3) & ~3) + 63) & ~static_cast<size_t>(63)) +
            static_cast<size_t>(plan.grid) * plan.n_off * (plan.spp + 1) * plan.spill_rows;
 }
 
 bool make_resident_plan(int L, int R, int Hkv, int d, int c, int C, int n_max, int max_ctas, int smem_limit,
                         ResidentPlan* plan) {
-    // chunk sizes that divide a panel of 60 or 64 keys and leave at least two chunks in it; the others (and token
-    // level, where a partial sum per chunk would be the score matrix itself) take other kernels
+    // The chunk sizes that are compiled in: of those that divide a panel of 60 or 64 keys, 5, 10 and 20 of the method's
+    // ablation and the page sizes 8, 16 and 32. 3, 4, 6, 12, 15 and 30 divide 60 as well and would fit; each costs two
+    // kernels here, two in model_kernel.cu and 3 MB of library. They and the sizes that divide neither take the kernels of
+    // score.cu (32768 tokens, 128 rows: c = 15 88 us, c = 16 here 29), token level token_kernel.cu.
     if (c != 5 && c != 8 && c != 10 && c != 16 && c != 20 && c != 32) return false;
     if (R < 1 || R > 256 || (d != 64 && d != 128) || L < 1 || C < 1 || Hkv < 1 || Hkv > kResidentMaxHeads) return false;
     if (max_ctas < Hkv) return false;
     ResidentPlan p{};
     p.c_static = c;
-    p.n_mt = R > 128 ? 2 : 1;
     const int tile = 2 * panel_keys(c);
     p.spp = panel_keys(c) / c;
     p.tile = tile;
     p.n_tiles = (L + tile - 1) / tile;
-    p.cph = max_ctas / Hkv;
+    // More than 128 rows as two scoring heads where all panels of such a head stay on chip (see the top of this file); chunk
+    // scores alone (no positions to fill) always as two query tiles, which leave nothing to add afterwards.
+    const int halves = max_ctas / (2 * Hkv) < p.n_tiles ? max_ctas / (2 * Hkv) : p.n_tiles;
+    if (R > 128 && n_max > 0 && halves > 0 && 2 * Hkv <= kResidentMaxHeads) {
+        const int t = (p.n_tiles + halves - 1) / halves;
+        p.shift = 2 * t * p.spp <= kRPartCols ? 1 : 0;
+    }
+    p.n_mt = R > 128 && p.shift == 0 ? 2 : 1;
+    p.cph = max_ctas / (Hkv << p.shift);
     if (p.cph > p.n_tiles) p.cph = p.n_tiles;                       // a CTA without keys would only lengthen the hand-overs
-    p.grid = p.cph * Hkv;
+    p.grid = p.cph * (Hkv << p.shift);
     p.t_max = (p.n_tiles + p.cph - 1) / p.cph;
     const int n_pl = 2 * p.n_mt * p.t_max;                          // panels of a CTA
     p.n_on = kRPartCols / p.spp;
@@ -599,7 +619,7 @@ bool make_resident_plan(int L, int R, int Hkv, int d, int c, int C, int n_max, i
     p.smem_bytes = 1024 + p.off_misc + kRMiscBytes;
     // after scoring the ring holds the row sums of the chunk scores, then the selection scratch and the kept positions
     if (static_cast<size_t>(p.n_mt) * 4 * p.t_max * (tile / c) * 4 > static_cast<size_t>(p.ring_bytes)) return false;
-    const size_t own = static_cast<size_t>(n_max) / p.cph + 1;      // kept positions of a CTA
+    const size_t own = static_cast<size_t>(n_max) / (p.cph << p.shift) + 1;      // kept positions of a CTA
     const size_t sel_bytes = ((sizeof(SelectSmem) + 127) & ~size_t(127)) + ((own * 4 + 127) & ~size_t(127));
     if (sel_bytes > static_cast<size_t>(p.ring_bytes)) return false;
     *plan = p;
@@ -612,8 +632,7 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     a.L = io.L; a.P = io.L - io.w; a.w = io.w; a.R = io.R; a.d = io.d; a.n_mt = plan.n_mt;
     a.sl2 = io.sl2;
     a.cph = plan.cph; a.n_tiles = plan.n_tiles; a.n_stages = plan.n_stages;
-    a.q_box_rows = io.R < 128 ? io.R : 128;
-    a.k_box_rows = io.L < plan.tile ? io.L : plan.tile;
+    a.shift = plan.shift; a.q_rows = resident_q_box_rows(plan, io.R);
     a.C = io.C; a.k = io.k; a.n_max = io.n_max; a.Hkv = io.Hkv;
     a.n_on = plan.n_on; a.n_off = plan.n_off; a.spill_rows = plan.spill_rows;
     a.off_ring = plan.off_ring; a.ring_bytes = plan.ring_bytes; a.off_pmax = plan.off_pmax; a.off_misc = plan.off_misc;
@@ -632,7 +651,7 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     float* scores = io.scratch + static_cast<size_t>(plan.grid) * plan.n_mt * 256;
     a.scores = io.out_scores ? io.out_scores : scores;
     a.score_row = io.out_scores ? io.C : (io.C + 3) & ~3;
-    a.spill = scores + ((static_cast<size_t>(io.Hkv) * ((io.C + 3) & ~3) + 63) & ~static_cast<size_t>(63));
+    a.spill = scores + (((static_cast<size_t>(io.Hkv) << plan.shift) * ((io.C + 3) & ~3) + 63) & ~static_cast<size_t>(63));
     a.counters = io.counters;
     const bool big = plan.n_mt == 2 || plan.n_off > 0;
     const void* kern = nullptr;

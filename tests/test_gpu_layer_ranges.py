@@ -61,6 +61,17 @@ def test_layer_and_chunk_scores(ck, Hq, Hkv, d, L, w, c):
     assert np.array_equal(sidx.cpu().numpy(), idx) and torch.equal(sK, oK) and torch.equal(sV, oV)
 
 
+# More than 128 rows: two scoring heads of half the rows where all their panels stay on chip, else two query tiles. Odd numbers of
+# rows, the last length of the one form and the first of the other (32 KV heads: two CTAs a half, 21 tiles each hold 252 chunk slots),
+# more KV heads than a hand-over counter per half leaves room for.
+@pytest.mark.parametrize("Hq,Hkv,d,L,w,c", [
+    (3, 1, 64, 900, 43, 10), (5, 1, 128, 1003, 51, 5), (14, 2, 128, 130, 32, 16), (128, 32, 64, 2 * 21 * 120, 64, 10),
+    (128, 32, 64, 2 * 21 * 120 + 1, 64, 10), (160, 80, 64, 700, 65, 20), (64, 8, 128, 300, 32, 32),
+])
+def test_layer_with_more_than_128_rows(ck, Hq, Hkv, d, L, w, c):
+    test_layer_and_chunk_scores(ck, Hq, Hkv, d, L, w, c)
+
+
 # a model call's CTA takes ceil(ceil(L / tile) / (144 / Hkv)) key tiles of every layer; its ring of partial sums continues in
 # scratch where a layer and eight panels more do not fit on chip, and always has both forms with two query tiles
 MODEL_CASES = [
