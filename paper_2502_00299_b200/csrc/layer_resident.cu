@@ -80,9 +80,8 @@ struct ResArgs {
     int q_rows;                        // rows of a box of the query tensor map: 128, fewer, or the half's
     float sl2;                         // log2(e) / sqrt(d)
     int cph;                           // CTAs per scoring head (a KV head, or one of its halves)
-    int n_tiles;                       // accumulator tiles per head
     int n_stages;
-    int C, k, n_max, Hkv;
+    int k, n_max, Hkv;
     int off_ring, ring_bytes, off_pmax, off_misc;   // dynamic shared memory layout (bytes from the aligned base)
     int n_on, n_off;                   // panels of a CTA kept on chip; room for panels in scratch
     int spill_rows;                    // rows of a panel's record in scratch
@@ -106,9 +105,10 @@ struct ResArgs {
     __device__ unsigned* cnt_b(int h) const { return counters + 16 + kResidentMaxHeads + h; }      // hand-over 4 of a KV head
     __device__ int* status() const { return reinterpret_cast<int*>(counters) - kResidentCountersOffset / sizeof(int); }
 };
-// The launch costs the host more with more parameter bytes than this: 488 -> 504 bytes took 0.45 us of a serving layer's 30.3
-// (a launch between other kernels' launches; hence the addresses above that follow from one pointer).
-static_assert(2 * sizeof(CUtensorMap) + sizeof(ResArgs) <= 488, "kernel parameters");
+// A launch that comes between others costs the host more or less with the size of the parameters. A serving layer (window queries,
+// then this; 30 us a pass) against the 488 bytes of an older form, padded and timed in turn: 464 bytes +0.35 us, 472 and 480
+// -0.1 to -0.3, 488 +0.2, 496 to 520 +0.3 to +0.45, 544 -0.2. What follows from other members is computed in the kernel.
+static_assert(2 * sizeof(CUtensorMap) + sizeof(ResArgs) == 480, "kernel parameters");
 
 // One thread publishes this CTA's arrival on `counter` and waits until `target` CTAs have arrived.
 // Block-wide: every thread calls it; returns false if the wait was abandoned.
@@ -169,7 +169,8 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     const int n_rows = BIG ? a.R : (a.shift ? (row0 ? a.R - row0 : a.q_rows) : a.R);   // rows of the scoring head
     // tiles are dealt out rounding up, so the head's last CTA - whose last panels take the slow, masked path -
     // is never one of those that get an extra tile
-    const int t_begin = (a.n_tiles * part + a.cph - 1) / a.cph, t_end = (a.n_tiles * (part + 1) + a.cph - 1) / a.cph;
+    const int n_tiles = (a.L + TILE - 1) / TILE, C = (a.P + C_STATIC - 1) / C_STATIC;
+    const int t_begin = (n_tiles * part + a.cph - 1) / a.cph, t_end = (n_tiles * (part + 1) + a.cph - 1) / a.cph;
     const int nt = t_end - t_begin;
     const int n_mt = BIG ? a.n_mt : 1;
     const bool two = n_mt == 2;                      // two query tiles
@@ -482,7 +483,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         __syncthreads();
         const int ch0 = t_begin * (TILE / C_STATIC);     // this CTA's first chunk
         for (int lc = threadIdx.x; lc < n_local; lc += kRThreads)
-            if (ch0 + lc < a.C) {
+            if (ch0 + lc < C) {
                 const float* r = red + lc;
                 float t = (r[0] + r[n_local]) + (r[2 * n_local] + r[3 * n_local]);
                 if (two) t += (r[4 * n_local] + r[5 * n_local]) + (r[6 * n_local] + r[7 * n_local]);
@@ -504,16 +505,16 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         int32_t* out_idx = a.out_idx + static_cast<size_t>(hkv) * a.n_max;
         const size_t idx_bytes = (static_cast<size_t>(r_end - r_begin) * 4 + 127) & ~size_t(127);
         uint32_t* kbuf = reinterpret_cast<uint32_t*>(ring + kSelBytes + idx_bytes);
-        const bool fits = kSelBytes + idx_bytes + static_cast<size_t>(a.C) * 4 <= static_cast<size_t>(a.ring_bytes);
-        if (min(a.k, a.C) <= kSelCap && a.C <= kSelMaxChunks && (fits || a.C <= kRThreads * 16)) {
-            if (a.C <= kRThreads * 8)
-                select_core<8>(sc, sc2, a.C, a.k, ss, nullptr);
-            else if (a.C <= kRThreads * 16)
-                select_core<16>(sc, sc2, a.C, a.k, ss, nullptr);
+        const bool fits = kSelBytes + idx_bytes + static_cast<size_t>(C) * 4 <= static_cast<size_t>(a.ring_bytes);
+        if (min(a.k, C) <= kSelCap && C <= kSelMaxChunks && (fits || C <= kRThreads * 16)) {
+            if (C <= kRThreads * 8)
+                select_core<8>(sc, sc2, C, a.k, ss, nullptr);
+            else if (C <= kRThreads * 16)
+                select_core<16>(sc, sc2, C, a.k, ss, nullptr);
             else
-                select_core<0>(sc, sc2, a.C, a.k, ss, kbuf);
+                select_core<0>(sc, sc2, C, a.k, ss, kbuf);
             // every CTA holds the head's kept chunks: it expands, writes and gathers its own share of the positions
-            const int n_tok = select_tokens(a.P, C_STATIC, a.C, a.k, ss, a.tok_cap);
+            const int n_tok = select_tokens(a.P, C_STATIC, C, a.k, ss, a.tok_cap);
             for (int n = r_begin + threadIdx.x; n < r_end; n += kRThreads) {
                 const int pos = select_position(ss, n, n_tok, C_STATIC, a.P, a.w);
                 sidx[n - r_begin] = pos;
@@ -521,7 +522,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             }
         } else {
             // very many chunks: every CTA of the head writes the same positions to out_idx and takes its share from there
-            select_head_rows(sc, sc2, a.L, a.w, C_STATIC, a.C, a.k, a.n_max, out_idx, ss, fits ? kbuf : nullptr, a.tok_cap);
+            select_head_rows(sc, sc2, a.L, a.w, C_STATIC, C, a.k, a.n_max, out_idx, ss, fits ? kbuf : nullptr, a.tok_cap);
             for (int n = r_begin + threadIdx.x; n < r_end; n += kRThreads) sidx[n - r_begin] = out_idx[n];
         }
         __syncthreads();
@@ -631,9 +632,9 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     ResArgs a{};
     a.L = io.L; a.P = io.L - io.w; a.w = io.w; a.R = io.R; a.d = io.d; a.n_mt = plan.n_mt;
     a.sl2 = io.sl2;
-    a.cph = plan.cph; a.n_tiles = plan.n_tiles; a.n_stages = plan.n_stages;
+    a.cph = plan.cph; a.n_stages = plan.n_stages;
     a.shift = plan.shift; a.q_rows = resident_q_box_rows(plan, io.R);
-    a.C = io.C; a.k = io.k; a.n_max = io.n_max; a.Hkv = io.Hkv;
+    a.k = io.k; a.n_max = io.n_max; a.Hkv = io.Hkv;
     a.n_on = plan.n_on; a.n_off = plan.n_off; a.spill_rows = plan.spill_rows;
     a.off_ring = plan.off_ring; a.ring_bytes = plan.ring_bytes; a.off_pmax = plan.off_pmax; a.off_misc = plan.off_misc;
     a.K = static_cast<const uint4*>(io.K); a.V = static_cast<const uint4*>(io.V);
