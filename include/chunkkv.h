@@ -35,7 +35,9 @@
  *   - Scratch memory: scoring needs device scratch of chunkkv_workspace_bytes(...) bytes. The
  *     library never allocates and never frees: the caller hands it a buffer once with
  *     chunkkv_set_workspace (a set-up call), and every entry point that scores returns
- *     CHUNKKV_ENOWORKSPACE while no buffer, or too small a buffer, is set. Calls that use the
+ *     CHUNKKV_ENOWORKSPACE while no buffer, or too small a buffer, is set. (A buffer below that
+ *     size may still hold another kernel's scratch: the call then runs that one, and chunk scores
+ *     may differ in their last bits.) Calls that use the
  *     scratch of one device must be ordered on the GPU (same stream, or otherwise serialised):
  *     concurrent calls would share it. Lanes and pipes (below) take their scratch per object.
  */
@@ -102,9 +104,9 @@ CHUNKKV_API int chunkkv_device_status(void* stream);
  * Steps "observe-window attention scores" and "chunk score calculation" (Algorithm 3; Algorithm 1
  * "Observe Window Calculation" / "Chunk Attention Score Calculation").
  *   out_chunk_scores [Hkv, C] f32   required
- *   out_token_scores [Hkv, P] f32   optional (NULL to skip); computed by a second pass of the
- *                                   same kernels with chunk size 1, so it costs scratch for
- *                                   chunk size 1 as well
+ *   out_token_scores [Hkv, P] f32   optional (NULL to skip); needs the scratch of chunk size 1,
+ *                                   and the chunk scores are then sums of the token scores, so
+ *                                   their last bits may differ from a call without token scores
  * With P == 0 nothing is written.
  */
 CHUNKKV_API int chunkkv_score(const void* q_obs, const void* K, int L, int Hq, int Hkv, int d, int w, int c,
@@ -202,8 +204,8 @@ CHUNKKV_API int chunkkv_compress_layer(const void* q_obs, const void* K, const v
  *   [L, Hkv, d] has token stride Hkv * d and head stride d. Strides are in bf16 elements, multiples
  *   of 8 and at least d; K and V 16-byte aligned. The outputs are packed as usual. With the packed
  *   strides (d and L * d) this is chunkkv_compress_layer itself; otherwise the one-launch layer kernel
- *   where the shape fits it (chunk sizes 10 and 20, up to 128 score rows per scoring head), else separate
- *   score / select / gather launches. Returns CHUNKKV_EINVAL_SHAPE for other strides.
+ *   where the shape fits it (chunk sizes 5, 8, 10, 16, 20 and 32), else separate score / select / gather
+ *   launches. Returns CHUNKKV_EINVAL_SHAPE for other strides.
  */
 CHUNKKV_API int chunkkv_window_queries(const void* qkv, long long row_elems, int T, int Hq, int Hkv, int d, int w,
                                        const float* cos_rows, const float* sin_rows, void* out_q_obs, void* stream);
@@ -253,8 +255,8 @@ CHUNKKV_API int chunkkv_compress_model(int n_layers, const void* const* q_obs, c
  * chunkkv_compress_model on keys and values that are not packed [Hkv, L, d] (the same strides, in bf16
  * elements, for every layer: see chunkkv_compress_layer_strided; a token-major cache [L, Hkv, d] has
  * token stride Hkv * d and head stride d). Outputs are packed. The persistent kernel scores through
- * tensor maps with those strides and copies the kept rows one row at a time; shapes it does not take
- * run layer by layer. No counterpart in the paper: it is Algorithm 2 on another memory layout.
+ * tensor maps with those strides and fetches the kept rows a chunk at a time through others; shapes it
+ * does not take run layer by layer. No counterpart in the paper: it is Algorithm 2 on another memory layout.
  */
 CHUNKKV_API int chunkkv_compress_model_strided(int n_layers, const void* const* q_obs, const void* const* K,
                                                const void* const* V, int L, int Hq, int Hkv, int d, int w, int c,
@@ -286,7 +288,8 @@ CHUNKKV_API int chunkkv_compress_model_paged(int n_layers, const void* const* q_
  * out_V for these two calls; a kept clipped last chunk leaves -1 / zero-row padding at the end.
  * Chunk grid, tie-break, layouts, ownership and error codes are those of chunkkv_select and
  * chunkkv_compress_layer (no index reuse argument: reuse layers call chunkkv_compress_layer or
- * chunkkv_gather with these indices). Scoring, selection and gathering run as three launches.
+ * chunkkv_gather with these indices). One launch of the layer kernel where the shape fits it, else
+ * scoring, selection and gathering as separate launches.
  */
 CHUNKKV_API int chunkkv_budget_from_ratio(int L, double ratio);
 CHUNKKV_API int chunkkv_num_kept_chunks_alg1(int L, int w, int c, int budget);

@@ -927,6 +927,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
 }  // namespace
 
 bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, ModelPlan* plan) {
+    // the chunk sizes that are compiled in, as in layer_resident.cu
     if (c != 5 && c != 8 && c != 10 && c != 16 && c != 20 && c != 32) return false;
     if (R < 1 || R > 256 || (d != 64 && d != 128) || L < 1 || C < 1 || k < 1 || Hkv < 1 || Hkv > kResidentMaxHeads)
         return false;

@@ -8,10 +8,8 @@
 
 namespace chunkkv {
 
-constexpr int kRTile = 120;                  // keys per accumulator tile
-constexpr int kRUmmaN = 128;                 // UMMA N (a multiple of 16): the last 8 columns are never read
+constexpr int kRUmmaN = 128;                 // UMMA N (a multiple of 16): a tile of 120 keys leaves the last 8 columns unread
 constexpr int kRPanel = 60;                  // keys per epilogue panel (half a tile)
-constexpr int kRStageBytes = kRTile * 128;   // one stage = 120 keys x 64 dims, 128-byte swizzled rows
 constexpr int kRMaxStages = 14;
 constexpr int kRPartCol0 = 256;              // tensor-memory column of the first chunk partial sum
 constexpr int kRPartCols = 256;
