@@ -649,7 +649,7 @@ def run_ours(args, wl):
             "algorithmic_bytes": bytes5, "GB/s": bytes5 / (ms5 * 1e-3) / 1e9,
             "frac_of_measured_peak": bytes5 / (ms5 * 1e-3) / 1e9 / peak,
             "note": "8 chunkkv_compress_model calls (one per sequence, 27 computed + 53 reusing layers each), sequences one "
-                    "after another; sequences too long for the persistent kernel's tensor-memory budget run layer by layer"}
+                    "after another, all through the persistent kernel"}
         del calls5, outs5
         torch.cuda.empty_cache()
 
