@@ -506,13 +506,8 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         const size_t idx_bytes = (static_cast<size_t>(r_end - r_begin) * 4 + 127) & ~size_t(127);
         uint32_t* kbuf = reinterpret_cast<uint32_t*>(ring + kSelBytes + idx_bytes);
         const bool fits = kSelBytes + idx_bytes + static_cast<size_t>(C) * 4 <= static_cast<size_t>(a.ring_bytes);
-        if (min(a.k, C) <= kSelCap && C <= kSelMaxChunks && (fits || C <= kRThreads * 16)) {
-            if (C <= kRThreads * 8)
-                select_core<8>(sc, sc2, C, a.k, ss, nullptr);
-            else if (C <= kRThreads * 16)
-                select_core<16>(sc, sc2, C, a.k, ss, nullptr);
-            else
-                select_core<0>(sc, sc2, C, a.k, ss, kbuf);
+        if (min(a.k, C) <= kSelCap && C <= kSelMaxChunks && (fits || C <= kRThreads * select_reg_keys(kSelLayer))) {
+            select_kept<kSelLayer>(sc, sc2, C, a.k, ss, kbuf);
             // every CTA holds the head's kept chunks: it expands, writes and gathers its own share of the positions
             const int n_tok = select_tokens(a.P, C_STATIC, C, a.k, ss, a.tok_cap);
             for (int n = r_begin + threadIdx.x; n < r_end; n += kRThreads) {

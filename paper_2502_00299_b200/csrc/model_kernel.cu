@@ -252,12 +252,8 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
             if (!flag[0]) return false;
             const float* sc = p.scores + (static_cast<size_t>(s) * p.Hkv + hkv) * p.n_mt * p.Cpad;
             const float* sc2 = p.n_mt == 2 ? sc + p.Cpad : nullptr;
-            if (p.C <= kMThreads * 8)
-                select_core<8>(sc, sc2, p.C, p.k, ss, nullptr);
-            else if (p.C <= kMThreads * 16)
-                select_core<16>(sc, sc2, p.C, p.k, ss, nullptr);
-            else if (p.sel_keys_fit)
-                select_core<0>(sc, sc2, p.C, p.k, ss, kbuf);
+            if (p.sel_keys_fit || p.C <= kMThreads * select_reg_keys(kSelModel))
+                select_kept<kSelModel>(sc, sc2, p.C, p.k, ss, kbuf);
             else
                 select_head_rows(sc, sc2, p.L, p.w, C_STATIC, p.C, p.k, p.n_max, p.layer[li].out_idx + static_cast<size_t>(hkv) * p.n_max,
                                  ss, nullptr);

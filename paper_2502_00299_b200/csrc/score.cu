@@ -858,20 +858,16 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             const float* sc2 = a.kv_shift ? sc + la.C : nullptr;        // the head's second scoring head
             int32_t* out = la.out_idx + static_cast<size_t>(h) * la.n_max;
             const bool sel_staged = min(la.k, la.C) <= kSelCap && la.C <= kSelMaxChunks;
-            if (sel_staged && la.C <= kThreads * 8) {
-                select_head<8>(sc, sc2, a.L, a.w, a.c, la.C, la.k, la.n_max, out, ss, nullptr);
-            } else {
-                // keys go to the idle dynamic shared memory behind the selection scratch; if they do
-                // not fit there (token-level selection of very long sequences) they replace the
-                // chunk scores, which nothing reads after the selection
-                uint32_t* kbuf = reinterpret_cast<uint32_t*>(dyn + ((sizeof(SelectSmem) + 127) & ~size_t(127)));
-                const bool fits = static_cast<size_t>(la.C) * 4 + sizeof(SelectSmem) + 256 <= static_cast<size_t>(g.dyn_bytes);
-                if (fits && sel_staged)
-                    select_head<0>(sc, sc2, a.L, a.w, a.c, la.C, la.k, la.n_max, out, ss, kbuf);
-                else
-                    select_head_rows(sc, sc2, a.L, a.w, a.c, la.C, la.k, la.n_max, out, ss,
-                                     fits ? kbuf : reinterpret_cast<uint32_t*>(const_cast<float*>(sc)));
-            }
+            // the keys of many chunks go to the idle dynamic shared memory behind the selection scratch; if they do
+            // not fit there (token-level selection of very long sequences) they replace the
+            // chunk scores, which nothing reads after the selection
+            uint32_t* kbuf = reinterpret_cast<uint32_t*>(dyn + ((sizeof(SelectSmem) + 127) & ~size_t(127)));
+            const bool fits = static_cast<size_t>(la.C) * 4 + sizeof(SelectSmem) + 256 <= static_cast<size_t>(g.dyn_bytes);
+            if (sel_staged && (fits || la.C <= kThreads * select_reg_keys(kSelScratch)))
+                select_head<kSelScratch>(sc, sc2, a.L, a.w, a.c, la.C, la.k, la.n_max, out, ss, kbuf);
+            else
+                select_head_rows(sc, sc2, a.L, a.w, a.c, la.C, la.k, la.n_max, out, ss,
+                                 fits ? kbuf : reinterpret_cast<uint32_t*>(const_cast<float*>(sc)));
         }
         if (rows_elsewhere) return;
         if (!solo) {

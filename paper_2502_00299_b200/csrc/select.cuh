@@ -7,8 +7,8 @@
 // ties go to the lower chunk id. Token positions are written directly in ascending order: no
 // mask, no sort.
 //
-// select_core (keys in registers or in shared memory): the threshold comes from an adaptive radix select (2048
-// equal sub-intervals of [min key, max key], repeated on the sub-interval that holds the k-th largest
+// select_kept (keys in registers, or in shared memory where there are many a thread): an adaptive radix select
+// (2048 equal sub-intervals of [min key, max key], repeated on the sub-interval that holds the k-th largest
 // until few enough keys remain to rank directly).
 //
 // select_head_rows (keys nowhere or in a buffer of any kind; any number of kept chunks): 8 bits of the key at a time in
@@ -17,9 +17,9 @@
 // adds its totals once; any other bin, and every bin of the later passes, takes one
 // shared-memory atomic per key.
 //
-// In both, each warp owns a contiguous block of chunk ids and walks it in rows of 32 consecutive ids, one
-// per lane: accesses are coalesced and the order inside a row is the lane order; ranks come from warp ballots plus the
-// warps' (#above, #equal) totals.
+// Keys in registers: a thread owns a run of consecutive ids. Otherwise each warp owns a contiguous block of chunk ids and walks
+// it in rows of 32 consecutive ids, one per lane: accesses are coalesced and the order inside a row is the lane order; ranks
+// come from warp ballots plus the warps' (#above, #equal) totals.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -42,6 +42,9 @@ struct SelectSmem {
     int n_cand;
     int need_eq;
     int last_kept;
+    alignas(16) int found[4];               // sub-interval of the k-th largest key, its rank in it, keys in it
+    unsigned long long last;                // last candidate that is kept
+    int kept_cand[kSelMaxWarps];            // kept candidates of a warp's ids
 };
 
 __device__ __forceinline__ uint32_t select_order_key(float x) {
@@ -49,11 +52,9 @@ __device__ __forceinline__ uint32_t select_order_key(float x) {
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);     // larger float <=> larger key
 }
 
-// The one-CTA selection proper: leaves the ids of the kept chunks in ascending order in sm.sel (kk = min(k, C) of
-// them; kk <= kSelCap, C <= kSelMaxChunks) and sm.last_kept. All threads of the CTA must call this (it uses __syncthreads);
-// blockDim.x must be a multiple of 32, at least 512 and at most 1024.
-// KPT > 0: every thread keeps up to KPT keys in registers, which needs C <= blockDim.x * KPT and kbuf is not used.
-// KPT = 0: the keys live in kbuf (shared memory, room for C).
+// The one-CTA selection proper (select_regs, select_core; select_kept takes the one that fits): leaves the ids of the kept
+// chunks in ascending order in sm.sel (kk = min(k, C) of them; kk <= kSelCap, C <= kSelMaxChunks) and sm.last_kept. All threads
+// of the CTA must call this (it uses __syncthreads); blockDim.x must be a multiple of 32, at least 512 and at most 1024.
 // sc2 != NULL: the head's scores are sc[ch] + sc2[ch] (a KV head scored as two heads of half the rows).
 //
 // The k-th largest key is found by an adaptive radix select: the keys of interest always lie in a
@@ -64,17 +65,229 @@ __device__ __forceinline__ uint32_t select_order_key(float x) {
 // ranked against each other directly. Ties and degenerate inputs (all keys equal) end with
 // span = 0, i.e. a single key value. Exact for any input.
 //
-// What bounds it is a chain of latencies - about ten block-wide steps on a few thousand keys - and, inside the steps,
-// instructions that a quarter of the lanes execute at a time (population counts, shared atomics). Keys in registers: a
-// thread owns a run of KPT or fewer consecutive ids - loaded 16 bytes at a time where the scores are aligned and the run is KPT
-// long, else one by one - so that the order inside a warp is one packed prefix sum over its lanes and the list is written without branches. Keys in shared
-// memory: warp v owns a block of consecutive ids and walks it in rows of 32, one id per lane, with ballots for the order.
-// Totals of warps are combined by one shared-memory read per lane and a warp reduction.
-// 3274 keys, 640 threads, in clocks: 11.2k with scalar loads (2.2k), a loop over the warps for the minimum and maximum
-// (1.1k) and branches per key for the candidates (1.2k) and the list (2.1k); 7.2k in this form (a selector CTA of the model kernel; 12.2k there before).
+// What bounds it is a chain of latencies - seven or eight block-wide steps on a few thousand keys - and, inside the steps,
+// the instructions that all warps issue. select_regs: a thread owns a run of KPT consecutive ids, so that a warp without
+// ids leaves out the work on keys, loads are 8 or 16 bytes wide, and the order inside a warp is one packed prefix sum over its
+// lanes. Candidates are ranked by (key, id) at once, so that ties need no counting of their own and the prefix sum over the keys
+// above them runs in the same step as their collection. select_core: registers with runs padded to four ids, or shared memory
+// (warp v owns a block of consecutive ids and walks it in rows of 32, one id per lane, with ballots for the order); the ties are
+// counted in a step more. In clocks, 576 threads, scores from the L2, a cold instruction cache, select_core -> select_regs: 204 keys
+// 5.7k -> 4.0k, 816 5.5k -> 4.5k, 1636 6.0k -> 4.6k, 3274 6.6k -> 6.3k, 6550 15.0k -> 9.0k (runs padded to 16 ids were loaded one by
+// one), 13104 20.2k (in shared memory) -> 14.8k. The layer kernel with it: 2048 tokens, 2 heads 13.0 -> 12.4 us; 65536 tokens,
+// 2 heads 26.5 -> 23.0; 131072 tokens, 8 heads, 128 rows 88 -> 82.
 constexpr int kSelBins = 2048;
 constexpr int kSelCandCap = 128;
 
+// Keys in registers: thread t owns the ids [t KPT, (t + 1) KPT), C <= blockDim.x KPT.
+template <int KPT>
+__device__ __forceinline__ void select_regs(const float* sc, const float* sc2, int C, int k, SelectSmem& sm) {
+    constexpr unsigned kFull = 0xffffffffu;
+    static_assert(KPT <= 32, "a run's flags fit a word");
+    const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
+    const int kk = min(k, C);
+    if (tid == 0) { sm.last_kept = k >= C && kk > 0; sm.n_cand = 0; }
+    if (k >= C || kk <= 0) {
+        for (int ch = tid; ch < kk; ch += nt) sm.sel[ch] = static_cast<unsigned short>(ch);
+        __syncthreads();
+        return;
+    }
+    int* hist = reinterpret_cast<int*>(&sm.whist[0][0]);                            // kSelBins counters
+    unsigned long long* cand = reinterpret_cast<unsigned long long*>(&sm.sel[0]);   // kSelCandCap keys with ids (sel is written later)
+    const int id0 = tid * KPT, own = min(KPT, C - id0);      // this thread's ids; own <= 0: none
+    const bool warp_on = warp * (32 * KPT) < C;              // this thread's warp has ids
+    uint32_t keys[KPT];
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    {
+        float v[KPT];
+        constexpr int W = KPT % 4 == 0 ? 4 : 2;              // floats a load
+        auto load = [&](const float* p, float* o) {
+            if constexpr (W == 4) {
+                const float4 f = __ldcg(reinterpret_cast<const float4*>(p));
+                o[0] = f.x; o[1] = f.y; o[2] = f.z; o[3] = f.w;
+            } else {
+                const float2 f = __ldcg(reinterpret_cast<const float2*>(p));
+                o[0] = f.x; o[1] = f.y;
+            }
+        };
+        const bool vec = ((reinterpret_cast<uintptr_t>(sc) | reinterpret_cast<uintptr_t>(sc2)) & (4u * W - 1u)) == 0;
+        if (own == KPT && vec) {
+#pragma unroll
+            for (int u = 0; u < KPT; u += W) load(sc + id0 + u, &v[u]);
+            if (sc2 != nullptr) {
+                float v2[KPT];
+#pragma unroll
+                for (int u = 0; u < KPT; u += W) load(sc2 + id0 + u, &v2[u]);
+#pragma unroll
+                for (int u = 0; u < KPT; ++u) v[u] += v2[u];
+            }
+        } else if (own > 0) {
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) v[u] = u < own ? __ldcg(sc + id0 + u) : 0.f;
+            if (sc2 != nullptr) {
+#pragma unroll
+                for (int u = 0; u < KPT; ++u) v[u] += u < own ? __ldcg(sc2 + id0 + u) : 0.f;
+            }
+        }
+        for (int i = tid; i < kSelBins / 4; i += nt) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
+        for (int i = tid; i < kSelMaxWarps; i += nt) sm.kept_cand[i] = 0;
+        for (int i = tid; i < kSelCandCap; i += nt) cand[i] = 0ull;
+        if (warp_on) {
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) {
+                const bool in = u < own;
+                keys[u] = in ? select_order_key(v[u]) : 0u;
+                if (in) { lo = min(lo, keys[u]); hi = max(hi, keys[u]); }
+            }
+            lo = __reduce_min_sync(kFull, lo);
+            hi = __reduce_max_sync(kFull, hi);
+        }
+    }
+    if (lane == 0) sm.warp_sums[warp] = (static_cast<unsigned long long>(hi) << 32) | lo;
+    __syncthreads();
+    const unsigned long long mm = sm.warp_sums[lane < nwarps ? lane : 0];
+    uint32_t base = __reduce_min_sync(kFull, static_cast<uint32_t>(mm));
+    uint32_t span = __reduce_max_sync(kFull, static_cast<uint32_t>(mm >> 32)) - base;
+    int need = k, n_bin = 0;        // the need-th largest of the n_bin keys in [base, base + span] is the k-th largest of all
+    for (int round = 0;; ++round) {
+        const int shift = max(0, 21 - __clz(span));          // (span >> shift) < kSelBins
+        if (round > 0) {
+            for (int i = tid; i < kSelBins / 4; i += nt) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
+            __syncthreads();
+        }
+        if (warp_on) {
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) {
+                const uint32_t dlt = keys[u] - base;         // (a key below base wraps to more than span: base + span is a key's value)
+                if (u < own && dlt <= span) atomicAdd(&hist[dlt >> shift], 1);
+            }
+        }
+        __syncthreads();
+        // thread t < 512 owns bins 2047 - 4t .. 2044 - 4t, so a prefix over threads counts from the top
+        int cnt[4] = {0, 0, 0, 0}, sum = 0, inc = 0;
+        if (tid < kSelBins / 4) {
+            const int4 b4 = *reinterpret_cast<const int4*>(hist + kSelBins - 4 - 4 * tid);
+            cnt[0] = b4.w; cnt[1] = b4.z; cnt[2] = b4.y; cnt[3] = b4.x;
+            sum = (cnt[0] + cnt[1]) + (cnt[2] + cnt[3]);
+            inc = sum;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int n = __shfl_up_sync(kFull, inc, off);
+                if (lane >= off) inc += n;
+            }
+            if (lane == 31) sm.warp_tot[warp] = inc;
+        }
+        __syncthreads();
+        if (tid < kSelBins / 4) {
+            inc += __reduce_add_sync(kFull, lane < warp ? sm.warp_tot[lane] : 0);
+            if (inc - sum < need && need <= inc) {           // exactly one thread
+                int ab = inc - sum, q = 0, cq = cnt[0];
+#pragma unroll
+                for (int t = 0; t < 3; ++t)                  // (unrolled: cnt stays in registers)
+                    if (q == t && ab + cnt[t] < need) { ab += cnt[t]; q = t + 1; cq = cnt[t + 1]; }
+                *reinterpret_cast<int4*>(&sm.found) = make_int4(kSelBins - 1 - 4 * tid - q, need - ab, cq, 0);
+            }
+        }
+        __syncthreads();
+        const int4 f = *reinterpret_cast<const int4*>(&sm.found);
+        n_bin = f.z;
+        need = f.y;
+        const uint32_t sub = static_cast<uint32_t>(f.x) << shift;
+        base += sub;
+        span = min((1u << shift) - 1u, span - sub);
+        if (n_bin <= kSelCandCap || span == 0u) break;
+    }
+    // The keys above the interval are kept, and `need` of those in it, the candidates. Few candidates: they are ranked by key and
+    // id. Many equal ones: the first `need` of them in the order of ids.
+    const bool ranked = n_bin <= kSelCandCap;
+    const uint32_t top = base + span;
+    unsigned above = 0, hits = 0;   // this thread's keys above the interval, and in it (bit u: id0 + u)
+    unsigned before = 0;            // (#candidates << 16 | #above) in the warp before this thread
+    if (warp_on) {
+#pragma unroll
+        for (int u = 0; u < KPT; ++u) {
+            above |= keys[u] > top ? 1u << u : 0u;           // (ids past the last one have key 0)
+            hits |= u < own && keys[u] - base <= span ? 1u << u : 0u;
+        }
+        const unsigned mine = __popc(above) | __popc(hits) << 16;
+        unsigned inc = mine;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const unsigned n = __shfl_up_sync(kFull, inc, off);
+            if (lane >= off) inc += n;
+        }
+        if (lane == 31) sm.warp_tot[warp] = static_cast<int>(inc);
+        before = inc - mine;
+        if (ranked && __any_sync(kFull, hits != 0)) {        // (one atomic a warp; the order of the candidates does not matter)
+            int at = 0;
+            if (lane == 31) at = atomicAdd(&sm.n_cand, static_cast<int>(inc >> 16));
+            at = __shfl_sync(kFull, at, 31) + static_cast<int>(before >> 16);
+#pragma unroll
+            for (int u = 0; u < KPT; ++u)
+                if (hits >> u & 1u) cand[at++] = static_cast<unsigned long long>(keys[u]) << 32 | static_cast<uint32_t>(~(id0 + u));
+        }
+    } else if (lane == 31) {
+        sm.warp_tot[warp] = 0;
+    }
+    __syncthreads();
+    if (ranked) {
+        if (tid < n_bin) {
+            const unsigned long long v = cand[tid];          // larger key first, then lower id: all different
+            int gt = 0;
+            const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(cand);
+#pragma unroll 8
+            for (int i = 0; i < (n_bin + 1) / 2; ++i) { const ulonglong2 x = c2[i]; gt += x.x > v; gt += x.y > v; }
+            if (gt < need) {
+                const int id = static_cast<int>(~static_cast<uint32_t>(v));
+                atomicAdd(&sm.kept_cand[id / (32 * KPT)], 1);
+                if (gt == need - 1) sm.last = v;
+            }
+        }
+        __syncthreads();
+    }
+    if (warp_on) {
+        const unsigned tot = lane < warp ? static_cast<unsigned>(sm.warp_tot[lane]) : 0u;
+        unsigned kept = above;
+        int rank;
+        if (ranked) {
+            const unsigned ex = __reduce_add_sync(kFull, (tot & 0xffffu) + (lane < warp ? static_cast<unsigned>(sm.kept_cand[lane]) : 0u));
+            rank = static_cast<int>(ex + (before & 0xffffu));
+            if (__any_sync(kFull, hits != 0)) {
+                const unsigned long long last = sm.last;
+                unsigned kh = 0;
+                if (hits != 0) {
+#pragma unroll
+                    for (int u = 0; u < KPT; ++u)
+                        if (hits >> u & 1u) kh |= (static_cast<unsigned long long>(keys[u]) << 32 | static_cast<uint32_t>(~(id0 + u))) >= last ? 1u << u : 0u;
+                }
+                const int mh = __popc(kh);
+                int ih = mh;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int n = __shfl_up_sync(kFull, ih, off);
+                    if (lane >= off) ih += n;
+                }
+                rank += ih - mh;
+                kept |= kh;
+            }
+        } else {
+            const unsigned ex = __reduce_add_sync(kFull, tot) + before;
+            const int eq_before = static_cast<int>(ex >> 16);
+            rank = static_cast<int>(ex & 0xffffu) + min(eq_before, need);
+            int room = max(0, need - eq_before);
+#pragma unroll
+            for (int u = 0; u < KPT; ++u)
+                if (hits >> u & 1u) { kept |= room > 0 ? 1u << u : 0u; --room; }
+        }
+#pragma unroll
+        for (int u = 0; u < KPT; ++u)
+            if (kept >> u & 1u) sm.sel[rank + __popc(kept & ((1u << u) - 1u))] = static_cast<unsigned short>(id0 + u);
+        if (own > 0 && id0 + own == C && (kept >> (own - 1) & 1u)) sm.last_kept = 1;
+    }
+    __syncthreads();
+}
+
+// KPT > 0: up to KPT keys a thread in registers, in runs padded to four ids (C <= blockDim.x KPT; kbuf is not used). KPT = 0: the keys
+// live in kbuf (shared memory, room for C).
 template <int KPT>
 __device__ __forceinline__ void select_core(const float* sc, const float* sc2, int C, int k, SelectSmem& sm, uint32_t* kbuf) {
     constexpr unsigned kFull = 0xffffffffu;
@@ -301,6 +514,34 @@ __device__ __forceinline__ void select_core(const float* sc, const float* sc2, i
     __syncthreads();
 }
 
+// The selection, by the number of keys a thread has to take; kbuf: room for C keys in shared memory, used beyond
+// select_reg_keys() keys a thread. The layer kernel and select.cu take select_regs throughout. The other kernels have no registers
+// to spare beside their own: with select_regs for 6 keys or more the model kernel spills and a call with 5994 chunks is 8 %
+// slower, so it takes that form up to 4 keys a thread (32 layers of 4096 tokens 348 -> 311 us, 16 layers of 20000 tokens in chunks
+// of 16 228 -> 206); the kernels of score.cu spill with any of it.
+// (All inlined: as a function its register convention made the kernels' scoring loops spill, 2 to 10 % of a model call.)
+enum SelectIn { kSelScratch, kSelModel, kSelLayer };      // the kernels of score.cu, the model kernel, the layer kernel or select.cu
+__host__ __device__ constexpr int select_reg_keys(SelectIn where) { return where == kSelLayer ? 24 : (where == kSelModel ? 16 : 8); }
+template <SelectIn WHERE>
+__device__ __forceinline__ void select_kept(const float* sc, const float* sc2, int C, int k, SelectSmem& sm, uint32_t* kbuf) {
+    const int per = (C + static_cast<int>(blockDim.x) - 1) / static_cast<int>(blockDim.x);
+    if (per > select_reg_keys(WHERE)) return select_core<0>(sc, sc2, C, k, sm, kbuf);
+    if constexpr (WHERE != kSelScratch) {
+        // the shortest run that covers the ids: the longer ones leave more warps without any, and a step's time goes with the
+        // keys of the busiest scheduler (816 keys: runs of 2 4.5k clocks, of 4 5.2k; 1636 keys: of 4 4.6k, of 8 5.7k)
+        if (per <= 2) return select_regs<2>(sc, sc2, C, k, sm);
+        if (per <= 4) return select_regs<4>(sc, sc2, C, k, sm);
+    }
+    if constexpr (WHERE == kSelLayer) {
+        if (per <= 8) return select_regs<8>(sc, sc2, C, k, sm);
+        if (per <= 16) return select_regs<16>(sc, sc2, C, k, sm);
+        select_regs<24>(sc, sc2, C, k, sm);
+    } else {
+        if (WHERE == kSelScratch || per <= 8) return select_core<8>(sc, sc2, C, k, sm, nullptr);
+        if constexpr (WHERE == kSelModel) select_core<16>(sc, sc2, C, k, sm, nullptr);
+    }
+}
+
 // Tokens of the kept chunks that are emitted: every kept chunk is full except possibly chunk C - 1, which can only be
 // the last kept one. tok_cap: at most this many, lowest positions first (Algorithm 1 keeps the first L_max - w
 // selected tokens); no cap by default.
@@ -316,11 +557,11 @@ __device__ __forceinline__ int select_position(const SelectSmem& sm, int n, int 
     return n < n_tok + w ? P + (n - n_tok) : -1;
 }
 
-// The whole selection of a head into out[n_max], keys in registers (KPT > 0) or in kbuf; conditions as select_core.
-template <int KPT>
+// The whole selection of a head into out[n_max]; conditions as select_kept.
+template <SelectIn WHERE>
 __device__ __forceinline__ void select_head(const float* sc, const float* sc2, int L, int w, int c, int C, int k, int n_max,
                                             int32_t* out, SelectSmem& sm, uint32_t* kbuf, int tok_cap = 0x7fffffff) {
-    select_core<KPT>(sc, sc2, C, k, sm, kbuf);
+    select_kept<WHERE>(sc, sc2, C, k, sm, kbuf);
     const int P = L - w, n_tok = select_tokens(P, c, C, k, sm, tok_cap);
     for (int n = threadIdx.x; n < n_max; n += blockDim.x) out[n] = select_position(sm, n, n_tok, c, P, w);
     __syncthreads();     // shared state may be reused by the caller

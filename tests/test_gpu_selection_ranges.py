@@ -97,3 +97,32 @@ def test_select_with_all_scores_equal_and_with_two_values(ck, C, k):
         want = ora.select_chunks(x[h].double().cpu().numpy(), k)
         assert np.array_equal(idx[h][:k * c], (want[:, None] * c + np.arange(c)).ravel())
         assert idx[h][k * c:].tolist() == list(range(L - w, L))
+
+
+# Chunk counts at the ends of the runs of ids that a thread holds (2, 4, 8, 16, 24): 576 threads in the layer kernel, 512 in chunkkv_select
+@pytest.mark.parametrize("C,k", [(1, 1), (31, 30), (575, 1), (1152, 100), (1153, 1152), (2304, 700), (2305, 300), (4608, 4000),
+                                 (4609, 900), (9216, 1), (9217, 800), (13824, 600), (13825, 700)])
+def test_layer_selection_at_the_ends_of_runs(ck, C, k):
+    w, c, d = 16, 5, 64
+    L = C * c + w - (3 if C > 1 else 0)                 # (a clipped last chunk)
+    q, K, V = _random(4, 1, d, L, w, seed=C)
+    s = ora.chunk_scores(ora.token_scores(q, K, 4, 1, w), c)
+    oK, oV, idx = ck.compress_layer(*map(to_dev, (q, K, V)), 4, w, c, w + c * k)
+    assert ck.device_status() == 0
+    assert_selection_matches(idx.cpu().numpy(), s, L, w, c, w + c * k)
+    assert_gather_exact(bits_of(oK), bits_of(oV), idx.cpu().numpy(), K, V)
+
+
+@pytest.mark.parametrize("C", [2, 33, 511, 1024, 1025, 2048, 2049, 4095, 4096])
+def test_select_at_the_ends_of_runs(ck, C):
+    L, w, c = 2 * C + 3, 3, 2
+    g = torch.Generator(device="cuda").manual_seed(C)
+    x = torch.randn(4, C, device="cuda", generator=g)                                  # head 0: all different
+    x[1] = torch.randint(0, 3, (C,), device="cuda", generator=g).float()               # many ties
+    x[2] = torch.where(torch.rand(C, device="cuda", generator=g) < 0.9, -float("inf"), x[0])
+    x[3] = torch.where(torch.rand(C, device="cuda", generator=g) < 0.1, 1e30 * x[0], 1e-30 * x[0])
+    for k in sorted({1, C // 3 + 1, C - 1, C}):
+        idx = ck.select(x, L, w, c, w + c * k).cpu().numpy()
+        for h in range(4):
+            want = ora.select_chunks(x[h].double().cpu().numpy(), k)
+            assert np.array_equal(idx[h][:k * c], (want[:, None] * c + np.arange(c)).ravel())
