@@ -384,6 +384,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
             const uint32_t qbar = smem_u32(&ctl.qfull);
             const uint32_t q_bytes = static_cast<uint32_t>(n_mt * KB * p.q_box_rows) * 128u;
             const uint32_t k_bytes = static_cast<uint32_t>(p.k_box_rows) * 128u;
+            const uint64_t first = l2_policy_evict_first();
             uint32_t st = 0, st_par = 1;
             int issued = 0;
             bool ok = true;
@@ -403,7 +404,9 @@ model_kernel(const __grid_constant__ ModelParams p) {
                         if (!ok) break;
                         const uint32_t bar = smem_u32(&ctl.full[st]);
                         mbar_arrive_expect_tx(bar, k_bytes);
-                        tma_load_3d(k_base + st * STAGE, &p.tm_k[s], bar, kb * 64, t * TILE, hkv);
+                        // (big variant: the keys leave the L2 to the ring in scratch; 16 layers of 30000 tokens, c = 5, 403 -> 381 us)
+                        if constexpr (BIG) tma_load_3d_hint(k_base + st * STAGE, &p.tm_k[s], bar, kb * 64, t * TILE, hkv, first);
+                        else tma_load_3d(k_base + st * STAGE, &p.tm_k[s], bar, kb * 64, t * TILE, hkv);
                         ++issued;
                         if (++st == n_stages) { st = 0; st_par ^= 1u; }
                     }
