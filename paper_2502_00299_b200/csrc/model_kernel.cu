@@ -939,8 +939,12 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_
     p.tile = 2 * panel_keys(c);
     p.spp = panel_keys(c) / c;
     p.n_tiles = (L + p.tile - 1) / p.tile;
-    // a few CTAs do nothing but select (they take the SMs the scoring grid would leave idle anyway)
+    // a few CTAs do nothing but select (four take the SMs the scoring grid would leave idle anyway)
     p.n_sel = Hkv < 4 ? Hkv : 4;
+    // Five to eight heads on short contexts: a selector each. With two heads a selector the two selections (about 5k clocks each)
+    // are longer than the scoring of a layer up to six tiles a CTA, and the scoring CTA a head gives up costs less: 32 layers of
+    // 4096 tokens 309 -> 287 us, 16 of 7000 (256 rows) 192 -> 183, 16 of 2100 157 -> 145, 16 of 11000 (indices shared by two) 121 -> 114.
+    if (Hkv > 4 && Hkv <= 8 && max_ctas >= 2 * Hkv && p.n_tiles <= 6 * ((max_ctas - Hkv) / Hkv)) p.n_sel = Hkv;
     if (max_ctas - p.n_sel < Hkv) p.n_sel = max_ctas - Hkv;
     p.cph = (max_ctas - p.n_sel) / Hkv;
     if (p.cph > p.n_tiles) p.cph = p.n_tiles;
