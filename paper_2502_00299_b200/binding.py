@@ -1,4 +1,7 @@
-"""ctypes binding of the C ABI declared in include/chunkkv.h (argument marshalling only)."""
+"""Binding of the C ABI declared in include/chunkkv.h (argument marshalling only).
+
+Calls that a program makes per layer or per model go through ``_native`` (csrc/native.cpp), which answers None for arguments
+other than plain tensors and ints and for whatever fails a check; those, and all other calls, go through ctypes here."""
 from __future__ import annotations
 
 import ctypes
@@ -109,10 +112,19 @@ def _load() -> ctypes.CDLL:
 
 lib = _load()
 
+from . import _native  # noqa: E402  (linked against the library loaded above)
+
 
 def _check(status: int, where: str) -> None:
     if status != 0:
         raise ChunkKVError(status, where)
+
+
+def _done(r, where: str):
+    """The result of a ``_native`` call that was taken: an int is the status of the C ABI."""
+    if type(r) is int:
+        raise ChunkKVError(r, where)
+    return r
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -166,10 +178,12 @@ def set_workspace(buf: Optional[torch.Tensor]) -> None:
     if buf is None:
         _check(lib.chunkkv_set_workspace(None, 0), "chunkkv_set_workspace")
         _workspaces.pop(dev, None)
+        _native.note_workspace(dev, 0)
     else:
         _check(lib.chunkkv_set_workspace(buf.data_ptr(), buf.numel() * buf.element_size()),
                "chunkkv_set_workspace")
         _workspaces[dev] = buf
+        _native.note_workspace(dev, buf.numel())
 
 
 def ensure_workspace(L: int, Hq: int, Hkv: int, d: int, w: int, c: int) -> None:
@@ -194,6 +208,9 @@ def device_status(stream: Optional[torch.cuda.Stream] = None) -> int:
 def score(q_obs: torch.Tensor, K: torch.Tensor, w: int, c: int, want_token_scores: bool = False,
           stream: Optional[torch.cuda.Stream] = None) -> Tuple[torch.Tensor, Optional[torch.Tensor]]:
     """chunk scores [Hkv, C] f32 (and token scores [Hkv, P] f32 if asked)."""
+    r = _native.score(q_obs, K, w, c, want_token_scores, stream)
+    if r is not None:
+        return _done(r, "chunkkv_score")
     _dev(q_obs, torch.bfloat16, "q_obs"); _dev(K, torch.bfloat16, "K")
     Hq, d = q_obs.shape[0], q_obs.shape[2]
     Hkv, L = K.shape[0], K.shape[1]
@@ -248,6 +265,9 @@ def compress_layer_alg1(q_obs: torch.Tensor, K: torch.Tensor, V: torch.Tensor, H
                         out_idx: Optional[torch.Tensor] = None,
                         stream: Optional[torch.cuda.Stream] = None) -> Tuple[torch.Tensor, torch.Tensor, torch.Tensor]:
     """out_K, out_V [Hkv, n_max, d], idx [Hkv, n_max] for one layer under Algorithm 1's budget rule."""
+    r = _native.layer_alg1(q_obs, K, V, Hq, w, c, budget, out_K, out_V, out_idx, stream)
+    if r is not None:
+        return _done(r, "chunkkv_compress_layer_alg1")
     _dev(q_obs, torch.bfloat16, "q_obs"); _dev(K, torch.bfloat16, "K"); _dev(V, torch.bfloat16, "V")
     Hkv, L, d = K.shape
     n_max = out_len_alg1(L, w, c, budget)
@@ -286,6 +306,9 @@ def compress_layer(q_obs: Optional[torch.Tensor], K: torch.Tensor, V: torch.Tens
                    stream: Optional[torch.cuda.Stream] = None,
                    ) -> Tuple[torch.Tensor, torch.Tensor, torch.Tensor]:
     """One layer: score -> chunk-sum -> top-k -> gather, or gather only with ``reuse_idx``."""
+    r = _native.layer(q_obs, K, V, Hq, w, c, budget, reuse_idx, out_K, out_V, out_idx, stream)
+    if r is not None:
+        return _done(r, "chunkkv_compress_layer")
     _dev(K, torch.bfloat16, "K"); _dev(V, torch.bfloat16, "V")
     if q_obs is not None:
         _dev(q_obs, torch.bfloat16, "q_obs")
@@ -312,6 +335,9 @@ def window_queries(qkv: torch.Tensor, Hq: int, Hkv: int, d: int, w: int, cos_row
                    sin_rows: torch.Tensor, stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
     """q_obs [Hq, w, d] bf16 from the last w rows of a fused QKV activation [T, row_elems] bf16,
     with the rotary embedding of those rows applied (cos_rows, sin_rows [w, d / 2] f32)."""
+    r = _native.window_queries(qkv, Hq, Hkv, d, w, cos_rows, sin_rows, stream)
+    if r is not None:
+        return _done(r, "chunkkv_window_queries")
     _dev(qkv, torch.bfloat16, "qkv"); _dev(cos_rows, torch.float32, "cos_rows"); _dev(sin_rows, torch.float32, "sin_rows")
     T, row_elems = qkv.shape
     out = torch.empty((Hq, w, d), dtype=torch.bfloat16, device=qkv.device)
@@ -339,6 +365,9 @@ def compress_layer_strided(q_obs: Optional[torch.Tensor], K: torch.Tensor, V: to
     """One layer on K / V given as [Hkv, L, d] *views* with arbitrary token and head strides (the last
     dimension contiguous), e.g. ``cache.permute(1, 0, 2)`` of a token-major cache [L, Hkv, d]. Outputs
     are packed [Hkv, n_max, d]."""
+    r = _native.layer_strided(q_obs, K, V, Hq, w, c, budget, reuse_idx, out_K, out_V, out_idx, stream)
+    if r is not None:
+        return _done(r, "chunkkv_compress_layer_strided")
     for t, name in ((K, "K"), (V, "V")):
         if not (t.is_cuda and t.dtype == torch.bfloat16 and t.dim() == 3 and t.stride(2) == 1):
             raise ValueError(f"{name}: a CUDA bf16 [Hkv, L, d] view with a contiguous last dimension is required")
@@ -369,6 +398,9 @@ def compress_layer_paged(q_obs: Optional[torch.Tensor], K: torch.Tensor, V: torc
                          reuse_idx: Optional[torch.Tensor] = None, out_idx: Optional[torch.Tensor] = None,
                          stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
     """One layer into a paged cache; returns idx [Hkv, n_max]."""
+    r = _native.layer_paged(q_obs, K, V, Hq, w, c, budget, block_table, cache_K, cache_V, reuse_idx, out_idx, stream)
+    if r is not None:
+        return _done(r, "chunkkv_compress_layer_paged")
     Hkv, L, d = K.shape
     n_max = out_len(L, w, c, budget)
     if reuse_idx is None:
@@ -533,6 +565,9 @@ def compress_model(layers: Sequence[Tuple[Optional[torch.Tensor], torch.Tensor, 
     chunkkv_compress_model call; with one chunk size per layer (chunk-level layers followed by
     token-level ones, c = 1) it is the same call sequence over chunkkv_compress_layer, a layer that
     reuses indices taking its source layer's chunk size. Only marshalling lives here."""
+    r = _native.model(layers, Hq, w, c, budget, n_reuse, stream, outs, False)
+    if r is not None:
+        return _done(r, "chunkkv_compress_model")
     n = len(layers)
     if not isinstance(c, int):
         cs = [int(v) for v in c]
@@ -581,6 +616,9 @@ def compress_model_strided(layers: Sequence[Tuple[Optional[torch.Tensor], torch.
                            ) -> List[Tuple[torch.Tensor, torch.Tensor, torch.Tensor]]:
     """compress_model on K / V given as [Hkv, L, d] views that share one set of token and head strides
     (last dimension contiguous), e.g. ``cache.permute(1, 0, 2)`` of token-major caches [L, Hkv, d]."""
+    r = _native.model(layers, Hq, w, c, budget, n_reuse, stream, outs, True)
+    if r is not None:
+        return _done(r, "chunkkv_compress_model_strided")
     n = len(layers)
     K0, V0 = layers[0][1], layers[0][2]
     Hkv, L, d = K0.shape

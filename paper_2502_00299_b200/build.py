@@ -1,4 +1,4 @@
-"""Build libchunkkv.so (CUDA, sm_100a) in-tree with nvcc.
+"""Build libchunkkv.so (CUDA, sm_100a) with nvcc and the binding's native part with g++, in-tree.
 
 Usage: ``python -m paper_2502_00299_b200.build [--force]``. Objects go to ``_build/`` inside the
 package; the shared library is written next to this file so that it ships with the package.
@@ -10,11 +10,13 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 BUILD_DIR = os.path.join(PKG_DIR, "_build")
 LIB_PATH = os.path.join(PKG_DIR, "libchunkkv.so")
+NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")      # extension module used by binding.py
 INCLUDE_DIR = os.path.join(os.path.dirname(PKG_DIR), "include")
 SOURCES = ("api.cu", "score.cu", "layer_resident.cu", "model_kernel.cu", "token_kernel.cu", "select.cu", "select_cluster.cu", "gather.cu", "diagnostics.cu", "score_noalloc.cu")
 NVCC_FLAGS = [
@@ -37,7 +39,32 @@ def _deps_mtime() -> float:
 
 
 def is_current() -> bool:
-    return os.path.exists(LIB_PATH) and os.path.getmtime(LIB_PATH) >= _deps_mtime()
+    return all(os.path.exists(p) and os.path.getmtime(p) >= _deps_mtime() for p in (LIB_PATH, NATIVE_PATH))
+
+
+def _compile_native() -> str:
+    import torch
+    root = os.path.dirname(os.path.abspath(torch.__file__))
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    obj = os.path.join(BUILD_DIR, "native.o")
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(root, "include"),
+           "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"), "-isystem", os.path.join(cuda, "include"),
+           "-c", os.path.join(CSRC, "native.cpp"), "-o", obj]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"g++ failed on native.cpp:\n{res.stdout}\n{res.stderr}")
+    return obj
+
+
+def _link_native(obj: str) -> None:
+    import torch
+    lib = os.path.join(os.path.dirname(os.path.abspath(torch.__file__)), "lib")
+    cmd = ["g++", "-shared", "-o", NATIVE_PATH, obj, "-L", PKG_DIR, "-l:libchunkkv.so", "-Wl,-rpath,$ORIGIN", "-L", lib, "-ltorch_python", "-ltorch",
+           "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"link of _native.so failed:\n{res.stdout}\n{res.stderr}")
 
 
 def _compile(src: str, verbose: bool) -> str:
@@ -55,16 +82,18 @@ def _compile(src: str, verbose: bool) -> str:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every kernel for sm_100a and link the shared library. Returns its path."""
+    """Compile every kernel for sm_100a and link the shared library and the extension module. Returns the library's path."""
     if not force and not verbose and is_current():
         return LIB_PATH
     os.makedirs(BUILD_DIR, exist_ok=True)
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as pool:
+    with cf.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as pool:
+        native = pool.submit(_compile_native)
         objs = list(pool.map(lambda s: _compile(s, verbose), SOURCES))
     cmd = [_nvcc(), "-Wno-deprecated-gpu-targets", "-shared", "-o", LIB_PATH, *objs, "-lcudart"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError(f"link failed:\n{res.stdout}\n{res.stderr}")
+    _link_native(native.result())
     return LIB_PATH
 
 

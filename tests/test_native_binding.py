@@ -1,0 +1,102 @@
+"""The binding's native calls (csrc/native.cpp): what they decline goes the general way, and both ways give the same results."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2502_00299_b200 as ck
+from paper_2502_00299_b200 import binding
+
+CALLS = ("layer", "layer_strided", "layer_alg1", "layer_paged", "window_queries", "score", "model")
+
+
+def test_declined_arguments_raise_what_the_general_way_raises():
+    x = torch.zeros(2, 64, 64, dtype=torch.bfloat16)               # not on a GPU
+    for call in (lambda: ck.compress_layer(x, x, x, 4, 16, 8, 32), lambda: ck.compress_layer_strided(x, x, x, 4, 16, 8, 32),
+                 lambda: ck.compress_layer_alg1(x, x, x, 4, 16, 8, 32), lambda: ck.score(x, x, 16, 8),
+                 lambda: ck.compress_model([(x, x, x)], 4, 16, 8, 32), lambda: ck.compress_model_strided([(x, x, x)], 4, 16, 8, 32),
+                 lambda: ck.window_queries(x[0], 1, 1, 64, 16, x[0], x[0])):
+        with pytest.raises(ValueError):
+            call()
+    with pytest.raises(AttributeError):
+        ck.compress_layer(None, None, None, 4, 16, 8, 32)
+    for name in CALLS:
+        with pytest.raises(TypeError):
+            getattr(binding._native, name)(1, 2, 3)
+
+
+def _general(monkeypatch):
+    for name in CALLS:
+        monkeypatch.setattr(binding._native, name, lambda *a: None)
+
+
+def _cases(g):
+    Hq, Hkv, d, L, w, c, budget = 8, 2, 64, 1111, 16, 10, 200
+    bf = torch.bfloat16
+    q, K, V = (torch.randn(*s, device="cuda", generator=g).to(bf) for s in ((Hq, w, d), (Hkv, L, d), (Hkv, L, d)))
+    n = ck.out_len(L, w, c, budget)
+    tm = [t.permute(1, 0, 2).contiguous().permute(1, 0, 2) for t in (K, V)]
+    idx = torch.stack([torch.randperm(L, device="cuda", generator=g)[:n].sort().values for _ in range(Hkv)]).to(torch.int32)
+    outs = lambda: (torch.zeros(Hkv, n, d, dtype=bf, device="cuda"), torch.zeros(Hkv, n, d, dtype=bf, device="cuda"),
+                    torch.zeros(Hkv, n, dtype=torch.int32, device="cuda"))
+    kw = lambda o: dict(out_K=o[0], out_V=o[1], out_idx=o[2])
+    table = torch.randperm(20, device="cuda", generator=g)[:-(-n // 16)].to(torch.int32)
+    qkv = torch.randn(300, (Hq + 2 * Hkv) * d, device="cuda", generator=g).to(bf)
+    ang = torch.rand(w, d // 2, device="cuda", generator=g)
+    side = torch.cuda.Stream()
+
+    def paged(**more):
+        cache = [torch.zeros(20, 16, Hkv, d, dtype=bf, device="cuda") for _ in range(2)]
+        return [ck.compress_layer_paged(q, K, V, Hq, w, c, budget, table, *cache, **more), *cache]
+
+    def on_side():
+        side.wait_stream(torch.cuda.current_stream())
+        r = ck.compress_layer(q, K, V, Hq, w, c, budget, stream=side, **kw(outs()))
+        torch.cuda.current_stream().wait_stream(side)
+        return r
+    layers = [(q, K, V), (None, V, K), (q, V, K)]
+    strided = [(q, tm[0], tm[1]), (None, tm[1], tm[0])]
+    return [lambda: ck.compress_layer(q, K, V, Hq, w, c, budget), lambda: ck.compress_layer(q, K, V, Hq, w, c, budget, **kw(outs())),
+            lambda: ck.compress_layer(None, K, V, Hq, w, c, budget, reuse_idx=idx), lambda: ck.compress_layer(q, K, V, Hq, w, 1, budget),
+            lambda: ck.compress_layer(q, K, V, np.int64(Hq), w, c, np.int32(budget)), on_side,
+            lambda: ck.compress_layer_strided(q, *tm, Hq, w, c, budget), lambda: ck.compress_layer_strided(None, *tm, Hq, w, c, budget, reuse_idx=idx),
+            lambda: ck.compress_layer_alg1(q, K, V, Hq, w, c, budget), lambda: paged(), lambda: paged(reuse_idx=idx),
+            lambda: [ck.window_queries(qkv, Hq, Hkv, d, w, ang.cos(), ang.sin())], lambda: ck.score(q, K, w, c)[:1],
+            lambda: ck.score(q, K, w, c, want_token_scores=True),
+            lambda: sum(ck.compress_model(layers, Hq, w, c, budget, 2), ()),
+            lambda: sum(ck.compress_model(layers, Hq, w, c, budget, 2, outs=[outs() for _ in layers]), ()),
+            lambda: sum(ck.compress_model(tuple(layers), Hq, w, c, budget, 2, outs=tuple(list(outs()) for _ in layers)), ()),
+            lambda: sum(ck.compress_model_strided(strided, Hq, w, c, budget, 2), ())]
+
+
+@pytest.mark.gpu
+def test_native_and_general_results_are_the_same(monkeypatch):
+    cases = _cases(torch.Generator(device="cuda").manual_seed(5))
+    native = [call() for call in cases]
+    _general(monkeypatch)
+    for i, (got, call) in enumerate(zip(native, cases)):
+        want = call()
+        assert len(got) == len(want), i
+        for x, y in zip(got, want):
+            assert x.shape == y.shape and x.dtype == y.dtype and x.device == y.device and torch.equal(x, y), i
+    assert ck.device_status() == 0
+
+
+@pytest.mark.gpu
+def test_native_errors_and_growing_scratch():
+    g = torch.Generator(device="cuda").manual_seed(6)
+    q, K, V = (torch.randn(*s, device="cuda", generator=g).to(torch.bfloat16) for s in ((8, 16, 64), (2, 900, 64), (2, 900, 64)))
+    for bad in (dict(budget=4), dict(c=0), dict(w=901)):             # sizes
+        with pytest.raises(ck.ChunkKVError) as e:
+            ck.compress_layer(q, K, V, 8, **{**dict(w=16, c=10, budget=100), **bad})
+        assert e.value.status == -2
+    with pytest.raises(ck.ChunkKVError) as e:                        # a status of the C ABI
+        ck.compress_layer(None, K, V, 8, 16, 10, 100)
+    assert e.value.status == -1 and "chunkkv_compress_layer" in str(e.value)
+    with pytest.raises(ValueError):
+        ck.compress_layer(q, K.transpose(0, 1), V, 8, 16, 10, 100)
+    ck.set_workspace(torch.empty(8192, dtype=torch.uint8, device="cuda"))
+    want = ck.compress_layer(q, K, V, 8, 16, 10, 100)                # too small: replaced by a larger one
+    assert binding._workspaces[torch.cuda.current_device()].numel() > 8192
+    for x, y in zip(ck.compress_layer(q, K, V, 8, 16, 10, 100), want):
+        assert torch.equal(x, y)
+    assert ck.device_status() == 0
