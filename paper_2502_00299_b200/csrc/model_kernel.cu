@@ -37,6 +37,7 @@
 #include "select.cuh"
 
 #include <math_constants.h>
+#include <type_traits>
 
 namespace chunkkv {
 
@@ -765,18 +766,34 @@ model_kernel(const __grid_constant__ ModelParams p) {
             if (!wait_counter_warp(p.cnt_a + hkv, static_cast<unsigned>(s + 1) * p.cph, abort_flag)) break;
             if constexpr (!BIG) {
                 // the head's records straight from the L2 (they were written by other SMs; every lane has
-                // acquired the counter), nine CTAs' worth of loads in flight per lane
+                // acquired the counter), nine CTAs' worth of loads in flight per lane. Up to 64 rows each half of the warp
+                // takes every other record (2 heads: 69 CTAs, 32 layers of 8192 tokens 487 -> 335 us).
                 const float* src = p.cta_stat + (static_cast<size_t>(s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * 256;
                 float M[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}, S[4] = {0.f, 0.f, 0.f, 0.f};
-                for (int j0 = 0; j0 < p.cph; j0 += 9) {
-                    float4 m[9], l[9];
+                auto fold = [&](const float* from, auto stride, int n) {
+                    constexpr int kStride = decltype(stride)::value;
+                    for (int j0 = 0; j0 < n; j0 += 9) {
+                        float4 m[9], l[9];
 #pragma unroll
-                    for (int j = 0; j < 9; ++j) {
-                        const int jj = min(j0 + j, p.cph - 1);
-                        m[j] = __ldcg(reinterpret_cast<const float4*>(src + static_cast<size_t>(jj) * 256 + r0));
-                        l[j] = __ldcg(reinterpret_cast<const float4*>(src + static_cast<size_t>(jj) * 256 + 128 + r0));
+                        for (int j = 0; j < 9; ++j) {
+                            const int jj = min(j0 + j, n - 1);
+                            m[j] = __ldcg(reinterpret_cast<const float4*>(from + static_cast<size_t>(jj) * kStride));
+                            l[j] = __ldcg(reinterpret_cast<const float4*>(from + static_cast<size_t>(jj) * kStride + 128));
+                        }
+                        merge_batch<9>(M, S, m, l, n - j0);
                     }
-                    merge_batch<9>(M, S, m, l, p.cph - j0);
+                };
+                if (p.R > 64) {
+                    fold(src + r0, std::integral_constant<int, 256>{}, p.cph);
+                } else {
+                    const int sub = lane >> 4;
+                    fold(src + sub * 256 + (r0 & 63), std::integral_constant<int, 512>{}, (p.cph - sub + 1) >> 1);
+                    __syncwarp();
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const float mo = __shfl_xor_sync(0xffffffffu, M[r], 16), so = __shfl_xor_sync(0xffffffffu, S[r], 16);
+                        merge_ml(M[r], S[r], mo, so);
+                    }
                 }
                 float* gm = gstat + (s & 1) * 256;
                 *reinterpret_cast<float4*>(gm + r0) = make_float4(M[0], M[1], M[2], M[3]);
