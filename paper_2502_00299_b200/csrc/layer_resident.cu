@@ -134,7 +134,10 @@ __device__ __forceinline__ bool head_handover(unsigned* counter, unsigned target
 
 // BIG: two query tiles, or panels in scratch. A variant of its own: the code for either, present but not taken, costs
 // the other shapes 1.5 us of 34 (32K tokens, 128 rows).
-template <int C_STATIC, bool BIG>
+// FEW: up to 64 rows and more than kRManyCtas CTAs a head, for the reading of row statistics; a variant of its own for the same reason
+// (as a run-time choice it costs every other shape 0.1 us of 12 to 30).
+constexpr int kRManyCtas = 20;
+template <int C_STATIC, bool BIG, bool FEW>
 __global__ void __launch_bounds__(kRThreads, 1)
 layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                       const ResArgs a) {
@@ -370,50 +373,81 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 
     // ---- 3. row statistics of the head, then this CTA's chunk scores
     if (ok) {
-        // 512 threads: four (one query tile) or two (two tiles) slices of the records per row
-        const int n_sl = two ? 2 : 4;
-        if (threadIdx.x < 512) {
-            const int i = threadIdx.x & 127, sl = (threadIdx.x >> 7) & (n_sl - 1), mt = two ? threadIdx.x >> 8 : 0;
-            const size_t step = static_cast<size_t>(n_mt) * 256;
-            const float* src = a.cta_stat + (static_cast<size_t>(hs) * a.cph * n_mt + mt) * 256 + i;
+        // Up to 64 rows and more CTAs a head than four slices of records read in one round trip (2 heads: 74): eight slices
+        // of 64 rows, two round trips to the L2 instead of four (8192 tokens 14.3 -> 13.5 us, 65536 tokens 23.3 -> 22.3).
+        if constexpr (FEW) {
             float M = -CUDART_INF_F, Ls = 0.f;
-            // records in flight per thread: enough for one round trip where a head has 18 CTAs (8 heads)
-            constexpr int kF = BIG ? 9 : 5;
-            for (int j0 = sl; j0 < a.cph; j0 += kF * n_sl) {
-                float rm[kF], rl[kF];
+            if (threadIdx.x < 512) {
+                const float* src = a.cta_stat + static_cast<size_t>(hs) * a.cph * 256 + (threadIdx.x & 63);
+#pragma unroll 1
+                for (int j0 = threadIdx.x >> 6; j0 < a.cph; j0 += 40) {
+                    float rm[5], rl[5];
 #pragma unroll
-                for (int u = 0; u < kF; ++u) {
-                    const int j = j0 + n_sl * u;
-                    rm[u] = (j < a.cph) ? __ldcg(src + j * step) : -CUDART_INF_F;
-                    rl[u] = (j < a.cph) ? __ldcg(src + j * step + 128) : 0.f;
+                    for (int u = 0; u < 5; ++u) {
+                        const int j = j0 + 8 * u;
+                        rm[u] = (j < a.cph) ? __ldcg(src + j * 256) : -CUDART_INF_F;
+                        rl[u] = (j < a.cph) ? __ldcg(src + j * 256 + 128) : 0.f;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 5; ++u) merge_ml(M, Ls, rm[u], rl[u]);
                 }
-                float bm = M;
-#pragma unroll
-                for (int u = 0; u < kF; ++u) bm = fmaxf(bm, rm[u]);
-                float acc = (M == -CUDART_INF_F) ? 0.f : Ls * ex2_approx(M - bm);
-#pragma unroll
-                for (int u = 0; u < kF; ++u) acc += (rm[u] == -CUDART_INF_F) ? 0.f : rl[u] * ex2_approx(rm[u] - bm);
-                M = bm;
-                Ls = acc;
+                slice[threadIdx.x] = M;
+                slice[512 + threadIdx.x] = Ls;
             }
-            slice[((threadIdx.x >> 7) * 2 + 0) * 128 + i] = M;
-            slice[((threadIdx.x >> 7) * 2 + 1) * 128 + i] = Ls;
+            __syncthreads();
+            if (threadIdx.x < 64) {
+#pragma unroll
+                for (int s = 1; s < 8; ++s) merge_ml(M, Ls, slice[s * 64 + threadIdx.x], slice[512 + s * 64 + threadIdx.x]);
+                gm[threadIdx.x] = M;
+                ginv[threadIdx.x] = 1.0f / Ls;
+            }
         }
-        __syncthreads();
-        if (static_cast<int>(threadIdx.x) < n_mt * 128) {
-            const int i = threadIdx.x & 127, s0 = (threadIdx.x >> 7) * n_sl;
-            float M = -CUDART_INF_F, Ls = 0.f;
+        // 512 threads: four (one query tile) or two (two tiles) slices of the records per row
+        if constexpr (!FEW) {
+            const int n_sl = two ? 2 : 4;
+            if (threadIdx.x < 512) {
+                const int i = threadIdx.x & 127, sl = (threadIdx.x >> 7) & (n_sl - 1), mt = two ? threadIdx.x >> 8 : 0;
+                const size_t step = static_cast<size_t>(n_mt) * 256;
+                const float* src = a.cta_stat + (static_cast<size_t>(hs) * a.cph * n_mt + mt) * 256 + i;
+                float M = -CUDART_INF_F, Ls = 0.f;
+                // records in flight per thread: enough for one round trip where a head has 18 CTAs (8 heads)
+                constexpr int kF = BIG ? 9 : 5;
+                for (int j0 = sl; j0 < a.cph; j0 += kF * n_sl) {
+                    float rm[kF], rl[kF];
 #pragma unroll
-            for (int s = 0; s < 4; ++s)
-                if (s >= s0 && s < s0 + n_sl) M = fmaxf(M, slice[(s * 2) * 128 + i]);
+                    for (int u = 0; u < kF; ++u) {
+                        const int j = j0 + n_sl * u;
+                        rm[u] = (j < a.cph) ? __ldcg(src + j * step) : -CUDART_INF_F;
+                        rl[u] = (j < a.cph) ? __ldcg(src + j * step + 128) : 0.f;
+                    }
+                    float bm = M;
 #pragma unroll
-            for (int s = 0; s < 4; ++s)
-                if (s >= s0 && s < s0 + n_sl) {
-                    const float m = slice[(s * 2) * 128 + i];
-                    Ls += (m == -CUDART_INF_F) ? 0.f : slice[(s * 2 + 1) * 128 + i] * ex2_approx(m - M);
+                    for (int u = 0; u < kF; ++u) bm = fmaxf(bm, rm[u]);
+                    float acc = (M == -CUDART_INF_F) ? 0.f : Ls * ex2_approx(M - bm);
+#pragma unroll
+                    for (int u = 0; u < kF; ++u) acc += (rm[u] == -CUDART_INF_F) ? 0.f : rl[u] * ex2_approx(rm[u] - bm);
+                    M = bm;
+                    Ls = acc;
                 }
-            gm[threadIdx.x] = M;
-            ginv[threadIdx.x] = 1.0f / Ls;       // rows >= R are never used
+                slice[((threadIdx.x >> 7) * 2 + 0) * 128 + i] = M;
+                slice[((threadIdx.x >> 7) * 2 + 1) * 128 + i] = Ls;
+            }
+            __syncthreads();
+            if (static_cast<int>(threadIdx.x) < n_mt * 128) {
+                const int i = threadIdx.x & 127, s0 = (threadIdx.x >> 7) * n_sl;
+                float M = -CUDART_INF_F, Ls = 0.f;
+#pragma unroll
+                for (int s = 0; s < 4; ++s)
+                    if (s >= s0 && s < s0 + n_sl) M = fmaxf(M, slice[(s * 2) * 128 + i]);
+#pragma unroll
+                for (int s = 0; s < 4; ++s)
+                    if (s >= s0 && s < s0 + n_sl) {
+                        const float m = slice[(s * 2) * 128 + i];
+                        Ls += (m == -CUDART_INF_F) ? 0.f : slice[(s * 2 + 1) * 128 + i] * ex2_approx(m - M);
+                    }
+                gm[threadIdx.x] = M;
+                ginv[threadIdx.x] = 1.0f / Ls;       // rows >= R are never used
+            }
         }
         __syncthreads();
         // chunk scores of this CTA's key range: partial sums x exp2(m_panel - m_i) / l_i, summed over
@@ -558,10 +592,12 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     }
 }
 
+// 0: small, 1: big, 2: small with few rows
 template <int C_STATIC>
-const void* kernel_of(bool big) {
-    return big ? reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, true>)
-               : reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, false>);
+const void* kernel_of(int variant) {
+    return variant == 1 ? reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, true, false>)
+         : variant == 2 ? reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, false, true>)
+                        : reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, false, false>);
 }
 
 }  // namespace
@@ -652,20 +688,20 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     a.score_row = io.out_scores ? io.C : (io.C + 3) & ~3;
     a.spill = scores + (((static_cast<size_t>(io.Hkv) << plan.shift) * ((io.C + 3) & ~3) + 63) & ~static_cast<size_t>(63));
     a.counters = io.counters;
-    const bool big = plan.n_mt == 2 || plan.n_off > 0;
+    const int variant = plan.n_mt == 2 || plan.n_off > 0 ? 1 : (io.R <= 64 && plan.cph > kRManyCtas ? 2 : 0);
     const void* kern = nullptr;
     int v = 0;
     switch (plan.c_static) {
-        case 5: kern = kernel_of<5>(big); v = 0; break;
-        case 8: kern = kernel_of<8>(big); v = 1; break;
-        case 10: kern = kernel_of<10>(big); v = 2; break;
-        case 16: kern = kernel_of<16>(big); v = 3; break;
-        case 20: kern = kernel_of<20>(big); v = 4; break;
-        case 32: kern = kernel_of<32>(big); v = 5; break;
+        case 5: kern = kernel_of<5>(variant); v = 0; break;
+        case 8: kern = kernel_of<8>(variant); v = 1; break;
+        case 10: kern = kernel_of<10>(variant); v = 2; break;
+        case 16: kern = kernel_of<16>(variant); v = 3; break;
+        case 20: kern = kernel_of<20>(variant); v = 4; break;
+        case 32: kern = kernel_of<32>(variant); v = 5; break;
         default: return cudaErrorInvalidValue;
     }
-    v += big ? 6 : 0;
-    static int smem_set[12][64] = {{0}};
+    v += 6 * variant;
+    static int smem_set[18][64] = {{0}};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
