@@ -128,3 +128,11 @@ def test_token_scores_and_chunk_scores_with_and_without_them(ck, Hq, Hkv, d, L, 
     assert_scores_close(ts.cpu().numpy(), t, R, L, "token scores")
     assert_scores_close(cs.cpu().numpy(), s, R, L, "chunk scores beside token scores")
     assert_scores_close(alone.cpu().numpy(), s, R, L, "chunk scores alone")
+
+
+# Up to 64 rows and more than 20 CTAs a head read the head's row statistics in a variant of their own: its first row and CTA counts,
+# the last ones before it, one round trip of records (40) and its first beyond, every CTA of the GPU for one head.
+@pytest.mark.parametrize("Hq,w,d,tiles", [(1, 1, 64, 21), (3, 11, 64, 20), (4, 16, 128, 21), (4, 16, 64, 40), (2, 32, 64, 41), (5, 13, 64, 41),
+                                          (4, 16, 64, 148), (1, 64, 128, 81)])
+def test_layer_with_few_rows_and_many_ctas(ck, Hq, w, d, tiles):
+    test_layer_and_chunk_scores(ck, Hq, 1, d, 120 * tiles - 7, w, 10)
