@@ -142,6 +142,13 @@ def _dev(t: torch.Tensor, dtype: torch.dtype, name: str) -> torch.Tensor:
     return t
 
 
+def _sized(t: torch.Tensor, dtype: torch.dtype, n: int, name: str) -> torch.Tensor:
+    """_dev with at least n elements: the kernels read or write that many."""
+    if _dev(t, dtype, name).numel() < n:
+        raise ValueError(f"{name} must have at least {n} elements")
+    return t
+
+
 def strerror(status: int) -> str:
     return lib.chunkkv_strerror(status).decode()
 
@@ -346,6 +353,16 @@ def window_queries(qkv: torch.Tensor, Hq: int, Hkv: int, d: int, w: int, cos_row
     return out
 
 
+def _paged(block_table: torch.Tensor, cache_K: torch.Tensor, cache_V: torch.Tensor, Hkv: int, d: int, n_max: int) -> None:
+    """The paged destination of n_max rows a head: caches [pages, page_size, Hkv, d], a table with an entry per page used."""
+    _dev(cache_K, torch.bfloat16, "cache_K")
+    rows = cache_K.shape[0] * cache_K.shape[1]
+    for t, name in ((cache_K, "cache_K"), (cache_V, "cache_V")):
+        _sized(t, torch.bfloat16, rows * Hkv * d, name)
+    if cache_K.shape[1] > 0:
+        _sized(block_table, torch.int32, -(-n_max // cache_K.shape[1]), "block_table")
+
+
 def gather_paged(K: torch.Tensor, V: torch.Tensor, idx: torch.Tensor, block_table: torch.Tensor, cache_K: torch.Tensor,
                  cache_V: torch.Tensor, stream: Optional[torch.cuda.Stream] = None) -> None:
     """Kept rows into a paged cache [num_pages, page_size, Hkv, d] through block_table (int32)."""
@@ -401,8 +418,15 @@ def compress_layer_paged(q_obs: Optional[torch.Tensor], K: torch.Tensor, V: torc
     r = _native.layer_paged(q_obs, K, V, Hq, w, c, budget, block_table, cache_K, cache_V, reuse_idx, out_idx, stream)
     if r is not None:
         return _done(r, "chunkkv_compress_layer_paged")
+    _dev(K, torch.bfloat16, "K")
     Hkv, L, d = K.shape
     n_max = out_len(L, w, c, budget)
+    _sized(V, torch.bfloat16, K.numel(), "V")
+    if q_obs is not None:
+        _sized(q_obs, torch.bfloat16, Hq * w * d, "q_obs")
+    if reuse_idx is not None:
+        _sized(reuse_idx, torch.int32, Hkv * n_max, "reuse_idx")
+    _paged(block_table, cache_K, cache_V, Hkv, d, n_max)
     if reuse_idx is None:
         ensure_workspace(L, Hq, Hkv, d, w, c)
     if out_idx is None:

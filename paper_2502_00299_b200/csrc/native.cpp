@@ -39,6 +39,12 @@ const at::Tensor& checked(PyObject* o, at::ScalarType type) {
     if (!t.is_cuda() || t.scalar_type() != type || !t.is_contiguous()) throw Decline{};
     return t;
 }
+// The same with at least `need` elements.
+const at::Tensor& sized(PyObject* o, at::ScalarType type, long long need) {
+    const at::Tensor& t = checked(o, type);
+    if (t.numel() < need) throw Decline{};
+    return t;
+}
 int narrow(long long v) {
     if (v < INT_MIN || v > INT_MAX) throw Decline{};
     return static_cast<int>(v);
@@ -201,14 +207,19 @@ PyObject* layer_alg1(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // layer_paged(q_obs, K, V, Hq, w, c, budget, block_table, cache_K, cache_V, reuse_idx, out_idx, stream) -> idx
 PyObject* layer_paged(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 13, [&]() -> PyObject* {
-        const at::Tensor &K = tensor(a[1]), &V = tensor(a[2]), &bt = tensor(a[7]), &cK = tensor(a[8]), &cV = tensor(a[9]);
+        const at::Tensor &K = checked(a[1], at::kBFloat16), &cK = checked(a[8], at::kBFloat16);
         if (K.dim() != 3 || cK.dim() < 2) throw Decline{};
-        const void* q = a[0] == Py_None ? nullptr : tensor(a[0]).data_ptr();
-        const int32_t* reuse = a[10] == Py_None ? nullptr : static_cast<const int32_t*>(tensor(a[10]).data_ptr());
         const int Hkv = narrow(K.size(0)), L = narrow(K.size(1)), d = narrow(K.size(2));
         const int Hq = integer(a[3]), w = integer(a[4]), c = integer(a[5]), budget = integer(a[6]);
         const int n_max = chunkkv_out_len(L, w, c, budget);
         if (n_max < 0) throw Decline{};
+        const long long page = narrow(cK.size(1)), pages = narrow(cK.size(0)), n_idx = static_cast<long long>(Hkv) * n_max;
+        if (page < 1) throw Decline{};
+        const at::Tensor &V = sized(a[2], at::kBFloat16, K.numel()), &bt = sized(a[7], at::kInt, (n_max + page - 1) / page);
+        const at::Tensor& cV = sized(a[9], at::kBFloat16, pages * page * Hkv * d);
+        if (cK.numel() < pages * page * Hkv * d) throw Decline{};
+        const void* q = a[0] == Py_None ? nullptr : sized(a[0], at::kBFloat16, static_cast<long long>(Hq) * w * d).data_ptr();
+        const int32_t* reuse = a[10] == Py_None ? nullptr : static_cast<const int32_t*>(sized(a[10], at::kInt, n_idx).data_ptr());
         if (reuse == nullptr) room(chunkkv_workspace_bytes(L, Hq, Hkv, d, w, c));
         void* s = stream_of(a[12]);
         Ref oI;
@@ -216,9 +227,9 @@ PyObject* layer_paged(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const void *k = K.data_ptr(), *v = V.data_ptr();
         const int32_t* table = static_cast<const int32_t*>(bt.data_ptr());
         void *pK = cK.data_ptr(), *pV = cV.data_ptr();
-        const int page = narrow(cK.size(1)), pages = narrow(cK.size(0));
         const int st = unlocked([&] {
-            return chunkkv_compress_layer_paged(q, k, v, L, Hq, Hkv, d, w, c, budget, reuse, table, page, pages, pK, pV, pI, s);
+            return chunkkv_compress_layer_paged(q, k, v, L, Hq, Hkv, d, w, c, budget, reuse, table, static_cast<int>(page),
+                                                static_cast<int>(pages), pK, pV, pI, s);
         });
         if (st != 0) return PyLong_FromLong(st);
         Py_INCREF(oI.p);

@@ -12,6 +12,7 @@ CALLS = ("layer", "layer_strided", "layer_alg1", "layer_paged", "window_queries"
 def test_declined_arguments_raise_what_the_general_way_raises():
     x = torch.zeros(2, 64, 64, dtype=torch.bfloat16)               # not on a GPU
     for call in (lambda: ck.compress_layer(x, x, x, 4, 16, 8, 32), lambda: ck.compress_layer_strided(x, x, x, 4, 16, 8, 32),
+                 lambda: ck.compress_layer_paged(x, x, x, 4, 16, 8, 32, x, x[None], x[None]),
                  lambda: ck.compress_layer_alg1(x, x, x, 4, 16, 8, 32), lambda: ck.score(x, x, 16, 8),
                  lambda: ck.compress_model([(x, x, x)], 4, 16, 8, 32), lambda: ck.compress_model_strided([(x, x, x)], 4, 16, 8, 32),
                  lambda: ck.window_queries(x[0], 1, 1, 64, 16, x[0], x[0])):
@@ -22,6 +23,70 @@ def test_declined_arguments_raise_what_the_general_way_raises():
     for name in CALLS:
         with pytest.raises(TypeError):
             getattr(binding._native, name)(1, 2, 3)
+
+
+class Fake:
+    """What the general way looks at of a CUDA tensor; nothing is behind it."""
+
+    def __init__(self, *shape, dtype=torch.bfloat16, cuda=True, contiguous=True):
+        self.shape, self.dtype, self.is_cuda, self.device, self._contiguous = torch.Size(shape), dtype, cuda, torch.device("cuda"), contiguous
+
+    def is_contiguous(self):
+        return self._contiguous
+
+    def numel(self):
+        return self.shape.numel()
+
+    def dim(self):
+        return len(self.shape)
+
+    def stride(self, i):
+        return self.shape[i + 1:].numel()
+
+    def data_ptr(self):
+        raise AssertionError("the pointer of a tensor that should have been refused")
+
+
+def _refused(call, good, bad):
+    """`good` passes the checks (and ends where a device is asked for, in data_ptr where there is one); each of `bad` in its place does not."""
+    with pytest.raises((RuntimeError, AssertionError)):
+        call(**good)
+    for name, values in bad.items():
+        for v in values:
+            with pytest.raises(ValueError, match=name):
+                call(**{**good, name: v})
+
+
+def test_paged_layer_call_checks_its_tensors():
+    Hq, Hkv, d, L, w, c, budget, page = 8, 2, 64, 300, 16, 10, 100, 16
+    n = ck.out_len(L, w, c, budget)
+    i32 = torch.int32
+    good = dict(q_obs=Fake(Hq, w, d), K=Fake(Hkv, L, d), V=Fake(Hkv, L, d), block_table=Fake(-(-n // page), dtype=i32),
+                cache_K=Fake(9, page, Hkv, d), cache_V=Fake(9, page, Hkv, d))
+    kinds = lambda *s: [Fake(*s, cuda=False), Fake(*s, dtype=torch.float16), Fake(*s, contiguous=False)]
+    bad = {"q_obs": kinds(Hq, w, d) + [Fake(Hq, w - 1, d)], "K": kinds(Hkv, L, d), "V": kinds(Hkv, L, d) + [Fake(Hkv, L - 1, d)],
+           "block_table": [Fake(9, dtype=torch.int64), Fake(9, dtype=i32, cuda=False), Fake(-(-n // page) - 1, dtype=i32)],
+           "cache_K": kinds(9, page, Hkv, d) + [Fake(9, page, 1, d)], "cache_V": kinds(9, page, Hkv, d) + [Fake(8, page, Hkv, d)]}
+    call = lambda **k: ck.compress_layer_paged(k.pop("q_obs"), k.pop("K"), k.pop("V"), Hq, w, c, budget, **k)
+    _refused(call, good, bad)
+    idx = Fake(Hkv, n, dtype=i32)
+    _refused(call, {**good, "q_obs": None, "reuse_idx": idx}, {"reuse_idx": [Fake(Hkv, n, dtype=torch.int64), Fake(Hkv, n - 1, dtype=i32)]})
+
+
+@pytest.mark.gpu
+def test_native_paged_layer_call_declines_what_the_general_way_refuses():
+    Hq, Hkv, d, L, w, c, budget = 8, 2, 64, 300, 16, 10, 100
+    n, bf = ck.out_len(L, w, c, budget), torch.bfloat16
+    ck.ensure_workspace(L, Hq, Hkv, d, w, c)
+    z = lambda *s, dtype=bf: torch.zeros(*s, dtype=dtype, device="cuda")
+    good = [z(Hq, w, d), z(Hkv, L, d), z(Hkv, L, d), Hq, w, c, budget, torch.arange(9, dtype=torch.int32, device="cuda"), z(9, 16, Hkv, d), z(9, 16, Hkv, d),
+            None, None, None]
+    assert binding._native.layer_paged(*good) is not None
+    for i, t in ((0, z(Hq, w - 1, d)), (1, z(Hkv, d, L).transpose(1, 2)), (1, z(Hkv, L, d).cpu()), (2, z(Hkv, L - 1, d)), (2, z(Hkv, L, d, dtype=torch.float16)),
+                 (7, torch.arange(9, device="cuda")), (7, good[7][:6]), (7, good[7].cpu()), (8, z(9, 16, 1, d)), (9, z(8, 16, Hkv, d)),
+                 (9, z(9, Hkv, 16, d).transpose(1, 2)), (10, z(Hkv, n, dtype=torch.int64)), (10, z(Hkv, n - 1, dtype=torch.int32))):
+        assert binding._native.layer_paged(*[t if j == i else x for j, x in enumerate(good)]) is None, i
+    assert ck.device_status() == 0
 
 
 def _general(monkeypatch):
