@@ -278,6 +278,7 @@ def compress_layer_alg1(q_obs: torch.Tensor, K: torch.Tensor, V: torch.Tensor, H
     _dev(q_obs, torch.bfloat16, "q_obs"); _dev(K, torch.bfloat16, "K"); _dev(V, torch.bfloat16, "V")
     Hkv, L, d = K.shape
     n_max = out_len_alg1(L, w, c, budget)
+    _outputs(Hkv * n_max, d, out_K, out_V, out_idx)
     ensure_workspace(L, Hq, Hkv, d, w, c)
     if out_K is None:
         out_K = torch.empty((Hkv, n_max, d), dtype=torch.bfloat16, device=K.device)
@@ -297,6 +298,7 @@ def gather(K: torch.Tensor, V: torch.Tensor, idx: torch.Tensor,
     _dev(K, torch.bfloat16, "K"); _dev(V, torch.bfloat16, "V"); _dev(idx, torch.int32, "idx")
     Hkv, L, d = K.shape
     n_max = idx.shape[1]
+    _outputs(Hkv * n_max, d, out_K, out_V, None)
     if out_K is None:
         out_K = torch.empty((Hkv, n_max, d), dtype=torch.bfloat16, device=K.device)
     if out_V is None:
@@ -323,6 +325,7 @@ def compress_layer(q_obs: Optional[torch.Tensor], K: torch.Tensor, V: torch.Tens
         _dev(reuse_idx, torch.int32, "reuse_idx")
     Hkv, L, d = K.shape
     n_max = out_len(L, w, c, budget)
+    _outputs(Hkv * n_max, d, out_K, out_V, out_idx)
     dev = K.device
     if reuse_idx is None:
         ensure_workspace(L, Hq, Hkv, d, w, c)
@@ -351,6 +354,13 @@ def window_queries(qkv: torch.Tensor, Hq: int, Hkv: int, d: int, w: int, cos_row
     _check(lib.chunkkv_window_queries(qkv.data_ptr(), row_elems, T, Hq, Hkv, d, w, cos_rows.data_ptr(),
                                       sin_rows.data_ptr(), out.data_ptr(), _stream(stream)), "chunkkv_window_queries")
     return out
+
+
+def _outputs(n_row: int, d: int, out_K: Optional[torch.Tensor], out_V: Optional[torch.Tensor], out_idx: Optional[torch.Tensor]) -> None:
+    """Outputs that the caller gave: n_row rows of keys and values, n_row positions."""
+    for t, dtype, n, name in ((out_K, torch.bfloat16, n_row * d, "out_K"), (out_V, torch.bfloat16, n_row * d, "out_V"), (out_idx, torch.int32, n_row, "out_idx")):
+        if t is not None:
+            _sized(t, dtype, n, name)
 
 
 def _paged(block_table: torch.Tensor, cache_K: torch.Tensor, cache_V: torch.Tensor, Hkv: int, d: int, n_max: int) -> None:
@@ -394,6 +404,7 @@ def compress_layer_strided(q_obs: Optional[torch.Tensor], K: torch.Tensor, V: to
         _dev(reuse_idx, torch.int32, "reuse_idx")
     Hkv, L, d = K.shape
     n_max = out_len(L, w, c, budget)
+    _outputs(Hkv * n_max, d, out_K, out_V, out_idx)
     dev = K.device
     if reuse_idx is None:
         ensure_workspace(L, Hq, Hkv, d, w, c)
@@ -427,6 +438,7 @@ def compress_layer_paged(q_obs: Optional[torch.Tensor], K: torch.Tensor, V: torc
     if reuse_idx is not None:
         _sized(reuse_idx, torch.int32, Hkv * n_max, "reuse_idx")
     _paged(block_table, cache_K, cache_V, Hkv, d, n_max)
+    _outputs(Hkv * n_max, d, None, None, out_idx)
     if reuse_idx is None:
         ensure_workspace(L, Hq, Hkv, d, w, c)
     if out_idx is None:
@@ -483,6 +495,7 @@ class Lane:
         """chunkkv_compress_layer_lane on this lane's stream."""
         Hkv, L, d = K.shape
         n_max = out_len(L, w, c, budget)
+        _outputs(Hkv * n_max, d, out_K, out_V, out_idx)
         dev = K.device
         with torch.cuda.stream(self.stream):
             if out_K is None:
@@ -524,6 +537,7 @@ class Pipe:
         """chunkkv_pipe_layer; the outputs are complete after join()."""
         Hkv, L, d = K.shape
         n_max = out_len(L, w, c, budget)
+        _outputs(Hkv * n_max, d, out_K, out_V, out_idx)
         dev = K.device
         with torch.cuda.stream(self.stream):
             if out_K is None:
@@ -620,6 +634,9 @@ def compress_model(layers: Sequence[Tuple[Optional[torch.Tensor], torch.Tensor, 
         outs = [(torch.empty((Hkv, n_max, d), dtype=torch.bfloat16, device=dev),
                  torch.empty((Hkv, n_max, d), dtype=torch.bfloat16, device=dev),
                  torch.empty((Hkv, n_max), dtype=torch.int32, device=dev)) for _ in range(n)]
+    else:
+        for o in outs:
+            _outputs(Hkv * n_max, d, o[0], o[1], o[2])
     _ensure_bytes(int(lib.chunkkv_model_workspace_bytes(n, L, Hq, Hkv, d, w, c, budget, n_reuse)))
     arr = ctypes.c_void_p * n
     qa = arr(*[None if t[0] is None else t[0].data_ptr() for t in layers])
@@ -660,6 +677,9 @@ def compress_model_strided(layers: Sequence[Tuple[Optional[torch.Tensor], torch.
         outs = [(torch.empty((Hkv, n_max, d), dtype=torch.bfloat16, device=dev),
                  torch.empty((Hkv, n_max, d), dtype=torch.bfloat16, device=dev),
                  torch.empty((Hkv, n_max), dtype=torch.int32, device=dev)) for _ in range(n)]
+    else:
+        for o in outs:
+            _outputs(Hkv * n_max, d, o[0], o[1], o[2])
     _ensure_bytes(max(int(lib.chunkkv_model_workspace_bytes(n, L, Hq, Hkv, d, w, c, budget, n_reuse)),
                       workspace_bytes(L, Hq, Hkv, d, w, c)))
     arr = ctypes.c_void_p * n
@@ -696,6 +716,9 @@ def compress_model_paged(layers: Sequence[Tuple[Optional[torch.Tensor], torch.Te
     dev = layers[0][1].device
     if out_idx is None:
         out_idx = [torch.empty((Hkv, n_max), dtype=torch.int32, device=dev) for _ in range(n)]
+    else:
+        for t in out_idx:
+            _outputs(Hkv * n_max, d, None, None, t)
     _ensure_bytes(max(int(lib.chunkkv_model_workspace_bytes(n, L, Hq, Hkv, d, w, c, budget, n_reuse)),
                       workspace_bytes(L, Hq, Hkv, d, w, c)))
     arr = ctypes.c_void_p * n

@@ -83,8 +83,9 @@ struct Ref {                             // an owned reference
     Ref& operator=(const Ref&) = delete;
     ~Ref() { Py_XDECREF(p); }
     template <class Make>
-    void* set(PyObject* given, Make make) {      // the given output or a new one; its address
+    void* set(PyObject* given, at::ScalarType type, long long n, Make make) {      // the given output (n elements of `type`) or a new one; its address
         if (given != Py_None) {
+            sized(given, type, n);
             p = given;
             Py_INCREF(p);
         } else {
@@ -141,12 +142,13 @@ PyObject* layer(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int Hq = integer(a[3]), w = integer(a[4]), c = integer(a[5]), budget = integer(a[6]);
         const int n_max = chunkkv_out_len(L, w, c, budget);
         if (n_max < 0) throw Decline{};
+        const long long n_row = static_cast<long long>(Hkv) * n_max;
         if (reuse == nullptr) room(chunkkv_workspace_bytes(L, Hq, Hkv, d, w, c));
         void* s = stream_of(a[11]);
         Ref oK, oV, oI;
-        void* pK = oK.set(a[8], [&] { return rows(K, Hkv, n_max, d); });
-        void* pV = oV.set(a[9], [&] { return rows(K, Hkv, n_max, d); });
-        int32_t* pI = static_cast<int32_t*>(oI.set(a[10], [&] { return ids(K, Hkv, n_max); }));
+        void* pK = oK.set(a[8], at::kBFloat16, n_row * d, [&] { return rows(K, Hkv, n_max, d); });
+        void* pV = oV.set(a[9], at::kBFloat16, n_row * d, [&] { return rows(K, Hkv, n_max, d); });
+        int32_t* pI = static_cast<int32_t*>(oI.set(a[10], at::kInt, n_row, [&] { return ids(K, Hkv, n_max); }));
         const void *k = K.data_ptr(), *v = V.data_ptr();
         const int st = unlocked([&] { return chunkkv_compress_layer(q, k, v, L, Hq, Hkv, d, w, c, budget, reuse, pK, pV, pI, s); });
         if (st != 0) return PyLong_FromLong(st);
@@ -166,12 +168,13 @@ PyObject* layer_strided(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int Hq = integer(a[3]), w = integer(a[4]), c = integer(a[5]), budget = integer(a[6]);
         const int n_max = chunkkv_out_len(L, w, c, budget);
         if (n_max < 0) throw Decline{};
+        const long long n_row = static_cast<long long>(Hkv) * n_max;
         if (reuse == nullptr) room(chunkkv_workspace_bytes(L, Hq, Hkv, d, w, c));
         void* s = stream_of(a[11]);
         Ref oK, oV, oI;
-        void* pK = oK.set(a[8], [&] { return rows(K, Hkv, n_max, d); });
-        void* pV = oV.set(a[9], [&] { return rows(K, Hkv, n_max, d); });
-        int32_t* pI = static_cast<int32_t*>(oI.set(a[10], [&] { return ids(K, Hkv, n_max); }));
+        void* pK = oK.set(a[8], at::kBFloat16, n_row * d, [&] { return rows(K, Hkv, n_max, d); });
+        void* pV = oV.set(a[9], at::kBFloat16, n_row * d, [&] { return rows(K, Hkv, n_max, d); });
+        int32_t* pI = static_cast<int32_t*>(oI.set(a[10], at::kInt, n_row, [&] { return ids(K, Hkv, n_max); }));
         const void *k = K.data_ptr(), *v = V.data_ptr();
         const long long kt = K.stride(1), kh = K.stride(0), vt = V.stride(1), vh = V.stride(0);
         const int st = unlocked([&] {
@@ -191,12 +194,13 @@ PyObject* layer_alg1(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int Hq = integer(a[3]), w = integer(a[4]), c = integer(a[5]), budget = integer(a[6]);
         const int n_max = chunkkv_out_len_alg1(L, w, c, budget);
         if (n_max < 0) throw Decline{};
+        const long long n_row = static_cast<long long>(Hkv) * n_max;
         room(chunkkv_workspace_bytes(L, Hq, Hkv, d, w, c));
         void* s = stream_of(a[10]);
         Ref oK, oV, oI;
-        void* pK = oK.set(a[7], [&] { return rows(K, Hkv, n_max, d); });
-        void* pV = oV.set(a[8], [&] { return rows(K, Hkv, n_max, d); });
-        int32_t* pI = static_cast<int32_t*>(oI.set(a[9], [&] { return ids(K, Hkv, n_max); }));
+        void* pK = oK.set(a[7], at::kBFloat16, n_row * d, [&] { return rows(K, Hkv, n_max, d); });
+        void* pV = oV.set(a[8], at::kBFloat16, n_row * d, [&] { return rows(K, Hkv, n_max, d); });
+        int32_t* pI = static_cast<int32_t*>(oI.set(a[9], at::kInt, n_row, [&] { return ids(K, Hkv, n_max); }));
         const void *pq = q.data_ptr(), *k = K.data_ptr(), *v = V.data_ptr();
         const int st = unlocked([&] { return chunkkv_compress_layer_alg1(pq, k, v, L, Hq, Hkv, d, w, c, budget, pK, pV, pI, s); });
         if (st != 0) return PyLong_FromLong(st);
@@ -213,17 +217,17 @@ PyObject* layer_paged(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int Hq = integer(a[3]), w = integer(a[4]), c = integer(a[5]), budget = integer(a[6]);
         const int n_max = chunkkv_out_len(L, w, c, budget);
         if (n_max < 0) throw Decline{};
-        const long long page = narrow(cK.size(1)), pages = narrow(cK.size(0)), n_idx = static_cast<long long>(Hkv) * n_max;
+        const long long page = narrow(cK.size(1)), pages = narrow(cK.size(0)), n_row = static_cast<long long>(Hkv) * n_max;
         if (page < 1) throw Decline{};
         const at::Tensor &V = sized(a[2], at::kBFloat16, K.numel()), &bt = sized(a[7], at::kInt, (n_max + page - 1) / page);
         const at::Tensor& cV = sized(a[9], at::kBFloat16, pages * page * Hkv * d);
         if (cK.numel() < pages * page * Hkv * d) throw Decline{};
         const void* q = a[0] == Py_None ? nullptr : sized(a[0], at::kBFloat16, static_cast<long long>(Hq) * w * d).data_ptr();
-        const int32_t* reuse = a[10] == Py_None ? nullptr : static_cast<const int32_t*>(sized(a[10], at::kInt, n_idx).data_ptr());
+        const int32_t* reuse = a[10] == Py_None ? nullptr : static_cast<const int32_t*>(sized(a[10], at::kInt, n_row).data_ptr());
         if (reuse == nullptr) room(chunkkv_workspace_bytes(L, Hq, Hkv, d, w, c));
         void* s = stream_of(a[12]);
         Ref oI;
-        int32_t* pI = static_cast<int32_t*>(oI.set(a[11], [&] { return ids(K, Hkv, n_max); }));
+        int32_t* pI = static_cast<int32_t*>(oI.set(a[11], at::kInt, n_row, [&] { return ids(K, Hkv, n_max); }));
         const void *k = K.data_ptr(), *v = V.data_ptr();
         const int32_t* table = static_cast<const int32_t*>(bt.data_ptr());
         void *pK = cK.data_ptr(), *pV = cV.data_ptr();
@@ -247,7 +251,7 @@ PyObject* window_queries(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const long long row = x.size(1);
         void* s = stream_of(a[7]);
         Ref out;
-        void* p = out.set(Py_None, [&] { return rows(x, Hq, w, d); });
+        void* p = out.set(Py_None, at::kBFloat16, 0, [&] { return rows(x, Hq, w, d); });
         const void* px = x.data_ptr();
         const float *pc = static_cast<const float*>(co.data_ptr()), *ps = static_cast<const float*>(si.data_ptr());
         const int st = unlocked([&] { return chunkkv_window_queries(px, row, T, Hq, Hkv, d, w, pc, ps, p, s); });
@@ -271,9 +275,9 @@ PyObject* score(PyObject*, PyObject* const* a, Py_ssize_t n) {
         void* s = stream_of(a[5]);
         const auto f32 = at::TensorOptions().dtype(at::kFloat).device(K.device());
         Ref cs, ts;
-        float* pc = static_cast<float*>(cs.set(Py_None, [&] { return at::empty({Hkv, C}, f32); }));
+        float* pc = static_cast<float*>(cs.set(Py_None, at::kFloat, 0, [&] { return at::empty({Hkv, C}, f32); }));
         float* pt = nullptr;
-        if (tokens) pt = static_cast<float*>(ts.set(Py_None, [&] { return at::empty({Hkv, L - w}, f32); }));
+        if (tokens) pt = static_cast<float*>(ts.set(Py_None, at::kFloat, 0, [&] { return at::empty({Hkv, L - w}, f32); }));
         const void *pq = q.data_ptr(), *pk = K.data_ptr();
         const int st = unlocked([&] { return chunkkv_score(pq, pk, L, Hq, Hkv, d, w, c, pt, pc, s); });
         if (st != 0) return PyLong_FromLong(st);
@@ -324,6 +328,7 @@ PyObject* model(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int Hq = integer(a[1]), w = integer(a[2]), c = integer(a[3]), budget = integer(a[4]), n_reuse = integer(a[5]);
         const int n_max = chunkkv_out_len(L, w, c, budget);
         if (n_max < 0) throw Decline{};
+        const long long n_row = static_cast<long long>(Hkv) * n_max;
         const int nl = narrow(layers.n);
         const size_t need = chunkkv_model_workspace_bytes(nl, L, Hq, Hkv, d, w, c, budget, n_reuse);
         room(need > 0 ? need : 1);
@@ -336,9 +341,9 @@ PyObject* model(PyObject*, PyObject* const* a, Py_ssize_t n) {
             const at::Tensor& like = tensor(Items(layers.p[0]).p[1]);
             for (Py_ssize_t i = 0; i < layers.n; ++i) {
                 Ref x, y, z;
-                oK[i] = x.set(Py_None, [&] { return rows(like, Hkv, n_max, d); });
-                oV[i] = y.set(Py_None, [&] { return rows(like, Hkv, n_max, d); });
-                oI[i] = static_cast<int32_t*>(z.set(Py_None, [&] { return ids(like, Hkv, n_max); }));
+                oK[i] = x.set(Py_None, at::kBFloat16, 0, [&] { return rows(like, Hkv, n_max, d); });
+                oV[i] = y.set(Py_None, at::kBFloat16, 0, [&] { return rows(like, Hkv, n_max, d); });
+                oI[i] = static_cast<int32_t*>(z.set(Py_None, at::kInt, 0, [&] { return ids(like, Hkv, n_max); }));
                 PyObject* t = PyTuple_Pack(3, x.p, y.p, z.p);
                 if (t == nullptr) throw Decline{};
                 PyList_SET_ITEM(res.p, i, t);
@@ -350,9 +355,9 @@ PyObject* model(PyObject*, PyObject* const* a, Py_ssize_t n) {
                 if (!PyTuple_CheckExact(outs.p[i])) throw Decline{};
                 const Items o(outs.p[i]);
                 if (o.n != 3) throw Decline{};
-                oK[i] = tensor(o.p[0]).data_ptr();
-                oV[i] = tensor(o.p[1]).data_ptr();
-                oI[i] = static_cast<int32_t*>(tensor(o.p[2]).data_ptr());
+                oK[i] = sized(o.p[0], at::kBFloat16, n_row * d).data_ptr();
+                oV[i] = sized(o.p[1], at::kBFloat16, n_row * d).data_ptr();
+                oI[i] = static_cast<int32_t*>(sized(o.p[2], at::kInt, n_row).data_ptr());
                 Py_INCREF(outs.p[i]);
                 PyList_SET_ITEM(res.p, i, outs.p[i]);
             }

@@ -73,6 +73,46 @@ def test_paged_layer_call_checks_its_tensors():
     _refused(call, {**good, "q_obs": None, "reuse_idx": idx}, {"reuse_idx": [Fake(Hkv, n, dtype=torch.int64), Fake(Hkv, n - 1, dtype=i32)]})
 
 
+def test_given_outputs_are_checked():
+    Hq, Hkv, d, L, w, c, budget = 8, 2, 64, 300, 16, 10, 100
+    i32 = torch.int32
+    q, K, V = Fake(Hq, w, d), Fake(Hkv, L, d), Fake(Hkv, L, d)
+    for call, n in ((ck.compress_layer, ck.out_len(L, w, c, budget)), (ck.compress_layer_strided, ck.out_len(L, w, c, budget)),
+                    (ck.compress_layer_alg1, ck.out_len_alg1(L, w, c, budget)), (ck.compress_model, ck.out_len(L, w, c, budget)),
+                    (ck.compress_model_strided, ck.out_len(L, w, c, budget))):
+        rows = lambda: Fake(Hkv, n, d)
+        kinds = lambda *s: [Fake(*s, cuda=False), Fake(*s, dtype=torch.float32), Fake(*s, contiguous=False), Fake(s[0], s[1] - 1, *s[2:])]
+        bad = {"out_K": kinds(Hkv, n, d), "out_V": kinds(Hkv, n, d), "out_idx": [Fake(Hkv, n, dtype=torch.int64), Fake(Hkv, n - 1, dtype=i32), Fake(Hkv, n, dtype=i32, cuda=False)]}
+        if call in (ck.compress_model, ck.compress_model_strided):
+            one = lambda out_K, out_V, out_idx: call([(q, K, V)] * 2, Hq, w, c, budget, 2, outs=[(rows(), rows(), Fake(Hkv, n, dtype=i32)), (out_K, out_V, out_idx)])
+        else:
+            one = lambda **k: call(q, K, V, Hq, w, c, budget, **k)
+        _refused(one, dict(out_K=rows(), out_V=rows(), out_idx=Fake(Hkv, n, dtype=i32)), bad)
+    n = 40
+    _refused(lambda **k: ck.gather(K, V, Fake(Hkv, n, dtype=i32), **k), dict(out_K=Fake(Hkv, n, d), out_V=Fake(Hkv, n, d)),
+             {"out_K": [Fake(Hkv, n - 1, d)], "out_V": [Fake(Hkv, n, d, cuda=False)]})
+
+
+@pytest.mark.gpu
+def test_native_calls_decline_outputs_that_the_general_way_refuses():
+    Hq, Hkv, d, L, w, c, budget = 8, 2, 64, 300, 16, 10, 100
+    n, n1, bf, i32 = ck.out_len(L, w, c, budget), ck.out_len_alg1(L, w, c, budget), torch.bfloat16, torch.int32
+    ck.set_workspace(torch.empty(64 << 20, dtype=torch.uint8, device="cuda"))
+    z = lambda *s, dtype=bf: torch.zeros(*s, dtype=dtype, device="cuda")
+    q, K, V, sizes = z(Hq, w, d), z(Hkv, L, d), z(Hkv, L, d), (Hq, w, c, budget)
+    N = binding._native
+    calls = [(lambda *o: N.layer(q, K, V, *sizes, None, *o, None), n), (lambda *o: N.layer_strided(q, K, V, *sizes, None, *o, None), n),
+             (lambda *o: N.layer_alg1(q, K, V, *sizes, *o, None), n1), (lambda *o: N.model([(q, K, V)], *sizes, 1, None, [o], False), n),
+             (lambda *o: N.model([(q, K, V)], *sizes, 1, None, [o], True), n)]
+    for call, m in calls:
+        good = [z(Hkv, m, d), z(Hkv, m, d), z(Hkv, m, dtype=i32)]
+        assert call(*good) is not None
+        for i, t in ((0, z(Hkv, m, d).cpu()), (0, z(Hkv, m - 1, d)), (0, z(Hkv, d, m).transpose(1, 2)), (1, z(Hkv, m, d, dtype=torch.float16)), (1, z(Hkv, m - 1, d)),
+                     (2, z(Hkv, m, dtype=torch.int64)), (2, z(Hkv, m - 1, dtype=i32)), (2, z(Hkv, m, dtype=i32).cpu())):
+            assert call(*[t if j == i else x for j, x in enumerate(good)]) is None, i
+    assert ck.device_status() == 0
+
+
 @pytest.mark.gpu
 def test_native_paged_layer_call_declines_what_the_general_way_refuses():
     Hq, Hkv, d, L, w, c, budget = 8, 2, 64, 300, 16, 10, 100
