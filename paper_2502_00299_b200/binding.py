@@ -221,6 +221,7 @@ def score(q_obs: torch.Tensor, K: torch.Tensor, w: int, c: int, want_token_score
     _dev(q_obs, torch.bfloat16, "q_obs"); _dev(K, torch.bfloat16, "K")
     Hq, d = q_obs.shape[0], q_obs.shape[2]
     Hkv, L = K.shape[0], K.shape[1]
+    _sized(q_obs, torch.bfloat16, Hq * w * d, "q_obs"); _sized(K, torch.bfloat16, Hkv * L * d, "K")
     C = num_chunks(L, w, c)
     ensure_workspace(L, Hq, Hkv, d, w, c)
     if want_token_scores:
@@ -278,6 +279,7 @@ def compress_layer_alg1(q_obs: torch.Tensor, K: torch.Tensor, V: torch.Tensor, H
     _dev(q_obs, torch.bfloat16, "q_obs"); _dev(K, torch.bfloat16, "K"); _dev(V, torch.bfloat16, "V")
     Hkv, L, d = K.shape
     n_max = out_len_alg1(L, w, c, budget)
+    _inputs(q_obs, Hq * w * d, V, K.numel())
     _outputs(Hkv * n_max, d, out_K, out_V, out_idx)
     ensure_workspace(L, Hq, Hkv, d, w, c)
     if out_K is None:
@@ -298,6 +300,7 @@ def gather(K: torch.Tensor, V: torch.Tensor, idx: torch.Tensor,
     _dev(K, torch.bfloat16, "K"); _dev(V, torch.bfloat16, "V"); _dev(idx, torch.int32, "idx")
     Hkv, L, d = K.shape
     n_max = idx.shape[1]
+    _inputs(None, 0, V, K.numel()); _sized(idx, torch.int32, Hkv * n_max, "idx")
     _outputs(Hkv * n_max, d, out_K, out_V, None)
     if out_K is None:
         out_K = torch.empty((Hkv, n_max, d), dtype=torch.bfloat16, device=K.device)
@@ -325,6 +328,7 @@ def compress_layer(q_obs: Optional[torch.Tensor], K: torch.Tensor, V: torch.Tens
         _dev(reuse_idx, torch.int32, "reuse_idx")
     Hkv, L, d = K.shape
     n_max = out_len(L, w, c, budget)
+    _inputs(q_obs, Hq * w * d, V, K.numel(), reuse_idx, Hkv * n_max)
     _outputs(Hkv * n_max, d, out_K, out_V, out_idx)
     dev = K.device
     if reuse_idx is None:
@@ -350,10 +354,18 @@ def window_queries(qkv: torch.Tensor, Hq: int, Hkv: int, d: int, w: int, cos_row
         return _done(r, "chunkkv_window_queries")
     _dev(qkv, torch.bfloat16, "qkv"); _dev(cos_rows, torch.float32, "cos_rows"); _dev(sin_rows, torch.float32, "sin_rows")
     T, row_elems = qkv.shape
+    _sized(cos_rows, torch.float32, w * (d // 2), "cos_rows"); _sized(sin_rows, torch.float32, w * (d // 2), "sin_rows")
     out = torch.empty((Hq, w, d), dtype=torch.bfloat16, device=qkv.device)
     _check(lib.chunkkv_window_queries(qkv.data_ptr(), row_elems, T, Hq, Hkv, d, w, cos_rows.data_ptr(),
                                       sin_rows.data_ptr(), out.data_ptr(), _stream(stream)), "chunkkv_window_queries")
     return out
+
+
+def _inputs(q_obs: Optional[torch.Tensor], n_q: int, V: Optional[torch.Tensor], n_V: int, reuse_idx: Optional[torch.Tensor] = None, n_idx: int = 0) -> None:
+    """Inputs beside K: the window queries, values of K's size, another layer's positions."""
+    for t, dtype, n, name in ((q_obs, torch.bfloat16, n_q, "q_obs"), (V, torch.bfloat16, n_V, "V"), (reuse_idx, torch.int32, n_idx, "reuse_idx")):
+        if t is not None:
+            _sized(t, dtype, n, name)
 
 
 def _outputs(n_row: int, d: int, out_K: Optional[torch.Tensor], out_V: Optional[torch.Tensor], out_idx: Optional[torch.Tensor]) -> None:
@@ -379,6 +391,8 @@ def gather_paged(K: torch.Tensor, V: torch.Tensor, idx: torch.Tensor, block_tabl
     _dev(K, torch.bfloat16, "K"); _dev(V, torch.bfloat16, "V"); _dev(idx, torch.int32, "idx")
     _dev(block_table, torch.int32, "block_table"); _dev(cache_K, torch.bfloat16, "cache_K"); _dev(cache_V, torch.bfloat16, "cache_V")
     Hkv, L, d = K.shape
+    _inputs(None, 0, V, K.numel()); _sized(idx, torch.int32, Hkv * idx.shape[1], "idx")
+    _paged(block_table, cache_K, cache_V, Hkv, d, idx.shape[1])
     _check(lib.chunkkv_gather_paged(K.data_ptr(), V.data_ptr(), idx.data_ptr(), L, Hkv, d, idx.shape[1],
                                     block_table.data_ptr(), cache_K.shape[1], cache_K.shape[0], cache_K.data_ptr(),
                                     cache_V.data_ptr(), _stream(stream)), "chunkkv_gather_paged")
@@ -404,6 +418,9 @@ def compress_layer_strided(q_obs: Optional[torch.Tensor], K: torch.Tensor, V: to
         _dev(reuse_idx, torch.int32, "reuse_idx")
     Hkv, L, d = K.shape
     n_max = out_len(L, w, c, budget)
+    _inputs(q_obs, Hq * w * d, None, 0, reuse_idx, Hkv * n_max)
+    if any(V.shape[i] < K.shape[i] for i in range(3)):
+        raise ValueError("V must be as large as K")
     _outputs(Hkv * n_max, d, out_K, out_V, out_idx)
     dev = K.device
     if reuse_idx is None:
@@ -432,11 +449,7 @@ def compress_layer_paged(q_obs: Optional[torch.Tensor], K: torch.Tensor, V: torc
     _dev(K, torch.bfloat16, "K")
     Hkv, L, d = K.shape
     n_max = out_len(L, w, c, budget)
-    _sized(V, torch.bfloat16, K.numel(), "V")
-    if q_obs is not None:
-        _sized(q_obs, torch.bfloat16, Hq * w * d, "q_obs")
-    if reuse_idx is not None:
-        _sized(reuse_idx, torch.int32, Hkv * n_max, "reuse_idx")
+    _inputs(q_obs, Hq * w * d, V, K.numel(), reuse_idx, Hkv * n_max)
     _paged(block_table, cache_K, cache_V, Hkv, d, n_max)
     _outputs(Hkv * n_max, d, None, None, out_idx)
     if reuse_idx is None:
@@ -493,8 +506,9 @@ class Lane:
                        out_idx: Optional[torch.Tensor] = None,
                        ) -> Tuple[torch.Tensor, torch.Tensor, torch.Tensor]:
         """chunkkv_compress_layer_lane on this lane's stream."""
-        Hkv, L, d = K.shape
+        Hkv, L, d = _dev(K, torch.bfloat16, "K").shape
         n_max = out_len(L, w, c, budget)
+        _inputs(q_obs, Hq * w * d, V, K.numel(), reuse_idx, Hkv * n_max)
         _outputs(Hkv * n_max, d, out_K, out_V, out_idx)
         dev = K.device
         with torch.cuda.stream(self.stream):
@@ -535,8 +549,9 @@ class Pipe:
               out_K: Optional[torch.Tensor] = None, out_V: Optional[torch.Tensor] = None,
               out_idx: Optional[torch.Tensor] = None) -> Tuple[torch.Tensor, torch.Tensor, torch.Tensor]:
         """chunkkv_pipe_layer; the outputs are complete after join()."""
-        Hkv, L, d = K.shape
+        Hkv, L, d = _dev(K, torch.bfloat16, "K").shape
         n_max = out_len(L, w, c, budget)
+        _inputs(q_obs, Hq * w * d, V, K.numel())
         _outputs(Hkv * n_max, d, out_K, out_V, out_idx)
         dev = K.device
         with torch.cuda.stream(self.stream):
@@ -625,7 +640,7 @@ def compress_model(layers: Sequence[Tuple[Optional[torch.Tensor], torch.Tensor, 
     for q, K, V in layers:
         _dev(K, torch.bfloat16, "K"); _dev(V, torch.bfloat16, "V")
         if q is not None:
-            _dev(q, torch.bfloat16, "q_obs")
+            _sized(q, torch.bfloat16, Hq * w * d, "q_obs")
         if tuple(K.shape) != (Hkv, L, d) or tuple(V.shape) != (Hkv, L, d):
             raise ValueError("all layers must share one K/V shape")
     n_max = out_len(L, w, c, budget)
@@ -670,7 +685,7 @@ def compress_model_strided(layers: Sequence[Tuple[Optional[torch.Tensor], torch.
                     and (t.stride(1), t.stride(0)) == st):
                 raise ValueError(f"{name}: CUDA bf16 [Hkv, L, d] views with the same strides in every layer are required")
         if q is not None:
-            _dev(q, torch.bfloat16, "q_obs")
+            _sized(q, torch.bfloat16, Hq * w * d, "q_obs")
     n_max = out_len(L, w, c, budget)
     dev = K0.device
     if outs is None:
@@ -706,13 +721,17 @@ def compress_model_paged(layers: Sequence[Tuple[Optional[torch.Tensor], torch.Te
     for q, K, V in layers:
         _dev(K, torch.bfloat16, "K"); _dev(V, torch.bfloat16, "V")
         if q is not None:
-            _dev(q, torch.bfloat16, "q_obs")
+            _sized(q, torch.bfloat16, Hq * w * d, "q_obs")
     page_size, num_pages = caches[0][0].shape[1], caches[0][0].shape[0]
     for (cK, cV), bt in zip(caches, block_tables):
         _dev(cK, torch.bfloat16, "cache_K"); _dev(cV, torch.bfloat16, "cache_V"); _dev(bt, torch.int32, "block_table")
         if cK.shape[0] != num_pages or cK.shape[1] != page_size:
             raise ValueError("all layers' caches must share page_size and num_pages")
     n_max = out_len(L, w, c, budget)
+    for (q, K, V), (cK, cV), bt in zip(layers, caches, block_tables):
+        _sized(K, torch.bfloat16, Hkv * L * d, "K")
+        _inputs(None, 0, V, Hkv * L * d)
+        _paged(bt, cK, cV, Hkv, d, n_max)
     dev = layers[0][1].device
     if out_idx is None:
         out_idx = [torch.empty((Hkv, n_max), dtype=torch.int32, device=dev) for _ in range(n)]

@@ -134,15 +134,16 @@ PyObject* note_workspace(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // layer(q_obs, K, V, Hq, w, c, budget, reuse_idx, out_K, out_V, out_idx, stream) -> (out_K, out_V, out_idx)
 PyObject* layer(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 12, [&]() -> PyObject* {
-        const at::Tensor &K = checked(a[1], at::kBFloat16), &V = checked(a[2], at::kBFloat16);
-        const void* q = a[0] == Py_None ? nullptr : checked(a[0], at::kBFloat16).data_ptr();
-        const int32_t* reuse = a[7] == Py_None ? nullptr : static_cast<const int32_t*>(checked(a[7], at::kInt).data_ptr());
+        const at::Tensor& K = checked(a[1], at::kBFloat16);
         if (K.dim() != 3) throw Decline{};
+        const at::Tensor& V = sized(a[2], at::kBFloat16, K.numel());
         const int Hkv = narrow(K.size(0)), L = narrow(K.size(1)), d = narrow(K.size(2));
         const int Hq = integer(a[3]), w = integer(a[4]), c = integer(a[5]), budget = integer(a[6]);
         const int n_max = chunkkv_out_len(L, w, c, budget);
         if (n_max < 0) throw Decline{};
         const long long n_row = static_cast<long long>(Hkv) * n_max;
+        const void* q = a[0] == Py_None ? nullptr : sized(a[0], at::kBFloat16, static_cast<long long>(Hq) * w * d).data_ptr();
+        const int32_t* reuse = a[7] == Py_None ? nullptr : static_cast<const int32_t*>(sized(a[7], at::kInt, n_row).data_ptr());
         if (reuse == nullptr) room(chunkkv_workspace_bytes(L, Hq, Hkv, d, w, c));
         void* s = stream_of(a[11]);
         Ref oK, oV, oI;
@@ -162,13 +163,15 @@ PyObject* layer_strided(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor &K = tensor(a[1]), &V = tensor(a[2]);
         for (const at::Tensor* t : {&K, &V})
             if (!t->is_cuda() || t->scalar_type() != at::kBFloat16 || t->dim() != 3 || t->stride(2) != 1) throw Decline{};
-        const void* q = a[0] == Py_None ? nullptr : checked(a[0], at::kBFloat16).data_ptr();
-        const int32_t* reuse = a[7] == Py_None ? nullptr : static_cast<const int32_t*>(checked(a[7], at::kInt).data_ptr());
+        for (int i = 0; i < 3; ++i)
+            if (V.size(i) < K.size(i)) throw Decline{};
         const int Hkv = narrow(K.size(0)), L = narrow(K.size(1)), d = narrow(K.size(2));
         const int Hq = integer(a[3]), w = integer(a[4]), c = integer(a[5]), budget = integer(a[6]);
         const int n_max = chunkkv_out_len(L, w, c, budget);
         if (n_max < 0) throw Decline{};
         const long long n_row = static_cast<long long>(Hkv) * n_max;
+        const void* q = a[0] == Py_None ? nullptr : sized(a[0], at::kBFloat16, static_cast<long long>(Hq) * w * d).data_ptr();
+        const int32_t* reuse = a[7] == Py_None ? nullptr : static_cast<const int32_t*>(sized(a[7], at::kInt, n_row).data_ptr());
         if (reuse == nullptr) room(chunkkv_workspace_bytes(L, Hq, Hkv, d, w, c));
         void* s = stream_of(a[11]);
         Ref oK, oV, oI;
@@ -188,13 +191,15 @@ PyObject* layer_strided(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // layer_alg1(q_obs, K, V, Hq, w, c, budget, out_K, out_V, out_idx, stream) -> (out_K, out_V, out_idx)
 PyObject* layer_alg1(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 11, [&]() -> PyObject* {
-        const at::Tensor &q = checked(a[0], at::kBFloat16), &K = checked(a[1], at::kBFloat16), &V = checked(a[2], at::kBFloat16);
+        const at::Tensor& K = checked(a[1], at::kBFloat16);
         if (K.dim() != 3) throw Decline{};
+        const at::Tensor& V = sized(a[2], at::kBFloat16, K.numel());
         const int Hkv = narrow(K.size(0)), L = narrow(K.size(1)), d = narrow(K.size(2));
         const int Hq = integer(a[3]), w = integer(a[4]), c = integer(a[5]), budget = integer(a[6]);
         const int n_max = chunkkv_out_len_alg1(L, w, c, budget);
         if (n_max < 0) throw Decline{};
         const long long n_row = static_cast<long long>(Hkv) * n_max;
+        const at::Tensor& q = sized(a[0], at::kBFloat16, static_cast<long long>(Hq) * w * d);
         room(chunkkv_workspace_bytes(L, Hq, Hkv, d, w, c));
         void* s = stream_of(a[10]);
         Ref oK, oV, oI;
@@ -247,7 +252,7 @@ PyObject* window_queries(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor &x = checked(a[0], at::kBFloat16), &co = checked(a[5], at::kFloat), &si = checked(a[6], at::kFloat);
         if (x.dim() != 2) throw Decline{};
         const int T = narrow(x.size(0)), Hq = integer(a[1]), Hkv = integer(a[2]), d = integer(a[3]), w = integer(a[4]);
-        if (Hq < 0 || w < 0 || d < 0) throw Decline{};
+        if (Hq < 0 || w < 0 || d < 0 || co.numel() < static_cast<long long>(w) * (d / 2) || si.numel() < static_cast<long long>(w) * (d / 2)) throw Decline{};
         const long long row = x.size(1);
         void* s = stream_of(a[7]);
         Ref out;
@@ -269,6 +274,7 @@ PyObject* score(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int Hq = narrow(q.size(0)), d = narrow(q.size(2)), Hkv = narrow(K.size(0)), L = narrow(K.size(1));
         const int w = integer(a[2]), c = integer(a[3]), C = chunkkv_num_chunks(L, w, c);
         if (C < 0 || !PyBool_Check(a[4])) throw Decline{};
+        if (q.numel() < static_cast<long long>(Hq) * w * d || K.numel() < static_cast<long long>(Hkv) * L * d) throw Decline{};
         const bool tokens = a[4] == Py_True;
         room(chunkkv_workspace_bytes(L, Hq, Hkv, d, w, c));
         if (tokens) room(chunkkv_workspace_bytes(L, Hq, Hkv, d, w, 1));
@@ -302,6 +308,7 @@ PyObject* model(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const Items layers(a[0]);
         const bool strided = a[8] == Py_True;
         if (layers.n < 1) throw Decline{};
+        const int Hq = integer(a[1]), w = integer(a[2]);
         std::vector<const void*> q(layers.n), k(layers.n), v(layers.n);
         std::vector<void*> oK(layers.n), oV(layers.n);
         std::vector<int32_t*> oI(layers.n);
@@ -323,9 +330,9 @@ PyObject* model(PyObject*, PyObject* const* a, Py_ssize_t n) {
                 }
                 (j == 1 ? k : v)[i] = x.data_ptr();
             }
-            q[i] = t.p[0] == Py_None ? nullptr : checked(t.p[0], at::kBFloat16).data_ptr();
+            q[i] = t.p[0] == Py_None ? nullptr : sized(t.p[0], at::kBFloat16, static_cast<long long>(Hq) * w * d).data_ptr();
         }
-        const int Hq = integer(a[1]), w = integer(a[2]), c = integer(a[3]), budget = integer(a[4]), n_reuse = integer(a[5]);
+        const int c = integer(a[3]), budget = integer(a[4]), n_reuse = integer(a[5]);
         const int n_max = chunkkv_out_len(L, w, c, budget);
         if (n_max < 0) throw Decline{};
         const long long n_row = static_cast<long long>(Hkv) * n_max;

@@ -93,6 +93,56 @@ def test_given_outputs_are_checked():
              {"out_K": [Fake(Hkv, n - 1, d)], "out_V": [Fake(Hkv, n, d, cuda=False)]})
 
 
+def test_inputs_that_are_too_small_are_refused():
+    Hq, Hkv, d, L, w, c, budget, n = 8, 2, 64, 300, 16, 10, 100, 96
+    assert ck.out_len(L, w, c, budget) == n
+    i32, f32 = torch.int32, torch.float32
+    good = dict(q_obs=Fake(Hq, w, d), K=Fake(Hkv, L, d), V=Fake(Hkv, L, d))
+    bad = {"q_obs": [Fake(Hq, w - 1, d)], "V": [Fake(Hkv, L - 1, d), Fake(1, L, d)]}
+    sizes = (Hq, w, c, budget)
+    for call in (ck.compress_layer, ck.compress_layer_strided, ck.compress_layer_alg1):
+        _refused(lambda q_obs, K, V: call(q_obs, K, V, *sizes), good, bad)
+    for call in (ck.compress_layer, ck.compress_layer_strided):
+        _refused(lambda reuse_idx: call(None, good["K"], good["V"], *sizes, reuse_idx=reuse_idx), dict(reuse_idx=Fake(Hkv, n, dtype=i32)),
+                 {"reuse_idx": [Fake(Hkv, n - 1, dtype=i32)]})
+    for call in (ck.compress_model, ck.compress_model_strided):
+        _refused(lambda q_obs, K, V: call([(q_obs, K, V)], *sizes), good, {"q_obs": bad["q_obs"]})
+    _refused(lambda q_obs, K: ck.score(q_obs, K, w, c), dict(q_obs=good["q_obs"], K=good["K"]), {"q_obs": bad["q_obs"], "K": [Fake(Hkv, L, d - 1)]})
+    _refused(lambda V, idx: ck.gather(good["K"], V, idx), dict(V=good["V"], idx=Fake(Hkv, n, dtype=i32)), {"V": bad["V"], "idx": [Fake(1, n, dtype=i32)]})
+    _refused(lambda cos_rows, sin_rows: ck.window_queries(Fake(L, (Hq + 2 * Hkv) * d), Hq, Hkv, d, w, cos_rows, sin_rows),
+             dict(cos_rows=Fake(w, d // 2, dtype=f32), sin_rows=Fake(w, d // 2, dtype=f32)),
+             {"cos_rows": [Fake(w - 1, d // 2, dtype=f32)], "sin_rows": [Fake(w - 1, d // 2, dtype=f32)]})
+    table, cache = Fake(6, dtype=i32), lambda h=Hkv: Fake(9, 16, h, d)
+    _refused(lambda V, block_table, cache_V: ck.gather_paged(good["K"], V, Fake(Hkv, n, dtype=i32), block_table, cache(), cache_V),
+             dict(V=good["V"], block_table=table, cache_V=cache()), {"V": bad["V"], "block_table": [Fake(5, dtype=i32)], "cache_V": [cache(1)]})
+    _refused(lambda V, block_table, cache_V: ck.compress_model_paged([(good["q_obs"], good["K"], V)], *sizes, [block_table], [(cache(), cache_V)]),
+             dict(V=good["V"], block_table=table, cache_V=cache()), {"V": bad["V"], "block_table": [Fake(5, dtype=i32)], "cache_V": [cache(1)]})
+
+
+@pytest.mark.gpu
+def test_native_calls_decline_inputs_that_are_too_small():
+    Hq, Hkv, d, L, w, c, budget = 8, 2, 64, 300, 16, 10, 100
+    n, bf = ck.out_len(L, w, c, budget), torch.bfloat16
+    ck.set_workspace(torch.empty(64 << 20, dtype=torch.uint8, device="cuda"))
+    z = lambda *s, dtype=bf: torch.zeros(*s, dtype=dtype, device="cuda")
+    q, K, V, sizes, N = z(Hq, w, d), z(Hkv, L, d), z(Hkv, L, d), (Hq, w, c, budget), binding._native
+    idx, ang = z(Hkv, n, dtype=torch.int32), z(w, d // 2, dtype=torch.float32)
+    less = lambda t: t.flatten()[:-1].contiguous()
+    few = z(Hq, w - 1, d)
+    for call, args in ((lambda *a: N.layer(*a, *sizes, None, None, None, None, None), (q, K, V)), (lambda *a: N.layer_alg1(*a, *sizes, None, None, None, None), (q, K, V)),
+                       (lambda r: N.layer(None, K, V, *sizes, r, None, None, None, None), (idx,)), (lambda q: N.score(q, K, w, c, True, None), (q,)),
+                       (lambda a, b: N.window_queries(z(L, (Hq + 2 * Hkv) * d), Hq, Hkv, d, w, a, b, None), (ang, ang))):
+        assert call(*args) is not None
+        for i, t in enumerate(args):
+            if t is not K:
+                small = few if t is q else less(t)
+                assert call(*[small if j == i else x for j, x in enumerate(args)]) is None, i
+    for strided in (False, True):
+        assert N.model([(q, K, V)], *sizes, 1, None, None, strided) is not None and N.model([(few, K, V)], *sizes, 1, None, None, strided) is None
+    assert N.layer_strided(q, K, V[:, 1:], *sizes, None, None, None, None, None) is None
+    assert ck.device_status() == 0
+
+
 @pytest.mark.gpu
 def test_native_calls_decline_outputs_that_the_general_way_refuses():
     Hq, Hkv, d, L, w, c, budget = 8, 2, 64, 300, 16, 10, 100
