@@ -18,6 +18,7 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <climits>
+#include <memory>
 #include <vector>
 
 #include "../../include/chunkkv.h"
@@ -96,12 +97,14 @@ struct Ref {                             // an owned reference
     }
 };
 
+// Runs `call` without the interpreter lock, which is held again however it ends.
 template <class Call>
 int unlocked(Call call) {
-    PyThreadState* save = PyEval_SaveThread();
-    const int st = call();
-    PyEval_RestoreThread(save);
-    return st;
+    struct Unlock {
+        PyThreadState* save = PyEval_SaveThread();
+        ~Unlock() { PyEval_RestoreThread(save); }
+    } unlock;
+    return call();
 }
 
 // Runs `body`, which returns a new reference; None for what it declines. (A C++ exception is one of torch's about a tensor: the
@@ -291,14 +294,18 @@ PyObject* score(PyObject*, PyObject* const* a, Py_ssize_t n) {
     });
 }
 
-// The items of a list or tuple, borrowed.
+// The items of a list or tuple as they are now, with a reference to each: an allocation can run Python code (a dispatch mode, a
+// finalizer), which may change the list.
 struct Items {
+    Ref own;
     PyObject** p;
     Py_ssize_t n;
     explicit Items(PyObject* o) {
         if (!PyList_CheckExact(o) && !PyTuple_CheckExact(o)) throw Decline{};
-        p = PySequence_Fast_ITEMS(o);
-        n = PySequence_Fast_GET_SIZE(o);
+        own.p = PySequence_Tuple(o);
+        if (own.p == nullptr) throw Decline{};
+        p = PySequence_Fast_ITEMS(own.p);
+        n = PySequence_Fast_GET_SIZE(own.p);
     }
 };
 
@@ -314,8 +321,9 @@ PyObject* model(PyObject*, PyObject* const* a, Py_ssize_t n) {
         std::vector<int32_t*> oI(layers.n);
         int Hkv = 0, L = 0, d = 0;
         long long st[4] = {0, 0, 0, 0};
+        std::vector<std::unique_ptr<Items>> held;       // the layers' and the outputs' tensors, until the call has been queued
         for (Py_ssize_t i = 0; i < layers.n; ++i) {
-            const Items t(layers.p[i]);
+            const Items& t = *held.emplace_back(std::make_unique<Items>(layers.p[i]));
             if (t.n != 3) throw Decline{};
             for (int j = 1; j < 3; ++j) {
                 const at::Tensor& x = strided ? tensor(t.p[j]) : checked(t.p[j], at::kBFloat16);
@@ -345,7 +353,7 @@ PyObject* model(PyObject*, PyObject* const* a, Py_ssize_t n) {
         res.p = PyList_New(layers.n);
         if (res.p == nullptr) throw Decline{};
         if (a[7] == Py_None) {
-            const at::Tensor& like = tensor(Items(layers.p[0]).p[1]);
+            const at::Tensor& like = tensor(held[0]->p[1]);
             for (Py_ssize_t i = 0; i < layers.n; ++i) {
                 Ref x, y, z;
                 oK[i] = x.set(Py_None, at::kBFloat16, 0, [&] { return rows(like, Hkv, n_max, d); });
@@ -360,7 +368,7 @@ PyObject* model(PyObject*, PyObject* const* a, Py_ssize_t n) {
             if (outs.n != layers.n) throw Decline{};
             for (Py_ssize_t i = 0; i < layers.n; ++i) {
                 if (!PyTuple_CheckExact(outs.p[i])) throw Decline{};
-                const Items o(outs.p[i]);
+                const Items& o = *held.emplace_back(std::make_unique<Items>(outs.p[i]));
                 if (o.n != 3) throw Decline{};
                 oK[i] = sized(o.p[0], at::kBFloat16, n_row * d).data_ptr();
                 oV[i] = sized(o.p[1], at::kBFloat16, n_row * d).data_ptr();

@@ -2,6 +2,7 @@
 import numpy as np
 import pytest
 import torch
+from torch.utils._python_dispatch import TorchDispatchMode
 
 import paper_2502_00299_b200 as ck
 from paper_2502_00299_b200 import binding
@@ -254,4 +255,33 @@ def test_native_errors_and_growing_scratch():
     assert binding._workspaces[torch.cuda.current_device()].numel() > 8192
     for x, y in zip(ck.compress_layer(q, K, V, 8, 16, 10, 100), want):
         assert torch.equal(x, y)
+    assert ck.device_status() == 0
+
+
+class _Empties(TorchDispatchMode):
+    """Empties a list when a tensor is allocated."""
+
+    def __init__(self, victim):
+        super().__init__()
+        self.victim, self.hits = victim, 0
+
+    def __torch_dispatch__(self, func, types, args=(), kwargs=None):
+        if "empty" in str(func):
+            self.hits += 1
+            self.victim.clear()
+        return func(*args, **(kwargs or {}))
+
+
+@pytest.mark.gpu
+def test_layers_list_that_changes_while_outputs_are_allocated():
+    g = torch.Generator(device="cuda").manual_seed(7)
+    make = lambda *s: torch.randn(*s, device="cuda", generator=g).to(torch.bfloat16)
+    xs = [(make(8, 16, 64), make(2, 900, 64), make(2, 900, 64)) for _ in range(3)]
+    ck.set_workspace(torch.empty(64 << 20, dtype=torch.uint8, device="cuda"))
+    want = ck.compress_model(xs, 8, 16, 10, 100)
+    layers = [list(x) for x in xs]
+    with _Empties(layers) as mode:
+        got = binding._native.model(layers, 8, 16, 10, 100, 1, None, None, False)
+    assert mode.hits == 9 and layers == [] and len(got) == 3
+    assert all(torch.equal(a, b) for x, y in zip(got, want) for a, b in zip(x, y))
     assert ck.device_status() == 0
