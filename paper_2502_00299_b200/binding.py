@@ -176,6 +176,7 @@ def workspace_bytes(L: int, Hq: int, Hkv: int, d: int, w: int, c: int) -> int:
 
 
 _workspaces = {}      # device index -> uint8 tensor currently handed to the library
+_native.scratch(_workspaces)
 
 
 def set_workspace(buf: Optional[torch.Tensor]) -> None:
@@ -185,12 +186,10 @@ def set_workspace(buf: Optional[torch.Tensor]) -> None:
     if buf is None:
         _check(lib.chunkkv_set_workspace(None, 0), "chunkkv_set_workspace")
         _workspaces.pop(dev, None)
-        _native.note_workspace(dev, 0)
     else:
         _check(lib.chunkkv_set_workspace(buf.data_ptr(), buf.numel() * buf.element_size()),
                "chunkkv_set_workspace")
         _workspaces[dev] = buf
-        _native.note_workspace(dev, buf.numel())
 
 
 def ensure_workspace(L: int, Hq: int, Hkv: int, d: int, w: int, c: int) -> None:

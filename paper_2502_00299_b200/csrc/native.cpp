@@ -8,7 +8,7 @@
 // They take what programs normally pass - plain tensors and plain ints - and answer None for everything else (subclasses,
 // other number types, tensors that fail a check, a scratch buffer that has to grow, an active torch-function mode), before
 // anything is queued: the Python function then goes its general way, which raises the errors. A status of the C ABI other
-// than 0 is returned as an int. Nothing is kept between calls but the size of the scratch that each device was given.
+// than 0 is returned as an int. Nothing is kept between calls but the dict in which the binding keeps its scratch tensors.
 #include <Python.h>
 
 #include <ATen/ATen.h>
@@ -25,8 +25,7 @@
 
 namespace {
 
-constexpr int kMaxDevices = 64;
-long long g_ws_bytes[kMaxDevices];       // scratch handed to the library per device (under the interpreter lock)
+PyObject* g_scratch = nullptr;           // the binding's dict of the scratch tensors handed to the library, by device
 
 // What a call cannot take: the caller returns None.
 struct Decline {};
@@ -68,8 +67,11 @@ void* stream_of(PyObject* o) {
     return s;
 }
 void room(size_t need) {
-    const int dev = c10::cuda::current_device();
-    if (need == 0 || dev < 0 || dev >= kMaxDevices || g_ws_bytes[dev] < static_cast<long long>(need)) throw Decline{};
+    PyObject* dev = g_scratch != nullptr && need > 0 ? PyLong_FromLong(c10::cuda::current_device()) : nullptr;
+    if (dev == nullptr) throw Decline{};
+    PyObject* buf = PyDict_GetItemWithError(g_scratch, dev);       // (borrowed)
+    Py_DECREF(dev);
+    if (buf == nullptr || !THPVariable_Check(buf) || THPVariable_Unpack(buf).numel() < static_cast<long long>(need)) throw Decline{};
 }
 at::Tensor rows(const at::Tensor& like, long long heads, long long n, long long d) {
     return at::empty({heads, n, d}, at::TensorOptions().dtype(at::kBFloat16).device(like.device()));
@@ -124,14 +126,16 @@ PyObject* guarded(Py_ssize_t n, Py_ssize_t want, Body body) {
     }
 }
 
-// note_workspace(device, bytes)
-PyObject* note_workspace(PyObject*, PyObject* const* a, Py_ssize_t n) {
-    if (n != 2) { PyErr_SetString(PyExc_TypeError, "2 arguments expected"); return nullptr; }
-    const long dev = PyLong_AsLong(a[0]);
-    const long long bytes = PyLong_AsLongLong(a[1]);
-    if (PyErr_Occurred()) return nullptr;
-    if (dev >= 0 && dev < kMaxDevices) g_ws_bytes[dev] = bytes;
-    Py_RETURN_NONE;
+// scratch(dict): the dict in which the binding keeps the scratch tensors; returns the one in use
+PyObject* scratch(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (n > 1 || (n == 1 && !PyDict_CheckExact(a[0]))) { PyErr_SetString(PyExc_TypeError, "a dict expected"); return nullptr; }
+    if (n == 1) {
+        Py_INCREF(a[0]);
+        Py_XSETREF(g_scratch, a[0]);
+    }
+    PyObject* r = g_scratch != nullptr ? g_scratch : Py_None;
+    Py_INCREF(r);
+    return r;
 }
 
 // layer(q_obs, K, V, Hq, w, c, budget, reuse_idx, out_K, out_V, out_idx, stream) -> (out_K, out_V, out_idx)
@@ -391,7 +395,7 @@ PyObject* model(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 PyMethodDef kMethods[] = {
 #define CKV_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(name)), METH_FASTCALL, nullptr}
-    CKV_METHOD(note_workspace), CKV_METHOD(layer), CKV_METHOD(layer_strided), CKV_METHOD(layer_alg1), CKV_METHOD(layer_paged),
+    CKV_METHOD(scratch), CKV_METHOD(layer), CKV_METHOD(layer_strided), CKV_METHOD(layer_alg1), CKV_METHOD(layer_paged),
     CKV_METHOD(window_queries), CKV_METHOD(score), CKV_METHOD(model), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_native", "Per-call part of the binding (see binding.py).", -1, kMethods, nullptr, nullptr, nullptr, nullptr};
 

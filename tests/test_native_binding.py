@@ -1,4 +1,8 @@
 """The binding's native calls (csrc/native.cpp): what they decline goes the general way, and both ways give the same results."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -7,6 +11,7 @@ from torch.utils._python_dispatch import TorchDispatchMode
 import paper_2502_00299_b200 as ck
 from paper_2502_00299_b200 import binding
 
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CALLS = ("layer", "layer_strided", "layer_alg1", "layer_paged", "window_queries", "score", "model")
 
 
@@ -285,3 +290,10 @@ def test_layers_list_that_changes_while_outputs_are_allocated():
     assert mode.hits == 9 and layers == [] and len(got) == 3
     assert all(torch.equal(a, b) for x, y in zip(got, want) for a, b in zip(x, y))
     assert ck.device_status() == 0
+
+
+def test_scratch_is_looked_up_where_the_binding_keeps_it():
+    # (loaded again, the binding has no scratch, and the native calls must not take the old one for granted)
+    code = ("import importlib; from paper_2502_00299_b200 import binding as b; t = b._native.scratch(); assert t is b._workspaces; "
+            "b = importlib.reload(b); assert b._native.scratch() is b._workspaces is not t")
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
