@@ -1,14 +1,19 @@
 """Binding of the C ABI declared in include/chunkkv.h (argument marshalling only).
 
 Calls that a program makes per layer or per model go through ``_native`` (csrc/native.cpp), which answers None for arguments
-other than plain tensors and ints and for whatever fails a check; those, and all other calls, go through ctypes here."""
+other than plain tensors and ints and for whatever fails a check; those, and all other calls, go through ctypes here. Without that
+module (built for another torch or Python) every call does."""
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
+import warnings
 from typing import List, Optional, Sequence, Tuple
 
 import torch
+
+from .build import native_path
 
 LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libchunkkv.so")
 
@@ -112,7 +117,28 @@ def _load() -> ctypes.CDLL:
 
 lib = _load()
 
-from . import _native  # noqa: E402  (linked against the library loaded above)
+class _General:
+    """In the place of the extension module: declines every call."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
+def _load_native():
+    """The extension module (it is linked against the library loaded above)."""
+    path = native_path()
+    try:
+        spec = importlib.util.spec_from_file_location(f"{__package__}._native", path)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        return mod
+    except ImportError as e:
+        warnings.warn(f"{path} cannot be loaded ({e}): calls take about 15 us longer on the host. Build it with "
+                      "`python -m paper_2502_00299_b200.build`.", RuntimeWarning)
+        return _General()
+
+
+_native = _load_native()
 
 
 def _check(status: int, where: str) -> None:

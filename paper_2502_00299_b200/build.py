@@ -16,13 +16,18 @@ PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 BUILD_DIR = os.path.join(PKG_DIR, "_build")
 LIB_PATH = os.path.join(PKG_DIR, "libchunkkv.so")
-NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")      # extension module used by binding.py
 INCLUDE_DIR = os.path.join(os.path.dirname(PKG_DIR), "include")
 SOURCES = ("api.cu", "score.cu", "layer_resident.cu", "model_kernel.cu", "token_kernel.cu", "select.cu", "select_cluster.cu", "gather.cu", "diagnostics.cu", "score_noalloc.cu")
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
     "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "--expt-relaxed-constexpr",
 ]
+
+
+def native_path() -> str:
+    """The extension module used by binding.py. Its name holds the versions of torch and Python that it was built for and that run now."""
+    import torch
+    return os.path.join(PKG_DIR, f"_native-torch{torch.__version__}{sysconfig.get_config_var('EXT_SUFFIX')}")
 
 
 def _nvcc() -> str:
@@ -39,7 +44,7 @@ def _deps_mtime() -> float:
 
 
 def is_current() -> bool:
-    return all(os.path.exists(p) and os.path.getmtime(p) >= _deps_mtime() for p in (LIB_PATH, NATIVE_PATH))
+    return all(os.path.exists(p) and os.path.getmtime(p) >= _deps_mtime() for p in (LIB_PATH, native_path()))
 
 
 def _compile_native() -> str:
@@ -60,11 +65,14 @@ def _compile_native() -> str:
 def _link_native(obj: str) -> None:
     import torch
     lib = os.path.join(os.path.dirname(os.path.abspath(torch.__file__)), "lib")
-    cmd = ["g++", "-shared", "-o", NATIVE_PATH, obj, "-L", PKG_DIR, "-l:libchunkkv.so", "-Wl,-rpath,$ORIGIN", "-L", lib, "-ltorch_python", "-ltorch",
+    for f in os.listdir(PKG_DIR):                      # of other versions
+        if f.startswith("_native") and f.endswith(".so"):
+            os.remove(os.path.join(PKG_DIR, f))
+    cmd = ["g++", "-shared", "-o", native_path(), obj, "-L", PKG_DIR, "-l:libchunkkv.so", "-Wl,-rpath,$ORIGIN", "-L", lib, "-ltorch_python", "-ltorch",
            "-ltorch_cpu", "-lc10", "-lc10_cuda"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
-        raise RuntimeError(f"link of _native.so failed:\n{res.stdout}\n{res.stderr}")
+        raise RuntimeError(f"link of {native_path()} failed:\n{res.stdout}\n{res.stderr}")
 
 
 def _compile(src: str, verbose: bool) -> str:

@@ -9,7 +9,7 @@ import torch
 from torch.utils._python_dispatch import TorchDispatchMode
 
 import paper_2502_00299_b200 as ck
-from paper_2502_00299_b200 import binding
+from paper_2502_00299_b200 import binding, build
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CALLS = ("layer", "layer_strided", "layer_alg1", "layer_paged", "window_queries", "score", "model")
@@ -297,3 +297,14 @@ def test_scratch_is_looked_up_where_the_binding_keeps_it():
     code = ("import importlib; from paper_2502_00299_b200 import binding as b; t = b._native.scratch(); assert t is b._workspaces; "
             "b = importlib.reload(b); assert b._native.scratch() is b._workspaces is not t")
     subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
+
+
+def test_without_the_native_part_calls_go_the_general_way(monkeypatch):
+    monkeypatch.setattr(torch, "__version__", "0.0.1")              # built for another torch
+    assert not build.is_current()
+    with pytest.warns(RuntimeWarning, match="paper_2502_00299_b200.build"):
+        none = binding._load_native()
+    for name in CALLS:
+        assert getattr(none, name)(1, 2, 3) is None
+    monkeypatch.undo()
+    assert binding._load_native().scratch.__name__ == "scratch" and build.is_current()
