@@ -15,7 +15,7 @@ constexpr size_t kSelBytes = (sizeof(SelectSmem) + 127) & ~size_t(127);
 __global__ void __launch_bounds__(kSelThreads)
 select_kernel(const float* __restrict__ scores, int L, int w, int c, int C, int k, int n_max,
               int32_t* __restrict__ out_idx, int key_bytes, bool staged, int tok_cap) {
-    extern __shared__ uint8_t smem_raw[];
+    extern __shared__ __align__(128) uint8_t smem_raw[];      // (SelectSmem is read 16 bytes at a time)
     SelectSmem& sm = *reinterpret_cast<SelectSmem*>(smem_raw);
     uint32_t* kbuf = reinterpret_cast<uint32_t*>(smem_raw + kSelBytes);
     const int h = blockIdx.x;
@@ -38,7 +38,7 @@ cudaError_t launch_select(const float* scores, int L, int Hkv, int w, int c, int
         select_kernel<<<Hkv, kSelThreads, kSelBytes, stream>>>(scores, L, w, c, C, k, n_max, out_idx, 0, true, tok_cap);
         return cudaGetLastError();
     }
-    // more: the keys of a head live in dynamic shared memory if they fit beside the static scratch
+    // more: the keys of a head live in dynamic shared memory if they fit behind the selection scratch
     // (beyond the 48 KB every kernel may use, so the kernel opts in), else they are recomputed
     const size_t want = static_cast<size_t>(C) * 4;
     int key_bytes = 0, dev = 0, optin = 0;
