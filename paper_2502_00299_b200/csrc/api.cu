@@ -310,12 +310,13 @@ int run_score(DeviceCtx& ctx, const void* q_obs, const void* K, int L, int Hq, i
 
 // Scratch floats of the scoring kernels for a shape: the larger of the score-only launch and the
 // fused layer launch (which always uses one CTA per SM and so may keep more per-CTA records).
-size_t scratch_floats_for(const DeviceCtx& ctx, int L, int R, int Hkv, int d, int c) {
+// reserve: never less for a longer sequence.
+size_t scratch_floats_for(const DeviceCtx& ctx, int L, int R, int Hkv, int d, int c, bool reserve) {
     ScorePlan plan;
     size_t n = 0;
     for (int full = 0; full < 2; ++full) {
         if (!make_score_plan(L, R, Hkv, d, c, ctx.num_sms, smem_budget(ctx), full != 0, &plan)) return 0;
-        const size_t f = score_scratch_floats(plan, Hkv, R);
+        const size_t f = reserve ? score_reserve_floats(plan, Hkv, R, ctx.num_sms) : score_scratch_floats(plan, Hkv, R);
         n = f > n ? f : n;
     }
     return n;
@@ -323,10 +324,10 @@ size_t scratch_floats_for(const DeviceCtx& ctx, int L, int R, int Hkv, int d, in
 
 // Bytes of scratch of the calls that score with the kernels of score.cu: the chunk scores of the KV heads, those of the
 // scoring heads, and the kernels' own scratch.
-size_t score_path_bytes(const DeviceCtx& ctx, int L, int Hq, int Hkv, int d, int w, int c) {
+size_t score_path_bytes(const DeviceCtx& ctx, int L, int Hq, int Hkv, int d, int w, int c, bool reserve = false) {
     const ScoreShape sh = score_shape(Hq, Hkv, w);
     const int C = (L - w + c - 1) / c;
-    const size_t floats = scratch_floats_for(ctx, L, sh.Rs, sh.Hs, d, c) + round64(static_cast<size_t>(Hkv) * C) +
+    const size_t floats = scratch_floats_for(ctx, L, sh.Rs, sh.Hs, d, c, reserve) + round64(static_cast<size_t>(Hkv) * C) +
                           round64(static_cast<size_t>(sh.Hs) * C);
     return kHeaderBytes + floats * sizeof(float);
 }
@@ -890,14 +891,27 @@ size_t chunkkv_model_workspace_bytes(int n_layers, int L, int Hq, int Hkv, int d
     std::lock_guard<std::mutex> lk(g_mu);
     DeviceCtx* ctx;
     if (get_ctx(&ctx) != CHUNKKV_OK) return 0;
-    const int C = (L - w + c - 1) / c;
-    const int k = chunkkv_num_kept_chunks(L, w, c, budget);
-    ModelPlan mp;
-    size_t need = per_layer;
-    if (C > 0 && k > 0 && make_model_plan(L, w * (Hq / Hkv), Hkv, d, c, C, k, ctx->num_sms, smem_budget(*ctx), &mp)) {
-        const size_t m = kHeaderBytes + model_scratch_floats(mp, Hkv, C, model_launch_computes(n_layers, reuse_depth), true) * sizeof(float);
-        need = m > need ? m : need;
+    // never less for a longer sequence: see score_reserve_floats and model_reserve_floats
+    const size_t score_path = score_path_bytes(*ctx, L, Hq, Hkv, d, w, c, true);
+    auto persistent = [&](int len) {
+        const int C = (len - w + c - 1) / c, k = chunkkv_num_kept_chunks(len, w, c, budget);
+        return C > 0 && k > 0 ? model_reserve_floats(len, w * (Hq / Hkv), Hkv, d, c, C, k, ctx->num_sms, smem_budget(*ctx),
+                                                     model_launch_computes(n_layers, reuse_depth))
+                              : 0;
+    };
+    size_t floats = persistent(L);
+    if (floats == 0 && L > w && persistent(w + 1) > 0) {
+        // the persistent kernel takes shorter sequences only (its limits on chunks): the longest of them
+        int fits = w + 1, fails = L;
+        while (fails - fits > 1) {
+            const int mid = fits + (fails - fits) / 2;
+            (persistent(mid) > 0 ? fits : fails) = mid;
+        }
+        floats = persistent(fits);
     }
+    size_t need = per_layer > score_path ? per_layer : score_path;
+    const size_t m = floats > 0 ? kHeaderBytes + floats * sizeof(float) : 0;
+    need = m > need ? m : need;
     return need;
 }
 

@@ -53,6 +53,8 @@ bool make_score_plan(int L, int R, int Hkv, int d, int c, int num_sms, int smem_
 
 // Scratch floats needed for a plan (panel maxima + CTA records + partial sums), per layer.
 size_t score_scratch_floats(const ScorePlan& plan, int Hkv, int R);
+// At least that, and never smaller for a longer sequence.
+size_t score_reserve_floats(const ScorePlan& plan, int Hkv, int R, int num_sms);
 
 // Points the scratch pointers of `args` into `base` (score_scratch_floats floats).
 void score_scratch_layout(const ScorePlan& plan, int Hkv, int R, float* base, ScoreArgs* args);
@@ -164,9 +166,12 @@ struct ModelLayerIO {
     bool computes;        // false: gather with the indices of the nearest computed layer before it
 };
 
-bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, ModelPlan* plan);
-// What a launch uses; with `reserve` what a caller is told to provide, which a shorter sequence never exceeds.
-size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute, bool reserve = false);
+// n_sel: selector CTAs (0: as many as are best).
+bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, ModelPlan* plan, int n_sel = 0);
+// What a launch uses.
+size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute);
+// What a caller is told to provide, which a shorter sequence never exceeds; 0 for a shape that the kernel does not take.
+size_t model_reserve_floats(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, int n_compute);
 // layers[0] must compute; tm_q / tm_k hold one tensor map per computed layer, in order; tm_rk / tm_rv one per layer (boxes
 // of one chunk's rows) where keys and values are not packed, else NULL.
 cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtensorMap* tm_q, const CUtensorMap* tm_k,

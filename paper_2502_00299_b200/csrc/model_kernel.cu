@@ -942,7 +942,12 @@ model_kernel(const __grid_constant__ ModelParams p) {
 
 }  // namespace
 
-bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, ModelPlan* plan) {
+// Tiles up to which five to eight heads have a selector CTA each (see make_model_plan).
+static int selector_each_tiles(int Hkv, int max_ctas) {
+    return Hkv > 4 && Hkv <= 8 && max_ctas >= 2 * Hkv ? 6 * ((max_ctas - Hkv) / Hkv) : 0;
+}
+
+bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, ModelPlan* plan, int n_sel) {
     // the chunk sizes that are compiled in, as in layer_resident.cu
     if (c != 5 && c != 8 && c != 10 && c != 16 && c != 20 && c != 32) return false;
     if (R < 1 || R > 256 || (d != 64 && d != 128) || L < 1 || C < 1 || k < 1 || Hkv < 1 || Hkv > kResidentMaxHeads)
@@ -961,7 +966,8 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_
     // Five to eight heads on short contexts: a selector each. With two heads a selector the two selections (about 5k clocks each)
     // are longer than the scoring of a layer up to six tiles a CTA, and the scoring CTA a head gives up costs less: 32 layers of
     // 4096 tokens 309 -> 287 us, 16 of 7000 (256 rows) 192 -> 183, 16 of 2100 157 -> 145, 16 of 11000 (indices shared by two) 121 -> 114.
-    if (Hkv > 4 && Hkv <= 8 && max_ctas >= 2 * Hkv && p.n_tiles <= 6 * ((max_ctas - Hkv) / Hkv)) p.n_sel = Hkv;
+    if (p.n_tiles <= selector_each_tiles(Hkv, max_ctas)) p.n_sel = Hkv;
+    if (n_sel > 0) p.n_sel = n_sel;
     if (max_ctas - p.n_sel < Hkv) p.n_sel = max_ctas - Hkv;
     p.cph = (max_ctas - p.n_sel) / Hkv;
     if (p.cph > p.n_tiles) p.cph = p.n_tiles;
@@ -1025,10 +1031,29 @@ static size_t model_spill_floats(const ModelPlan& plan, int ring) {
     return ((ring - plan.ring_on) * n_w + 4 * (4 - n_w)) * (plan.spp + 1) * 32;
 }
 
-size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute, bool reserve) {
+static size_t model_floats(const ModelPlan& plan, int Hkv, int C, int n_compute, int ring) {
     return static_cast<size_t>(2) * plan.grid * plan.n_mt * 256 + static_cast<size_t>(n_compute) * Hkv * plan.n_mt * ((C + 3) & ~3) +
            static_cast<size_t>(n_compute) * Hkv * (plan.sel_row_bytes / 4) + 64 +
-           static_cast<size_t>(plan.n_score) * model_spill_floats(plan, reserve ? plan.ring_reserve : plan.ring);
+           static_cast<size_t>(plan.n_score) * model_spill_floats(plan, ring);
+}
+
+size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute) {
+    return model_floats(plan, Hkv, C, n_compute, plan.ring);
+}
+
+size_t model_reserve_floats(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, int n_compute) {
+    // A grid with a given number of selectors never shrinks for a longer sequence, nor does its ring_reserve; the two numbers of
+    // selectors that a shorter sequence may have are both provided for.
+    size_t need = 0;
+    ModelPlan p;
+    if (make_model_plan(L, R, Hkv, d, c, C, k, max_ctas, smem_limit, &p, Hkv < 4 ? Hkv : 4))
+        need = model_floats(p, Hkv, C, n_compute, p.ring_reserve);
+    const long long each = static_cast<long long>(selector_each_tiles(Hkv, max_ctas)) * 2 * panel_keys(c);
+    if (each > 0 && make_model_plan(each < L ? static_cast<int>(each) : L, R, Hkv, d, c, C, k, max_ctas, smem_limit, &p, Hkv)) {
+        const size_t m = model_floats(p, Hkv, C, n_compute, p.ring_reserve);
+        need = m > need ? m : need;
+    }
+    return need;
 }
 
 template <int C_STATIC>

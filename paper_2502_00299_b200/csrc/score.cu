@@ -1084,6 +1084,14 @@ size_t score_scratch_floats(const ScorePlan& plan, int Hkv, int R) {
            static_cast<size_t>(Hkv) * 512 + panels * plan.spp * R;
 }
 
+size_t score_reserve_floats(const ScorePlan& plan, int Hkv, int R, int num_sms) {
+    // The records of the CTAs (grid * hs_max of them) for the largest grid and the most heads a CTA that any length has: between
+    // 15/16 of the SMs and all of them, at most 256, and one head more than divide evenly.
+    const int most = num_sms < 256 ? num_sms : 256, least = most - most / 16;
+    const size_t records = static_cast<size_t>(plan.grid) * plan.hs_max, any = static_cast<size_t>(most) * ((Hkv + least - 1) / least + 1);
+    return score_scratch_floats(plan, Hkv, R) + (any > records ? (any - records) * (kGroups * 256) : 0);
+}
+
 void score_scratch_layout(const ScorePlan& plan, int Hkv, int R, float* base, ScoreArgs* args) {
     const size_t panels = static_cast<size_t>(Hkv) * plan.n_panels;
     args->stat_m = base;

@@ -69,6 +69,28 @@ def test_model_scratch_never_shrinks_for_a_longer_sequence(ck, Hq, Hkv, w, c):
     assert all(a <= b for a, b in zip(need, need[1:])), [L for L, a, b in zip(sorted(lens)[1:], need, need[1:]) if a > b][:5]
 
 
+# Either side of the length up to which five to eight heads have a selector CTA each (6 tiles of 120 keys a CTA)
+@pytest.mark.parametrize("Hkv,L", [(5, 20160), (6, 16560), (7, 14400), (8, 12240)])
+def test_model_call_in_scratch_sized_for_a_longer_sequence(ck, Hkv, L):
+    d, w, c = 64, 8, 10
+    budget = w + c * (L // (12 * c))
+    ws = Guarded((int(ck.lib.chunkkv_model_workspace_bytes(2, L + 1, Hkv, Hkv, d, w, c, budget, 1)),), torch.uint8)
+    for n in (L, L + 1):
+        xs = [_layer(Hkv, Hkv, d, n, w, seed=n + i) for i in range(2)]
+        ck.set_workspace(None)
+        want = [ck.compress_layer(*x, Hkv, w, c, budget) for x in xs]
+        n_max = ck.out_len(n, w, c, budget)
+        outs = [(torch.empty(Hkv, n_max, d, dtype=torch.bfloat16, device="cuda"), torch.empty(Hkv, n_max, d, dtype=torch.bfloat16, device="cuda"),
+                 torch.empty(Hkv, n_max, dtype=torch.int32, device="cuda")) for _ in xs]
+        arr = ctypes.c_void_p * 2
+        ck.set_workspace(ws.t)
+        st = ck.lib.chunkkv_compress_model(2, *[arr(*[x[j].data_ptr() for x in xs]) for j in range(3)], n, Hkv, Hkv, d, w, c, budget, 1,
+                                           *[arr(*[o[j].data_ptr() for o in outs]) for j in range(3)], None)
+        assert st == 0 and ck.device_status() == 0
+        assert all(torch.equal(a, b) for o, v in zip(outs, want) for a, b in zip(o, v))
+    ws.check("model scratch")
+
+
 @pytest.mark.parametrize("Hq,c,L,refused", [(8, 10, 20000, True), (8, 20, 20000, True), (8, 16, 20000, False), (8, 5, 9000, False),
                                             (8, 10, 120000, False)])
 def test_model_call_on_a_scratch_of_the_layer_calls(ck, Hq, c, L, refused):
