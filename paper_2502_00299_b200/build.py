@@ -75,15 +75,19 @@ def _link_native(obj: str) -> None:
         raise RuntimeError(f"link of {native_path()} failed:\n{res.stdout}\n{res.stderr}")
 
 
+def report_path(src: str) -> str:
+    """What ptxas said of a source file's kernels (registers, spills, shared memory)."""
+    return os.path.join(BUILD_DIR, src.replace(".cu", ".ptxas.txt"))
+
+
 def _compile(src: str, verbose: bool) -> str:
     obj = os.path.join(BUILD_DIR, src.replace(".cu", ".o"))
-    cmd = [_nvcc(), *NVCC_FLAGS, "-I", INCLUDE_DIR, "-c", os.path.join(CSRC, src), "-o", obj]
-    if verbose:
-        cmd.insert(1, "-Xptxas")
-        cmd.insert(2, "-v")
+    cmd = [_nvcc(), *NVCC_FLAGS, "-Xptxas", "-v", "-I", INCLUDE_DIR, "-c", os.path.join(CSRC, src), "-o", obj]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError(f"nvcc failed on {src}:\n{res.stdout}\n{res.stderr}")
+    with open(report_path(src), "w") as f:
+        f.write(res.stderr)
     if verbose:
         sys.stderr.write(res.stderr)
     return obj

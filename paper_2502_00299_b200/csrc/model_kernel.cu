@@ -288,7 +288,9 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
 
 // BIG: two query tiles, or a ring that reaches into scratch. A variant of its own, so that the kernel for up to 128 rows
 // carries none of it.
-template <int C_STATIC, bool BIG>
+// FEW: up to 64 rows and more than nine CTAs a head, for the reading of row statistics. A variant of its own: as a run-time choice it
+// made the general form spill (bytes of stores / loads at c = 10: 16 / 28 instead of none, at 16: 32 / 44 instead of 20 / 20).
+template <int C_STATIC, bool BIG, bool FEW>
 __global__ void __launch_bounds__(kMThreads, 1)
 model_kernel(const __grid_constant__ ModelParams p) {
     constexpr int WP = panel_keys(C_STATIC);
@@ -766,7 +768,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
             if (!wait_counter_warp(p.cnt_a + hkv, static_cast<unsigned>(s + 1) * p.cph, abort_flag)) break;
             if constexpr (!BIG) {
                 // the head's records straight from the L2 (they were written by other SMs; every lane has
-                // acquired the counter), nine CTAs' worth of loads in flight per lane. Up to 64 rows each half of the warp
+                // acquired the counter), nine CTAs' worth of loads in flight per lane. FEW: each half of the warp
                 // takes every other record (2 heads: 69 CTAs, 32 layers of 8192 tokens 487 -> 335 us).
                 const float* src = p.cta_stat + (static_cast<size_t>(s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * 256;
                 float M[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}, S[4] = {0.f, 0.f, 0.f, 0.f};
@@ -783,7 +785,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                         merge_batch<9>(M, S, m, l, n - j0);
                     }
                 };
-                if (p.R > 64) {
+                if constexpr (!FEW) {
                     fold(src + r0, std::integral_constant<int, 256>{}, p.cph);
                 } else {
                     const int sub = lane >> 4;
@@ -1056,9 +1058,12 @@ size_t model_reserve_floats(int L, int R, int Hkv, int d, int c, int C, int k, i
     return need;
 }
 
+// 0: small, 1: big, 2: small with few rows
 template <int C_STATIC>
-static const void* model_kernel_of(bool big) {
-    return big ? reinterpret_cast<const void*>(model_kernel<C_STATIC, true>) : reinterpret_cast<const void*>(model_kernel<C_STATIC, false>);
+static const void* model_kernel_of(int variant) {
+    return variant == 1 ? reinterpret_cast<const void*>(model_kernel<C_STATIC, true, false>)
+         : variant == 2 ? reinterpret_cast<const void*>(model_kernel<C_STATIC, false, true>)
+                        : reinterpret_cast<const void*>(model_kernel<C_STATIC, false, false>);
 }
 
 cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtensorMap* tm_q, const CUtensorMap* tm_k,
@@ -1109,19 +1114,21 @@ cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtenso
     p.cnt_b = io.counters + 16 + kResidentMaxHeads;
     p.cnt_c = io.counters + 16 + 2 * kResidentMaxHeads;
     p.status = io.status;
+    // (nine records are one round trip, which half a warp does not shorten)
+    const int variant = plan.big ? 1 : (io.R <= 64 && plan.cph > 9 ? 2 : 0);
     const void* kern = nullptr;
     int v = 0;
     switch (plan.c_static) {
-        case 5: kern = model_kernel_of<5>(plan.big); v = 0; break;
-        case 8: kern = model_kernel_of<8>(plan.big); v = 1; break;
-        case 10: kern = model_kernel_of<10>(plan.big); v = 2; break;
-        case 16: kern = model_kernel_of<16>(plan.big); v = 3; break;
-        case 20: kern = model_kernel_of<20>(plan.big); v = 4; break;
-        case 32: kern = model_kernel_of<32>(plan.big); v = 5; break;
+        case 5: kern = model_kernel_of<5>(variant); v = 0; break;
+        case 8: kern = model_kernel_of<8>(variant); v = 1; break;
+        case 10: kern = model_kernel_of<10>(variant); v = 2; break;
+        case 16: kern = model_kernel_of<16>(variant); v = 3; break;
+        case 20: kern = model_kernel_of<20>(variant); v = 4; break;
+        case 32: kern = model_kernel_of<32>(variant); v = 5; break;
         default: break;
     }
-    v += plan.big ? 6 : 0;
-    static int smem_set[12][64] = {{0}};
+    v += 6 * variant;
+    static int smem_set[18][64] = {{0}};
     int dev = 0;
     cudaError_t e = kern != nullptr ? cudaGetDevice(&dev) : cudaErrorInvalidValue;
     if (e == cudaSuccess && (dev < 0 || dev >= 64 || smem_set[v][dev] < plan.smem_bytes)) {
