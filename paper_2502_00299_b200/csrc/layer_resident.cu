@@ -219,7 +219,12 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 for (int kb = 0; kb < KB; ++kb)
                     tma_load_3d(q_base + static_cast<uint32_t>(mt * KB + kb) * kRQTileBytes, &tm_q, qbar, kb * 64, row0 + mt * 128, hkv);
             const uint32_t k_bytes = static_cast<uint32_t>(min(a.L, TILE)) * 128u;
-            const uint64_t first = l2_policy_evict_first();
+            // Panels in scratch: the keys leave the L2 to their records, unless the kept key rows, which the gather reads again, are
+            // the larger part. us without -> with the hint: 131072 tokens, 256 rows, c = 20, 3 % kept (47 MB of records, 8 MB of rows) 124 -> 115;
+            // 52088 tokens, 64 rows, c = 5, 16 % (14 MB, 17 MB) 55.7 -> 54.0; 131072 tokens, 64 rows, c = 5, 25 % (48 MB, 67 MB) 146.7 -> 149.2;
+            // 120859 tokens, 128 rows, c = 20, 18 % (8 MB, 45 MB) 92.4 -> 98.3.
+            const bool keys_leave = 3ll * a.n_max * a.Hkv * a.d * 2 < 4ll * a.n_off * (SPP + 1) * a.spill_rows * 4 * gridDim.x;
+            const uint64_t policy = keys_leave ? l2_policy_evict_first() : l2_policy_evict_normal();
             uint32_t st = 0, st_par = 1;
             int issued = 0;
             bool ok = true;
@@ -229,8 +234,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                     if (!ok) break;
                     const uint32_t bar = smem_u32(&ctl.full[st]);
                     mbar_arrive_expect_tx(bar, k_bytes);
-                    // (panels in scratch: the keys leave the L2 to them; 128K tokens, 256 rows 127 -> 115 to 123 us)
-                    if (BIG && a.n_off > 0) tma_load_3d_hint(k_base + st * STAGE, &tm_k, bar, kb * 64, t * TILE, hkv, first);
+                    if constexpr (BIG) tma_load_3d_hint(k_base + st * STAGE, &tm_k, bar, kb * 64, t * TILE, hkv, policy);
                     else tma_load_3d(k_base + st * STAGE, &tm_k, bar, kb * 64, t * TILE, hkv);
                     ++issued;
                     if (++st == n_stages) { st = 0; st_par ^= 1u; }

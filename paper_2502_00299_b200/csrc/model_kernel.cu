@@ -387,7 +387,9 @@ model_kernel(const __grid_constant__ ModelParams p) {
             const uint32_t qbar = smem_u32(&ctl.qfull);
             const uint32_t q_bytes = static_cast<uint32_t>(n_mt * KB * p.q_box_rows) * 128u;
             const uint32_t k_bytes = static_cast<uint32_t>(p.k_box_rows) * 128u;
-            const uint64_t first = l2_policy_evict_first();
+            // A ring that continues in scratch: the keys leave the L2 to it (30000 tokens, 128 rows, c = 5 222 -> 217 us, 256 rows, c = 10 246 -> 241). On chip
+            // there is nothing to keep, and the row copies of the next layer read kept key rows (16000 tokens, 224 rows, c = 20, 25 % kept: 320 -> 321 us with the hint).
+            const uint64_t policy = p.ring > p.ring_on ? l2_policy_evict_first() : l2_policy_evict_normal();
             uint32_t st = 0, st_par = 1;
             int issued = 0;
             bool ok = true;
@@ -407,8 +409,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                         if (!ok) break;
                         const uint32_t bar = smem_u32(&ctl.full[st]);
                         mbar_arrive_expect_tx(bar, k_bytes);
-                        // (big variant: the keys leave the L2 to the ring in scratch; 16 layers of 30000 tokens, c = 5, 403 -> 381 us)
-                        if constexpr (BIG) tma_load_3d_hint(k_base + st * STAGE, &p.tm_k[s], bar, kb * 64, t * TILE, hkv, first);
+                        if constexpr (BIG) tma_load_3d_hint(k_base + st * STAGE, &p.tm_k[s], bar, kb * 64, t * TILE, hkv, policy);
                         else tma_load_3d(k_base + st * STAGE, &p.tm_k[s], bar, kb * 64, t * TILE, hkv);
                         ++issued;
                         if (++st == n_stages) { st = 0; st_par ^= 1u; }

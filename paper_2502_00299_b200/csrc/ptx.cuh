@@ -99,6 +99,11 @@ __device__ __forceinline__ uint64_t l2_policy_evict_first() {
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
+__device__ __forceinline__ uint64_t l2_policy_evict_normal() {
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
 // Stores and loads of scratch that is written once and read once a little later: keep it in L2
 // ahead of streamed data, and let it go once it has been read.
 __device__ __forceinline__ uint64_t l2_policy_evict_last() {
