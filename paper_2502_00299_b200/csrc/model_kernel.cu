@@ -229,7 +229,7 @@ __device__ __forceinline__ bool wait_counter(const unsigned* counter, unsigned t
 // and of every layer that reuses its indices (and zero rows behind the kept rows, which exist
 // only when the clipped last chunk is kept), publishes the kept-chunk list for the scoring CTAs'
 // copy threads and announces it on the head's third counter.
-template <int C_STATIC>
+template <int C_STATIC, SelectIn WHERE>
 __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn, int* flag_smem) {
     SelectSmem& ss = *reinterpret_cast<SelectSmem*>(dyn);
     constexpr size_t kSelBytes = (sizeof(SelectSmem) + 127) & ~size_t(127);
@@ -253,8 +253,8 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
             if (!flag[0]) return false;
             const float* sc = p.scores + (static_cast<size_t>(s) * p.Hkv + hkv) * p.n_mt * p.Cpad;
             const float* sc2 = p.n_mt == 2 ? sc + p.Cpad : nullptr;
-            if (p.sel_keys_fit || p.C <= kMThreads * select_reg_keys(kSelModel))
-                select_kept<kSelModel>(sc, sc2, p.C, p.k, ss, kbuf);
+            if (p.sel_keys_fit || p.C <= kMThreads * select_reg_keys(WHERE))
+                select_kept<WHERE>(sc, sc2, p.C, p.k, ss, kbuf);
             else
                 select_head_rows(sc, sc2, p.L, p.w, C_STATIC, p.C, p.k, p.n_max, p.layer[li].out_idx + static_cast<size_t>(hkv) * p.n_max,
                                  ss, nullptr);
@@ -325,7 +325,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
         __syncthreads();
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        const bool s_ok = selector_loop<C_STATIC>(p, dyn, ctl.sel_flag);
+        const bool s_ok = selector_loop<C_STATIC, BIG && C_STATIC == 8 ? kSelModelCore : kSelModel>(p, dyn, ctl.sel_flag);
         __syncthreads();
         if (threadIdx.x == 0) {
             if (!s_ok) atomicExch(p.status, 1);

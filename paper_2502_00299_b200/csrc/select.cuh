@@ -518,15 +518,18 @@ __device__ __forceinline__ void select_core(const float* sc, const float* sc2, i
 // select_reg_keys() keys a thread. The layer kernel and select.cu take select_regs throughout. The other kernels have no registers
 // to spare beside their own: with select_regs for 6 keys or more the model kernel spills and a call with 5994 chunks is 8 %
 // slower, so it takes that form up to 4 keys a thread (32 layers of 4096 tokens 348 -> 311 us, 16 layers of 20000 tokens in chunks
-// of 16 228 -> 206); the kernels of score.cu spill with any of it.
+// of 16 228 -> 206); the kernels of score.cu spill with any of it, and so does the model kernel's big variant for chunks of 8 (30 bytes
+// a thread instead of 28; 12000 tokens, 224 rows 303 -> 308 us, 24000 tokens, 256 rows 270 -> 279; the big variants of the other sizes are 0.5 to
+// 2 % faster with it).
 // (All inlined: as a function its register convention made the kernels' scoring loops spill, 2 to 10 % of a model call.)
-enum SelectIn { kSelScratch, kSelModel, kSelLayer };      // the kernels of score.cu, the model kernel, the layer kernel or select.cu
-__host__ __device__ constexpr int select_reg_keys(SelectIn where) { return where == kSelLayer ? 24 : (where == kSelModel ? 16 : 8); }
+// the kernels of score.cu, the model kernel (kSelModelCore: without select_regs), the layer kernel or select.cu
+enum SelectIn { kSelScratch, kSelModel, kSelModelCore, kSelLayer };
+__host__ __device__ constexpr int select_reg_keys(SelectIn where) { return where == kSelLayer ? 24 : (where == kSelScratch ? 8 : 16); }
 template <SelectIn WHERE>
 __device__ __forceinline__ void select_kept(const float* sc, const float* sc2, int C, int k, SelectSmem& sm, uint32_t* kbuf) {
     const int per = (C + static_cast<int>(blockDim.x) - 1) / static_cast<int>(blockDim.x);
     if (per > select_reg_keys(WHERE)) return select_core<0>(sc, sc2, C, k, sm, kbuf);
-    if constexpr (WHERE != kSelScratch) {
+    if constexpr (WHERE == kSelModel || WHERE == kSelLayer) {
         // the shortest run that covers the ids: the longer ones leave more warps without any, and a step's time goes with the
         // keys of the busiest scheduler (816 keys: runs of 2 4.5k clocks, of 4 5.2k; 1636 keys: of 4 4.6k, of 8 5.7k)
         if (per <= 2) return select_regs<2>(sc, sc2, C, k, sm);
@@ -538,7 +541,7 @@ __device__ __forceinline__ void select_kept(const float* sc, const float* sc2, i
         select_regs<24>(sc, sc2, C, k, sm);
     } else {
         if (WHERE == kSelScratch || per <= 8) return select_core<8>(sc, sc2, C, k, sm, nullptr);
-        if constexpr (WHERE == kSelModel) select_core<16>(sc, sc2, C, k, sm, nullptr);
+        if constexpr (WHERE != kSelScratch) select_core<16>(sc, sc2, C, k, sm, nullptr);
     }
 }
 
