@@ -955,7 +955,7 @@ static int compress_model_impl(int n_layers, const void* const* q_obs, const voi
         if (st != CHUNKKV_OK) return st;
         // paged outputs run layer by layer: the one-launch layer kernel places rows through the block table with all
         // its threads, which measured faster (35 us per layer) than the persistent kernel's copy warp doing it (41 us)
-        if (!paged && C > 0 && k > 0 && make_model_plan(L, R, Hkv, d, c, C, k, ctx->num_sms, smem_budget(*ctx), &mp)) {
+        if (!paged && C > 0 && k > 0 && make_model_plan(L, R, Hkv, d, c, C, k, reuse_depth < n_layers ? reuse_depth : n_layers, ctx->num_sms, smem_budget(*ctx), &mp)) {
             st = ensure_workspace(*ctx, model_scratch_floats(mp, Hkv, C, model_launch_computes(n_layers, reuse_depth)) * sizeof(float));
             if (st != CHUNKKV_OK && model_scratch_required(ctx->num_sms, L, R, Hq / Hkv, Hkv, c)) return st;
             persistent = st == CHUNKKV_OK;

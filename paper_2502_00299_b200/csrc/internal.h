@@ -166,8 +166,8 @@ struct ModelLayerIO {
     bool computes;        // false: gather with the indices of the nearest computed layer before it
 };
 
-// n_sel: selector CTAs (0: as many as are best).
-bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, ModelPlan* plan, int n_sel = 0);
+// reuse: layers that share a computed layer's indices, itself included; n_sel: selector CTAs (0: as many as are best).
+bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int reuse, int max_ctas, int smem_limit, ModelPlan* plan, int n_sel = 0);
 // What a launch uses.
 size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute);
 // What a caller is told to provide, which a shorter sequence never exceeds; 0 for a shape that the kernel does not take.

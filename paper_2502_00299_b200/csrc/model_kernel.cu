@@ -950,7 +950,7 @@ static int selector_each_tiles(int Hkv, int max_ctas) {
     return Hkv > 4 && Hkv <= 8 && max_ctas >= 2 * Hkv ? 6 * ((max_ctas - Hkv) / Hkv) : 0;
 }
 
-bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, ModelPlan* plan, int n_sel) {
+bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int reuse, int max_ctas, int smem_limit, ModelPlan* plan, int n_sel) {
     // the chunk sizes that are compiled in, as in layer_resident.cu
     if (c != 5 && c != 8 && c != 10 && c != 16 && c != 20 && c != 32) return false;
     if (R < 1 || R > 256 || (d != 64 && d != 128) || L < 1 || C < 1 || k < 1 || Hkv < 1 || Hkv > kResidentMaxHeads)
@@ -967,9 +967,21 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int max_
     // a few CTAs do nothing but select (four take the SMs the scoring grid would leave idle anyway)
     p.n_sel = Hkv < 4 ? Hkv : 4;
     // Five to eight heads on short contexts: a selector each. With two heads a selector the two selections (about 5k clocks each)
-    // are longer than the scoring of a layer up to six tiles a CTA, and the scoring CTA a head gives up costs less: 32 layers of
-    // 4096 tokens 309 -> 287 us, 16 of 7000 (256 rows) 192 -> 183, 16 of 2100 157 -> 145, 16 of 11000 (indices shared by two) 121 -> 114.
-    if (p.n_tiles <= selector_each_tiles(Hkv, max_ctas)) p.n_sel = Hkv;
+    // are longer than the scoring of a layer up to six tiles a CTA. Speed with a selector each over four (10 % kept; 64, 128 and 256 rows):
+    //   5 heads  1.04 to 1.19   6 heads  1.00 to 1.19   7 heads  1.04 to 1.17   8 heads  0.99 to 1.26
+    // Six and eight heads give up a scoring CTA a head for it, which then copies rows no longer either. Where much is copied for each
+    // selection that costs more: 8 heads, 4 tiles a CTA, indices shared by three layers, chunks of 8 0.91 to 0.95, of 16 0.93; a quarter
+    // kept, chunks of 5 0.96 to 0.98. So they have to stay below 15 kept chunks to copy a CTA and selection and, beyond two tiles, 27 % of
+    // the rows; within that 0.985 to 1.26. Five and seven heads need no such line (0.996 and more with a quarter kept and indices shared
+    // by three).
+    // (Two sets of layers in turn, inputs of 3 x 200 MB and more, graph replays. More heads keep four selectors; where the line
+    // lies for them has not been worked out.)
+    if (p.n_tiles <= selector_each_tiles(Hkv, max_ctas)) {
+        const int cph = (max_ctas - Hkv) / Hkv;
+        const long long copied = static_cast<long long>(reuse) * kk;
+        const bool light = copied <= 15ll * cph && (p.n_tiles <= 2 * cph || copied * c * 100 <= 27ll * L);
+        if (light || cph == (max_ctas - 4) / Hkv) p.n_sel = Hkv;
+    }
     if (n_sel > 0) p.n_sel = n_sel;
     if (max_ctas - p.n_sel < Hkv) p.n_sel = max_ctas - Hkv;
     p.cph = (max_ctas - p.n_sel) / Hkv;
@@ -1049,10 +1061,10 @@ size_t model_reserve_floats(int L, int R, int Hkv, int d, int c, int C, int k, i
     // selectors that a shorter sequence may have are both provided for.
     size_t need = 0;
     ModelPlan p;
-    if (make_model_plan(L, R, Hkv, d, c, C, k, max_ctas, smem_limit, &p, Hkv < 4 ? Hkv : 4))
+    if (make_model_plan(L, R, Hkv, d, c, C, k, 1, max_ctas, smem_limit, &p, Hkv < 4 ? Hkv : 4))
         need = model_floats(p, Hkv, C, n_compute, p.ring_reserve);
     const long long each = static_cast<long long>(selector_each_tiles(Hkv, max_ctas)) * 2 * panel_keys(c);
-    if (each > 0 && make_model_plan(each < L ? static_cast<int>(each) : L, R, Hkv, d, c, C, k, max_ctas, smem_limit, &p, Hkv)) {
+    if (each > 0 && make_model_plan(each < L ? static_cast<int>(each) : L, R, Hkv, d, c, C, k, 1, max_ctas, smem_limit, &p, Hkv)) {
         const size_t m = model_floats(p, Hkv, C, n_compute, p.ring_reserve);
         need = m > need ? m : need;
     }

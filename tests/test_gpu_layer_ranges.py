@@ -136,3 +136,39 @@ def test_token_scores_and_chunk_scores_with_and_without_them(ck, Hq, Hkv, d, L, 
                                           (4, 16, 64, 148), (1, 64, 128, 81)])
 def test_layer_with_few_rows_and_many_ctas(ck, Hq, w, d, tiles):
     test_layer_and_chunk_scores(ck, Hq, 1, d, 120 * tiles - 7, w, 10)
+
+
+# Five to eight heads have a selector CTA each up to six tiles a scoring CTA (28, 23, 20 and 17 CTAs a head), six and eight only while
+# few chunks and rows are copied for a selection: the last length of the one form and the first of the other, one and two query
+# tiles, either side of 15 chunks a CTA (indices shared by two and three layers) and of 27 % of the rows.
+@pytest.mark.parametrize("Hq,Hkv,L,w,c,n_layers,n_reuse,kept", [
+    (5, 5, 28 * 6 * 120, 8, 10, 3, 1, 0.05), (5, 5, 28 * 6 * 120 + 1, 8, 10, 3, 1, 0.05), (6, 6, 23 * 6 * 120, 8, 10, 3, 1, 0.05),
+    (6, 6, 23 * 6 * 120 + 1, 8, 10, 3, 1, 0.05), (14, 7, 20 * 6 * 128, 32, 16, 3, 2, 0.1), (14, 7, 20 * 6 * 128 + 1, 32, 16, 3, 2, 0.1),
+    (64, 8, 17 * 6 * 120, 32, 20, 2, 1, 0.05), (64, 8, 17 * 6 * 120 + 1, 32, 20, 2, 1, 0.05), (7, 7, 600, 16, 5, 3, 1, 0.3), (6, 6, 121, 8, 8, 2, 1, 0.5),
+    (16, 8, 17 * 3 * 120 - 5, 16, 10, 4, 2, 0.205), (16, 8, 17 * 3 * 120 - 5, 16, 10, 4, 2, 0.22), (16, 8, 17 * 4 * 120, 16, 20, 4, 1, 0.26),
+    (16, 8, 17 * 4 * 120, 16, 20, 4, 1, 0.28), (16, 8, 17 * 2 * 120, 16, 32, 4, 3, 0.25), (8, 8, 17 * 2 * 120, 16, 5, 4, 3, 0.25),
+    (40, 8, 17 * 4 * 128, 26, 8, 3, 50, 0.1),
+])
+def test_model_call_with_five_to_eight_heads(ck, Hq, Hkv, L, w, c, n_layers, n_reuse, kept):
+    budget = w + c * int(kept * L / c)
+    x = [_layer(Hq, Hkv, 64, L, w, c, budget, seed=i)[1] for i in range(2)]
+    on = [tuple(to_dev(t) for t in (a.q_obs, a.K, a.V)) for a in x]
+    outs = ck.compress_model([on[i % 2] for i in range(n_layers)], Hq, w, c, budget, n_reuse)
+    assert ck.device_status() == 0
+    for l, (oK, oV, idx) in enumerate(outs):
+        src = l // n_reuse * n_reuse
+        assert_gather_exact(bits_of(oK), bits_of(oV), idx.cpu().numpy(), x[l % 2].K, x[l % 2].V)
+        if l != src:
+            assert torch.equal(idx, outs[src][2])
+        elif l < 2:
+            s = ora.chunk_scores(ora.token_scores(x[l].q_obs, x[l].K, Hq, Hkv, w), c)
+            assert_selection_matches(idx.cpu().numpy(), s, L, w, c, budget)
+        else:                                             # (the layers of a pair have the same inputs)
+            assert torch.equal(idx, outs[l - 2][2] if n_reuse == 1 else ck.compress_layer(*on[l % 2], Hq, w, c, budget)[2])
+
+
+# Up to 64 rows and more than nine CTAs a head read the head's row statistics in a variant of their own (148 SMs, four selectors)
+@pytest.mark.parametrize("Hq,Hkv,L,w", [(64, 16, 9 * 120, 16), (56, 14, 10 * 120, 16), (70, 14, 10 * 120 - 3, 13), (14, 14, 10 * 120 - 119, 1),
+                                        (56, 14, 9 * 120, 16), (3, 1, 2500, 21)])
+def test_model_call_with_few_rows(ck, Hq, Hkv, L, w):
+    test_model_call(ck, Hq, Hkv, 64, L, w, 10, 2, 1)
