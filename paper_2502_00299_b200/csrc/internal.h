@@ -182,6 +182,7 @@ cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtenso
 struct TokenPlan {
     int n_mt, Hs;         // scoring heads per KV head (1 or 2: more than 128 rows), in all
     int grid, cph, n_tiles, n_tiles_prefix, n_stages, smem_bytes, off_ring, off_misc;
+    bool whole;           // a ring stage is a whole tile of keys, else 64 dims of it
 };
 struct TokenIO {
     int L, w, R, d;       // R = w * Hq / Hkv query rows per KV head

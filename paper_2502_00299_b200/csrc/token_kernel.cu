@@ -14,9 +14,9 @@
 // and four warps to meet on every panel: 15 us of a 32768-token layer's pass 2, 128 rows, against the
 // special-function unit's 7; the layer went from 56.7 to 49.6 us.) Each of the four epilogue groups has an accumulator of its own, 128 keys x 128 rows.
 // A KV head with more than 128 query rows is scored as two heads of 128 and the rest.
-// What bounds it is the hand-over of products to the epilogue and back; a ring stage is a whole tile, so that the issuing thread
-// waits on one barrier and commits one stage per tile instead of one per 64 dims (a satisfied wait costs it 58 clocks): 62261 tokens,
-// 128 rows, with their chunk scores 52.4 -> 50.7 us, a token-level layer of 32768 tokens 47.0 -> 46.4.
+// What bounds it is the hand-over of products to the epilogue and back. With whole tiles as ring stages the issuing thread waits on
+// one barrier and commits one stage per tile instead of one per 64 dims (a satisfied wait costs it 58 clocks), but the ring holds
+// five tiles instead of five and a half and frees them later. Which is faster: make_token_plan.
 #include "internal.h"
 #include "panels.cuh"
 #include "ptx.cuh"
@@ -60,6 +60,8 @@ struct TokArgs {
     int* status;
 };
 
+// WHOLE: a ring stage is a whole tile, else 64 dims of it.
+template <bool WHOLE>
 __global__ void __launch_bounds__(kTThreads, 1)
 token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const TokArgs a) {
@@ -80,7 +82,7 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     float* inv = misc + 2176;          // [128] 1 / l_i
     volatile int* abort_flag = &ctl.abort_flag;
     const uint32_t n_stages = static_cast<uint32_t>(a.n_stages);
-    const uint32_t stage = kTHalfBytes * static_cast<uint32_t>(KB);      // a whole tile: 64 dims after 64 dims
+    const uint32_t stage = WHOLE ? kTHalfBytes * static_cast<uint32_t>(KB) : kTHalfBytes;      // (64 dims after 64 dims)
 
     const int hs = blockIdx.x / a.cph, part = blockIdx.x - hs * a.cph;
     const int hkv = a.n_mt == 2 ? hs >> 1 : hs, row0 = a.n_mt == 2 ? (hs & 1) * 128 : 0;
@@ -126,22 +128,28 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             mbar_arrive_expect_tx(qbar, static_cast<uint32_t>(KB * a.q_box_rows) * 128u);
             for (int kb = 0; kb < KB; ++kb)
                 tma_load_3d(q_base + static_cast<uint32_t>(kb) * kRQTileBytes, &tm_q, qbar, kb * 64, row0, hkv);   // (rows past R arrive as zeros)
-            const uint32_t k_bytes = static_cast<uint32_t>(KB * a.k_box_rows) * 128u;
+            const uint32_t k_bytes = static_cast<uint32_t>((WHOLE ? KB : 1) * a.k_box_rows) * 128u;
             uint32_t st = 0, st_par = 1;
             int issued = 0;
             bool ok = true;
             for (int pass = 0; pass < 2 && ok; ++pass) {
                 // pass 2 walks the tiles backwards: the keys read last in pass 1 are the ones still in L2
                 const int n_pass = pass == 0 ? nt : nt2;
-                for (int i = 0; i < n_pass; ++i) {
+                for (int i = 0; i < n_pass && ok; ++i) {
                     const int t = pass == 0 ? t_begin + i : t_begin + nt2 - 1 - i;
-                    ok = mbar_wait(smem_u32(&ctl.empty[st]), st_par, abort_flag);
-                    if (!ok) break;
-                    const uint32_t bar = smem_u32(&ctl.full[st]);
-                    mbar_arrive_expect_tx(bar, k_bytes);
-                    for (int kb = 0; kb < KB; ++kb) tma_load_3d(k_base + st * stage + kb * kTHalfBytes, &tm_k, bar, kb * 64, t * kTTile, hkv);
-                    ++issued;
-                    if (++st == n_stages) { st = 0; st_par ^= 1u; }
+                    for (int kb = 0; kb < KB; ++kb) {
+                        const uint32_t bar = smem_u32(&ctl.full[st]);
+                        if (!WHOLE || kb == 0) {
+                            ok = mbar_wait(smem_u32(&ctl.empty[st]), st_par, abort_flag);
+                            if (!ok) break;
+                            mbar_arrive_expect_tx(bar, k_bytes);
+                        }
+                        tma_load_3d(k_base + st * stage + (WHOLE ? kb * kTHalfBytes : 0u), &tm_k, bar, kb * 64, t * kTTile, hkv);
+                        if (!WHOLE || kb == KB - 1) {
+                            ++issued;
+                            if (++st == n_stages) { st = 0; st_par ^= 1u; }
+                        }
+                    }
                 }
             }
             if (!ok) {
@@ -167,22 +175,31 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 tc_fence_after();
                 const uint32_t d_addr = tmem_base + static_cast<uint32_t>(buf * 128);
                 const bool keys_first = tg >= nt;        // pass 2: lanes are keys
-                ok = mbar_wait(smem_u32(&ctl.full[st]), st_par, abort_flag);
-                if (!ok) break;
-                tc_fence_after();
 #pragma unroll
                 for (int kb = 0; kb < 2; ++kb) {
                     if (kb >= KB) break;
-                    const uint64_t k_desc = umma_desc_sw128(k_base + st * stage + kb * kTHalfBytes);
+                    if (!WHOLE || kb == 0) {
+                        ok = mbar_wait(smem_u32(&ctl.full[st]), st_par, abort_flag);
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
+                    const uint64_t k_desc = umma_desc_sw128(k_base + st * stage + (WHOLE ? kb * kTHalfBytes : 0u));
                     const uint64_t q_desc = umma_desc_sw128(q_base + static_cast<uint32_t>(kb) * kRQTileBytes);
                     const uint64_t a_desc = keys_first ? k_desc : q_desc, b_desc = keys_first ? q_desc : k_desc;
 #pragma unroll
                     for (int k4 = 0; k4 < 4; ++k4)
                         umma_bf16(d_addr, a_desc + 2u * k4, b_desc + 2u * k4, IDESC, (kb > 0 || k4 > 0) ? 1u : 0u);
+                    if (!WHOLE) {
+                        umma_commit(smem_u32(&ctl.empty[st]));
+                        if (++st == n_stages) { st = 0; st_par ^= 1u; }
+                    }
                 }
+                if (!ok) break;
                 umma_commit(smem_u32(&ctl.tfull[buf]));
-                umma_commit(smem_u32(&ctl.empty[st]));
-                if (++st == n_stages) { st = 0; st_par ^= 1u; }
+                if (WHOLE) {
+                    umma_commit(smem_u32(&ctl.empty[st]));
+                    if (++st == n_stages) { st = 0; st_par ^= 1u; }
+                }
             }
         }
     } else {
@@ -365,10 +382,15 @@ bool make_token_plan(int L, int w, int R, int Hkv, int d, int max_ctas, int smem
     const int KB = d / 64;
     const int q_bytes = KB * kRQTileBytes;
     const int fixed = 1024 + q_bytes + 1024 + kTMiscBytes;
-    const int stage = KB * static_cast<int>(kTHalfBytes);
+    // Whole tiles as stages for one scoring head a KV head and more than ten tiles a CTA, us with stages of 64 dims -> of whole
+    // tiles, d = 128, with the chunk sums: 8 heads, 128 rows 32768 tokens 40.2 -> 39.8, 46657 51.0 -> 50.5, 90000 78.5 -> 77; 4 heads, 112 rows
+    // 56490 37.2 -> 36.8. Not for less: 8 heads, 64 rows 16000 22.8 -> 23.1; 4 heads, 112 rows 32768 29.1 -> 29.5, 46657 (ten tiles) 34.9 -> 35.2;
+    // nor for the two scoring heads of more than 128 rows: 4 heads, 224 rows 46657 41.1 -> 41.5, 8 heads, 256 rows 32768 51.5 -> 52.0.
+    p.whole = KB == 1 || (n_mt == 1 && p.n_tiles > 10 * p.cph);
+    const int stage = (p.whole ? KB : 1) * static_cast<int>(kTHalfBytes);
     int ns = (smem_limit - fixed) / stage;
     if (ns > kRMaxStages) ns = kRMaxStages;
-    if (ns < 2) return false;
+    if (ns < (p.whole ? 2 : 2 * KB)) return false;
     p.n_stages = ns;
     p.off_ring = q_bytes;
     p.off_misc = p.off_ring + ns * stage + 1024;
@@ -391,12 +413,14 @@ cudaError_t launch_token_scores(const TokenPlan& plan, const CUtensorMap& tm_q, 
     a.exits = io.counters;
     a.cnt_a = io.counters + 16;
     a.status = io.status;
-    static int smem_set[64] = {0};
+    const void* kern = plan.whole ? reinterpret_cast<const void*>(token_scores_kernel<true>) : reinterpret_cast<const void*>(token_scores_kernel<false>);
+    static int smem_all[2][64] = {{0}};
+    int* smem_set = smem_all[plan.whole ? 1 : 0];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || smem_set[dev] < plan.smem_bytes) {
-        e = cudaFuncSetAttribute(token_scores_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.smem_bytes);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) smem_set[dev] = plan.smem_bytes;
     }
@@ -415,7 +439,7 @@ cudaError_t launch_token_scores(const TokenPlan& plan, const CUtensorMap& tm_q, 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(token_scores_kernel), params);
+    return cudaLaunchKernelExC(&cfg, kern, params);
 }
 
 }  // namespace chunkkv

@@ -172,3 +172,9 @@ def test_model_call_with_five_to_eight_heads(ck, Hq, Hkv, L, w, c, n_layers, n_r
                                         (56, 14, 9 * 120, 16), (3, 1, 2500, 21)])
 def test_model_call_with_few_rows(ck, Hq, Hkv, L, w):
     test_model_call(ck, Hq, Hkv, 64, L, w, 10, 2, 1)
+
+
+# d = 128: a ring stage is 64 dims of a tile up to ten tiles a CTA (four CTAs a head of 32) and for two scoring heads, else a whole tile
+@pytest.mark.parametrize("Hq,Hkv,L,w", [(32, 32, 40 * 128, 4), (32, 32, 40 * 128 + 1, 4), (64, 32, 4 * 23 * 128 - 77, 16), (160, 32, 2 * 11 * 128 + 5, 32)])
+def test_token_scores_with_either_ring_stage(ck, Hq, Hkv, L, w):
+    test_token_scores_and_chunk_scores_with_and_without_them(ck, Hq, Hkv, 128, L, w, 7)

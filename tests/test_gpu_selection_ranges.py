@@ -126,3 +126,33 @@ def test_select_at_the_ends_of_runs(ck, C):
         for h in range(4):
             want = ora.select_chunks(x[h].double().cpu().numpy(), k)
             assert np.array_equal(idx[h][:k * c], (want[:, None] * c + np.arange(c)).ravel())
+
+
+# The same with the scores of two scoring heads added (136 rows of an even group of heads)
+@pytest.mark.parametrize("C,k", [(575, 3), (1152, 700), (1153, 1), (2304, 90), (2305, 2300), (4608, 500), (4609, 1000)])
+def test_layer_selection_of_two_scoring_heads_at_the_ends_of_runs(ck, C, k):
+    w, c, d = 17, 10, 64
+    L = C * c + w - 4
+    q, K, V = _random(8, 1, d, L, w, seed=C)
+    s = ora.chunk_scores(ora.token_scores(q, K, 8, 1, w), c)
+    oK, oV, idx = ck.compress_layer(*map(to_dev, (q, K, V)), 8, w, c, w + c * k)
+    assert ck.device_status() == 0
+    assert_selection_matches(idx.cpu().numpy(), s, L, w, c, w + c * k)
+    assert_gather_exact(bits_of(oK), bits_of(oV), idx.cpu().numpy(), K, V)
+
+
+# A selector of the model kernel has 640 threads: runs of 2 and 4 ids, 8 and 16 keys a thread, then shared memory; small and big (two
+# query tiles) variants, the big one for chunks of 8 without runs
+@pytest.mark.parametrize("Hq,c", [(4, 5), (16, 10), (16, 8)])
+@pytest.mark.parametrize("C,k", [(1280, 300), (1281, 1280), (2560, 1), (2561, 800), (5120, 5000), (5121, 400), (10240, 700), (10241, 900)])
+def test_model_selection_at_the_ends_of_runs(ck, Hq, c, C, k):
+    w, d = 10, 64
+    L = C * c + w - 3
+    q, K, V = _random(Hq, 1, d, L, w, seed=C + c)
+    s = ora.chunk_scores(ora.token_scores(q, K, Hq, 1, w), c)
+    x = tuple(map(to_dev, (q, K, V)))
+    outs = ck.compress_model([x, x], Hq, w, c, w + c * k)
+    assert ck.device_status() == 0
+    assert_selection_matches(outs[0][2].cpu().numpy(), s, L, w, c, w + c * k)
+    assert_gather_exact(bits_of(outs[0][0]), bits_of(outs[0][1]), outs[0][2].cpu().numpy(), K, V)
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
