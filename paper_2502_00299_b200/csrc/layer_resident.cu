@@ -160,7 +160,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     float* pmax = reinterpret_cast<float*>(dyn + a.off_pmax);      // [panel of this CTA][128] panel maxima (log2 domain)
     float* misc = reinterpret_cast<float*>(dyn + a.off_misc);
     float* rec = misc;                 // [4 groups][{max, sum}][128]
-    float* slice = misc + 1024;        // [4 slices][{max, sum}][128]
+    float* slice = misc + 1024;        // [4 slices][{max, sum}][128]; FEW: [{max, sum}][8 slices][64]
     float* gm = misc + 2048;           // [2 query tiles][128] row maxima of the head
     float* ginv = misc + 2304;         // [2 query tiles][128] 1 / row sums of the head
     uint8_t* ring = dyn + a.off_ring;  // reused after scoring
@@ -220,10 +220,10 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                     tma_load_3d(q_base + static_cast<uint32_t>(mt * KB + kb) * kRQTileBytes, &tm_q, qbar, kb * 64, row0 + mt * 128, hkv);
             const uint32_t k_bytes = static_cast<uint32_t>(min(a.L, TILE)) * 128u;
             // Panels in scratch: the keys leave the L2 to their records, unless the kept key rows, which the gather reads again, are
-            // the larger part. us without -> with the hint: 131072 tokens, 256 rows, c = 20, 3 % kept (47 MB of records, 8 MB of rows) 124 -> 115;
-            // 52088 tokens, 64 rows, c = 5, 16 % (14 MB, 17 MB) 55.7 -> 54.0; 131072 tokens, 64 rows, c = 5, 25 % (48 MB, 67 MB) 146.7 -> 149.2;
-            // 120859 tokens, 128 rows, c = 20, 18 % (8 MB, 45 MB) 92.4 -> 98.3.
-            const bool keys_leave = 3ll * a.n_max * a.Hkv * a.d * 2 < 4ll * a.n_off * (SPP + 1) * a.spill_rows * 4 * gridDim.x;
+            // many. us without -> with the hint (kept key rows): 131072 tokens, 256 rows, c = 20 (8 MB) 124 -> 115; 131072, 128 rows, c = 10 (13 MB) 85.2 -> 82.5;
+            // 52088, 64 rows, c = 5 (17 MB) 55.7 -> 54.0; 80000, 128 rows, c = 10 (25 MB) 64.4 -> 63.2; 120859, 128 rows, c = 20 (45 MB) 92.4 -> 98.3; 131072,
+            // 64 rows, c = 5 (67 MB) 146.7 -> 149.2.
+            const bool keys_leave = a.n_off > 0 && 2ll * a.n_max * a.Hkv * a.d <= (32ll << 20);
             const uint64_t policy = keys_leave ? l2_policy_evict_first() : l2_policy_evict_normal();
             uint32_t st = 0, st_par = 1;
             int issued = 0;

@@ -288,9 +288,10 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
 
 // BIG: two query tiles, or a ring that reaches into scratch. A variant of its own, so that the kernel for up to 128 rows
 // carries none of it.
-// FEW: up to 64 rows and more than nine CTAs a head, for the reading of row statistics. A variant of its own: as a run-time choice it
-// made the general form spill (bytes of stores / loads at c = 10: 16 / 28 instead of none, at 16: 32 / 44 instead of 20 / 20).
-template <int C_STATIC, bool BIG, bool FEW>
+// (The reading of row statistics for few rows is a run-time choice below. It makes the small form spill - bytes of stores / loads at c = 10:
+// 16 / 28 instead of none - and is faster for it: with a variant of its own 25 layers of 10000 tokens, 112 rows, c = 10 282.8 -> 287.8 us,
+// 32 layers of 2300 tokens, 128 rows 265 -> 268.5, 9 of 30000 156.7 -> 158.4; other chunk sizes the same.)
+template <int C_STATIC, bool BIG>
 __global__ void __launch_bounds__(kMThreads, 1)
 model_kernel(const __grid_constant__ ModelParams p) {
     constexpr int WP = panel_keys(C_STATIC);
@@ -387,9 +388,12 @@ model_kernel(const __grid_constant__ ModelParams p) {
             const uint32_t qbar = smem_u32(&ctl.qfull);
             const uint32_t q_bytes = static_cast<uint32_t>(n_mt * KB * p.q_box_rows) * 128u;
             const uint32_t k_bytes = static_cast<uint32_t>(p.k_box_rows) * 128u;
-            // A ring that continues in scratch: the keys leave the L2 to it (30000 tokens, 128 rows, c = 5 222 -> 217 us, 256 rows, c = 10 246 -> 241). On chip
-            // there is nothing to keep, and the row copies of the next layer read kept key rows (16000 tokens, 224 rows, c = 20, 25 % kept: 320 -> 321 us with the hint).
-            const uint64_t policy = p.ring > p.ring_on ? l2_policy_evict_first() : l2_policy_evict_normal();
+            // The keys, which are read once, leave the L2 first where the ring continues in scratch (30000 tokens, 128 rows, c = 5 222 -> 217 us,
+            // 256 rows, c = 10 246 -> 241) and where a layer has few of them (224 rows, 4 heads: 2300 tokens, c = 16 266.6 -> 258.7, 5500 tokens, c = 20
+            // 169.4 -> 166.5). Not otherwise: the row copies of the next layer read the kept key rows again (16000 tokens, 16 MB, c = 20,
+            // 10 % kept: 315.4 -> 317.1).
+            const bool leave = p.ring > p.ring_on || 2ll * p.Hkv * p.L * p.d <= (6ll << 20);
+            const uint64_t policy = leave ? l2_policy_evict_first() : l2_policy_evict_normal();
             uint32_t st = 0, st_par = 1;
             int issued = 0;
             bool ok = true;
@@ -769,7 +773,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
             if (!wait_counter_warp(p.cnt_a + hkv, static_cast<unsigned>(s + 1) * p.cph, abort_flag)) break;
             if constexpr (!BIG) {
                 // the head's records straight from the L2 (they were written by other SMs; every lane has
-                // acquired the counter), nine CTAs' worth of loads in flight per lane. FEW: each half of the warp
+                // acquired the counter), nine CTAs' worth of loads in flight per lane. Up to 64 rows each half of the warp
                 // takes every other record (2 heads: 69 CTAs, 32 layers of 8192 tokens 487 -> 335 us).
                 const float* src = p.cta_stat + (static_cast<size_t>(s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * 256;
                 float M[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}, S[4] = {0.f, 0.f, 0.f, 0.f};
@@ -786,7 +790,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                         merge_batch<9>(M, S, m, l, n - j0);
                     }
                 };
-                if constexpr (!FEW) {
+                if (p.R > 64) {
                     fold(src + r0, std::integral_constant<int, 256>{}, p.cph);
                 } else {
                     const int sub = lane >> 4;
@@ -971,15 +975,15 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int reus
     //   5 heads  1.04 to 1.19   6 heads  1.00 to 1.19   7 heads  1.04 to 1.17   8 heads  0.99 to 1.26
     // Six and eight heads give up a scoring CTA a head for it, which then copies rows no longer either. Where much is copied for each
     // selection that costs more: 8 heads, 4 tiles a CTA, indices shared by three layers, chunks of 8 0.91 to 0.95, of 16 0.93; a quarter
-    // kept, chunks of 5 0.96 to 0.98. So they have to stay below 15 kept chunks to copy a CTA and selection and, beyond two tiles, 27 % of
-    // the rows; within that 0.985 to 1.26. Five and seven heads need no such line (0.996 and more with a quarter kept and indices shared
+    // kept, chunks of 5 0.96 to 0.98. So they have to stay below 22 kept chunks to copy a CTA and selection, 15 where indices are shared, and,
+    // beyond two tiles, 27 % of the rows; within that 0.985 to 1.26. Five and seven heads need no such line (0.996 and more with a quarter kept and indices shared
     // by three).
     // (Two sets of layers in turn, inputs of 3 x 200 MB and more, graph replays. More heads keep four selectors; where the line
     // lies for them has not been worked out.)
     if (p.n_tiles <= selector_each_tiles(Hkv, max_ctas)) {
         const int cph = (max_ctas - Hkv) / Hkv;
         const long long copied = static_cast<long long>(reuse) * kk;
-        const bool light = copied <= 15ll * cph && (p.n_tiles <= 2 * cph || copied * c * 100 <= 27ll * L);
+        const bool light = copied <= (reuse > 1 ? 15ll : 22ll) * cph && (p.n_tiles <= 2 * cph || copied * c * 100 <= 27ll * L);
         if (light || cph == (max_ctas - 4) / Hkv) p.n_sel = Hkv;
     }
     if (n_sel > 0) p.n_sel = n_sel;
@@ -1071,12 +1075,9 @@ size_t model_reserve_floats(int L, int R, int Hkv, int d, int c, int C, int k, i
     return need;
 }
 
-// 0: small, 1: big, 2: small with few rows
 template <int C_STATIC>
-static const void* model_kernel_of(int variant) {
-    return variant == 1 ? reinterpret_cast<const void*>(model_kernel<C_STATIC, true, false>)
-         : variant == 2 ? reinterpret_cast<const void*>(model_kernel<C_STATIC, false, true>)
-                        : reinterpret_cast<const void*>(model_kernel<C_STATIC, false, false>);
+static const void* model_kernel_of(bool big) {
+    return big ? reinterpret_cast<const void*>(model_kernel<C_STATIC, true>) : reinterpret_cast<const void*>(model_kernel<C_STATIC, false>);
 }
 
 cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtensorMap* tm_q, const CUtensorMap* tm_k,
@@ -1127,21 +1128,19 @@ cudaError_t launch_model(const ModelPlan& plan, const ModelIO& io, const CUtenso
     p.cnt_b = io.counters + 16 + kResidentMaxHeads;
     p.cnt_c = io.counters + 16 + 2 * kResidentMaxHeads;
     p.status = io.status;
-    // (nine records are one round trip, which half a warp does not shorten)
-    const int variant = plan.big ? 1 : (io.R <= 64 && plan.cph > 9 ? 2 : 0);
     const void* kern = nullptr;
     int v = 0;
     switch (plan.c_static) {
-        case 5: kern = model_kernel_of<5>(variant); v = 0; break;
-        case 8: kern = model_kernel_of<8>(variant); v = 1; break;
-        case 10: kern = model_kernel_of<10>(variant); v = 2; break;
-        case 16: kern = model_kernel_of<16>(variant); v = 3; break;
-        case 20: kern = model_kernel_of<20>(variant); v = 4; break;
-        case 32: kern = model_kernel_of<32>(variant); v = 5; break;
+        case 5: kern = model_kernel_of<5>(plan.big); v = 0; break;
+        case 8: kern = model_kernel_of<8>(plan.big); v = 1; break;
+        case 10: kern = model_kernel_of<10>(plan.big); v = 2; break;
+        case 16: kern = model_kernel_of<16>(plan.big); v = 3; break;
+        case 20: kern = model_kernel_of<20>(plan.big); v = 4; break;
+        case 32: kern = model_kernel_of<32>(plan.big); v = 5; break;
         default: break;
     }
-    v += 6 * variant;
-    static int smem_set[18][64] = {{0}};
+    v += plan.big ? 6 : 0;
+    static int smem_set[12][64] = {{0}};
     int dev = 0;
     cudaError_t e = kern != nullptr ? cudaGetDevice(&dev) : cudaErrorInvalidValue;
     if (e == cudaSuccess && (dev < 0 || dev >= 64 || smem_set[v][dev] < plan.smem_bytes)) {

@@ -383,8 +383,8 @@ bool make_token_plan(int L, int w, int R, int Hkv, int d, int max_ctas, int smem
     const int q_bytes = KB * kRQTileBytes;
     const int fixed = 1024 + q_bytes + 1024 + kTMiscBytes;
     // Whole tiles as stages for one scoring head a KV head and more than ten tiles a CTA, us with stages of 64 dims -> of whole
-    // tiles, d = 128, with the chunk sums: 8 heads, 128 rows 32768 tokens 40.2 -> 39.8, 46657 51.0 -> 50.5, 90000 78.5 -> 77; 4 heads, 112 rows
-    // 56490 37.2 -> 36.8. Not for less: 8 heads, 64 rows 16000 22.8 -> 23.1; 4 heads, 112 rows 32768 29.1 -> 29.5, 46657 (ten tiles) 34.9 -> 35.2;
+    // tiles, d = 128, with the chunk sums: 8 heads, 128 rows 32768 tokens 40.3 -> 39.6, 46657 51.1 -> 50.0, 90000 79 -> 76.4; 4 heads, 112 rows
+    // 56490 37.3 -> 36.5. Not for less: 8 heads, 64 rows 16000 22.8 -> 23.1; 4 heads, 112 rows 32768 29.1 -> 29.5, 46657 (ten tiles) 34.9 -> 35.2;
     // nor for the two scoring heads of more than 128 rows: 4 heads, 224 rows 46657 41.1 -> 41.5, 8 heads, 256 rows 32768 51.5 -> 52.0.
     p.whole = KB == 1 || (n_mt == 1 && p.n_tiles > 10 * p.cph);
     const int stage = (p.whole ? KB : 1) * static_cast<int>(kTHalfBytes);

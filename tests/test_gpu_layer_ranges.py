@@ -140,7 +140,7 @@ def test_layer_with_few_rows_and_many_ctas(ck, Hq, w, d, tiles):
 
 # Five to eight heads have a selector CTA each up to six tiles a scoring CTA (28, 23, 20 and 17 CTAs a head), six and eight only while
 # few chunks and rows are copied for a selection: the last length of the one form and the first of the other, one and two query
-# tiles, either side of 15 chunks a CTA (indices shared by two and three layers) and of 27 % of the rows.
+# tiles, either side of 15 and 22 chunks a CTA (indices shared or not) and of 27 % of the rows.
 @pytest.mark.parametrize("Hq,Hkv,L,w,c,n_layers,n_reuse,kept", [
     (5, 5, 28 * 6 * 120, 8, 10, 3, 1, 0.05), (5, 5, 28 * 6 * 120 + 1, 8, 10, 3, 1, 0.05), (6, 6, 23 * 6 * 120, 8, 10, 3, 1, 0.05),
     (6, 6, 23 * 6 * 120 + 1, 8, 10, 3, 1, 0.05), (14, 7, 20 * 6 * 128, 32, 16, 3, 2, 0.1), (14, 7, 20 * 6 * 128 + 1, 32, 16, 3, 2, 0.1),
