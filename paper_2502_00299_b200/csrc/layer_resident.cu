@@ -136,8 +136,9 @@ __device__ __forceinline__ bool head_handover(unsigned* counter, unsigned target
 // the other shapes 1.5 us of 34 (32K tokens, 128 rows).
 // FEW: up to 64 rows and more than kRManyCtas CTAs a head, for the reading of row statistics; a variant of its own for the same reason
 // (as a run-time choice it costs every other shape 0.1 us of 12 to 30).
+// WIDE: more than 16 chunks a thread (9216 a head), for the selection, whose bodies for them would slow the scoring of the others.
 constexpr int kRManyCtas = 20;
-template <int C_STATIC, bool BIG, bool FEW>
+template <int C_STATIC, bool BIG, bool FEW, bool WIDE>
 __global__ void __launch_bounds__(kRThreads, 1)
 layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                       const ResArgs a) {
@@ -547,8 +548,9 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         const size_t idx_bytes = (static_cast<size_t>(r_end - r_begin) * 4 + 127) & ~size_t(127);
         uint32_t* kbuf = reinterpret_cast<uint32_t*>(ring + kSelBytes + idx_bytes);
         const bool fits = kSelBytes + idx_bytes + static_cast<size_t>(C) * 4 <= static_cast<size_t>(a.ring_bytes);
-        if (min(a.k, C) <= kSelCap && C <= kSelMaxChunks && (fits || C <= kRThreads * select_reg_keys(kSelLayer))) {
-            select_kept<kSelLayer>(sc, sc2, C, a.k, ss, kbuf);
+        constexpr SelectIn kIn = WIDE ? kSelLayerWide : kSelLayer;
+        if (min(a.k, C) <= kSelCap && C <= kSelMaxChunks && ((WIDE && fits) || C <= kRThreads * select_reg_keys(kIn))) {
+            select_kept<kIn>(sc, sc2, C, a.k, ss, kbuf);
             // every CTA holds the head's kept chunks: it expands, writes and gathers its own share of the positions
             const int n_tok = select_tokens(a.P, C_STATIC, C, a.k, ss, a.tok_cap);
             for (int n = r_begin + threadIdx.x; n < r_end; n += kRThreads) {
@@ -596,12 +598,17 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     }
 }
 
-// 0: small, 1: big, 2: small with few rows
-template <int C_STATIC>
+// variant: 0 small, 1 big, 2 small with few rows
+template <int C_STATIC, bool WIDE>
 const void* kernel_of(int variant) {
-    return variant == 1 ? reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, true, false>)
-         : variant == 2 ? reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, false, true>)
-                        : reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, false, false>);
+    return variant == 1 ? reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, true, false, WIDE>)
+         : variant == 2 ? reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, false, true, WIDE>)
+                        : reinterpret_cast<const void*>(layer_resident_kernel<C_STATIC, false, false, WIDE>);
+}
+
+template <int C_STATIC>
+const void* kernel_of(int variant, bool wide) {
+    return wide ? kernel_of<C_STATIC, true>(variant) : kernel_of<C_STATIC, false>(variant);
 }
 
 }  // namespace
@@ -693,19 +700,20 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     a.spill = scores + (((static_cast<size_t>(io.Hkv) << plan.shift) * ((io.C + 3) & ~3) + 63) & ~static_cast<size_t>(63));
     a.counters = io.counters;
     const int variant = plan.n_mt == 2 || plan.n_off > 0 ? 1 : (io.R <= 64 && plan.cph > kRManyCtas ? 2 : 0);
+    const bool wide = io.out_idx != nullptr && io.C > kRThreads * select_reg_keys(kSelLayer);
     const void* kern = nullptr;
     int v = 0;
     switch (plan.c_static) {
-        case 5: kern = kernel_of<5>(variant); v = 0; break;
-        case 8: kern = kernel_of<8>(variant); v = 1; break;
-        case 10: kern = kernel_of<10>(variant); v = 2; break;
-        case 16: kern = kernel_of<16>(variant); v = 3; break;
-        case 20: kern = kernel_of<20>(variant); v = 4; break;
-        case 32: kern = kernel_of<32>(variant); v = 5; break;
+        case 5: kern = kernel_of<5>(variant, wide); v = 0; break;
+        case 8: kern = kernel_of<8>(variant, wide); v = 1; break;
+        case 10: kern = kernel_of<10>(variant, wide); v = 2; break;
+        case 16: kern = kernel_of<16>(variant, wide); v = 3; break;
+        case 20: kern = kernel_of<20>(variant, wide); v = 4; break;
+        case 32: kern = kernel_of<32>(variant, wide); v = 5; break;
         default: return cudaErrorInvalidValue;
     }
-    v += 6 * variant;
-    static int smem_set[18][64] = {{0}};
+    v += 6 * (variant + (wide ? 3 : 0));
+    static int smem_set[36][64] = {{0}};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;

@@ -21,8 +21,8 @@ select_kernel(const float* __restrict__ scores, int L, int w, int c, int C, int 
     const int h = blockIdx.x;
     const float* sc = scores + static_cast<size_t>(h) * C;
     int32_t* out = out_idx + static_cast<size_t>(h) * n_max;
-    if (staged && (key_bytes > 0 || C <= kSelThreads * select_reg_keys(kSelLayer)))
-        select_head<kSelLayer>(sc, nullptr, L, w, c, C, k, n_max, out, sm, kbuf, tok_cap);
+    if (staged && (key_bytes > 0 || C <= kSelThreads * select_reg_keys(kSelAlone)))
+        select_head<kSelAlone>(sc, nullptr, L, w, c, C, k, n_max, out, sm, kbuf, tok_cap);
     else
         select_head_rows(sc, nullptr, L, w, c, C, k, n_max, out, sm, key_bytes > 0 ? kbuf : nullptr, tok_cap);
 }
@@ -34,7 +34,7 @@ cudaError_t launch_select(const float* scores, int L, int Hkv, int w, int c, int
     // thousands of chunks per head: eight CTAs per head
     if (select_cluster_applies(C, k)) return launch_select_cluster(scores, L, Hkv, w, c, C, k, n_max, out_idx, stream, tok_cap);
     const bool staged = (k < C ? k : C) <= kSelCap && C <= kSelMaxChunks;
-    if (staged && C <= kSelThreads * select_reg_keys(kSelLayer)) {
+    if (staged && C <= kSelThreads * select_reg_keys(kSelAlone)) {
         select_kernel<<<Hkv, kSelThreads, kSelBytes, stream>>>(scores, L, w, c, C, k, n_max, out_idx, 0, true, tok_cap);
         return cudaGetLastError();
     }

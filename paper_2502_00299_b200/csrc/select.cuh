@@ -521,25 +521,42 @@ __device__ __forceinline__ void select_core(const float* sc, const float* sc2, i
 // of 16 228 -> 206); the kernels of score.cu spill with any of it, and so does the model kernel's big variant for chunks of 8 (30 bytes
 // a thread instead of 28; 12000 tokens, 224 rows 303 -> 308 us, 24000 tokens, 256 rows 270 -> 279; the big variants of the other sizes are 0.5 to
 // 2 % faster with it).
-// (All inlined: as a function its register convention made the kernels' scoring loops spill, 2 to 10 % of a model call.)
-// the kernels of score.cu, the model kernel (kSelModelCore: without select_regs), the layer kernel or select.cu
-enum SelectIn { kSelScratch, kSelModel, kSelModelCore, kSelLayer };
-__host__ __device__ constexpr int select_reg_keys(SelectIn where) { return where == kSelLayer ? 24 : (where == kSelScratch ? 8 : 16); }
+// What else is compiled into a kernel changes how its scoring loops are scheduled, without a spill: the layer kernel with the bodies for more
+// than 16 keys a thread beside the others is slower at 80000 tokens (28 query heads, 112 rows, chunks of 32 35.7 -> 36.6 us), so those are a variant of
+// it.
+// (All inlined: as a function its register convention made the kernels' scoring loops spill, 2 to 10 % of a model call; the layer
+// kernel does not spill with it, but is 1 to 2 % slower.)
+enum SelectIn {
+    kSelScratch,        // the kernels of score.cu
+    kSelModel,          // the model kernel
+    kSelModelCore,      // the same without select_regs
+    kSelLayer,          // the layer kernel, at most 16 keys a thread
+    kSelLayerWide,      // the layer kernel, more
+    kSelAlone           // select.cu
+};
+__host__ __device__ constexpr int select_reg_keys(SelectIn where) {
+    return where == kSelLayerWide || where == kSelAlone ? 24 : (where == kSelScratch ? 8 : 16);
+}
+
 template <SelectIn WHERE>
 __device__ __forceinline__ void select_kept(const float* sc, const float* sc2, int C, int k, SelectSmem& sm, uint32_t* kbuf) {
     const int per = (C + static_cast<int>(blockDim.x) - 1) / static_cast<int>(blockDim.x);
-    if (per > select_reg_keys(WHERE)) return select_core<0>(sc, sc2, C, k, sm, kbuf);
-    if constexpr (WHERE == kSelModel || WHERE == kSelLayer) {
+    if constexpr (WHERE != kSelLayer) {
+        if (per > select_reg_keys(WHERE)) return select_core<0>(sc, sc2, C, k, sm, kbuf);
+    }
+    if constexpr (WHERE == kSelModel || WHERE == kSelLayer || WHERE == kSelAlone) {
         // the shortest run that covers the ids: the longer ones leave more warps without any, and a step's time goes with the
         // keys of the busiest scheduler (816 keys: runs of 2 4.5k clocks, of 4 5.2k; 1636 keys: of 4 4.6k, of 8 5.7k)
         if (per <= 2) return select_regs<2>(sc, sc2, C, k, sm);
         if (per <= 4) return select_regs<4>(sc, sc2, C, k, sm);
     }
-    if constexpr (WHERE == kSelLayer) {
+    if constexpr (WHERE == kSelLayer || WHERE == kSelAlone) {
         if (per <= 8) return select_regs<8>(sc, sc2, C, k, sm);
-        if (per <= 16) return select_regs<16>(sc, sc2, C, k, sm);
+        if (WHERE == kSelLayer || per <= 16) return select_regs<16>(sc, sc2, C, k, sm);
+    }
+    if constexpr (WHERE == kSelLayerWide || WHERE == kSelAlone) {
         select_regs<24>(sc, sc2, C, k, sm);
-    } else {
+    } else if constexpr (WHERE != kSelLayer) {
         if (WHERE == kSelScratch || per <= 8) return select_core<8>(sc, sc2, C, k, sm, nullptr);
         if constexpr (WHERE != kSelScratch) select_core<16>(sc, sc2, C, k, sm, nullptr);
     }

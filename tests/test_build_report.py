@@ -25,7 +25,7 @@ def _spills(src):
 
 def test_layer_kernels_do_not_spill():
     spills = _spills("layer_resident.cu")
-    assert sum("layer_resident_kernel" in k for k in spills) == 18 and not any(spills.values()), spills
+    assert sum("layer_resident_kernel" in k for k in spills) == 36 and not any(spills.values()), spills
 
 
 # (two query tiles, or a ring that continues in scratch; the selection's longer bodies would spill here too)
