@@ -774,7 +774,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
             if constexpr (!BIG) {
                 // the head's records straight from the L2 (they were written by other SMs; every lane has
                 // acquired the counter), nine CTAs' worth of loads in flight per lane. Up to 64 rows each half of the warp
-                // takes every other record (2 heads: 69 CTAs, 32 layers of 8192 tokens 487 -> 335 us).
+                // takes every other record (2 heads: 69 CTAs, 32 layers of 8192 tokens 490 -> 330 us with the selection by runs).
                 const float* src = p.cta_stat + (static_cast<size_t>(s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * 256;
                 float M[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}, S[4] = {0.f, 0.f, 0.f, 0.f};
                 auto fold = [&](const float* from, auto stride, int n) {
