@@ -257,37 +257,28 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         // ------------------------------------------------------------------ UMMA issuer
         if (elect_one() && nt > 0) {
             bool ok = mbar_wait(smem_u32(&ctl.qfull), 0, abort_flag);
+            const uint64_t q_desc = umma_desc_sw128(q_base), k_desc = umma_desc_sw128(k_base);
+            const bool both = KB == 2;                   // d is 64 or 128: one or two stages a tile
             uint32_t st = 0, st_par = 0;
             for (int ti = 0, vt = 0; ti < nt && ok; ++ti) {
-                uint32_t st_kb[2] = {0u, 0u};
-#pragma unroll
-                for (int kb = 0; kb < 2; ++kb) {          // d is 64 or 128: one or two 64-element blocks
-                    if (kb >= KB || !ok) break;
-                    ok = mbar_wait(smem_u32(&ctl.full[st]), st_par, abort_flag);
-                    st_kb[kb] = st;
-                    if (++st == n_stages) { st = 0; st_par ^= 1u; }
-                }
-                for (int mt = 0; mt < n_mt && ok; ++mt, ++vt) {
+                const uint32_t s0 = st, p0 = st_par;
+                if (++st == n_stages) { st = 0; st_par ^= 1u; }
+                const uint32_t s1 = both ? st : s0, p1 = both ? st_par : p0;
+                if (both && ++st == n_stages) { st = 0; st_par ^= 1u; }
+                for (int mt = 0; mt < n_mt; ++mt, ++vt) {
                     const int buf = vt & 1, use = vt >> 1;
-                    ok = mbar_wait(smem_u32(&ctl.tempty[buf]), (use & 1) ^ 1, abort_flag);
+                    const uint32_t tempty = smem_u32(&ctl.tempty[buf]), te_par = (use & 1) ^ 1;
+                    ok = mt == 0 ? mbar_wait3(smem_u32(&ctl.full[s0]), p0, smem_u32(&ctl.full[s1]), p1, tempty, te_par, abort_flag)
+                                 : mbar_wait(tempty, te_par, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t d_addr = tmem_base + static_cast<uint32_t>(buf * kRUmmaN);
-#pragma unroll
-                    for (int kb = 0; kb < 2; ++kb) {
-                        if (kb >= KB) break;
-                        const uint64_t b_desc = umma_desc_sw128(k_base + st_kb[kb] * STAGE);
-                        const uint64_t a_desc = umma_desc_sw128(q_base + static_cast<uint32_t>(mt * KB + kb) * kRQTileBytes);
-#pragma unroll
-                        for (int k4 = 0; k4 < 4; ++k4)      // k-steps advance the start address by 32 bytes
-                            umma_bf16(d_addr, a_desc + 2u * k4, b_desc + 2u * k4, IDESC, (kb > 0 || k4 > 0) ? 1u : 0u);
-                    }
+                    issue_products(tmem_base + static_cast<uint32_t>(buf * kRUmmaN), q_desc + static_cast<uint32_t>(mt * KB) * (kRQTileBytes >> 4),
+                                   k_desc + s0 * (STAGE >> 4), k_desc + s1 * (STAGE >> 4), both, IDESC);
                     umma_commit(smem_u32(&ctl.tfull[buf]));
                 }
                 if (!ok) break;
-#pragma unroll
-                for (int kb = 0; kb < 2; ++kb)
-                    if (kb < KB) umma_commit(smem_u32(&ctl.empty[st_kb[kb]]));
+                umma_commit(smem_u32(&ctl.empty[s0]));
+                if (both) umma_commit(smem_u32(&ctl.empty[s1]));
             }
         }
     } else {

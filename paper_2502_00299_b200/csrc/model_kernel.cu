@@ -434,6 +434,8 @@ model_kernel(const __grid_constant__ ModelParams p) {
     } else if (warp == 1) {
         // ------------------------------------------------------------------ UMMA issuer
         if (elect_one() && nt > 0) {
+            const uint64_t q_desc = umma_desc_sw128(q_base), k_desc = umma_desc_sw128(k_base);
+            const bool both = KB == 2;                   // d is 64 or 128: one or two stages a tile
             uint32_t st = 0, st_par = 0;
             uint32_t buf = 0, aslot = 0, e_slot = kMAccSlots - kMAccBufs, e_par = 1;   // small: accumulator, (accumulator, group) slot; slot to wait for
             int vg = 0;                  // virtual tiles issued so far (all layers); the epilogue pair vg & 1 reads tile vg
@@ -441,61 +443,43 @@ model_kernel(const __grid_constant__ ModelParams p) {
             for (int s = 0; s < p.n_compute && ok; ++s) {
                 ok = mbar_wait(smem_u32(&ctl.qfull), s & 1, abort_flag);
                 for (int ti = 0; ti < nt && ok; ++ti) {
-                    uint32_t st_kb[2] = {0u, 0u};
-#pragma unroll
-                    for (int kb = 0; kb < 2; ++kb) {
-                        if (kb >= KB || !ok) break;
-                        ok = mbar_wait(smem_u32(&ctl.full[st]), st_par, abort_flag);
-                        st_kb[kb] = st;
-                        if (++st == n_stages) { st = 0; st_par ^= 1u; }
-                    }
-                    if (!ok) break;
-                    for (int mt = 0; mt < n_mt && ok; ++mt, ++vg) {
-                        if constexpr (BIG) {
+                    const uint32_t s0 = st, p0 = st_par;
+                    if (++st == n_stages) { st = 0; st_par ^= 1u; }
+                    const uint32_t s1 = both ? st : s0, p1 = both ? st_par : p0;
+                    if (both && ++st == n_stages) { st = 0; st_par ^= 1u; }
+                    const uint32_t full0 = smem_u32(&ctl.full[s0]), full1 = smem_u32(&ctl.full[s1]);
+                    if constexpr (BIG) {
+                        for (int mt = 0; mt < n_mt; ++mt, ++vg) {
                             const uint32_t ab = vg & 1;
-                            ok = mbar_wait(smem_u32(&ctl.tempty[ab]), ((vg >> 1) & 1) ^ 1, abort_flag);
+                            const uint32_t tempty = smem_u32(&ctl.tempty[ab]), te_par = ((vg >> 1) & 1) ^ 1;
+                            ok = mt == 0 ? mbar_wait3(full0, p0, full1, p1, tempty, te_par, abort_flag) : mbar_wait(tempty, te_par, abort_flag);
                             if (!ok) break;
                             tc_fence_after();
-                            const uint32_t d_addr = tmem_base + ab * kRUmmaN;
-#pragma unroll
-                            for (int kb = 0; kb < 2; ++kb) {
-                                if (kb >= KB) break;
-                                const uint64_t b_desc = umma_desc_sw128(k_base + st_kb[kb] * STAGE);
-                                const uint64_t a_desc = umma_desc_sw128(q_base + static_cast<uint32_t>(mt * KB + kb) * kRQTileBytes);
-#pragma unroll
-                                for (int k4 = 0; k4 < 4; ++k4)
-                                    umma_bf16(d_addr, a_desc + 2u * k4, b_desc + 2u * k4, IDESC, (kb > 0 || k4 > 0) ? 1u : 0u);
-                            }
+                            issue_products(tmem_base + ab * kRUmmaN, q_desc + static_cast<uint32_t>(mt * KB) * (kRQTileBytes >> 4),
+                                           k_desc + s0 * (STAGE >> 4), k_desc + s1 * (STAGE >> 4), both, IDESC);
                             umma_commit(smem_u32(&ctl.tfull[ab]));
-                        } else {
+                        }
+                    } else {
 #pragma unroll
-                            for (int half = 0; half < 2; ++half) {
-                                // a panel goes to accumulator (panel number % 3), which the third panel before it used last:
-                                // wait until that one's group has read it (the first three panels find a fresh barrier)
-                                ok = mbar_wait(smem_u32(&ctl.tempty[e_slot]), e_par, abort_flag);
-                                if (++e_slot == kMAccSlots) { e_slot = 0; e_par ^= 1u; }
-                                if (!ok) break;
-                                tc_fence_after();
-                                const uint32_t d_addr = tmem_base + buf * kMAccN;
-#pragma unroll
-                                for (int kb = 0; kb < 2; ++kb) {
-                                    if (kb >= KB) break;
-                                    const uint64_t b_desc = umma_desc_sw128(k_base + st_kb[kb] * STAGE + static_cast<uint32_t>(half * ACC1 * 128));
-                                    const uint64_t a_desc = umma_desc_sw128(q_base + static_cast<uint32_t>(kb) * kRQTileBytes);
-#pragma unroll
-                                    for (int k4 = 0; k4 < 4; ++k4)
-                                        umma_bf16(d_addr, a_desc + 2u * k4, b_desc + 2u * k4, IDESC, (kb > 0 || k4 > 0) ? 1u : 0u);
-                                }
-                                umma_commit(smem_u32(&ctl.tfull[aslot]));
-                                if (++buf == kMAccBufs) buf = 0;
-                                if (++aslot == kMAccSlots) aslot = 0;
-                            }
+                        for (int half = 0; half < 2; ++half) {
+                            // a panel goes to accumulator (panel number % 3), which the third panel before it used last:
+                            // wait until that one's group has read it (the first three panels find a fresh barrier)
+                            const uint32_t tempty = smem_u32(&ctl.tempty[e_slot]);
+                            ok = half == 0 ? mbar_wait3(full0, p0, full1, p1, tempty, e_par, abort_flag) : mbar_wait(tempty, e_par, abort_flag);
+                            if (++e_slot == kMAccSlots) { e_slot = 0; e_par ^= 1u; }
+                            if (!ok) break;
+                            tc_fence_after();
+                            const uint32_t half_off = static_cast<uint32_t>(half * ACC1 * 128) >> 4;
+                            issue_products(tmem_base + buf * kMAccN, q_desc, k_desc + s0 * (STAGE >> 4) + half_off, k_desc + s1 * (STAGE >> 4) + half_off,
+                                           both, IDESC);
+                            umma_commit(smem_u32(&ctl.tfull[aslot]));
+                            if (++buf == kMAccBufs) buf = 0;
+                            if (++aslot == kMAccSlots) aslot = 0;
                         }
                     }
                     if (!ok) break;
-#pragma unroll
-                    for (int kb = 0; kb < 2; ++kb)
-                        if (kb < KB) umma_commit(smem_u32(&ctl.empty[st_kb[kb]]));
+                    umma_commit(smem_u32(&ctl.empty[s0]));
+                    if (both) umma_commit(smem_u32(&ctl.empty[s1]));
                 }
                 if (ok) umma_commit(smem_u32(&ctl.qempty));       // every UMMA of this layer has read the Q tile
             }

@@ -69,6 +69,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// Bounded waits for three phases. The first tests travel together: a test takes some 60 clocks to come back, and a thread
+// that issues products waits for phases which mostly lie behind it.
+__device__ __forceinline__ bool mbar_wait3(uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1, uint32_t bar2, uint32_t par2,
+                                           volatile int* abort_flag) {
+    const bool r0 = mbar_try_wait(bar0, par0), r1 = mbar_try_wait(bar1, par1), r2 = mbar_try_wait(bar2, par2);
+    return (r0 || mbar_wait(bar0, par0, abort_flag)) && (r1 || mbar_wait(bar1, par1, abort_flag)) && (r2 || mbar_wait(bar2, par2, abort_flag));
+}
+__device__ __forceinline__ bool mbar_wait2(uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1, volatile int* abort_flag) {
+    const bool r0 = mbar_try_wait(bar0, par0), r1 = mbar_try_wait(bar1, par1);
+    return (r0 || mbar_wait(bar0, par0, abort_flag)) && (r1 || mbar_wait(bar1, par1, abort_flag));
+}
+
 // ----------------------------------------------------------------------------- TMA
 __device__ __forceinline__ void prefetch_tmap(const void* tmap) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");

@@ -18,6 +18,17 @@ constexpr int kRQTileBytes = 128 * 128;
 // Keys per epilogue panel (half a tile) for a chunk size: a multiple of it, so that no chunk straddles panels.
 __host__ __device__ constexpr int panel_keys(int c) { return (c == 8 || c == 16 || c == 32) ? 64 : kRPanel; }
 
+// One accumulator tile: the products of 64 or 128 dims, four of 16 dims per ring stage (k-steps advance the start address by 32
+// bytes). The descriptors come ready made, so that the issuing thread only adds constants between two products.
+__device__ __forceinline__ void issue_products(uint32_t d_addr, uint64_t q_desc, uint64_t k_desc0, uint64_t k_desc1, bool both, uint32_t idesc) {
+#pragma unroll
+    for (int k4 = 0; k4 < 4; ++k4) umma_bf16(d_addr, q_desc + 2u * k4, k_desc0 + 2u * k4, idesc, k4 > 0 ? 1u : 0u);
+    if (both) {
+#pragma unroll
+        for (int k4 = 0; k4 < 4; ++k4) umma_bf16(d_addr, q_desc + (kRQTileBytes >> 4) + 2u * k4, k_desc1 + 2u * k4, idesc, 1u);
+    }
+}
+
 // A panel's chunk partial sums to and from consecutive tensor-memory columns.
 template <int N>
 __device__ __forceinline__ void part_store(uint32_t taddr, const float (&p)[N]) {
