@@ -397,27 +397,36 @@ model_kernel(const __grid_constant__ ModelParams p) {
             uint32_t st = 0, st_par = 1;
             int issued = 0;
             bool ok = true;
+            // A layer's first key tiles go ahead of its queries: the Q tile is free only when the last product of the layer before has
+            // read it, and by then the stages that were free earlier hold keys. Before this, the K stream stopped at every layer until the
+            // ring had run empty (5.5k of 30.5k clocks a layer of 32768 tokens, 128 rows). As many stages as are not the layer before's last tile
+            // (its products end together with the Q tile's use).
+            const int n_k = nt * KB, q_at = min(n_k, p.n_stages - KB);
             for (int s = 0; s < p.n_compute && ok; ++s) {
                 prefetch_tmap(&p.tm_q[s]);
                 prefetch_tmap(&p.tm_k[s]);
-                // the Q tile is free again once the last UMMA of the previous layer has read it
-                if (s > 0) ok = mbar_wait(smem_u32(&ctl.qempty), (s - 1) & 1, abort_flag);
-                if (!ok) break;
-                mbar_arrive_expect_tx(qbar, q_bytes);
-                for (int mt = 0; mt < n_mt; ++mt)    // (rows past R of the second tile arrive as zeros)
-                    for (int kb = 0; kb < KB; ++kb)
-                        tma_load_3d(q_base + static_cast<uint32_t>(mt * KB + kb) * kRQTileBytes, &p.tm_q[s], qbar, kb * 64, mt * 128, hkv);
-                for (int t = t_begin; t < t_end && ok; ++t) {
-                    for (int kb = 0; kb < KB; ++kb) {
-                        ok = mbar_wait(smem_u32(&ctl.empty[st]), st_par, abort_flag);
+                for (int mt = 0; mt < n_mt; ++mt)
+                    for (int kb = 0; kb < KB; ++kb) tma_prefetch_3d(&p.tm_q[s], kb * 64, mt * 128, hkv);
+                int t = t_begin, kb = 0;
+                for (int i = 0; i <= n_k; ++i) {
+                    if (i == (s == 0 ? 0 : q_at)) {
+                        if (s > 0) ok = mbar_wait(smem_u32(&ctl.qempty), (s - 1) & 1, abort_flag);
                         if (!ok) break;
-                        const uint32_t bar = smem_u32(&ctl.full[st]);
-                        mbar_arrive_expect_tx(bar, k_bytes);
-                        if constexpr (BIG) tma_load_3d_hint(k_base + st * STAGE, &p.tm_k[s], bar, kb * 64, t * TILE, hkv, policy);
-                        else tma_load_3d(k_base + st * STAGE, &p.tm_k[s], bar, kb * 64, t * TILE, hkv);
-                        ++issued;
-                        if (++st == n_stages) { st = 0; st_par ^= 1u; }
+                        mbar_arrive_expect_tx(qbar, q_bytes);
+                        for (int mt = 0; mt < n_mt; ++mt)    // (rows past R of the second tile arrive as zeros)
+                            for (int b = 0; b < KB; ++b)
+                                tma_load_3d(q_base + static_cast<uint32_t>(mt * KB + b) * kRQTileBytes, &p.tm_q[s], qbar, b * 64, mt * 128, hkv);
                     }
+                    if (i == n_k) break;
+                    ok = mbar_wait(smem_u32(&ctl.empty[st]), st_par, abort_flag);
+                    if (!ok) break;
+                    const uint32_t bar = smem_u32(&ctl.full[st]);
+                    mbar_arrive_expect_tx(bar, k_bytes);
+                    if constexpr (BIG) tma_load_3d_hint(k_base + st * STAGE, &p.tm_k[s], bar, kb * 64, t * TILE, hkv, policy);
+                    else tma_load_3d(k_base + st * STAGE, &p.tm_k[s], bar, kb * 64, t * TILE, hkv);
+                    ++issued;
+                    if (++st == n_stages) { st = 0; st_par ^= 1u; }
+                    if (++kb == KB) { kb = 0; ++t; }
                 }
             }
             if (!ok) {
