@@ -328,12 +328,8 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 else if (active)
                     spill_store<SPP + 1, 0>(a.spill + at * ((SPP + 1) * a.spill_rows), a.spill_rows, row, rec_, keep);
             }
-            // fold into the running record: l is relative to m2, run_l to run_m
-            const float nm = fmaxf(run_m, m2);
-            const float s_old = (run_m == -CUDART_INF_F) ? 0.f : ex2_approx(run_m - nm);
-            const float s_new = (m2 == -CUDART_INF_F) ? 0.f : ex2_approx(m2 - nm);
-            run_l = run_l * s_old + l * s_new;
-            run_m = nm;
+            // the running record: l is relative to m2, run_l to run_m
+            merge_ml(run_m, run_l, m2, l);
         }
         tmem_st_wait();
         rec[(grp * 2 + 0) * 128 + row] = active ? run_m : -CUDART_INF_F;
@@ -358,7 +354,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             for (int g = 0; g < 4; ++g)
                 if (g >= g0 && g < g1) {
                     const float m = rec[(g * 2) * 128 + i];
-                    Ls += (m == -CUDART_INF_F) ? 0.f : rec[(g * 2 + 1) * 128 + i] * ex2_approx(m - M);
+                    Ls += rec[(g * 2 + 1) * 128 + i] * exp2_int(m - M);
                 }
             float* dst = a.cta_stat + (static_cast<size_t>(blockIdx.x) * n_mt + (threadIdx.x >> 7)) * 256;
             dst[i] = M;
@@ -419,9 +415,9 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                     float bm = M;
 #pragma unroll
                     for (int u = 0; u < kF; ++u) bm = fmaxf(bm, rm[u]);
-                    float acc = (M == -CUDART_INF_F) ? 0.f : Ls * ex2_approx(M - bm);
+                    float acc = Ls * exp2_int(M - bm);
 #pragma unroll
-                    for (int u = 0; u < kF; ++u) acc += (rm[u] == -CUDART_INF_F) ? 0.f : rl[u] * ex2_approx(rm[u] - bm);
+                    for (int u = 0; u < kF; ++u) acc += rl[u] * exp2_int(rm[u] - bm);
                     M = bm;
                     Ls = acc;
                 }
@@ -439,7 +435,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 for (int s = 0; s < 4; ++s)
                     if (s >= s0 && s < s0 + n_sl) {
                         const float m = slice[(s * 2) * 128 + i];
-                        Ls += (m == -CUDART_INF_F) ? 0.f : slice[(s * 2 + 1) * 128 + i] * ex2_approx(m - M);
+                        Ls += slice[(s * 2 + 1) * 128 + i] * exp2_int(m - M);
                     }
                 gm[threadIdx.x] = M;
                 ginv[threadIdx.x] = 1.0f / Ls;       // rows >= R are never used
@@ -500,7 +496,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 #pragma unroll
                 for (int u = 0; u < PPB; ++u) {
                     const bool have = active && grp + 4 * (b0 + u) < n_pl;
-                    const float f = have ? ex2_approx(pm[u] - mi) * li : 0.f;
+                    const float f = have ? exp2_int(pm[u] - mi) * li : 0.f;
 #pragma unroll
                     for (int s = 0; s < SPP; ++s) v[u * SPP + s] = have ? v[u * SPP + s] * f : 0.f;
                 }

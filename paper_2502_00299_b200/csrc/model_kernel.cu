@@ -163,10 +163,9 @@ __device__ __forceinline__ void bulk_wait_read() {
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // Fold N (max, sum-of-exp2) records into (M, S), one row each of four rows at a time: the new maximum
-// first, then N independent exponentials (a short dependency chain, unlike N merges in sequence).
+// first, then N independent factors (a short dependency chain, unlike N merges in sequence).
 template <int N>
 __device__ __forceinline__ void merge_batch(float (&M)[4], float (&S)[4], const float4 (&m)[N], const float4 (&l)[N], int n) {
-    const float ninf = -CUDART_INF_F;
     float nm[4] = {M[0], M[1], M[2], M[3]};
 #pragma unroll
     for (int j = 0; j < N; ++j)
@@ -177,14 +176,14 @@ __device__ __forceinline__ void merge_batch(float (&M)[4], float (&S)[4], const 
             nm[3] = fmaxf(nm[3], m[j].w);
         }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) S[r] = (M[r] == ninf) ? 0.f : S[r] * ex2_approx(M[r] - nm[r]);
+    for (int r = 0; r < 4; ++r) S[r] *= exp2_int(M[r] - nm[r]);
 #pragma unroll
     for (int j = 0; j < N; ++j)
         if (j < n) {
-            S[0] += (m[j].x == ninf) ? 0.f : l[j].x * ex2_approx(m[j].x - nm[0]);
-            S[1] += (m[j].y == ninf) ? 0.f : l[j].y * ex2_approx(m[j].y - nm[1]);
-            S[2] += (m[j].z == ninf) ? 0.f : l[j].z * ex2_approx(m[j].z - nm[2]);
-            S[3] += (m[j].w == ninf) ? 0.f : l[j].w * ex2_approx(m[j].w - nm[3]);
+            S[0] += l[j].x * exp2_int(m[j].x - nm[0]);
+            S[1] += l[j].y * exp2_int(m[j].y - nm[1]);
+            S[2] += l[j].z * exp2_int(m[j].z - nm[2]);
+            S[3] += l[j].w * exp2_int(m[j].w - nm[3]);
         }
 #pragma unroll
     for (int r = 0; r < 4; ++r) M[r] = nm[r];
@@ -570,9 +569,9 @@ model_kernel(const __grid_constant__ ModelParams p) {
                         float bm = M;
 #pragma unroll
                         for (int j = 0; j < 9; ++j) bm = fmaxf(bm, rm[j]);
-                        float acc = (M == -CUDART_INF_F) ? 0.f : S * ex2_approx(M - bm);
+                        float acc = S * exp2_int(M - bm);
 #pragma unroll
-                        for (int j = 0; j < 9; ++j) acc += (rm[j] == -CUDART_INF_F) ? 0.f : rl[j] * ex2_approx(rm[j] - bm);
+                        for (int j = 0; j < 9; ++j) acc += rl[j] * exp2_int(rm[j] - bm);
                         M = bm;
                         S = acc;
                     }
@@ -623,7 +622,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
 #pragma unroll
                 for (int u = 0; u < PPB; ++u) {
                     const bool have = active && b0 + u < own;
-                    const float f = have ? ex2_approx(pm[u] - mi) * li : 0.f;
+                    const float f = have ? exp2_int(pm[u] - mi) * li : 0.f;
 #pragma unroll
                     for (int q = 0; q < SPP; ++q) v[u * SPP + q] = have ? v[u * SPP + q] * f : 0.f;
                 }
@@ -695,11 +694,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                     part_store<SPP>(lane_addr + static_cast<uint32_t>(PART0 + slot * SPP), pr);
                     pmax[slot * 128 + row] = m2;
                 }
-                const float nm = fmaxf(run_m, m2);
-                const float s_old = (run_m == -CUDART_INF_F) ? 0.f : ex2_approx(run_m - nm);
-                const float s_new = (m2 == -CUDART_INF_F) ? 0.f : ex2_approx(m2 - nm);
-                run_l = run_l * s_old + l * s_new;
-                run_m = nm;
+                merge_ml(run_m, run_l, m2, l);
             }
         };
         // end of slot s: this group's (max, sum) per row -> shared memory; the statistics warp merges the four

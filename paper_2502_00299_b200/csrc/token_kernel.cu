@@ -234,11 +234,7 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                     panel_fast<8, kTPanel>(v, a.sl2, emit, &m2, &l);
                 else
                     panel_static_tail<8, kTPanel>(v, a.sl2, emit, j0, a.P, last_visible, &m2, &l);
-                const float nm = fmaxf(run_m, m2);
-                const float s_old = (run_m == -CUDART_INF_F) ? 0.f : ex2_approx(run_m - nm);
-                const float s_new = (m2 == -CUDART_INF_F) ? 0.f : ex2_approx(m2 - nm);
-                run_l = run_l * s_old + l * s_new;
-                run_m = nm;
+                merge_ml(run_m, run_l, m2, l);
             }
         }
         rec[(grp * 2 + 0) * 128 + row] = active ? run_m : -CUDART_INF_F;
