@@ -77,6 +77,7 @@ __host__ __device__ constexpr int model_copy_slots(int c, int d) {
     const int n = 40960 / (4 * c * d);
     return n > kMSlots ? kMSlots : (n < 3 ? 3 : n);
 }
+constexpr int kMOwnMerge = 36;                     // CTAs a head up to which the epilogue threads merge their rows' records
 constexpr int kBarGroup = 2;                       // named barriers 2 .. 5: the four warps of an epilogue group
 
 struct ModelCtl {
@@ -90,8 +91,9 @@ struct ModelCtl {
     unsigned long long gfull[kMSlots];
     unsigned long long sfull;          // a kept-chunk list has landed in shared memory (copy thread)
     unsigned long long stat_full[2];   // m_i and 1 / l_i of a slot are in shared memory (statistics warps -> epilogue)
-    unsigned long long pub_done[2];    // every epilogue warp has stored its part of the slot's record (-> statistics warp)
+    unsigned long long pub_done[2];    // the slot's record is stored, 32 rows an arrival (-> statistics warp)
     unsigned long long sc_done[2];     // every epilogue warp has stored its chunk scores of the slot (-> statistics warp)
+    int pub_count[2][2][4];            // epilogue warps that have left their part of a slot's record: [slot parity][query tile][32 rows]
     uint32_t tmem_base;
     int abort_flag;
     int sel_flag[2];                   // selector CTAs: wait result, abort flag
@@ -346,6 +348,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
     const int n_mt = BIG ? p.n_mt : 1;
     const bool two = n_mt == 2;
     const int n_vt = two ? 2 * nt : nt;              // virtual tiles of this CTA per layer
+    const bool own_merge = BIG || p.cph <= kMOwnMerge;      // epilogue threads merge their rows' records themselves
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.n_stages; ++s) {
@@ -363,9 +366,10 @@ model_kernel(const __grid_constant__ ModelParams p) {
         mbar_init(smem_u32(&ctl.stat_full[0]), 1);
         mbar_init(smem_u32(&ctl.stat_full[1]), 1);
         for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&ctl.pub_done[b]), 16);
+            mbar_init(smem_u32(&ctl.pub_done[b]), 4 * n_mt);
             mbar_init(smem_u32(&ctl.sc_done[b]), 16);
         }
+        for (int i = 0; i < 16; ++i) (&ctl.pub_count[0][0][0])[i] = 0;
         ctl.abort_flag = 0;
         fence_mbar_init();
         fence_proxy_async();
@@ -550,10 +554,10 @@ model_kernel(const __grid_constant__ ModelParams p) {
                 if (!__shfl_sync(0xffffffffu, ready, 0)) ok = false;   // (the failed wait has raised the abort flag)
                 __syncwarp();          // orders the other lanes' reads below behind the wait; a shuffle alone does not
                 tmem_st_wait();
-                if constexpr (BIG) {
+                if (own_merge) {
                     // every record of the head is there (the statistics warp has seen the count): each thread merges those of
-                    // its row, straight from the L2. 18 records of two query tiles took the statistics warp 8 us beside four
-                    // busy warps, 128 threads a group take 1.5.
+                    // its row, straight from the L2. 18 records took the statistics warp 3 us of a layer's 16 beside four busy
+                    // warps (two query tiles: 8), a group's 128 threads take 0.5; with very many it is the warp's again, which no one waits for.
                     float M = -CUDART_INF_F, S = 0.f;
                     const size_t step = static_cast<size_t>(n_mt) * 256;
                     const float* src = p.cta_stat + ((static_cast<size_t>(c_s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * n_mt +
@@ -579,7 +583,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                     gstat[grp * 256 + 128 + row] = 1.0f / S;
                 }
             }
-            const float* gm = gstat + (BIG ? grp : c_s & 1) * 256;
+            const float* gm = gstat + (own_merge ? grp : c_s & 1) * 256;
             const float mi = gm[row], li = gm[128 + row];
             float* rb = rg + c_par * (4 * kMBlkSlots);
             if (own > 0) {
@@ -697,16 +701,36 @@ model_kernel(const __grid_constant__ ModelParams p) {
                 merge_ml(run_m, run_l, m2, l);
             }
         };
-        // end of slot s: this group's (max, sum) per row -> shared memory; the statistics warp merges the four
-        // groups, stores the CTA's record and announces it (no block-wide barrier on the scoring warps' path)
+        // end of slot s: this group's (max, sum) per row -> shared memory. The last of the groups' warps that hold the same 32 rows
+        // merges their parts and stores them; the statistics warp announces the CTA's record when all of it is there (no
+        // block-wide barrier on the scoring warps' path).
         auto publish = [&](int s) {
             float* rc = rec + (s & 1) * 3072;
             rc[(grp * 2 + 0) * 128 + row] = active ? run_m : -CUDART_INF_F;
             rc[(grp * 2 + 1) * 128 + row] = active ? run_l : 0.f;
             run_m = -CUDART_INF_F;
             run_l = 0.f;
+            __threadfence_block();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&ctl.pub_done[s & 1]));
+            const int mt = two ? pair : 0, n_g = two ? 2 : 4;
+            int* cnt = &ctl.pub_count[s & 1][mt][quarter];
+            int old = 0;
+            if (lane == 0) old = atomicAdd(cnt, 1);
+            if (__shfl_sync(0xffffffffu, old, 0) == n_g - 1) {
+                __threadfence_block();
+                float M = -CUDART_INF_F, S = 0.f;
+#pragma unroll
+                for (int g = 0; g < 4; ++g)
+                    if (g < n_g) merge_ml(M, S, rc[((mt * 2 + g) * 2) * 128 + row], rc[((mt * 2 + g) * 2 + 1) * 128 + row]);
+                float* dst = p.cta_stat + ((static_cast<size_t>(s & 1) * gridDim.x + blockIdx.x) * n_mt + mt) * 256;
+                dst[row] = M;
+                dst[128 + row] = S;
+                __syncwarp();
+                if (lane == 0) {
+                    *cnt = 0;
+                    mbar_arrive(smem_u32(&ctl.pub_done[s & 1]));
+                }
+            }
         };
         for (int s = 0; s <= p.n_compute && alive; ++s) {
             if (s < p.n_compute) do_layer(s);
@@ -734,32 +758,10 @@ model_kernel(const __grid_constant__ ModelParams p) {
                 w_ok = mbar_wait(smem_u32(&ctl.pub_done[s & 1]), static_cast<uint32_t>(s >> 1) & 1u, abort_flag);
             if (!__shfl_sync(0xffffffffu, w_ok, 0)) break;
             __syncwarp();              // (as above: the other lanes read what the epilogue warps left in shared memory)
-            {
-                // every epilogue warp has left its group's (max, sum) per row in shared memory: merge the
-                // four groups (this lane: rows 4 lane .. 4 lane + 3), store the CTA's record and announce it.
-                // release: the record stores of the whole warp, ordered by __syncwarp, are visible to whoever
-                // sees the count
-                const float* rc = rec + (s & 1) * 3072;
-                for (int mt = 0; mt < n_mt; ++mt) {
-                    float Mo[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}, So[4] = {0.f, 0.f, 0.f, 0.f};
-                    float4 m[4], l[4];
-                    const int n_g = two ? 2 : 4;         // groups that scored this query tile
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        const int gg = two ? mt * 2 + (g & 1) : g;
-                        m[g] = *reinterpret_cast<const float4*>(rc + (gg * 2) * 128 + r0);
-                        l[g] = *reinterpret_cast<const float4*>(rc + (gg * 2 + 1) * 128 + r0);
-                    }
-                    merge_batch<4>(Mo, So, m, l, n_g);
-                    float* dst = p.cta_stat + ((static_cast<size_t>(s & 1) * gridDim.x + blockIdx.x) * n_mt + mt) * 256;
-                    *reinterpret_cast<float4*>(dst + r0) = make_float4(Mo[0], Mo[1], Mo[2], Mo[3]);
-                    *reinterpret_cast<float4*>(dst + 128 + r0) = make_float4(So[0], So[1], So[2], So[3]);
-                }
-                __syncwarp();
-            }
+            // release, behind the wait that acquired what the epilogue warps stored: the record is visible to whoever sees the count
             if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.cnt_a + hkv) : "memory");
             if (!wait_counter_warp(p.cnt_a + hkv, static_cast<unsigned>(s + 1) * p.cph, abort_flag)) break;
-            if constexpr (!BIG) {
+            if (!own_merge) {
                 // the head's records straight from the L2 (they were written by other SMs; every lane has
                 // acquired the counter), nine CTAs' worth of loads in flight per lane. Up to 64 rows each half of the warp
                 // takes every other record (2 heads: 69 CTAs, 32 layers of 8192 tokens 490 -> 330 us with the selection by runs).
