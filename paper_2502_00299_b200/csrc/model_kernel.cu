@@ -17,7 +17,7 @@
 //                  on with the next layer; when the head's row statistics have arrived (normally long
 //                  before they are needed) it contracts the partial sums it wrote itself over the rows
 //                  into chunk scores of the CTA's key range (global memory)
-//   warp 18        one thread: for each computed layer, once a selector CTA has published the head's
+//   warp 18        for each computed layer, once a selector CTA has published the head's
 //                  kept-chunk list, moves this CTA's share of the kept K/V rows with bulk asynchronous
 //                  copies (global -> shared -> global, whole chunks at a time) - for the computed
 //                  layer and for every following layer that reuses its indices
@@ -809,46 +809,53 @@ model_kernel(const __grid_constant__ ModelParams p) {
         }
     } else if (warp == 18) {
         // ------------------------------------------------------------------ tail: row copies
-        // One thread: waits until the selector CTA has published the head's kept-chunk list of a
-        // slot, fetches the list, and moves this CTA's share of the rows - whole chunks and window
-        // pieces - through the staging slots with bulk copies, for the computed layer and for every
-        // layer that reuses its indices. Rows that are not adjacent in memory (e.g. token-major caches)
+        // Once the selector CTA has published the head's kept-chunk list of a slot, this warp fetches the list and moves this
+        // CTA's share of the rows - whole chunks and window pieces - through the staging slots with bulk copies, for the computed
+        // layer and for every layer that reuses its indices. Rows that are not adjacent in memory (e.g. token-major caches)
         // arrive through tensor maps whose box is a chunk: one copy as well, whatever the strides.
-        if (lane == 0) {
-            uint8_t* tbase = dyn + p.off_tail;
-            int* row = reinterpret_cast<int*>(tbase);        // [4 + kkpad]: n_tok, -, -, -, kept chunk ids
-            const uint32_t stage0 = smem_u32(tbase + p.sel_row_bytes);
-            const int* sel = row + 4;
-            const int Q = p.cph, q = part;                   // CTAs of this KV head
-            constexpr uint32_t kSl = C_STATIC <= 10 ? kMSlots : 0;   // staging slots where every head dim has the most
-            const uint32_t n_slots = kSl ? kSl : static_cast<uint32_t>(p.copy_slots);
-            const int kk = min(p.k, p.C);
-            const int wu = (p.w + C_STATIC - 1) / C_STATIC;  // the window as pseudo-chunks of up to c rows
-            const int U = kk + wu;                           // copy units of the head
-            const int u_begin = static_cast<int>(static_cast<long long>(U) * q / Q);
-            const int u_end = static_cast<int>(static_cast<long long>(U) * (q + 1) / Q);
-            const int n_units = u_end - u_begin;
-            const uint32_t row_bytes = static_cast<uint32_t>(p.d) * 2u;
-            const uint32_t half_slot = static_cast<uint32_t>(p.stage_slot_bytes) / 2u;
-            uint32_t g_issued = 0;                           // units loaded so far (all layers): slot = g % n_slots
-            bool ok = true;
-            for (int li = 0; li < p.n_layers && ok;) {
-                const int s = p.layer[li].slot;
-                {
-                    ok = wait_counter(p.cnt_c + hkv, static_cast<unsigned>(s + 1), abort_flag, 200);
-                    if (ok) {
-                        asm volatile("fence.acq_rel.gpu;" ::: "memory");
-                        const uint32_t bar = smem_u32(&ctl.sfull);
-                        mbar_arrive_expect_tx(bar, static_cast<uint32_t>(p.sel_row_bytes));
-                        // the list was written with ordinary stores by the selector CTA
-                        asm volatile("fence.proxy.async.global;" ::: "memory");
-                        bulk_load(smem_u32(row), p.sel_rows + (static_cast<size_t>(s) * p.Hkv + hkv) * (p.sel_row_bytes / 4),
-                                  static_cast<uint32_t>(p.sel_row_bytes), bar);
-                    }
+        // The units of all these layers are one sequence; a round takes `lanes` of them, a lane each, through one of n_sets sets of
+        // slots, so that a set is loaded while the others are stored. What bounds this warp is not the copies but its own instructions,
+        // which wait for their turn beside 16 busy warps: one thread took 630 ns a unit, of which 60 waiting for copies (32768
+        // tokens; 420 ns when nothing else ran), more than the scoring took where two layers share a list.
+        uint8_t* tbase = dyn + p.off_tail;
+        int* row = reinterpret_cast<int*>(tbase);            // [4 + kkpad]: n_tok, -, -, -, kept chunk ids
+        const uint32_t stage0 = smem_u32(tbase + p.sel_row_bytes);
+        const int* sel = row + 4;
+        const int Q = p.cph, q = part;                       // CTAs of this KV head
+        constexpr int kSl = C_STATIC <= 10 ? kMSlots : 0;    // staging slots where every head dim has the most
+        const int n_slots = kSl ? kSl : p.copy_slots;
+        const int lanes = n_slots >= 4 ? n_slots / 2 : 1, n_sets = n_slots >= 4 ? 2 : n_slots;
+        const int kk = min(p.k, p.C);
+        const int wu = (p.w + C_STATIC - 1) / C_STATIC;      // the window as pseudo-chunks of up to c rows
+        const int U = kk + wu;                               // copy units of the head
+        const int u_begin = static_cast<int>(static_cast<long long>(U) * q / Q);
+        const int u_end = static_cast<int>(static_cast<long long>(U) * (q + 1) / Q);
+        const int n_units = u_end - u_begin;
+        const uint32_t row_bytes = static_cast<uint32_t>(p.d) * 2u;
+        const uint32_t half_slot = static_cast<uint32_t>(p.stage_slot_bytes) / 2u;
+        uint32_t phase = 0;                                  // parity of this lane's next wait, a bit per set
+        bool ok = true;
+        for (int li = 0; li < p.n_layers;) {
+            const int s = p.layer[li].slot;
+            int lj_end = li + 1;
+            while (lj_end < p.n_layers && !p.layer[lj_end].computes) ++lj_end;
+            if (lane == 0) {
+                ok = wait_counter(p.cnt_c + hkv, static_cast<unsigned>(s + 1), abort_flag, 200);
+                if (ok) {
+                    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+                    const uint32_t bar = smem_u32(&ctl.sfull);
+                    mbar_arrive_expect_tx(bar, static_cast<uint32_t>(p.sel_row_bytes));
+                    // the list was written with ordinary stores by the selector CTA
+                    asm volatile("fence.proxy.async.global;" ::: "memory");
+                    bulk_load(smem_u32(row), p.sel_rows + (static_cast<size_t>(s) * p.Hkv + hkv) * (p.sel_row_bytes / 4),
+                              static_cast<uint32_t>(p.sel_row_bytes), bar);
                 }
-                if (ok) ok = mbar_wait(smem_u32(&ctl.sfull), static_cast<uint32_t>(s) & 1u, abort_flag);
-                if (!ok) break;
-                const int n_tok = row[0];
+            }
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            if (ok) ok = mbar_wait(smem_u32(&ctl.sfull), static_cast<uint32_t>(s) & 1u, abort_flag);
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+            const int n_tok = row[0];
+            if (lane < lanes && n_units > 0) {
                 auto unit = [&](int u, int& src_row, int& dst_row, int& rows) {
                     if (u < kk) {
                         src_row = sel[u] * C_STATIC;
@@ -861,63 +868,68 @@ model_kernel(const __grid_constant__ ModelParams p) {
                         rows = min(C_STATIC, p.L - src_row);
                     }
                 };
-                int lj = li;
-                do {
-                    const ModelLayer& ly = p.layer[lj];
-                    const char* Kh = reinterpret_cast<const char*>(ly.K) + static_cast<size_t>(hkv) * p.L * row_bytes;
-                    const char* Vh = reinterpret_cast<const char*>(ly.V) + static_cast<size_t>(hkv) * p.L * row_bytes;
-                    char* oK = reinterpret_cast<char*>(ly.out_K) + static_cast<size_t>(hkv) * p.n_max * row_bytes;
-                    char* oV = reinterpret_cast<char*>(ly.out_V) + static_cast<size_t>(hkv) * p.n_max * row_bytes;
-                    int loaded = 0;
-                    auto issue_load = [&](int idx) {
-                        int sr, dr, rows;
-                        unit(u_begin + idx, sr, dr, rows);
-                        const uint32_t slot = (g_issued + idx) % n_slots;
-                        const uint32_t bar = smem_u32(&ctl.gfull[slot]);
-                        const uint32_t dst = stage0 + slot * p.stage_slot_bytes;
-                        if (!p.strided) {
-                            const uint32_t bytes = static_cast<uint32_t>(rows) * row_bytes;
-                            mbar_arrive_expect_tx(bar, 2u * bytes);
-                            bulk_load(dst, Kh + static_cast<size_t>(sr) * row_bytes, bytes, bar);
-                            bulk_load(dst + half_slot, Vh + static_cast<size_t>(sr) * row_bytes, bytes, bar);
-                        } else {
-                            // (a box is always whole: rows past the chunk's or window's end are not stored, past L they are zeros)
-                            mbar_arrive_expect_tx(bar, 2u * static_cast<uint32_t>(p.copy_box_bytes));
-                            tma_load_3d(dst, &p.tm_rk[lj], bar, 0, sr, hkv);
-                            tma_load_3d(dst + half_slot, &p.tm_rv[lj], bar, 0, sr, hkv);
-                        }
-                    };
-                    // loads run n_slots - 1 units ahead of the stores
-                    for (; loaded < n_units && loaded < static_cast<int>(n_slots) - 1; ++loaded) issue_load(loaded);
-                    for (int idx = 0; idx < n_units && ok; ++idx) {
-                        const uint32_t gi = g_issued + idx;
-                        const uint32_t slot = gi % n_slots;
-                        ok = mbar_wait(smem_u32(&ctl.gfull[slot]), (gi / n_slots) & 1u, abort_flag);
-                        if (!ok) break;
-                        int sr, dr, rows;
-                        unit(u_begin + idx, sr, dr, rows);
+                auto issue_load = [&](int lj, int idx, int set) {
+                    int sr, dr, rows;
+                    unit(u_begin + idx, sr, dr, rows);
+                    const uint32_t slot = static_cast<uint32_t>(set * lanes + lane);
+                    const uint32_t bar = smem_u32(&ctl.gfull[slot]);
+                    const uint32_t dst = stage0 + slot * p.stage_slot_bytes;
+                    if (!p.strided) {
+                        const ModelLayer& ly = p.layer[lj];
+                        const size_t from = (static_cast<size_t>(hkv) * p.L + sr) * row_bytes;
                         const uint32_t bytes = static_cast<uint32_t>(rows) * row_bytes;
-                        {
-                            bulk_store(oK + static_cast<size_t>(dr) * row_bytes, stage0 + slot * p.stage_slot_bytes, bytes);
-                            bulk_store(oV + static_cast<size_t>(dr) * row_bytes, stage0 + slot * p.stage_slot_bytes + half_slot, bytes);
-                            bulk_commit();
-                        }
-                        if (loaded < n_units) {
-                            // the slot the next load takes was stored one unit ago: all but the newest group have been read
-                            bulk_wait_read<1>();
-                            issue_load(loaded);
-                            ++loaded;
-                        }
+                        mbar_arrive_expect_tx(bar, 2u * bytes);
+                        bulk_load(dst, reinterpret_cast<const char*>(ly.K) + from, bytes, bar);
+                        bulk_load(dst + half_slot, reinterpret_cast<const char*>(ly.V) + from, bytes, bar);
+                    } else {
+                        // (a box is always whole: rows past the chunk's or window's end are not stored, past L they are zeros)
+                        mbar_arrive_expect_tx(bar, 2u * static_cast<uint32_t>(p.copy_box_bytes));
+                        tma_load_3d(dst, &p.tm_rk[lj], bar, 0, sr, hkv);
+                        tma_load_3d(dst + half_slot, &p.tm_rv[lj], bar, 0, sr, hkv);
                     }
-                    bulk_wait_read<0>();          // the slots are reused by the next layer's first loads
-                    g_issued += static_cast<uint32_t>(n_units);
-                    ++lj;
-                } while (ok && lj < p.n_layers && !p.layer[lj].computes);
-                li = lj;
+                };
+                // this lane's next unit to load, and to store: (layer, unit of the CTA's share), `lanes` units apart
+                int lj_l = li, ix_l = lane, lj_s = li, ix_s = lane, set = 0;
+                auto next = [&](int& lj, int& ix) {
+                    ix += lanes;
+                    while (ix >= n_units) { ix -= n_units; ++lj; }
+                };
+                while (ix_l >= n_units) { ix_l -= n_units; ++lj_l; }
+                lj_s = lj_l;
+                ix_s = ix_l;
+                for (int i = 0; i < n_sets && lj_l < lj_end; ++i) {
+                    issue_load(lj_l, ix_l, i);
+                    next(lj_l, ix_l);
+                }
+                while (lj_s < lj_end) {
+                    const uint32_t slot = static_cast<uint32_t>(set * lanes + lane);
+                    ok = mbar_wait(smem_u32(&ctl.gfull[slot]), phase >> set & 1u, abort_flag);
+                    if (!ok) break;
+                    phase ^= 1u << set;
+                    int sr, dr, rows;
+                    unit(u_begin + ix_s, sr, dr, rows);
+                    const ModelLayer& ly = p.layer[lj_s];
+                    const uint32_t bytes = static_cast<uint32_t>(rows) * row_bytes, from = stage0 + slot * p.stage_slot_bytes;
+                    const size_t to = (static_cast<size_t>(hkv) * p.n_max + dr) * row_bytes;
+                    bulk_store(reinterpret_cast<char*>(ly.out_K) + to, from, bytes);
+                    bulk_store(reinterpret_cast<char*>(ly.out_V) + to, from + half_slot, bytes);
+                    bulk_commit();
+                    if (lj_l < lj_end) {
+                        bulk_wait_read<0>();                 // the slot is loaded again
+                        issue_load(lj_l, ix_l, set);
+                        next(lj_l, ix_l);
+                    }
+                    next(lj_s, ix_s);
+                    if (++set == n_sets) set = 0;
+                }
+                bulk_wait_read<0>();                         // the slots are reused by the next list's first loads
             }
-            bulk_wait_all();
-            if (!ok) ctl.abort_flag = 1;
+            __syncwarp();                                    // (and the list itself)
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+            li = lj_end;
         }
+        bulk_wait_all();
+        if (!ok) ctl.abort_flag = 1;
     }
 
     tc_fence_before();
