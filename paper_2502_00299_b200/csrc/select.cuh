@@ -44,7 +44,6 @@ struct SelectSmem {
     int last_kept;
     alignas(16) int found[4];               // sub-interval of the k-th largest key, its rank in it, keys in it
     unsigned long long last;                // last candidate that is kept
-    int kept_cand[kSelMaxWarps];            // kept candidates of a warp's ids
 };
 
 __device__ __forceinline__ uint32_t select_order_key(float x) {
@@ -67,14 +66,14 @@ __device__ __forceinline__ uint32_t select_order_key(float x) {
 //
 // What bounds it is a chain of latencies - seven or eight block-wide steps on a few thousand keys - and, inside the steps,
 // the instructions that all warps issue. select_regs: a thread owns a run of KPT consecutive ids, so that a warp without
-// ids leaves out the work on keys, loads are 8 or 16 bytes wide, and the order inside a warp is one packed prefix sum over its
-// lanes. Candidates are ranked by (key, id) at once, so that ties need no counting of their own and the prefix sum over the keys
-// above them runs in the same step as their collection. select_core: registers with runs padded to four ids, or shared memory
+// ids leaves out the work on keys, loads are 8 or 16 bytes wide, and the order inside a warp is one prefix sum over its
+// lanes. Candidates are ranked by (key, id) at once, so that ties need no counting of their own. select_core: registers with runs padded to four ids, or shared memory
 // (warp v owns a block of consecutive ids and walks it in rows of 32, one id per lane, with ballots for the order); the ties are
 // counted in a step more. In clocks, 576 threads, scores from the L2, a cold instruction cache, select_core -> select_regs: 204 keys
 // 5.7k -> 4.0k, 816 5.5k -> 4.5k, 1636 6.0k -> 4.6k, 3274 6.6k -> 6.3k, 6550 15.0k -> 9.0k (runs padded to 16 ids were loaded one by
-// one), 13104 20.2k (in shared memory) -> 14.8k. The layer kernel with it: 2048 tokens, 2 heads 13.0 -> 12.4 us; 65536 tokens,
-// 2 heads 26.5 -> 23.0; 131072 tokens, 8 heads, 128 rows 88 -> 82.
+// one), 13104 20.2k (in shared memory) -> 14.8k. Then the last kept candidate was found first, so that one comparison a key and one
+// prefix sum give the kept ids (two of each before), and four lanes rank a candidate: from the candidates' bin to the list 2.3k -> 1.8k
+// clocks (204 and 819 keys); a layer of 2048 tokens, 2 heads 12.28 -> 11.84 us, of 8192 16.7 -> 16.3, of 32768 29.5 -> 29.2.
 constexpr int kSelBins = 2048;
 constexpr int kSelCandCap = 128;
 
@@ -129,7 +128,6 @@ __device__ __forceinline__ void select_regs(const float* sc, const float* sc2, i
             }
         }
         for (int i = tid; i < kSelBins / 4; i += nt) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
-        for (int i = tid; i < kSelMaxWarps; i += nt) sm.kept_cand[i] = 0;
         for (int i = tid; i < kSelCandCap; i += nt) cand[i] = 0ull;
         if (warp_on) {
 #pragma unroll
@@ -196,81 +194,86 @@ __device__ __forceinline__ void select_regs(const float* sc, const float* sc2, i
         span = min((1u << shift) - 1u, span - sub);
         if (n_bin <= kSelCandCap || span == 0u) break;
     }
-    // The keys above the interval are kept, and `need` of those in it, the candidates. Few candidates: they are ranked by key and
-    // id. Many equal ones: the first `need` of them in the order of ids.
-    const bool ranked = n_bin <= kSelCandCap;
-    const uint32_t top = base + span;
-    unsigned above = 0, hits = 0;   // this thread's keys above the interval, and in it (bit u: id0 + u)
-    unsigned before = 0;            // (#candidates << 16 | #above) in the warp before this thread
-    if (warp_on) {
+    // The keys above the interval are kept, and `need` of those in it, the candidates. Few candidates: they are ranked against
+    // each other by key and id, which gives the last one kept. Many equal ones: the first `need` of them in the order of ids.
+    unsigned kept = 0;              // this thread's kept keys (bit u: id0 + u)
+    int rank = 0;                   // kept keys before them
+    if (n_bin <= kSelCandCap) {
+        if (warp_on) {
+            unsigned hits = 0;
 #pragma unroll
-        for (int u = 0; u < KPT; ++u) {
-            above |= keys[u] > top ? 1u << u : 0u;           // (ids past the last one have key 0)
-            hits |= u < own && keys[u] - base <= span ? 1u << u : 0u;
-        }
-        const unsigned mine = __popc(above) | __popc(hits) << 16;
-        unsigned inc = mine;
+            for (int u = 0; u < KPT; ++u) hits |= u < own && keys[u] - base <= span ? 1u << u : 0u;
+            if (hits != 0) {                                     // (the order of the candidates does not matter)
+                int at = atomicAdd(&sm.n_cand, __popc(hits));
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const unsigned n = __shfl_up_sync(kFull, inc, off);
-            if (lane >= off) inc += n;
-        }
-        if (lane == 31) sm.warp_tot[warp] = static_cast<int>(inc);
-        before = inc - mine;
-        if (ranked && __any_sync(kFull, hits != 0)) {        // (one atomic a warp; the order of the candidates does not matter)
-            int at = 0;
-            if (lane == 31) at = atomicAdd(&sm.n_cand, static_cast<int>(inc >> 16));
-            at = __shfl_sync(kFull, at, 31) + static_cast<int>(before >> 16);
-#pragma unroll
-            for (int u = 0; u < KPT; ++u)
-                if (hits >> u & 1u) cand[at++] = static_cast<unsigned long long>(keys[u]) << 32 | static_cast<uint32_t>(~(id0 + u));
-        }
-    } else if (lane == 31) {
-        sm.warp_tot[warp] = 0;
-    }
-    __syncthreads();
-    if (ranked) {
-        if (tid < n_bin) {
-            const unsigned long long v = cand[tid];          // larger key first, then lower id: all different
-            int gt = 0;
-            const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(cand);
-#pragma unroll 8
-            for (int i = 0; i < (n_bin + 1) / 2; ++i) { const ulonglong2 x = c2[i]; gt += x.x > v; gt += x.y > v; }
-            if (gt < need) {
-                const int id = static_cast<int>(~static_cast<uint32_t>(v));
-                atomicAdd(&sm.kept_cand[id / (32 * KPT)], 1);
-                if (gt == need - 1) sm.last = v;
+                for (int u = 0; u < KPT; ++u)
+                    if (hits >> u & 1u) cand[at++] = static_cast<unsigned long long>(keys[u]) << 32 | static_cast<uint32_t>(~(id0 + u));
             }
         }
         __syncthreads();
-    }
-    if (warp_on) {
-        const unsigned tot = lane < warp ? static_cast<unsigned>(sm.warp_tot[lane]) : 0u;
-        unsigned kept = above;
-        int rank;
-        if (ranked) {
-            const unsigned ex = __reduce_add_sync(kFull, (tot & 0xffffu) + (lane < warp ? static_cast<unsigned>(sm.kept_cand[lane]) : 0u));
-            rank = static_cast<int>(ex + (before & 0xffffu));
-            if (__any_sync(kFull, hits != 0)) {
-                const unsigned long long last = sm.last;
-                unsigned kh = 0;
-                if (hits != 0) {
+        if (warp * 8 < n_bin) {                                  // four lanes a candidate
+            const int ci = tid >> 2;
+            const unsigned long long v = ci < n_bin ? cand[ci] : 0ull;   // larger key first, then lower id: all different
+            int gt = 0;
+            const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(cand);
+#pragma unroll 4
+            for (int i = tid & 3; i < (n_bin + 1) / 2; i += 4) { const ulonglong2 x = c2[i]; gt += x.x > v; gt += x.y > v; }
+            gt += __shfl_xor_sync(kFull, gt, 1);
+            gt += __shfl_xor_sync(kFull, gt, 2);
+            if ((tid & 3) == 0 && ci < n_bin && gt == need - 1) sm.last = v;
+        }
+        __syncthreads();
+        if (warp_on) {
+            const unsigned long long last = sm.last;
+            const uint32_t last_key = static_cast<uint32_t>(last >> 32);
+            const int last_id = static_cast<int>(~static_cast<uint32_t>(last));
 #pragma unroll
-                    for (int u = 0; u < KPT; ++u)
-                        if (hits >> u & 1u) kh |= (static_cast<unsigned long long>(keys[u]) << 32 | static_cast<uint32_t>(~(id0 + u))) >= last ? 1u << u : 0u;
+            for (int u = 0; u < KPT; ++u)                        // (ids past the last one have key 0 and come behind every candidate)
+                kept |= keys[u] > last_key || (keys[u] == last_key && id0 + u <= last_id) ? 1u << u : 0u;
+            int total;
+            if constexpr (KPT <= 4) {
+                total = 0;
+#pragma unroll
+                for (int u = 0; u < KPT; ++u) {
+                    const unsigned m = __ballot_sync(kFull, kept >> u & 1u);
+                    rank += __popc(m & ((1u << lane) - 1u));
+                    total += __popc(m);
                 }
-                const int mh = __popc(kh);
-                int ih = mh;
+            } else {
+                total = __popc(kept);
 #pragma unroll
                 for (int off = 1; off < 32; off <<= 1) {
-                    const int n = __shfl_up_sync(kFull, ih, off);
-                    if (lane >= off) ih += n;
+                    const int n = __shfl_up_sync(kFull, total, off);
+                    if (lane >= off) total += n;
                 }
-                rank += ih - mh;
-                kept |= kh;
+                rank = total - __popc(kept);
             }
-        } else {
-            const unsigned ex = __reduce_add_sync(kFull, tot) + before;
+            if (lane == 31) sm.warp_tot[warp] = total;
+        }
+        __syncthreads();
+        if (warp_on) rank += __reduce_add_sync(kFull, lane < warp ? sm.warp_tot[lane] : 0);
+    } else {
+        const uint32_t top = base + span;
+        unsigned hits = 0;              // keys in the interval
+        unsigned inc = 0, mine = 0;     // (#candidates << 16 | #above)
+        if (warp_on) {
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) {
+                kept |= keys[u] > top ? 1u << u : 0u;
+                hits |= u < own && keys[u] - base <= span ? 1u << u : 0u;
+            }
+            mine = __popc(kept) | __popc(hits) << 16;
+            inc = mine;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const unsigned n = __shfl_up_sync(kFull, inc, off);
+                if (lane >= off) inc += n;
+            }
+            if (lane == 31) sm.warp_tot[warp] = static_cast<int>(inc);
+        }
+        __syncthreads();
+        if (warp_on) {
+            const unsigned ex = __reduce_add_sync(kFull, lane < warp ? static_cast<unsigned>(sm.warp_tot[lane]) : 0u) + inc - mine;
             const int eq_before = static_cast<int>(ex >> 16);
             rank = static_cast<int>(ex & 0xffffu) + min(eq_before, need);
             int room = max(0, need - eq_before);
@@ -278,6 +281,8 @@ __device__ __forceinline__ void select_regs(const float* sc, const float* sc2, i
             for (int u = 0; u < KPT; ++u)
                 if (hits >> u & 1u) { kept |= room > 0 ? 1u << u : 0u; --room; }
         }
+    }
+    if (warp_on) {
 #pragma unroll
         for (int u = 0; u < KPT; ++u)
             if (kept >> u & 1u) sm.sel[rank + __popc(kept & ((1u << u) - 1u))] = static_cast<unsigned short>(id0 + u);
