@@ -41,15 +41,13 @@ struct PagedDst {
 
 // Work item `item` of `n_items` (a CTA-sized slab of rows of one head); threads = nthreads
 // (a multiple of VPR). VPR = 16-byte vectors per row: 8 (d = 64) or 16 (d = 128).
-// FRESH_IDX: the indices were written earlier in the same kernel launch, so they must not be
-// read through the non-coherent path. k_row_vecs / v_row_vecs: 16-byte vectors between consecutive
+// index_at(n): the source row of compacted position n (-1: none). k_row_vecs / v_row_vecs: 16-byte vectors between consecutive
 // source rows of a head (VPR for packed rows; more for a token-major cache).
-template <int VPR, bool FRESH_IDX>
-__device__ __forceinline__ void gather_rows(const uint4* __restrict__ Kh, const uint4* __restrict__ Vh,
-                                            const int32_t* ih, int L, int n_max, int n0, int tid, int nthreads,
-                                            uint4* __restrict__ oK, uint4* __restrict__ oV, int32_t* idx_copy,
-                                            long long k_row_vecs = VPR, long long v_row_vecs = VPR,
-                                            PagedDst pg = PagedDst{nullptr, 0, 0, 0, 0}) {
+template <int VPR, class IndexAt>
+__device__ __forceinline__ void gather_rows_at(const uint4* __restrict__ Kh, const uint4* __restrict__ Vh,
+                                               IndexAt index_at, int L, int n_max, int n0, int tid, int nthreads,
+                                               uint4* __restrict__ oK, uint4* __restrict__ oV, int32_t* idx_copy,
+                                               long long k_row_vecs, long long v_row_vecs, PagedDst pg) {
     const int rows_per_pass = nthreads / VPR;
     const int vec = tid % VPR, sub = tid / VPR;
     const unsigned long long policy = gather_policy();
@@ -58,8 +56,7 @@ __device__ __forceinline__ void gather_rows(const uint4* __restrict__ Kh, const 
 #pragma unroll
     for (int u = 0; u < kGatherRowsPerThread; ++u) {
         const int n = n0 + u * rows_per_pass + sub;
-        if (n < n_max) src[u] = FRESH_IDX ? __ldcg(ih + n) : ih[n];
-        else src[u] = -1;
+        src[u] = n < n_max ? index_at(n) : -1;
     }
 #pragma unroll
     for (int u = 0; u < kGatherRowsPerThread; ++u) {
@@ -85,6 +82,17 @@ __device__ __forceinline__ void gather_rows(const uint4* __restrict__ Kh, const 
             if (idx_copy != nullptr && vec == 0) idx_copy[n] = src[u];
         }
     }
+}
+
+// The same with the indices in memory. FRESH_IDX: they were written earlier in the same kernel launch, so they must not be
+// read through the non-coherent path.
+template <int VPR, bool FRESH_IDX>
+__device__ __forceinline__ void gather_rows(const uint4* __restrict__ Kh, const uint4* __restrict__ Vh,
+                                            const int32_t* ih, int L, int n_max, int n0, int tid, int nthreads,
+                                            uint4* __restrict__ oK, uint4* __restrict__ oV, int32_t* idx_copy,
+                                            long long k_row_vecs = VPR, long long v_row_vecs = VPR) {
+    gather_rows_at<VPR>(Kh, Vh, [&](int n) { return FRESH_IDX ? __ldcg(ih + n) : ih[n]; }, L, n_max, n0, tid, nthreads, oK, oV, idx_copy,
+                        k_row_vecs, v_row_vecs, PagedDst{nullptr, 0, 0, 0, 0});
 }
 
 }  // namespace chunkkv

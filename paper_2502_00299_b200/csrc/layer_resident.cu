@@ -31,11 +31,11 @@
 //
 //   1. score      TMA -> tcgen05.mma (128 rows x 120 or 128 keys per accumulator tile) -> epilogue
 //                 warps: one exponential per score element, chunk sums to tensor memory
-//   2. hand-over  the CTAs of a scoring head publish their per-row (max, sum) and wait for one
-//                 another on a per-head counter (bounded wait)
+//   2. hand-over  the CTAs of a scoring head publish their per-row (max, sum) and take one another's: words that carry
+//                 the launch's tag beside the value, or (lanes) a per-head counter (bounded waits)
 //   3. contract   every CTA merges the head's records into m_i and 1 / l_i and contracts its own
 //                 partial sums over the rows: chunk scores of its key range -> global memory
-//   4. hand-over  per KV head, until all of its chunk scores are there (bounded wait)
+//   4. hand-over  per KV head, until all of its chunk scores are there (tagged words or a counter, bounded wait)
 //   5. select     every CTA of the KV head runs the same exact top-k over the head's chunk scores
 //                 and so holds the kept chunks in shared memory without a third wait
 //   6. gather     the head's output positions are split evenly over its CTAs: each expands its
@@ -68,15 +68,31 @@ struct ResCtl {
     unsigned long long tfull[2];
     unsigned long long tempty[2];
     unsigned long long qfull;
+    int rec_count[2][4];               // epilogue warps that have left their part of the CTA's record: [query tile][32 rows]
     uint32_t tmem_base;
+    uint32_t tag;                      // this launch's tag (0: not known yet)
     int abort_flag;
     int wait_ok;
 };
 
+// Hand-overs of the launches that have the GPU to themselves carry their data (tagged words), which leaves out the release, the
+// counter and the read behind it: two round trips of the L2 for each of the two (2048 tokens, 2 heads 11.84 -> 11.06 us, 8192 16.3 -> 15.4,
+// 32768 29.2 -> 28.7, 9 CTAs a head 15.6 -> 14.6, 74 22.26 -> 21.31). The tag is the launch's number, so nothing
+// has to be cleared. Launches that share the GPU with others of their kind (lanes) keep the counters and their own scratch.
+constexpr int kXScores = 65536;        // chunk scores of all scoring heads that fit (more: the second hand-over by counters)
+struct Exchange {
+    uint32_t last_tag;                 // of the launches that have ended; advanced by a launch's last CTA
+    alignas(128) ulonglong2 record[kResidentMaxHeads * 2 * 128];   // [CTA, query tile][row]: maximum, sum
+    ulonglong2 score[kXScores / 2];    // [scoring head][score_row / 2]
+};
+__device__ Exchange g_exchange;
+enum { kDirectRecords = 1, kDirectScores = 2 };
+
 struct ResArgs {
     int L, P, w, R, d;                 // R rows per KV head
-    int n_mt;                          // 128-row query tiles per KV head (1 or 2)
-    int shift;                         // 1: the rows of a KV head are scored as two heads of q_rows and the rest
+    short n_mt;                        // 128-row query tiles per KV head (1 or 2)
+    short shift;                       // 1: the rows of a KV head are scored as two heads of q_rows and the rest
+    int direct;                        // hand-overs that go through g_exchange
     int q_rows;                        // rows of a box of the query tensor map: 128, fewer, or the half's
     float sl2;                         // log2(e) / sqrt(d)
     int cph;                           // CTAs per scoring head (a KV head, or one of its halves)
@@ -109,6 +125,120 @@ struct ResArgs {
 // then this; 30 us a pass) against the 488 bytes of an older form, padded and timed in turn: 464 bytes +0.35 us, 472 and 480
 // -0.1 to -0.3, 488 +0.2, 496 to 520 +0.3 to +0.45, 544 -0.2. What follows from other members is computed in the kernel.
 static_assert(2 * sizeof(CUtensorMap) + sizeof(ResArgs) == 480, "kernel parameters");
+
+// Up to KF records of a row (one every `step`, from `src`) in one round trip, as often as it takes until all of them carry this
+// launch's tag; merged into (M, S). False: given up.
+template <int KF>
+__device__ __forceinline__ bool take_records(const ulonglong2* src, size_t step, int n, uint32_t tag, float& M, float& S, volatile int* abort_flag) {
+    ulonglong2 r[KF];
+    unsigned missing = (1u << n) - 1u;
+    long long t0 = 0;
+    for (uint32_t it = 1;; ++it) {
+#pragma unroll
+        for (int u = 0; u < KF; ++u)
+            if (missing >> u & 1u) r[u] = ld_tagged2(src + u * step);
+#pragma unroll
+        for (int u = 0; u < KF; ++u)
+            if ((missing >> u & 1u) && tagged_is(r[u].x, tag) && tagged_is(r[u].y, tag)) missing &= ~(1u << u);
+        if (missing == 0u) break;
+        if ((it & 63u) == 0u) {
+            if (t0 == 0) t0 = clock64();
+            if (*abort_flag) return false;
+            if (clock64() - t0 > kWaitLimitClocks) { *abort_flag = 1; return false; }
+        }
+    }
+    float bm = M;
+#pragma unroll
+    for (int u = 0; u < KF; ++u)
+        if (u < n) bm = fmaxf(bm, tagged_value(r[u].x));
+    float acc = S * exp2_int(M - bm);
+#pragma unroll
+    for (int u = 0; u < KF; ++u)
+        if (u < n) acc += tagged_value(r[u].y) * exp2_int(tagged_value(r[u].x) - bm);
+    M = bm;
+    S = acc;
+    return true;
+}
+
+// The head's chunk scores from the exchange into shared memory as order keys, two a word pair, as they arrive (src2: added); this thread's
+// smallest and largest key. False: given up.
+__device__ __forceinline__ bool take_scores(const ulonglong2* src, const ulonglong2* src2, int C, uint32_t tag, uint32_t* kbuf, uint32_t& lo,
+                                            uint32_t& hi, volatile int* abort_flag) {
+    constexpr int KP = 3;                // pairs in flight: one round trip up to 3456 chunks
+    const int pairs = (C + 1) >> 1;
+    for (int p0 = threadIdx.x; p0 < pairs; p0 += KP * kRThreads) {
+        ulonglong2 a[KP], b[KP];
+        unsigned missing = 0;
+#pragma unroll
+        for (int u = 0; u < KP; ++u) missing |= p0 + u * kRThreads < pairs ? 1u << u : 0u;
+        const unsigned all = missing;
+        long long t0 = 0;
+        for (uint32_t it = 1;; ++it) {
+#pragma unroll
+            for (int u = 0; u < KP; ++u)
+                if (missing >> u & 1u) {
+                    a[u] = ld_tagged2(src + p0 + u * kRThreads);
+                    if (src2 != nullptr) b[u] = ld_tagged2(src2 + p0 + u * kRThreads);
+                }
+#pragma unroll
+            for (int u = 0; u < KP; ++u)
+                if (missing >> u & 1u) {
+                    const bool one = 2 * (p0 + u * kRThreads) + 1 == C;        // (no second chunk)
+                    if (tagged_is(a[u].x, tag) && (one || tagged_is(a[u].y, tag)) &&
+                        (src2 == nullptr || (tagged_is(b[u].x, tag) && (one || tagged_is(b[u].y, tag)))))
+                        missing &= ~(1u << u);
+                }
+            if (missing == 0u) break;
+            if ((it & 63u) == 0u) {
+                if (t0 == 0) t0 = clock64();
+                if (*abort_flag) return false;
+                if (clock64() - t0 > kWaitLimitClocks) { *abort_flag = 1; return false; }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < KP; ++u)
+            if (all >> u & 1u) {
+                const int ch = 2 * (p0 + u * kRThreads);
+                float x = tagged_value(a[u].x), y = tagged_value(a[u].y);
+                if (src2 != nullptr) { x += tagged_value(b[u].x); y += tagged_value(b[u].y); }
+                const uint32_t kx = select_order_key(x), ky = select_order_key(y);
+                *reinterpret_cast<uint2*>(kbuf + ch) = make_uint2(kx, ky);
+                lo = min(lo, kx);
+                hi = max(hi, kx);
+                if (ch + 1 < C) { lo = min(lo, ky); hi = max(hi, ky); }
+            }
+    }
+    return true;
+}
+// The same from global memory, behind a hand-over by counters (rows padded to a multiple of four chunks).
+__device__ __forceinline__ void load_scores(const float* sc, const float* sc2, int C, uint32_t* kbuf, uint32_t& lo, uint32_t& hi) {
+    constexpr int KP = 4;
+    const int pairs = (C + 1) >> 1;
+    for (int p0 = threadIdx.x; p0 < pairs; p0 += KP * kRThreads) {
+        float2 v[KP];
+#pragma unroll
+        for (int u = 0; u < KP; ++u) v[u] = __ldcg(reinterpret_cast<const float2*>(sc) + min(p0 + u * kRThreads, pairs - 1));
+        if (sc2 != nullptr) {
+#pragma unroll
+            for (int u = 0; u < KP; ++u) {
+                const float2 x = __ldcg(reinterpret_cast<const float2*>(sc2) + min(p0 + u * kRThreads, pairs - 1));
+                v[u].x += x.x;
+                v[u].y += x.y;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < KP; ++u) {
+            const int ch = 2 * (p0 + u * kRThreads);
+            if (ch < C) {
+                const uint32_t kx = select_order_key(v[u].x), ky = select_order_key(v[u].y);
+                *reinterpret_cast<uint2*>(kbuf + ch) = make_uint2(kx, ky);
+                lo = min(lo, kx);
+                hi = max(hi, kx);
+                if (ch + 1 < C) { lo = min(lo, ky); hi = max(hi, ky); }
+            }
+        }
+    }
+}
 
 // One thread publishes this CTA's arrival on `counter` and waits until `target` CTAs have arrived.
 // Block-wide: every thread calls it; returns false if the wait was abandoned.
@@ -190,6 +320,8 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             mbar_init(smem_u32(&ctl.tempty[b]), 8);      // one arrival per warp of the pair that reads the buffer
         }
         mbar_init(smem_u32(&ctl.qfull), 1);
+        for (int i = 0; i < 8; ++i) (&ctl.rec_count[0][0])[i] = 0;
+        ctl.tag = 0u;
         ctl.abort_flag = 0;
         ctl.wait_ok = 1;
         prefetch_tmap(&tm_q);            // (kernel parameters: not written by the kernel ahead of this one)
@@ -256,7 +388,10 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     } else if (warp == 1) {
         // ------------------------------------------------------------------ UMMA issuer
         if (elect_one() && nt > 0) {
+            uint32_t last_tag;               // (the launch before has ended: griddepcontrol.wait)
+            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(last_tag) : "l"(&g_exchange.last_tag) : "memory");
             bool ok = mbar_wait(smem_u32(&ctl.qfull), 0, abort_flag);
+            *const_cast<volatile uint32_t*>(&ctl.tag) = last_tag + 1u;
             const uint64_t q_desc = umma_desc_sw128(q_base), k_desc = umma_desc_sw128(k_base);
             const bool both = KB == 2;                   // d is 64 or 128: one or two stages a tile
             uint32_t st = 0, st_par = 0;
@@ -295,11 +430,13 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
         const uint64_t keep = l2_policy_evict_last();
         float run_m = -CUDART_INF_F, run_l = 0.f;
+        bool scored = true;
         for (int vt = pair; vt < n_vt; vt += 2) {
             const int use = vt >> 1, ti = two ? use : vt;
             bool ready = true;                           // one lane polls, the warp follows
             if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[pair]), use & 1, abort_flag);
-            if (!__shfl_sync(0xffffffffu, ready, 0)) break;
+            scored = __shfl_sync(0xffffffffu, ready, 0);
+            if (!scored) break;
             tc_fence_after();
             float v[WP];
             load_panel<WP>(lane_addr + static_cast<uint32_t>(pair * kRUmmaN + half * WP), v);
@@ -334,6 +471,44 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         tmem_st_wait();
         rec[(grp * 2 + 0) * 128 + row] = active ? run_m : -CUDART_INF_F;
         rec[(grp * 2 + 1) * 128 + row] = active ? run_l : 0.f;
+
+        // ---- 2. (hand-over that carries its data) The last of the warps that hold the same 32 rows merges their parts and stores them; then
+        // every thread takes its share of the records of one row of the head: a slice a group, the slices are put together below.
+        // Up to 64 rows and more CTAs a head than four slices of records read in one round trip (2 heads: 74): eight slices of 64 rows.
+        if (a.direct != 0 && scored) {
+            __threadfence_block();
+            __syncwarp();
+            const int mt = two ? pair : 0, n_g = two ? 2 : 4;
+            uint32_t tag = 0u;
+            while (!*abort_flag && (tag = *const_cast<volatile uint32_t*>(&ctl.tag)) == 0u) {}
+            int old = 0;
+            if (lane == 0) old = atomicAdd(&ctl.rec_count[mt][quarter], 1);
+            if (__shfl_sync(0xffffffffu, old, 0) == n_g - 1) {
+                __threadfence_block();
+                float M = -CUDART_INF_F, S = 0.f;
+#pragma unroll
+                for (int g = 0; g < 4; ++g)
+                    if (g < n_g) merge_ml(M, S, rec[((mt * 2 + g) * 2) * 128 + row], rec[((mt * 2 + g) * 2 + 1) * 128 + row]);
+                if (tag != 0u) st_tagged2(&g_exchange.record[(static_cast<size_t>(blockIdx.x) * n_mt + mt) * 128 + row], M, S, tag);
+            }
+            constexpr int KF = BIG ? 9 : 5;              // records in flight per thread: one round trip where a head has 18 CTAs (8 heads)
+            const int n_sl = FEW ? 8 : (two ? 2 : 4), sl = FEW ? grp * 2 + (quarter >> 1) : (two ? half : grp);
+            const int prow = FEW ? (quarter & 1) * 32 + lane : row;
+            float M = -CUDART_INF_F, S = 0.f;
+            if (tag != 0u && (FEW ? prow < n_rows : active)) {
+                const size_t step = static_cast<size_t>(n_mt) * 128;
+                const ulonglong2* src = g_exchange.record + (static_cast<size_t>(hs) * a.cph * n_mt + mt) * 128 + prow;
+                for (int j0 = sl; j0 < a.cph; j0 += KF * n_sl)
+                    if (!take_records<KF>(src + j0 * step, n_sl * step, min(KF, (a.cph - j0 + n_sl - 1) / n_sl), tag, M, S, abort_flag)) break;
+            }
+            if constexpr (FEW) {
+                slice[sl * 64 + prow] = M;
+                slice[512 + sl * 64 + prow] = S;
+            } else {
+                slice[(grp * 2 + 0) * 128 + row] = M;
+                slice[(grp * 2 + 1) * 128 + row] = S;
+            }
+        }
     }
 
     tc_fence_before();
@@ -341,8 +516,8 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     tc_fence_after();
     bool ok = ctl.abort_flag == 0;
 
-    // ---- 2. this CTA's (max, sum) per row -> global memory; wait for the head's other CTAs
-    if (ok) {
+    // ---- 2. (by counters) this CTA's (max, sum) per row -> global memory; wait for the head's other CTAs
+    if (ok && a.direct == 0) {
         if (static_cast<int>(threadIdx.x) < n_mt * 128) {
             const int i = threadIdx.x & 127;
             const int g0 = two ? (threadIdx.x >> 7) * 2 : 0, g1 = two ? g0 + 2 : 4;   // groups that scored this query tile
@@ -365,8 +540,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 
     // ---- 3. row statistics of the head, then this CTA's chunk scores
     if (ok) {
-        // Up to 64 rows and more CTAs a head than four slices of records read in one round trip (2 heads: 74): eight slices
-        // of 64 rows, two round trips to the L2 instead of four (8192 tokens 14.3 -> 13.5 us, 65536 tokens 23.3 -> 22.3).
+        if (a.direct == 0) {
         if constexpr (FEW) {
             float M = -CUDART_INF_F, Ls = 0.f;
             if (threadIdx.x < 512) {
@@ -442,6 +616,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             }
         }
         __syncthreads();
+        }
         // chunk scores of this CTA's key range: partial sums x exp2(m_panel - m_i) / l_i, summed over
         // the rows. A thread holds one row of up to 32 chunk slots at a time (PPB panels of its
         // group: panels grp, grp + 4, ...); a transposing warp reduction leaves lane j with the sum
@@ -456,7 +631,23 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             const bool active = mt * 128 + row < n_rows;
             const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
             const int srow = active ? row : 0;           // (rows that do not exist have no record)
-            const float mi = gm[mt * 128 + row], li = ginv[mt * 128 + row];
+            float mi, li;                                // the row's maximum and 1 / sum in the head (rows >= R: never used)
+            if (a.direct == 0) {
+                mi = gm[mt * 128 + row];
+                li = ginv[mt * 128 + row];
+            } else {
+                float M = -CUDART_INF_F, S = 0.f;
+                if constexpr (FEW) {
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) merge_ml(M, S, slice[u * 64 + (row & 63)], slice[512 + u * 64 + (row & 63)]);
+                } else {
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+                        if (!two || (g >> 1) == mt) merge_ml(M, S, slice[(g * 2) * 128 + row], slice[(g * 2 + 1) * 128 + row]);
+                }
+                mi = M;
+                li = 1.0f / S;
+            }
             const uint64_t drop = l2_policy_evict_first();   // the sums in scratch are dead once read
             constexpr int PPB = 32 / SPP;                // panels per block of up to 32 values
             for (int b0 = 0; grp + 4 * b0 < n_pl; b0 += PPB) {
@@ -516,55 +707,82 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 const float* r = red + lc;
                 float t = (r[0] + r[n_local]) + (r[2 * n_local] + r[3 * n_local]);
                 if (two) t += (r[4 * n_local] + r[5 * n_local]) + (r[6 * n_local] + r[7 * n_local]);
-                a.scores[static_cast<size_t>(hs) * a.score_row + ch0 + lc] = t;
+                const size_t at = static_cast<size_t>(hs) * a.score_row + ch0 + lc;
+                if (a.direct & kDirectScores) st_tagged(reinterpret_cast<unsigned long long*>(g_exchange.score) + at, t, ctl.tag);
+                else a.scores[at] = t;
             }
     }
     // ---- 4. wait for the KV head's other CTAs, 5. select, 6. gather
-    if (ok && a.out_idx != nullptr) ok = head_handover(a.cnt_b(hkv), static_cast<unsigned>(a.cph << (BIG ? 0 : a.shift)), ctl);
+    if (ok && a.out_idx != nullptr) {
+        if (a.direct & kDirectScores) __syncthreads();       // (the sums above are read; the ring is written again)
+        else ok = head_handover(a.cnt_b(hkv), static_cast<unsigned>(a.cph << (BIG ? 0 : a.shift)), ctl);
+    }
     if (ok && a.out_idx != nullptr) {
         SelectSmem& ss = *reinterpret_cast<SelectSmem*>(ring);
         constexpr size_t kSelBytes = (sizeof(SelectSmem) + 127) & ~size_t(127);
         const int shift = BIG ? 0 : a.shift;
-        const float* sc = a.scores + (static_cast<size_t>(hkv) << shift) * a.score_row;
+        const size_t row_at = (static_cast<size_t>(hkv) << shift) * a.score_row;
+        const float* sc = a.scores + row_at;
         const float* sc2 = shift ? sc + a.score_row : nullptr;           // the other half's chunk scores are added
         const int Q = a.cph << shift, q = (hs & shift) * a.cph + part;   // CTAs of this KV head
         const int r_begin = static_cast<int>(static_cast<long long>(a.n_max) * q / Q);
         const int r_end = static_cast<int>(static_cast<long long>(a.n_max) * (q + 1) / Q);
-        int32_t* sidx = reinterpret_cast<int32_t*>(ring + kSelBytes);          // kept positions [r_begin, r_end) of the head
         int32_t* out_idx = a.out_idx + static_cast<size_t>(hkv) * a.n_max;
-        const size_t idx_bytes = (static_cast<size_t>(r_end - r_begin) * 4 + 127) & ~size_t(127);
-        uint32_t* kbuf = reinterpret_cast<uint32_t*>(ring + kSelBytes + idx_bytes);
-        const bool fits = kSelBytes + idx_bytes + static_cast<size_t>(C) * 4 <= static_cast<size_t>(a.ring_bytes);
-        constexpr SelectIn kIn = WIDE ? kSelLayerWide : kSelLayer;
-        if (min(a.k, C) <= kSelCap && C <= kSelMaxChunks && ((WIDE && fits) || C <= kRThreads * select_reg_keys(kIn))) {
-            select_kept<kIn>(sc, sc2, C, a.k, ss, kbuf);
-            // every CTA holds the head's kept chunks: it expands, writes and gathers its own share of the positions
-            const int n_tok = select_tokens(a.P, C_STATIC, C, a.k, ss, a.tok_cap);
-            for (int n = r_begin + threadIdx.x; n < r_end; n += kRThreads) {
-                const int pos = select_position(ss, n, n_tok, C_STATIC, a.P, a.w);
-                sidx[n - r_begin] = pos;
-                out_idx[n] = pos;
-            }
+        uint32_t* kbuf = reinterpret_cast<uint32_t*>(ring + kSelBytes);
+        const bool fits = kSelBytes + (static_cast<size_t>(C) + 4) * 4 <= static_cast<size_t>(a.ring_bytes);
+        // every CTA holds the head's kept chunks: it expands, writes and gathers its own share of the positions
+        bool listed = min(a.k, C) <= kSelCap && C <= kSelMaxChunks && fits;
+        if constexpr (WIDE) {
+            if (listed) select_kept<kSelLayerWide>(sc, sc2, C, a.k, ss, kbuf);
         } else {
-            // very many chunks: every CTA of the head writes the same positions to out_idx and takes its share from there
-            select_head_rows(sc, sc2, a.L, a.w, C_STATIC, C, a.k, a.n_max, out_idx, ss, fits ? kbuf : nullptr, a.tok_cap);
-            for (int n = r_begin + threadIdx.x; n < r_end; n += kRThreads) sidx[n - r_begin] = out_idx[n];
+            listed = listed && C <= kRThreads * select_reg_keys(kSelLayer);
+            if (listed && !select_all(C, a.k, ss)) {
+                uint32_t lo = 0xffffffffu, hi = 0u;
+                select_clear(ss);
+                if (a.direct & kDirectScores) {
+                    const ulonglong2* x = g_exchange.score + row_at / 2;
+                    take_scores(x, shift ? x + a.score_row / 2 : nullptr, C, ctl.tag, kbuf, lo, hi, abort_flag);
+                } else {
+                    load_scores(sc, sc2, C, kbuf, lo, hi);
+                }
+                lo = __reduce_min_sync(0xffffffffu, lo);
+                hi = __reduce_max_sync(0xffffffffu, hi);
+                if (lane == 0) ss.warp_sums[warp] = (static_cast<unsigned long long>(hi) << 32) | lo;
+                __syncthreads();
+                ok = ctl.abort_flag == 0;
+                if (ok) {
+                    const int per = (C + kRThreads - 1) / kRThreads;
+                    if (per <= 2) select_staged<2>(kbuf, C, a.k, ss);
+                    else if (per <= 4) select_staged<4>(kbuf, C, a.k, ss);
+                    else if (per <= 8) select_staged<8>(kbuf, C, a.k, ss);
+                    else select_staged<16>(kbuf, C, a.k, ss);
+                }
+            }
         }
-        __syncthreads();
-        const int vpr = a.d >> 3;
-        const int rows_per_pass = (kRThreads / vpr) * kGatherRowsPerThread;
-        // packed outputs: this head's block; paged outputs: the cache base (rows are placed through the block table)
-        const PagedDst pg{a.block_table, a.page_size, a.num_pages, a.Hkv, hkv};
-        const size_t head_out = a.block_table ? 0 : static_cast<size_t>(hkv) * a.n_max;
-        for (int n0 = r_begin; n0 < r_end; n0 += rows_per_pass) {
-            if (vpr == 16)
-                gather_rows<16, false>(a.K + static_cast<size_t>(hkv) * a.k_head, a.V + static_cast<size_t>(hkv) * a.v_head,
-                                       sidx - r_begin, a.L, r_end, n0, threadIdx.x, kRThreads, a.out_K + head_out * 16,
-                                       a.out_V + head_out * 16, nullptr, a.k_row, a.v_row, pg);
-            else
-                gather_rows<8, false>(a.K + static_cast<size_t>(hkv) * a.k_head, a.V + static_cast<size_t>(hkv) * a.v_head,
-                                      sidx - r_begin, a.L, r_end, n0, threadIdx.x, kRThreads, a.out_K + head_out * 8,
-                                      a.out_V + head_out * 8, nullptr, a.k_row, a.v_row, pg);
+        // very many chunks: every CTA of the head writes the same positions to out_idx and takes its share from there
+        if (!listed) {
+            select_head_rows(sc, sc2, a.L, a.w, C_STATIC, C, a.k, a.n_max, out_idx, ss, fits ? kbuf : nullptr, a.tok_cap);
+            __syncthreads();
+        }
+        if (ok) {
+            const int n_tok = listed ? select_tokens(a.P, C_STATIC, C, a.k, ss, a.tok_cap) : 0;
+            auto index_at = [&](int n) { return listed ? select_position(ss, n, n_tok, C_STATIC, a.P, a.w) : __ldcg(out_idx + n); };
+            int32_t* idx_out = listed ? out_idx : nullptr;
+            const int vpr = a.d >> 3;
+            const int rows_per_pass = (kRThreads / vpr) * kGatherRowsPerThread;
+            // packed outputs: this head's block; paged outputs: the cache base (rows are placed through the block table)
+            const PagedDst pg{a.block_table, a.page_size, a.num_pages, a.Hkv, hkv};
+            const size_t head_out = a.block_table ? 0 : static_cast<size_t>(hkv) * a.n_max;
+            const uint4* Kh = a.K + static_cast<size_t>(hkv) * a.k_head;
+            const uint4* Vh = a.V + static_cast<size_t>(hkv) * a.v_head;
+            for (int n0 = r_begin; n0 < r_end; n0 += rows_per_pass) {
+                if (vpr == 16)
+                    gather_rows_at<16>(Kh, Vh, index_at, a.L, r_end, n0, threadIdx.x, kRThreads, a.out_K + head_out * 16, a.out_V + head_out * 16,
+                                       idx_out, a.k_row, a.v_row, pg);
+                else
+                    gather_rows_at<8>(Kh, Vh, index_at, a.L, r_end, n0, threadIdx.x, kRThreads, a.out_K + head_out * 8, a.out_V + head_out * 8,
+                                      idx_out, a.k_row, a.v_row, pg);
+            }
         }
     }
     // tensor memory has not been read since the barrier after the contraction (or after scoring)
@@ -580,6 +798,17 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         if (old + 1u == gridDim.x) {
             for (int h = 0; h < a.Hkv << a.shift; ++h) { *a.cnt_a(h) = 0u; *a.cnt_b(h) = 0u; }
             *a.exits() = 0u;
+            if (a.direct != 0) {
+                // the next launch's tag; before it starts over at 1, words of old launches that were never written again are cleared
+                uint32_t t = *const_cast<volatile uint32_t*>(&ctl.tag);
+                if (t == 0u) t = *const_cast<volatile uint32_t*>(&g_exchange.last_tag) + 1u;      // (this CTA gave up before it knew)
+                if (t == 0xffffffffu) {
+                    for (ulonglong2& x : g_exchange.record) x = make_ulonglong2(0ull, 0ull);
+                    for (ulonglong2& x : g_exchange.score) x = make_ulonglong2(0ull, 0ull);
+                    t = 0u;
+                }
+                g_exchange.last_tag = t;
+            }
             __threadfence();
         }
     }
@@ -661,11 +890,14 @@ bool make_resident_plan(int L, int R, int Hkv, int d, int c, int C, int n_max, i
 
 cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                                   const ResidentIO& io, cudaStream_t stream) {
+    const bool wide = io.out_idx != nullptr && io.C > kRThreads * select_reg_keys(kSelLayer);
     ResArgs a{};
-    a.L = io.L; a.P = io.L - io.w; a.w = io.w; a.R = io.R; a.d = io.d; a.n_mt = plan.n_mt;
+    a.L = io.L; a.P = io.L - io.w; a.w = io.w; a.R = io.R; a.d = io.d; a.n_mt = static_cast<short>(plan.n_mt);
     a.sl2 = io.sl2;
     a.cph = plan.cph; a.n_stages = plan.n_stages;
-    a.shift = plan.shift; a.q_rows = resident_q_box_rows(plan, io.R);
+    a.direct = io.cooperative ? 0
+             : kDirectRecords | (io.out_idx != nullptr && !wide && static_cast<long long>(io.Hkv << plan.shift) * ((io.C + 3) & ~3) <= kXScores ? kDirectScores : 0);
+    a.shift = static_cast<short>(plan.shift); a.q_rows = resident_q_box_rows(plan, io.R);
     a.k = io.k; a.n_max = io.n_max; a.Hkv = io.Hkv;
     a.n_on = plan.n_on; a.n_off = plan.n_off; a.spill_rows = plan.spill_rows;
     a.off_ring = plan.off_ring; a.ring_bytes = plan.ring_bytes; a.off_pmax = plan.off_pmax; a.off_misc = plan.off_misc;
@@ -687,7 +919,6 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     a.spill = scores + (((static_cast<size_t>(io.Hkv) << plan.shift) * ((io.C + 3) & ~3) + 63) & ~static_cast<size_t>(63));
     a.counters = io.counters;
     const int variant = plan.n_mt == 2 || plan.n_off > 0 ? 1 : (io.R <= 64 && plan.cph > kRManyCtas ? 2 : 0);
-    const bool wide = io.out_idx != nullptr && io.C > kRThreads * select_reg_keys(kSelLayer);
     const void* kern = nullptr;
     int v = 0;
     switch (plan.c_static) {

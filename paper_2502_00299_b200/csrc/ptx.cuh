@@ -168,6 +168,25 @@ __device__ __forceinline__ void spill_load(const float* p, int rows, int row, fl
         asm volatile("ld.global.cg.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v[o]) : "l"(p + o * n + row), "l"(policy));
 }
 
+// Values handed to other SMs with a tag in the same 64-bit word: who reads the tag has the value, so that one round trip through
+// the L2 replaces a release, a counter and a read. The upper half is the tag, the lower the value; two words a vector.
+__device__ __forceinline__ unsigned long long tagged(float v, uint32_t tag) {
+    return static_cast<unsigned long long>(tag) << 32 | __float_as_uint(v);
+}
+__device__ __forceinline__ void st_tagged(unsigned long long* p, float v, uint32_t tag) {
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(tagged(v, tag)) : "memory");
+}
+__device__ __forceinline__ void st_tagged2(ulonglong2* p, float v0, float v1, uint32_t tag) {
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(tagged(v0, tag)), "l"(tagged(v1, tag)) : "memory");
+}
+__device__ __forceinline__ ulonglong2 ld_tagged2(const ulonglong2* p) {
+    ulonglong2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float tagged_value(unsigned long long w) { return __uint_as_float(static_cast<uint32_t>(w)); }
+__device__ __forceinline__ bool tagged_is(unsigned long long w, uint32_t tag) { return static_cast<uint32_t>(w >> 32) == tag; }
+
 // ----------------------------------------------------------------------------- tcgen05
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst),

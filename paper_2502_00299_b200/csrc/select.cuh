@@ -77,71 +77,34 @@ __device__ __forceinline__ uint32_t select_order_key(float x) {
 constexpr int kSelBins = 2048;
 constexpr int kSelCandCap = 128;
 
-// Keys in registers: thread t owns the ids [t KPT, (t + 1) KPT), C <= blockDim.x KPT.
+// Scratch of a selection of k of C > k keys (every thread; before the barrier ahead of select_keys).
+__device__ __forceinline__ void select_clear(SelectSmem& sm) {
+    const int nt = blockDim.x, tid = threadIdx.x;
+    if (tid == 0) { sm.last_kept = 0; sm.n_cand = 0; }
+    for (int i = tid; i < kSelBins / 4; i += nt) reinterpret_cast<int4*>(&sm.whist[0][0])[i] = make_int4(0, 0, 0, 0);
+    for (int i = tid; i < kSelCandCap; i += nt) reinterpret_cast<unsigned long long*>(&sm.sel[0])[i] = 0ull;
+}
+// k >= C or nothing to keep: no keys are needed. Every thread; true if that was it.
+__device__ __forceinline__ bool select_all(int C, int k, SelectSmem& sm) {
+    const int kk = min(k, C);
+    if (k < C && kk > 0) return false;
+    if (threadIdx.x == 0) sm.last_kept = kk > 0;
+    for (int ch = threadIdx.x; ch < kk; ch += blockDim.x) sm.sel[ch] = static_cast<unsigned short>(ch);
+    __syncthreads();
+    return true;
+}
+
+// Keys in registers: thread t owns the ids [t KPT, (t + 1) KPT), C <= blockDim.x KPT; keys of ids past the last one are 0.
+// Behind a barrier after select_clear and after every warp has left its smallest and largest key in sm.warp_sums.
 template <int KPT>
-__device__ __forceinline__ void select_regs(const float* sc, const float* sc2, int C, int k, SelectSmem& sm) {
+__device__ __forceinline__ void select_keys(const uint32_t (&keys)[KPT], int C, int k, SelectSmem& sm) {
     constexpr unsigned kFull = 0xffffffffu;
     static_assert(KPT <= 32, "a run's flags fit a word");
     const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = nt >> 5;
-    const int kk = min(k, C);
-    if (tid == 0) { sm.last_kept = k >= C && kk > 0; sm.n_cand = 0; }
-    if (k >= C || kk <= 0) {
-        for (int ch = tid; ch < kk; ch += nt) sm.sel[ch] = static_cast<unsigned short>(ch);
-        __syncthreads();
-        return;
-    }
     int* hist = reinterpret_cast<int*>(&sm.whist[0][0]);                            // kSelBins counters
     unsigned long long* cand = reinterpret_cast<unsigned long long*>(&sm.sel[0]);   // kSelCandCap keys with ids (sel is written later)
     const int id0 = tid * KPT, own = min(KPT, C - id0);      // this thread's ids; own <= 0: none
     const bool warp_on = warp * (32 * KPT) < C;              // this thread's warp has ids
-    uint32_t keys[KPT];
-    uint32_t lo = 0xffffffffu, hi = 0u;
-    {
-        float v[KPT];
-        constexpr int W = KPT % 4 == 0 ? 4 : 2;              // floats a load
-        auto load = [&](const float* p, float* o) {
-            if constexpr (W == 4) {
-                const float4 f = __ldcg(reinterpret_cast<const float4*>(p));
-                o[0] = f.x; o[1] = f.y; o[2] = f.z; o[3] = f.w;
-            } else {
-                const float2 f = __ldcg(reinterpret_cast<const float2*>(p));
-                o[0] = f.x; o[1] = f.y;
-            }
-        };
-        const bool vec = ((reinterpret_cast<uintptr_t>(sc) | reinterpret_cast<uintptr_t>(sc2)) & (4u * W - 1u)) == 0;
-        if (own == KPT && vec) {
-#pragma unroll
-            for (int u = 0; u < KPT; u += W) load(sc + id0 + u, &v[u]);
-            if (sc2 != nullptr) {
-                float v2[KPT];
-#pragma unroll
-                for (int u = 0; u < KPT; u += W) load(sc2 + id0 + u, &v2[u]);
-#pragma unroll
-                for (int u = 0; u < KPT; ++u) v[u] += v2[u];
-            }
-        } else if (own > 0) {
-#pragma unroll
-            for (int u = 0; u < KPT; ++u) v[u] = u < own ? __ldcg(sc + id0 + u) : 0.f;
-            if (sc2 != nullptr) {
-#pragma unroll
-                for (int u = 0; u < KPT; ++u) v[u] += u < own ? __ldcg(sc2 + id0 + u) : 0.f;
-            }
-        }
-        for (int i = tid; i < kSelBins / 4; i += nt) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
-        for (int i = tid; i < kSelCandCap; i += nt) cand[i] = 0ull;
-        if (warp_on) {
-#pragma unroll
-            for (int u = 0; u < KPT; ++u) {
-                const bool in = u < own;
-                keys[u] = in ? select_order_key(v[u]) : 0u;
-                if (in) { lo = min(lo, keys[u]); hi = max(hi, keys[u]); }
-            }
-            lo = __reduce_min_sync(kFull, lo);
-            hi = __reduce_max_sync(kFull, hi);
-        }
-    }
-    if (lane == 0) sm.warp_sums[warp] = (static_cast<unsigned long long>(hi) << 32) | lo;
-    __syncthreads();
     const unsigned long long mm = sm.warp_sums[lane < nwarps ? lane : 0];
     uint32_t base = __reduce_min_sync(kFull, static_cast<uint32_t>(mm));
     uint32_t span = __reduce_max_sync(kFull, static_cast<uint32_t>(mm >> 32)) - base;
@@ -289,6 +252,87 @@ __device__ __forceinline__ void select_regs(const float* sc, const float* sc2, i
         if (own > 0 && id0 + own == C && (kept >> (own - 1) & 1u)) sm.last_kept = 1;
     }
     __syncthreads();
+}
+
+// The same, keys from global memory.
+template <int KPT>
+__device__ __forceinline__ void select_regs(const float* sc, const float* sc2, int C, int k, SelectSmem& sm) {
+    constexpr unsigned kFull = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (select_all(C, k, sm)) return;
+    const int id0 = tid * KPT, own = min(KPT, C - id0);
+    uint32_t keys[KPT];
+    uint32_t lo = 0xffffffffu, hi = 0u;
+    {
+        float v[KPT];
+        constexpr int W = KPT % 4 == 0 ? 4 : 2;              // floats a load
+        auto load = [&](const float* p, float* o) {
+            if constexpr (W == 4) {
+                const float4 f = __ldcg(reinterpret_cast<const float4*>(p));
+                o[0] = f.x; o[1] = f.y; o[2] = f.z; o[3] = f.w;
+            } else {
+                const float2 f = __ldcg(reinterpret_cast<const float2*>(p));
+                o[0] = f.x; o[1] = f.y;
+            }
+        };
+        const bool vec = ((reinterpret_cast<uintptr_t>(sc) | reinterpret_cast<uintptr_t>(sc2)) & (4u * W - 1u)) == 0;
+        if (own == KPT && vec) {
+#pragma unroll
+            for (int u = 0; u < KPT; u += W) load(sc + id0 + u, &v[u]);
+            if (sc2 != nullptr) {
+                float v2[KPT];
+#pragma unroll
+                for (int u = 0; u < KPT; u += W) load(sc2 + id0 + u, &v2[u]);
+#pragma unroll
+                for (int u = 0; u < KPT; ++u) v[u] += v2[u];
+            }
+        } else if (own > 0) {
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) v[u] = u < own ? __ldcg(sc + id0 + u) : 0.f;
+            if (sc2 != nullptr) {
+#pragma unroll
+                for (int u = 0; u < KPT; ++u) v[u] += u < own ? __ldcg(sc2 + id0 + u) : 0.f;
+            }
+        }
+        select_clear(sm);
+        if (warp * (32 * KPT) < C) {
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) {
+                const bool in = u < own;
+                keys[u] = in ? select_order_key(v[u]) : 0u;
+                if (in) { lo = min(lo, keys[u]); hi = max(hi, keys[u]); }
+            }
+            lo = __reduce_min_sync(kFull, lo);
+            hi = __reduce_max_sync(kFull, hi);
+        }
+    }
+    if (lane == 0) sm.warp_sums[warp] = (static_cast<unsigned long long>(hi) << 32) | lo;
+    __syncthreads();
+    select_keys<KPT>(keys, C, k, sm);
+}
+
+// The same, keys in shared memory (16-byte aligned, room for a multiple of four behind the last one).
+template <int KPT>
+__device__ __forceinline__ void select_staged(const uint32_t* kbuf, int C, int k, SelectSmem& sm) {
+    const int id0 = threadIdx.x * KPT;
+    uint32_t keys[KPT];
+    if (static_cast<int>(threadIdx.x >> 5) * (32 * KPT) < C) {
+        constexpr int W = KPT % 4 == 0 ? 4 : 2;
+#pragma unroll
+        for (int u = 0; u < KPT; u += W) {
+            if constexpr (W == 4) {
+                const uint4 x = id0 + u < C ? *reinterpret_cast<const uint4*>(kbuf + id0 + u) : make_uint4(0u, 0u, 0u, 0u);
+                keys[u] = x.x; keys[u + 1] = x.y; keys[u + 2] = x.z; keys[u + 3] = x.w;
+            } else {
+                const uint2 x = id0 + u < C ? *reinterpret_cast<const uint2*>(kbuf + id0 + u) : make_uint2(0u, 0u);
+                keys[u] = x.x; keys[u + 1] = x.y;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < KPT; ++u)
+            if (id0 + u >= C) keys[u] = 0u;
+    }
+    select_keys<KPT>(keys, C, k, sm);
 }
 
 // KPT > 0: up to KPT keys a thread in registers, in runs padded to four ids (C <= blockDim.x KPT; kbuf is not used). KPT = 0: the keys
