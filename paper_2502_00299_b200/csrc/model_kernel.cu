@@ -246,9 +246,7 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
         for (int hkv = sid; hkv < p.Hkv; hkv += p.n_sel) {
             if (threadIdx.x == 0) {
                 const unsigned target = static_cast<unsigned>(s + 1) * p.cph;
-                const bool w_ok = wait_counter(p.cnt_b + hkv, target, flag + 1, 100);
-                asm volatile("fence.acq_rel.gpu;" ::: "memory");
-                flag[0] = w_ok ? 1 : 0;
+                flag[0] = wait_counter(p.cnt_b + hkv, target, flag + 1, 100) ? 1 : 0;      // (acquires; the barrier passes it on)
             }
             __syncthreads();
             if (!flag[0]) return false;
@@ -260,10 +258,14 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
                 select_head_rows(sc, sc2, p.L, p.w, C_STATIC, p.C, p.k, p.n_max, p.layer[li].out_idx + static_cast<size_t>(hkv) * p.n_max,
                                  ss, nullptr);
             const int n_tok = select_tokens(p.P, C_STATIC, p.C, p.k, ss);
-            // the kept-chunk list for the copy threads: [n_tok, -, -, -, chunk ids]
+            // the kept-chunk list for the copy warps: [n_tok, -, -, -, chunk ids]. It is announced before the positions are written, which nothing
+            // in this launch reads, and by another warp than the one that waits for the next head: a release waits for the stores before it.
             int* row = p.sel_rows + (static_cast<size_t>(s) * p.Hkv + hkv) * row_ints;
             if (threadIdx.x == 0) row[0] = n_tok;
             for (int r = threadIdx.x; r < kk; r += kMThreads) row[4 + r] = ss.sel[r];
+            __syncthreads();
+            if (threadIdx.x == kMThreads - 32)      // release: the list is visible to whoever sees the count
+                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.cnt_c + hkv) : "memory");
             const int vpr = p.d >> 3;
             for (int n = threadIdx.x; n < p.n_max; n += kMThreads) {
                 const int pos = select_position(ss, n, n_tok, C_STATIC, p.P, p.w);
@@ -276,11 +278,6 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
                     uint4* zv = p.layer[lj].out_V + (static_cast<size_t>(hkv) * p.n_max + n_tok + p.w) * vpr;
                     for (int i = threadIdx.x; i < nz; i += kMThreads) { zk[i] = make_uint4(0, 0, 0, 0); zv[i] = make_uint4(0, 0, 0, 0); }
                 }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                unsigned old;   // release: the list and the positions written above are visible to whoever sees the count
-                asm volatile("atom.add.release.gpu.u32 %0, [%1], 1;" : "=r"(old) : "l"(p.cnt_c + hkv) : "memory");
-            }
         }
         li = lj_end;
     }
