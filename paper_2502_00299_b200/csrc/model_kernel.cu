@@ -949,9 +949,12 @@ model_kernel(const __grid_constant__ ModelParams p) {
 
 }  // namespace
 
-// Tiles up to which five to eight heads have a selector CTA each (see make_model_plan).
-static int selector_each_tiles(int Hkv, int max_ctas) {
-    return Hkv > 4 && Hkv <= 8 && max_ctas >= 2 * Hkv ? 6 * ((max_ctas - Hkv) / Hkv) : 0;
+// Selector CTAs: four take the SMs that eight scoring heads leave idle anyway; more of them, one a head up to 16, where that costs the
+// scoring nothing (below); 0: no such choice.
+constexpr int kMSelFew = 4, kMSelMany = 16;
+static int many_selectors(int Hkv, int max_ctas) {
+    const int n = Hkv < kMSelMany ? Hkv : kMSelMany;
+    return Hkv > kMSelFew && max_ctas - n >= Hkv ? n : 0;
 }
 
 bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int reuse, int max_ctas, int smem_limit, ModelPlan* plan, int n_sel) {
@@ -968,23 +971,26 @@ bool make_model_plan(int L, int R, int Hkv, int d, int c, int C, int k, int reus
     p.tile = 2 * panel_keys(c);
     p.spp = panel_keys(c) / c;
     p.n_tiles = (L + p.tile - 1) / p.tile;
-    // a few CTAs do nothing but select (four take the SMs the scoring grid would leave idle anyway)
-    p.n_sel = Hkv < 4 ? Hkv : 4;
-    // Five to eight heads on short contexts: a selector each. With two heads a selector the two selections (about 5k clocks each)
-    // are longer than the scoring of a layer up to six tiles a CTA. Speed with a selector each over four (10 % kept; 64, 128 and 256 rows):
-    //   5 heads  1.04 to 1.19   6 heads  1.00 to 1.19   7 heads  1.04 to 1.17   8 heads  0.99 to 1.26
-    // Six and eight heads give up a scoring CTA a head for it, which then copies rows no longer either. Where much is copied for each
-    // selection that costs more: 8 heads, 4 tiles a CTA, indices shared by three layers, chunks of 8 0.91 to 0.95, of 16 0.93; a quarter
-    // kept, chunks of 5 0.96 to 0.98. So they have to stay below 22 kept chunks to copy a CTA and selection, 15 where indices are shared, and,
-    // beyond two tiles, 27 % of the rows; within that 0.985 to 1.26. Five and seven heads need no such line (0.996 and more with a quarter kept and indices shared
-    // by three).
-    // (Two sets of layers in turn, inputs of 3 x 200 MB and more, graph replays. More heads keep four selectors; where the line
-    // lies for them has not been worked out.)
-    if (p.n_tiles <= selector_each_tiles(Hkv, max_ctas)) {
-        const int cph = (max_ctas - Hkv) / Hkv;
-        const long long copied = static_cast<long long>(reuse) * kk;
-        const bool light = copied <= (reuse > 1 ? 15ll : 22ll) * cph && (p.n_tiles <= 2 * cph || copied * c * 100 <= 27ll * L);
-        if (light || cph == (max_ctas - 4) / Hkv) p.n_sel = Hkv;
+    // What a layer takes with n selectors, ns: scoring (a chain of latencies and some 1.1 us a product of a tile), the selections of one
+    // selector's heads, the copies of one CTA's units, whichever is longest; fitted to calls of 2048 to 42450 tokens. As many selectors as there are
+    // if that is at most 4 % more: their lists come sooner, which shortens the end of the launch. us with four -> with one a head (16
+    // at most), 10 % kept: 8 heads, 128 rows 4096 tokens x12 102.5 -> 93.5, 16000 x12 138 -> 130, 20000 x8 116 -> 108; 256 rows 16000 x12 237 -> 232;
+    // 12 heads 2048 x9 99 -> 68, 16000 x6 118.5 -> 107; 16 heads 2048 140 -> 84 (x9, 4096), 32 heads 240 -> 89, 8192 297 -> 180. Where a CTA gets another
+    // tile or the copies are the longest, four are better: 8 heads, 256 rows 8192 tokens x12 144 -> 154, 32768 x8 280 -> 294; 128 rows, chunks of 5,
+    // a fifth kept, indices shared by two, 12000 x12 141 -> 143; 24 heads 32768 x6, a fifth kept, shared by three 298 -> 308.
+    p.n_sel = Hkv < kMSelFew ? Hkv : kMSelFew;
+    const int many = many_selectors(Hkv, max_ctas);
+    if (many > 0) {
+        auto layer_ns = [&](int n) {
+            int cph = (max_ctas - n) / Hkv;
+            if (cph > p.n_tiles) cph = p.n_tiles;
+            const long long score = 3500 + 1100ll * p.n_mt * ((p.n_tiles + cph - 1) / cph);
+            const long long select = static_cast<long long>((Hkv + n - 1) / n) * (4000 + C * 4ll / 5);
+            const long long copy = static_cast<long long>(reuse) * kk * (200 + 13 * c) / cph;
+            const long long longer = score > select ? score : select;
+            return longer > copy ? longer : copy;
+        };
+        if (max_ctas - kMSelFew < Hkv || 100 * layer_ns(many) <= 104 * layer_ns(kMSelFew)) p.n_sel = many;
     }
     if (n_sel > 0) p.n_sel = n_sel;
     if (max_ctas - p.n_sel < Hkv) p.n_sel = max_ctas - Hkv;
@@ -1061,17 +1067,15 @@ size_t model_scratch_floats(const ModelPlan& plan, int Hkv, int C, int n_compute
 }
 
 size_t model_reserve_floats(int L, int R, int Hkv, int d, int c, int C, int k, int max_ctas, int smem_limit, int n_compute) {
-    // A grid with a given number of selectors never shrinks for a longer sequence, nor does its ring_reserve; the two numbers of
-    // selectors that a shorter sequence may have are both provided for.
+    // A grid with a given number of selectors never shrinks for a longer sequence, nor does its ring_reserve; either number of
+    // selectors that a sequence may have is provided for.
     size_t need = 0;
     ModelPlan p;
-    if (make_model_plan(L, R, Hkv, d, c, C, k, 1, max_ctas, smem_limit, &p, Hkv < 4 ? Hkv : 4))
-        need = model_floats(p, Hkv, C, n_compute, p.ring_reserve);
-    const long long each = static_cast<long long>(selector_each_tiles(Hkv, max_ctas)) * 2 * panel_keys(c);
-    if (each > 0 && make_model_plan(each < L ? static_cast<int>(each) : L, R, Hkv, d, c, C, k, 1, max_ctas, smem_limit, &p, Hkv)) {
-        const size_t m = model_floats(p, Hkv, C, n_compute, p.ring_reserve);
-        need = m > need ? m : need;
-    }
+    for (const int n : {Hkv < kMSelFew ? Hkv : kMSelFew, many_selectors(Hkv, max_ctas)})
+        if (n > 0 && make_model_plan(L, R, Hkv, d, c, C, k, 1, max_ctas, smem_limit, &p, n)) {
+            const size_t m = model_floats(p, Hkv, C, n_compute, p.ring_reserve);
+            need = m > need ? m : need;
+        }
     return need;
 }
 
