@@ -243,9 +243,9 @@ int run_score(DeviceCtx& ctx, const void* q_obs, const void* K, int L, int Hq, i
     TokenPlan tplan;
     const int rows = w * (Hq / Hkv);
     if (c == 1 && make_token_plan(L, w, rows, Hkv, d, ctx.num_sms, smem_budget(ctx), &tplan)) {
-        // token scores: two passes over the keys in one launch, nothing but row records in scratch
+        // token scores: two passes over the keys in one launch, no scratch but the second half of rows
         const size_t pair_t = tplan.n_mt == 2 ? round64(static_cast<size_t>(tplan.Hs) * C) : 0;
-        const size_t tfloats = extra_payload_floats + pair_t + static_cast<size_t>(tplan.grid) * 256;
+        const size_t tfloats = extra_payload_floats + pair_t;
         int st2 = ensure_workspace(ctx, tfloats * sizeof(float));
         if (st2 != CHUNKKV_OK) return st2;
         float* payload = reinterpret_cast<float*>(static_cast<char*>(ctx.ws) + kHeaderBytes);
@@ -261,7 +261,6 @@ int run_score(DeviceCtx& ctx, const void* q_obs, const void* K, int L, int Hq, i
         io.L = L; io.w = w; io.R = rows; io.d = d;
         io.sl2 = static_cast<float>(1.4426950408889634 / sqrt(static_cast<double>(d)));
         io.token_scores = head_scores;
-        io.scratch = payload + extra_payload_floats + pair_t;
         io.counters = reinterpret_cast<unsigned*>(static_cast<char*>(ctx.ws) + kResidentCountersOffset);
         io.status = static_cast<int*>(ctx.ws);
         cudaError_t e2;

@@ -188,7 +188,6 @@ struct TokenIO {
     int L, w, R, d;       // R = w * Hq / Hkv query rows per KV head
     float sl2;
     float* token_scores;  // [Hs][P]
-    float* scratch;       // grid * 256 floats
     unsigned* counters;   // header + kResidentCountersOffset
     int* status;
 };

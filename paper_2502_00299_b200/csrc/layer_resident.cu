@@ -75,7 +75,7 @@ struct ResCtl {
     int wait_ok;
 };
 
-// Hand-overs of the launches that have the GPU to themselves carry their data (tagged words), which leaves out the release, the
+// Hand-overs of the launches that have the GPU to themselves carry their data (tagged words, resident.cuh), which leaves out the release, the
 // counter and the read behind it: two round trips of the L2 for each of the two (2048 tokens, 2 heads 11.84 -> 11.06 us, 8192 16.3 -> 15.4,
 // 32768 29.2 -> 28.7, 9 CTAs a head 15.6 -> 14.6, 74 22.26 -> 21.31). The tag is the launch's number, so nothing
 // has to be cleared. Launches that share the GPU with others of their kind (lanes) keep the counters and their own scratch.
@@ -84,6 +84,10 @@ struct Exchange {
     uint32_t last_tag;                 // of the launches that have ended; advanced by a launch's last CTA
     alignas(128) ulonglong2 record[kResidentMaxHeads * 2 * 128];   // [CTA, query tile][row]: maximum, sum
     ulonglong2 score[kXScores / 2];    // [scoring head][score_row / 2]
+    __device__ void clear() {
+        for (ulonglong2& x : record) x = make_ulonglong2(0ull, 0ull);
+        for (ulonglong2& x : score) x = make_ulonglong2(0ull, 0ull);
+    }
 };
 __device__ Exchange g_exchange;
 enum { kDirectRecords = 1, kDirectScores = 2 };
@@ -125,40 +129,6 @@ struct ResArgs {
 // then this; 30 us a pass) against the 488 bytes of an older form, padded and timed in turn: 464 bytes +0.35 us, 472 and 480
 // -0.1 to -0.3, 488 +0.2, 496 to 520 +0.3 to +0.45, 544 -0.2. What follows from other members is computed in the kernel.
 static_assert(2 * sizeof(CUtensorMap) + sizeof(ResArgs) == 480, "kernel parameters");
-
-// Up to KF records of a row (one every `step`, from `src`) in one round trip, as often as it takes until all of them carry this
-// launch's tag; merged into (M, S). False: given up.
-template <int KF>
-__device__ __forceinline__ bool take_records(const ulonglong2* src, size_t step, int n, uint32_t tag, float& M, float& S, volatile int* abort_flag) {
-    ulonglong2 r[KF];
-    unsigned missing = (1u << n) - 1u;
-    long long t0 = 0;
-    for (uint32_t it = 1;; ++it) {
-#pragma unroll
-        for (int u = 0; u < KF; ++u)
-            if (missing >> u & 1u) r[u] = ld_tagged2(src + u * step);
-#pragma unroll
-        for (int u = 0; u < KF; ++u)
-            if ((missing >> u & 1u) && tagged_is(r[u].x, tag) && tagged_is(r[u].y, tag)) missing &= ~(1u << u);
-        if (missing == 0u) break;
-        if ((it & 63u) == 0u) {
-            if (t0 == 0) t0 = clock64();
-            if (*abort_flag) return false;
-            if (clock64() - t0 > kWaitLimitClocks) { *abort_flag = 1; return false; }
-        }
-    }
-    float bm = M;
-#pragma unroll
-    for (int u = 0; u < KF; ++u)
-        if (u < n) bm = fmaxf(bm, tagged_value(r[u].x));
-    float acc = S * exp2_int(M - bm);
-#pragma unroll
-    for (int u = 0; u < KF; ++u)
-        if (u < n) acc += tagged_value(r[u].y) * exp2_int(tagged_value(r[u].x) - bm);
-    M = bm;
-    S = acc;
-    return true;
-}
 
 // The head's chunk scores from the exchange into shared memory as order keys, two a word pair, as they arrive (src2: added); this thread's
 // smallest and largest key. False: given up.
@@ -388,8 +358,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     } else if (warp == 1) {
         // ------------------------------------------------------------------ UMMA issuer
         if (elect_one() && nt > 0) {
-            uint32_t last_tag;               // (the launch before has ended: griddepcontrol.wait)
-            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(last_tag) : "l"(&g_exchange.last_tag) : "memory");
+            const uint32_t last_tag = ld_relaxed(&g_exchange.last_tag);       // (the launch before has ended: griddepcontrol.wait)
             bool ok = mbar_wait(smem_u32(&ctl.qfull), 0, abort_flag);
             *const_cast<volatile uint32_t*>(&ctl.tag) = last_tag + 1u;
             const uint64_t q_desc = umma_desc_sw128(q_base), k_desc = umma_desc_sw128(k_base);
@@ -480,7 +449,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             __syncwarp();
             const int mt = two ? pair : 0, n_g = two ? 2 : 4;
             uint32_t tag = 0u;
-            while (!*abort_flag && (tag = *const_cast<volatile uint32_t*>(&ctl.tag)) == 0u) {}
+            while (!*abort_flag && (tag = *const_cast<volatile uint32_t*>(&ctl.tag)) == 0u) {}      // (the issuer's first wait at most)
             int old = 0;
             if (lane == 0) old = atomicAdd(&ctl.rec_count[mt][quarter], 1);
             if (__shfl_sync(0xffffffffu, old, 0) == n_g - 1) {
@@ -799,15 +768,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             for (int h = 0; h < a.Hkv << a.shift; ++h) { *a.cnt_a(h) = 0u; *a.cnt_b(h) = 0u; }
             *a.exits() = 0u;
             if (a.direct != 0) {
-                // the next launch's tag; before it starts over at 1, words of old launches that were never written again are cleared
-                uint32_t t = *const_cast<volatile uint32_t*>(&ctl.tag);
-                if (t == 0u) t = *const_cast<volatile uint32_t*>(&g_exchange.last_tag) + 1u;      // (this CTA gave up before it knew)
-                if (t == 0xffffffffu) {
-                    for (ulonglong2& x : g_exchange.record) x = make_ulonglong2(0ull, 0ull);
-                    for (ulonglong2& x : g_exchange.score) x = make_ulonglong2(0ull, 0ull);
-                    t = 0u;
-                }
-                g_exchange.last_tag = t;
+                advance_tag(g_exchange, *const_cast<volatile uint32_t*>(&ctl.tag));
             }
             __threadfence();
         }

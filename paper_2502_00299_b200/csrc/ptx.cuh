@@ -184,6 +184,11 @@ __device__ __forceinline__ ulonglong2 ld_tagged2(const ulonglong2* p) {
     asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ float tagged_value(unsigned long long w) { return __uint_as_float(static_cast<uint32_t>(w)); }
 __device__ __forceinline__ bool tagged_is(unsigned long long w, uint32_t tag) { return static_cast<uint32_t>(w >> 32) == tag; }
 

@@ -91,4 +91,50 @@ __device__ __forceinline__ void merge_ml(float& M, float& S, float m, float s) {
     M = nm;
 }
 
+// Up to KF records of a row (one every `step`, from `src`) in one round trip, as often as it takes until all of them carry this
+// launch's tag; merged into (M, S). False: given up.
+template <int KF>
+__device__ __forceinline__ bool take_records(const ulonglong2* src, size_t step, int n, uint32_t tag, float& M, float& S, volatile int* abort_flag) {
+    ulonglong2 r[KF];
+    unsigned missing = (1u << n) - 1u;
+    long long t0 = 0;
+    for (uint32_t it = 1;; ++it) {
+#pragma unroll
+        for (int u = 0; u < KF; ++u)
+            if (missing >> u & 1u) r[u] = ld_tagged2(src + u * step);
+#pragma unroll
+        for (int u = 0; u < KF; ++u)
+            if ((missing >> u & 1u) && tagged_is(r[u].x, tag) && tagged_is(r[u].y, tag)) missing &= ~(1u << u);
+        if (missing == 0u) break;
+        if ((it & 63u) == 0u) {
+            if (t0 == 0) t0 = clock64();
+            if (*abort_flag) return false;
+            if (clock64() - t0 > kWaitLimitClocks) { *abort_flag = 1; return false; }
+        }
+    }
+    float bm = M;
+#pragma unroll
+    for (int u = 0; u < KF; ++u)
+        if (u < n) bm = fmaxf(bm, tagged_value(r[u].x));
+    float acc = S * exp2_int(M - bm);
+#pragma unroll
+    for (int u = 0; u < KF; ++u)
+        if (u < n) acc += tagged_value(r[u].y) * exp2_int(tagged_value(r[u].x) - bm);
+    M = bm;
+    S = acc;
+    return true;
+}
+
+// The last CTA of a launch makes its tag the last one used (tag 0: this CTA gave up before it knew it). Before the tags start over at 1,
+// words of old launches that were never written again are cleared.
+template <class X>
+__device__ __forceinline__ void advance_tag(X& x, uint32_t tag) {
+    if (tag == 0u) tag = ld_relaxed(&x.last_tag) + 1u;
+    if (tag == 0xffffffffu) {
+        x.clear();
+        tag = 0u;
+    }
+    x.last_tag = tag;
+}
+
 }  // namespace chunkkv

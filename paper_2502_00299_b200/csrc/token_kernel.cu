@@ -4,8 +4,8 @@
 //
 // With one chunk per key the per-(chunk, row) partial sums of the other kernels would be the whole
 // score matrix, so this kernel walks its keys twice instead, in one launch: pass 1 only folds the
-// per-row (max, sum) of the CTA's key range; the CTAs of a head exchange those records (one
-// bounded hand-over per head); pass 2 recomputes the same tiles (the keys come back from L2),
+// per-row (max, sum) of the CTA's key range; the CTAs of a head exchange those records (words
+// that carry the launch's tag, bounded waits); pass 2 recomputes the same tiles (the keys come back from L2),
 // normalises every element with the final row statistics and sums over the rows. Pass 1 multiplies
 // query rows x keys (a thread owns a row, so maximum and sum over keys stay in the thread); pass 2 multiplies
 // keys x query rows - the same two shared-memory operands with their roles exchanged - so that a thread owns a
@@ -42,10 +42,21 @@ struct TokCtl {
     unsigned long long tfull[kTBufs];
     unsigned long long tempty[kTBufs];
     unsigned long long qfull;
+    int rec_count[4];                  // epilogue warps that have left their part of the CTA's record (32 rows each)
     uint32_t tmem_base;
+    uint32_t tag;                      // this launch's tag (0: not known yet)
     int abort_flag;
-    int wait_ok;
 };
+
+// The hand-over of row statistics, as tagged words (resident.cuh): this kernel only runs with the GPU to itself.
+struct TokExchange {
+    uint32_t last_tag;
+    alignas(128) ulonglong2 record[kResidentMaxHeads * 128];       // [CTA][row]: maximum, sum
+    __device__ void clear() {
+        for (ulonglong2& x : record) x = make_ulonglong2(0ull, 0ull);
+    }
+};
+__device__ TokExchange g_tok_exchange;
 
 struct TokArgs {
     int L, P, w, R, Hs, d;
@@ -53,9 +64,7 @@ struct TokArgs {
     float sl2;
     int cph, n_tiles, n_tiles_prefix, n_stages, q_box_rows, k_box_rows;
     int off_ring, off_misc;
-    float* cta_stat;       // [grid][{max, sum}][128]
     float* token_scores;   // [Hs][P]
-    unsigned* cnt_a;       // [Hs]
     unsigned* exits;
     int* status;
 };
@@ -101,8 +110,9 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             mbar_init(smem_u32(&ctl.tempty[b]), 4);
         }
         mbar_init(smem_u32(&ctl.qfull), 1);
+        for (int i = 0; i < 4; ++i) ctl.rec_count[i] = 0;
+        ctl.tag = 0u;
         ctl.abort_flag = 0;
-        ctl.wait_ok = 1;
         prefetch_tmap(&tm_q);            // (kernel parameters: not written by the kernel ahead of this one)
         prefetch_tmap(&tm_k);
         fence_mbar_init();
@@ -165,8 +175,10 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ UMMA issuer
-        if (elect_one() && nt > 0) {
-            bool ok = mbar_wait(smem_u32(&ctl.qfull), 0, abort_flag);
+        if (elect_one()) {
+            const uint32_t last_tag = ld_relaxed(&g_tok_exchange.last_tag);   // (the launch before has ended: griddepcontrol.wait)
+            bool ok = nt == 0 || mbar_wait(smem_u32(&ctl.qfull), 0, abort_flag);
+            *const_cast<volatile uint32_t*>(&ctl.tag) = last_tag + 1u;
             uint32_t st = 0, st_par = 0;
             for (int tg = 0; tg < nt + nt2 && ok; ++tg) {
                 const int buf = tg % kTBufs, use = tg / kTBufs;
@@ -213,10 +225,12 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         int tg = grp;                                    // this group's next tile, counted over both passes; tile tg uses accumulator tg % 4
         // ---- pass 1: (max, sum of exp2) per row over this CTA's keys
         float run_m = -CUDART_INF_F, run_l = 0.f;
+        bool scored = true;
         for (; tg < nt; tg += kTBufs) {
             bool ready = true;
             if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[grp]), (tg / kTBufs) & 1, abort_flag);
-            if (!__shfl_sync(0xffffffffu, ready, 0)) break;
+            scored = __shfl_sync(0xffffffffu, ready, 0);
+            if (!scored) break;
             tc_fence_after();
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
@@ -239,52 +253,34 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
         rec[(grp * 2 + 0) * 128 + row] = active ? run_m : -CUDART_INF_F;
         rec[(grp * 2 + 1) * 128 + row] = active ? run_l : 0.f;
-        named_barrier(1, 512);
-        bool ok = ctl.abort_flag == 0;               // same answer in every epilogue thread
-        // ---- the head's row statistics: publish, wait for the head's other CTAs, merge
-        if (ok) {
-            if (et < 128) {
-                float M = -CUDART_INF_F, Ls = 0.f;
+        // ---- the head's row statistics: the last of the warps that hold the same 32 rows merges their parts and stores them; every
+        // thread then takes a quarter of the records of one row of the head, and the quarters are put together
+        if (scored) {
+            __threadfence_block();
+            __syncwarp();
+            uint32_t tag = 0u;
+            while (!*abort_flag && (tag = *const_cast<volatile uint32_t*>(&ctl.tag)) == 0u) {}      // (the issuer's first wait at most)
+            int old = 0;
+            if (lane == 0) old = atomicAdd(&ctl.rec_count[quarter], 1);
+            if (__shfl_sync(0xffffffffu, old, 0) == 3) {
+                __threadfence_block();
+                float M = -CUDART_INF_F, S = 0.f;
 #pragma unroll
-                for (int g = 0; g < 4; ++g) merge_ml(M, Ls, rec[(g * 2) * 128 + et], rec[(g * 2 + 1) * 128 + et]);
-                float* dst = a.cta_stat + static_cast<size_t>(blockIdx.x) * 256;
-                dst[et] = M;
-                dst[128 + et] = Ls;
+                for (int g = 0; g < 4; ++g) merge_ml(M, S, rec[(g * 2) * 128 + row], rec[(g * 2 + 1) * 128 + row]);
+                if (tag != 0u) st_tagged2(&g_tok_exchange.record[static_cast<size_t>(blockIdx.x) * 128 + row], M, S, tag);
             }
-            named_barrier(1, 512);
-            if (et == 0) {
-                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.cnt_a + hs) : "memory");
-                bool w_ok = true;
-                const long long t0 = clock64();
-                for (;;) {
-                    unsigned cur;
-                    asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(cur) : "l"(a.cnt_a + hs) : "memory");
-                    if (cur >= static_cast<unsigned>(a.cph)) break;
-                    if (clock64() - t0 > kWaitLimitClocks) { w_ok = false; ctl.abort_flag = 1; break; }
-                }
-                ctl.wait_ok = w_ok ? 1 : 0;
+            float M = -CUDART_INF_F, S = 0.f;
+            if (tag != 0u && active) {
+                const ulonglong2* src = g_tok_exchange.record + static_cast<size_t>(hs) * a.cph * 128 + row;
+                for (int j0 = grp; j0 < a.cph; j0 += 20)             // five records in flight
+                    if (!take_records<5>(src + j0 * 128, 4 * 128, min(5, (a.cph - j0 + 3) / 4), tag, M, S, abort_flag)) break;
             }
-            named_barrier(1, 512);
-            ok = ctl.wait_ok != 0;
+            slice[(grp * 2 + 0) * 128 + row] = M;
+            slice[(grp * 2 + 1) * 128 + row] = S;
         }
+        named_barrier(1, 512);
+        const bool ok = ctl.abort_flag == 0;         // same answer in every epilogue thread
         if (ok) {
-            const int i = et & 127, sl = et >> 7;
-            const float* src = a.cta_stat + static_cast<size_t>(hs) * a.cph * 256 + i;
-            float M = -CUDART_INF_F, Ls = 0.f;
-            for (int j0 = sl; j0 < a.cph; j0 += 20) {        // five records in flight per thread
-                float rm[5], rl[5];
-#pragma unroll
-                for (int u = 0; u < 5; ++u) {
-                    const int j = j0 + 4 * u;
-                    rm[u] = (j < a.cph) ? __ldcg(src + static_cast<size_t>(j) * 256) : -CUDART_INF_F;
-                    rl[u] = (j < a.cph) ? __ldcg(src + static_cast<size_t>(j) * 256 + 128) : 0.f;
-                }
-#pragma unroll
-                for (int u = 0; u < 5; ++u) merge_ml(M, Ls, rm[u], rl[u]);
-            }
-            slice[(sl * 2 + 0) * 128 + i] = M;
-            slice[(sl * 2 + 1) * 128 + i] = Ls;
-            named_barrier(1, 512);
             if (et < 128) {
                 float M2 = -CUDART_INF_F, L2 = 0.f;
 #pragma unroll
@@ -355,8 +351,8 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (ctl.abort_flag) atomicExch(a.status, 1);
         const unsigned old = atomicAdd(a.exits, 1u);
         if (old + 1u == gridDim.x) {
-            for (int h = 0; h < a.Hs; ++h) a.cnt_a[h] = 0u;
             *a.exits = 0u;
+            advance_tag(g_tok_exchange, *const_cast<volatile uint32_t*>(&ctl.tag));
             __threadfence();
         }
     }
@@ -404,10 +400,8 @@ cudaError_t launch_token_scores(const TokenPlan& plan, const CUtensorMap& tm_q, 
     a.q_box_rows = 128;                  // (rows past R arrive as zeros)
     a.k_box_rows = io.L < kTTile ? io.L : kTTile;
     a.off_ring = plan.off_ring; a.off_misc = plan.off_misc;
-    a.cta_stat = io.scratch;
     a.token_scores = io.token_scores;
     a.exits = io.counters;
-    a.cnt_a = io.counters + 16;
     a.status = io.status;
     const void* kern = plan.whole ? reinterpret_cast<const void*>(token_scores_kernel<true>) : reinterpret_cast<const void*>(token_scores_kernel<false>);
     static int smem_all[2][64] = {{0}};
