@@ -402,9 +402,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         bool scored = true;
         for (int vt = pair; vt < n_vt; vt += 2) {
             const int use = vt >> 1, ti = two ? use : vt;
-            bool ready = true;                           // one lane polls, the warp follows
-            if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[pair]), use & 1, abort_flag);
-            scored = __shfl_sync(0xffffffffu, ready, 0);
+            scored = mbar_wait_warp(smem_u32(&ctl.tfull[pair]), use & 1, abort_flag);
             if (!scored) break;
             tc_fence_after();
             float v[WP];

@@ -666,9 +666,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
                 const int aslot = BIG ? pair : pc % kMAccSlots;
                 const int use = BIG ? (vg0 + vt) >> 1 : pc / kMAccSlots;
                 const int acol = BIG ? pair * kRUmmaN + half * WP : (pc % kMAccBufs) * kMAccN + half * COL1;
-                bool ready = true;
-                if (lane == 0) ready = mbar_wait(smem_u32(&ctl.tfull[aslot]), use & 1, abort_flag);
-                if (!__shfl_sync(0xffffffffu, ready, 0)) { ok = false; continue; }
+                if (!mbar_wait_warp(smem_u32(&ctl.tfull[aslot]), use & 1, abort_flag)) { ok = false; continue; }
                 tc_fence_after();
                 float v[WP];
                 load_panel<WP>(lane_addr + static_cast<uint32_t>(acol), v);

@@ -69,6 +69,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// Bounded wait of a whole warp: every lane tests once (the phase mostly lies behind it already), then one lane polls.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    bool ready = true;
+    if ((threadIdx.x & 31) == 0) ready = mbar_wait(bar, parity, abort_flag);
+    ready = __shfl_sync(0xffffffffu, ready, 0);
+    __syncwarp();
+    return ready;
+}
+
 // Bounded waits for three phases. The first tests travel together: a test takes some 60 clocks to come back, and a thread
 // that issues products waits for phases which mostly lie behind it.
 __device__ __forceinline__ bool mbar_wait3(uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1, uint32_t bar2, uint32_t par2,
