@@ -496,7 +496,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             for (int g = 0; g < 4; ++g)
                 if (g >= g0 && g < g1) {
                     const float m = rec[(g * 2) * 128 + i];
-                    Ls += rec[(g * 2 + 1) * 128 + i] * exp2_int(m - M);
+                    Ls += rec[(g * 2 + 1) * 128 + i] * ex2_below(m, M);
                 }
             float* dst = a.cta_stat + (static_cast<size_t>(blockIdx.x) * n_mt + (threadIdx.x >> 7)) * 256;
             dst[i] = M;
@@ -556,9 +556,9 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                     float bm = M;
 #pragma unroll
                     for (int u = 0; u < kF; ++u) bm = fmaxf(bm, rm[u]);
-                    float acc = Ls * exp2_int(M - bm);
+                    float acc = Ls * ex2_below(M, bm);
 #pragma unroll
-                    for (int u = 0; u < kF; ++u) acc += rl[u] * exp2_int(rm[u] - bm);
+                    for (int u = 0; u < kF; ++u) acc += rl[u] * ex2_below(rm[u], bm);
                     M = bm;
                     Ls = acc;
                 }
@@ -576,7 +576,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 for (int s = 0; s < 4; ++s)
                     if (s >= s0 && s < s0 + n_sl) {
                         const float m = slice[(s * 2) * 128 + i];
-                        Ls += slice[(s * 2 + 1) * 128 + i] * exp2_int(m - M);
+                        Ls += slice[(s * 2 + 1) * 128 + i] * ex2_below(m, M);
                     }
                 gm[threadIdx.x] = M;
                 ginv[threadIdx.x] = 1.0f / Ls;       // rows >= R are never used
@@ -654,7 +654,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 #pragma unroll
                 for (int u = 0; u < PPB; ++u) {
                     const bool have = active && grp + 4 * (b0 + u) < n_pl;
-                    const float f = have ? exp2_int(pm[u] - mi) * li : 0.f;
+                    const float f = have ? ex2_approx(pm[u] - mi) * li : 0.f;
 #pragma unroll
                     for (int s = 0; s < SPP; ++s) v[u * SPP + s] = have ? v[u * SPP + s] * f : 0.f;
                 }

@@ -178,14 +178,14 @@ __device__ __forceinline__ void merge_batch(float (&M)[4], float (&S)[4], const 
             nm[3] = fmaxf(nm[3], m[j].w);
         }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) S[r] *= exp2_int(M[r] - nm[r]);
+    for (int r = 0; r < 4; ++r) S[r] *= ex2_below(M[r], nm[r]);
 #pragma unroll
     for (int j = 0; j < N; ++j)
         if (j < n) {
-            S[0] += l[j].x * exp2_int(m[j].x - nm[0]);
-            S[1] += l[j].y * exp2_int(m[j].y - nm[1]);
-            S[2] += l[j].z * exp2_int(m[j].z - nm[2]);
-            S[3] += l[j].w * exp2_int(m[j].w - nm[3]);
+            S[0] += l[j].x * ex2_below(m[j].x, nm[0]);
+            S[1] += l[j].y * ex2_below(m[j].y, nm[1]);
+            S[2] += l[j].z * ex2_below(m[j].z, nm[2]);
+            S[3] += l[j].w * ex2_below(m[j].w, nm[3]);
         }
 #pragma unroll
     for (int r = 0; r < 4; ++r) M[r] = nm[r];
@@ -571,9 +571,9 @@ model_kernel(const __grid_constant__ ModelParams p) {
                         float bm = M;
 #pragma unroll
                         for (int j = 0; j < kF; ++j) bm = fmaxf(bm, rm[j]);
-                        float acc = S * exp2_int(M - bm);
+                        float acc = S * ex2_below(M, bm);
 #pragma unroll
-                        for (int j = 0; j < kF; ++j) acc += rl[j] * exp2_int(rm[j] - bm);
+                        for (int j = 0; j < kF; ++j) acc += rl[j] * ex2_below(rm[j], bm);
                         M = bm;
                         S = acc;
                     }
@@ -624,7 +624,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
 #pragma unroll
                 for (int u = 0; u < PPB; ++u) {
                     const bool have = active && b0 + u < own;
-                    const float f = have ? exp2_int(pm[u] - mi) * li : 0.f;
+                    const float f = have ? ex2_approx(pm[u] - mi) * li : 0.f;
 #pragma unroll
                     for (int q = 0; q < SPP; ++q) v[u * SPP + q] = have ? v[u * SPP + q] * f : 0.f;
                 }

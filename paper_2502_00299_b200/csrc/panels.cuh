@@ -1,7 +1,6 @@
 // Epilogue panels of the scoring kernels: one thread owns one query row of a panel of WP score
 // columns (keys), pulled from tensor memory into registers. For that row it takes the panel
-// maximum (in the log2 domain, rounded to an integer: what the exponents are relative to, so that records of several panels, groups
-// and CTAs are merged with exact powers of two), exponentiates every visible element once relative to it, and sums the exponentials per
+// maximum, exponentiates every visible element once relative to it, and sums the exponentials per
 // chunk of C keys (ChunkKV Algorithm 3, "Vectorized Chunk Score Calculation", before the softmax
 // normaliser is known). What happens to a chunk's partial sum is the caller's business: `emit(ch,
 // value)` is called once per chunk slot of the panel with a compile-time-unrolled `ch`.
@@ -40,7 +39,7 @@ __device__ __forceinline__ void panel_fast(float (&v)[WP], float sl2, Emit emit,
     // (a row whose keys of the panel all have the logit -inf: a finite maximum, so that the exponents are -inf and not
     // -inf + inf; as the third operand it costs nothing, where selecting cost 1 to 2 % of the calls that exponentials bound)
     const float mx = fmax3(m0, m1, -3.402823466e38f);
-    const float ref = rintf(mx * sl2), neg_m2 = -ref;
+    const float neg_m2 = -mx * sl2;
     float l = 0.f;
     if constexpr (C % 2 == 0) {
         // Two columns per instruction: scale-and-shift and the chunk sums run on packed pairs
@@ -88,7 +87,7 @@ __device__ __forceinline__ void panel_fast(float (&v)[WP], float sl2, Emit emit,
             l += acc;
         }
     }
-    *out_m = ref;
+    *out_m = mx * sl2;
     *out_l = l;
 }
 
@@ -116,7 +115,7 @@ __device__ __forceinline__ void panel_static_tail(const float (&v)[WP], float sl
     }
     if constexpr (WP % 2 == 1) mx0 = (WP - 1 < n_vis) ? fmaxf(mx0, v[WP - 1]) : mx0;
     const float mx = fmaxf(mx0, mx1);
-    const float ref = rintf(mx * sl2), neg_m2 = (mx == -CUDART_INF_F) ? 0.f : -ref;
+    const float neg_m2 = (mx == -CUDART_INF_F) ? 0.f : -mx * sl2;
     float l0 = 0.f, l1 = 0.f, acc = 0.f;
 #pragma unroll
     for (int u = 0; u < WP; ++u) {
@@ -130,7 +129,7 @@ __device__ __forceinline__ void panel_static_tail(const float (&v)[WP], float sl
         }
     }
     const float l = l0 + l1;
-    *out_m = ref;
+    *out_m = (mx == -CUDART_INF_F) ? -CUDART_INF_F : mx * sl2;
     *out_l = l;
 }
 

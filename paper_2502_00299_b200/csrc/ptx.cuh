@@ -352,10 +352,9 @@ __device__ __forceinline__ float ex2_approx(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// 2^k for an integer k <= 0 held as a float; 0 below 2^-126 and for NaN (the difference of two infinities). Exact, and without
-// the special-function unit: 12582912 + 127 moves k + 127 into the low bits of the sum, the shift makes it an exponent.
-__device__ __forceinline__ float exp2_int(float k) {
-    return __int_as_float(__float_as_int(fmaxf(k, -127.f) + 12583039.f) << 23);
+// 2^(m - M) of two maxima, m <= M; 0 where m is -inf (nothing yet).
+__device__ __forceinline__ float ex2_below(float m, float M) {
+    return m == __int_as_float(0xff800000) ? 0.f : ex2_approx(m - M);
 }
 // Packed pairs of fp32 (sm_100 executes fma/add on two fp32 per lane per instruction).
 __device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
