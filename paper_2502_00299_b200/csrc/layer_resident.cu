@@ -81,7 +81,8 @@ struct ResCtl {
 // has to be cleared. Launches that share the GPU with others of their kind (lanes) keep the counters and their own scratch.
 constexpr int kXScores = 65536;        // chunk scores of all scoring heads that fit (more: the second hand-over by counters)
 struct Exchange {
-    uint32_t last_tag;                 // of the launches that have ended; advanced by a launch's last CTA
+    uint32_t last_tag;                 // of the launches so far
+    uint32_t started;                  // CTAs of this launch that have taken its tag
     alignas(128) ulonglong2 record[kResidentMaxHeads * 2 * 128];   // [CTA, query tile][row]: maximum, sum
     ulonglong2 score[kXScores / 2];    // [scoring head][score_row / 2]
     __device__ void clear() {
@@ -358,9 +359,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     } else if (warp == 1) {
         // ------------------------------------------------------------------ UMMA issuer
         if (elect_one() && nt > 0) {
-            const uint32_t last_tag = ld_relaxed(&g_exchange.last_tag);       // (the launch before has ended: griddepcontrol.wait)
             bool ok = mbar_wait(smem_u32(&ctl.qfull), 0, abort_flag);
-            *const_cast<volatile uint32_t*>(&ctl.tag) = last_tag + 1u;
             const uint64_t q_desc = umma_desc_sw128(q_base), k_desc = umma_desc_sw128(k_base);
             const bool both = KB == 2;                   // d is 64 or 128: one or two stages a tile
             uint32_t st = 0, st_par = 0;
@@ -398,6 +397,8 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         const int last_visible = a.P + ((row0 + qrow) % a.w);     // this row sees keys j <= P + r (all < L)
         const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
         const uint64_t keep = l2_policy_evict_last();
+        // (behind griddepcontrol.wait; beside the first keys' way here, which the issuing thread should not wait for twice)
+        if (a.direct != 0 && threadIdx.x == 64) *const_cast<volatile uint32_t*>(&ctl.tag) = take_tag(g_exchange);
         float run_m = -CUDART_INF_F, run_l = 0.f;
         bool scored = true;
         for (int vt = pair; vt < n_vt; vt += 2) {
@@ -447,7 +448,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             __syncwarp();
             const int mt = two ? pair : 0, n_g = two ? 2 : 4;
             uint32_t tag = 0u;
-            while (!*abort_flag && (tag = *const_cast<volatile uint32_t*>(&ctl.tag)) == 0u) {}      // (the issuer's first wait at most)
+            while (!*abort_flag && (tag = *const_cast<volatile uint32_t*>(&ctl.tag)) == 0u) {}      // (long there)
             int old = 0;
             if (lane == 0) old = atomicAdd(&ctl.rec_count[mt][quarter], 1);
             if (__shfl_sync(0xffffffffu, old, 0) == n_g - 1) {
@@ -759,15 +760,14 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     }
     if (threadIdx.x == 0) {
         if (!ok) atomicExch(a.status(), 1);
-        // The last CTA to leave clears the hand-over counters for the next launch. (After an
+        // The last CTA to leave clears the hand-over counters for the next launch, if there were any. (After an
         // abandoned wait the counters are left as they are; chunkkv_device_status clears them.)
-        const unsigned old = atomicAdd(a.exits(), 1u);
-        if (old + 1u == gridDim.x) {
+        const bool counted = a.direct == 0 || (a.direct == kDirectRecords && a.out_idx != nullptr);
+        const bool last_tag = a.direct != 0 && ctl.tag == kLastTag;
+        if ((counted || last_tag) && atomicAdd(a.exits(), 1u) + 1u == gridDim.x) {
             for (int h = 0; h < a.Hkv << a.shift; ++h) { *a.cnt_a(h) = 0u; *a.cnt_b(h) = 0u; }
             *a.exits() = 0u;
-            if (a.direct != 0) {
-                advance_tag(g_exchange, *const_cast<volatile uint32_t*>(&ctl.tag));
-            }
+            if (last_tag) end_tags(g_exchange);
             __threadfence();
         }
     }

@@ -50,7 +50,8 @@ struct TokCtl {
 
 // The hand-over of row statistics, as tagged words (resident.cuh): this kernel only runs with the GPU to itself.
 struct TokExchange {
-    uint32_t last_tag;
+    uint32_t last_tag;                 // of the launches so far
+    uint32_t started;                  // CTAs of this launch that have taken its tag
     alignas(128) ulonglong2 record[kResidentMaxHeads * 128];       // [CTA][row]: maximum, sum
     __device__ void clear() {
         for (ulonglong2& x : record) x = make_ulonglong2(0ull, 0ull);
@@ -175,10 +176,8 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ UMMA issuer
-        if (elect_one()) {
-            const uint32_t last_tag = ld_relaxed(&g_tok_exchange.last_tag);   // (the launch before has ended: griddepcontrol.wait)
-            bool ok = nt == 0 || mbar_wait(smem_u32(&ctl.qfull), 0, abort_flag);
-            *const_cast<volatile uint32_t*>(&ctl.tag) = last_tag + 1u;
+        if (elect_one() && nt > 0) {
+            bool ok = mbar_wait(smem_u32(&ctl.qfull), 0, abort_flag);
             uint32_t st = 0, st_par = 0;
             for (int tg = 0; tg < nt + nt2 && ok; ++tg) {
                 const int buf = tg % kTBufs, use = tg / kTBufs;
@@ -223,6 +222,8 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const int last_visible = a.P + ((row0 + row) % a.w);
         const uint32_t acc = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(grp * 128);
         int tg = grp;                                    // this group's next tile, counted over both passes; tile tg uses accumulator tg % 4
+        // (behind griddepcontrol.wait; beside the first keys' way here, which the issuing thread should not wait for twice)
+        if (et == 0) *const_cast<volatile uint32_t*>(&ctl.tag) = take_tag(g_tok_exchange);
         // ---- pass 1: (max, sum of exp2) per row over this CTA's keys
         float run_m = -CUDART_INF_F, run_l = 0.f;
         bool scored = true;
@@ -259,7 +260,7 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             __threadfence_block();
             __syncwarp();
             uint32_t tag = 0u;
-            while (!*abort_flag && (tag = *const_cast<volatile uint32_t*>(&ctl.tag)) == 0u) {}      // (the issuer's first wait at most)
+            while (!*abort_flag && (tag = *const_cast<volatile uint32_t*>(&ctl.tag)) == 0u) {}      // (long there)
             int old = 0;
             if (lane == 0) old = atomicAdd(&ctl.rec_count[quarter], 1);
             if (__shfl_sync(0xffffffffu, old, 0) == 3) {
@@ -349,10 +350,9 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     }
     if (threadIdx.x == 0) {
         if (ctl.abort_flag) atomicExch(a.status, 1);
-        const unsigned old = atomicAdd(a.exits, 1u);
-        if (old + 1u == gridDim.x) {
+        if (ctl.tag == kLastTag && atomicAdd(a.exits, 1u) + 1u == gridDim.x) {
             *a.exits = 0u;
-            advance_tag(g_tok_exchange, *const_cast<volatile uint32_t*>(&ctl.tag));
+            end_tags(g_tok_exchange);
             __threadfence();
         }
     }
