@@ -720,9 +720,12 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 ok = ctl.abort_flag == 0;
                 if (ok) {
                     const int per = (C + kRThreads - 1) / kRThreads;
+                    // (runs of 6 and 12 as well: 3274 chunks 28.94 -> 28.59 us a layer, 6550 20.98 -> 20.65)
                     if (per <= 2) select_staged<2>(kbuf, C, a.k, ss);
                     else if (per <= 4) select_staged<4>(kbuf, C, a.k, ss);
+                    else if (per <= 6) select_staged<6>(kbuf, C, a.k, ss);
                     else if (per <= 8) select_staged<8>(kbuf, C, a.k, ss);
+                    else if (per <= 12) select_staged<12>(kbuf, C, a.k, ss);
                     else select_staged<16>(kbuf, C, a.k, ss);
                 }
             }
