@@ -56,13 +56,32 @@ select_cluster_kernel(const float* __restrict__ scores, int L, int w, int c, int
     constexpr int nwarps = kCsThreads / 32;
 
     // CTA r owns chunk ids [r S, (r + 1) S); thread t of it a contiguous run of at most kCsKpt ids
-    const int S = (C + kCsCtas - 1) / kCsCtas;
+    // (shares and runs are whole vectors of four: loaded one by one, a run's scores take as many requests as it has ids, 32 sectors each)
+    const int S = ((C + kCsCtas - 1) / kCsCtas + 3) & ~3;
     const int s0 = min(r * S, C), s1 = min(s0 + S, C);
-    const int per = (S + kCsThreads - 1) / kCsThreads;
+    const int per = ((S + kCsThreads - 1) / kCsThreads + 3) & ~3;
     const int c0 = min(s0 + tid * per, s1), c1 = min(c0 + per, s1);
     uint32_t keys[kCsKpt];
+    const bool vec = (reinterpret_cast<uintptr_t>(sc) & 15u) == 0;
 #pragma unroll
-    for (int u = 0; u < kCsKpt; ++u) keys[u] = (c0 + u < c1) ? select_order_key(__ldcg(sc + c0 + u)) : 0u;
+    for (int u = 0; u < kCsKpt; u += 4) {
+        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (vec && c0 + u + 4 <= c1) {
+            f = __ldcg(reinterpret_cast<const float4*>(sc + c0 + u));
+        } else {
+            if (c0 + u < c1) f.x = __ldcg(sc + c0 + u);
+            if (c0 + u + 1 < c1) f.y = __ldcg(sc + c0 + u + 1);
+            if (c0 + u + 2 < c1) f.z = __ldcg(sc + c0 + u + 2);
+            if (c0 + u + 3 < c1) f.w = __ldcg(sc + c0 + u + 3);
+        }
+        keys[u] = select_order_key(f.x);
+        keys[u + 1] = select_order_key(f.y);
+        keys[u + 2] = select_order_key(f.z);
+        keys[u + 3] = select_order_key(f.w);
+    }
+#pragma unroll
+    for (int u = 0; u < kCsKpt; ++u)
+        if (c0 + u >= c1) keys[u] = 0u;
 
     // ---- smallest and largest key of the head
     uint32_t lo = 0xffffffffu, hi = 0u;
