@@ -22,9 +22,9 @@
 // many CTAs gather, and K's second reading is an L2 hit. Past that the partial sums in scratch would double as well.
 //
 // What bounds it (8 KV heads, d 128, B200): up to 128 rows the DRAM stream of K while scoring (12 of
-// 30 us on the device at 32K tokens, c = 10) and then a chain of latencies (two hand-overs, selection, gather);
+// 28.6 us on the device at 32K tokens, c = 10) and then a chain of latencies (two hand-overs, selection, gather);
 // beyond 128 rows the special-function unit (one exponential per score element, 16 per clock and
-// SM: 78 % of that rate while scoring). Against the kernel of score.cu, which keeps every partial sum
+// SM: 80 % of that rate while scoring; 86 % is what this pipeline reaches with nothing else to do). Against the kernel of score.cu, which keeps every partial sum
 // in scratch, loads K once per query tile and takes run-time chunk sizes: c = 16, 32768 tokens, 256 rows
 // 121 -> 41 us; c = 20, 131072 tokens, 256 rows 161 -> 139 us; chunk scores alone (c = 10, 32768
 // tokens, 128 rows, four launches) 32 -> 20 us.
@@ -509,81 +509,81 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     // ---- 3. row statistics of the head, then this CTA's chunk scores
     if (ok) {
         if (a.direct == 0) {
-        if constexpr (FEW) {
-            float M = -CUDART_INF_F, Ls = 0.f;
-            if (threadIdx.x < 512) {
-                const float* src = a.cta_stat + static_cast<size_t>(hs) * a.cph * 256 + (threadIdx.x & 63);
+            if constexpr (FEW) {
+                float M = -CUDART_INF_F, Ls = 0.f;
+                if (threadIdx.x < 512) {
+                    const float* src = a.cta_stat + static_cast<size_t>(hs) * a.cph * 256 + (threadIdx.x & 63);
 #pragma unroll 1
-                for (int j0 = threadIdx.x >> 6; j0 < a.cph; j0 += 40) {
-                    float rm[5], rl[5];
+                    for (int j0 = threadIdx.x >> 6; j0 < a.cph; j0 += 40) {
+                        float rm[5], rl[5];
 #pragma unroll
-                    for (int u = 0; u < 5; ++u) {
-                        const int j = j0 + 8 * u;
-                        rm[u] = (j < a.cph) ? __ldcg(src + j * 256) : -CUDART_INF_F;
-                        rl[u] = (j < a.cph) ? __ldcg(src + j * 256 + 128) : 0.f;
+                        for (int u = 0; u < 5; ++u) {
+                            const int j = j0 + 8 * u;
+                            rm[u] = (j < a.cph) ? __ldcg(src + j * 256) : -CUDART_INF_F;
+                            rl[u] = (j < a.cph) ? __ldcg(src + j * 256 + 128) : 0.f;
+                        }
+#pragma unroll
+                        for (int u = 0; u < 5; ++u) merge_ml(M, Ls, rm[u], rl[u]);
                     }
-#pragma unroll
-                    for (int u = 0; u < 5; ++u) merge_ml(M, Ls, rm[u], rl[u]);
+                    slice[threadIdx.x] = M;
+                    slice[512 + threadIdx.x] = Ls;
                 }
-                slice[threadIdx.x] = M;
-                slice[512 + threadIdx.x] = Ls;
+                __syncthreads();
+                if (threadIdx.x < 64) {
+#pragma unroll
+                    for (int s = 1; s < 8; ++s) merge_ml(M, Ls, slice[s * 64 + threadIdx.x], slice[512 + s * 64 + threadIdx.x]);
+                    gm[threadIdx.x] = M;
+                    ginv[threadIdx.x] = 1.0f / Ls;
+                }
+            }
+            // 512 threads: four (one query tile) or two (two tiles) slices of the records per row
+            if constexpr (!FEW) {
+                const int n_sl = two ? 2 : 4;
+                if (threadIdx.x < 512) {
+                    const int i = threadIdx.x & 127, sl = (threadIdx.x >> 7) & (n_sl - 1), mt = two ? threadIdx.x >> 8 : 0;
+                    const size_t step = static_cast<size_t>(n_mt) * 256;
+                    const float* src = a.cta_stat + (static_cast<size_t>(hs) * a.cph * n_mt + mt) * 256 + i;
+                    float M = -CUDART_INF_F, Ls = 0.f;
+                    // records in flight per thread: enough for one round trip where a head has 18 CTAs (8 heads)
+                    constexpr int kF = BIG ? 9 : 5;
+                    for (int j0 = sl; j0 < a.cph; j0 += kF * n_sl) {
+                        float rm[kF], rl[kF];
+#pragma unroll
+                        for (int u = 0; u < kF; ++u) {
+                            const int j = j0 + n_sl * u;
+                            rm[u] = (j < a.cph) ? __ldcg(src + j * step) : -CUDART_INF_F;
+                            rl[u] = (j < a.cph) ? __ldcg(src + j * step + 128) : 0.f;
+                        }
+                        float bm = M;
+#pragma unroll
+                        for (int u = 0; u < kF; ++u) bm = fmaxf(bm, rm[u]);
+                        float acc = Ls * ex2_below(M, bm);
+#pragma unroll
+                        for (int u = 0; u < kF; ++u) acc += rl[u] * ex2_below(rm[u], bm);
+                        M = bm;
+                        Ls = acc;
+                    }
+                    slice[((threadIdx.x >> 7) * 2 + 0) * 128 + i] = M;
+                    slice[((threadIdx.x >> 7) * 2 + 1) * 128 + i] = Ls;
+                }
+                __syncthreads();
+                if (static_cast<int>(threadIdx.x) < n_mt * 128) {
+                    const int i = threadIdx.x & 127, s0 = (threadIdx.x >> 7) * n_sl;
+                    float M = -CUDART_INF_F, Ls = 0.f;
+#pragma unroll
+                    for (int s = 0; s < 4; ++s)
+                        if (s >= s0 && s < s0 + n_sl) M = fmaxf(M, slice[(s * 2) * 128 + i]);
+#pragma unroll
+                    for (int s = 0; s < 4; ++s)
+                        if (s >= s0 && s < s0 + n_sl) {
+                            const float m = slice[(s * 2) * 128 + i];
+                            Ls += slice[(s * 2 + 1) * 128 + i] * ex2_below(m, M);
+                        }
+                    gm[threadIdx.x] = M;
+                    ginv[threadIdx.x] = 1.0f / Ls;       // rows >= R are never used
+                }
             }
             __syncthreads();
-            if (threadIdx.x < 64) {
-#pragma unroll
-                for (int s = 1; s < 8; ++s) merge_ml(M, Ls, slice[s * 64 + threadIdx.x], slice[512 + s * 64 + threadIdx.x]);
-                gm[threadIdx.x] = M;
-                ginv[threadIdx.x] = 1.0f / Ls;
-            }
-        }
-        // 512 threads: four (one query tile) or two (two tiles) slices of the records per row
-        if constexpr (!FEW) {
-            const int n_sl = two ? 2 : 4;
-            if (threadIdx.x < 512) {
-                const int i = threadIdx.x & 127, sl = (threadIdx.x >> 7) & (n_sl - 1), mt = two ? threadIdx.x >> 8 : 0;
-                const size_t step = static_cast<size_t>(n_mt) * 256;
-                const float* src = a.cta_stat + (static_cast<size_t>(hs) * a.cph * n_mt + mt) * 256 + i;
-                float M = -CUDART_INF_F, Ls = 0.f;
-                // records in flight per thread: enough for one round trip where a head has 18 CTAs (8 heads)
-                constexpr int kF = BIG ? 9 : 5;
-                for (int j0 = sl; j0 < a.cph; j0 += kF * n_sl) {
-                    float rm[kF], rl[kF];
-#pragma unroll
-                    for (int u = 0; u < kF; ++u) {
-                        const int j = j0 + n_sl * u;
-                        rm[u] = (j < a.cph) ? __ldcg(src + j * step) : -CUDART_INF_F;
-                        rl[u] = (j < a.cph) ? __ldcg(src + j * step + 128) : 0.f;
-                    }
-                    float bm = M;
-#pragma unroll
-                    for (int u = 0; u < kF; ++u) bm = fmaxf(bm, rm[u]);
-                    float acc = Ls * ex2_below(M, bm);
-#pragma unroll
-                    for (int u = 0; u < kF; ++u) acc += rl[u] * ex2_below(rm[u], bm);
-                    M = bm;
-                    Ls = acc;
-                }
-                slice[((threadIdx.x >> 7) * 2 + 0) * 128 + i] = M;
-                slice[((threadIdx.x >> 7) * 2 + 1) * 128 + i] = Ls;
-            }
-            __syncthreads();
-            if (static_cast<int>(threadIdx.x) < n_mt * 128) {
-                const int i = threadIdx.x & 127, s0 = (threadIdx.x >> 7) * n_sl;
-                float M = -CUDART_INF_F, Ls = 0.f;
-#pragma unroll
-                for (int s = 0; s < 4; ++s)
-                    if (s >= s0 && s < s0 + n_sl) M = fmaxf(M, slice[(s * 2) * 128 + i]);
-#pragma unroll
-                for (int s = 0; s < 4; ++s)
-                    if (s >= s0 && s < s0 + n_sl) {
-                        const float m = slice[(s * 2) * 128 + i];
-                        Ls += slice[(s * 2 + 1) * 128 + i] * ex2_below(m, M);
-                    }
-                gm[threadIdx.x] = M;
-                ginv[threadIdx.x] = 1.0f / Ls;       // rows >= R are never used
-            }
-        }
-        __syncthreads();
         }
         // chunk scores of this CTA's key range: partial sums x exp2(m_panel - m_i) / l_i, summed over
         // the rows. A thread holds one row of up to 32 chunk slots at a time (PPB panels of its

@@ -21,9 +21,10 @@
 //                  kept-chunk list, moves this CTA's share of the kept K/V rows with bulk asynchronous
 //                  copies (global -> shared -> global, whole chunks at a time) - for the computed
 //                  layer and for every following layer that reuses its indices
-//   warp 19        row statistics: merges the groups' records, stores and announces the CTA's record,
-//                  waits (bounded) for the head's other CTAs, merges their records into m_i and 1 / l_i
-//                  for the contraction, and announces the CTA's chunk scores when they are stored
+//   warp 19        announces the CTA's record of row statistics, which the last of the epilogue warps that hold the same
+//                  32 rows stores, waits (bounded) for the head's other CTAs - the epilogue threads merge the head's
+//                  records for the contraction, this warp itself where a head has very many CTAs - and
+//                  announces the CTA's chunk scores when they are stored
 // The CTAs after the scoring CTAs are selectors: exact top-k per head, out_idx, kept-chunk lists.
 //
 // So while the selectors and copy threads work on layer l, the other warps already score layer l + 1:
@@ -742,10 +743,9 @@ model_kernel(const __grid_constant__ ModelParams p) {
         if (!ok && lane == 0) ctl.abort_flag = 1;
     } else if (warp == 19) {
         // ------------------------------------------------------------------ statistics warp
-        // Per slot: merge the groups' records into the CTA's record, store and announce it, wait (bounded)
-        // until every CTA of the scoring head has done the same, read their records from the L2, merge
-        // them into m_i and 1 / l_i - four rows per lane - and hand the result to the epilogue; then
-        // announce the CTA's chunk scores once the epilogue has stored them.
+        // Per slot: announce the CTA's record once it is stored, wait (bounded) until every CTA of the scoring head has
+        // announced its own, let the epilogue merge them - or, with very many CTAs a head, merge them here into m_i and
+        // 1 / l_i, four rows per lane - and announce the CTA's chunk scores once the epilogue has stored them.
         const int r0 = 4 * lane;
         bool ok = true;
         for (int s = 0; s < p.n_compute && ok; ++s) {
