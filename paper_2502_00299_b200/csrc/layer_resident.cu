@@ -453,10 +453,13 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             if (lane == 0) old = atomicAdd(&ctl.rec_count[mt][quarter], 1);
             if (__shfl_sync(0xffffffffu, old, 0) == n_g - 1) {
                 __threadfence_block();
-                float M = -CUDART_INF_F, S = 0.f;
+                float M = -CUDART_INF_F, S = 0.f, m[4], l[4];
 #pragma unroll
-                for (int g = 0; g < 4; ++g)
-                    if (g < n_g) merge_ml(M, S, rec[((mt * 2 + g) * 2) * 128 + row], rec[((mt * 2 + g) * 2 + 1) * 128 + row]);
+                for (int g = 0; g < 4; ++g) {
+                    m[g] = g < n_g ? rec[((mt * 2 + g) * 2) * 128 + row] : -CUDART_INF_F;
+                    l[g] = g < n_g ? rec[((mt * 2 + g) * 2 + 1) * 128 + row] : 0.f;
+                }
+                merge_records(M, S, m, l);
                 if (tag != 0u) st_tagged2(&g_exchange.record[(static_cast<size_t>(blockIdx.x) * n_mt + mt) * 128 + row], M, S, tag);
             }
             constexpr int KF = BIG ? 9 : 5;              // records in flight per thread: one round trip where a head has 18 CTAs (8 heads)
@@ -467,7 +470,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 const size_t step = static_cast<size_t>(n_mt) * 128;
                 const ulonglong2* src = g_exchange.record + (static_cast<size_t>(hs) * a.cph * n_mt + mt) * 128 + prow;
                 for (int j0 = sl; j0 < a.cph; j0 += KF * n_sl)
-                    if (!take_records<KF>(src + j0 * step, n_sl * step, min(KF, (a.cph - j0 + n_sl - 1) / n_sl), tag, M, S, abort_flag)) break;
+                    if (!take_records<KF, FEW>(src + j0 * step, n_sl * step, min(KF, (a.cph - j0 + n_sl - 1) / n_sl), tag, M, S, abort_flag)) break;
             }
             if constexpr (FEW) {
                 slice[sl * 64 + prow] = M;
@@ -609,9 +612,14 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
 #pragma unroll
                     for (int u = 0; u < 8; ++u) merge_ml(M, S, slice[u * 64 + (row & 63)], slice[512 + u * 64 + (row & 63)]);
                 } else {
+                    float m[4], l[4];
 #pragma unroll
-                    for (int g = 0; g < 4; ++g)
-                        if (!two || (g >> 1) == mt) merge_ml(M, S, slice[(g * 2) * 128 + row], slice[(g * 2 + 1) * 128 + row]);
+                    for (int g = 0; g < 4; ++g) {
+                        const bool mine = !two || (g >> 1) == mt;
+                        m[g] = mine ? slice[(g * 2) * 128 + row] : -CUDART_INF_F;
+                        l[g] = mine ? slice[(g * 2 + 1) * 128 + row] : 0.f;
+                    }
+                    merge_records(M, S, m, l);
                 }
                 mi = M;
                 li = 1.0f / S;

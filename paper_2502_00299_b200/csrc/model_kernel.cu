@@ -715,10 +715,13 @@ model_kernel(const __grid_constant__ ModelParams p) {
             if (lane == 0) old = atomicAdd(cnt, 1);
             if (__shfl_sync(0xffffffffu, old, 0) == n_g - 1) {
                 __threadfence_block();
-                float M = -CUDART_INF_F, S = 0.f;
+                float M = -CUDART_INF_F, S = 0.f, m[4], l[4];
 #pragma unroll
-                for (int g = 0; g < 4; ++g)
-                    if (g < n_g) merge_ml(M, S, rc[((mt * 2 + g) * 2) * 128 + row], rc[((mt * 2 + g) * 2 + 1) * 128 + row]);
+                for (int g = 0; g < 4; ++g) {
+                    m[g] = g < n_g ? rc[((mt * 2 + g) * 2) * 128 + row] : -CUDART_INF_F;
+                    l[g] = g < n_g ? rc[((mt * 2 + g) * 2 + 1) * 128 + row] : 0.f;
+                }
+                merge_records(M, S, m, l);
                 float* dst = p.cta_stat + ((static_cast<size_t>(s & 1) * gridDim.x + blockIdx.x) * n_mt + mt) * 256;
                 dst[row] = M;
                 dst[128 + row] = S;

@@ -91,9 +91,22 @@ __device__ __forceinline__ void merge_ml(float& M, float& S, float m, float s) {
     M = nm;
 }
 
+// The same for N records at a time: the largest maximum first, then each record's sum with one factor.
+template <int N>
+__device__ __forceinline__ void merge_records(float& M, float& S, const float (&m)[N], const float (&l)[N]) {
+    float bm = M;
+#pragma unroll
+    for (int u = 0; u < N; ++u) bm = fmaxf(bm, m[u]);
+    float acc = S * ex2_below(M, bm);
+#pragma unroll
+    for (int u = 0; u < N; ++u) acc += l[u] * ex2_below(m[u], bm);
+    M = bm;
+    S = acc;
+}
+
 // Up to KF records of a row (one every `step`, from `src`) in one round trip, as often as it takes until all of them carry this
-// launch's tag; merged into (M, S). False: given up.
-template <int KF>
+// launch's tag; merged into (M, S), all at once or one after the other. False: given up.
+template <int KF, bool IN_TURN>
 __device__ __forceinline__ bool take_records(const ulonglong2* src, size_t step, int n, uint32_t tag, float& M, float& S, volatile int* abort_flag) {
     ulonglong2 r[KF];
     unsigned missing = (1u << n) - 1u;
@@ -112,16 +125,18 @@ __device__ __forceinline__ bool take_records(const ulonglong2* src, size_t step,
             if (clock64() - t0 > kWaitLimitClocks) { *abort_flag = 1; return false; }
         }
     }
-    float bm = M;
+    float m[KF], l[KF];
 #pragma unroll
-    for (int u = 0; u < KF; ++u)
-        if (u < n) bm = fmaxf(bm, tagged_value(r[u].x));
-    float acc = S * ex2_below(M, bm);
+    for (int u = 0; u < KF; ++u) {
+        m[u] = u < n ? tagged_value(r[u].x) : __int_as_float(0xff800000);
+        l[u] = u < n ? tagged_value(r[u].y) : 0.f;
+    }
+    if constexpr (IN_TURN) {
 #pragma unroll
-    for (int u = 0; u < KF; ++u)
-        if (u < n) acc += tagged_value(r[u].y) * ex2_below(tagged_value(r[u].x), bm);
-    M = bm;
-    S = acc;
+        for (int u = 0; u < KF; ++u) merge_ml(M, S, m[u], l[u]);
+    } else {
+        merge_records(M, S, m, l);
+    }
     return true;
 }
 

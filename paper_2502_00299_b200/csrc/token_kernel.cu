@@ -274,7 +274,7 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             if (tag != 0u && active) {
                 const ulonglong2* src = g_tok_exchange.record + static_cast<size_t>(hs) * a.cph * 128 + row;
                 for (int j0 = grp; j0 < a.cph; j0 += 20)             // five records in flight
-                    if (!take_records<5>(src + j0 * 128, 4 * 128, min(5, (a.cph - j0 + 3) / 4), tag, M, S, abort_flag)) break;
+                    if (!take_records<5, true>(src + j0 * 128, 4 * 128, min(5, (a.cph - j0 + 3) / 4), tag, M, S, abort_flag)) break;
             }
             slice[(grp * 2 + 0) * 128 + row] = M;
             slice[(grp * 2 + 1) * 128 + row] = S;
