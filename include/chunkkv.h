@@ -40,6 +40,8 @@
  *     may differ in their last bits.) Calls that use the
  *     scratch of one device must be ordered on the GPU (same stream, or otherwise serialised):
  *     concurrent calls would share it. Lanes and pipes (below) take their scratch per object.
+ *     (Calls outside lanes also hand values from SM to SM through 1.4 MB of device memory that is
+ *     part of the library's image, in the same order.)
  */
 #ifndef CHUNKKV_H_
 #define CHUNKKV_H_
