@@ -93,6 +93,17 @@ struct Exchange {
 __device__ Exchange g_exchange;
 enum { kDirectRecords = 1, kDirectScores = 2 };
 
+// After scoring the ring holds the selection's scratch, then the head's keys if they fit. A CTA lists the head's kept chunks where the
+// list has room for them and, but for the wide variant, a thread takes all of its keys at once; else it works on the scores in global
+// memory. Chunk scores go through g_exchange only where every CTA lists, so the host asks the same function as the kernel.
+constexpr size_t kRSelBytes = (sizeof(SelectSmem) + 127) & ~size_t(127);
+__host__ __device__ constexpr bool keys_fit(int C, int ring_bytes) {
+    return kRSelBytes + (static_cast<size_t>(C) + 4) * 4 <= static_cast<size_t>(ring_bytes);
+}
+__host__ __device__ constexpr bool lists_kept(bool wide, int C, int k, int ring_bytes) {
+    return (k < C ? k : C) <= kSelCap && C <= kSelMaxChunks && keys_fit(C, ring_bytes) && (wide || C <= kRThreads * select_reg_keys(kSelLayer));
+}
+
 struct ResArgs {
     int L, P, w, R, d;                 // R rows per KV head
     short n_mt;                        // 128-row query tiles per KV head (1 or 2)
@@ -695,7 +706,6 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
     }
     if (ok && a.out_idx != nullptr) {
         SelectSmem& ss = *reinterpret_cast<SelectSmem*>(ring);
-        constexpr size_t kSelBytes = (sizeof(SelectSmem) + 127) & ~size_t(127);
         const int shift = BIG ? 0 : a.shift;
         const size_t row_at = (static_cast<size_t>(hkv) << shift) * a.score_row;
         const float* sc = a.scores + row_at;
@@ -704,14 +714,12 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         const int r_begin = static_cast<int>(static_cast<long long>(a.n_max) * q / Q);
         const int r_end = static_cast<int>(static_cast<long long>(a.n_max) * (q + 1) / Q);
         int32_t* out_idx = a.out_idx + static_cast<size_t>(hkv) * a.n_max;
-        uint32_t* kbuf = reinterpret_cast<uint32_t*>(ring + kSelBytes);
-        const bool fits = kSelBytes + (static_cast<size_t>(C) + 4) * 4 <= static_cast<size_t>(a.ring_bytes);
+        uint32_t* kbuf = reinterpret_cast<uint32_t*>(ring + kRSelBytes);
         // every CTA holds the head's kept chunks: it expands, writes and gathers its own share of the positions
-        bool listed = min(a.k, C) <= kSelCap && C <= kSelMaxChunks && fits;
+        const bool listed = lists_kept(WIDE, C, a.k, a.ring_bytes);
         if constexpr (WIDE) {
             if (listed) select_kept<kSelLayerWide>(sc, sc2, C, a.k, ss, kbuf);
         } else {
-            listed = listed && C <= kRThreads * select_reg_keys(kSelLayer);
             if (listed && !select_all(C, a.k, ss)) {
                 uint32_t lo = 0xffffffffu, hi = 0u;
                 select_clear(ss);
@@ -738,9 +746,9 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 }
             }
         }
-        // very many chunks: every CTA of the head writes the same positions to out_idx and takes its share from there
+        // very many chunks, or very many kept: every CTA of the head writes the same positions to out_idx and takes its share from there
         if (!listed) {
-            select_head_rows(sc, sc2, a.L, a.w, C_STATIC, C, a.k, a.n_max, out_idx, ss, fits ? kbuf : nullptr, a.tok_cap);
+            select_head_rows(sc, sc2, a.L, a.w, C_STATIC, C, a.k, a.n_max, out_idx, ss, keys_fit(C, a.ring_bytes) ? kbuf : nullptr, a.tok_cap);
             __syncthreads();
         }
         if (ok) {
@@ -866,7 +874,8 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     a.sl2 = io.sl2;
     a.cph = plan.cph; a.n_stages = plan.n_stages;
     a.direct = io.cooperative ? 0
-             : kDirectRecords | (io.out_idx != nullptr && !wide && static_cast<long long>(io.Hkv << plan.shift) * ((io.C + 3) & ~3) <= kXScores ? kDirectScores : 0);
+             : kDirectRecords | (io.out_idx != nullptr && !wide && lists_kept(false, io.C, io.k, plan.ring_bytes) &&
+                               static_cast<long long>(io.Hkv << plan.shift) * ((io.C + 3) & ~3) <= kXScores ? kDirectScores : 0);
     a.shift = static_cast<short>(plan.shift); a.q_rows = resident_q_box_rows(plan, io.R);
     a.k = io.k; a.n_max = io.n_max; a.Hkv = io.Hkv;
     a.n_on = plan.n_on; a.n_off = plan.n_off; a.spill_rows = plan.spill_rows;
