@@ -14,6 +14,7 @@ namespace chunkkv {
 constexpr size_t kHeaderBytes = 2048;
 constexpr size_t kResidentCountersOffset = 192;
 constexpr int kResidentMaxHeads = 148;   // three counter arrays of this length follow the exit counter
+constexpr int kExchangeCtas = 160;       // CTAs of a launch whose row records the tables of tagged words hold
 
 // Geometry of one scoring launch, fixed on the host.
 struct ScorePlan {
@@ -125,6 +126,8 @@ bool make_resident_plan(int L, int R, int Hkv, int d, int c, int C, int n_max, i
                         ResidentPlan* plan);
 // Rows of a box of the query tensor map.
 inline int resident_q_box_rows(const ResidentPlan& plan, int R) { return plan.shift ? (R + 1) / 2 : (R < 128 ? R : 128); }
+// Whether the launch's row records fit the table of tagged words (a GPU with more SMs: counters instead).
+inline bool resident_tagged(const ResidentPlan& plan) { return plan.grid <= kExchangeCtas; }
 size_t resident_scratch_floats(const ResidentPlan& plan, int Hkv, int C);
 cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                                   const ResidentIO& io, cudaStream_t stream);

@@ -83,7 +83,7 @@ constexpr int kXScores = 65536;        // chunk scores of all scoring heads that
 struct Exchange {
     uint32_t last_tag;                 // of the launches so far
     uint32_t started;                  // CTAs of this launch that have taken its tag
-    alignas(128) ulonglong2 record[kResidentMaxHeads * 2 * 128];   // [CTA, query tile][row]: maximum, sum
+    alignas(128) ulonglong2 record[kExchangeCtas * 2 * 128];   // [CTA, query tile][row]: maximum, sum
     ulonglong2 score[kXScores / 2];    // [scoring head][score_row / 2]
     __device__ void clear() {
         for (ulonglong2& x : record) x = make_ulonglong2(0ull, 0ull);
@@ -873,7 +873,7 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     a.L = io.L; a.P = io.L - io.w; a.w = io.w; a.R = io.R; a.d = io.d; a.n_mt = static_cast<short>(plan.n_mt);
     a.sl2 = io.sl2;
     a.cph = plan.cph; a.n_stages = plan.n_stages;
-    a.direct = io.cooperative ? 0
+    a.direct = io.cooperative || !resident_tagged(plan) ? 0
              : kDirectRecords | (io.out_idx != nullptr && !wide && lists_kept(false, io.C, io.k, plan.ring_bytes) &&
                                static_cast<long long>(io.Hkv << plan.shift) * ((io.C + 3) & ~3) <= kXScores ? kDirectScores : 0);
     a.shift = static_cast<short>(plan.shift); a.q_rows = resident_q_box_rows(plan, io.R);

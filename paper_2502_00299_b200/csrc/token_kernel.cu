@@ -52,7 +52,7 @@ struct TokCtl {
 struct TokExchange {
     uint32_t last_tag;                 // of the launches so far
     uint32_t started;                  // CTAs of this launch that have taken its tag
-    alignas(128) ulonglong2 record[kResidentMaxHeads * 128];       // [CTA][row]: maximum, sum
+    alignas(128) ulonglong2 record[kExchangeCtas * 128];   // [CTA][row]: maximum, sum
     __device__ void clear() {
         for (ulonglong2& x : record) x = make_ulonglong2(0ull, 0ull);
     }
@@ -367,7 +367,7 @@ bool make_token_plan(int L, int w, int R, int Hkv, int d, int max_ctas, int smem
     TokenPlan p{};
     p.n_mt = n_mt;
     p.Hs = Hs;
-    p.cph = max_ctas / Hs;
+    p.cph = (max_ctas < kExchangeCtas ? max_ctas : kExchangeCtas) / Hs;
     p.grid = p.cph * Hs;
     p.n_tiles = (L + kTTile - 1) / kTTile;
     p.n_tiles_prefix = (L - w + kTTile - 1) / kTTile;
