@@ -40,8 +40,10 @@
  *     may differ in their last bits.) Calls that use the
  *     scratch of one device must be ordered on the GPU (same stream, or otherwise serialised):
  *     concurrent calls would share it. Lanes and pipes (below) take their scratch per object.
- *     (Calls outside lanes also hand values from SM to SM through 1.4 MB of device memory that is
- *     part of the library's image, in the same order.)
+ *     (Calls outside lanes also hand values from SM to SM through 1.2 MB of device memory that is
+ *     part of the library's image. Each scratch that calls are captured on into a CUDA graph has
+ *     such words of its own, so graphs over different scratch may run side by side and beside
+ *     other calls; from the ninth such scratch of a device on, calls on it are slower.)
  */
 #ifndef CHUNKKV_H_
 #define CHUNKKV_H_

@@ -32,6 +32,9 @@ struct DeviceCtx {
     int smem_optin = 0;
     void* ws = nullptr;        // scratch handed over with chunkkv_set_workspace (header + payload)
     size_t ws_bytes = 0;
+    Exchange* slots = nullptr;                            // the device's sets of tagged words
+    int slot = -1;                                        // the one that calls on `ws` use; -1: none is left
+    const void* captured_on[kExchangeSlots] = {nullptr};  // the scratch of captured calls that use a set
     std::vector<ProfileRec> recs;
     float prof_ms[CHUNKKV_PROFILE_SLOTS] = {0, 0, 0, 0};
     int prof_n[CHUNKKV_PROFILE_SLOTS] = {0, 0, 0, 0};
@@ -95,6 +98,31 @@ int ensure_workspace(DeviceCtx& c, size_t payload_bytes) {
     if (c.ws != nullptr && c.ws_bytes >= need) return CHUNKKV_OK;
     return CHUNKKV_ENOWORKSPACE;
 }
+
+// Calls on one scratch are ordered, and another scratch is only set when the device is idle; but captured calls run whenever
+// their graph does, beside the calls on another scratch. So a scratch that calls were captured on keeps its set of tagged words for
+// good (known by its address: a later buffer at that address could not be used beside it either), and while none of the sets is
+// left for a scratch, its calls hand over by counters in the scratch. Caller holds g_mu; once per launch.
+Exchange* take_exchange(DeviceCtx& c, cudaStream_t stream) {
+    if (c.slot < 0) return nullptr;
+    if (c.captured_on[c.slot] == nullptr) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(stream, &cap);
+        if (e != cudaSuccess) cudaGetLastError();
+        if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) c.captured_on[c.slot] = c.ws;
+    }
+    return exchange_slot(c.slots, c.slot);
+}
+int find_exchange(const DeviceCtx& c, const void* ws) {
+    for (int i = 0; i < kExchangeSlots; ++i)
+        if (c.captured_on[i] == ws) return i;
+    for (int i = 0; i < kExchangeSlots; ++i)
+        if (c.captured_on[i] == nullptr) return i;
+    return -1;
+}
+
+// The token kernel has no other hand-over: without a set of tagged words token-level calls take the kernels of score.cu.
+bool token_kernel_runs(const DeviceCtx& c) { return c.ws == nullptr || c.slot >= 0; }
 
 // How the R = w * Hq / Hkv window rows of a KV head are scored. Rows are independent (each has its
 // own softmax) and chunk scores are sums over rows, so more than 128 rows of an even number of
@@ -201,6 +229,7 @@ int try_resident(DeviceCtx& ctx, char* base, size_t bytes, const ResidentCall& r
     io.scratch = reinterpret_cast<float*>(base + kHeaderBytes);
     io.counters = reinterpret_cast<unsigned*>(base + kResidentCountersOffset);
     io.cooperative = rc.cooperative;
+    if (!rc.cooperative) io.exchange = take_exchange(ctx, stream);
     io.k_row_elems = rc.kt; io.k_head_elems = rc.kh; io.v_row_elems = rc.vt; io.v_head_elems = rc.vh;
     io.block_table = rc.block_table; io.page_size = rc.page_size; io.num_pages = rc.num_pages;
     io.tok_cap = rc.tok_cap;
@@ -242,7 +271,7 @@ int run_score(DeviceCtx& ctx, const void* q_obs, const void* K, int L, int Hq, i
     }
     TokenPlan tplan;
     const int rows = w * (Hq / Hkv);
-    if (c == 1 && make_token_plan(L, w, rows, Hkv, d, ctx.num_sms, smem_budget(ctx), &tplan)) {
+    if (c == 1 && token_kernel_runs(ctx) && make_token_plan(L, w, rows, Hkv, d, ctx.num_sms, smem_budget(ctx), &tplan)) {
         // token scores: two passes over the keys in one launch, no scratch but the second half of rows
         const size_t pair_t = tplan.n_mt == 2 ? round64(static_cast<size_t>(tplan.Hs) * C) : 0;
         const size_t tfloats = extra_payload_floats + pair_t;
@@ -261,6 +290,7 @@ int run_score(DeviceCtx& ctx, const void* q_obs, const void* K, int L, int Hq, i
         io.L = L; io.w = w; io.R = rows; io.d = d;
         io.sl2 = static_cast<float>(1.4426950408889634 / sqrt(static_cast<double>(d)));
         io.token_scores = head_scores;
+        io.exchange = take_exchange(ctx, stream);
         io.counters = reinterpret_cast<unsigned*>(static_cast<char*>(ctx.ws) + kResidentCountersOffset);
         io.status = static_cast<int*>(ctx.ws);
         cudaError_t e2;
@@ -459,16 +489,20 @@ int chunkkv_set_workspace(void* dev_ptr, size_t bytes) {
     if (dev_ptr == nullptr) {
         ctx->ws = nullptr;
         ctx->ws_bytes = 0;
+        ctx->slot = -1;
         return CHUNKKV_OK;
     }
     if ((reinterpret_cast<uintptr_t>(dev_ptr) & 255u) != 0) return CHUNKKV_EINVAL_ALIGN;
     if (bytes < kHeaderBytes) return CHUNKKV_ENOWORKSPACE;
+    e = exchange_slots(&ctx->slots);
+    if (e != cudaSuccess) return cuda_fail(e);
     e = cudaMemset(dev_ptr, 0, kHeaderBytes);
     if (e != cudaSuccess) return cuda_fail(e);
     e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_fail(e);
     ctx->ws = dev_ptr;
     ctx->ws_bytes = bytes;
+    ctx->slot = find_exchange(*ctx, dev_ptr);
     return CHUNKKV_OK;
 }
 
@@ -485,6 +519,8 @@ int chunkkv_device_status(void* stream) {
     if (e != cudaSuccess) return cuda_fail(e);
     if (flag != 0) {
         cudaMemset(ctx->ws, 0, kHeaderBytes);   // status word and grid-barrier words
+        // (the tag stays, so that old words stay old; calls that were not ordered may have left a count)
+        if (ctx->slot >= 0) cudaMemset(exchange_tags(exchange_slot(ctx->slots, ctx->slot)) + 1, 0, sizeof(uint32_t));
         return CHUNKKV_EDEVICE;
     }
     return CHUNKKV_OK;
@@ -621,7 +657,7 @@ static int compress_impl(const void* q_obs, const void* K, const void* V, int L,
         ScorePlan plan;
         TokenPlan tplan;
         // token-level layers on the whole GPU: the two-pass token-score kernel, then select and gather
-        const bool token_path = c == 1 && lane == nullptr && rows_elsewhere == nullptr &&
+        const bool token_path = c == 1 && token_kernel_runs(*ctx) && lane == nullptr && rows_elsewhere == nullptr &&
                                 make_token_plan(L, w, w * (Hq / Hkv), Hkv, d, ctx->num_sms, smem_budget(*ctx), &tplan);
         if (!token_path && make_score_plan(L, R, sh.Hs, d, c, ctas, smem_budget(*ctx), true, &plan)) {
             // One cooperative launch for the whole layer.

@@ -14,7 +14,14 @@ namespace chunkkv {
 constexpr size_t kHeaderBytes = 2048;
 constexpr size_t kResidentCountersOffset = 192;
 constexpr int kResidentMaxHeads = 148;   // three counter arrays of this length follow the exit counter
-constexpr int kExchangeCtas = 160;       // CTAs of a launch whose row records the tables of tagged words hold
+constexpr int kExchangeCtas = 160;       // CTAs of a launch whose row records a table of tagged words holds
+constexpr int kExchangeSlots = 8;        // sets of such tables on a device
+
+// A set of tagged words (resident.cuh), in device memory of the library's image.
+struct Exchange;
+cudaError_t exchange_slots(Exchange** slots);                // the current device's; loads the module, so for set-up calls
+Exchange* exchange_slot(Exchange* slots, int slot);
+uint32_t* exchange_tags(Exchange* x);                        // last tag, CTAs that have taken the tag of a launch under way
 
 // Geometry of one scoring launch, fixed on the host.
 struct ScorePlan {
@@ -110,6 +117,7 @@ struct ResidentIO {
     float* out_scores = nullptr;   // [Hkv, C]; NULL: in scratch
     float* scratch;       // resident_scratch_floats() floats
     unsigned* counters;   // header + kResidentCountersOffset (the status word is the header's first)
+    Exchange* exchange = nullptr;  // tagged words of the calls on this scratch; NULL: hand-overs by counters
     bool cooperative;     // cooperative launch (lanes: several launches share the GPU) instead of a programmatic dependent one
     // elements between consecutive rows of a head and between heads of K and of V; 0 = packed [Hkv, L, d]
     long long k_row_elems = 0, k_head_elems = 0, v_row_elems = 0, v_head_elems = 0;
@@ -191,6 +199,7 @@ struct TokenIO {
     int L, w, R, d;       // R = w * Hq / Hkv query rows per KV head
     float sl2;
     float* token_scores;  // [Hs][P]
+    Exchange* exchange;   // tagged words of the calls on this scratch
     unsigned* counters;   // header + kResidentCountersOffset
     int* status;
 };

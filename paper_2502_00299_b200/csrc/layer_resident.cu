@@ -75,27 +75,12 @@ struct ResCtl {
     int wait_ok;
 };
 
-// Hand-overs of the launches that have the GPU to themselves carry their data (tagged words, resident.cuh), which leaves out the release, the
-// counter and the read behind it: two round trips of the L2 for each of the two (2048 tokens, 2 heads 11.84 -> 11.06 us, 8192 16.3 -> 15.4,
-// 32768 29.2 -> 28.7, 9 CTAs a head 15.6 -> 14.6, 74 22.26 -> 21.31). The tag is the launch's number, so nothing
-// has to be cleared. Launches that share the GPU with others of their kind (lanes) keep the counters and their own scratch.
-constexpr int kXScores = 65536;        // chunk scores of all scoring heads that fit (more: the second hand-over by counters)
-struct Exchange {
-    uint32_t last_tag;                 // of the launches so far
-    uint32_t started;                  // CTAs of this launch that have taken its tag
-    alignas(128) ulonglong2 record[kExchangeCtas * 2 * 128];   // [CTA, query tile][row]: maximum, sum
-    ulonglong2 score[kXScores / 2];    // [scoring head][score_row / 2]
-    __device__ void clear() {
-        for (ulonglong2& x : record) x = make_ulonglong2(0ull, 0ull);
-        for (ulonglong2& x : score) x = make_ulonglong2(0ull, 0ull);
-    }
-};
-__device__ Exchange g_exchange;
+__device__ Exchange g_exchange[kExchangeSlots];
 enum { kDirectRecords = 1, kDirectScores = 2 };
 
 // After scoring the ring holds the selection's scratch, then the head's keys if they fit. A CTA lists the head's kept chunks where the
 // list has room for them and, but for the wide variant, a thread takes all of its keys at once; else it works on the scores in global
-// memory. Chunk scores go through g_exchange only where every CTA lists, so the host asks the same function as the kernel.
+// memory. Chunk scores go through the exchange only where every CTA lists, so the host asks the same function as the kernel.
 constexpr size_t kRSelBytes = (sizeof(SelectSmem) + 127) & ~size_t(127);
 __host__ __device__ constexpr bool keys_fit(int C, int ring_bytes) {
     return kRSelBytes + (static_cast<size_t>(C) + 4) * 4 <= static_cast<size_t>(ring_bytes);
@@ -108,7 +93,7 @@ struct ResArgs {
     int L, P, w, R, d;                 // R rows per KV head
     short n_mt;                        // 128-row query tiles per KV head (1 or 2)
     short shift;                       // 1: the rows of a KV head are scored as two heads of q_rows and the rest
-    int direct;                        // hand-overs that go through g_exchange
+    int direct;                        // hand-overs that go through the exchange
     int q_rows;                        // rows of a box of the query tensor map: 128, fewer, or the half's
     float sl2;                         // log2(e) / sqrt(d)
     int cph;                           // CTAs per scoring head (a KV head, or one of its halves)
@@ -126,7 +111,10 @@ struct ResArgs {
     uint4* out_K;
     uint4* out_V;
     int32_t* out_idx;
-    float* cta_stat;                   // [grid, n_mt, {max, sum}, 128]
+    union {
+        float* cta_stat;               // [grid, n_mt, {max, sum}, 128] (hand-over by counters)
+        Exchange* x;                   // (direct != 0)
+    };
     float* scores;                     // [Hkv, score_row]
     int score_row;                     // C, or C rounded up to a multiple of 4 in scratch (16-byte aligned rows)
     float* spill;                      // [grid, n_off, (chunk slots per panel + 1) * spill_rows]: chunk sums, panel maximum
@@ -409,7 +397,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
         const uint64_t keep = l2_policy_evict_last();
         // (behind griddepcontrol.wait; beside the first keys' way here, which the issuing thread should not wait for twice)
-        if (a.direct != 0 && threadIdx.x == 64) *const_cast<volatile uint32_t*>(&ctl.tag) = take_tag(g_exchange);
+        if (a.direct != 0 && threadIdx.x == 64) *const_cast<volatile uint32_t*>(&ctl.tag) = take_tag(*a.x);
         float run_m = -CUDART_INF_F, run_l = 0.f;
         bool scored = true;
         for (int vt = pair; vt < n_vt; vt += 2) {
@@ -471,7 +459,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                     l[g] = g < n_g ? rec[((mt * 2 + g) * 2 + 1) * 128 + row] : 0.f;
                 }
                 merge_records(M, S, m, l);
-                if (tag != 0u) st_tagged2(&g_exchange.record[(static_cast<size_t>(blockIdx.x) * n_mt + mt) * 128 + row], M, S, tag);
+                if (tag != 0u) st_tagged2(&a.x->record[(static_cast<size_t>(blockIdx.x) * n_mt + mt) * 128 + row], M, S, tag);
             }
             constexpr int KF = BIG ? 9 : 5;              // records in flight per thread: one round trip where a head has 18 CTAs (8 heads)
             const int n_sl = FEW ? 8 : (two ? 2 : 4), sl = FEW ? grp * 2 + (quarter >> 1) : (two ? half : grp);
@@ -479,7 +467,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             float M = -CUDART_INF_F, S = 0.f;
             if (tag != 0u && (FEW ? prow < n_rows : active)) {
                 const size_t step = static_cast<size_t>(n_mt) * 128;
-                const ulonglong2* src = g_exchange.record + (static_cast<size_t>(hs) * a.cph * n_mt + mt) * 128 + prow;
+                const ulonglong2* src = a.x->record + (static_cast<size_t>(hs) * a.cph * n_mt + mt) * 128 + prow;
                 for (int j0 = sl; j0 < a.cph; j0 += KF * n_sl)
                     if (!take_records<KF, FEW>(src + j0 * step, n_sl * step, min(KF, (a.cph - j0 + n_sl - 1) / n_sl), tag, M, S, abort_flag)) break;
             }
@@ -695,7 +683,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 float t = (r[0] + r[n_local]) + (r[2 * n_local] + r[3 * n_local]);
                 if (two) t += (r[4 * n_local] + r[5 * n_local]) + (r[6 * n_local] + r[7 * n_local]);
                 const size_t at = static_cast<size_t>(hs) * a.score_row + ch0 + lc;
-                if (a.direct & kDirectScores) st_tagged(reinterpret_cast<unsigned long long*>(g_exchange.score) + at, t, ctl.tag);
+                if (a.direct & kDirectScores) st_tagged(reinterpret_cast<unsigned long long*>(a.x->score) + at, t, ctl.tag);
                 else a.scores[at] = t;
             }
     }
@@ -724,7 +712,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
                 uint32_t lo = 0xffffffffu, hi = 0u;
                 select_clear(ss);
                 if (a.direct & kDirectScores) {
-                    const ulonglong2* x = g_exchange.score + row_at / 2;
+                    const ulonglong2* x = a.x->score + row_at / 2;
                     take_scores(x, shift ? x + a.score_row / 2 : nullptr, C, ctl.tag, kbuf, lo, hi, abort_flag);
                 } else {
                     load_scores(sc, sc2, C, kbuf, lo, hi);
@@ -786,7 +774,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
         if ((counted || last_tag) && atomicAdd(a.exits(), 1u) + 1u == gridDim.x) {
             for (int h = 0; h < a.Hkv << a.shift; ++h) { *a.cnt_a(h) = 0u; *a.cnt_b(h) = 0u; }
             *a.exits() = 0u;
-            if (last_tag) end_tags(g_exchange);
+            if (last_tag) end_tags(*a.x);
             __threadfence();
         }
     }
@@ -806,6 +794,10 @@ const void* kernel_of(int variant, bool wide) {
 }
 
 }  // namespace
+
+cudaError_t exchange_slots(Exchange** slots) { return cudaGetSymbolAddress(reinterpret_cast<void**>(slots), g_exchange); }
+Exchange* exchange_slot(Exchange* slots, int slot) { return slots + slot; }
+uint32_t* exchange_tags(Exchange* x) { return &x->last_tag; }
 
 size_t resident_scratch_floats(const ResidentPlan& plan, int Hkv, int C) {
     return static_cast<size_t>(plan.grid) * plan.n_mt * 256 + (((static_cast<size_t>(Hkv) << plan.shift) * ((C + 3) & ~3) + 63) & ~static_cast<size_t>(63)) +
@@ -873,7 +865,7 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
     a.L = io.L; a.P = io.L - io.w; a.w = io.w; a.R = io.R; a.d = io.d; a.n_mt = static_cast<short>(plan.n_mt);
     a.sl2 = io.sl2;
     a.cph = plan.cph; a.n_stages = plan.n_stages;
-    a.direct = io.cooperative || !resident_tagged(plan) ? 0
+    a.direct = io.cooperative || io.exchange == nullptr || !resident_tagged(plan) ? 0
              : kDirectRecords | (io.out_idx != nullptr && !wide && lists_kept(false, io.C, io.k, plan.ring_bytes) &&
                                static_cast<long long>(io.Hkv << plan.shift) * ((io.C + 3) & ~3) <= kXScores ? kDirectScores : 0);
     a.shift = static_cast<short>(plan.shift); a.q_rows = resident_q_box_rows(plan, io.R);
@@ -891,7 +883,8 @@ cudaError_t launch_layer_resident(const ResidentPlan& plan, const CUtensorMap& t
         a.v_head = io.v_head_elems ? io.v_head_elems / 8 : static_cast<long long>(io.L) * vpr;
     }
     a.out_K = static_cast<uint4*>(io.out_K); a.out_V = static_cast<uint4*>(io.out_V); a.out_idx = io.out_idx;
-    a.cta_stat = io.scratch;
+    if (a.direct != 0) a.x = io.exchange;
+    else a.cta_stat = io.scratch;
     float* scores = io.scratch + static_cast<size_t>(plan.grid) * plan.n_mt * 256;
     a.scores = io.out_scores ? io.out_scores : scores;
     a.score_row = io.out_scores ? io.C : (io.C + 3) & ~3;

@@ -140,14 +140,30 @@ __device__ __forceinline__ bool take_records(const ulonglong2* src, size_t step,
     return true;
 }
 
+// Hand-overs of the launches that have the GPU to themselves carry their data, which leaves out the release, the
+// counter and the read behind it: two round trips of the L2 for each of the two (2048 tokens, 2 heads 11.84 -> 11.06 us, 8192 16.3 -> 15.4,
+// 32768 29.2 -> 28.7, 9 CTAs a head 15.6 -> 14.6, 74 22.26 -> 21.31). The tag is the launch's number, so nothing
+// has to be cleared. Launches that share the GPU with others of their kind (lanes) keep the counters and their own scratch.
+// Launches on one scratch buffer are ordered, so one set of words each is enough; whose words a call gets: api.cu, take_exchange.
+constexpr int kXScores = 65536;        // chunk scores of all scoring heads that fit (more: the second hand-over by counters)
+struct Exchange {
+    uint32_t last_tag;                 // of the launches so far
+    uint32_t started;                  // CTAs of this launch that have taken its tag
+    alignas(128) ulonglong2 record[kExchangeCtas * 2 * 128];       // [CTA, query tile][row]: maximum, sum
+    ulonglong2 score[kXScores / 2];    // [scoring head][score_row / 2]
+    __device__ void clear() {
+        for (ulonglong2& x : record) x = make_ulonglong2(0ull, 0ull);
+        for (ulonglong2& x : score) x = make_ulonglong2(0ull, 0ull);
+    }
+};
+
 // A launch's tag is the number after the last launch's. One thread of every CTA takes it at its start; the last of them to have done so
 // makes it the last one used, while the keys are under way: nothing is left for the end of the launch, for which the next one waits
 // (the last CTA to leave counted itself out, stored and fenced: 2048 tokens, 2 heads 10.99 -> 10.21 us, 8192 15.4 -> 14.8, 4096 with 4 heads
 // 13.1 -> 12.4). The last tag of all is the exception:
 // at that launch's end words of old launches that were never written again are cleared (end_tags), before the tags start over at 1.
 constexpr uint32_t kLastTag = 0xffffffffu;
-template <class X>
-__device__ __forceinline__ uint32_t take_tag(X& x) {
+__device__ __forceinline__ uint32_t take_tag(Exchange& x) {
     const uint32_t tag = ld_relaxed(&x.last_tag) + 1u;
     uint32_t old;
     asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(&x.started) : "memory");
@@ -157,8 +173,7 @@ __device__ __forceinline__ uint32_t take_tag(X& x) {
     }
     return tag;
 }
-template <class X>
-__device__ __forceinline__ void end_tags(X& x) {
+__device__ __forceinline__ void end_tags(Exchange& x) {
     x.clear();
     x.last_tag = 0u;
 }

@@ -48,17 +48,6 @@ struct TokCtl {
     int abort_flag;
 };
 
-// The hand-over of row statistics, as tagged words (resident.cuh): this kernel only runs with the GPU to itself.
-struct TokExchange {
-    uint32_t last_tag;                 // of the launches so far
-    uint32_t started;                  // CTAs of this launch that have taken its tag
-    alignas(128) ulonglong2 record[kExchangeCtas * 128];   // [CTA][row]: maximum, sum
-    __device__ void clear() {
-        for (ulonglong2& x : record) x = make_ulonglong2(0ull, 0ull);
-    }
-};
-__device__ TokExchange g_tok_exchange;
-
 struct TokArgs {
     int L, P, w, R, Hs, d;
     int n_mt;              // scoring heads per KV head (1 or 2): scoring head v scores rows [128 (v % n_mt), ...) of KV head v / n_mt
@@ -66,6 +55,7 @@ struct TokArgs {
     int cph, n_tiles, n_tiles_prefix, n_stages, q_box_rows, k_box_rows;
     int off_ring, off_misc;
     float* token_scores;   // [Hs][P]
+    Exchange* x;           // row records as tagged words: this kernel only runs with the GPU to itself
     unsigned* exits;
     int* status;
 };
@@ -223,7 +213,7 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const uint32_t acc = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(grp * 128);
         int tg = grp;                                    // this group's next tile, counted over both passes; tile tg uses accumulator tg % 4
         // (behind griddepcontrol.wait; beside the first keys' way here, which the issuing thread should not wait for twice)
-        if (et == 0) *const_cast<volatile uint32_t*>(&ctl.tag) = take_tag(g_tok_exchange);
+        if (et == 0) *const_cast<volatile uint32_t*>(&ctl.tag) = take_tag(*a.x);
         // ---- pass 1: (max, sum of exp2) per row over this CTA's keys
         float run_m = -CUDART_INF_F, run_l = 0.f;
         bool scored = true;
@@ -268,11 +258,11 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 float M = -CUDART_INF_F, S = 0.f;
 #pragma unroll
                 for (int g = 0; g < 4; ++g) merge_ml(M, S, rec[(g * 2) * 128 + row], rec[(g * 2 + 1) * 128 + row]);
-                if (tag != 0u) st_tagged2(&g_tok_exchange.record[static_cast<size_t>(blockIdx.x) * 128 + row], M, S, tag);
+                if (tag != 0u) st_tagged2(&a.x->record[static_cast<size_t>(blockIdx.x) * 128 + row], M, S, tag);
             }
             float M = -CUDART_INF_F, S = 0.f;
             if (tag != 0u && active) {
-                const ulonglong2* src = g_tok_exchange.record + static_cast<size_t>(hs) * a.cph * 128 + row;
+                const ulonglong2* src = a.x->record + static_cast<size_t>(hs) * a.cph * 128 + row;
                 for (int j0 = grp; j0 < a.cph; j0 += 20)             // five records in flight
                     if (!take_records<5, true>(src + j0 * 128, 4 * 128, min(5, (a.cph - j0 + 3) / 4), tag, M, S, abort_flag)) break;
             }
@@ -352,7 +342,7 @@ token_scores_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         if (ctl.abort_flag) atomicExch(a.status, 1);
         if (ctl.tag == kLastTag && atomicAdd(a.exits, 1u) + 1u == gridDim.x) {
             *a.exits = 0u;
-            end_tags(g_tok_exchange);
+            end_tags(*a.x);
             __threadfence();
         }
     }
@@ -401,6 +391,7 @@ cudaError_t launch_token_scores(const TokenPlan& plan, const CUtensorMap& tm_q, 
     a.k_box_rows = io.L < kTTile ? io.L : kTTile;
     a.off_ring = plan.off_ring; a.off_misc = plan.off_misc;
     a.token_scores = io.token_scores;
+    a.x = io.exchange;
     a.exits = io.counters;
     a.status = io.status;
     const void* kern = plan.whole ? reinterpret_cast<const void*>(token_scores_kernel<true>) : reinterpret_cast<const void*>(token_scores_kernel<false>);
