@@ -446,8 +446,7 @@ layer_resident_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_con
             __threadfence_block();
             __syncwarp();
             const int mt = two ? pair : 0, n_g = two ? 2 : 4;
-            uint32_t tag = 0u;
-            while (!*abort_flag && (tag = *const_cast<volatile uint32_t*>(&ctl.tag)) == 0u) {}      // (long there)
+            const uint32_t tag = wait_tag(&ctl.tag, abort_flag);
             int old = 0;
             if (lane == 0) old = atomicAdd(&ctl.rec_count[mt][quarter], 1);
             if (__shfl_sync(0xffffffffu, old, 0) == n_g - 1) {

@@ -173,6 +173,19 @@ __device__ __forceinline__ uint32_t take_tag(Exchange& x) {
     }
     return tag;
 }
+// The tag as the CTA's other threads wait for it (bounded); 0: given up. It is mostly long there.
+__device__ __forceinline__ uint32_t wait_tag(const volatile uint32_t* tag, volatile int* abort_flag) {
+    uint32_t v;
+    long long t0 = 0;
+    for (uint32_t it = 1; (v = *tag) == 0u; ++it) {
+        if (*abort_flag) return 0u;
+        if ((it & 63u) == 0u) {
+            if (t0 == 0) t0 = clock64();
+            if (clock64() - t0 > kWaitLimitClocks) { *abort_flag = 1; return 0u; }
+        }
+    }
+    return v;
+}
 __device__ __forceinline__ void end_tags(Exchange& x) {
     x.clear();
     x.last_tag = 0u;
