@@ -526,6 +526,19 @@ int chunkkv_device_status(void* stream) {
     return CHUNKKV_OK;
 }
 
+// Not part of the API: for the tests of the end of the tags (resident.cuh), which 2^32 - 1 launches on a set of words take otherwise. The
+// words must hold no later tag.
+CHUNKKV_API int chunkkv_test_last_tag(unsigned last_tag) {
+    std::lock_guard<std::mutex> lk(g_mu);
+    DeviceCtx* ctx;
+    int st = get_ctx(&ctx);
+    if (st != CHUNKKV_OK) return st;
+    if (ctx->slot < 0) return CHUNKKV_ENOWORKSPACE;
+    cudaError_t e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaMemcpy(exchange_tags(exchange_slot(ctx->slots, ctx->slot)), &last_tag, sizeof(last_tag), cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? CHUNKKV_OK : cuda_fail(e);
+}
+
 int chunkkv_score(const void* q_obs, const void* K, int L, int Hq, int Hkv, int d, int w, int c,
                   float* out_token_scores, float* out_chunk_scores, void* stream) {
     if (w < 1 || c < 1 || L < w) return CHUNKKV_EINVAL_SHAPE;
