@@ -848,7 +848,8 @@ bool make_resident_plan(int L, int R, int Hkv, int d, int c, int C, int n_max, i
     p.off_pmax = p.off_ring + p.ring_bytes;
     p.off_misc = p.off_pmax + pmax_bytes;
     p.smem_bytes = 1024 + p.off_misc + kRMiscBytes;
-    // after scoring the ring holds the row sums of the chunk scores, then the selection scratch and the kept positions
+    // After scoring the ring holds the row sums of the chunk scores, then the selection's scratch and keys. (A CTA's kept positions, which it
+    // once held as well, still have to have room: calls with more of them stay with the kernels of score.cu.)
     if (static_cast<size_t>(p.n_mt) * 4 * p.t_max * (tile / c) * 4 > static_cast<size_t>(p.ring_bytes)) return false;
     const size_t own = static_cast<size_t>(n_max) / (p.cph << p.shift) + 1;      // kept positions of a CTA
     const size_t sel_bytes = ((sizeof(SelectSmem) + 127) & ~size_t(127)) + ((own * 4 + 127) & ~size_t(127));

@@ -564,7 +564,8 @@ __device__ __forceinline__ void select_core(const float* sc, const float* sc2, i
 }
 
 // The selection, by the number of keys a thread has to take; kbuf: room for C keys in shared memory, used beyond
-// select_reg_keys() keys a thread. The layer kernel and select.cu take select_regs throughout. The other kernels have no registers
+// select_reg_keys() keys a thread. select.cu and the layer kernel's wide variant take select_regs up to there (the layer kernel takes its keys from
+// shared memory otherwise: select_staged). The other kernels have no registers
 // to spare beside their own: with select_regs for 6 keys or more the model kernel spills and a call with 5994 chunks is 8 %
 // slower, so it takes that form up to 4 keys a thread (32 layers of 4096 tokens 348 -> 311 us, 16 layers of 20000 tokens in chunks
 // of 16 228 -> 206); the kernels of score.cu spill with any of it, and so does the model kernel's big variant for chunks of 8 (30 bytes
@@ -579,7 +580,7 @@ enum SelectIn {
     kSelScratch,        // the kernels of score.cu
     kSelModel,          // the model kernel
     kSelModelCore,      // the same without select_regs
-    kSelLayer,          // the layer kernel, at most 16 keys a thread
+    kSelLayer,          // the layer kernel, at most 16 keys a thread (select_staged, not select_kept)
     kSelLayerWide,      // the layer kernel, more
     kSelAlone           // select.cu
 };
@@ -589,23 +590,22 @@ __host__ __device__ constexpr int select_reg_keys(SelectIn where) {
 
 template <SelectIn WHERE>
 __device__ __forceinline__ void select_kept(const float* sc, const float* sc2, int C, int k, SelectSmem& sm, uint32_t* kbuf) {
+    static_assert(WHERE != kSelLayer, "takes its keys from shared memory");
     const int per = (C + static_cast<int>(blockDim.x) - 1) / static_cast<int>(blockDim.x);
-    if constexpr (WHERE != kSelLayer) {
-        if (per > select_reg_keys(WHERE)) return select_core<0>(sc, sc2, C, k, sm, kbuf);
-    }
-    if constexpr (WHERE == kSelModel || WHERE == kSelLayer || WHERE == kSelAlone) {
+    if (per > select_reg_keys(WHERE)) return select_core<0>(sc, sc2, C, k, sm, kbuf);
+    if constexpr (WHERE == kSelModel || WHERE == kSelAlone) {
         // the shortest run that covers the ids: the longer ones leave more warps without any, and a step's time goes with the
         // keys of the busiest scheduler (816 keys: runs of 2 4.5k clocks, of 4 5.2k; 1636 keys: of 4 4.6k, of 8 5.7k)
         if (per <= 2) return select_regs<2>(sc, sc2, C, k, sm);
         if (per <= 4) return select_regs<4>(sc, sc2, C, k, sm);
     }
-    if constexpr (WHERE == kSelLayer || WHERE == kSelAlone) {
+    if constexpr (WHERE == kSelAlone) {
         if (per <= 8) return select_regs<8>(sc, sc2, C, k, sm);
-        if (WHERE == kSelLayer || per <= 16) return select_regs<16>(sc, sc2, C, k, sm);
+        if (per <= 16) return select_regs<16>(sc, sc2, C, k, sm);
     }
     if constexpr (WHERE == kSelLayerWide || WHERE == kSelAlone) {
         select_regs<24>(sc, sc2, C, k, sm);
-    } else if constexpr (WHERE != kSelLayer) {
+    } else {
         if (WHERE == kSelScratch || per <= 8) return select_core<8>(sc, sc2, C, k, sm, nullptr);
         if constexpr (WHERE != kSelScratch) select_core<16>(sc, sc2, C, k, sm, nullptr);
     }
