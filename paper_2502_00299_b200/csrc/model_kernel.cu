@@ -23,8 +23,7 @@
 //                  layer and for every following layer that reuses its indices
 //   warp 19        announces the CTA's record of row statistics, which the last of the epilogue warps that hold the same
 //                  32 rows stores, waits (bounded) for the head's other CTAs - the epilogue threads merge the head's
-//                  records for the contraction, this warp itself where a head has very many CTAs - and
-//                  announces the CTA's chunk scores when they are stored
+//                  records for the contraction - and announces the CTA's chunk scores when they are stored
 // The CTAs after the scoring CTAs are selectors: exact top-k per head, out_idx, kept-chunk lists.
 //
 // So while the selectors and copy threads work on layer l, the other warps already score layer l + 1:
@@ -38,7 +37,6 @@
 #include "select.cuh"
 
 #include <math_constants.h>
-#include <type_traits>
 
 namespace chunkkv {
 
@@ -78,7 +76,6 @@ __host__ __device__ constexpr int model_copy_slots(int c, int d) {
     const int n = 40960 / (4 * c * d);
     return n > kMSlots ? kMSlots : (n < 3 ? 3 : n);
 }
-constexpr int kMOwnMerge = 36;                     // CTAs a head up to which the epilogue threads merge their rows' records
 constexpr int kBarGroup = 2;                       // named barriers 2 .. 5: the four warps of an epilogue group
 
 struct ModelCtl {
@@ -164,33 +161,6 @@ __device__ __forceinline__ void bulk_wait_read() {
     asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
-// Fold N (max, sum-of-exp2) records into (M, S), one row each of four rows at a time: the new maximum
-// first, then N independent factors (a short dependency chain, unlike N merges in sequence).
-template <int N>
-__device__ __forceinline__ void merge_batch(float (&M)[4], float (&S)[4], const float4 (&m)[N], const float4 (&l)[N], int n) {
-    float nm[4] = {M[0], M[1], M[2], M[3]};
-#pragma unroll
-    for (int j = 0; j < N; ++j)
-        if (j < n) {
-            nm[0] = fmaxf(nm[0], m[j].x);
-            nm[1] = fmaxf(nm[1], m[j].y);
-            nm[2] = fmaxf(nm[2], m[j].z);
-            nm[3] = fmaxf(nm[3], m[j].w);
-        }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) S[r] *= ex2_below(M[r], nm[r]);
-#pragma unroll
-    for (int j = 0; j < N; ++j)
-        if (j < n) {
-            S[0] += l[j].x * ex2_below(m[j].x, nm[0]);
-            S[1] += l[j].y * ex2_below(m[j].y, nm[1]);
-            S[2] += l[j].z * ex2_below(m[j].z, nm[2]);
-            S[3] += l[j].w * ex2_below(m[j].w, nm[3]);
-        }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) M[r] = nm[r];
-}
 
 // Bounded wait of a whole warp on a counter that only grows: every lane performs the acquire load, so
 // each lane's later loads are ordered behind the arrivals it has seen. Lane 0 keeps the time limit.
@@ -287,9 +257,6 @@ __device__ __forceinline__ bool selector_loop(const ModelParams& p, uint8_t* dyn
 
 // BIG: two query tiles, or a ring that reaches into scratch. A variant of its own, so that the kernel for up to 128 rows
 // carries none of it.
-// (The reading of row statistics for few rows is a run-time choice below. It makes the small form spill - bytes of stores / loads at c = 10:
-// 16 / 28 instead of none - and is faster for it: with a variant of its own 25 layers of 10000 tokens, 112 rows, c = 10 282.8 -> 287.8 us,
-// 32 layers of 2300 tokens, 128 rows 265 -> 268.5, 9 of 30000 156.7 -> 158.4; other chunk sizes the same.)
 template <int C_STATIC, bool BIG>
 __global__ void __launch_bounds__(kMThreads, 1)
 model_kernel(const __grid_constant__ ModelParams p) {
@@ -314,7 +281,7 @@ model_kernel(const __grid_constant__ ModelParams p) {
     float* pmax = reinterpret_cast<float*>(dyn + p.off_pmax);
     float* misc = reinterpret_cast<float*>(dyn + p.off_misc);
     float* rec = misc;                 // [4 groups][{max, sum}][128]; the odd slots' copy sits at misc + 3072
-    float* gstat = misc + 1024;        // [2 (slot parity)][{m_i, 1 / l_i}][128]; big variant: [4 groups][{m_i, 1 / l_i}][128]
+    float* gstat = misc + 1024;        // [4 groups][{m_i, 1 / l_i}][128]
     float* red = misc + 2048;          // [4 groups][block parity][4 lane quarters][kMBlkSlots]
     volatile int* abort_flag = &ctl.abort_flag;
     const uint32_t n_stages = static_cast<uint32_t>(p.n_stages);
@@ -346,7 +313,6 @@ model_kernel(const __grid_constant__ ModelParams p) {
     const int n_mt = BIG ? p.n_mt : 1;
     const bool two = n_mt == 2;
     const int n_vt = two ? 2 * nt : nt;              // virtual tiles of this CTA per layer
-    const bool own_merge = BIG || p.cph <= kMOwnMerge;      // epilogue threads merge their rows' records themselves
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.n_stages; ++s) {
@@ -552,37 +518,36 @@ model_kernel(const __grid_constant__ ModelParams p) {
                 if (!__shfl_sync(0xffffffffu, ready, 0)) ok = false;   // (the failed wait has raised the abort flag)
                 __syncwarp();          // orders the other lanes' reads below behind the wait; a shuffle alone does not
                 tmem_st_wait();
-                if (own_merge) {
-                    // every record of the head is there (the statistics warp has seen the count): each thread merges those of
-                    // its row, straight from the L2. 18 records took the statistics warp 3 us of a layer's 16 beside four busy
-                    // warps (two query tiles: 8), a group's 128 threads take 0.5; with very many it is the warp's again, which no one waits for.
-                    float M = -CUDART_INF_F, S = 0.f;
-                    const size_t step = static_cast<size_t>(n_mt) * 256;
-                    const float* src = p.cta_stat + ((static_cast<size_t>(c_s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * n_mt +
-                                                     (two ? pair : 0)) * 256 + row;
-                    constexpr int kF = BIG ? 9 : 18;         // records in flight (18 in the small form: 2048 tokens 111 -> 108 us; in the big one 42450 tokens 1174 -> 1207)
-                    for (int j0 = 0; ok && j0 < p.cph; j0 += kF) {
-                        float rm[kF], rl[kF];
+                // every record of the head is there (the statistics warp has seen the count): each thread merges those of
+                // its row, straight from the L2. 18 records took the statistics warp 3 us of a layer's 16 beside four busy
+                // warps (two query tiles: 8), a group's 128 threads take 0.5. With very many as well, up to 144 of one head, although each of the
+                // four groups reads them all: 128 rows, 2 heads, 32 layers of 8192 tokens 454 -> 276 us, 1 head, 12000 tokens 594 -> 323.
+                float M = -CUDART_INF_F, S = 0.f;
+                const size_t step = static_cast<size_t>(n_mt) * 256;
+                const float* src = p.cta_stat + ((static_cast<size_t>(c_s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * n_mt +
+                                                 (two ? pair : 0)) * 256 + row;
+                constexpr int kF = BIG ? 9 : 18;         // records in flight (18 in the small form: 2048 tokens 111 -> 108 us; in the big one 42450 tokens 1174 -> 1207)
+                for (int j0 = 0; ok && j0 < p.cph; j0 += kF) {
+                    float rm[kF], rl[kF];
 #pragma unroll
-                        for (int j = 0; j < kF; ++j) {
-                            const bool in = j0 + j < p.cph;
-                            rm[j] = in ? __ldcg(src + (j0 + j) * step) : -CUDART_INF_F;
-                            rl[j] = in ? __ldcg(src + (j0 + j) * step + 128) : 0.f;
-                        }
-                        float bm = M;
-#pragma unroll
-                        for (int j = 0; j < kF; ++j) bm = fmaxf(bm, rm[j]);
-                        float acc = S * ex2_below(M, bm);
-#pragma unroll
-                        for (int j = 0; j < kF; ++j) acc += rl[j] * ex2_below(rm[j], bm);
-                        M = bm;
-                        S = acc;
+                    for (int j = 0; j < kF; ++j) {
+                        const bool in = j0 + j < p.cph;
+                        rm[j] = in ? __ldcg(src + (j0 + j) * step) : -CUDART_INF_F;
+                        rl[j] = in ? __ldcg(src + (j0 + j) * step + 128) : 0.f;
                     }
-                    gstat[grp * 256 + row] = M;                // (read back by this thread only)
-                    gstat[grp * 256 + 128 + row] = 1.0f / S;
+                    float bm = M;
+#pragma unroll
+                    for (int j = 0; j < kF; ++j) bm = fmaxf(bm, rm[j]);
+                    float acc = S * ex2_below(M, bm);
+#pragma unroll
+                    for (int j = 0; j < kF; ++j) acc += rl[j] * ex2_below(rm[j], bm);
+                    M = bm;
+                    S = acc;
                 }
+                gstat[grp * 256 + row] = M;                // (read back by this thread only)
+                gstat[grp * 256 + 128 + row] = 1.0f / S;
             }
-            const float* gm = gstat + (own_merge ? grp : c_s & 1) * 256;
+            const float* gm = gstat + grp * 256;
             const float mi = gm[row], li = gm[128 + row];
             float* rb = rg + c_par * (4 * kMBlkSlots);
             if (own > 0) {
@@ -747,54 +712,17 @@ model_kernel(const __grid_constant__ ModelParams p) {
     } else if (warp == 19) {
         // ------------------------------------------------------------------ statistics warp
         // Per slot: announce the CTA's record once it is stored, wait (bounded) until every CTA of the scoring head has
-        // announced its own, let the epilogue merge them - or, with very many CTAs a head, merge them here into m_i and
-        // 1 / l_i, four rows per lane - and announce the CTA's chunk scores once the epilogue has stored them.
-        const int r0 = 4 * lane;
+        // announced its own, let the epilogue merge them, and announce the CTA's chunk scores once the epilogue has stored them.
         bool ok = true;
         for (int s = 0; s < p.n_compute && ok; ++s) {
             bool w_ok = true;
             if (lane == 0)
                 w_ok = mbar_wait(smem_u32(&ctl.pub_done[s & 1]), static_cast<uint32_t>(s >> 1) & 1u, abort_flag);
             if (!__shfl_sync(0xffffffffu, w_ok, 0)) break;
-            __syncwarp();              // (as above: the other lanes read what the epilogue warps left in shared memory)
+            __syncwarp();
             // release, behind the wait that acquired what the epilogue warps stored: the record is visible to whoever sees the count
             if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.cnt_a + hkv) : "memory");
             if (!wait_counter_warp(p.cnt_a + hkv, static_cast<unsigned>(s + 1) * p.cph, abort_flag)) break;
-            if (!own_merge) {
-                // the head's records straight from the L2 (they were written by other SMs; every lane has
-                // acquired the counter), nine CTAs' worth of loads in flight per lane. Up to 64 rows each half of the warp
-                // takes every other record (2 heads: 69 CTAs, 32 layers of 8192 tokens 490 -> 330 us with the selection by runs).
-                const float* src = p.cta_stat + (static_cast<size_t>(s & 1) * gridDim.x + static_cast<size_t>(hkv) * p.cph) * 256;
-                float M[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F}, S[4] = {0.f, 0.f, 0.f, 0.f};
-                auto fold = [&](const float* from, auto stride, int n) {
-                    constexpr int kStride = decltype(stride)::value;
-                    for (int j0 = 0; j0 < n; j0 += 9) {
-                        float4 m[9], l[9];
-#pragma unroll
-                        for (int j = 0; j < 9; ++j) {
-                            const int jj = min(j0 + j, n - 1);
-                            m[j] = __ldcg(reinterpret_cast<const float4*>(from + static_cast<size_t>(jj) * kStride));
-                            l[j] = __ldcg(reinterpret_cast<const float4*>(from + static_cast<size_t>(jj) * kStride + 128));
-                        }
-                        merge_batch<9>(M, S, m, l, n - j0);
-                    }
-                };
-                if (p.R > 64) {
-                    fold(src + r0, std::integral_constant<int, 256>{}, p.cph);
-                } else {
-                    const int sub = lane >> 4;
-                    fold(src + sub * 256 + (r0 & 63), std::integral_constant<int, 512>{}, (p.cph - sub + 1) >> 1);
-                    __syncwarp();
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const float mo = __shfl_xor_sync(0xffffffffu, M[r], 16), so = __shfl_xor_sync(0xffffffffu, S[r], 16);
-                        merge_ml(M[r], S[r], mo, so);
-                    }
-                }
-                float* gm = gstat + (s & 1) * 256;
-                *reinterpret_cast<float4*>(gm + r0) = make_float4(M[0], M[1], M[2], M[3]);
-                *reinterpret_cast<float4*>(gm + 128 + r0) = make_float4(1.0f / S[0], 1.0f / S[1], 1.0f / S[2], 1.0f / S[3]);
-            }
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(smem_u32(&ctl.stat_full[s & 1]));
