@@ -90,7 +90,7 @@ CHUNKKV_API size_t chunkkv_workspace_bytes(int L, int Hq, int Hkv, int d, int w,
 
 /*
  * Set-up: use caller-owned device memory (256-byte aligned, on the current device) as scratch for
- * all later calls on this device. Its first 256 bytes hold the library's device status word and
+ * all later calls on this device. Its first 2048 bytes hold the library's device status word and
  * hand-over counters and are cleared by this call. This is the one call that synchronises the
  * device (work queued earlier may still be using the previous buffer). Passing (NULL, 0) detaches
  * the buffer. The caller keeps ownership and must keep the buffer alive while calls may use it.
@@ -324,7 +324,7 @@ CHUNKKV_API int chunkkv_jaccard(const int32_t* idx_a, const int32_t* idx_b, int 
  * bandwidth-bound scoring and gathering of the others.
  *
  *   chunkkv_lane_bytes          scratch a lane needs for a shape with a CTA budget (0 = all SMs)
- *   chunkkv_lane_init           clears the lane's 256-byte header (queued on `stream`); call once
+ *   chunkkv_lane_init           clears the lane's header (queued on `stream`); call once
  *                               before first use, and again before using the lane with a different
  *                               CTA budget
  *   chunkkv_compress_layer_lane chunkkv_compress_layer with the lane's scratch and at most

@@ -383,7 +383,7 @@ size_t score_with_scratch_bytes(int L, int Hq, int Hkv, int d, int w, int c) {
     return get_ctx(&ctx) == CHUNKKV_OK ? score_path_bytes(*ctx, L, Hq, Hkv, d, w, c) : 0;
 }
 
-// Scoring into caller-supplied scratch (256-byte header + payload). Used by the fixed-scratch
+// Scoring into caller-supplied scratch (header + payload). Used by the fixed-scratch
 // entry point; allocates nothing and records no profiling events.
 int score_with_scratch(const void* q_obs, const void* K, int L, int Hq, int Hkv, int d, int w, int c,
                        float* out_scores, void* scratch, size_t scratch_bytes, cudaStream_t stream) {

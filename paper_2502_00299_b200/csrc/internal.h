@@ -246,7 +246,7 @@ cudaError_t launch_pair_sum(const float* in, float* out, int Hkv, int C, cudaStr
 cudaError_t launch_gather_shared_sms(const void* K, const void* V, const int32_t* idx, int L, int Hkv, int d,
                                      int n_max, void* out_K, void* out_V, int num_sms, cudaStream_t stream);
 
-// Scoring (score + finalisation kernels) into caller-supplied scratch: a 256-byte header whose
+// Scoring (score + finalisation kernels) into caller-supplied scratch: a header whose
 // first word is the device status word, then the payload. Returns a CHUNKKV_* status;
 // CHUNKKV_ETOOLARGE if scratch_bytes is too small. Allocates nothing.
 size_t score_with_scratch_bytes(int L, int Hq, int Hkv, int d, int w, int c);

@@ -69,8 +69,9 @@ def test_model_scratch_never_shrinks_for_a_longer_sequence(ck, Hq, Hkv, w, c):
     assert all(a <= b for a, b in zip(need, need[1:])), [L for L, a, b in zip(sorted(lens)[1:], need, need[1:]) if a > b][:5]
 
 
-# Either side of the length up to which five to eight heads have a selector CTA each (6 tiles of 120 keys a CTA)
-@pytest.mark.parametrize("Hkv,L", [(5, 20160), (6, 16560), (7, 14400), (8, 12240)])
+# Either side of lengths at which a tile more a CTA is due, and with it more or fewer selector CTAs: 6 heads 6 -> 4, 8 heads 8 -> 4 and back, 12
+# heads 12 -> 4, 16 heads 16 -> 4 (5 and 7 heads keep as many)
+@pytest.mark.parametrize("Hkv,L", [(5, 20160), (6, 16560), (7, 14400), (8, 12240), (8, 10200), (8, 10698), (12, 14520), (16, 15360)])
 def test_model_call_in_scratch_sized_for_a_longer_sequence(ck, Hkv, L):
     d, w, c = 64, 8, 10
     budget = w + c * (L // (12 * c))
