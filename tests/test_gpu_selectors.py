@@ -13,6 +13,8 @@ pytestmark = pytest.mark.gpu
     (8, 8, 64, 1000, 8, 10, 100, 1), (8, 8, 64, 8200, 8, 10, 4000, 3), (64, 8, 64, 4100, 32, 10, 400, 1),
     (12, 12, 64, 700, 8, 5, 150, 2), (16, 16, 64, 1500, 8, 16, 300, 1), (20, 20, 64, 900, 8, 10, 120, 1), (33, 33, 64, 600, 8, 20, 100, 2),
     (140, 140, 64, 300, 4, 10, 50, 1),
+    # either side of a change: 8 -> 4, twice
+    (64, 8, 64, 4080, 32, 10, 400, 1), (64, 8, 64, 4081, 32, 10, 400, 1), (8, 8, 64, 10200, 8, 10, 100, 1), (8, 8, 64, 10201, 8, 10, 100, 1),
 ])
 def test_model_call(Hq, Hkv, d, L, w, c, budget, reuse):
     import paper_2502_00299_b200 as ck
